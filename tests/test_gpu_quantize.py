@@ -149,3 +149,28 @@ def test_random_hadamard_recipe_matches_the_oracle_byte_for_byte(case):
         assert np.linalg.norm(back - x) / np.linalg.norm(x) < 0.2
     finally:
         h.close()
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("rows,cols,pad", [(16, 64, 0), (16, 64, 8), (33, 64, 4), (130, 1088, 64), (70, 2112, 16), (64, 16448, 4), (3, 16448, 64), (4096, 2112, 0)])
+def test_tensor_amax_sees_every_element(ctx, dtype, rows, cols, pad):
+    """The tensor scale is amax / 2688 whichever element is the largest: corners, the ends of a row, a middle row, and every
+    column of one row (operands of one short row group, rows of several segments, strided rows whose starts do or do not
+    allow 16-byte loads).  The columns beyond the operand hold larger values and must not count."""
+    B, h = ctx
+    if dtype == torch.bfloat16 and pad % 8:
+        pad += 4                                     # the library wants rows on 16-byte boundaries
+    full = torch.rand((rows, cols + pad), device="cuda").to(dtype)
+    full[:, cols:] = 1000.0
+    x = full[:, :cols]
+    spots = {(0, 0), (0, cols - 1), (rows - 1, 0), (rows - 1, cols - 1), (rows // 2, cols // 2)} | {(rows // 3, c) for c in range(0, cols, max(1, cols // 37))}
+    for r, c in sorted(spots):
+        old = x[r, c].clone()
+        x[r, c] = -7.0
+        t, _ = h.quantize_nvfp4(x)
+        assert t.tensor_scale.item() == float(np.float32(7.0) / np.float32(2688.0)), (r, c)
+        x[r, c] = old
+    x[rows - 1, cols // 2] = float("nan")
+    h.quantize_nvfp4(x)
+    torch.cuda.synchronize()
+    assert h.device_status() != 0
