@@ -12,6 +12,8 @@
 // All four quantized cross terms of the paper's expansion are kept.
 #include "common.cuh"
 
+#include <cuda_fp16.h>
+
 bool metis_gemm_tc_can_fuse(const metis_nvfp4_t* a, const metis_nvfp4_t* b);
 metis_status_t metis_launch_gemm_tc_fused(metis_context* ctx, const metis_nvfp4_t* a, const metis_nvfp4_t* b, void* d,
                                           int d_dtype, int64_t ldd, const void* lx, const void* rx, int kx, cudaStream_t s);
@@ -332,108 +334,310 @@ rank_update_kernel(const float* __restrict__ y0, int64_t M, int64_t N, int kc, c
 // G (n x m, FP32 or BF16, as produced by the wgrad product) and a dequantized factor F stored k x len:
 //   TRANS = 0:  out[t][r] = scale_t * sum_c G[r][c] F[t][c]      (r over n, c over m:  dL/dV from U)
 //   TRANS = 1:  out[t][r] = scale_t * sum_c G[c][r] F[t][c]      (r over m, c over n:  dL/dU from V)
-// scale_t = sigma_t.  One CTA owns 32 values of r and walks c in chunks of 32; FP32 FMAs, fixed summation
-// order (deterministic).  With `other` given (the factor lying along r), the CTA also writes its partial of
-//   dsigma[t] = sum_r other[t][r] * (sum_c ...)   to ds_part[blockIdx.x][t].
-constexpr int FG_ROWS = 32, FG_CHUNK = 32;
-template <int KT, bool TRANS>                           // KT = ceil(k / 8) outputs per thread
-__global__ void __launch_bounds__(256)
-factor_grad_kernel(const void* __restrict__ gsrc, int g_dtype, int64_t ldg, int64_t n_r, int64_t n_c, int k, int t0, int k_all,
+// scale_t = sigma_t.  With `other` given (the factor lying along r), a strip also writes its partial of
+//   dsigma[t] = sum_r other[t][r] * (sum_c ...)   to ds_part[strip][t].
+//
+// A contraction whose large operand is read once: bound by the bytes of G.  A factor entry without its tensor scale
+// is an E2M1 x E4M3 product and exact in BF16, an FP32 gradient is three BF16 terms, so the products of mma.sync are
+// exact and only the FP32 sums round.  The tensor core truncates its sums, so an accumulator runs over one chunk (12 adds)
+// and is then added to an FP32 total.  A CTA owns a strip of 64 values of r; its four warps are 2 (r) x 2 (halves of a
+// chunk of 128 values of c), and the CTAs of a cluster divide the chunks; the 2 * cluster totals of a strip are added in a
+// fixed order at the end (shared memory, then distributed shared memory).
+// G goes from global memory straight into fragment registers - every element is used by exactly one thread; the
+// contraction index (and, for TRANS, r) is permuted so that each load is 16 bytes and a warp's loads cover whole
+// 64 / 128-byte runs - and the factor chunk is dequantized into shared memory, double-buffered.
+constexpr int FG_ROWS = 64, FG_CHUNK = 128, FG_KW = FG_CHUNK / 64, FG_THREADS = 64 * FG_KW, FG_PITCH = FG_CHUNK + 16;    // pitch: 8 words mod 32, conflict-free 64-bit fragment loads
+constexpr int fg_smem(int nt) {
+  const int stage = 2 * 8 * nt * FG_PITCH * 2, red = FG_KW * FG_ROWS * (8 * nt + 1) * 4;
+  return stage > red ? stage : red;
+}
+
+__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// the next BF16 term of a pair of floats; x and y become what is left
+__device__ __forceinline__ uint32_t take_bf16x2(float& x, float& y) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
+  x -= __uint_as_float(w << 16);
+  y -= __uint_as_float(w & 0xFFFF0000u);
+  return w;
+}
+// four consecutive elements of G from index `off` on (VEC: 16-byte aligned FP32, 8-byte aligned BF16)
+template <typename T, bool VEC>
+__device__ __forceinline__ float4 fg_load4(const T* g, int64_t off, bool in) {
+  float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  if (!in) return v;
+  if (sizeof(T) == 4) {
+    const float* f = reinterpret_cast<const float*>(g) + off;
+    if (VEC) v = __ldg(reinterpret_cast<const float4*>(f));
+    else v = make_float4(f[0], f[1], f[2], f[3]);
+  } else {
+    const uint16_t* f = reinterpret_cast<const uint16_t*>(g) + off;
+    uint2 w;
+    if (VEC) w = __ldg(reinterpret_cast<const uint2*>(f));
+    else w = make_uint2((uint32_t)f[0] | ((uint32_t)f[1] << 16), (uint32_t)f[2] | ((uint32_t)f[3] << 16));
+    v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
+  }
+  return v;
+}
+
+// the two E2M1 codes of the low byte as FP16 (exact)
+__device__ __forceinline__ __half2 e2m1x2_to_half2(uint32_t byte) {
+  uint32_t w;
+  asm("{ .reg .b8 t; cvt.u8.u32 t, %1; cvt.rn.f16x2.e2m1x2 %0, t; }" : "=r"(w) : "r"(byte));
+  return *reinterpret_cast<const __half2*>(&w);
+}
+
+template <int NT, bool TRANS, typename T, bool VEC>     // NT = ceil(k / 8) groups of eight factor vectors, at most 8
+__global__ void __launch_bounds__(FG_THREADS, NT <= 4 ? 3 : 2)
+factor_grad_kernel(const T* __restrict__ gsrc, int64_t ldg, int64_t n_r, int64_t n_c, int k, int t0, int k_all,
                    const uint8_t* f_codes, const uint8_t* f_sf, int f_layout, const float* f_ts,
                    const uint8_t* o_codes, const uint8_t* o_sf, int o_layout, const float* o_ts,
                    const float* __restrict__ sigma, float* __restrict__ out, float* __restrict__ ds_part) {
   // factor vectors t0 .. t0 + k - 1 of k_all (a launch handles at most 64 of them)
-  __shared__ float gs[FG_ROWS][FG_CHUNK + 1];
-  __shared__ __align__(16) float fs[FG_CHUNK][8 * KT + 4];
-  __shared__ float red[8][8 * KT];
-  const int tid = threadIdx.x, r = tid >> 3, tg = tid & 7;
-  const int64_t r0 = (int64_t)blockIdx.x * FG_ROWS;
-  const float fts = *f_ts;
-  float acc[KT];
+  extern __shared__ __align__(16) unsigned char fg_sm[];
+  __nv_bfloat16* fs = reinterpret_cast<__nv_bfloat16*>(fg_sm);                   // [2][8 NT][FG_PITCH]
+  float* red = reinterpret_cast<float*>(fg_sm);                                  // [FG_KW][FG_ROWS][8 NT + 1], after the loop
+  constexpr int RP = 8 * NT + 1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
+  const int mw = warp & 1, kw = warp >> 1;
+  uint32_t rank, csize;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(csize));
+  const int64_t strip = blockIdx.x / csize, r0 = strip * FG_ROWS + 32 * mw;
+  const int chunks = (int)((n_c + FG_CHUNK - 1) / FG_CHUNK), per = (chunks + (int)csize - 1) / (int)csize;
+  const int ch0 = (int)rank * per, ch1 = min(chunks, ch0 + per);
+
+  // A step is 16 values of c: slots {2q, 2q+1, 2q+8, 2q+9} of a fragment hold c = base + 4q .. 4q + 3.
+  //   TRANS = 0: one load is four values of c of row r0 + 16 i + g (+ 8)
+  //   TRANS = 1: one load is r0 + 4g .. 4g + 3 of one c; rows g / g + 8 of fragment i are r0 + 4g + 2i / + 1
+  // Offsets of the four loads at c = 0, and what one value of c adds.
+  int64_t off[4];
+  bool row_in[4];
 #pragma unroll
-  for (int j = 0; j < KT; ++j) acc[j] = 0.0f;
-  for (int64_t c0 = 0; c0 < n_c; c0 += FG_CHUNK) {
-    // tile of G: element (rr, cc) of this chunk
-    for (int o = tid; o < FG_ROWS * FG_CHUNK; o += 256) {
-      const int a = o >> 5, b = o & 31;                 // b runs along the contiguous axis of G
-      const int rr = TRANS ? b : a, cc = TRANS ? a : b;
-      const int64_t gr = r0 + rr, gc = c0 + cc;
-      float v = 0.0f;
-      if (gr < n_r && gc < n_c) {
-        const int64_t off = TRANS ? gc * ldg + gr : gr * ldg + gc;
-        v = g_dtype == METIS_BF16 ? __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(gsrc)[off])
-                                  : reinterpret_cast<const float*>(gsrc)[off];
+  for (int u = 0; u < 4; ++u) {
+    const int64_t r = TRANS ? r0 + 4 * g : r0 + 16 * (u >> 1) + 8 * (u & 1) + g;
+    row_in[u] = r < n_r;
+    off[u] = TRANS ? (4 * q + u) * ldg + r : r * ldg + 4 * q;
+  }
+  const int64_t c_stride = TRANS ? ldg : 1;
+  auto load_step = [&](float4 (&v)[4], int64_t c0) {
+    const int64_t base = c0 * c_stride;
+    const int64_t c_left = n_c - c0 - 4 * q;             // n_c is a multiple of 16: a load is inside or outside as a whole
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = fg_load4<T, VEC>(gsrc, base + off[u], row_in[u] && c_left > (TRANS ? u : 0));
+  };
+  const bool wide_codes = (reinterpret_cast<uintptr_t>(f_codes) & 7u) == 0;      // n_c is a multiple of 16: every block is then aligned
+  // factor chunk ch, dequantized without the tensor scale; rows beyond k and values of c beyond n_c are zero
+  auto stage = [&](int ch, int buf) {
+    const int64_t c_base = (int64_t)ch * FG_CHUNK;
+    for (int o = tid; o < 8 * NT * (FG_CHUNK / 16); o += FG_THREADS) {
+      const int t = o / (FG_CHUNK / 16), b = o % (FG_CHUNK / 16);
+      const int64_t c = c_base + 16 * b;
+      uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+      if (t < k && c < n_c) {
+        const uint8_t* src = f_codes + (int64_t)(t0 + t) * (n_c / 2) + c / 2;
+        uint2 code;
+        if (wide_codes) code = *reinterpret_cast<const uint2*>(src);
+        else code = make_uint2(src[0] | (src[1] << 8) | (src[2] << 16) | ((uint32_t)src[3] << 24), src[4] | (src[5] << 8) | (src[6] << 16) | ((uint32_t)src[7] << 24));
+        // E2M1 pairs to FP16 in one conversion; the products with the block scale have six significant bits and lie
+        // between 2^-10 and 2688, so they are exact in FP16 and in BF16
+        const __half2 sc = __float2half2_rn(metis_e4m3_value(f_sf[metis_sf_offset(t0 + t, c / 16, n_c / 16, f_layout)]));
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float2 v = __half22float2(__hmul2(e2m1x2_to_half2((j < 4 ? code.x : code.y) >> (8 * (j & 3))), sc));
+          const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+          w[j] = *reinterpret_cast<const uint32_t*>(&h);
+        }
       }
-      gs[rr][cc] = v;
+      uint4* dst = reinterpret_cast<uint4*>(fs + (buf * 8 * NT + t) * FG_PITCH + 16 * b);
+      dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+      dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
     }
-    for (int o = tid; o < FG_CHUNK * 8 * KT; o += 256) {
-      const int t = o >> 5, cc = o & 31;
-      fs[cc][t] = (t < k && c0 + cc < n_c) ? deq_at(f_codes, f_sf, f_layout, n_c, t0 + t, c0 + cc) : 0.0f;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int cc = 0; cc < FG_CHUNK; ++cc) {
-      const float gv = gs[r][cc];
+  };
+  float acc[2][NT][4], total[2][NT][4];
 #pragma unroll
-      for (int j = 0; j < KT; ++j) acc[j] = fmaf(gv, fs[cc][tg * KT + j], acc[j]);
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[i][j][e] = total[i][j][e] = 0.0f;
+  // two steps of G are on their way while the two before them are multiplied
+  float4 v_buf[2][2][4];
+  if (ch0 < ch1) {
+    const int64_t c_first = (int64_t)ch0 * FG_CHUNK + 64 * kw;
+    load_step(v_buf[0][0], c_first); load_step(v_buf[0][1], c_first + 16);
+    stage(ch0, 0);
+  }
+  __syncthreads();
+  for (int ch = ch0; ch < ch1; ++ch) {
+    const int buf = (ch - ch0) & 1;
+    const int64_t c_w = (int64_t)ch * FG_CHUNK + 64 * kw;
+#pragma unroll
+    for (int hs = 0; hs < 2; ++hs) {
+      const int64_t c_next = hs == 0 ? c_w + 32 : c_w + FG_CHUNK;               // beyond n_c the loads return zeros
+      if (hs == 0 || ch + 1 < ch1) { load_step(v_buf[hs ^ 1][0], c_next); load_step(v_buf[hs ^ 1][1], c_next + 16); }
+      if (hs == 0 && ch + 1 < ch1) stage(ch + 1, buf ^ 1);
+#pragma unroll
+      for (int st = 0; st < 2; ++st) {
+        const float4 (&v)[4] = v_buf[hs][st];
+        float ax[2][4][2];                                                       // [fragment][register][pair]
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          if (TRANS) {
+            const float* e0 = reinterpret_cast<const float*>(&v[0]) + 2 * i; const float* e1 = reinterpret_cast<const float*>(&v[1]) + 2 * i;
+            const float* e2 = reinterpret_cast<const float*>(&v[2]) + 2 * i; const float* e3 = reinterpret_cast<const float*>(&v[3]) + 2 * i;
+            ax[i][0][0] = e0[0]; ax[i][0][1] = e1[0]; ax[i][1][0] = e0[1]; ax[i][1][1] = e1[1];
+            ax[i][2][0] = e2[0]; ax[i][2][1] = e3[0]; ax[i][3][0] = e2[1]; ax[i][3][1] = e3[1];
+          } else {
+            ax[i][0][0] = v[2 * i].x; ax[i][0][1] = v[2 * i].y; ax[i][1][0] = v[2 * i + 1].x; ax[i][1][1] = v[2 * i + 1].y;
+            ax[i][2][0] = v[2 * i].z; ax[i][2][1] = v[2 * i].w; ax[i][3][0] = v[2 * i + 1].z; ax[i][3][1] = v[2 * i + 1].w;
+          }
+        }
+        uint32_t bf[NT][2];
+#pragma unroll
+        for (int j = 0; j < NT; ++j) {
+          const uint2 w = *reinterpret_cast<const uint2*>(fs + (buf * 8 * NT + 8 * j + g) * FG_PITCH + 64 * kw + 32 * hs + 16 * st + 4 * q);
+          bf[j][0] = w.x; bf[j][1] = w.y;
+        }
+#pragma unroll
+        for (int term = 0; term < (sizeof(T) == 4 ? 3 : 1); ++term) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            uint32_t a[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) a[e] = take_bf16x2(ax[i][e][0], ax[i][e][1]);
+#pragma unroll
+            for (int j = 0; j < NT; ++j) mma_16816(acc[i][j], a, bf[j][0], bf[j][1]);
+          }
+        }
+      }
     }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < NT; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) { total[i][j][e] += acc[i][j][e]; acc[i][j][e] = 0.0f; }
     __syncthreads();
   }
-  const int64_t gr = r0 + r;
+  // ---- sums of the halves, then of the cluster's CTAs ----
 #pragma unroll
-  for (int j = 0; j < KT; ++j) {
-    const int t = tg * KT + j;
-    acc[j] *= fts;
-    if (t < k && gr < n_r) out[(int64_t)(t0 + t) * n_r + gr] = acc[j] * sigma[t0 + t];
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int row = 32 * mw + (TRANS ? 4 * g + 2 * i + (e >> 1) : 16 * i + g + 8 * (e >> 1));
+        red[(kw * FG_ROWS + row) * RP + 8 * j + 2 * q + (e & 1)] = total[i][j][e];
+      }
+  __syncthreads();
+  for (int o = tid; o < FG_ROWS * 8 * NT; o += FG_THREADS) {
+    const int row = o / (8 * NT), t = o % (8 * NT);
+    float v = red[row * RP + t];
+#pragma unroll
+    for (int w = 1; w < FG_KW; ++w) v += red[(w * FG_ROWS + row) * RP + t];
+    red[row * RP + t] = v;
   }
-  if (ds_part != nullptr) {
-    const float ots = *o_ts;
-    // sum over the CTA's 32 rows in a fixed order: 4 rows per warp by shuffles, then 8 warps through shared memory
+  asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+  // CTA `rank` finishes the factor vectors t = rank, rank + csize, ..., one warp per vector
+  const float fts = *f_ts, ots = ds_part != nullptr ? *o_ts : 0.0f;
+  const uint32_t red_addr = (uint32_t)__cvta_generic_to_shared(red);
+  for (int t = (int)rank + (int)csize * warp; t < k; t += (int)csize * (FG_THREADS / 32)) {
+    float ds = 0.0f;
 #pragma unroll
-    for (int j = 0; j < KT; ++j) {
-      const int t = tg * KT + j;
-      float v = (t < k && gr < n_r) ? acc[j] * deq_at(o_codes, o_sf, o_layout, n_r, t0 + t, gr) * ots : 0.0f;
-      v += __shfl_xor_sync(0xFFFFFFFFu, v, 8);
-      v += __shfl_xor_sync(0xFFFFFFFFu, v, 16);
-      if ((tid & 31) < 8) red[tid >> 5][t] = v;
-    }
-    __syncthreads();
-    if (tid < k) {
+    for (int h = 0; h < 2; ++h) {
+      const int row = lane + 32 * h;
+      const int64_t r = strip * FG_ROWS + row;
       float v = 0.0f;
+      for (uint32_t c = 0; c < csize; ++c) {
+        uint32_t peer;
+        float x;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(red_addr + (uint32_t)(row * RP + t) * 4u), "r"(c));
+        asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(peer));
+        v += x;
+      }
+      v *= fts;
+      if (r < n_r) {
+        out[(int64_t)(t0 + t) * n_r + r] = v * sigma[t0 + t];
+        if (ds_part != nullptr) ds += v * deq_at(o_codes, o_sf, o_layout, n_r, t0 + t, r) * ots;
+      }
+    }
+    if (ds_part != nullptr) {
 #pragma unroll
-      for (int w = 0; w < 8; ++w) v += red[w][tid];
-      ds_part[(int64_t)blockIdx.x * k_all + t0 + tid] = v;
+      for (int o = 16; o > 0; o >>= 1) ds += __shfl_xor_sync(0xFFFFFFFFu, ds, o);
+      if (lane == 0) ds_part[strip * k_all + t0 + t] = ds;
     }
   }
+  asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");   // peers may still be reading
 }
 
-// dsigma[t] = sum over the partials, in order
-__global__ void factor_grad_sigma_kernel(const float* __restrict__ part, int n_part, int k, float* __restrict__ ds) {
-  const int t = threadIdx.x;
+// dsigma[t] = sum over the partials, one warp per t (each lane every 32nd partial, then a fixed tree)
+__global__ void __launch_bounds__(256)
+factor_grad_sigma_kernel(const float* __restrict__ part, int n_part, int k, float* __restrict__ ds) {
+  const int t = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (t >= k) return;
   float v = 0.0f;
-  for (int i = 0; i < n_part; ++i) v += part[(int64_t)i * k + t];
-  ds[t] = v;
+  for (int i = lane; i < n_part; i += 32) v += part[(int64_t)i * k + t];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  if (lane == 0) ds[t] = v;
+}
+
+template <int NT, bool TRANS, typename T, bool VEC>
+metis_status_t launch_factor_grad_nt(cudaStream_t s, const T* g, int64_t ldg, int64_t n_r, int64_t n_c, int kg, int t0, int k, const metis_nvfp4_t* f,
+                                     const metis_nvfp4_t* o, const float* sigma, float* out, float* ds_part) {
+  // CTAs of a cluster divide the contraction until the grid holds the chip's resident CTAs (a strip's work is the whole
+  // contraction: without the split 64 strips of a 4096-wide operand would leave more than half of the SMs idle)
+  const int64_t strips = metis_ceil_div(n_r, FG_ROWS), chunks = metis_ceil_div(n_c, FG_CHUNK);
+  unsigned csize = 1;
+  while (csize < 8 && strips * csize < 3 * 148 && 2 * csize <= chunks) csize *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(strips * csize)); cfg.blockDim = dim3(FG_THREADS); cfg.dynamicSmemBytes = (size_t)fg_smem(NT); cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  METIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, factor_grad_kernel<NT, TRANS, T, VEC>, g, ldg, n_r, n_c, kg, t0, k, (const uint8_t*)f->codes, (const uint8_t*)f->scales,
+      (int)f->sf_layout, (const float*)f->tensor_scale, (const uint8_t*)(o ? o->codes : nullptr), (const uint8_t*)(o ? o->scales : nullptr),
+      (int)(o ? o->sf_layout : 0), (const float*)(o ? o->tensor_scale : nullptr), sigma, out, ds_part));
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+
+template <bool TRANS, typename T, bool VEC>
+metis_status_t launch_factor_grad_t(cudaStream_t s, const T* g, int64_t ldg, int64_t n_r, int64_t n_c, int k, const metis_nvfp4_t* f, const metis_nvfp4_t* o,
+                                    const float* sigma, float* out, float* ds_part) {
+  for (int t0 = 0; t0 < k; t0 += 64) {                  // at most 64 factor vectors per pass over the gradient
+    const int kg = k - t0 < 64 ? k - t0 : 64;
+#define METIS_FG(NT) METIS_TRY((launch_factor_grad_nt<NT, TRANS, T, VEC>(s, g, ldg, n_r, n_c, kg, t0, k, f, o, sigma, out, ds_part)))
+    if (kg <= 8) METIS_FG(1);
+    else if (kg <= 16) METIS_FG(2);
+    else if (kg <= 32) METIS_FG(4);
+    else if (kg <= 48) METIS_FG(6);
+    else METIS_FG(8);
+#undef METIS_FG
+  }
+  return METIS_OK;
 }
 
 template <bool TRANS>
 metis_status_t launch_factor_grad(cudaStream_t s, const void* g, int g_dtype, int64_t ldg, int64_t n_r, int64_t n_c, int k,
                                   const metis_nvfp4_t* f, const metis_nvfp4_t* o, const float* sigma, float* out, float* ds_part) {
-  const unsigned grid = (unsigned)metis_ceil_div(n_r, FG_ROWS);
-#define METIS_FG(KT) factor_grad_kernel<KT, TRANS><<<grid, 256, 0, s>>>(g, g_dtype, ldg, n_r, n_c, kg, t0, k, f->codes, f->scales, f->sf_layout, \
-    f->tensor_scale, o ? o->codes : nullptr, o ? o->scales : nullptr, o ? o->sf_layout : 0, o ? o->tensor_scale : nullptr, sigma, out, ds_part)
-  for (int t0 = 0; t0 < k; t0 += 64) {                  // at most 64 factor vectors per pass over the gradient
-    const int kg = k - t0 < 64 ? k - t0 : 64;
-    switch ((kg + 7) / 8) {
-      case 1: METIS_FG(1); break; case 2: METIS_FG(2); break; case 3: METIS_FG(3); break; case 4: METIS_FG(4); break;
-      case 5: METIS_FG(5); break; case 6: METIS_FG(6); break; case 7: METIS_FG(7); break; case 8: METIS_FG(8); break;
-      default: return METIS_ERR_SHAPE;
-    }
-    METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(cudaGetLastError());
+  // four elements per load when every row starts on the boundary of such a load; element by element otherwise
+  if (g_dtype == METIS_BF16) {
+    const __nv_bfloat16* gb = reinterpret_cast<const __nv_bfloat16*>(g);
+    const bool vec = (reinterpret_cast<uintptr_t>(g) & 7u) == 0 && ldg % 4 == 0;
+    return vec ? launch_factor_grad_t<TRANS, __nv_bfloat16, true>(s, gb, ldg, n_r, n_c, k, f, o, sigma, out, ds_part)
+               : launch_factor_grad_t<TRANS, __nv_bfloat16, false>(s, gb, ldg, n_r, n_c, k, f, o, sigma, out, ds_part);
   }
-#undef METIS_FG
-  return METIS_OK;
+  const float* gf = reinterpret_cast<const float*>(g);
+  const bool vec = metis_aligned16(g) && ldg % 4 == 0;
+  return vec ? launch_factor_grad_t<TRANS, float, true>(s, gf, ldg, n_r, n_c, k, f, o, sigma, out, ds_part)
+             : launch_factor_grad_t<TRANS, float, false>(s, gf, ldg, n_r, n_c, k, f, o, sigma, out, ds_part);
 }
 
 // the host-side checks of factor_grads, callable before anything is enqueued
@@ -463,7 +667,7 @@ metis_status_t factor_grads(metis_context* ctx, const void* dw, int dw_dtype, in
     METIS_TRY(launch_factor_grad<false>(s, dw, dw_dtype, lddw, n, m, w->k, rq, d_sigma ? lq : nullptr, w->sigma, d_left,
                                         d_sigma ? part : nullptr));
     if (d_sigma) {
-      factor_grad_sigma_kernel<<<1, 256, 0, s>>>(part, (int)n_part, w->k, d_sigma); METIS_COUNT_LAUNCH();
+      factor_grad_sigma_kernel<<<(unsigned)metis_ceil_div(w->k, 8), 256, 0, s>>>(part, (int)n_part, w->k, d_sigma); METIS_COUNT_LAUNCH();
       METIS_CUDA_TRY(cudaGetLastError());
     }
   }
@@ -599,6 +803,14 @@ metis_status_t split_gemm(metis_context* ctx, const Side& a, const Side& b, void
 
 metis_status_t metis_linear_set_attrs() {
   METIS_CUDA_TRY(cudaFuncSetAttribute(rank_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * 2 * 128 * 68)));
+#define METIS_FG_ATTR(NT, TR, T, V) METIS_CUDA_TRY(cudaFuncSetAttribute(factor_grad_kernel<NT, TR, T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, fg_smem(NT)))
+#define METIS_FG_ATTRS(NT) \
+  METIS_FG_ATTR(NT, false, float, true); METIS_FG_ATTR(NT, false, float, false); METIS_FG_ATTR(NT, true, float, true); METIS_FG_ATTR(NT, true, float, false); \
+  METIS_FG_ATTR(NT, false, __nv_bfloat16, true); METIS_FG_ATTR(NT, false, __nv_bfloat16, false); METIS_FG_ATTR(NT, true, __nv_bfloat16, true); \
+  METIS_FG_ATTR(NT, true, __nv_bfloat16, false)
+  METIS_FG_ATTRS(1); METIS_FG_ATTRS(2); METIS_FG_ATTRS(4); METIS_FG_ATTRS(6); METIS_FG_ATTRS(8);
+#undef METIS_FG_ATTRS
+#undef METIS_FG_ATTR
   return METIS_OK;
 }
 

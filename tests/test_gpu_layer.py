@@ -152,6 +152,37 @@ def test_factor_gradients(ctx, dw_dtype):
                 "dS": rel_fro(d_sigma.cpu().numpy(), ds)}, (xo, xq), (wo, wq), (do, dq), base_tol=base)
 
 
+@pytest.mark.parametrize("l,n,m,k,dtype,pad", [
+    (128, 64, 64, 4, torch.float32, 0),            # one strip, one ragged chunk, the smallest rank
+    (128, 320, 2112, 20, torch.float32, 2),        # rows that start off the 16-byte boundary: element loads
+    (128, 2112, 320, 36, torch.bfloat16, 2),
+    (256, 1088, 960, 64, torch.bfloat16, 0),
+    (256, 576, 1024, 68, torch.float32, 0),        # more than 64 vectors: a second pass with four of them
+    (256, 9536, 192, 8, torch.float32, 0),         # a long contraction for few columns: clusters of eight
+])
+def test_factor_gradient_strips_and_chunks(ctx, l, n, m, k, dtype, pad):
+    """The contractions against float64 from the library's own dw and factors.  Every product is exact and a partial sum runs
+    over at most a few hundred FP32 additions of at most twelve tensor-core adds each: 2e-6 of the result in norm."""
+    from gpu_util import rel_fro, nv_dequant
+    B, h = ctx
+    torch.manual_seed(n + k)
+    xo = h.split(torch.randn(l, m, device="cuda").to(torch.bfloat16), 0, 0)
+    do = h.split(torch.randn(l, n, device="cuda").to(torch.bfloat16), 0, 0)
+    wo = B.Operand(n, m, k)
+    wo.left_q, wo.right_q = h.quantize_nvfp4(torch.randn(k, n, device="cuda"))[0], h.quantize_nvfp4(torch.randn(k, m, device="cuda"))[0]
+    wo.sigma.copy_(torch.rand(k, device="cuda") + 0.5)
+    fg = (torch.full((k, n), float("nan"), device="cuda"), torch.full((k,), float("nan"), device="cuda"), torch.full((k, m), float("nan"), device="cuda"))
+    dw = torch.empty((n, m + pad), dtype=dtype, device="cuda")[:, :m]
+    h.linear_bwd(do, xo, wo, need_dx=False, out=(None, dw), factor_grads=fg)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    dwn = dw.float().cpu().numpy().astype(np.float64)
+    lq, rq, sig = nv_dequant(wo.left_q)[:k].T, nv_dequant(wo.right_q)[:k].T, wo.sigma.cpu().numpy().astype(np.float64)
+    assert rel_fro(fg[0].cpu().numpy().T, (dwn @ rq) * sig) < 2e-6
+    assert rel_fro(fg[2].cpu().numpy().T, (dwn.T @ lq) * sig) < 2e-6
+    assert rel_fro(fg[1].cpu().numpy(), np.einsum("jt,ji,it->t", lq, dwn, rq)) < 1e-5
+
+
 def test_factor_gradients_need_the_weight_gradient(ctx):
     from gpu_util import to_dev_bf16
     B, h = ctx
