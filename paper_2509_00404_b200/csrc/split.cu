@@ -7,6 +7,7 @@
 //   with the NVFP4 quantizer in both block orientations -> factor rotation, sign fix, factor quantization.
 #include "quant_tile.cuh"
 #include "bigrank.cuh"
+#include "small_eig.cuh"
 
 metis_status_t metis_launch_residual_tc(metis_context* ctx, const void* x, const float* coef, int k, int kp,
                                         const metis_qt::QuantParams& qp, const float* amax_src, float* ts_out0, float* ts_out1,
@@ -14,8 +15,8 @@ metis_status_t metis_launch_residual_tc(metis_context* ctx, const void* x, const
 
 namespace {
 
-constexpr int MAXQ = 72;                               // k + p at most (k = 64 with p = 8)
-constexpr size_t JACOBI_SMEM = sizeof(double) * MAXQ * (MAXQ + 1);
+constexpr int MAXQ = metis_small::MAXQ;                // k + p at most (k = 64 with p = 8)
+constexpr int LP = metis_small::PITCH;                 // row pitch of a factor in shared memory
 
 // ------------------------------------------------------------------------------------------------
 __global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, int64_t rows, uint64_t seed, int full) {
@@ -60,214 +61,77 @@ __global__ void reduce_partials_kernel(const float* __restrict__ zp, int n_chunk
 // ------------------------------------------------------------------------------------------------
 // Gram partials in FP64: part[p][i][j] = sum over the p-th slab of rows r of v(r,i) v(r,j),
 // v(r,i) = V[r*stride_row + i*stride_vec].
-constexpr int GR_TILE = 32;
-constexpr int GR_PITCH = MAXQ + 2;                      // doubles per tile row: even, so that 4-wide groups stay 16-byte aligned
-constexpr int GR_NB = (MAXQ + 3) / 4;                   // 4 x 4 output blocks per dimension
+// On the FP64 tensor cores: 64 rows at a time are converted to FP64 in shared memory (FP32 -> FP64 conversions are a slow-rate
+// instruction: once per element), a warp owns up to six lower 8 x 8 tiles of the result.  As FP64 multiply-adds
+// from shared memory the same slabs took 8.4 us (4096 x 40) and 24 us (16384 x 40).
+constexpr int GR_TILE = 64;
+constexpr int GR_TPW = 6;                               // tiles per warp: 45 lower tiles at n = 72 over eight warps
 __global__ void __launch_bounds__(256)
 gram_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t stride_row, int64_t stride_vec,
             int64_t rows_per_part, double* __restrict__ part, const int* __restrict__ skip) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;                 // second CholeskyQR pass not needed (see chol_kernel)
-  // The tile is converted to FP64 once when it is staged (FP32 -> FP64 conversions are a slow-rate instruction).
-  // A thread owns 4 x 4 blocks of the output: eight shared-memory loads feed sixteen multiply-adds, which keeps
-  // the kernel off the shared-memory pipe that bounds a one-output-per-thread formulation.
-  __shared__ __align__(16) double tile[GR_TILE][GR_PITCH];
-  const int tid = threadIdx.x;
+  __shared__ double tile[GR_TILE][LP];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q4 = lane & 3;
   const int64_t r_begin = (int64_t)blockIdx.x * rows_per_part;
   const int64_t r_end = min(n_rows, r_begin + rows_per_part);
-  const int nb = (n + 3) / 4, n_blocks = nb * nb;
-  constexpr int BPT = (GR_NB * GR_NB + 255) / 256;      // blocks per thread at the largest n
-  // With at most 128 output blocks (n <= 44) two threads share a block, each taking half of the tile's rows; their
-  // partial sums are added once at the end (second half first into shared memory: a fixed order).
-  const bool halved = 2 * n_blocks <= 256;
-  const int half = halved ? tid / n_blocks : 0;         // 0 or 1 (threads beyond 2 * n_blocks idle)
-  const int rr_begin = halved ? half * (GR_TILE / 2) : 0, rr_end = halved ? rr_begin + GR_TILE / 2 : GR_TILE;
-  double acc[BPT][4][4];
+  const int n8 = (n + 7) & ~7, tiles = (n8 / 8) * (n8 / 8 + 1) / 2;
+  int t_i[GR_TPW], t_j[GR_TPW];
+  double acc[GR_TPW][2][2];                             // even and odd steps: two chains in flight
 #pragma unroll
-  for (int b = 0; b < BPT; ++b)
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[b][i][j] = 0.0;
-  for (int i = tid; i < GR_TILE * (GR_PITCH - n); i += 256) {                    // columns n .. pitch-1 stay zero
-    const int rr = i / (GR_PITCH - n), ii = n + i % (GR_PITCH - n);
-    tile[rr][ii] = 0.0;
+  for (int u = 0; u < GR_TPW; ++u) {
+    const int o = warp + 8 * u;
+    int ti = 0;
+    while ((ti + 1) * (ti + 2) / 2 <= o) ++ti;
+    t_i[u] = ti; t_j[u] = o - ti * (ti + 1) / 2;
+    acc[u][0][0] = acc[u][0][1] = acc[u][1][0] = acc[u][1][1] = 0.0;
   }
+  for (int i = tid; i < GR_TILE * (n8 - n); i += 256) tile[i / (n8 - n)][n + i % (n8 - n)] = 0.0;
   for (int64_t r0 = r_begin; r0 < r_end; r0 += GR_TILE) {
-    for (int i = tid; i < GR_TILE * n; i += 256) {
-      int rr, ii;
-      if (stride_row == 1) { rr = i % GR_TILE; ii = i / GR_TILE; } else { ii = i % n; rr = i / n; }
-      tile[rr][ii] = (r0 + rr < r_end) ? (double)v[(r0 + rr) * stride_row + ii * stride_vec] : 0.0;
+    if (stride_row == 1) {
+      for (int i = tid; i < GR_TILE * n; i += 256) {
+        const int rr = i % GR_TILE, ii = i / GR_TILE;
+        tile[rr][ii] = r0 + rr < r_end ? (double)v[r0 + rr + ii * stride_vec] : 0.0;
+      }
+    } else {
+      for (int i = tid; i < GR_TILE * n; i += 256) {
+        const int ii = i % n, rr = i / n;
+        tile[rr][ii] = r0 + rr < r_end ? (double)v[(r0 + rr) * stride_row + ii * stride_vec] : 0.0;
+      }
     }
     __syncthreads();
 #pragma unroll
-    for (int b = 0; b < BPT; ++b) {
-      const int o = halved ? tid - half * n_blocks : tid + b * 256;
-      if (o < n_blocks && half < 2 && (!halved || b == 0)) {
-        const int bi = o / nb, bj = o % nb;
-#pragma unroll 4
-        for (int rr = rr_begin; rr < rr_end; ++rr) {
-          const double2 a01 = *reinterpret_cast<const double2*>(&tile[rr][4 * bi]), a23 = *reinterpret_cast<const double2*>(&tile[rr][4 * bi + 2]);
-          const double2 b01 = *reinterpret_cast<const double2*>(&tile[rr][4 * bj]), b23 = *reinterpret_cast<const double2*>(&tile[rr][4 * bj + 2]);
-          const double av[4] = {a01.x, a01.y, a23.x, a23.y}, bv[4] = {b01.x, b01.y, b23.x, b23.y};
+    for (int u = 0; u < GR_TPW; ++u) {
+      if (warp + 8 * u < tiles) {
+        const double* pa = &tile[q4][8 * t_i[u] + g];
+        const double* pb = &tile[q4][8 * t_j[u] + g];
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[b][i][j] += av[i] * bv[j];
+        for (int kk = 0; kk < GR_TILE; kk += 8) {
+          metis_small::dmma(acc[u][0], pa[kk * LP], pb[kk * LP]);
+          metis_small::dmma(acc[u][1], pa[(kk + 4) * LP], pb[(kk + 4) * LP]);
         }
       }
     }
     __syncthreads();
   }
-  if (halved) {
-    double* scratch = &tile[0][0];                      // the tile is free now: GR_TILE * GR_PITCH >= 16 * 128 doubles
-    const int o = tid - half * n_blocks;
-    if (half == 1 && o < n_blocks) {
+  double* out = part + (int64_t)blockIdx.x * n * n;
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+  for (int u = 0; u < GR_TPW; ++u) {
+    if (warp + 8 * u < tiles) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) scratch[o * 16 + i * 4 + j] = acc[0][i][j];
-    }
-    __syncthreads();
-    if (half == 0 && o < n_blocks) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[0][i][j] += scratch[o * 16 + i * 4 + j];
-    }
-  }
-#pragma unroll
-  for (int b = 0; b < BPT; ++b) {
-    const int o = halved ? tid : tid + b * 256;
-    if (o < n_blocks && (!halved || b == 0)) {
-      const int bi = o / nb, bj = o % nb;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (4 * bi + i < n && 4 * bj + j < n) part[(int64_t)blockIdx.x * n * n + (4 * bi + i) * n + 4 * bj + j] = acc[b][i][j];
+      for (int e = 0; e < 2; ++e) {
+        const int i = 8 * t_i[u] + g, j = 8 * t_j[u] + 2 * q4 + e;
+        const double x = acc[u][0][e] + acc[u][1][e];
+        if (i < n && j < n) {
+          out[i * n + j] = x;
+          if (t_i[u] != t_j[u]) out[j * n + i] = x;
+        }
+      }
     }
   }
 }
 
 // ------------------------------------------------------------------------------------------------
-__device__ __forceinline__ double chol_rsqrt(double x) {
-  // scale into the FP32 range by an even power of two, seed with rsqrtf, two Newton steps in FP64
-  int e;
-  const double mant = frexp(x, &e);                     // x = mant * 2^e, mant in [0.5, 1)
-  const int e2 = e & ~1;
-  const double xs = ldexp(mant, e - e2);                // in [0.5, 2)
-  double y = (double)rsqrtf((float)xs);
-  y = y * (1.5 - 0.5 * xs * y * y);
-  y = y * (1.5 - 0.5 * xs * y * y);
-  return ldexp(y, -(e2 / 2));
-}
-
-__device__ __forceinline__ double fast_rsqrt_wide(double x) { return chol_rsqrt(x); }
-
-// 1/x in FP64: the hardware's 20-bit FP64 reciprocal seed and three Newton steps
-__device__ __forceinline__ double chol_rcp(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = y * (2.0 - x * y);
-  y = y * (2.0 - x * y);
-  y = y * (2.0 - x * y);
-  return y;
-}
-
-// In-place Cholesky of the n x n lower triangle of Y (row pitch P doubles) by the first 256 threads of the CTA.
-// Right-looking with the column scaling deferred: step j only subtracts  Y[a][j] Y[b][j] / Y[j][j]  from the
-// trailing triangle (one barrier per column, a reciprocal instead of a square root in the serial chain); the
-// columns are divided by sqrt(pivot) together at the end.  The matrix lives in registers for the whole
-// factorisation - thread (ty, tx) of a 16 x 16 grid keeps the elements (ty + 16u, tx + 16v) - and a step reads
-// only column j and the reciprocal of its pivot, which their owners publish through shared memory before the
-// barrier of the step before; the step itself has no data-dependent branch.  A pivot not above `tol` marks a
-// dependent column: its reciprocal is published as zero, so it takes no part in the updates, and it ends as a
-// zero column with inv_out[j] = 0.
-template <int P>
-__device__ __forceinline__ void cta_cholesky(double (*Y)[P], int n, double tol, double* inv_out, double* dmin_out, int nthr) {
-  constexpr int NB = (MAXQ + 15) / 16;
-  __shared__ double colbuf[2][16 * NB];
-  __shared__ double rd_s[2];
-  const int tid = threadIdx.x, ty = (tid >> 4) & 15, tx = tid & 15;
-  const bool worker = tid < 256;
-  double r[NB][NB];
-#pragma unroll
-  for (int u = 0; u < NB; ++u)
-#pragma unroll
-    for (int v = 0; v <= u; ++v) {
-      const int a = ty + 16 * u, b = tx + 16 * v;
-      r[u][v] = (worker && a < n && b <= a) ? Y[a][b] : 0.0;
-    }
-  if (worker && tx == 0) {
-#pragma unroll
-    for (int u = 0; u < NB; ++u) colbuf[0][ty + 16 * u] = r[u][0];
-  }
-  if (tid == 0) { const double d0 = r[0][0]; rd_s[0] = d0 > tol ? chol_rcp(d0) : 0.0; }
-  __syncthreads();
-  // Steps in phases of sixteen: during phase w (columns 16w .. 16w+15) only the register blocks u, v >= w still
-  // change, so the unrolled block loops shrink from phase to phase (an instruction stream a thread does not run
-  // costs nothing; one it runs predicated-off still costs its issue slots).
-#pragma unroll
-  for (int w = 0; w < NB; ++w) {
-    if (16 * w < n) {
-      const int j_end = min(n, 16 * w + 16);
-      for (int j = 16 * w; j < j_end; ++j) {
-        if (worker) {
-          const double* cb = colbuf[j & 1];
-          const double rd = rd_s[j & 1];                // 0 for a dependent column: the step is a no-op
-          const int jn = j + 1;
-          double la[NB], lb[NB];
-#pragma unroll
-          for (int u = w; u < NB; ++u)
-            if (16 * u < n) { la[u] = cb[ty + 16 * u] * rd; lb[u] = cb[tx + 16 * u]; }
-#pragma unroll
-          for (int u = w; u < NB; ++u)
-#pragma unroll
-            for (int v = w; v <= u; ++v)
-              if (16 * u < n) {
-                const int a = ty + 16 * u, b = tx + 16 * v;
-                if (a > j && b > j && b <= a) r[u][v] -= la[u] * lb[v];
-                if (b == jn) colbuf[jn & 1][a] = r[u][v];
-                if (b == jn && a == jn) { const double dn = r[u][v]; rd_s[jn & 1] = dn > tol ? chol_rcp(dn) : 0.0; }
-              }
-        }
-        __syncthreads();
-      }
-    }
-  }
-  if (worker) {
-#pragma unroll
-    for (int u = 0; u < NB; ++u)
-#pragma unroll
-      for (int v = 0; v <= u; ++v) {
-        const int a = ty + 16 * u, b = tx + 16 * v;
-        if (a < n && b <= a) Y[a][b] = r[u][v];
-      }
-  }
-  __syncthreads();
-  double dj = 0.0, inv = 0.0;
-  if (tid < n) {
-    dj = Y[tid][tid];
-    inv = dj > tol ? chol_rsqrt(dj) : 0.0;
-    inv_out[tid] = inv;
-  }
-  if (dmin_out != nullptr && tid < 32) {                // smallest accepted pivot
-    double dm = 1e300;
-    for (int i = tid; i < n; i += 32) { const double v = Y[i][i]; if (v > tol) dm = fmin(dm, v); }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dm = fmin(dm, __shfl_xor_sync(0xFFFFFFFFu, dm, o));
-    if (tid == 0) *dmin_out = dm;
-  }
-  __syncthreads();
-  for (int o = tid; o < n * n; o += nthr) {
-    const int i = o / n, j = o % n;
-    if (i > j) Y[i][j] *= inv_out[j];
-  }
-  if (tid < n) Y[tid][tid] = dj * inv;                  // sqrt(pivot), or 0 for a dependent column
-  __syncthreads();
-}
-
 // One CholeskyQR pass, step 1 (one CTA): G (one Gram partial) = L L^T in FP64; writes L (q x q, row-major,
 // upper part unused) and the reciprocal pivots.  A pivot below 1e-13 of the largest diagonal marks a
 // dependent sketch column: its reciprocal is stored as zero, so the corresponding column of H = Z L^-T
@@ -277,11 +141,15 @@ chol_kernel(const double* __restrict__ g, int q, double* __restrict__ l_out, dou
             const int* __restrict__ skip, int* __restrict__ well_conditioned) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;
-  __shared__ double L[MAXQ][MAXQ + 1];
+  __shared__ double L[MAXQ][LP];
   __shared__ double gmax_s;
   __shared__ double dmin_s;
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  for (int o = tid; o < q * q; o += 256) L[o / q][o % q] = g[o];
+  const int q8 = (q + 7) & ~7;
+  for (int o = tid; o < q8 * q8; o += 256) {
+    const int i = o / q8, j = o % q8;
+    L[i][j] = i < q && j < q ? g[i * q + j] : 0.0;
+  }
   __syncthreads();
   if (tid < 32) {
     double gm = 0.0;
@@ -293,7 +161,7 @@ chol_kernel(const double* __restrict__ g, int q, double* __restrict__ l_out, dou
   __syncthreads();
   const double tol = 1e-13 * gmax_s;
   __shared__ double inv_s[MAXQ];
-  cta_cholesky<MAXQ + 1>(L, q, tol, inv_s, &dmin_s, 256);
+  metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, 256);
   if (tid < q) invd_out[tid] = inv_s[tid];
   // With every pivot above 1e-8 of the largest diagonal the FP64 factorisation leaves Z L^-T orthonormal to
   // ~1e-8 already, below the FP32 rounding of its storage: the caller's second pass is then skipped.
@@ -303,11 +171,11 @@ chol_kernel(const double* __restrict__ g, int q, double* __restrict__ l_out, dou
 
 // One CholeskyQR pass, steps 0 and 1 in one CTA, for a sketch short enough to sit in shared memory as FP64 (the
 // row-sampled case: a few hundred rows): G = Z^T Z and its Cholesky factor without a trip through global memory.
-// The Gram phase computes the lower 4 x 4 blocks only; S threads (adjacent lanes) share a block, each taking
-// every S-th row, and add their partial sums with shuffles in a fixed order.
+// The Gram matrix is formed on the FP64 tensor cores, a warp per lower 8 x 8 tile (as FP64 multiply-adds from shared memory
+// it took half of the kernel: 22 -> 9 us at 160 x 40 with the panel factorisation).
 constexpr int GC_THREADS = 512;
-constexpr size_t GC_MAX_SMEM = 144 * 1024;              // beside ~45 KiB of static shared memory
-__host__ __device__ inline int gram_chol_pitch(int q) { return 4 * ((q + 3) / 4) + 2; }
+constexpr size_t GC_MAX_SMEM = 176 * 1024;              // beside ~45 KiB of static shared memory: 288 sampled rows at q = 72
+__host__ __device__ inline int gram_chol_pitch(int q) { return ((q + 7) & ~7) + 4; }   // 4 or 12 mod 16: conflict-free fragment loads
 __host__ inline size_t gram_chol_smem(int64_t n_s, int q) { return (size_t)n_s * gram_chol_pitch(q) * sizeof(double); }
 // Well-conditioned sketch (every pivot above 1e-8 of the largest diagonal: Z L^-T is orthonormal to ~1e-8 already):
 // the kernel writes L and the reciprocal pivots and clears *applied; apply_chol_kernel, on many CTAs, does the
@@ -319,58 +187,33 @@ gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ l_o
                  int* __restrict__ applied) {
   metis_pdl_wait();
   extern __shared__ __align__(16) double zs[];
-  __shared__ double L[MAXQ][MAXQ + 1];
+  __shared__ double L[MAXQ][LP];
   __shared__ double gmax_s;
   __shared__ double dmin_s;
   __shared__ double inv_s[MAXQ];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nb = (q + 3) / 4, zp = gram_chol_pitch(q);
+  const int q8 = (q + 7) & ~7, zp = gram_chol_pitch(q);
   for (int o = tid; o < n_s * zp; o += GC_THREADS) {
     const int r = o / zp, c = o - r * zp;
     zs[o] = c < q ? (double)z[(int64_t)r * q + c] : 0.0;
   }
-  const int blocks = nb * (nb + 1) / 2;
-  int S = 1;
-  while (2 * S * blocks <= GC_THREADS && S < 32) S *= 2;
-  const int o = tid / S, part = tid - o * S;
-  int bi = 0;
-  while ((bi + 1) * (bi + 2) / 2 <= o) ++bi;
-  const int bj = o - bi * (bi + 1) / 2;
-  const bool active = o < blocks;
+  const int g = lane >> 2, q4 = lane & 3, tiles = (q8 / 8) * (q8 / 8 + 1) / 2;
   bool solved_here = false;
   __syncthreads();
   for (int pass = 0; pass < 2; ++pass) {
-    double acc[4][4];
+    for (int o = warp; o < tiles; o += GC_THREADS / 32) {
+      int ti = 0;
+      while ((ti + 1) * (ti + 2) / 2 <= o) ++ti;
+      const int tj = o - ti * (ti + 1) / 2;
+      double acc[4][2] = {};
+      const double* pa = zs + q4 * zp + 8 * ti + g;
+      const double* pb = zs + q4 * zp + 8 * tj + g;
+      for (int r0 = 0; r0 < n_s; r0 += 16) {               // n_s is a multiple of 16
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    if (active) {
-      const double* pa = zs + 4 * bi;
-      const double* pb = zs + 4 * bj;
-#pragma unroll 2
-      for (int rr = part; rr < n_s; rr += S) {
-        const double2 a01 = *reinterpret_cast<const double2*>(pa + rr * zp), a23 = *reinterpret_cast<const double2*>(pa + rr * zp + 2);
-        const double2 b01 = *reinterpret_cast<const double2*>(pb + rr * zp), b23 = *reinterpret_cast<const double2*>(pb + rr * zp + 2);
-        const double av[4] = {a01.x, a01.y, a23.x, a23.y}, bv[4] = {b01.x, b01.y, b23.x, b23.y};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] += av[i] * bv[j];
+        for (int u = 0; u < 4; ++u) metis_small::dmma(acc[u], pa[(r0 + 4 * u) * zp], pb[(r0 + 4 * u) * zp]);
       }
-    }
-    for (int off = S >> 1; off > 0; off >>= 1) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += __shfl_xor_sync(0xFFFFFFFFu, acc[i][j], off);
-    }
-    if (active && part == 0) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (4 * bi + i < q && 4 * bj + j < q) L[4 * bi + i][4 * bj + j] = acc[i][j];
+      for (int e = 0; e < 2; ++e) L[8 * ti + g][8 * tj + 2 * q4 + e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
     }
     __syncthreads();
     if (tid < 32) {
@@ -382,7 +225,7 @@ gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ l_o
     }
     __syncthreads();
     const double tol = 1e-13 * gmax_s;
-    cta_cholesky<MAXQ + 1>(L, q, tol, inv_s, &dmin_s, GC_THREADS);
+    metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, GC_THREADS);
     if (pass == 0 && dmin_s > 1e-8 * gmax_s) break;
     // z_row <- z_row L^-T in shared memory, one warp per row (the recurrence of apply_chol_kernel)
     solved_here = true;
@@ -423,7 +266,7 @@ apply_chol_kernel(float* __restrict__ z, int64_t n_rows, int q, const double* __
                   const int* __restrict__ skip) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;
-  __shared__ double L[MAXQ][MAXQ + 1];
+  __shared__ double L[MAXQ][LP];
   __shared__ double inv_s[MAXQ];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int o = tid; o < q * q; o += 256) L[o / q][o % q] = l[o];
@@ -508,173 +351,6 @@ project_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __r
       if (col < cols) dst[(int64_t)(2 * j + jg) * cols + col] = acc0[j];
       if (col + 1 < cols) dst[(int64_t)(2 * j + jg) * cols + col + 1] = acc1[j];
     }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Symmetric positive semi-definite eigen-decomposition (n <= MAXQ) in FP64, one CTA.
-// G = L L^T (Cholesky, dependent columns zeroed), then one-sided (Hestenes) Jacobi on the columns of Y = L:
-// plane rotations make the columns mutually orthogonal, Y J1 J2 ... = U Sigma, so G = Y Y^T = U Sigma^2 U^T:
-// eigenvalues are the squared column norms and eigenvectors the normalised columns.  Working on the
-// Cholesky factor needs one matrix instead of two (no separate eigenvector accumulation), one barrier per
-// round, and converges in few sweeps.  Each round pairs the columns into n/2 disjoint couples (round-robin
-// tournament); a couple is handled by LANES threads that split the rows, reduce the inner product with
-// shuffles and rotate their rows in registers.
-// Input: Gram matrix (ld x ld, leading n x n block used).  Output: eigenvalues descending, eigenvectors as
-// columns of evecs[n][n].
-__device__ __forceinline__ void jacobi_pair(int I, int step, int np, int* p, int* q) {
-  int a, b;
-  if (I == 0) { a = 0; b = (step % (np - 1)) + 1; }
-  else { a = ((step + I) % (np - 1)) + 1; b = ((step + np - 1 - I) % (np - 1)) + 1; }
-  *p = min(a, b); *q = max(a, b);
-}
-
-// 1/sqrt(x) in FP64 from an FP32 seed and two Newton steps (x in the FP32 range; relative error ~1e-16).
-__device__ __forceinline__ double fast_rsqrt(double x) {
-  double y = (double)rsqrtf((float)x);
-  y = y * (1.5 - 0.5 * x * y * y);
-  y = y * (1.5 - 0.5 * x * y * y);
-  return y;
-}
-
-template <int R, int LANES>                             // lanes per couple (8 or 16), rows per lane: ceil(n / LANES)
-__global__ void __launch_bounds__(LANES == 8 ? (R > 8 ? 288 : 256) : (128 * R > 256 ? 128 * R : 256), 1)
-jacobi_eig_kernel(const double* __restrict__ g, int n, int ld, float exit_cos2, double* __restrict__ evals,
-                  double* __restrict__ evecs) {
-  metis_pdl_wait();
-  extern __shared__ __align__(16) unsigned char jsm[];
-  double (*Y)[MAXQ + 1] = reinterpret_cast<double (*)[MAXQ + 1]>(jsm);
-  __shared__ double lam[MAXQ];
-  __shared__ double gmax_s;
-  __shared__ int order[MAXQ];
-  __shared__ uint8_t pairs[MAXQ][MAXQ / 2][2];          // [round][couple] -> (p, q)
-  constexpr int NTHR = LANES == 8 ? (R > 8 ? 288 : 256) : (128 * R > 256 ? 128 * R : 256);
-  const int tid = threadIdx.x;
-  const int np = n + (n & 1), half = np / 2;
-  for (int o = tid; o < np * np; o += NTHR) {
-    const int i = o / np, j = o % np;
-    Y[i][j] = (i < n && j < n) ? 0.5 * (g[i * ld + j] + g[j * ld + i]) : 0.0;
-  }
-  for (int o = tid; o < (np - 1) * half; o += NTHR) {
-    int p, q;
-    jacobi_pair(o % half, o / half, np, &p, &q);
-    pairs[o / half][o % half][0] = (uint8_t)p; pairs[o / half][o % half][1] = (uint8_t)q;
-  }
-  __syncthreads();
-  // ---- Cholesky, lower factor in place; the strict upper triangle is cleared afterwards ----
-  if (tid < 32) {
-    double gm = 0.0;
-    for (int i = tid; i < n; i += 32) gm = fmax(gm, Y[i][i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, o));
-    if (tid == 0) gmax_s = gm;
-  }
-  __syncthreads();
-  const double tol = 1e-14 * gmax_s;
-  cta_cholesky<MAXQ + 1>(Y, n, tol, lam, nullptr, NTHR);
-  for (int o = tid; o < np * np; o += NTHR) {
-    const int i = o / np, j = o % np;
-    if (j > i) Y[i][j] = 0.0;
-  }
-  __syncthreads();
-  // ---- one-sided Jacobi on the columns of Y ----
-  // FP64 is kept for what sets the accuracy of the result - the columns themselves and the orthonormality of
-  // each applied rotation - and FP32 is used for what only steers convergence: the carried column norms, the
-  // rotation angle and the convergence measure.  (FP64 instructions are the slow ones in this latency chain.)
-  // Norms are carried along and recomputed exactly at the start of every sweep, so a round needs a single
-  // inner product per couple.  A sweep whose largest cos^2 between paired columns was below exit_cos2 is the
-  // last one: convergence is quadratic, so its own rotations leave the columns orthogonal to about exit_cos2.
-  float* lamf = reinterpret_cast<float*>(lam);          // FP32 norms during the sweeps (lam is reused below)
-  const int m = tid / LANES, sub = tid % LANES;         // couple index, row slice
-  const bool active = m < half;
-  const int mc = min(m, MAXQ / 2 - 1);                  // table column of this couple slot (idle slots beyond the table share the last)
-  for (int sweep = 0; sweep < 16; ++sweep) {
-    if (tid < np) {
-      double a0 = 0.0, a1 = 0.0;
-      int i = 0;
-      for (; i + 1 < np; i += 2) { a0 += Y[i][tid] * Y[i][tid]; a1 += Y[i + 1][tid] * Y[i + 1][tid]; }
-      if (i < np) a0 += Y[i][tid] * Y[i][tid];
-      lamf[tid] = (float)(a0 + a1);
-    }
-    __syncthreads();
-    int p = active ? pairs[0][m][0] : 0, q = active ? pairs[0][m][1] : 0;
-    bool above = false;                                 // some couple of this slot had cos^2 above exit_cos2 in this sweep
-    for (int step = 0; step < np - 1; ++step) {
-      {
-        // every lane takes part in the shuffles; lanes of couples beyond n/2 carry zeros and write nothing
-        double yp[R], yq[R];
-        double c = 0.0;
-#pragma unroll
-        for (int t = 0; t < R; ++t) {
-          const int i = sub + LANES * t;
-          yp[t] = (active && i < np) ? Y[i][p] : 0.0;
-          yq[t] = (active && i < np) ? Y[i][q] : 0.0;
-          c += yp[t] * yq[t];
-        }
-#pragma unroll
-        for (int o = LANES / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xFFFFFFFFu, c, o);
-        const float a = lamf[p], b = lamf[q], cf = (float)c;
-        // next round's couple, fetched early (after the last round, and for idle couple slots, the table entry is
-        // unused filler: it is inside the array and never used as an index)
-        const int pn = pairs[step + 1][mc][0], qn = pairs[step + 1][mc][1];
-        // rotate only if the two columns are not yet orthogonal to working precision (cos^2 > 1e-26)
-        if (active && cf * cf > 1e-26f * (a * b)) {
-          // tan(theta) = 2c / (d + sign(d) sqrt(d^2 + 4c^2)), d = b - a: the smaller root, |theta| <= pi/4.  These
-          // FP32 quantities only steer convergence, so the fast reciprocal and reciprocal square root are enough.
-          // with cos(2 theta) = |d| / hyp and sin(2 theta) = +-2c / hyp:  cos^2(theta) = (1 + cos 2theta) / 2,
-          // sin(theta) = sin(2 theta) / (2 cos theta): two reciprocal square roots, no division
-          const float d = b - a, c2 = 2.0f * cf;
-          const float h2 = fmaf(c2, c2, d * d);
-          const float rh = rsqrtf(h2);
-          const float cc = fmaf(0.5f * fabsf(d), rh, 0.5f);
-          const float rs = rsqrtf(cc);
-          const float c32 = cc * rs, s32 = (d < 0.0f ? -c2 : c2) * (0.5f * rh) * rs;
-          const float tf = s32 * rs;                      // tan(theta), for the carried norms
-          // (c32, s32) is a unit vector to ~1e-7; one Newton step on 1/sqrt(c^2 + s^2) in FP64 makes it one to ~1e-14
-          const double cd = (double)c32, sd = (double)s32;
-          const double scale = 1.5 - 0.5 * (cd * cd + sd * sd);
-          const double cs = cd * scale, sn = sd * scale;
-#pragma unroll
-          for (int tt = 0; tt < R; ++tt) {
-            const int i = sub + LANES * tt;
-            if (i < np) {
-              Y[i][p] = cs * yp[tt] - sn * yq[tt];
-              Y[i][q] = sn * yp[tt] + cs * yq[tt];
-            }
-          }
-          // |y_p'|^2 = a - t c, |y_q'|^2 = b + t c for the exact rotation.  Every lane of the couple holds the same
-          // numbers and stores them (one value per address): no lane-dependent branch inside the round.
-          const float tc = tf * cf;
-          lamf[p] = a - tc;
-          lamf[q] = b + tc;
-          above |= cf * cf > exit_cos2 * (a * b);
-        }
-        p = pn; q = qn;
-      }
-      __syncthreads();
-    }
-    if (!__syncthreads_or(above ? 1 : 0)) break;        // no couple above the threshold: this was the last sweep
-  }
-  // ---- eigenvalues = squared column norms, eigenvectors = normalised columns ----
-  if (tid < n) {
-    double a = 0.0;
-    for (int i = 0; i < n; ++i) a += Y[i][tid] * Y[i][tid];
-    lam[tid] = a;
-    order[tid] = tid;                                   // stays a valid index if NaNs make the ranks below collide
-  }
-  __syncthreads();
-  if (tid < n) {
-    const double li = lam[tid];
-    int rank = 0;
-    for (int j = 0; j < n; ++j) rank += (lam[j] > li) || (lam[j] == li && j < tid);
-    order[rank] = tid;
-  }
-  __syncthreads();
-  if (tid < n) evals[tid] = lam[order[tid]];
-  for (int o = tid; o < n * n; o += NTHR) {
-    const int i = o / n, j = order[o % n];
-    const double l2 = lam[j];
-    evecs[o] = l2 > 0.0 ? Y[i][j] * fast_rsqrt_wide(l2) : 0.0;
-  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1530,18 +1206,16 @@ int gram_parts(int64_t n_rows, int64_t* rows_per_part) {
   return (int)metis_ceil_div(n_rows, rpp);
 }
 
-void launch_jacobi(cudaStream_t s, const double* g, int n, int ld, float exit_cos2, double* evals, double* evecs) {
-  // sixteen lanes per couple: 8 lanes (longer per-thread instruction streams) and 32 lanes (five shuffle stages, up
-  // to 1024 threads at the barrier) both measured slower
-  const int np = n + (n & 1);
-  switch ((np + 15) / 16) {
-    case 1: (void)(metis_launch_pdl((jacobi_eig_kernel<1, 16>), dim3(1), dim3(256), (size_t)(JACOBI_SMEM), s, g, n, ld, exit_cos2, evals, evecs)); break;
-    case 2: (void)(metis_launch_pdl((jacobi_eig_kernel<2, 16>), dim3(1), dim3(256), (size_t)(JACOBI_SMEM), s, g, n, ld, exit_cos2, evals, evecs)); break;
-    case 3: (void)(metis_launch_pdl((jacobi_eig_kernel<3, 16>), dim3(1), dim3(384), (size_t)(JACOBI_SMEM), s, g, n, ld, exit_cos2, evals, evecs)); break;
-    case 4: (void)(metis_launch_pdl((jacobi_eig_kernel<4, 16>), dim3(1), dim3(512), (size_t)(JACOBI_SMEM), s, g, n, ld, exit_cos2, evals, evecs)); break;
-    default: (void)(metis_launch_pdl((jacobi_eig_kernel<5, 16>), dim3(1), dim3(640), (size_t)(JACOBI_SMEM), s, g, n, ld, exit_cos2, evals, evecs)); break;
+metis_status_t launch_eig(cudaStream_t s, const double* g, int n, int ld, double* evals, double* evecs) {
+  const size_t smem = metis_small::eig_smem(n);
+#define METIS_EIG(NT8) case NT8: METIS_CUDA_TRY(metis_launch_pdl((metis_small::eig_kernel<NT8>), dim3(1), dim3(metis_small::EIG_THREADS), smem, s, g, n, ld, evals, evecs)); break
+  switch ((n + 7) / 8) {
+    METIS_EIG(1); METIS_EIG(2); METIS_EIG(3); METIS_EIG(4); METIS_EIG(5); METIS_EIG(6); METIS_EIG(7); METIS_EIG(8); METIS_EIG(9);
+    default: return METIS_ERR_SHAPE;
   }
+#undef METIS_EIG
   METIS_COUNT_LAUNCH();
+  return METIS_OK;
 }
 
 template <int NJ4>
@@ -1549,13 +1223,6 @@ void launch_project(dim3 grid, cudaStream_t s, const __nv_bfloat16* x, int64_t c
                     const float* h, int rpp, float* mp) {
   (void)(metis_launch_pdl((project_kernel<NJ4>), dim3(grid), dim3(256), (size_t)(0), s, x, cols, idx, n_s, q, h, rpp, mp)); METIS_COUNT_LAUNCH();
 }
-
-int jacobi_threads(int n) {
-  const int half = (n + 1) / 2;
-  int t = (half * half + 31) / 32 * 32;
-  return t < 64 ? 64 : t;
-}
-
 
 // ------------------------------------------------------------------------------------------------
 // Wide sketches (k + p above MAXQ or k above 64, up to 272 / 256): the same decomposition on kernels that tile over
@@ -1811,11 +1478,9 @@ int64_t metis_default_sample_count(int64_t rows, int32_t q) {
 
 metis_status_t metis_split_set_attrs() {
   using namespace metis_qt;
-  METIS_CUDA_TRY(cudaFuncSetAttribute(jacobi_eig_kernel<1, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JACOBI_SMEM));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(jacobi_eig_kernel<2, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JACOBI_SMEM));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(jacobi_eig_kernel<3, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JACOBI_SMEM));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(jacobi_eig_kernel<4, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JACOBI_SMEM));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(jacobi_eig_kernel<5, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)JACOBI_SMEM));
+#define METIS_EIG_ATTR(NT8) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_small::eig_kernel<NT8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_small::eig_smem(8 * NT8)))
+  METIS_EIG_ATTR(1); METIS_EIG_ATTR(2); METIS_EIG_ATTR(3); METIS_EIG_ATTR(4); METIS_EIG_ATTR(5); METIS_EIG_ATTR(6); METIS_EIG_ATTR(7); METIS_EIG_ATTR(8); METIS_EIG_ATTR(9);
+#undef METIS_EIG_ATTR
   METIS_CUDA_TRY(cudaFuncSetAttribute(coeff_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * 9 * 32 * 64)));
   METIS_CUDA_TRY(cudaFuncSetAttribute(coeff_mma_kernel<48>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * 9 * 32 * 48)));
   METIS_CUDA_TRY(cudaFuncSetAttribute(residual_quant_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true)));
@@ -2100,7 +1765,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     int64_t rpp; const int parts = gram_parts(cols, &rpp);
     METIS_CUDA_TRY(metis_launch_pdl((gram_kernel), dim3(parts), dim3(256), (size_t)(0), s, m, cols, q, 1, cols, rpp, gram, nullptr)); METIS_COUNT_LAUNCH();
     METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(q * q, 32)), dim3(128), (size_t)(0), s, gram, parts, q * q, gram1, nullptr)); METIS_COUNT_LAUNCH();
-    launch_jacobi(s, gram1, q, q, 1e-8f, evals, evecs);
+    METIS_TRY(launch_eig(s, gram1, q, q, evals, evecs));
   }
   METIS_CUDA_TRY(metis_launch_pdl((right_basis_kernel), dim3((unsigned)metis_ceil_div(cols, RB_COLS)), dim3(256), (size_t)(0), s, m, cols, q, k, evals, evecs, basis,
                                                                           full ? out->sigma : nullptr)); METIS_COUNT_LAUNCH();
@@ -2168,7 +1833,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   if (!full) {
     // (7) Rayleigh-Ritz on C^T C (Gram partials came out of the broadcast pass), rotate both factors
     METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(kp * kp, 32)), dim3(128), (size_t)(0), sf, gram_c, n_cta_c, kp * kp, gram1, nullptr)); METIS_COUNT_LAUNCH();
-    launch_jacobi(sf, gram1, k, kp, 1e-6f, evals2, evecs2);
+    METIS_TRY(launch_eig(sf, gram1, k, kp, evals2, evecs2));
     METIS_CUDA_TRY(metis_launch_pdl((right_rotate_kernel), dim3(dim3(n_cand, (k + 7) / 8)), dim3(256), (size_t)(0), sf, basis, cols, k, evecs2, out->right, cand_v, cand_i)); METIS_COUNT_LAUNCH();
     METIS_CUDA_TRY(metis_launch_pdl((sign_fix_kernel), dim3(dim3(n_cand, k)), dim3(256), (size_t)(0), sf, out->right, cols, k, cand_v, cand_i, n_cand, sign, amax + 2)); METIS_COUNT_LAUNCH();
     METIS_CUDA_TRY(metis_launch_pdl((left_rotate_kernel), dim3(dim3((unsigned)metis_ceil_div(rows, 64), (unsigned)((kp + 15) / 16))), dim3(256), (size_t)(0), sf, coef, rows, k, k, 1, kp, evecs2, evals2, sign,

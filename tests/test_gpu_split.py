@@ -376,3 +376,31 @@ def test_non_finite_operand_is_reported_in_the_device_status(bad):
             assert not (h.device_status() & B.DEV_TIMEOUT), kind
         finally:
             h.close()
+
+
+@pytest.mark.parametrize("k,p", [(4, 1), (4, 4), (8, 3), (12, 0), (20, 5), (32, 8), (36, 7), (60, 5), (64, 8)])
+@pytest.mark.parametrize("spectrum", ["geometric", "equal", "close", "decades"])
+def test_eigen_solver_sizes_and_spectra(ctx, k, p, spectrum):
+    """Every padding of the small eigen-solver (k + p and k against multiples of eight, odd sizes), with separated, equal,
+    nearly equal and widely graded singular values: the factors are orthonormal and L^T X R is diagonal.  Bounds: FP32 storage of a
+    unit vector of 512 / 320 entries, 2^-24 each, times the coefficients' accumulation over 320 columns - 1e-6 for what
+    a FULL split returns."""
+    B, h = ctx
+    g = torch.Generator(device="cuda")
+    g.manual_seed(100 * k + p)
+    rows, cols = 512, 320
+    u = torch.linalg.qr(torch.randn((rows, k), generator=g, device="cuda", dtype=torch.float64))[0]
+    v = torch.linalg.qr(torch.randn((cols, k), generator=g, device="cuda", dtype=torch.float64))[0]
+    i = torch.arange(k, device="cuda", dtype=torch.float64)
+    s = {"geometric": 3000.0 * 10 ** (-i / k), "equal": 1000.0 + 0 * i, "close": 1000.0 * (1 + 1e-6 * i), "decades": 3000.0 * 10 ** (-3 * i / k)}[spectrum]
+    x = ((u * s) @ v.T + 0.05 * torch.randn((rows, cols), generator=g, device="cuda", dtype=torch.float64)).to(torch.bfloat16)
+    op = h.split(x, k, p, sketch=B.SKETCH_FULL, seed=11)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    left, right, sig, xd = op.left.double(), op.right.double(), op.sigma.double(), x.double()
+    eye = torch.eye(k, device="cuda", dtype=torch.float64)
+    assert (left @ left.T - eye).abs().max() < 1e-6 and (right @ right.T - eye).abs().max() < 1e-6
+    core = left @ xd @ right.T
+    assert (core - torch.diag(torch.diagonal(core))).abs().max() < 1e-6 * sig[0]
+    assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
+    assert bool((sig[:-1] >= sig[1:]).all())
