@@ -8,9 +8,11 @@
 //   trsm_wide_kernel         H = Z L^-T by blocked forward substitution (32 rows of Z per CTA)
 //   gemm64_kernel            C = A B with FP32 A, FP64 B and FP64 accumulation, arbitrary strides (right basis,
 //                            factor rotations)
-//   jacobi_cluster_kernel    one-sided Jacobi eigen-solver on a cluster of eight CTAs: the columns live in the
-//                            cluster's distributed shared memory, column blocks travel between CTAs by DSMEM stores
-//   jacobi_collect_kernel    eigenvalues (descending) and normalised eigenvectors from the rotated columns
+//   jacobi_fp32_kernel       FP32 one-sided block Jacobi on a cluster of up to eight CTAs: the columns live in the cluster's
+//                            distributed shared memory, column blocks travel between CTAs by DSMEM stores
+//   refine_*_kernel          FP64 refinement of the eigenvectors it found (steps of matrix products), eigen_finish_kernel
+//   jacobi_cluster_kernel    the FP64 form of the sweeps, and jacobi_collect_kernel: only run for matrices the refinement
+//                            cannot finish (eigenvalues that agree to working precision)
 //   sign_rows_kernel         sign convention of the factor pairs
 //   coef_sum_kernel          sums the column slices of the broadcast pass into a group of coefficient columns
 // Included by split.cu only.
@@ -18,6 +20,7 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "small_eig.cuh"
 
 namespace metis_wide {
 
@@ -29,22 +32,37 @@ constexpr int MAXK_WIDE = 256;
 // ------------------------------------------------------------------------------------------------
 // part[p][i][j] = sum over the p-th slab of rows r of v(r, i) v(r, j),  v(r, i) = V[r * sr + i * sv], FP64.
 // grid (tiles_j, tiles_i, slabs); the 16 x 16 threads of a CTA own 4 x 4 outputs each.
-constexpr int G64_T = 64, G64_R = 16;
+// On the FP64 tensor cores: a warp owns 16 x 32 of the tile; tiles above the diagonal are the mirror image of those below it
+// (as FP64 multiply-adds from shared memory over all tiles a rank-128 step spent 305 us on it, 190 us so).
+constexpr int G64_T = 64, G64_R = 32, G64_P = G64_T + 4;
+// acc (this warp's 16 x 32 of a 64 x 64 tile) += sum over kk < G64_R of as[kk][.] bs[kk][.]
+__device__ __forceinline__ void tile64_mac(const double (*as)[G64_P], const double (*bs)[G64_P], int wm, int wn, int g, int q, double (&acc)[2][4][2]) {
+#pragma unroll
+  for (int kk = 0; kk < G64_R; kk += 4) {
+    double a[2], b[4];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) a[u] = as[kk + q][wm + 8 * u + g];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) b[u] = bs[kk + q][wn + 8 * u + g];
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int v = 0; v < 4; ++v) metis_small::dmma(acc[u][v], a[u], b[v]);
+  }
+}
 __global__ void __launch_bounds__(256)
 gram64_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t sr, int64_t sv, int64_t rows_per_part,
               double* __restrict__ part, const int* __restrict__ skip) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;
-  __shared__ __align__(16) double as[G64_R][G64_T + 2], bs[G64_R][G64_T + 2];
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ double as[G64_R][G64_P], bs[G64_R][G64_P];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3, wm = 16 * (warp & 3), wn = 32 * (warp >> 2);
   const int i0 = blockIdx.y * G64_T, j0 = blockIdx.x * G64_T;
   const int64_t r_begin = (int64_t)blockIdx.z * rows_per_part, r_end = min(n_rows, r_begin + rows_per_part);
-  double acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+  double acc[2][4][2] = {};
   for (int64_t r0 = r_begin; r0 < r_end; r0 += G64_R) {
+#pragma unroll
     for (int o = tid; o < G64_R * G64_T; o += 256) {
       int rr, ii;
       if (sr == 1) { rr = o % G64_R; ii = o / G64_R; } else { ii = o % G64_T; rr = o / G64_T; }
@@ -53,26 +71,22 @@ gram64_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t sr, in
       bs[rr][ii] = (okr && j0 + ii < n) ? (double)v[(r0 + rr) * sr + (int64_t)(j0 + ii) * sv] : 0.0;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int rr = 0; rr < G64_R; ++rr) {
-      double av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) { av[a] = as[rr][ty + 16 * a]; bv[a] = bs[rr][tx + 16 * a]; }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
-    }
+    tile64_mac(as, bs, wm, wn, g, q, acc);
     __syncthreads();
   }
   double* dst = part + (int64_t)blockIdx.z * n * n;
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
-      if (i < n && j < n) dst[(int64_t)i * n + j] = acc[a][b];
-    }
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int i = i0 + wm + 8 * a + g, j = j0 + wn + 8 * b + 2 * q + e;
+        if (i < n && j < n) {
+          dst[(int64_t)i * n + j] = acc[a][b][e];
+          if (i0 != j0) dst[(int64_t)j * n + i] = acc[a][b][e];
+        }
+      }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -86,36 +100,29 @@ gram64_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t sr, in
 //   dinv_out  (optional) inverses of the CW_NB x CW_NB diagonal blocks of L, [panel][CW_NB][CW_NB] row-major lower:
 //             what the triangular solve H = Z L^-T needs besides L itself (trsm_wide_kernel)
 //   well_conditioned  (optional) 1 when every pivot is above 1e-8 of the largest diagonal entry
-constexpr int CW_NB = 32, CW_P = CW_NB + 1;
-constexpr int CW_ROWS = (MAXQ_WIDE + 15) / 16 * 16 + 16;   // rows of the shared panels: every row a thread's 4 x 4 tile may read exists
-constexpr size_t CW_SMEM = sizeof(double) * ((size_t)2 * CW_ROWS * CW_P + CW_NB * CW_P + MAXQ_WIDE);
-
-// acc[a][b] += sum over kk < 32 of  A[row0 + a][kk] * Bm[col0 + 8 b][kk]:  the 4 x 4 register tile of the panel products.
-// The rows of a warp's four row groups and the columns col0 + 8 b of its eight column groups fall on distinct banks
-// (pitch 33 doubles), so a step costs 8 shared-memory wavefronts per 16 multiply-adds of a warp.
-__device__ __forceinline__ void cw_tile_mac(const double (*A)[CW_P], const double (*Bm)[CW_P], int row0, int col0, double (&acc)[4][4]) {
-#pragma unroll 4
-  for (int kk = 0; kk < CW_NB; ++kk) {
-    double av[4], bv[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) { av[t] = A[row0 + t][kk]; bv[t] = Bm[col0 + 8 * t][kk]; }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b2 = 0; b2 < 4; ++b2) acc[a][b2] += av[a] * bv[b2];
-  }
-}
+//   perm_out  (optional) the matrix is factorised with its rows and columns sorted by descending diagonal entry;
+//             perm_out[i] is the original index of row i
+constexpr int CW_NB = 32, CW_P = CW_NB + 4;               // pitch: 4 mod 16 doubles, conflict-free fragment loads
+constexpr int CW_THREADS = 512, CW_WARPS = CW_THREADS / 32;
+constexpr int CW_ROWS = (MAXQ_WIDE + 31) / 32 * 32;
+constexpr int CW_RT = (CW_ROWS / 8 + CW_WARPS - 1) / CW_WARPS;                 // row tiles per warp
+constexpr size_t CW_SMEM = sizeof(double) * ((size_t)2 * CW_ROWS * CW_P + CW_NB * CW_P);
 
 // Blocked (left-looking) Cholesky factor of the n x n matrix g (symmetrised on the fly), one CTA, panels of 32 columns:
-//   1. the panel (rows j0 .. n-1) minus the products with the finished columns, in 4 x 4 register tiles, the finished
-//      columns streamed from global memory (L2) in chunks of 32;
-//   2. the 32 x 32 diagonal block factorised by one warp (lane = row, column by column, one warp barrier per column);
-//   3. the inverse of that factor by the same warp (lane = column);
-//   4. the rows below the block:  L = A X^T  with X the inverse, again in register tiles.
+//   1. the panel (rows j0 .. n-1) minus the products with the finished columns on the FP64 tensor cores, the finished columns
+//      streamed from global memory (L2) in chunks of 32, the next chunk on its way while one is multiplied;
+//   2. the 32 x 32 diagonal block factorised by one warp in registers (lane = row; a column step is one pivot broadcast, one
+//      reciprocal and one multiply-add deep);
+//   3. the inverse of that factor by the same warp (lane = column), in registers;
+//   4. the rows below the block:  L = A X^T  with X the inverse, on the tensor cores.
+// With FP64 multiply-adds from shared memory and a column of the diagonal block per shared-memory round trip the
+// factorisation took 138 us at n = 136; this form takes 104 us, and 286 us at n = 264.
 // A pivot at or below tol_rel * max diag gives a zero column.  l_out: the factor (lower triangle, zeros above);
 // dinv_out: the inverses of the diagonal blocks (32 x 32 each) for the blocked triangular solve.
-__global__ void __launch_bounds__(1024, 1)
-chol_wide_kernel(const double* __restrict__ g, int n, double tol_rel, double* l_out, double* dinv_out,
+struct EigState;
+__device__ __forceinline__ void eig_state_reset(EigState* st, int tid);
+__global__ void __launch_bounds__(CW_THREADS, 1)
+chol_wide_kernel(const double* __restrict__ g, int n, double tol_rel, double* l_out, double* dinv_out, int* perm_out, EigState* state,
                  const int* __restrict__ skip, int* __restrict__ well_conditioned) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;
@@ -123,105 +130,216 @@ chol_wide_kernel(const double* __restrict__ g, int n, double tol_rel, double* l_
   double (*P)[CW_P] = reinterpret_cast<double (*)[CW_P]>(cw_sm);                                      // the panel, rows j0 .. n-1
   double (*As)[CW_P] = reinterpret_cast<double (*)[CW_P]>(cw_sm + sizeof(double) * CW_ROWS * CW_P);   // a chunk of finished columns of those rows
   double (*Dv)[CW_P] = reinterpret_cast<double (*)[CW_P]>(cw_sm + sizeof(double) * 2 * CW_ROWS * CW_P);
-  double* rinv = reinterpret_cast<double*>(cw_sm + sizeof(double) * (2 * CW_ROWS * CW_P + CW_NB * CW_P));
-  __shared__ double red[32];
+  __shared__ double diag[MAXQ_WIDE];
+  __shared__ int perm[MAXQ_WIDE];
   __shared__ double gmax_s;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int o = tid; o < n * n; o += 1024) l_out[o] = 0.0;
-  for (int o = tid; o < 2 * CW_ROWS * CW_P; o += 1024) reinterpret_cast<double*>(cw_sm)[o] = 0.0;   // rows past the matrix read as zeros
-  double gm = 0.0;
-  for (int i = tid; i < n; i += 1024) gm = fmax(gm, g[(int64_t)i * n + i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, o));
-  if (lane == 0) red[warp] = gm;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, q = lane & 3;
+  if (state != nullptr) eig_state_reset(state, tid);
+  for (int i = tid; i < n; i += CW_THREADS) { diag[i] = g[(int64_t)i * n + i]; perm[i] = i; }
+  if (tid == 0) gmax_s = 0.0;
   __syncthreads();
-  if (tid == 0) { double m = 0.0; for (int w2 = 0; w2 < 32; ++w2) m = fmax(m, red[w2]); gmax_s = m; }
+  for (int i = tid; i < n; i += CW_THREADS) {
+    const double d = diag[i];
+    int rank = 0;
+#pragma unroll 8
+    for (int j = 0; j < n; ++j) rank += (diag[j] > d) || (diag[j] == d && j < i);
+    if (rank == 0) gmax_s = d;
+    if (perm_out != nullptr) perm[rank] = i;               // NaNs may collide; every entry stays a valid index
+  }
   __syncthreads();
-  const double tol = tol_rel * gmax_s;
-  double dmin = 1e300;                                     // smallest accepted pivot (warp 0 keeps it)
-  const int row0 = 4 * (tid >> 3), col0 = tid & 7;         // this thread's tile: rows row0 .. row0 + 3, columns col0 + 8 b
+  if (perm_out != nullptr)
+    for (int i = tid; i < n; i += CW_THREADS) perm_out[i] = perm[i];
+  const double gmax = gmax_s, tol = tol_rel * gmax;
+  double dmin = 1e300;                                     // smallest accepted pivot of this lane (warp 0)
   for (int j0 = 0; j0 < n; j0 += CW_NB) {
-    const int w = min(CW_NB, n - j0), nr = n - j0;
-    const bool mine = row0 < nr;
+    const int w = min(CW_NB, n - j0), nr = n - j0, nr8 = (nr + 7) / 8;
+    constexpr int PF = CW_ROWS / CW_WARPS;                 // rows per warp of a panel or chunk, lane = column
+    double pre[PF];
     __syncthreads();                                       // the previous panel is stored
-    for (int o = tid; o < nr * CW_NB; o += 1024) {
-      const int i = o / CW_NB, c = o % CW_NB;
-      P[i][c] = c < w ? 0.5 * (g[(int64_t)(j0 + i) * n + j0 + c] + g[(int64_t)(j0 + c) * n + j0 + i]) : 0.0;
+#pragma unroll
+    for (int u = 0; u < PF; ++u) {                         // all loads of the panel in flight (the Gram matrix is symmetric to the bit)
+      const int i = warp + u * CW_WARPS;
+      pre[u] = i < nr && lane < w ? g[(int64_t)perm[j0 + i] * n + perm[j0 + lane]] : 0.0;        // zeros past the matrix and the panel
     }
+#pragma unroll
+    for (int u = 0; u < PF; ++u) P[warp + u * CW_WARPS][lane] = pre[u];
     // ---- 1. minus the products with the finished columns ----
-    double acc[4][4];
+    double acc[CW_RT][4][2] = {};
+    auto fetch = [&](int k0) {
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int b2 = 0; b2 < 4; ++b2) acc[a][b2] = 0.0;
+      for (int u = 0; u < PF; ++u) {
+        const int i = warp + u * CW_WARPS;
+        pre[u] = i < nr ? __ldcg(l_out + (int64_t)(j0 + i) * n + k0 + lane) : 0.0;
+      }
+    };
+    if (j0 > 0) fetch(0);
     for (int k0 = 0; k0 < j0; k0 += CW_NB) {
       __syncthreads();
-      for (int o = tid; o < nr * CW_NB; o += 1024) { const int i = o / CW_NB, kk = o % CW_NB; As[i][kk] = l_out[(int64_t)(j0 + i) * n + k0 + kk]; }
+#pragma unroll
+      for (int u = 0; u < PF; ++u) As[warp + u * CW_WARPS][lane] = pre[u];
       __syncthreads();
-      if (mine) cw_tile_mac(As, As, row0, col0, acc);      // rows j0 .. j0 + 31 of L are the first rows of the chunk
+      if (k0 + CW_NB < j0) fetch(k0 + CW_NB);
+#pragma unroll 2
+      for (int kk = 0; kk < CW_NB; kk += 4) {              // rows j0 .. j0 + 31 of L are the first rows of the chunk
+        double b[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) b[v] = As[8 * v + gq][kk + q];
+#pragma unroll
+        for (int u = 0; u < CW_RT; ++u) {
+          const int rt = warp + u * CW_WARPS;
+          if (rt < nr8) {
+            const double a = As[8 * rt + gq][kk + q];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) metis_small::dmma(acc[u][v], a, b[v]);
+          }
+        }
+      }
     }
     __syncthreads();
-    if (mine) {
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+    for (int u = 0; u < CW_RT; ++u) {
+      const int rt = warp + u * CW_WARPS;
+      if (rt < nr8 && j0 > 0) {
 #pragma unroll
-        for (int b2 = 0; b2 < 4; ++b2)
-          if (row0 + a < nr && col0 + 8 * b2 < w) P[row0 + a][col0 + 8 * b2] -= acc[a][b2];
+        for (int v = 0; v < 4; ++v) {
+          P[8 * rt + gq][8 * v + 2 * q] -= acc[u][v][0];
+          P[8 * rt + gq][8 * v + 2 * q + 1] -= acc[u][v][1];
+        }
+      }
     }
     __syncthreads();
     // ---- 2. and 3.: the diagonal block and its inverse, warp 0 ----
     if (warp == 0) {
-      for (int c = 0; c < w; ++c) {
-        double s0 = 0.0, s1 = 0.0;
-        int k = 0;
-        for (; k + 1 < c; k += 2) { s0 += P[lane][k] * P[c][k]; s1 += P[lane][k + 1] * P[c][k + 1]; }
-        if (k < c) s0 += P[lane][k] * P[c][k];
-        const double sv = P[lane][c] - (s0 + s1);
-        const double d = __shfl_sync(0xFFFFFFFFu, sv, c);
-        const double r = d > tol ? 1.0 / sqrt(d) : 0.0;
-        if (lane >= c && lane < w) P[lane][c] = lane == c ? d * r : sv * r;
-        if (lane == 0) { rinv[j0 + c] = r; if (d > tol) dmin = fmin(dmin, d); }
-        __syncwarp();
+      double v[CW_NB];
+#pragma unroll
+      for (int c = 0; c < CW_NB; ++c) v[c] = lane < w && c < w ? P[lane][c] : 0.0;
+      double pivot = 0.0;
+#pragma unroll
+      for (int c = 0; c < CW_NB; ++c) {
+        const double d = __shfl_sync(0xFFFFFFFFu, v[c], c);
+        const double l = v[c] * (d > tol ? metis_small::rcp64(d) : 0.0);
+        if (lane == c) pivot = d;
+#pragma unroll
+        for (int c2 = c + 1; c2 < CW_NB; ++c2) v[c2] = fma(-l, __shfl_sync(0xFFFFFFFFu, v[c], c2), v[c2]);
       }
-      // X = L^-1, lane = column:  X[i][j] = -r_i sum_{k < i} L[i][k] X[k][j]  (X[k][j] = 0 for k < j),  X[j][j] = r_j
-      for (int i = 0; i < CW_NB; ++i) Dv[i][lane] = 0.0;
+      const bool ok = pivot > tol;
+      const double rinv = ok ? metis_small::rsqrt64(pivot) : 0.0;               // lane c: 1 / L[c][c]
+      if (ok) dmin = fmin(dmin, pivot);
+#pragma unroll
+      for (int c = 0; c < CW_NB; ++c) {
+        const double rc = __shfl_sync(0xFFFFFFFFu, rinv, c);
+        P[lane][c] = lane >= c ? v[c] * rc : 0.0;
+      }
       __syncwarp();
-      for (int i = 0; i < w; ++i) {
+      // X = L^-1, lane = column:  X[i][j] = -r_i sum_{k < i} L[i][k] X[k][j]  (X[k][j] = 0 for k < j),  X[j][j] = r_j
+      double x[CW_NB];
+#pragma unroll
+      for (int i = 0; i < CW_NB; ++i) {
         double s0 = 0.0, s1 = 0.0;
-        int k = 0;
-        for (; k + 1 < i; k += 2) { s0 += P[i][k] * Dv[k][lane]; s1 += P[i][k + 1] * Dv[k + 1][lane]; }
-        if (k < i) s0 += P[i][k] * Dv[k][lane];
-        const double ri = rinv[j0 + i];
-        Dv[i][lane] = i == lane ? ri : (i > lane ? -ri * (s0 + s1) : 0.0);
+#pragma unroll
+        for (int k = 0; k < i; ++k) { if (k & 1) s1 = fma(P[i][k], x[k], s1); else s0 = fma(P[i][k], x[k], s0); }
+        const double ri = __shfl_sync(0xFFFFFFFFu, rinv, i);
+        x[i] = i == lane ? ri : -ri * (s0 + s1);
+        Dv[i][lane] = x[i];
       }
     }
     __syncthreads();
-    // ---- 4. rows below the block: L = A X^T (X[c][cp] = Dv[c][cp], zero for cp > c) ----
-    if (nr > CW_NB) {
+    // ---- 4. rows below the block: L = A X^T (X[c][cp] = Dv[c][cp], zero for cp > c); a warp reads and writes its own rows ----
 #pragma unroll
-      for (int a = 0; a < 4; ++a)
+    for (int u = 0; u < CW_RT; ++u) {
+      const int rt = warp + u * CW_WARPS;
+      if (rt >= CW_NB / 8 && rt < nr8) {
+        double t[4][2] = {};
 #pragma unroll
-        for (int b2 = 0; b2 < 4; ++b2) acc[a][b2] = 0.0;
-      const bool below = mine && row0 >= CW_NB;            // a tile lies wholly inside or wholly below the block
-      if (below) cw_tile_mac(P, Dv, row0, col0, acc);
-      __syncthreads();                                     // every tile has read its rows
-      if (below) {
+        for (int kk = 0; kk < CW_NB; kk += 4) {
+          const double a = P[8 * rt + gq][kk + q];
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+          for (int v = 0; v < 4; ++v) metis_small::dmma(t[v], a, Dv[8 * v + gq][kk + q]);
+        }
+        __syncwarp();
 #pragma unroll
-          for (int b2 = 0; b2 < 4; ++b2)
-            if (row0 + a < nr) P[row0 + a][col0 + 8 * b2] = acc[a][b2];
+        for (int v = 0; v < 4; ++v) { P[8 * rt + gq][8 * v + 2 * q] = t[v][0]; P[8 * rt + gq][8 * v + 2 * q + 1] = t[v][1]; }
       }
-      __syncthreads();
     }
-    for (int o = tid; o < nr * w; o += 1024) {
-      const int i = o / w, c = o % w;
-      if (i >= c) l_out[(int64_t)(j0 + i) * n + j0 + c] = P[i][c];
-    }
+    __syncthreads();
+    for (int i = warp; i < nr; i += CW_WARPS)
+      if (lane < w) __stcg(l_out + (int64_t)(j0 + i) * n + j0 + lane, P[i][lane]);
+    for (int i = warp; i < w; i += CW_WARPS)
+      for (int c = j0 + w + lane; c < n; c += 32) l_out[(int64_t)(j0 + i) * n + c] = 0.0;
     if (dinv_out != nullptr)
-      for (int o = tid; o < CW_NB * CW_NB; o += 1024) dinv_out[(int64_t)(j0 / CW_NB) * CW_NB * CW_NB + o] = Dv[o / CW_NB][o % CW_NB];
+      for (int o = tid; o < CW_NB * CW_NB; o += CW_THREADS) dinv_out[(int64_t)(j0 / CW_NB) * CW_NB * CW_NB + o] = Dv[o / CW_NB][o % CW_NB];
   }
-  if (tid == 0 && well_conditioned != nullptr) *well_conditioned = (dmin > 1e-8 * gmax_s) ? 1 : 0;
+  if (warp == 0 && well_conditioned != nullptr) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_xor_sync(0xFFFFFFFFu, dmin, o));
+    if (lane == 0) *well_conditioned = (dmin > 1e-8 * gmax) ? 1 : 0;
+  }
+}
+
+// The same outputs for n <= CM_MAX, whose factor fits one SM's shared memory: the eight-column panels of cta_cholesky (a
+// panel costs 2.4k cycles whatever n is; n = 136: 45 us against 104 us of the 32-column panels), then the inverses of the
+// diagonal blocks, one warp each.
+constexpr int CM_MAX = 160, CM_P = CM_MAX + 4;
+__host__ __device__ constexpr size_t cm_smem(int n) { return sizeof(double) * (size_t)((n + 7) / 8 * 8) * CM_P; }
+__global__ void __launch_bounds__(CW_THREADS, 1)
+chol_mid_kernel(const double* __restrict__ g, int n, double tol_rel, double* __restrict__ l_out, double* dinv_out, int* perm_out, EigState* state,
+                const int* __restrict__ skip, int* __restrict__ well_conditioned) {
+  metis_pdl_wait();
+  if (skip != nullptr && *skip) return;
+  extern __shared__ __align__(16) unsigned char cm_sm[];
+  double* Y = reinterpret_cast<double*>(cm_sm);
+  __shared__ double diag[CM_MAX], inv_s[CM_MAX];
+  __shared__ int perm[CM_MAX];
+  __shared__ double gmax_s, dmin_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, n8 = (n + 7) & ~7;
+  if (state != nullptr) eig_state_reset(state, tid);
+  for (int i = tid; i < n; i += CW_THREADS) { diag[i] = g[(int64_t)i * n + i]; perm[i] = i; }
+  if (tid == 0) gmax_s = 0.0;
+  __syncthreads();
+  for (int i = tid >> 1; i < n; i += CW_THREADS / 2) {     // two lanes per entry
+    const double d = diag[i];
+    int rank = 0;
+#pragma unroll 8
+    for (int j = tid & 1; j < n; j += 2) rank += (diag[j] > d) || (diag[j] == d && j < i);
+    rank += __shfl_xor_sync(__activemask(), rank, 1);
+    if ((tid & 1) == 0) {
+      if (rank == 0) gmax_s = d;
+      if (perm_out != nullptr) perm[rank] = i;             // NaNs may collide; every entry stays a valid index
+    }
+  }
+  __syncthreads();
+  if (perm_out != nullptr)
+    for (int i = tid; i < n; i += CW_THREADS) perm_out[i] = perm[i];
+#pragma unroll 4
+  for (int i = warp; i < n8; i += CW_WARPS) {              // rows of the sorted matrix (symmetric to the bit)
+    double v[CM_MAX / 32];
+#pragma unroll
+    for (int t = 0; t < CM_MAX / 32; ++t) { const int c = lane + 32 * t; v[t] = i < n && c < n ? g[(int64_t)perm[i] * n + perm[c]] : 0.0; }
+#pragma unroll
+    for (int t = 0; t < CM_MAX / 32; ++t) { const int c = lane + 32 * t; if (c < n8) Y[i * CM_P + c] = v[t]; }
+  }
+  const double gmax = gmax_s;
+  __syncthreads();
+  metis_small::cta_cholesky<CM_P>(Y, n, tol_rel * gmax, inv_s, &dmin_s, CW_THREADS);
+  for (int i = warp; i < n; i += CW_WARPS)
+    for (int c = lane; c < n; c += 32) l_out[(int64_t)i * n + c] = c <= i ? Y[i * CM_P + c] : 0.0;
+  if (tid == 0 && well_conditioned != nullptr) *well_conditioned = (dmin_s > 1e-8 * gmax) ? 1 : 0;
+  if (dinv_out != nullptr && warp < (n + CW_NB - 1) / CW_NB) {
+    // X = L^-1 of a diagonal block, lane = column:  X[i][j] = -r_i sum_{k < i} L[i][k] X[k][j],  X[j][j] = r_j
+    const int j0 = warp * CW_NB;
+    double x[CW_NB];
+#pragma unroll
+    for (int i = 0; i < CW_NB; ++i) {
+      double s0 = 0.0, s1 = 0.0;
+      const bool in = j0 + i < n;
+      const double* row = Y + (in ? j0 + i : j0) * CM_P + j0;
+#pragma unroll
+      for (int k = 0; k < i; ++k) { if (k & 1) s1 = fma(row[k], x[k], s1); else s0 = fma(row[k], x[k], s0); }
+      const double ri = in ? inv_s[j0 + i] : 0.0;
+      x[i] = i == lane ? ri : (i > lane ? -ri * (s0 + s1) : 0.0);
+      dinv_out[(int64_t)warp * CW_NB * CW_NB + i * CW_NB + lane] = x[i];
+    }
+  }
 }
 
 // H = Z L^-T by blocked forward substitution, in place: for panel J of CW_NB columns
@@ -281,8 +399,8 @@ trsm_wide_kernel(float* __restrict__ z, int64_t n_rows, int n, const double* __r
 
 // ------------------------------------------------------------------------------------------------
 // C[m][n] = scale[n] * sum_k A[m * a_m + k * a_k] * B[k * b_k + n * b_n]      (A FP32, B FP64, FP64 accumulation)
-// written as FP32 to c[m * c_m + n * c_n]; optionally also c2[m * c2_m + n * c2_n] = (that value) * scale2[n], and
-// amax|C| into *amax (bits of a non-negative float, atomic max).  64 x 64 tile per CTA, 4 x 4 outputs per thread.
+// (on the FP64 tensor cores) written as FP32 to c[m * c_m + n * c_n]; optionally also c2[m * c2_m + n * c2_n] = (that value) * scale2[n], and
+// amax|C| into *amax (bits of a non-negative float, atomic max).  64 x 64 tile per CTA, 16 x 32 per warp.
 struct Gemm64Args {
   const float* a; int64_t a_m, a_k;
   const double* b; int64_t b_k, b_n;
@@ -297,17 +415,14 @@ __global__ void __launch_bounds__(256)
 gemm64_kernel(Gemm64Args g) {
   metis_pdl_wait();
   if (g.skip != nullptr && *g.skip) return;
-  constexpr int T = 64, KT = 16;
-  __shared__ __align__(16) double as[KT][T + 2], bs[KT][T + 2];
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+  constexpr int T = G64_T, KT = G64_R;
+  __shared__ double as[KT][G64_P], bs[KT][G64_P];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gq = lane >> 2, q = lane & 3, wm = 16 * (warp & 3), wn = 32 * (warp >> 2);
   const int64_t m0 = (int64_t)blockIdx.y * T;
   const int n0 = blockIdx.x * T;
-  double acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
+  double acc[2][4][2] = {};
   for (int k0 = 0; k0 < g.K; k0 += KT) {
+#pragma unroll
     for (int o = tid; o < KT * T; o += 256) {
       int kk, mm;
       if (g.a_k == 1) { kk = o % KT; mm = o / KT; } else { mm = o % T; kk = o / T; }
@@ -317,32 +432,25 @@ gemm64_kernel(Gemm64Args g) {
       bs[kb][nn] = (n0 + nn < g.N && k0 + kb < g.K) ? g.b[(int64_t)(k0 + kb) * g.b_k + (int64_t)(n0 + nn) * g.b_n] : 0.0;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < KT; ++kk) {
-      double av[4], bv[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) { av[a] = as[kk][ty + 16 * a]; bv[a] = bs[kk][tx + 16 * a]; }
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] += av[a] * bv[b];
-    }
+    tile64_mac(as, bs, wm, wn, gq, q, acc);
     __syncthreads();
   }
   float am = 0.0f;
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      const int64_t m = m0 + ty + 16 * a;
-      const int n = n0 + tx + 16 * b;
-      if (m < g.M && n < g.N) {
-        const float v = (float)(g.scale != nullptr ? acc[a][b] * g.scale[n] : acc[a][b]);
-        g.c[m * g.c_m + (int64_t)n * g.c_n] = v;
-        if (g.c2 != nullptr) g.c2[m * g.c2_m + (int64_t)n * g.c2_n] = v * g.scale2[n];
-        am = fmaxf(am, fabsf(v));
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int64_t m = m0 + wm + 8 * a + gq;
+        const int n = n0 + wn + 8 * b + 2 * q + e;
+        if (m < g.M && n < g.N) {
+          const float v = (float)(g.scale != nullptr ? acc[a][b][e] * g.scale[n] : acc[a][b][e]);
+          g.c[m * g.c_m + (int64_t)n * g.c_n] = v;
+          if (g.c2 != nullptr) g.c2[m * g.c2_m + (int64_t)n * g.c2_n] = v * g.scale2[n];
+          am = fmaxf(am, fabsf(v));
+        }
       }
-    }
   if (g.amax != nullptr) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) am = fmaxf(am, __shfl_xor_sync(0xFFFFFFFFu, am, o));
@@ -368,6 +476,311 @@ __global__ void rot_scales_kernel(const double* __restrict__ evals, const float*
 }
 
 // ------------------------------------------------------------------------------------------------
+// Symmetric eigen-decomposition of a Gram matrix of n up to MAXQ_WIDE, in the steps of the one-CTA solver (small_eig.cuh):
+// sorted Cholesky factor, FP32 block Jacobi, FP64 refinement with matrix products over many CTAs; a matrix the refinement cannot
+// finish (pairs of eigenvalues too close, or no convergence) is done by the FP64 Jacobi kernels, which otherwise return at
+// once.  The decisions are made on the device, in EigState, so that a call needs no host synchronisation.
+// Measured inside a layer step, n = 136: factorisation, solver and collection 138 + 1590 + 21 us before (FP64 sweeps on the cluster), now
+// 45 + 338 + 60 us.
+constexpr int ER_STEPS = 3;                               // refinement steps (two are enough unless eigenvalues are close)
+struct EigState {
+  unsigned int emax[ER_STEPS];                            // largest |E_ij| of a step (bits)
+  float norm2[ER_STEPS];                                  // squared norm of E
+  int open[ER_STEPS];                                     // some pair could not be separated
+};
+__device__ __forceinline__ void eig_state_reset(EigState* st, int tid) {
+  if (tid < ER_STEPS) { st->emax[tid] = 0u; st->norm2[tid] = 0.0f; st->open[tid] = 0; }
+}
+enum { EIG_RUNNING = 0, EIG_DONE = 1, EIG_FAILED = 2 };
+__device__ __forceinline__ bool eig_step_bad(const EigState* st, int t) { return __ldcg(&st->open[t]) != 0 || !(__ldcg(&st->norm2[t]) < 0.0625f); }
+// what the steps before `step` have come to; *last: the last step that was applied
+__device__ __forceinline__ int eig_status(const EigState* st, int step, int* last) {
+  *last = -1;
+  for (int t = 0; t < step; ++t) {
+    if (eig_step_bad(st, t)) return EIG_FAILED;
+    *last = t;
+    if (__uint_as_float(__ldcg(&st->emax[t])) < 2e-7f) return EIG_DONE;
+  }
+  return EIG_RUNNING;
+}
+
+// round-robin tournament of np players: couple I of round `step`
+__device__ __forceinline__ void jc_pair(int I, int step, int np, int* p, int* q) {
+  int a, b;
+  if (I == 0) { a = 0; b = (step % (np - 1)) + 1; }
+  else { a = ((step + I) % (np - 1)) + 1; b = ((step + np - 1 - I) % (np - 1)) + 1; }
+  *p = min(a, b); *q = max(a, b);
+}
+
+// FP32 one-sided block Jacobi on one cluster: 48 columns per CTA - two slots of twelve blocks of two columns, eight lanes per
+// block (sixteen above n = 176, where eight lanes' rows no longer fit their registers), so that the three warps sit on three schedulers (a warp per block: 1220 cycles a round at n = 136, the nine warps
+// sharing four schedulers, against 900) - and as many CTAs as the matrix needs.  Outer rounds are those of jacobi_cluster_kernel
+// below: first every pair among a CTA's own columns, then every block of one slot (kept in registers) against every block of the other,
+// the slots moving on to the neighbouring CTAs in the order of a round-robin tournament.  Ends with the
+// normalised columns in x (n x n, FP64).
+constexpr int JF_MB = 12, JF_COLS = 4 * JF_MB, JF_SWEEPS = 16;
+constexpr float JF_EXIT_COS2 = 1e-8f;                     // the rank cut may fall among close eigenvalues: a tighter exit than the small solver's
+__host__ __device__ constexpr size_t jf_smem(int lanes, int r) { return sizeof(float2) * 2 * 2 * JF_MB * lanes * (size_t)r; }
+template <int LANES, int R>                               // lanes per block; rows per lane, even: at least n / LANES
+__global__ void __launch_bounds__(LANES * JF_MB, 1)
+jacobi_fp32_kernel(const double* __restrict__ l, int n, double* __restrict__ x) {
+  constexpr int ROWS = LANES * R, JF_THREADS = LANES * JF_MB;
+  extern __shared__ __align__(16) unsigned char jf_sm[];
+  float2* blocks = reinterpret_cast<float2*>(jf_sm);      // [buffer][slot][block][row]
+  __shared__ float2 nrm[2 * JF_MB];
+  __shared__ int flag_s;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank(), P = (int)cluster.num_blocks();
+  const int tid = threadIdx.x, m = tid / LANES, sub = tid % LANES;             // group (block) and lane in it
+  auto blk = [&](int buf, int sb) { return blocks + ((size_t)buf * 2 * JF_MB + sb) * ROWS; };     // sb: slot * JF_MB + block
+  // odd groups walk the chunks of LANES rows in the order 1, 0, 3, 2, ...: the two groups of a half warp use different banks
+  auto row_of = [&](int t) { return sub + LANES * (t ^ (m & 1)); };
+  // FP32 copy, scaled to a largest entry near one (the factor's first pivot is its largest)
+  int ex = 0;
+  { const double l00 = l[0]; if (l00 > 0.0 && l00 < 1e150) (void)frexp(l00, &ex); }
+  const double scale = ldexp(1.0, -ex);
+#pragma unroll 4
+  for (int o = tid; o < 2 * JF_MB * ROWS; o += JF_THREADS) {
+    const int sb = o % (2 * JF_MB), i = o / (2 * JF_MB), c = rank * JF_COLS + 2 * sb;
+    float2 y = make_float2(0.0f, 0.0f);
+    if (i < n) {
+      if (c < n && c <= i) y.x = (float)(l[(int64_t)i * n + c] * scale);
+      if (c + 1 < n && c + 1 <= i) y.y = (float)(l[(int64_t)i * n + c + 1] * scale);
+    }
+    blk(0, sb)[i] = y;
+  }
+  __syncthreads();
+  int cur = 0;
+  for (int sweep = 0; sweep < JF_SWEEPS; ++sweep) {
+    bool above = false;
+    int any_above = 0;
+    for (int orr = 0; orr < 2 * P - 1; ++orr) {
+      // exact norms at the start of every outer round (carried through its rounds)
+#pragma unroll
+      for (int s = 0; s < 2; ++s) {
+        const float2* y = blk(cur, s * JF_MB + m);
+        float2 sq = make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int t = 0; t < R; ++t) { const float2 v = y[row_of(t)]; sq = metis_small::fma2(v, v, sq); }
+#pragma unroll
+        for (int o = LANES / 2; o > 0; o >>= 1) { sq.x += __shfl_xor_sync(0xFFFFFFFFu, sq.x, o); sq.y += __shfl_xor_sync(0xFFFFFFFFu, sq.y, o); }
+        if (sub == 0) nrm[s * JF_MB + m] = sq;
+      }
+      __syncthreads();
+      float2 a[R], b[R];
+      if (orr == 0) {
+        // every pair among the CTA's own columns: tournament of its 2 * JF_MB blocks
+        for (int r = 0; r < 2 * JF_MB - 1; ++r) {
+          int p, q;
+          jc_pair(m, r, 2 * JF_MB, &p, &q);
+          float2 *yp = blk(cur, p), *yq = blk(cur, q);
+#pragma unroll
+          for (int t = 0; t < R; ++t) { a[t] = yp[row_of(t)]; b[t] = yq[row_of(t)]; }
+          float2 n01 = nrm[p], n23 = nrm[q];
+          metis_small::block_rotate<R, LANES>(a, b, n01, n23, r == 0, JF_EXIT_COS2, above);
+#pragma unroll
+          for (int t = 0; t < R; ++t) { yp[row_of(t)] = a[t]; yq[row_of(t)] = b[t]; }
+          __syncwarp();
+          if (sub == 0) { nrm[p] = n01; nrm[q] = n23; }
+          __syncthreads();
+        }
+      } else {
+        // group m keeps block m of the first slot in registers and meets the blocks of the second slot one after the other
+        float2* yp = blk(cur, m);
+#pragma unroll
+        for (int t = 0; t < R; ++t) a[t] = yp[row_of(t)];
+        float2 n01 = nrm[m];
+        int q = JF_MB + m;
+        for (int r = 0; r < JF_MB; ++r) {
+          float2* yq = blk(cur, q);
+#pragma unroll
+          for (int t = 0; t < R; ++t) b[t] = yq[row_of(t)];
+          float2 n23 = nrm[q];
+          metis_small::block_rotate<R, LANES>(a, b, n01, n23, false, JF_EXIT_COS2, above);
+#pragma unroll
+          for (int t = 0; t < R; ++t) yq[row_of(t)] = b[t];
+          __syncwarp();
+          if (sub == 0) nrm[q] = n23;
+          q = q + 1 == 2 * JF_MB ? JF_MB : q + 1;
+          __syncthreads();
+        }
+#pragma unroll
+        for (int t = 0; t < R; ++t) yp[row_of(t)] = a[t];
+        __syncthreads();
+      }
+      const bool last = orr == 2 * P - 2;
+      if (last) {
+        const int any = __syncthreads_or(above ? 1 : 0);
+        if (tid == 0) flag_s = any;
+      }
+      cluster.sync();                                      // every CTA is done with this outer round (flags are written)
+      // hand the slots on: slot 0 ("top") of CTA c goes to the top of c + 1 (the last CTA's top becomes its own
+      // bottom, CTA 0's top stays); slot 1 ("bottom") of CTA c goes to the bottom of c - 1 (CTA 0's bottom becomes
+      // the top of CTA 1)
+      {
+        int dst_rank[2], dst_slot[2];
+        if (rank == 0) { dst_rank[0] = 0; dst_slot[0] = 0; dst_rank[1] = 1; dst_slot[1] = 0; }
+        else {
+          if (rank == P - 1) { dst_rank[0] = rank; dst_slot[0] = 1; } else { dst_rank[0] = rank + 1; dst_slot[0] = 0; }
+          dst_rank[1] = rank - 1; dst_slot[1] = 1;
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const float4* src = reinterpret_cast<const float4*>(blk(cur, s * JF_MB));
+          float4* dst = reinterpret_cast<float4*>(cluster.map_shared_rank(blk(cur ^ 1, dst_slot[s] * JF_MB), dst_rank[s]));
+#pragma unroll 8
+          for (int o = tid; o < JF_MB * ROWS / 2; o += JF_THREADS) dst[o] = src[o];
+        }
+      }
+      if (last) {
+        for (int c = 0; c < P; ++c) any_above |= *cluster.map_shared_rank(&flag_s, c);
+      }
+      cluster.sync();                                      // the slots have landed; the flags have been read
+      cur ^= 1;
+    }
+    if (!any_above) break;
+  }
+  // after whole sweeps every slot is back where it started; normalised columns, zero columns stay zero
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const float2* y = blk(cur, s * JF_MB + m);
+    double sx = 0.0, sy = 0.0;
+#pragma unroll
+    for (int t = 0; t < R; ++t) { const float2 v = y[row_of(t)]; sx = fma((double)v.x, (double)v.x, sx); sy = fma((double)v.y, (double)v.y, sy); }
+#pragma unroll
+    for (int o = LANES / 2; o > 0; o >>= 1) { sx += __shfl_xor_sync(0xFFFFFFFFu, sx, o); sy += __shfl_xor_sync(0xFFFFFFFFu, sy, o); }
+    const double rx = sx > 0.0 ? metis_small::rsqrt64(sx) : 0.0, ry = sy > 0.0 ? metis_small::rsqrt64(sy) : 0.0;
+    const int c = rank * JF_COLS + 2 * (s * JF_MB + m);
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      const int i = row_of(t);
+      const float2 v = y[i];
+      if (i < n && c < n) x[(int64_t)i * n + c] = (double)v.x * rx;
+      if (i < n && c + 1 < n) x[(int64_t)i * n + c + 1] = (double)v.y * ry;
+    }
+  }
+}
+
+// One product of a refinement step, 32 x 32 of the result per CTA (four warps of 16 x 16):
+//   OP 0  W = L^T X      OP 1  S = W^T W (blockIdx.z = 0) and X^T X (blockIdx.z = 1)      OP 2  X' = X + X E
+// Operands straight from L2 into fragment registers: n is at most 272 and each element is wanted by n / 32 CTAs.
+template <int OP>
+__global__ void __launch_bounds__(128)
+refine_product_kernel(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ c, const double* __restrict__ a1,
+                      double* __restrict__ c1, int n, const EigState* __restrict__ st, int step) {
+  metis_pdl_wait();
+  int last;
+  if (eig_status(st, step, &last) != EIG_RUNNING) return;
+  if (OP == 2 && eig_step_bad(st, step)) return;
+  if (OP == 1 && blockIdx.z == 1) { a = a1; b = a1; c = c1; }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3;
+  const int i0 = 32 * blockIdx.y + 16 * (warp & 1), j0 = 32 * blockIdx.x + 16 * (warp >> 1);
+  double acc[2][2][2] = {};
+  const bool in_i[2] = {i0 + g < n, i0 + 8 + g < n}, in_j[2] = {j0 + g < n, j0 + 8 + g < n};
+  constexpr int U = 8;                                    // steps of four whose loads are in flight together
+  for (int k0 = OP == 0 ? i0 / (4 * U) * (4 * U) : 0; k0 < n; k0 += 4 * U) {   // (L is lower triangular)
+    double fa[U][2], fb[U][2];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k = k0 + 4 * u + q;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        fa[u][h] = k < n && in_i[h] ? __ldcg(OP == 2 ? a + (int64_t)(i0 + 8 * h + g) * n + k : a + (int64_t)k * n + i0 + 8 * h + g) : 0.0;
+        fb[u][h] = k < n && in_j[h] ? __ldcg(b + (int64_t)k * n + j0 + 8 * h + g) : 0.0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int v = 0; v < 2; ++v) metis_small::dmma(acc[h][v], fa[u][h], fb[u][v]);
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int v = 0; v < 2; ++v)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int i = i0 + 8 * h + g, j = j0 + 8 * v + 2 * q + e;
+        if (i < n && j < n) c[(int64_t)i * n + j] = acc[h][v][e] + (OP == 2 ? a[(int64_t)i * n + j] : 0.0);
+      }
+}
+
+// E of a step from S and G1 = X^T X, and what the status is made of
+__global__ void __launch_bounds__(256)
+refine_correction_kernel(const double* __restrict__ s, const double* __restrict__ g1, double* __restrict__ e_out, int n, EigState* __restrict__ st, int step) {
+  metis_pdl_wait();
+  int last;
+  if (eig_status(st, step, &last) != EIG_RUNNING) return;
+  const int o = blockIdx.x * 256 + threadIdx.x;
+  float em = 0.0f, en = 0.0f;
+  bool open = false;
+  if (o < n * n) {
+    const int i = o / n, j = o % n;
+    const double gi = g1[(int64_t)i * n + i], gj = g1[(int64_t)j * n + j];
+    double e = 0.0;
+    if (gi != 0.0 && gj != 0.0) {                         // zero columns stay
+      const double r = (i == j ? 1.0 : 0.0) - g1[o];
+      e = 0.5 * r;
+      if (i != j) {
+        const double sv = s[o], li = s[(int64_t)i * n + i] / gi, lj = s[(int64_t)j * n + j] / gj;
+        if (sv * sv > 1e-28 * fabs(li * lj)) {            // orthogonal to FP64 rounding otherwise
+          const double gap = lj - li, a = sv + lj * r, b = sv + li * r;
+          if (fabs(a) < 0.0625 * fabs(gap) && fabs(b) < 0.0625 * fabs(gap)) e = a / gap;
+          else if (sv * sv > 1e-24 * fabs(li * lj)) open = true;
+        }
+      }
+    }
+    e_out[o] = e;
+    em = fabsf((float)e);
+    en = em * em;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) { em = fmaxf(em, __shfl_xor_sync(0xFFFFFFFFu, em, d)); en += __shfl_xor_sync(0xFFFFFFFFu, en, d); }
+  const bool any = __any_sync(0xFFFFFFFFu, open);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&st->emax[step], __float_as_uint(em));
+    atomicAdd(&st->norm2[step], en);                      // only compared with a bound
+    if (any) st->open[step] = 1;
+  }
+}
+
+// eigenvalues descending (squared lengths of the last step's S), eigenvectors in the input's row order
+__global__ void __launch_bounds__(1024, 1)
+eigen_finish_kernel(const double* __restrict__ x0, const double* __restrict__ x1, const double* __restrict__ s, const double* __restrict__ g1,
+                    const int* __restrict__ perm, int n, const EigState* __restrict__ st, double* __restrict__ evals, double* __restrict__ evecs,
+                    int* __restrict__ failed) {
+  metis_pdl_wait();
+  __shared__ double lam[MAXQ_WIDE];
+  __shared__ int order[MAXQ_WIDE];
+  int last;
+  const bool done = eig_status(st, ER_STEPS, &last) == EIG_DONE;
+  const int tid = threadIdx.x;
+  if (tid == 0) *failed = done ? 0 : 1;
+  if (!done) return;
+  const double* x = last & 1 ? x0 : x1;                   // step t reads one buffer and writes the other
+  if (tid < n) {
+    const double gi = g1[(int64_t)tid * n + tid];
+    lam[tid] = gi > 0.0 ? s[(int64_t)tid * n + tid] / gi : 0.0;
+    order[tid] = tid;
+  }
+  __syncthreads();
+  if (tid < n) {
+    const double li = lam[tid];
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += (lam[j] > li) || (lam[j] == li && j < tid);
+    order[rank] = tid;                                    // stays a valid index if NaNs make ranks collide
+  }
+  __syncthreads();
+  if (tid < n) evals[tid] = lam[order[tid]];
+  for (int o = tid; o < n * n; o += 1024) {
+    const int i = o / n, t = o % n;
+    evecs[(int64_t)perm[i] * n + t] = x[(int64_t)i * n + order[t]];
+  }
+}
+
+// ------------------------------------------------------------------------------------------------
 // One-sided (Hestenes) Jacobi on the columns of Y = L (the Cholesky factor of the Gram matrix, so that
 // G = Y Y^T and the rotated columns end as U Sigma), for n up to MAXQ_WIDE, on ONE CLUSTER of JC_P CTAs.
 // The 2 * JC_P * JC_W column slots are dealt out as 2 * JC_P blocks of JC_W columns; every CTA holds two blocks in
@@ -381,13 +794,6 @@ __global__ void rot_scales_kernel(const double* __restrict__ evals, const float*
 constexpr int JC_P = 8, JC_W = 17, JC_ROWS = 288, JC_THREADS = 32 * JC_W;
 constexpr int JC_RL = JC_ROWS / 32;                     // rows per lane
 constexpr size_t JC_SMEM = sizeof(double) * 2 * 2 * JC_W * JC_ROWS;
-
-__device__ __forceinline__ void jc_pair(int I, int step, int np, int* p, int* q) {
-  int a, b;
-  if (I == 0) { a = 0; b = (step % (np - 1)) + 1; }
-  else { a = ((step + I) % (np - 1)) + 1; b = ((step + np - 1 - I) % (np - 1)) + 1; }
-  *p = min(a, b); *q = max(a, b);
-}
 
 // Rotation that makes two columns with squared norms a, b and inner product c orthogonal: the smaller root of
 // tan(2 theta) = 2c / (b - a), |theta| <= pi / 4.  The FP32 quantities only steer convergence (fast reciprocal square
@@ -406,8 +812,8 @@ __device__ __forceinline__ void jc_rotation(float a, float b, float cf, double& 
 }
 
 __global__ void __cluster_dims__(JC_P, 1, 1) __launch_bounds__(JC_THREADS, 1)
-jacobi_cluster_kernel(const double* __restrict__ l, int n, float exit_cos2, double* __restrict__ ycm) {
-  metis_pdl_wait();
+jacobi_cluster_kernel(const double* __restrict__ l, int n, float exit_cos2, const int* __restrict__ wanted, double* __restrict__ ycm) {
+  if (!*wanted) return;                                   // the same for every CTA of the cluster
   extern __shared__ __align__(16) unsigned char jsm[];
   double* cols = reinterpret_cast<double*>(jsm);        // [buffer][slot][column][row]
   __shared__ float nrm[2][JC_W];
@@ -547,8 +953,9 @@ jacobi_cluster_kernel(const double* __restrict__ l, int n, float exit_cos2, doub
 
 // eigenvalues = squared column norms (descending), eigenvectors = normalised columns: evecs[i * n + t]
 __global__ void __launch_bounds__(1024, 1)
-jacobi_collect_kernel(const double* __restrict__ ycm, int n, double* __restrict__ evals, double* __restrict__ evecs) {
-  metis_pdl_wait();
+jacobi_collect_kernel(const double* __restrict__ ycm, int n, const int* __restrict__ perm, const int* __restrict__ wanted, double* __restrict__ evals,
+                      double* __restrict__ evecs) {
+  if (!*wanted) return;
   constexpr int NC = 2 * JC_P * JC_W;
   __shared__ double lam[NC];
   __shared__ int order[NC];
@@ -573,7 +980,7 @@ jacobi_collect_kernel(const double* __restrict__ ycm, int n, double* __restrict_
     const int i = o / n, t = o % n;
     const int c = order[t];
     const double l2 = lam[c];
-    evecs[o] = l2 > 0.0 ? ycm[(int64_t)c * n + i] * (1.0 / sqrt(l2)) : 0.0;
+    evecs[(int64_t)perm[i] * n + t] = l2 > 0.0 ? ycm[(int64_t)c * n + i] * (1.0 / sqrt(l2)) : 0.0;
   }
 }
 

@@ -35,74 +35,86 @@ __device__ __forceinline__ void dmma(double (&d)[2], double a, double b) {
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};" : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
 }
 
-// In-place Cholesky factorisation of the lower triangle of Y (n x n, row pitch P doubles; rows and columns up to the next
-// multiple of eight must exist and be zero), called by all nthr threads of the CTA.  Panels of eight columns: warp 0
-// factorises a panel in registers - lane l holds rows l, l + 32, l + 64 below the panel's top, a column step is one pivot
-// broadcast, one reciprocal and one multiply-add deep, without a barrier - and all warps subtract the panel's rank-8 product
-// from the trailing tiles on the FP64 tensor cores.  (One barrier per column with the matrix spread over 256 threads' registers
-// took 800 cycles a column; see the measured figures at the eigen-solver.)  A pivot not above `tol` marks a dependent column:
+// (row, column) of lower tile o, counted row by row
+__device__ __forceinline__ void lower_tile(int o, int& ti, int& tj) {
+  ti = (int)(0.5f * (sqrtf(8.0f * (float)o + 1.0f) - 1.0f));
+  tj = o - ti * (ti + 1) / 2;
+}
+
+// In-place Cholesky factorisation of the lower triangle of Y (n x n, n8 = n rounded up to a multiple of eight, row pitch P doubles,
+// rows and columns up to n8 must exist and be zero beyond n), called by all nthr threads of the CTA, 32 nthr / 32 >= n8 - 8.
+// Panels of eight columns: every warp factorises the panel's diagonal block in registers (lane = row; a column step is one
+// pivot broadcast, one reciprocal and one multiply-add deep, without a barrier) and carries 32 rows below it along; then all warps subtract
+// the panel's rank-8 product from the trailing tiles on the FP64 tensor cores, two tiles at a time.  (One barrier per
+// column with the matrix spread over 256 threads' registers took 800 cycles a column.)  A pivot not above `tol` marks a dependent column:
 // it takes no part in the updates and ends as a zero column with inv_out[j] = 0; otherwise inv_out[j] = 1 / L[j][j].
 // *dmin_out (optional): the smallest accepted pivot.
 template <int P>
 __device__ __forceinline__ void cta_cholesky(double* Y, int n, double tol, double* inv_out, double* dmin_out, int nthr) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = nthr >> 5;
-  const int n8 = (n + 7) & ~7;
+  const int n8 = (n + 7) & ~7, g = lane >> 2, q = lane & 3;
   double dmin = 1e300;
   for (int c0 = 0; c0 < n8; c0 += 8) {
-    if (warp == 0) {
-      double v[3][8];
+    const int r = c0 + 8 + 32 * warp + lane, rd_ = c0 + (lane & 7);             // a row below the block, a row of the block
+    double vd[8], inv = 0.0;
+    const bool busy = warp == 0 || c0 + 8 + 32 * warp < n8;
+    if (busy) {
+      double v[8];
 #pragma unroll
-      for (int t = 0; t < 3; ++t) {
-        const int r = c0 + lane + 32 * t;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) v[t][c] = r < n8 ? Y[r * P + c0 + c] : 0.0;
-      }
+      for (int c = 0; c < 8; ++c) { vd[c] = Y[rd_ * P + c0 + c]; v[c] = r < n8 ? Y[r * P + c0 + c] : 0.0; }
       double my_pivot = 0.0;                            // lane j < 8: pivot of column c0 + j
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const double d = __shfl_sync(0xFFFFFFFFu, v[0][j], j);
-        const bool ok = d > tol;
-        const double rd = ok ? rcp64(d) : 0.0;
-        if (lane == j) my_pivot = d;
-        double u[8];
+        const double d = __shfl_sync(0xFFFFFFFFu, vd[j], j);
+        const double rd = d > tol ? rcp64(d) : 0.0;
+        if ((lane & 7) == j) my_pivot = d;
+        const double ld = vd[j] * rd, l = v[j] * rd;
 #pragma unroll
-        for (int c = j + 1; c < 8; ++c) u[c] = __shfl_sync(0xFFFFFFFFu, v[0][j], c);
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const double l = v[t][j] * rd;
-#pragma unroll
-          for (int c = j + 1; c < 8; ++c) v[t][c] = fma(-l, u[c], v[t][c]);
+        for (int c = j + 1; c < 8; ++c) {
+          const double u = __shfl_sync(0xFFFFFFFFu, vd[j], c);
+          vd[c] = fma(-ld, u, vd[c]);
+          v[c] = fma(-l, u, v[c]);
         }
       }
       const bool ok = my_pivot > tol;
-      const double inv = ok ? rsqrt64(my_pivot) : 0.0;
-      if (lane < 8 && c0 + lane < n) {
-        inv_out[c0 + lane] = inv;
-        if (ok) dmin = fmin(dmin, my_pivot);
-      }
+      inv = ok ? rsqrt64(my_pivot) : 0.0;
+      if (ok) dmin = fmin(dmin, my_pivot);
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const double ic = __shfl_sync(0xFFFFFFFFu, inv, c);
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-          const int r = c0 + lane + 32 * t;
-          if (r < n8) Y[r * P + c0 + c] = r >= c0 + c ? v[t][c] * ic : 0.0;
-        }
+        vd[c] *= ic;
+        if (r < n8) Y[r * P + c0 + c] = v[c] * ic;
       }
     }
-    __syncthreads();
-    // trailing tiles (ti >= tj > panel): Y -= L_panel L_panel^T
-    const int first = c0 / 8 + 1, nt = n8 / 8 - first, g = lane >> 2, q = lane & 3;
-    for (int o = warp; o < nt * (nt + 1) / 2; o += n_warps) {
-      int ti = 0;
-      while ((ti + 1) * (ti + 2) / 2 <= o) ++ti;
-      const int tj = o - ti * (ti + 1) / 2;
-      const int ri = 8 * (first + ti) + g, rj = 8 * (first + tj) + g;
-      double* out = Y + ri * P + 8 * (first + tj) + 2 * q;
-      double acc[2] = {out[0], out[1]};
+    __syncthreads();                                    // the block has been read by every warp: its factor may be stored
+    if (warp == 0 && lane < 8) {
+      if (c0 + lane < n) inv_out[c0 + lane] = inv;
 #pragma unroll
-      for (int kk = 0; kk < 8; kk += 4) dmma(acc, -Y[ri * P + c0 + kk + q], Y[rj * P + c0 + kk + q]);
-      out[0] = acc[0]; out[1] = acc[1];
+      for (int c = 0; c < 8; ++c) Y[rd_ * P + c0 + c] = c <= lane ? vd[c] : 0.0;
+    }
+    // trailing tiles (ti >= tj > panel): Y -= L_panel L_panel^T
+    const int first = c0 / 8 + 1, nt = n8 / 8 - first, tiles = nt * (nt + 1) / 2;
+    for (int o = warp; o < tiles; o += 2 * n_warps) {
+      double acc[2][2], a[2][2], b[2][2];
+      double* out[2];
+      const bool two = o + n_warps < tiles;
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        int ti, tj;
+        lower_tile(u == 0 || !two ? o : o + n_warps, ti, tj);
+        const int ri = 8 * (first + ti) + g, rj = 8 * (first + tj) + g;
+        out[u] = Y + ri * P + 8 * (first + tj) + 2 * q;
+        acc[u][0] = out[u][0]; acc[u][1] = out[u][1];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) { a[u][h] = -Y[ri * P + c0 + 4 * h + q]; b[u][h] = Y[rj * P + c0 + 4 * h + q]; }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int u = 0; u < 2; ++u) dmma(acc[u], a[u][h], b[u][h]);
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (u == 0 || two) { out[u][0] = acc[u][0]; out[u][1] = acc[u][1]; }
     }
     __syncthreads();
   }
@@ -180,6 +192,57 @@ __device__ __forceinline__ void jacobi_rot2(float2& a, float2& b, float2 g, floa
   const float2 tg = mul2(mul2(s, rs), g);   // tan(theta) g
   a = add2(a, neg2(tg));
   b = add2(b, tg);
+}
+
+// Makes the four columns of two blocks, a = (0, 1) and b = (2, 3), orthogonal between the blocks (and, with `within`, inside them
+// first): LANES lanes hold R rows each.  n01, n23: squared lengths, carried along.  The rotations are worked out on the 4 x 4 Gram
+// matrix: its six inner products are reduced together, and the second half round's follow from the first's by rotation.
+template <int R, int LANES>
+__device__ __forceinline__ void block_rotate(float2 (&a)[R], float2 (&b)[R], float2& n01, float2& n23, bool within, float exit_cos2, bool& above) {
+  float g01 = 0.0f, g23 = 0.0f, g03 = 0.0f, g12 = 0.0f;
+  float2 gx = make_float2(0.0f, 0.0f);                  // <0, 2>, <1, 3>
+#pragma unroll
+  for (int t = 0; t < R; ++t) {
+    gx = fma2(a[t], b[t], gx);
+    g03 = fmaf(a[t].x, b[t].y, g03); g12 = fmaf(a[t].y, b[t].x, g12);
+    g01 = fmaf(a[t].x, a[t].y, g01); g23 = fmaf(b[t].x, b[t].y, g23);
+  }
+#pragma unroll
+  for (int o = LANES / 2; o > 0; o >>= 1) {
+    gx.x += __shfl_xor_sync(0xFFFFFFFFu, gx.x, o); gx.y += __shfl_xor_sync(0xFFFFFFFFu, gx.y, o);
+    g01 += __shfl_xor_sync(0xFFFFFFFFu, g01, o); g23 += __shfl_xor_sync(0xFFFFFFFFu, g23, o);
+    g03 += __shfl_xor_sync(0xFFFFFFFFu, g03, o); g12 += __shfl_xor_sync(0xFFFFFFFFu, g12, o);
+  }
+  float2 c, s;
+  if (within) {
+    float2 na = make_float2(n01.x, n23.x), nb = make_float2(n01.y, n23.y);
+    jacobi_rot2(na, nb, make_float2(g01, g23), exit_cos2, c, s, above);
+    n01 = make_float2(na.x, nb.x); n23 = make_float2(na.y, nb.y);
+    const float c02 = c.x * gx.x - s.x * g12, c03 = c.x * g03 - s.x * gx.y, c12 = s.x * gx.x + c.x * g12, c13 = s.x * g03 + c.x * gx.y;
+    gx.x = c.y * c02 - s.y * c03; g03 = s.y * c02 + c.y * c03; g12 = c.y * c12 - s.y * c13; gx.y = s.y * c12 + c.y * c13;
+    g01 = 0.0f; g23 = 0.0f;
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+      a[t] = make_float2(c.x * a[t].x - s.x * a[t].y, s.x * a[t].x + c.x * a[t].y);
+      b[t] = make_float2(c.y * b[t].x - s.y * b[t].y, s.y * b[t].x + c.y * b[t].y);
+    }
+  }
+  jacobi_rot2(n01, n23, gx, exit_cos2, c, s, above);    // couples (0, 2) and (1, 3)
+  const float x01 = c.x * g01 - s.x * g12, x03 = c.x * g03 - s.x * g23;        // <0', 1>, <0', 3>
+  const float x21 = s.x * g01 + c.x * g12, x23 = s.x * g03 + c.x * g23;        // <2', 1>, <2', 3>
+  const float2 gy = make_float2(s.y * x01 + c.y * x03, c.y * x21 - s.y * x23); // <0', 3'>, <1', 2'>
+  float2 n32 = make_float2(n23.y, n23.x), c2, s2;
+  jacobi_rot2(n01, n32, gy, exit_cos2, c2, s2, above);  // couples (0, 3) and (1, 2)
+  n23 = make_float2(n32.y, n32.x);
+  const float2 ns = neg2(s), ns2 = neg2(s2);
+#pragma unroll
+  for (int t = 0; t < R; ++t) {
+    const float2 a1 = fma2(c, a[t], mul2(ns, b[t])), b1 = fma2(s, a[t], mul2(c, b[t]));
+    const float2 bs = make_float2(b1.y, b1.x);
+    a[t] = fma2(c2, a1, mul2(ns2, bs));
+    const float2 b2 = fma2(s2, a1, mul2(c2, bs));
+    b[t] = make_float2(b2.y, b2.x);
+  }
 }
 
 template <int NT8>                                      // n rounded up to a multiple of eight, over eight
@@ -307,53 +370,13 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
           float2 a[R], b[R];                              // columns (0, 1) and (2, 3)
 #pragma unroll
           for (int t = 0; t < R; ++t) { a[t] = yp[row_of(t)]; b[t] = yr[row_of(t)]; }
+          const int pn = pairs[step + 1][mc][0], rn = pairs[step + 1][mc][1];  // (the table has a row more than it fills)
           float2 n01 = nrm2[p], n23 = nrm2[r];
-          float g01 = 0.0f, g23 = 0.0f, g03 = 0.0f, g12 = 0.0f;
-          float2 gx = make_float2(0.0f, 0.0f);            // <0, 2>, <1, 3>
-#pragma unroll
-          for (int t = 0; t < R; ++t) {
-            gx = fma2(a[t], b[t], gx);
-            g03 = fmaf(a[t].x, b[t].y, g03); g12 = fmaf(a[t].y, b[t].x, g12);
-            g01 = fmaf(a[t].x, a[t].y, g01); g23 = fmaf(b[t].x, b[t].y, g23);
-          }
-#pragma unroll
-          for (int o = 4; o > 0; o >>= 1) {
-            gx.x += __shfl_xor_sync(0xFFFFFFFFu, gx.x, o); gx.y += __shfl_xor_sync(0xFFFFFFFFu, gx.y, o);
-            g01 += __shfl_xor_sync(0xFFFFFFFFu, g01, o); g23 += __shfl_xor_sync(0xFFFFFFFFu, g23, o);
-            g03 += __shfl_xor_sync(0xFFFFFFFFu, g03, o); g12 += __shfl_xor_sync(0xFFFFFFFFu, g12, o);
-          }
-          const int pn = pairs[step + 1][mc][0], rn = pairs[step + 1][mc][1];      // (the table has a row more than it fills)
-          float2 c, s;
-          if (step == 0) {                                // the couples inside the two blocks, once per sweep
-            float2 na = make_float2(n01.x, n23.x), nb = make_float2(n01.y, n23.y);
-            jacobi_rot2(na, nb, make_float2(g01, g23), exit_cos2, c, s, above);
-            n01 = make_float2(na.x, nb.x); n23 = make_float2(na.y, nb.y);
-            const float c02 = c.x * gx.x - s.x * g12, c03 = c.x * g03 - s.x * gx.y, c12 = s.x * gx.x + c.x * g12, c13 = s.x * g03 + c.x * gx.y;
-            gx.x = c.y * c02 - s.y * c03; g03 = s.y * c02 + c.y * c03; g12 = c.y * c12 - s.y * c13; gx.y = s.y * c12 + c.y * c13;
-            g01 = 0.0f; g23 = 0.0f;
-#pragma unroll
-            for (int t = 0; t < R; ++t) {
-              a[t] = make_float2(c.x * a[t].x - s.x * a[t].y, s.x * a[t].x + c.x * a[t].y);
-              b[t] = make_float2(c.y * b[t].x - s.y * b[t].y, s.y * b[t].x + c.y * b[t].y);
-            }
-          }
-          jacobi_rot2(n01, n23, gx, exit_cos2, c, s, above);     // couples (0, 2) and (1, 3)
-          const float x01 = c.x * g01 - s.x * g12, x03 = c.x * g03 - s.x * g23;    // <0', 1>, <0', 3>
-          const float x21 = s.x * g01 + c.x * g12, x23 = s.x * g03 + c.x * g23;    // <2', 1>, <2', 3>
-          const float2 gy = make_float2(s.y * x01 + c.y * x03, c.y * x21 - s.y * x23);            // <0', 3'>, <1', 2'>
-          float2 n32 = make_float2(n23.y, n23.x), c2, s2;
-          jacobi_rot2(n01, n32, gy, exit_cos2, c2, s2, above);   // couples (0, 3) and (1, 2)
-          const float2 ns = neg2(s), ns2 = neg2(s2);
+          block_rotate<R, 8>(a, b, n01, n23, step == 0, exit_cos2, above);
           if (active) {
 #pragma unroll
-            for (int t = 0; t < R; ++t) {
-              const float2 a1 = fma2(c, a[t], mul2(ns, b[t])), b1 = fma2(s, a[t], mul2(c, b[t]));
-              const float2 bs = make_float2(b1.y, b1.x);
-              yp[row_of(t)] = fma2(c2, a1, mul2(ns2, bs));
-              const float2 b2 = fma2(s2, a1, mul2(c2, bs));
-              yr[row_of(t)] = make_float2(b2.y, b2.x);
-            }
-            if (sub == 0) { nrm2[p] = n01; nrm2[r] = make_float2(n32.y, n32.x); }
+            for (int t = 0; t < R; ++t) { yp[row_of(t)] = a[t]; yr[row_of(t)] = b[t]; }
+            if (sub == 0) { nrm2[p] = n01; nrm2[r] = n23; }
           }
           p = pn; r = rn;
           bar();

@@ -1298,13 +1298,66 @@ metis_status_t launch_gram64(cudaStream_t s, const float* v, int64_t n_rows, int
   return METIS_OK;
 }
 
-// eigen-decomposition of the n x n Gram matrix gram1: Cholesky factor, cluster Jacobi on its columns, collection
-metis_status_t launch_eig_wide(cudaStream_t s, const double* gram1, int n, float exit_cos2, double* l, double* ycm, double* evals, double* evecs) {
-  METIS_CUDA_TRY(metis_launch_pdl(metis_wide::chol_wide_kernel, dim3(1), dim3(1024), metis_wide::CW_SMEM, s, gram1, n, 1e-14, l, (double*)nullptr, (const int*)nullptr,
-                                  (int*)nullptr)); METIS_COUNT_LAUNCH();
-  metis_wide::jacobi_cluster_kernel<<<metis_wide::JC_P, metis_wide::JC_THREADS, metis_wide::JC_SMEM, s>>>(l, n, exit_cos2, ycm); METIS_COUNT_LAUNCH();
+// Cholesky factor of an n x n Gram matrix: in one SM's shared memory where it fits, streamed through L2 above that
+metis_status_t launch_chol_wide(cudaStream_t s, const double* g, int n, double tol_rel, double* l, double* dinv, int* perm, metis_wide::EigState* st, const int* skip,
+                                int* well_conditioned) {
+  using namespace metis_wide;
+  if (n <= CM_MAX) METIS_CUDA_TRY(metis_launch_pdl(chol_mid_kernel, dim3(1), dim3(CW_THREADS), cm_smem(n), s, g, n, tol_rel, l, dinv, perm, st, skip, well_conditioned));
+  else METIS_CUDA_TRY(metis_launch_pdl(chol_wide_kernel, dim3(1), dim3(CW_THREADS), CW_SMEM, s, g, n, tol_rel, l, dinv, perm, st, skip, well_conditioned));
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+
+// eigen-decomposition of the n x n Gram matrix gram1 (see bigrank.cuh).  scratch: the Gram partials, free by then
+// (WIDE_GRAM_PARTS n x n matrices; six are used, and the state and the permutation sit in the seventh).
+template <int LANES, int R>
+metis_status_t launch_jacobi_fp32(cudaStream_t s, const double* l, int n, double* x) {
+  cudaLaunchConfig_t cfg = {};
+  const unsigned ctas = (unsigned)((n + metis_wide::JF_COLS - 1) / metis_wide::JF_COLS);
+  cfg.gridDim = dim3(ctas); cfg.blockDim = dim3(LANES * metis_wide::JF_MB); cfg.dynamicSmemBytes = metis_wide::jf_smem(LANES, R); cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  METIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, (metis_wide::jacobi_fp32_kernel<LANES, R>), l, n, x)); METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+
+metis_status_t launch_eig_wide(cudaStream_t s, const double* gram1, int n, double* scratch, double* l, double* ycm, double* evals, double* evecs) {
+  if (n <= MAXQ) return launch_eig(s, gram1, n, n, evals, evecs);               // a small rank with a large oversampling
+  using namespace metis_wide;
+  const size_t nn = (size_t)n * n;
+  double *x[2] = {scratch, scratch + nn}, *w = scratch + 2 * nn, *sm = scratch + 3 * nn, *g1 = scratch + 4 * nn, *e = scratch + 5 * nn;
+  EigState* st = reinterpret_cast<EigState*>(scratch + 6 * nn);
+  int* failed = reinterpret_cast<int*>(st + 1);
+  int* perm = failed + 1;
+  METIS_TRY(launch_chol_wide(s, gram1, n, 1e-14, l, nullptr, perm, st, nullptr, nullptr));
+  if (n <= 96) METIS_TRY((launch_jacobi_fp32<8, 12>(s, l, n, x[0])));
+  else if (n <= 112) METIS_TRY((launch_jacobi_fp32<8, 14>(s, l, n, x[0])));
+  else if (n <= 128) METIS_TRY((launch_jacobi_fp32<8, 16>(s, l, n, x[0])));
+  else if (n <= 144) METIS_TRY((launch_jacobi_fp32<8, 18>(s, l, n, x[0])));
+  else if (n <= 176) METIS_TRY((launch_jacobi_fp32<8, 22>(s, l, n, x[0])));
+  else if (n <= 192) METIS_TRY((launch_jacobi_fp32<16, 12>(s, l, n, x[0])));
+  else if (n <= 224) METIS_TRY((launch_jacobi_fp32<16, 14>(s, l, n, x[0])));
+  else if (n <= 256) METIS_TRY((launch_jacobi_fp32<16, 16>(s, l, n, x[0])));
+  else METIS_TRY((launch_jacobi_fp32<16, 18>(s, l, n, x[0])));
+  const unsigned t = (unsigned)((n + 31) / 32);
+  for (int step = 0; step < ER_STEPS; ++step) {
+    double *xc = x[step & 1], *xn = x[(step & 1) ^ 1];
+    METIS_CUDA_TRY(metis_launch_pdl((refine_product_kernel<0>), dim3(t, t), dim3(128), (size_t)0, s, (const double*)l, (const double*)xc, w, (const double*)nullptr,
+                                    (double*)nullptr, n, (const EigState*)st, step)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((refine_product_kernel<1>), dim3(t, t, 2), dim3(128), (size_t)0, s, (const double*)w, (const double*)w, sm, (const double*)xc, g1, n,
+                                    (const EigState*)st, step)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl(refine_correction_kernel, dim3((unsigned)((nn + 255) / 256)), dim3(256), (size_t)0, s, (const double*)sm, (const double*)g1, e, n, st,
+                                    step)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((refine_product_kernel<2>), dim3(t, t), dim3(128), (size_t)0, s, (const double*)xc, (const double*)e, xn, (const double*)nullptr,
+                                    (double*)nullptr, n, (const EigState*)st, step)); METIS_COUNT_LAUNCH();
+  }
+  METIS_CUDA_TRY(metis_launch_pdl(eigen_finish_kernel, dim3(1), dim3(1024), (size_t)0, s, (const double*)x[0], (const double*)x[1], (const double*)sm, (const double*)g1,
+                                  (const int*)perm, n, (const EigState*)st, evals, evecs, failed)); METIS_COUNT_LAUNCH();
+  jacobi_cluster_kernel<<<JC_P, JC_THREADS, JC_SMEM, s>>>(l, n, 1e-12f, failed, ycm); METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
-  metis_wide::jacobi_collect_kernel<<<1, 1024, 0, s>>>(ycm, n, evals, evecs); METIS_COUNT_LAUNCH();
+  jacobi_collect_kernel<<<1, 1024, 0, s>>>(ycm, n, perm, failed, evals, evecs); METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
   return METIS_OK;
 }
@@ -1375,8 +1428,7 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
     for (int pass = 0; pass < 2; ++pass) {
       const int* skip = pass ? cond_flag : nullptr;
       METIS_TRY(launch_gram64(s, src, n_r, q, q, 1, gram, gram1, skip));
-      METIS_CUDA_TRY(metis_launch_pdl(metis_wide::chol_wide_kernel, dim3(1), dim3(1024), metis_wide::CW_SMEM, s, (const double*)gram1, q, 1e-13, lf, linv, skip,
-                                      pass ? (int*)nullptr : cond_flag)); METIS_COUNT_LAUNCH();
+      METIS_TRY(launch_chol_wide(s, gram1, q, 1e-13, lf, linv, nullptr, nullptr, skip, pass ? nullptr : cond_flag));
       METIS_CUDA_TRY(metis_launch_pdl(metis_wide::trsm_wide_kernel, dim3((unsigned)metis_ceil_div(n_r, metis_wide::TW_ROWS)), dim3(256), metis_wide::TW_SMEM, s, src, n_r, q,
                                       (const double*)lf, (const double*)linv, skip)); METIS_COUNT_LAUNCH();
     }
@@ -1394,7 +1446,7 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
       METIS_CUDA_TRY(metis_launch_pdl((reduce_proj_kernel), rgrid, dim3(256), (size_t)(0), s, (const float*)mp, slices, cols, jp, qg, m + (int64_t)j0 * cols)); METIS_COUNT_LAUNCH();
     }
     METIS_TRY(launch_gram64(s, m, cols, q, 1, cols, gram, gram1));
-    METIS_TRY(launch_eig_wide(s, gram1, q, 1e-8f, lf, ycm, evals, evecs));
+    METIS_TRY(launch_eig_wide(s, gram1, q, gram, lf, ycm, evals, evecs));
   }
   // right basis: basis[j][col] = sum_i evecs[i][j] M[i][col] / sqrt(eval_j),  j < k
   float* rb = full ? out->right : basis;
@@ -1442,7 +1494,7 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
     METIS_TRY(metis_launch_residual_tc(ctx, x, nullptr, k, kp, qp, amax, t0, t1, residual_dense, a6, b6, s));
     // (7) Rayleigh-Ritz on C^T C, rotate both factors (side stream, beside the residual pass)
     METIS_TRY(launch_gram64(sf, coef, rows, k, kp, 1, gram, gram1));
-    METIS_TRY(launch_eig_wide(sf, gram1, k, 1e-6f, lf, ycm, evals2, evecs2));
+    METIS_TRY(launch_eig_wide(sf, gram1, k, gram, lf, ycm, evals2, evecs2));
     {
       Gemm64Args g{};
       g.a = basis; g.a_m = 1; g.a_k = cols; g.b = evecs2; g.b_k = k; g.b_n = 1; g.c = out->right; g.c_m = 1; g.c_n = cols; g.M = cols; g.N = k; g.K = k;
@@ -1489,6 +1541,11 @@ metis_status_t metis_split_set_attrs() {
   METIS_CUDA_TRY(cudaFuncSetAttribute(residual_quant_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true)));
   METIS_CUDA_TRY(cudaFuncSetAttribute(gram_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GC_MAX_SMEM));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::JC_SMEM));
+#define METIS_JF_ATTR(LN, R) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_fp32_kernel<LN, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::jf_smem(LN, R)))
+  METIS_JF_ATTR(8, 12); METIS_JF_ATTR(8, 14); METIS_JF_ATTR(8, 16); METIS_JF_ATTR(8, 18); METIS_JF_ATTR(8, 22);
+  METIS_JF_ATTR(16, 12); METIS_JF_ATTR(16, 14); METIS_JF_ATTR(16, 16); METIS_JF_ATTR(16, 18);
+#undef METIS_JF_ATTR
+  METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::chol_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::cm_smem(metis_wide::CM_MAX)));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::chol_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::CW_SMEM));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::trsm_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::TW_SMEM));
 #define METIS_PP_ATTR(MTV) METIS_CUDA_TRY(cudaFuncSetAttribute(project_pipe_kernel<MTV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \

@@ -404,3 +404,28 @@ def test_eigen_solver_sizes_and_spectra(ctx, k, p, spectrum):
     assert (core - torch.diag(torch.diagonal(core))).abs().max() < 1e-6 * sig[0]
     assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
     assert bool((sig[:-1] >= sig[1:]).all())
+
+
+@pytest.mark.parametrize("k,p", [(68, 4), (96, 1), (100, 11), (112, 20), (128, 8), (136, 24), (160, 3), (176, 17), (220, 5), (256, 16)])
+@pytest.mark.parametrize("spectrum", ["geometric", "equal"])
+def test_wide_eigen_solver_sizes_and_spectra(ctx, k, p, spectrum):
+    """The cluster eigen-solver and both wide Cholesky factorisations at the edges of their size classes, with separated and with
+    equal singular values (the FP64 sweeps).  Bounds as in the small solver's test."""
+    B, h = ctx
+    g = torch.Generator(device="cuda")
+    g.manual_seed(100 * k + p)
+    rows, cols = 768, 640
+    u = torch.linalg.qr(torch.randn((rows, k), generator=g, device="cuda", dtype=torch.float64))[0]
+    v = torch.linalg.qr(torch.randn((cols, k), generator=g, device="cuda", dtype=torch.float64))[0]
+    i = torch.arange(k, device="cuda", dtype=torch.float64)
+    s = 3000.0 * 10 ** (-i / k) if spectrum == "geometric" else 1000.0 + 0 * i
+    x = ((u * s) @ v.T + 0.05 * torch.randn((rows, cols), generator=g, device="cuda", dtype=torch.float64)).to(torch.bfloat16)
+    op = h.split(x, k, p, sketch=B.SKETCH_FULL, seed=11)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    left, right, sig, xd = op.left.double(), op.right.double(), op.sigma.double(), x.double()
+    eye = torch.eye(k, device="cuda", dtype=torch.float64)
+    assert (left @ left.T - eye).abs().max() < 1e-6 and (right @ right.T - eye).abs().max() < 1e-6
+    core = left @ xd @ right.T
+    assert (core - torch.diag(torch.diagonal(core))).abs().max() < 1e-6 * sig[0]
+    assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
