@@ -323,8 +323,9 @@ metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t
 // Few long rows (the transposed split factors: k x len FP32, blocks along the contiguous dimension only): one
 // thread per block of 16, no tiles, no shared memory.  Threads beyond `rows` inside the last 128-row slab of the
 // tiled scale layout write zero scale bytes.
-__device__ __forceinline__ void rowblocks_body(const float* __restrict__ x, int64_t ld, const metis_qt::QuantParams& p,
-                                               const float* __restrict__ tscale_src, int tscale_is_amax, float* ts_out) {
+__device__ __forceinline__ void rowblocks_body(const float* x, int64_t ld, const metis_qt::QuantParams& p,
+                                               const float* __restrict__ tscale_src, int tscale_is_amax, float* ts_out,
+                                               const unsigned long long* __restrict__ keys, float* flip) {
   const int64_t bpr = p.cols / 16;
   const int64_t rows_pad = p.c_layout == METIS_SF_TILED ? (p.rows + 127) / 128 * 128 : p.rows;
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -340,6 +341,12 @@ __device__ __forceinline__ void rowblocks_body(const float* __restrict__ x, int6
   for (int i = 0; i < 4; ++i) {
     const float4 q = *reinterpret_cast<const float4*>(x + r * ld + b * 16 + i * 4);
     v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
+  }
+  if (keys != nullptr && (keys[r] & 1ull)) {               // the sign convention of the factor pair: this vector is flipped, in place
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] = -v[i];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<float4*>(flip + r * ld + b * 16 + i * 4) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
   }
   if (sr) {
     if (p.e_stride_c == 1 && (p.e_stride_r & 7) == 0) {
@@ -368,7 +375,7 @@ __device__ __forceinline__ void rowblocks_body(const float* __restrict__ x, int6
 __global__ void __launch_bounds__(256)
 quantize_rowblocks_kernel(const float* __restrict__ x, int64_t ld, metis_qt::QuantParams p, const float* __restrict__ tscale_src,
                           int tscale_is_amax, float* ts_out) {
-  rowblocks_body(x, ld, p, tscale_src, tscale_is_amax, ts_out);
+  rowblocks_body(x, ld, p, tscale_src, tscale_is_amax, ts_out, nullptr, nullptr);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -457,11 +464,13 @@ metis_status_t metis_launch_quantize_rht(metis_context* ctx, const void* x, int 
 }
 
 // two factor tensors in one launch (blockIdx.y selects): the left and right factors of a decomposition
-struct RowblocksJob { const float* x; int64_t ld; metis_qt::QuantParams p; const float* tscale_src; float* ts_out; };
+// (keys: the sign keys of the vectors, or nullptr; x is then flipped where the key says so)
+struct RowblocksJob { float* x; int64_t ld; metis_qt::QuantParams p; const float* tscale_src; float* ts_out; const unsigned long long* keys; };
 __global__ void __launch_bounds__(256)
 quantize_rowblocks_pair_kernel(RowblocksJob a, RowblocksJob b) {
   const RowblocksJob& j = blockIdx.y == 0 ? a : b;
-  rowblocks_body(j.x, j.ld, j.p, j.tscale_src, 1, j.ts_out);
+  metis_pdl_wait();
+  rowblocks_body(j.x, j.ld, j.p, j.tscale_src, 1, j.ts_out, j.keys, j.x);
 }
 
 metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, int rounding,
@@ -504,12 +513,13 @@ metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int
 
 // The two FP32 factor tensors of a decomposition (k x rows and k x cols, k <= 64, blocks along the long dimension,
 // tensor scale from each tensor's own amax) in one launch.
-metis_status_t metis_launch_quantize_factors(const float* left, int64_t rows, const float* right, int64_t cols, int k, int rounding,
+metis_status_t metis_launch_quantize_factors(float* left, int64_t rows, float* right, int64_t cols, int k, int rounding,
                                              uint64_t seed, const float* amax_left, const float* amax_right,
-                                             const metis_nvfp4_t* lq, const metis_nvfp4_t* rq, cudaStream_t s) {
+                                             const metis_nvfp4_t* lq, const metis_nvfp4_t* rq, cudaStream_t s, const unsigned long long* keys) {
   using namespace metis_qt;
   if (k <= 0 || k > 256 || rows % 16 || cols % 16) return METIS_ERR_SHAPE;
   RowblocksJob a{}, b{};
+  a.keys = b.keys = keys;
   a.x = left; a.ld = rows; a.tscale_src = amax_left; a.ts_out = lq->tensor_scale;
   a.p.rows = k; a.p.cols = rows; a.p.rounding = rounding; a.p.seed = seed; a.p.stream_id = METIS_STREAM_LEFT;
   a.p.e_stride_r = rows; a.p.e_stride_c = 1; a.p.c_codes = lq->codes; a.p.c_scales = lq->scales; a.p.c_layout = lq->sf_layout;
@@ -519,7 +529,6 @@ metis_status_t metis_launch_quantize_factors(const float* left, int64_t rows, co
   const int64_t pad_a = a.p.c_layout == METIS_SF_TILED ? (k + 127) / 128 * 128 : k, pad_b = b.p.c_layout == METIS_SF_TILED ? (k + 127) / 128 * 128 : k;
   const int64_t work_a = pad_a * (rows / 16), work_b = pad_b * (cols / 16);
   const unsigned gx = (unsigned)metis_ceil_div(work_a > work_b ? work_a : work_b, 256);
-  quantize_rowblocks_pair_kernel<<<dim3(gx, 2), 256, 0, s>>>(a, b); METIS_COUNT_LAUNCH();
-  METIS_CUDA_TRY(cudaGetLastError());
+  METIS_CUDA_TRY(metis_launch_pdl(quantize_rowblocks_pair_kernel, dim3(gx, 2), dim3(256), (size_t)0, s, a, b)); METIS_COUNT_LAUNCH();
   return METIS_OK;
 }

@@ -19,8 +19,14 @@ constexpr int MAXQ = metis_small::MAXQ;                // k + p at most (k = 64 
 constexpr int LP = metis_small::PITCH;                 // row pitch of a factor in shared memory
 
 // ------------------------------------------------------------------------------------------------
-__global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, int64_t rows, uint64_t seed, int full) {
+// The sampled rows; the first block of the one-CTA chain's call also clears what its later kernels accumulate into (a memset of
+// its own was a launch in front of every decomposition).
+__global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, int64_t rows, uint64_t seed, int full, float* __restrict__ amax, unsigned long long* __restrict__ keys) {
   metis_pdl_wait();
+  if (blockIdx.x == 0 && amax != nullptr && threadIdx.x < 64) {
+    if (threadIdx.x < 16) amax[threadIdx.x] = 0.0f;
+    keys[threadIdx.x] = 0ull;
+  }
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n_s) return;
   if (full) { idx[j] = j; return; }
@@ -351,47 +357,6 @@ project_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __r
       if (col < cols) dst[(int64_t)(2 * j + jg) * cols + col] = acc0[j];
       if (col + 1 < cols) dst[(int64_t)(2 * j + jg) * cols + col + 1] = acc1[j];
     }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Right basis from the small SVD: B[j][col] = sum_i Ut[i][j] M[i][col] / s_j, s_j = sqrt(eval_j); j < k.
-// Block = 64 columns x 4 groups of output vectors; a thread keeps four accumulators in flight.
-constexpr int RB_COLS = 32;
-__global__ void __launch_bounds__(256)
-right_basis_kernel(const float* __restrict__ m, int64_t cols, int q, int k, const double* __restrict__ evals,
-                   const double* __restrict__ evecs, float* __restrict__ basis, float* __restrict__ sigma_out) {
-  metis_pdl_wait();
-  // 32 columns per CTA; the CTA's slice of M is staged in shared memory first, so that all of its loads are in
-  // flight at once (read inside the accumulation loop they were one L2 round trip per term)
-  __shared__ double ut[MAXQ][64 + 1];                   // eigenvectors, the k <= 64 wanted columns
-  __shared__ double inv_s[64];
-  __shared__ float ms[MAXQ][RB_COLS];
-  const int tid = threadIdx.x, cx = tid & (RB_COLS - 1), jg = tid / RB_COLS;      // 8 groups of output vectors
-  const int64_t col0 = (int64_t)blockIdx.x * RB_COLS;
-  for (int o = tid; o < q * RB_COLS; o += 256) {
-    const int i = o / RB_COLS, c = o % RB_COLS;
-    ms[i][c] = col0 + c < cols ? m[(int64_t)i * cols + col0 + c] : 0.0f;
-  }
-  for (int o = tid; o < q * k; o += 256) ut[o / k][o % k] = evecs[(o / k) * q + o % k];
-  if (tid < k) {
-    const double s = sqrt(fmax(evals[tid], 0.0));
-    inv_s[tid] = s > 0.0 ? 1.0 / s : 0.0;
-    if (blockIdx.x == 0 && sigma_out != nullptr) sigma_out[tid] = (float)s;
-  }
-  __syncthreads();
-  const int64_t col = col0 + cx;
-  if (col >= cols) return;
-  for (int j0 = jg * 4; j0 < k; j0 += 32) {
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    for (int i = 0; i < q; ++i) {
-      const double v = (double)ms[i][cx];
-      a0 += ut[i][j0] * v; a1 += ut[i][j0 + 1] * v; a2 += ut[i][j0 + 2] * v; a3 += ut[i][j0 + 3] * v;
-    }
-    basis[(int64_t)j0 * cols + col] = (float)(a0 * inv_s[j0]);
-    if (j0 + 1 < k) basis[(int64_t)(j0 + 1) * cols + col] = (float)(a1 * inv_s[j0 + 1]);
-    if (j0 + 2 < k) basis[(int64_t)(j0 + 2) * cols + col] = (float)(a2 * inv_s[j0 + 2]);
-    if (j0 + 3 < k) basis[(int64_t)(j0 + 3) * cols + col] = (float)(a3 * inv_s[j0 + 3]);
-  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -993,138 +958,207 @@ project_pipe_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int
 }
 
 
-// right[j][col] = sum_i basis[i][col] * W[i][j] (W == nullptr: identity).  One thread per column; each CTA
-// also records, for every j, its entry of largest magnitude (signed value and column, lowest column on ties)
-// for the sign convention.
-__global__ void __launch_bounds__(256)
-right_rotate_kernel(const float* __restrict__ basis, int64_t cols, int k, const double* __restrict__ w,
-                    float* __restrict__ right, float* __restrict__ cand_v, int* __restrict__ cand_i) {
-  metis_pdl_wait();
-  __shared__ float wsm[MAXQ][MAXQ + 1];
-  __shared__ float red_v[8][MAXQ];
-  __shared__ int red_i[8][MAXQ];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (w) for (int o = tid; o < k * k; o += 256) wsm[o / k][o % k] = (float)w[o];
-  __syncthreads();
-  const int64_t col = (int64_t)blockIdx.x * 256 + tid;
-  // blockIdx.y owns the output vectors j = 8*blockIdx.y .. +7 (a CTA per 256 columns alone leaves most SMs idle)
-  const int j_begin = blockIdx.y * 8, j_end = min(k, j_begin + 8);
-  float bv[MAXQ];
-#pragma unroll
-  for (int i = 0; i < MAXQ; ++i) bv[i] = (i < k && col < cols) ? basis[(int64_t)i * cols + col] : 0.0f;
-  for (int j = j_begin; j < j_end; ++j) {
-    float v;
-    if (w) {
-      v = 0.0f;
-#pragma unroll
-      for (int i = 0; i < MAXQ; ++i) if (i < k) v = fmaf(bv[i], wsm[i][j], v);
-    } else {
-      v = 0.0f;
-#pragma unroll
-      for (int i = 0; i < MAXQ; ++i) if (i == j) v = bv[i];
-    }
-    if (col < cols) right[(int64_t)j * cols + col] = v;
-    float av = col < cols ? fabsf(v) : -1.0f, sv = v;            // magnitude for the contest, signed value for the decision
-    int ai = (int)min(col, (int64_t)0x7FFFFFFF);
-#pragma unroll
-    for (int sft = 16; sft > 0; sft >>= 1) {
-      const float ov = __shfl_xor_sync(0xFFFFFFFFu, av, sft);
-      const float os = __shfl_xor_sync(0xFFFFFFFFu, sv, sft);
-      const int oi = __shfl_xor_sync(0xFFFFFFFFu, ai, sft);
-      if (ov > av || (ov == av && oi < ai)) { av = ov; ai = oi; sv = os; }
-    }
-    if (lane == 0) { red_v[warp][j] = sv; red_i[warp][j] = ai; }
-  }
-  __syncthreads();
-  if (tid >= j_begin && tid < j_end) {
-    float sv = red_v[0][tid]; int ai = red_i[0][tid];
-    for (int wv = 1; wv < 8; ++wv) {
-      const float ov = red_v[wv][tid];
-      if (fabsf(ov) > fabsf(sv) || (fabsf(ov) == fabsf(sv) && red_i[wv][tid] < ai)) { sv = ov; ai = red_i[wv][tid]; }
-    }
-    cand_v[(int64_t)blockIdx.x * k + tid] = sv;                  // signed winner of this column chunk
-    cand_i[(int64_t)blockIdx.x * k + tid] = ai;
-  }
+// ------------------------------------------------------------------------------------------------
+// Factors from eigenvectors:  out[j][p] = scale_j sum_i src(i, p) W[i][j]  for a tile of 64 positions p (columns or rows of the
+// operand) and every j < k, on the FP64 tensor cores; i <= 72, j <= 64.  Used for the right basis (src = M, W = evecs), the left
+// factor (src = H or C) and the Rayleigh-Ritz rotation of the basis.  One kernel per stage of the chain does all that is
+// derived from the product - BF16 splits, the operands of the residual product, tensor amax, the sign decision - because the chain is
+// latency: the right basis, its sign, its splits, the left factor and its splits were six launches (28 us at
+// 4096 x 4096, k = 32; now 11 us in two), and beside a persistent residual pass, on the few SMs it leaves, FP32 multiply-adds with 72
+// registers of basis values a thread took 775 us for 28672 x 64.
+//
+// Sign convention: the entry of largest magnitude of a right vector (lowest index on ties) is positive.  The contest is an
+// atomic maximum over keys (magnitude bits, inverted column, sign), whatever the order of arrival; the factors stay
+// unsigned until the factor quantizer, which reads the key's sign and flips both (the residual C B^T does not see it).
+constexpr int FR_POS = 64, FR_P = FR_POS + 4, FR_OP = FR_POS + 1;
+__host__ __device__ constexpr size_t fr_smem(int n_in) { return sizeof(double) * 2 * (size_t)((n_in + 7) / 8 * 8 < 40 ? 40 : (n_in + 7) / 8 * 8) * FR_P; }
+__device__ __forceinline__ unsigned long long sign_key(float v, int64_t col) {
+  const uint32_t b = __float_as_uint(v);
+  return ((unsigned long long)(b & 0x7FFFFFFFu) << 32) | ((0x7FFFFFFFull - (unsigned long long)col) << 1) | (v < 0.0f ? 1ull : 0ull);
 }
 
-// Sign convention: the largest-magnitude entry of each right vector (lowest index on ties) is made positive.
-// grid (column chunks, k).  Every CTA re-derives the winner of its vector from the per-chunk candidates, whose
-// signed values were recorded before any flipping (the flips of other CTAs must not influence the decision).
-__global__ void __launch_bounds__(256)
-sign_fix_kernel(float* __restrict__ right, int64_t cols, int k, const float* __restrict__ cand_v,
-                const int* __restrict__ cand_i, int n_cand, float* __restrict__ sign_out, float* __restrict__ amax_out) {
-  metis_pdl_wait();
-  const int j = blockIdx.y;
-  float sv = 0.0f; int ai = 0x7FFFFFFF;
-  for (int c = 0; c < n_cand; ++c) {
-    const float v = cand_v[(int64_t)c * k + j]; const int i = cand_i[(int64_t)c * k + j];
-    if (fabsf(v) > fabsf(sv) || (fabsf(v) == fabsf(sv) && i < ai)) { sv = v; ai = i; }
-  }
-  const float sg = sv < 0.0f ? -1.0f : 1.0f;
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    sign_out[j] = sg;
-    // the winner's magnitude is the vector's amax: the factor's tensor scale needs the max over all vectors
-    if (amax_out != nullptr) atomicMax(reinterpret_cast<unsigned int*>(amax_out), __float_as_uint(fabsf(sv)));
-  }
-  const int64_t col = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (sg < 0.0f && col < cols) right[(int64_t)j * cols + col] = -right[(int64_t)j * cols + col];
-}
-
-// left[j][r] = sign_j * scale_j * sum_i coef(i, r) * W[i][j],  coef(i, r) = c[i*stride_i + r*stride_r]
-// scale_j = 1/sqrt(eval_j) when inv_sqrt_evals is given (Rayleigh-Ritz normalisation), else 1.
-// Also writes sigma_out[j] = sqrt(eval_j) when asked, and coef_rm[r][j] = left[j][r] * sigma_for_coef[j]
-// (row-major, kp columns, zero padded) when asked.
-__global__ void __launch_bounds__(256)
-left_rotate_kernel(const float* __restrict__ c, int64_t rows, int n_in, int k, int64_t stride_i, int64_t stride_r,
-                   const double* __restrict__ w, const double* __restrict__ evals_for_scale,
-                   const float* __restrict__ sign, float* __restrict__ left, float* __restrict__ sigma_out,
-                   float* __restrict__ coef_rm, int kp, const float* __restrict__ sigma_for_coef,
-                   float* __restrict__ amax_out) {
-  metis_pdl_wait();
-  __shared__ double ws[MAXQ][MAXQ + 1];
-  __shared__ double scl[MAXQ];
-  const int tid = threadIdx.x, rx = tid & 63, jg = tid >> 6;
-  for (int o = tid; o < n_in * n_in; o += 256) ws[o / n_in][o % n_in] = w[o];
-  if (tid < k) {
-    double s = 1.0;
-    if (evals_for_scale) {
-      const double lam = sqrt(fmax(evals_for_scale[tid], 0.0));
-      s = lam > 0.0 ? 1.0 / lam : 0.0;
-      if (blockIdx.x == 0 && blockIdx.y == 0 && sigma_out) sigma_out[tid] = (float)lam;
-    }
-    scl[tid] = s * (double)sign[tid];
-  }
-  __syncthreads();
-  const int64_t r = (int64_t)blockIdx.x * 64 + rx;
-  float am = 0.0f;
-  if (r < rows) {
-    for (int j0 = jg * 4 + 16 * blockIdx.y; j0 < kp; j0 += 16 * gridDim.y) {   // blockIdx.y: every gridDim.y-th group of 16 outputs
-      double a[4] = {0.0, 0.0, 0.0, 0.0};
-      if (j0 < k) {
+// Os[j][p] = (float)(scale[j] * sum); rows j in [k, 8 KT + 8) are zero.  src(i, p) = src[i * stride_i + p * stride_p], one of the strides 1.
+template <int KT>
+__device__ __forceinline__ void factor_tile(const float* __restrict__ src, int64_t n_pos, int64_t p0, int64_t stride_i, int64_t stride_p, int n_in,
+                                            const double* __restrict__ w, int ldw, int k, const double* scale, double* As, double* Ws, float* Os) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3, n8 = (n_in + 7) & ~7;
+  if (stride_p == 1) {
 #pragma unroll 4
-        for (int i = 0; i < n_in; ++i) {
-          const double v = (double)c[i * stride_i + r * stride_r];
-          a[0] += v * ws[i][j0]; a[1] += v * ws[i][j0 + 1]; a[2] += v * ws[i][j0 + 2]; a[3] += v * ws[i][j0 + 3];
-        }
-      }
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int j = j0 + t;
-        if (j < k) {
-          const float v = (float)(a[t] * scl[j]);
-          left[(int64_t)j * rows + r] = v;
-          am = fmaxf(am, fabsf(v));
-          if (coef_rm) coef_rm[r * kp + j] = v * sigma_for_coef[j];
-        } else if (coef_rm && j < kp) {
-          coef_rm[r * kp + j] = 0.0f;
-        }
-      }
+    for (int o = tid; o < n8 * FR_POS; o += 256) {
+      const int i = o / FR_POS, c = o % FR_POS;
+      As[i * FR_P + c] = i < n_in && p0 + c < n_pos ? (double)src[i * stride_i + p0 + c] : 0.0;
+    }
+  } else {
+#pragma unroll 4
+    for (int o = tid; o < n8 * FR_POS; o += 256) {
+      const int c = o / n8, i = o - c * n8;
+      As[i * FR_P + c] = i < n_in && p0 + c < n_pos ? (double)src[(p0 + c) * stride_p + i] : 0.0;
     }
   }
-  // amax|left| for the factor's tensor scale (order-independent atomic max on the float bits)
+#pragma unroll 4
+  for (int o = tid; o < n8 * 8 * KT; o += 256) {
+    const int i = o / (8 * KT), j = o % (8 * KT);
+    Ws[i * FR_P + j] = i < n_in && j < k ? w[i * ldw + j] : 0.0;
+  }
+  __syncthreads();
+  double acc[KT][2] = {};
+  for (int kk = 0; kk < n8; kk += 4) {
+    const double a = As[(kk + q) * FR_P + 8 * warp + g];
+#pragma unroll
+    for (int t = 0; t < KT; ++t) metis_small::dmma(acc[t], a, Ws[(kk + q) * FR_P + 8 * t + g]);
+  }
+  __syncthreads();                                      // Os lies over As
+#pragma unroll
+  for (int t = 0; t < KT; ++t)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int j = 8 * t + 2 * q + e;
+      Os[j * FR_OP + 8 * warp + g] = j < k ? (float)(scale != nullptr ? acc[t][e] * scale[j] : acc[t][e]) : 0.0f;
+    }
+  for (int o = tid; o < 8 * FR_OP; o += 256) Os[8 * KT * FR_OP + o] = 0.0f;
+  __syncthreads();
+}
+
+// the tile's entries into the sign contest and the tensor amax, one warp per vector
+__device__ __forceinline__ void sign_contest(const float* Os, int k, int64_t p0, int64_t n_pos, unsigned long long* keys, float* amax) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t top = 0u;
+  for (int j = warp; j < k; j += 8) {
+    unsigned long long key = p0 + lane < n_pos ? sign_key(Os[j * FR_OP + lane], p0 + lane) : 0ull;
+    if (p0 + lane + 32 < n_pos) { const unsigned long long o = sign_key(Os[j * FR_OP + lane + 32], p0 + lane + 32); key = o > key ? o : key; }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) { const unsigned long long x = __shfl_xor_sync(0xFFFFFFFFu, key, o); key = x > key ? x : key; }
+    if (lane == 0) atomicMax(keys + j, key);
+    top = max(top, (uint32_t)(key >> 32));
+  }
+  if (lane == 0 && top != 0u) atomicMax(reinterpret_cast<unsigned int*>(amax), top);
+}
+
+// Right basis B[j][col] = sum_i evecs[i][j] M[i][col] / s_j, s_j = sqrt(eval_j), and its BF16 splits (see basis_splits_kernel; bs,
+// bt and b6 are optional).  keys (FULL mode, where this is the right factor itself): the sign contest.
+template <int KT>
+__global__ void __launch_bounds__(256)
+basis_kernel(const float* __restrict__ m, int64_t cols, int q, int k, int kp, const double* __restrict__ evals, const double* __restrict__ evecs,
+             float* __restrict__ basis, __nv_bfloat16* __restrict__ bs, __nv_bfloat16* __restrict__ bt, __nv_bfloat16* __restrict__ b6, int kx,
+             float* __restrict__ sigma_out, unsigned long long* __restrict__ keys, float* __restrict__ amax_out) {
+  metis_pdl_wait();
+  extern __shared__ __align__(16) double fr_sm[];
+  __shared__ double scale[FR_POS];
+  double *As = fr_sm, *Ws = fr_sm + ((q + 7) / 8 * 8 < 40 ? 40 : (q + 7) / 8 * 8) * FR_P;
+  float* Os = reinterpret_cast<float*>(As);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int64_t p0 = (int64_t)blockIdx.x * FR_POS;
+  if (tid < k) {
+    const double sv = sqrt(fmax(evals[tid], 0.0));
+    scale[tid] = sv > 0.0 ? 1.0 / sv : 0.0;
+    if (blockIdx.x == 0 && sigma_out != nullptr) sigma_out[tid] = (float)sv;
+  }
+  factor_tile<KT>(m, cols, p0, cols, 1, q, evecs, q, k, scale, As, Ws, Os);
+  for (int o = tid; o < k * FR_POS; o += 256) {
+    const int j = o / FR_POS, c = o % FR_POS;
+    if (p0 + c < cols) basis[(int64_t)j * cols + p0 + c] = Os[j * FR_OP + c];
+  }
+  const int64_t col2 = p0 + 2 * lane;                   // a pair of columns (their number is a multiple of 16)
+  for (int j = warp; j < kp && bs != nullptr; j += 8) {
+    uint32_t h, l, l2;
+    split3(Os[j * FR_OP + 2 * lane], Os[j * FR_OP + 2 * lane + 1], h, l, l2);
+    if (col2 < cols) {
+      *reinterpret_cast<uint32_t*>(bs + (int64_t)j * cols + col2) = h;
+      *reinterpret_cast<uint32_t*>(bs + (int64_t)(kp + j) * cols + col2) = l;
+      *reinterpret_cast<uint32_t*>(bs + (int64_t)(2 * kp + j) * cols + col2) = l2;
+    }
+  }
+  for (int o = tid; o < FR_POS * (kp / 8); o += 256) {
+    const int c = o / (kp / 8), j0 = o % (kp / 8) * 8;  // consecutive threads: consecutive 16-byte groups of a column's row
+    const int64_t col = p0 + c;
+    if (col >= cols) break;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = Os[(j0 + e) * FR_OP + c];
+    uint4 h, l, l2;
+    metis_split3x8(v, h, l, l2);
+    if (bt != nullptr) {
+      *reinterpret_cast<uint4*>(bt + col * kp + j0) = h;
+      *reinterpret_cast<uint4*>(bt + (cols + col) * kp + j0) = l;
+      *reinterpret_cast<uint4*>(bt + (2 * cols + col) * kp + j0) = l2;
+    }
+    if (b6 != nullptr) {
+      __nv_bfloat16* dst = b6 + col * kx + j0;
+      *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + kp) = l; *reinterpret_cast<uint4*>(dst + 2 * kp) = h;
+      *reinterpret_cast<uint4*>(dst + 3 * kp) = l2; *reinterpret_cast<uint4*>(dst + 4 * kp) = h; *reinterpret_cast<uint4*>(dst + 5 * kp) = l;
+      if (j0 == 0)
+        for (int z = 6 * kp; z < kx; z += 8) *reinterpret_cast<uint4*>(b6 + col * kx + z) = make_uint4(0u, 0u, 0u, 0u);
+    }
+  }
+  if (keys != nullptr) sign_contest(Os, k, p0, cols, keys, amax_out);
+}
+
+// The factors of a decomposition, unsigned.  Blocks below n_right: right[j][col] = sum_i basis[i][col] W[i][j] and the sign contest;
+// the others: left[j][r] = s_j sum_i src[r * ld + i] W[i][j] with s_j = 1 / sqrt(eval_j) when evals is given (Rayleigh-Ritz; sigma_out = sqrt(eval_j)),
+// and from it the coefficients left * sigma of the residual product (FULL mode): as its BF16 operand a6, or as coef [r][kp].
+struct FactorsArgs {
+  const double* w; int ldw, n_in, k, kp;
+  const float* basis; int64_t cols; float* right; unsigned long long* keys; float* amax_right;
+  const float* src; int64_t ld, rows; const double* evals; float* left; float* sigma_out; float* amax_left;
+  const float* sigma_for_coef; float* coef; __nv_bfloat16* a6; int kx;
+};
+template <int KT>
+__global__ void __launch_bounds__(256)
+factors_kernel(FactorsArgs f, int n_right) {
+  metis_pdl_wait();
+  extern __shared__ __align__(16) double fr_sm[];
+  __shared__ double scale[FR_POS];
+  double *As = fr_sm, *Ws = fr_sm + ((f.n_in + 7) / 8 * 8 < 40 ? 40 : (f.n_in + 7) / 8 * 8) * FR_P;
+  float* Os = reinterpret_cast<float*>(As);
+  const int tid = threadIdx.x, k = f.k;
+  if ((int)blockIdx.x < n_right) {
+    const int64_t p0 = (int64_t)blockIdx.x * FR_POS;
+    factor_tile<KT>(f.basis, f.cols, p0, f.cols, 1, f.n_in, f.w, f.ldw, k, nullptr, As, Ws, Os);
+    for (int o = tid; o < k * FR_POS; o += 256) {
+      const int j = o / FR_POS, c = o % FR_POS;
+      if (p0 + c < f.cols) f.right[(int64_t)j * f.cols + p0 + c] = Os[j * FR_OP + c];
+    }
+    sign_contest(Os, k, p0, f.cols, f.keys, f.amax_right);
+    return;
+  }
+  const int64_t p0 = (int64_t)((int)blockIdx.x - n_right) * FR_POS;
+  if (f.evals != nullptr && tid < k) {
+    const double lam = sqrt(fmax(f.evals[tid], 0.0));
+    scale[tid] = lam > 0.0 ? 1.0 / lam : 0.0;
+    if ((int)blockIdx.x == n_right) f.sigma_out[tid] = (float)lam;
+  }
+  factor_tile<KT>(f.src, f.rows, p0, 1, f.ld, f.n_in, f.w, f.ldw, k, f.evals != nullptr ? scale : nullptr, As, Ws, Os);
+  float am = 0.0f;
+  for (int o = tid; o < k * FR_POS; o += 256) {
+    const int j = o / FR_POS, c = o % FR_POS;
+    const float v = Os[j * FR_OP + c];
+    if (p0 + c < f.rows) { f.left[(int64_t)j * f.rows + p0 + c] = v; am = fmaxf(am, fabsf(v)); }
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) am = fmaxf(am, __shfl_xor_sync(0xFFFFFFFFu, am, o));
-  if ((tid & 31) == 0 && amax_out != nullptr) atomicMax(reinterpret_cast<unsigned int*>(amax_out), __float_as_uint(am));
+  if ((tid & 31) == 0) atomicMax(reinterpret_cast<unsigned int*>(f.amax_left), __float_as_uint(am));
+  if (f.sigma_for_coef == nullptr) return;
+  const int kp = f.kp;
+  for (int o = tid; o < FR_POS * (kp / 8); o += 256) {
+    const int c = o / (kp / 8), j0 = o % (kp / 8) * 8;
+    const int64_t r = p0 + c;
+    if (r >= f.rows) break;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = j0 + e < k ? Os[(j0 + e) * FR_OP + c] * f.sigma_for_coef[j0 + e] : 0.0f;
+    if (f.a6 != nullptr) {
+      uint4 h, l, l2;
+      metis_split3x8(v, h, l, l2);
+      __nv_bfloat16* dst = f.a6 + r * f.kx + j0;
+      *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + kp) = h; *reinterpret_cast<uint4*>(dst + 2 * kp) = l;
+      *reinterpret_cast<uint4*>(dst + 3 * kp) = h; *reinterpret_cast<uint4*>(dst + 4 * kp) = l2; *reinterpret_cast<uint4*>(dst + 5 * kp) = l;
+      if (j0 == 0)
+        for (int z = 6 * kp; z < f.kx; z += 8) *reinterpret_cast<uint4*>(f.a6 + r * f.kx + z) = make_uint4(0u, 0u, 0u, 0u);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 8; ++e) f.coef[r * kp + j0 + e] = v[e];
+    }
+  }
 }
 
 // Columns per sketch CTA: a sampled sketch has few rows, so narrow chunks are what gives it enough CTAs; a full
@@ -1135,7 +1169,7 @@ int sketch_tc_cols(int q) { return q <= 48 ? 48 : 96; }
 int sketch_chunk_cols(int64_t n_s) { return n_s <= 512 ? 64 : SKM_COLS; }
 
 struct SplitWs {
-  size_t amax, idx, zp, omt, z, gram, gram1, linv, evals, evecs, mp, m, basis, coef, sign, cand_v, cand_i, evals2, evecs2, bs, bt,
+  size_t amax, idx, zp, omt, z, gram, gram1, linv, evals, evecs, mp, m, basis, coef, keys, evals2, evecs2, bs, bt,
       gram_c, part, a6, b6, hsp, total;
 };
 
@@ -1187,9 +1221,7 @@ SplitWs split_ws_layout(int64_t rows, int64_t cols, int k, int p, int64_t n_s) {
   w.bs = take(sizeof(__nv_bfloat16) * 3 * (size_t)kp * cols);
   w.bt = take(sizeof(__nv_bfloat16) * 3 * (size_t)kp * cols);
   w.gram_c = take(sizeof(double) * (size_t)metis_ceil_div(rows, 32) * kp * kp);
-  w.sign = take(sizeof(float) * MAXQ);
-  w.cand_v = take(sizeof(float) * MAXQ * (size_t)metis_ceil_div(cols, 256));
-  w.cand_i = take(sizeof(int) * MAXQ * (size_t)metis_ceil_div(cols, 256));
+  w.keys = take(sizeof(unsigned long long) * MAXQ);
   w.evals2 = take(sizeof(double) * MAXQ);
   w.evecs2 = take(sizeof(double) * MAXQ * MAXQ);
   w.total = off;
@@ -1222,6 +1254,39 @@ template <int NJ4>
 void launch_project(dim3 grid, cudaStream_t s, const __nv_bfloat16* x, int64_t cols, const int* idx, int n_s, int q,
                     const float* h, int rpp, float* mp) {
   (void)(metis_launch_pdl((project_kernel<NJ4>), dim3(grid), dim3(256), (size_t)(0), s, x, cols, idx, n_s, q, h, rpp, mp)); METIS_COUNT_LAUNCH();
+}
+
+template <int KT>
+metis_status_t launch_basis_kt(cudaStream_t s, int ctas, size_t smem, const float* m, int64_t cols, int q, int k, int kp, const double* evals, const double* evecs, float* basis,
+                               __nv_bfloat16* bs, __nv_bfloat16* bt, __nv_bfloat16* b6, int kx, float* sigma_out, unsigned long long* keys, float* amax_out) {
+  METIS_CUDA_TRY(metis_launch_pdl((basis_kernel<KT>), dim3((unsigned)ctas), dim3(256), smem, s, m, cols, q, k, kp, evals, evecs, basis, bs, bt, b6, kx, sigma_out, keys, amax_out));
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+template <typename... A>
+metis_status_t launch_basis(cudaStream_t s, int ctas, size_t smem, const float* m, int64_t cols, int q, int k, A... rest) {
+  switch ((k + 7) / 8) {
+    case 1: return launch_basis_kt<1>(s, ctas, smem, m, cols, q, k, rest...);
+    case 2: return launch_basis_kt<2>(s, ctas, smem, m, cols, q, k, rest...);
+    case 3: return launch_basis_kt<3>(s, ctas, smem, m, cols, q, k, rest...);
+    case 4: return launch_basis_kt<4>(s, ctas, smem, m, cols, q, k, rest...);
+    case 5: return launch_basis_kt<5>(s, ctas, smem, m, cols, q, k, rest...);
+    case 6: return launch_basis_kt<6>(s, ctas, smem, m, cols, q, k, rest...);
+    case 7: return launch_basis_kt<7>(s, ctas, smem, m, cols, q, k, rest...);
+    default: return launch_basis_kt<8>(s, ctas, smem, m, cols, q, k, rest...);
+  }
+}
+metis_status_t launch_factors(cudaStream_t s, const FactorsArgs& f, int n_right, int n_left) {
+  const dim3 grid((unsigned)(n_right + n_left));
+  const size_t smem = fr_smem(f.n_in);
+#define METIS_FACTORS(KT) METIS_CUDA_TRY(metis_launch_pdl((factors_kernel<KT>), grid, dim3(256), smem, s, f, n_right)); break
+  switch ((f.k + 7) / 8) {
+    case 1: METIS_FACTORS(1); case 2: METIS_FACTORS(2); case 3: METIS_FACTORS(3); case 4: METIS_FACTORS(4);
+    case 5: METIS_FACTORS(5); case 6: METIS_FACTORS(6); case 7: METIS_FACTORS(7); default: METIS_FACTORS(8);
+  }
+#undef METIS_FACTORS
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1401,7 +1466,8 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
   if (src_amax != nullptr) METIS_CUDA_TRY(cudaMemcpyAsync(amax, src_amax, sizeof(float), cudaMemcpyDeviceToDevice, s));
   const __nv_bfloat16* xr = x;
   if (!full) {
-    METIS_CUDA_TRY(metis_launch_pdl((sample_rows_kernel), dim3((unsigned)metis_ceil_div(n_s, 256)), dim3(256), (size_t)(0), s, idx, (int)n_s, rows, seed, 0)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((sample_rows_kernel), dim3((unsigned)metis_ceil_div(n_s, 256)), dim3(256), (size_t)(0), s, idx, (int)n_s, rows, seed, 0,
+                                    (float*)nullptr, (unsigned long long*)nullptr)); METIS_COUNT_LAUNCH();
     METIS_CUDA_TRY(metis_launch_pdl(metis_wide::gather_rows_kernel, dim3((unsigned)metis_ceil_div(n_s * (cols / 8), 256)), dim3(256), (size_t)0, s, x, cols,
                                     (const int*)idx, (int)n_s, xs)); METIS_COUNT_LAUNCH();
     xr = xs;
@@ -1530,6 +1596,10 @@ int64_t metis_default_sample_count(int64_t rows, int32_t q) {
 
 metis_status_t metis_split_set_attrs() {
   using namespace metis_qt;
+#define METIS_FR_ATTR(KT) METIS_CUDA_TRY(cudaFuncSetAttribute(basis_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fr_smem(MAXQ))); \
+  METIS_CUDA_TRY(cudaFuncSetAttribute(factors_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fr_smem(MAXQ)))
+  METIS_FR_ATTR(1); METIS_FR_ATTR(2); METIS_FR_ATTR(3); METIS_FR_ATTR(4); METIS_FR_ATTR(5); METIS_FR_ATTR(6); METIS_FR_ATTR(7); METIS_FR_ATTR(8);
+#undef METIS_FR_ATTR
 #define METIS_EIG_ATTR(NT8) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_small::eig_kernel<NT8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_small::eig_smem(8 * NT8)))
   METIS_EIG_ATTR(1); METIS_EIG_ATTR(2); METIS_EIG_ATTR(3); METIS_EIG_ATTR(4); METIS_EIG_ATTR(5); METIS_EIG_ATTR(6); METIS_EIG_ATTR(7); METIS_EIG_ATTR(8); METIS_EIG_ATTR(9);
 #undef METIS_EIG_ATTR
@@ -1692,9 +1762,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   float* m = reinterpret_cast<float*>(wsb + L.m);
   float* basis = reinterpret_cast<float*>(wsb + L.basis);
   float* coef = reinterpret_cast<float*>(wsb + L.coef);
-  float* sign = reinterpret_cast<float*>(wsb + L.sign);
-  float* cand_v = reinterpret_cast<float*>(wsb + L.cand_v);
-  int* cand_i = reinterpret_cast<int*>(wsb + L.cand_i);
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(wsb + L.keys);          // sign contest, one per vector
   double* evals2 = reinterpret_cast<double*>(wsb + L.evals2);
   double* evecs2 = reinterpret_cast<double*>(wsb + L.evecs2);
   __nv_bfloat16* bs = reinterpret_cast<__nv_bfloat16*>(wsb + L.bs);
@@ -1712,12 +1780,11 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   bool a6_ready = false;
   metis_context* ctx = h;
   const int kp = (k + 15) / 16 * 16;
-  // amax|x| for the residual's tensor scale: fused into the sketch pass (FULL) or the broadcast pass (SAMPLED)
-  METIS_CUDA_TRY(cudaMemsetAsync(amax, 0, 64, s));       // amax slots of x, left, right and the condition flag
+  // (1) row sample (clears the amax slots of x, left and right, the condition flag and the sign keys), (2) sketch (tensor cores; Omega
+  // generated per CTA into shared memory).  amax|x| for the residual's tensor scale: fused into the sketch pass (FULL) or
+  // the broadcast pass (SAMPLED).
+  METIS_CUDA_TRY(metis_launch_pdl((sample_rows_kernel), dim3((unsigned)metis_ceil_div(n_s, 256)), dim3(256), (size_t)(0), s, idx, (int)n_s, rows, seed, full ? 1 : 0, amax, keys)); METIS_COUNT_LAUNCH();
   if (src_amax != nullptr) METIS_CUDA_TRY(cudaMemcpyAsync(amax, src_amax, sizeof(float), cudaMemcpyDeviceToDevice, s));
-
-  // (1) row sample, (2) sketch (tensor cores; Omega generated per CTA into shared memory)
-  METIS_CUDA_TRY(metis_launch_pdl((sample_rows_kernel), dim3((unsigned)metis_ceil_div(n_s, 256)), dim3(256), (size_t)(0), s, idx, (int)n_s, rows, seed, full ? 1 : 0)); METIS_COUNT_LAUNCH();
   const int ccols = sketch_chunk_cols(n_s);
   const int chunks = (int)metis_ceil_div(cols, ccols);
   __nv_bfloat16* omt = reinterpret_cast<__nv_bfloat16*>(wsb + L.omt);
@@ -1824,20 +1891,21 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(q * q, 32)), dim3(128), (size_t)(0), s, gram, parts, q * q, gram1, nullptr)); METIS_COUNT_LAUNCH();
     METIS_TRY(launch_eig(s, gram1, q, q, evals, evecs));
   }
-  METIS_CUDA_TRY(metis_launch_pdl((right_basis_kernel), dim3((unsigned)metis_ceil_div(cols, RB_COLS)), dim3(256), (size_t)(0), s, m, cols, q, k, evals, evecs, basis,
-                                                                          full ? out->sigma : nullptr)); METIS_COUNT_LAUNCH();
-  // (5) coefficients of every row in the basis, (6) fused residual + quantizer
-  const int n_cand = (int)metis_ceil_div(cols, 256);
+  // (5) right basis and its splits; coefficients of every row in the basis, (6) fused residual + quantizer
   const int n_cta_c = (int)metis_ceil_div(rows, 32);
+  const int n_cta_cols = (int)metis_ceil_div(cols, FR_POS), n_cta_rows = (int)metis_ceil_div(rows, FR_POS);
+  float* rb = full ? out->right : basis;
+  __nv_bfloat16* btp = resid_tc ? nullptr : bt;
+  METIS_TRY(launch_basis(s, n_cta_cols, fr_smem(q), m, cols, q, k, kp, evals, evecs, rb, full ? (__nv_bfloat16*)nullptr : bs, btp, b6p, kx6, full ? out->sigma : nullptr, full ? keys : nullptr, amax + 2));
   if (full) {
-    // left = H U~_k, right = basis (sign fixed); coefficients = left * sigma
-    METIS_CUDA_TRY(metis_launch_pdl((right_rotate_kernel), dim3(dim3(n_cand, (k + 7) / 8)), dim3(256), (size_t)(0), s, basis, cols, k, nullptr, out->right, cand_v, cand_i)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((sign_fix_kernel), dim3(dim3(n_cand, k)), dim3(256), (size_t)(0), s, out->right, cols, k, cand_v, cand_i, n_cand, sign, amax + 2)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((basis_splits_kernel), dim3((unsigned)metis_ceil_div(cols, 128), (unsigned)(kp / 8)), dim3(128), (size_t)(0), s, out->right, cols, k, kp, bs, bt, b6p, kx6)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((left_rotate_kernel), dim3(dim3((unsigned)metis_ceil_div(rows, 64), (unsigned)((kp + 15) / 16))), dim3(256), (size_t)(0), s, z, rows, q, k, 1, q, evecs, nullptr, sign,
-                                                                            out->left, nullptr, coef, kp, out->sigma, amax + 1)); METIS_COUNT_LAUNCH();
+    // left = H U~_k; coefficients = left * sigma, as the residual product's operand where the tensor-core pass runs
+    FactorsArgs f{};
+    f.w = evecs; f.ldw = q; f.n_in = q; f.k = k; f.kp = kp;
+    f.src = z; f.ld = q; f.rows = rows; f.left = out->left; f.amax_left = amax + 1;
+    f.sigma_for_coef = out->sigma; f.coef = coef; f.a6 = a6p; f.kx = kx6;
+    METIS_TRY(launch_factors(s, f, 0, n_cta_rows));
+    a6_ready = resid_tc;
   } else {
-    METIS_CUDA_TRY(metis_launch_pdl((basis_splits_kernel), dim3((unsigned)metis_ceil_div(cols, 128), (unsigned)(kp / 8)), dim3(128), (size_t)(0), s, basis, cols, k, kp, bs, bt, b6p, kx6)); METIS_COUNT_LAUNCH();
     if (metis_coeff_tc_usable(x, bs, cols, kp)) {
       // tensor-core pass over x (column slices), then the slices are summed and the Gram partials formed
       METIS_TRY(metis_launch_coeff_tc(ctx, x, rows, cols, bs, kp, part, amax, 0, s));
@@ -1891,15 +1959,16 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     // (7) Rayleigh-Ritz on C^T C (Gram partials came out of the broadcast pass), rotate both factors
     METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(kp * kp, 32)), dim3(128), (size_t)(0), sf, gram_c, n_cta_c, kp * kp, gram1, nullptr)); METIS_COUNT_LAUNCH();
     METIS_TRY(launch_eig(sf, gram1, k, kp, evals2, evecs2));
-    METIS_CUDA_TRY(metis_launch_pdl((right_rotate_kernel), dim3(dim3(n_cand, (k + 7) / 8)), dim3(256), (size_t)(0), sf, basis, cols, k, evecs2, out->right, cand_v, cand_i)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((sign_fix_kernel), dim3(dim3(n_cand, k)), dim3(256), (size_t)(0), sf, out->right, cols, k, cand_v, cand_i, n_cand, sign, amax + 2)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((left_rotate_kernel), dim3(dim3((unsigned)metis_ceil_div(rows, 64), (unsigned)((kp + 15) / 16))), dim3(256), (size_t)(0), sf, coef, rows, k, k, 1, kp, evecs2, evals2, sign,
-                                                                            out->left, out->sigma, nullptr, kp, nullptr, amax + 1)); METIS_COUNT_LAUNCH();
+    FactorsArgs f{};
+    f.w = evecs2; f.ldw = k; f.n_in = k; f.k = k; f.kp = kp;
+    f.basis = basis; f.cols = cols; f.right = out->right; f.keys = keys; f.amax_right = amax + 2;
+    f.src = coef; f.ld = kp; f.rows = rows; f.evals = evals2; f.left = out->left; f.sigma_out = out->sigma; f.amax_left = amax + 1;
+    METIS_TRY(launch_factors(sf, f, n_cta_cols, n_cta_rows));
   }
   METIS_CUDA_TRY(cudaGetLastError());
-  // (8) quantize the factors (stored transposed: k x rows, k x cols; blocks along the long dimension)
+  // (8) apply the sign convention and quantize the factors (stored transposed: k x rows, k x cols; blocks along the long dimension)
   metis_nvfp4_t lq = out->left_q, rq = out->right_q;
   lq.rows = k; lq.k_len = rows; rq.rows = k; rq.k_len = cols;
-  METIS_TRY(metis_launch_quantize_factors(out->left, rows, out->right, cols, k, rounding, seed, amax + 1, amax + 2, &lq, &rq, sf));
+  METIS_TRY(metis_launch_quantize_factors(out->left, rows, out->right, cols, k, rounding, seed, amax + 1, amax + 2, &lq, &rq, sf, keys));
   return metis_join(ctx, s, 0);
 }
