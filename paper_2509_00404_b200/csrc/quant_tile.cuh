@@ -79,29 +79,40 @@ __device__ __forceinline__ uint32_t e2m1x8_rne(float a0, float a1, float a2, flo
   return w;
 }
 
-// Eight stochastically rounded codes in one word; thr[i] = draw_i << 16.  The same decision as metis_e2m1_sr,
-// arranged for the instruction mix of the SM (integer logic and compares issue at half the FP32 / IMAD rate):
+// What a 16-bit draw u contributes to the rounding of its element: (65535 - u) * 256 + 255, one byte permutation of the
+// COMPLEMENTED Philox word that holds the draw in its low (hi = false) or high half.
+__device__ __forceinline__ uint32_t sr_addend(uint32_t not_word, bool hi) { return __byte_perm(not_word, 0xFFu, hi ? 0x5324u : 0x5104u); }
+__device__ __forceinline__ uint32_t sr_addend16(uint32_t u16) { return ((~u16 & 0xFFFFu) << 8) | 0xFFu; }
+
+// Eight stochastically rounded codes in one word; add[i] = sr_addend of draw i.  The same decision as metis_e2m1_sr,
+// arranged for the instruction mix of the SM (integer logic, shifts and compares issue at half the FP32 / IMAD rate, and bound
+// this code):
 //   b = max(a, RU(a/2 + 1/2)) maps a < 1 onto [1/2, 1] (the E2M1 grid {0, 1/2, 1} becomes {1/2, 3/4, 1}: one
 //       mantissa bit per binade like the values from 1 up) and leaves a >= 1 alone, without a select;
-//   up = (bits(b) << 10) > thr compares the 22 mantissa bits below the grid bit with the draw, no masks;
-//   the magnitude code is (bits(b) >> 22) - 252 + up; the eight "- 252" are taken off the packed word at once;
+//   4 bits(b) + add: the 22 mantissa bits below the grid bit carry into it exactly when  frac * 65536 > u  (4 frac22 + (65535 - u) 256 +
+//       255 >= 2^24  <=>  frac22 > 64 u): comparison, selection and increment in one multiply-add;
+//   the magnitude code is then bits 24 .. 26, minus 4 modulo 8: the top bytes of four elements are gathered by byte permutations, the
+//       two words of even and odd elements are merged and the eight "- 4" taken off together;
 //   the sign nibbles are gathered with one funnel shift per element and masked once per word.
-__device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_t (&thr)[8]) {
-  uint32_t mag = 0u, sgn = 0u;
+// (Against a compare per element with the draw shifted up and codes packed one by one: quantize_kernel 472 -> 383 us at 16384 x 14336 with
+// both orientations, residual_tc_kernel 1060 -> 866 us at 16384 x 28672, k = 64.)
+__device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_t (&add)[8]) {
+  uint32_t s[8], sgn = 0u;
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
     const float a = fminf(fabsf(y[i]), 6.0f);
-    const uint32_t bits = __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f)));
-    const uint32_t t = (bits >> 22) + (((bits << 10) > thr[i]) ? 1u : 0u);
-    mag = mag * 16u + t;                                   // modulo 2^32: the excess of 252 per nibble is removed below
+    s[i] = __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f))) * 4u + add[i];
     sgn = __funnelshift_l(__float_as_uint(y[i]), sgn, 4);  // top nibble of y (sign and three exponent bits) shifted in
   }
-  return (mag - 252u * 0x11111111u) | (sgn & 0x88888888u);
+  const uint32_t even = __byte_perm(__byte_perm(s[0], s[2], 0x0073u), __byte_perm(s[4], s[6], 0x7300u), 0x7610u);
+  const uint32_t odd = __byte_perm(__byte_perm(s[1], s[3], 0x0073u), __byte_perm(s[5], s[7], 0x7300u), 0x7610u);
+  const uint32_t mag = ((even & 0x0F0F0F0Fu) | ((odd * 16u) & 0xF0F0F0F0u));
+  return ((mag & 0x77777777u) ^ 0x44444444u) | (sgn & 0x88888888u);
 }
 
 // encode_block with the multiplier looked up in a table filled by fill_r_table (same bytes as encode_block).
-// thr[i] = draw_i << 16 (only read with stochastic rounding).
-__device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&thr)[16], bool sr, float six_s_T,
+// add[i] = sr_addend of draw i (only read with stochastic rounding).
+__device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&add)[16], bool sr, float six_s_T,
                                                      const float* r_tab, uint32_t (&packed)[2]) {
   float m8[8];
 #pragma unroll
@@ -120,7 +131,7 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
     float y0[8], y1[8];
     uint32_t t0[8], t1[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { y0[i] = __fmul_rn(v[i], r); y1[i] = __fmul_rn(v[8 + i], r); t0[i] = thr[i]; t1[i] = thr[8 + i]; }
+    for (int i = 0; i < 8; ++i) { y0[i] = __fmul_rn(v[i], r); y1[i] = __fmul_rn(v[8 + i], r); t0[i] = add[i]; t1[i] = add[8 + i]; }
     packed[0] = e2m1x8_sr(y0, t0);
     packed[1] = e2m1x8_sr(y1, t1);
   }

@@ -79,10 +79,12 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
   extern __shared__ __align__(16) unsigned char smem[];
   T* tile = reinterpret_cast<T*>(smem);                                        // [TILE][TP]
   uint8_t* codes_s = smem + ((sizeof(T) * TILE * TP + 15) & ~(size_t)15);      // [TILE][QK_CP] row-block codes
-  uint8_t* sfr = codes_s + TILE * QK_CP;                                       // [TILE][8] scales of the row blocks
-  uint8_t* sfc = sfr + TILE * 8;                                               // [TILE][8] scales of the column blocks
+  // [TILE][8] scales of the column blocks, written out before pass 2 puts those of the row blocks in their place: with
+  // an area for each, two CTAs of the stochastic-rounding kernel fitted an SM instead of three
+  uint8_t* sfc = codes_s + TILE * QK_CP;
+  uint8_t* sfr = sfc;
   float* r_tab = reinterpret_cast<float*>(sfc + TILE * 8);                     // multiplier per scale byte
-  uint16_t* rnd = reinterpret_cast<uint16_t*>(r_tab + R_TABLE);                // [TILE][TILE] draws (SR only)
+  uint16_t* rnd = reinterpret_cast<uint16_t*>(r_tab + R_TABLE);                // [TILE][TILE] complemented draws (SR only)
 
   auto staged_row = [](int c) { return sizeof(T) == 2 ? (c >> 1) + 64 * (c & 1) : c; };
   // Scale bytes of the tile, from their staging area [stored row][8] to global memory.  The four blocks of a 64-element
@@ -184,26 +186,34 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       }
     }
     if (sr) {
+      uint32_t nw[8];                                      // complemented draws, two per word
       if (fast_draws && in) {
         const uint64_t e = (uint64_t)gr * (uint64_t)p.e_stride_r + (uint64_t)gc;
         const uint4 w0 = metis_philox_block(e >> 3, p.seed, p.stream_id), w1 = metis_philox_block((e >> 3) + 1, p.seed, p.stream_id);
-        const uint32_t ww[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
+        const uint32_t ww[8] = {~w0.x, ~w0.y, ~w0.z, ~w0.w, ~w1.x, ~w1.y, ~w1.z, ~w1.w};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) { u[2 * j] = ww[j] << 16; u[2 * j + 1] = ww[j] & 0xFFFF0000u; }   // thresholds: draw << 16
+        for (int j = 0; j < 8; ++j) nw[j] = ww[j];
       } else {
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          u[j] = in ? metis_draw_u16((uint64_t)gr * (uint64_t)p.e_stride_r + (uint64_t)(gc + j) * (uint64_t)p.e_stride_c, p.seed, p.stream_id) << 16 : 0u;
+        for (int j = 0; j < 8; ++j) {
+          uint32_t d[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            d[h] = in ? metis_draw_u16((uint64_t)gr * (uint64_t)p.e_stride_r + (uint64_t)(gc + 2 * j + h) * (uint64_t)p.e_stride_c, p.seed, p.stream_id) : 0u;
+          nw[j] = ~(d[0] | (d[1] << 16));
+        }
       }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) { u[2 * j] = sr_addend(nw[j], false); u[2 * j + 1] = sr_addend(nw[j], true); }
       if (want_r) {
         if (sizeof(T) == 2) {
           uint4* drow = reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(rnd) + r * 256);
-          drow[(2 * b) ^ (b >> 2)] = make_uint4((u[0] >> 16) | u[1], (u[2] >> 16) | u[3], (u[4] >> 16) | u[5], (u[6] >> 16) | u[7]);
-          drow[(2 * b + 1) ^ (b >> 2)] = make_uint4((u[8] >> 16) | u[9], (u[10] >> 16) | u[11], (u[12] >> 16) | u[13], (u[14] >> 16) | u[15]);
+          drow[(2 * b) ^ (b >> 2)] = make_uint4(nw[0], nw[1], nw[2], nw[3]);
+          drow[(2 * b + 1) ^ (b >> 2)] = make_uint4(nw[4], nw[5], nw[6], nw[7]);
         } else {
           uint32_t* dst = reinterpret_cast<uint32_t*>(rnd + r * TILE + b * 16);
 #pragma unroll
-          for (int j = 0; j < 8; ++j) dst[j] = (u[2 * j] >> 16) | u[2 * j + 1];
+          for (int j = 0; j < 8; ++j) dst[j] = nw[j];
         }
       }
     }
@@ -215,8 +225,10 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
     }
   }
   __syncthreads();
+  if (want_c) write_scales(p.c_scales, p.c_sf_bytes, p.c_layout, p.cols / 16, sfc, false, vrows, vcols, row0, col0 / 16);
   // ---- pass 2 ----
   if (want_r) {
+    __syncthreads();                                       // the column blocks' scales have been read
     if (sizeof(T) == 2) {
       // BF16 tile: a thread takes two adjacent columns (one 32-bit shared load per row) and four of the eight
       // row blocks, i.e. eight blocks in two rounds of four
@@ -235,7 +247,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const uint32_t w = reinterpret_cast<const uint32_t*>(rnd)[(b * 16 + i) * 64 + pw];
-            u0[i] = w << 16; u1[i] = w & 0xFFFF0000u;
+            u0[i] = sr_addend(w, false); u1[i] = sr_addend(w, true);
           }
         }
         uint32_t packed[2];
@@ -256,7 +268,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       for (int i = 0; i < 16; ++i) v[i] = reinterpret_cast<const float*>(tile)[(b * 16 + i) * TP + c];
       if (sr) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) u[i] = (uint32_t)rnd[(b * 16 + i) * TILE + c] << 16;
+        for (int i = 0; i < 16; ++i) u[i] = sr_addend((uint32_t)rnd[(b * 16 + i) * TILE + c], false);
       }
       uint32_t packed[2];
       const uint32_t byte = encode_block_tab(v, u, sr, six_s_T, r_tab, packed);
@@ -273,13 +285,12 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
     }
     write_scales(p.r_scales, p.r_sf_bytes, p.r_layout, p.rows / 16, sfr, true, vcols, vrows, col0, row0 / 16);
   }
-  if (want_c) write_scales(p.c_scales, p.c_sf_bytes, p.c_layout, p.cols / 16, sfc, false, vrows, vcols, row0, col0 / 16);
 }
 
 template <typename T>
 constexpr size_t quantize_smem(bool sr) {
   return ((sizeof(T) * metis_qt::TILE * (metis_qt::TILE + (sizeof(T) == 2 ? 0 : 1)) + 15) & ~(size_t)15) + metis_qt::TILE * QK_CP +
-         2 * metis_qt::TILE * 8 + sizeof(float) * metis_qt::R_TABLE + (sr ? sizeof(uint16_t) * metis_qt::TILE * metis_qt::TILE : 0);
+         metis_qt::TILE * 8 + sizeof(float) * metis_qt::R_TABLE + (sr ? sizeof(uint16_t) * metis_qt::TILE * metis_qt::TILE : 0);
 }
 
 }  // namespace

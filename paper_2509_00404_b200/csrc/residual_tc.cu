@@ -33,7 +33,7 @@ constexpr int X_BYTES = TM * TN * 2;                      // two 64-column boxes
 constexpr int N_EW = 16;                                  // epilogue warps: four TMEM lane quarters x four column quarters
 constexpr int PATCH_HALF = 16 * 20 + 16;                   // 16 rows of 20 floats; the second half starts 16 banks further
 constexpr int PATCH_F = 2 * PATCH_HALF;                   // floats per warp patch (32 rows x 16 columns)
-constexpr int PATCH_U = 32 * 18;                          // 16-bit draws per warp patch
+constexpr int PATCH_U = 2 * 336;                          // complemented 16-bit draws per warp patch: 32 rows of 20, the second 16 rows 32 further
 constexpr int NUM_THREADS = 64 + 32 * N_EW;               // producer, MMA issuer, epilogue warps
 constexpr size_t SMEM_BYTES = (size_t)RING * SLOT_BYTES + 2 * X_BYTES + N_EW * (PATCH_F * 4 + PATCH_U * 2) + 1024 + 256 + metis_qt::R_TABLE * 4;
 
@@ -177,7 +177,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     const int ew = warp - 2;                                // 0..15
     const int quarter = warp & 3, colq = ew >> 2;           // TMEM lane quarter (fixed by the warp id), column quarter
     float* patch = reinterpret_cast<float*>(gen_base + patch_off) + ew * PATCH_F;
-    uint16_t* upatch = reinterpret_cast<uint16_t*>(gen_base + patch_off + N_EW * PATCH_F * 4) + ew * PATCH_U;
+    uint32_t* upatch = reinterpret_cast<uint32_t*>(gen_base + patch_off + N_EW * PATCH_F * 4) + ew * (PATCH_U / 2);
     constexpr bool sr = SR;
     const int c_layout = FAST ? (int)METIS_SF_TILED : p.c_layout, r_layout = FAST ? (int)METIS_SF_TILED : p.r_layout;
     const float s_T = metis_tensor_scale(*g.amax_src);
@@ -232,7 +232,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       if (lane == 0) { mbar_arrive(tempty_bar(acc)); mbar_arrive(xempty_bar(xb)); }
       const bool step_ok = FAST || c0 < p.cols;                                      // false: the warp's columns lie outside the matrix
       const bool blk1_ok = FAST || c0 + 16 < p.cols;
-      uint32_t u[32];
+      uint32_t nw[16];                                      // complemented draws, two per word
       if (sr) {
         const uint64_t e0 = (uint64_t)row * (uint64_t)p.e_stride_r + (uint64_t)c0;        // multiple of 8
 #pragma unroll
@@ -240,7 +240,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           const uint4 w = metis_philox_block((e0 >> 3) + q4, p.seed, p.stream_id);
           const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) { u[8 * q4 + 2 * j] = ww[j] << 16; u[8 * q4 + 2 * j + 1] = ww[j] & 0xFFFF0000u; }   // thresholds: draw << 16
+          for (int j = 0; j < 4; ++j) nw[4 * q4 + j] = ~ww[j];
         }
       }
       if (!FAST && g.dense != nullptr && row_ok && step_ok) {
@@ -255,7 +255,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         float v0[16], v1[16];
         uint32_t u0[16], u1[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? u[i] : 0u; u1[i] = sr ? u[16 + i] : 0u; }
+        for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? metis_qt::sr_addend(nw[i >> 1], i & 1) : 0u; u1[i] = sr ? metis_qt::sr_addend(nw[8 + (i >> 1)], i & 1) : 0u; }
         uint32_t pk0[2], pk1[2];
         const uint32_t sb0 = encode_block_tab(v0, u0, sr, six_s_T, r_tab, pk0);
         const uint32_t sb1 = encode_block_tab(v1, u1, sr, six_s_T, r_tab, pk1);
@@ -281,6 +281,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         // blocks along the rows: the warp transposes its 32 x 32 values 16 columns at a time through its patch;
         // in each half lane l encodes the block of column l % 16, rows 16 * (l / 16) .. +15
         const int cb = lane & 15, rb = lane >> 4;
+        const uint32_t add_sel = (cb & 1) ? 0x5324u : 0x5104u;
         const bool rb_ok = FAST || slab_row0 + 16 * rb < p.rows;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
@@ -292,7 +293,8 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           }
           if (sr) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) upatch[lane * 18 + i] = (uint16_t)(u[16 * hf + i] >> 16);
+            for (int i = 0; i < 4; ++i)                     // rows of ten words, 8-byte stores: a half warp covers all banks
+              *reinterpret_cast<uint2*>(upatch + lane * 10 + (lane >> 4) * 16 + 2 * i) = make_uint2(nw[8 * hf + 2 * i], nw[8 * hf + 2 * i + 1]);
           }
           __syncwarp();
           const int64_t col = c0 + 16 * hf + cb;
@@ -302,7 +304,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             t[i] = patch[rb * PATCH_HALF + i * 20 + cb];
-            d[i] = sr ? (uint32_t)upatch[(16 * rb + i) * 18 + cb] << 16 : 0u;
+            d[i] = sr ? __byte_perm(upatch[rb * 176 + i * 10 + (cb >> 1)], 0xFFu, add_sel) : 0u;   // sr_addend of this column's half
           }
           uint32_t pk[2];
           const uint32_t sb = encode_block_tab(t, d, sr, six_s_T, r_tab, pk);
