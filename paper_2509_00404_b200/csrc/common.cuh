@@ -111,6 +111,26 @@ __device__ __forceinline__ uint4 metis_philox(uint32_t c0, uint32_t c1, uint32_t
   return make_uint4(c0, c1, c2, c3);
 }
 
+// The same draws for the kernels that make one per element: the round keys come ready from the kernel's parameters (an operand
+// of the exclusive-or instead of an addition per round and word) and a multiplication gives both halves at once.
+struct PhiloxKeys { uint32_t k0[10], k1[10]; };
+__host__ inline PhiloxKeys metis_philox_keys(uint64_t seed) {
+  PhiloxKeys k;
+  uint32_t a = (uint32_t)seed, b = (uint32_t)(seed >> 32);
+  for (int r = 0; r < 10; ++r) { k.k0[r] = a; k.k1[r] = b; a += 0x9E3779B9u; b += 0xBB67AE85u; }
+  return k;
+}
+__device__ __forceinline__ uint4 metis_philox_block_keys(uint64_t block_index, const PhiloxKeys& k, uint32_t stream) {
+  uint32_t c0 = (uint32_t)block_index, c1 = (uint32_t)(block_index >> 32), c2 = stream, c3 = 0u;
+#pragma unroll
+  for (int r = 0; r < 10; ++r) {
+    const uint64_t p0 = (uint64_t)0xD2511F53u * c0, p1 = (uint64_t)0xCD9E8D57u * c2;
+    c0 = (uint32_t)(p1 >> 32) ^ c1 ^ k.k0[r]; c2 = (uint32_t)(p0 >> 32) ^ c3 ^ k.k1[r];
+    c1 = (uint32_t)p1; c3 = (uint32_t)p0;
+  }
+  return make_uint4(c0, c1, c2, c3);
+}
+
 __device__ __forceinline__ uint4 metis_philox_block(uint64_t block_index, uint64_t seed, uint32_t stream) {
   return metis_philox((uint32_t)block_index, (uint32_t)(block_index >> 32), stream, 0u, (uint32_t)seed,
                       (uint32_t)(seed >> 32));

@@ -22,6 +22,7 @@ struct QuantParams {
   // debug build: extents of the scale buffers (the code buffers hold rows * cols / 2 bytes) and the status word
   int64_t c_sf_bytes, r_sf_bytes;
   uint32_t* dbg;
+  PhiloxKeys keys;                    // round keys of `seed` (filled where the element draws are made in bulk)
 };
 
 struct __align__(16) Stage {

@@ -63,7 +63,7 @@ amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, 
 //          stages the bytes; the transposed codes and both scale tiles are then written out coalesced
 constexpr int QK_CP = metis_qt::TILE / 2 + 8;                     // pitch of a staged row of row-block codes, bytes
 template <typename T, bool SR>   // T = __nv_bfloat16 or float: element type of the shared tile (= input type)
-__global__ void __launch_bounds__(metis_qt::THREADS, SR ? 3 : 4)
+__global__ void __launch_bounds__(metis_qt::THREADS, sizeof(T) == 4 ? (SR ? 2 : 3) : (SR ? 3 : 4))    // as many CTAs as their shared memory allows
 quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, const float* __restrict__ tscale_src,
                 int tscale_is_amax, float* ts_out0, float* ts_out1) {
   using namespace metis_qt;
@@ -71,14 +71,16 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
   //   BF16 tile and draws: rows of 256 bytes = 16 chunks of 16 bytes, chunk ch stored at ch ^ (ch >> 3): the eight
   //     lanes of a quarter warp store the even (or odd) chunks of one row, which the swizzle spreads over all banks;
   //     pass 2 reads 32 consecutive words of a row, a permutation of the chunks inside one 128-byte window.
-  //   FP32 tile: pitch 129 words.
+  //   FP32 tile: rows of 512 bytes = 32 chunks of 16 bytes, chunk ch stored at ch ^ (ch >> 3): the eight lanes of a quarter warp store
+  //     every fourth chunk of a row onto all banks; pass 2 reads 32 consecutive columns, a permutation inside one 128-byte window.
+  //     (Element stores into rows of 129 words met four to a bank; with them and unpipelined loads: 100 us at 14336 x 4096, 71 us now.)
   //   staged row-block codes: 72-byte rows; a BF16 thread owns two adjacent columns, so column c is staged in row
   //     (c >> 1) + 64 (c & 1) and the 32 lanes of a store write 32 consecutive rows (18 words apart: 16 lanes cover
   //     the 32 banks with their 8 bytes each).
-  constexpr int TP = sizeof(T) == 2 ? TILE : TILE + 1;           // tile pitch in elements
+  constexpr int TP = TILE;                                       // tile pitch in elements
   extern __shared__ __align__(16) unsigned char smem[];
   T* tile = reinterpret_cast<T*>(smem);                                        // [TILE][TP]
-  uint8_t* codes_s = smem + ((sizeof(T) * TILE * TP + 15) & ~(size_t)15);      // [TILE][QK_CP] row-block codes
+  uint8_t* codes_s = smem + sizeof(T) * TILE * TP;                             // [TILE][QK_CP] row-block codes
   // [TILE][8] scales of the column blocks, written out before pass 2 puts those of the row blocks in their place: with
   // an area for each, two CTAs of the stochastic-rounding kernel fitted an SM instead of three
   uint8_t* sfc = codes_s + TILE * QK_CP;
@@ -149,6 +151,16 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       }
     }
   }
+  // FP32: the block of the next round is loaded while this round's is encoded
+  float4 nxt[sizeof(T) == 4 ? 4 : 1];
+  auto load_fp32 = [&](int it) {
+    const int b = tid & 7, r = (tid >> 3) + 32 * it;
+    const bool in = r < vrows && b * 16 < vcols;
+    const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(x) + (row0 + r) * ld + col0 + b * 16);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) nxt[sizeof(T) == 4 ? j : 0] = in ? src[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  };
+  if (sizeof(T) == 4) load_fp32(0);
   __syncthreads();                                         // multiplier table complete (the tile loads are in flight)
 #pragma unroll
   for (int it = 0; it < 4; ++it) {
@@ -167,29 +179,22 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
         trow[(2 * b) ^ (b >> 2)] = q0;
         trow[(2 * b + 1) ^ (b >> 2)] = q1;
       }
-    } else if (in) {
-      const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(x) + gr * ld + gc);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { const float4 q = src[j]; v[4 * j] = q.x; v[4 * j + 1] = q.y; v[4 * j + 2] = q.z; v[4 * j + 3] = q.w; }
-      if (want_r) {
-        float* dst = reinterpret_cast<float*>(tile) + r * TP + b * 16;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) dst[j] = v[j];
-      }
     } else {
+      float4 q[4];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = 0.0f;
+      for (int j = 0; j < 4; ++j) { q[j] = nxt[sizeof(T) == 4 ? j : 0]; v[4 * j] = q[j].x; v[4 * j + 1] = q[j].y; v[4 * j + 2] = q[j].z; v[4 * j + 3] = q[j].w; }
+      if (it < 3) load_fp32(it + 1);
       if (want_r) {
-        T* dst = tile + r * TP + b * 16;
+        float4* trow = reinterpret_cast<float4*>(smem + r * 512);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) dst[j] = T(0.0f);
+        for (int j = 0; j < 4; ++j) trow[(4 * b + j) ^ (b >> 1)] = q[j];
       }
     }
     if (sr) {
       uint32_t nw[8];                                      // complemented draws, two per word
       if (fast_draws && in) {
         const uint64_t e = (uint64_t)gr * (uint64_t)p.e_stride_r + (uint64_t)gc;
-        const uint4 w0 = metis_philox_block(e >> 3, p.seed, p.stream_id), w1 = metis_philox_block((e >> 3) + 1, p.seed, p.stream_id);
+        const uint4 w0 = metis_philox_block_keys(e >> 3, p.keys, p.stream_id), w1 = metis_philox_block_keys((e >> 3) + 1, p.keys, p.stream_id);
         const uint32_t ww[8] = {~w0.x, ~w0.y, ~w0.z, ~w0.w, ~w1.x, ~w1.y, ~w1.z, ~w1.w};
 #pragma unroll
         for (int j = 0; j < 8; ++j) nw[j] = ww[j];
@@ -265,7 +270,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       float v[16];
       uint32_t u[16];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = reinterpret_cast<const float*>(tile)[(b * 16 + i) * TP + c];
+      for (int i = 0; i < 16; ++i) v[i] = reinterpret_cast<const float*>(tile)[(b * 16 + i) * TP + (((c >> 2) ^ (c >> 5)) << 2 | (c & 3))];
       if (sr) {
 #pragma unroll
         for (int i = 0; i < 16; ++i) u[i] = sr_addend((uint32_t)rnd[(b * 16 + i) * TILE + c], false);
@@ -289,7 +294,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
 
 template <typename T>
 constexpr size_t quantize_smem(bool sr) {
-  return ((sizeof(T) * metis_qt::TILE * (metis_qt::TILE + (sizeof(T) == 2 ? 0 : 1)) + 15) & ~(size_t)15) + metis_qt::TILE * QK_CP +
+  return sizeof(T) * metis_qt::TILE * metis_qt::TILE + metis_qt::TILE * QK_CP +
          metis_qt::TILE * 8 + sizeof(float) * metis_qt::R_TABLE + (sr ? sizeof(uint16_t) * metis_qt::TILE * metis_qt::TILE : 0);
 }
 
@@ -495,6 +500,7 @@ metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int
   QuantParams p{};
   p.rows = rows; p.cols = cols; p.rounding = rounding; p.seed = seed; p.stream_id = stream_id;
   p.e_stride_r = e_stride_r; p.e_stride_c = e_stride_c;
+  p.keys = metis_philox_keys(seed);
   if (by_cols) { p.c_codes = by_cols->codes; p.c_scales = by_cols->scales; p.c_layout = by_cols->sf_layout; p.c_sf_bytes = (int64_t)metis_sf_bytes(rows, cols, p.c_layout); }
   if (by_rows) { p.r_codes = by_rows->codes; p.r_scales = by_rows->scales; p.r_layout = by_rows->sf_layout; p.r_sf_bytes = (int64_t)metis_sf_bytes(cols, rows, p.r_layout); }
   p.dbg = dbg_status;

@@ -237,7 +237,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         const uint64_t e0 = (uint64_t)row * (uint64_t)p.e_stride_r + (uint64_t)c0;        // multiple of 8
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4) {
-          const uint4 w = metis_philox_block((e0 >> 3) + q4, p.seed, p.stream_id);
+          const uint4 w = metis_philox_block_keys((e0 >> 3) + q4, p.keys, p.stream_id);
           const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
           for (int j = 0; j < 4; ++j) nw[4 * q4 + j] = ~ww[j];
@@ -365,6 +365,7 @@ metis_status_t metis_launch_residual_tc(metis_context* ctx, const void* x, const
   METIS_TRY(make_map_bf16(ctx, &mb, b6, cols, kx, kx, TN));
   ResidArgs g{};
   g.p = qp;
+  g.p.keys = metis_philox_keys(qp.seed);
   g.p.c_sf_bytes = qp.c_codes ? (int64_t)metis_sf_bytes(rows, cols, qp.c_layout) : 0;
   g.p.r_sf_bytes = qp.r_codes ? (int64_t)metis_sf_bytes(cols, rows, qp.r_layout) : 0;
   g.amax_src = amax_src; g.ts_out0 = ts_out0; g.ts_out1 = ts_out1; g.dense = dense;
