@@ -78,7 +78,8 @@ splits6_kernel(const float* __restrict__ src, int64_t n, int k, int kp, int kx, 
 template <bool SR, bool FAST>
 __global__ void __launch_bounds__(NUM_THREADS, 1)
 residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_a,
-                   const __grid_constant__ CUtensorMap map_b, ResidArgs g) {
+                   const __grid_constant__ CUtensorMap map_b, const __grid_constant__ CUtensorMap map_cc, const __grid_constant__ CUtensorMap map_rc,
+                   ResidArgs g) {
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -179,6 +180,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     float* patch = reinterpret_cast<float*>(gen_base + patch_off) + ew * PATCH_F;
     uint32_t* upatch = reinterpret_cast<uint32_t*>(gen_base + patch_off + N_EW * PATCH_F * 4) + ew * (PATCH_U / 2);
     constexpr bool sr = SR;
+    static_assert(PATCH_F * 4 % 128 == 0 && PATCH_F * 4 >= 1024, "a warp's patch is the source of tensor copies");
     const int c_layout = FAST ? (int)METIS_SF_TILED : p.c_layout, r_layout = FAST ? (int)METIS_SF_TILED : p.r_layout;
     const float s_T = metis_tensor_scale(*g.amax_src);
     const float six_s_T = __fmul_rn(6.0f, s_T);
@@ -250,16 +252,19 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             METIS_DBG_GUARD(g.dev_status, (row * p.cols + c0 + 4 * j) * 4, 16, p.rows * p.cols * 4)
             *reinterpret_cast<float4*>(g.dense + row * p.cols + c0 + 4 * j) = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
       }
+      // FAST: a warp's codes - 32 rows of 16 bytes in either orientation - are staged in its patch and stored by tensor copies.  A
+      // lane's store goes to a row of its own, so as ordinary stores they cost the load / store pipe a wavefront per lane
+      // and were 40 % of what bounds the round-to-nearest kernel (77 - 85 % of the pipe's wavefronts).
+      uint32_t pk0[2] = {0u, 0u}, pk1[2] = {0u, 0u}, pkr[2][2];
       if (p.c_codes != nullptr && step_ok) {
         // blocks along the columns: two blocks of this row, from registers
         float v0[16], v1[16];
         uint32_t u0[16], u1[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? metis_qt::sr_addend(nw[i >> 1], i & 1) : 0u; u1[i] = sr ? metis_qt::sr_addend(nw[8 + (i >> 1)], i & 1) : 0u; }
-        uint32_t pk0[2], pk1[2];
         const uint32_t sb0 = encode_block_tab(v0, u0, sr, six_s_T, r_tab, pk0);
         const uint32_t sb1 = encode_block_tab(v1, u1, sr, six_s_T, r_tab, pk1);
-        if (row_ok) {
+        if (!FAST && row_ok) {
           uint8_t* cp = p.c_codes + row * c_kbytes + c0 / 2;
           METIS_DBG_GUARD(g.dev_status, row * c_kbytes + c0 / 2, blk1_ok ? 16 : 8, p.rows * c_kbytes) {
             if (blk1_ok) *reinterpret_cast<uint4*>(cp) = make_uint4(pk0[0], pk0[1], pk1[0], pk1[1]);
@@ -283,6 +288,10 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         const int cb = lane & 15, rb = lane >> 4;
         const uint32_t add_sel = (cb & 1) ? 0x5324u : 0x5104u;
         const bool rb_ok = FAST || slab_row0 + 16 * rb < p.rows;
+        if (FAST) {                                                          // the patch still feeds the last tile's copies until here
+          if (lane == 0) bulk_wait_read_all();
+          __syncwarp();
+        }
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
           {
@@ -308,7 +317,8 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           }
           uint32_t pk[2];
           const uint32_t sb = encode_block_tab(t, d, sr, six_s_T, r_tab, pk);
-          if (col_ok && rb_ok) METIS_DBG_GUARD(g.dev_status, col * r_kbytes + (slab_row0 + 16 * rb) / 2, 8, p.cols * r_kbytes)
+          pkr[hf][0] = pk[0]; pkr[hf][1] = pk[1];
+          if (!FAST && col_ok && rb_ok) METIS_DBG_GUARD(g.dev_status, col * r_kbytes + (slab_row0 + 16 * rb) / 2, 8, p.cols * r_kbytes)
             *reinterpret_cast<uint2*>(p.r_codes + col * r_kbytes + (slab_row0 + 16 * rb) / 2) = make_uint2(pk[0], pk[1]);
           if (rb_ok && (col_ok || r_layout == METIS_SF_TILED))               // padded columns of a 128-slab get zero scales
             METIS_DBG_GUARD(g.dev_status, metis_sf_offset(col, slab_row0 / 16 + rb, r_bpr, r_layout), 1, p.r_sf_bytes)
@@ -316,7 +326,29 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           __syncwarp();
         }
       }
+      if (FAST) {
+        if (p.r_codes == nullptr) {
+          if (lane == 0) bulk_wait_read_all();
+          __syncwarp();
+        }
+        uint4* stage_c = reinterpret_cast<uint4*>(patch);                    // [32 rows][16 bytes]
+        uint2* stage_r = reinterpret_cast<uint2*>(patch + 128);              // [32 columns][16 bytes]
+        stage_c[lane] = make_uint4(pk0[0], pk0[1], pk1[0], pk1[1]);
+        if (p.r_codes != nullptr) {
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) stage_r[(16 * hf + (lane & 15)) * 2 + (lane >> 4)] = make_uint2(pkr[hf][0], pkr[hf][1]);
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) {
+          const uint32_t src = base + (uint32_t)patch_off + (uint32_t)ew * (PATCH_F * 4);
+          if (p.c_codes != nullptr) tma_store_2d(&map_cc, src, (int)(c0 / 2), (int)slab_row0);
+          if (p.r_codes != nullptr) tma_store_2d(&map_rc, src + 512u, (int)(slab_row0 / 2), (int)c0);
+          bulk_commit();
+        }
+      }
     }
+    if (FAST && lane == 0) bulk_wait_all();
   }
 
   // ------------------------------- teardown ---------------------------------
@@ -334,6 +366,18 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 }
 
 }  // namespace
+
+// code matrix [rows][row_bytes], stored in patches of 32 rows x 16 bytes
+static metis_status_t make_map_codes(metis_context* ctx, CUtensorMap* map, const void* ptr, int64_t rows, int64_t row_bytes) {
+  const cuuint64_t dims[2] = {(cuuint64_t)row_bytes, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)row_bytes};
+  const cuuint32_t box[2] = {16, 32};
+  const cuuint32_t estr[2] = {1, 1};
+  const CUresult r = reinterpret_cast<EncodeTiledFn>(ctx->encode_tiled)(
+      map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+      CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? METIS_OK : METIS_ERR_CUDA;
+}
 
 int metis_residual_kx(int kp) { return (6 * kp + 63) / 64 * 64; }
 
@@ -371,9 +415,12 @@ metis_status_t metis_launch_residual_tc(metis_context* ctx, const void* x, const
   g.amax_src = amax_src; g.ts_out0 = ts_out0; g.ts_out1 = ts_out1; g.dense = dense;
   g.k_chunks = kx / BK;
   g.dev_status = ctx->dev_status;
-  const bool fast = rows % TM == 0 && cols % TN == 0 && dense == nullptr &&
+  const bool fast = rows % TM == 0 && cols % TN == 0 && dense == nullptr && metis_aligned16(qp.c_codes) && metis_aligned16(qp.r_codes) &&
                     (qp.c_codes == nullptr || (qp.c_layout == METIS_SF_TILED && reinterpret_cast<uintptr_t>(qp.c_scales) % 2 == 0)) &&
                     (qp.r_codes == nullptr || qp.r_layout == METIS_SF_TILED);
+  CUtensorMap mcc{}, mrc{};
+  if (fast && qp.c_codes != nullptr) METIS_TRY(make_map_codes(ctx, &mcc, qp.c_codes, rows, cols / 2));
+  if (fast && qp.r_codes != nullptr) METIS_TRY(make_map_codes(ctx, &mrc, qp.r_codes, cols, rows / 2));
   const bool sr = qp.rounding == METIS_ROUND_SR;
   const int64_t tiles = metis_ceil_div(rows, TM) * metis_ceil_div(cols, TN);
   // A persistent CTA fills its SM (216 KB of shared memory).  A few SMs are left free so that the small kernels
@@ -387,11 +434,11 @@ metis_status_t metis_launch_residual_tc(metis_context* ctx, const void* x, const
   const int usable = ctx->sm_count > 2 * reserve ? ctx->sm_count - reserve : ctx->sm_count;
   const int grid = (int)(tiles < usable ? tiles : usable);
   if (sr) {
-    if (fast) residual_tc_kernel<true, true><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, g);
-    else residual_tc_kernel<true, false><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, g);
+    if (fast) residual_tc_kernel<true, true><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
+    else residual_tc_kernel<true, false><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
   } else {
-    if (fast) residual_tc_kernel<false, true><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, g);
-    else residual_tc_kernel<false, false><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, g);
+    if (fast) residual_tc_kernel<false, true><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
+    else residual_tc_kernel<false, false><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
   }
   METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
