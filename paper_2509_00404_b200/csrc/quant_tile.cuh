@@ -95,13 +95,14 @@ __device__ __forceinline__ uint32_t sr_addend16(uint32_t u16) { return ((~u16 & 
 //   the magnitude code is then bits 24 .. 26, minus 4 modulo 8: the top bytes of four elements are gathered by byte permutations, the
 //       two words of even and odd elements are merged and the eight "- 4" taken off together;
 //   the sign nibbles are gathered with one funnel shift per element and masked once per word.
-// (Against a compare per element with the draw shifted up and codes packed one by one: quantize_kernel 472 -> 383 us at 16384 x 14336 with
-// both orientations, residual_tc_kernel 1060 -> 866 us at 16384 x 28672, k = 64.)
+// (Against a compare per element with the draw shifted up and codes packed one by one: residual_tc_kernel 236 -> 204 us at 8192 x 14336, k = 32, the
+// minimum per element below included; quantize_kernel 472 -> 371 us at 16384 x 14336 with both orientations, its third CTA per SM
+// included.)
 __device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_t (&add)[8]) {
   uint32_t s[8], sgn = 0u;
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
-    const float a = fminf(fabsf(y[i]), 6.0f);
+    const float a = fabsf(y[i]);                           // at most 6 (the caller has seen to it)
     s[i] = __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f))) * 4u + add[i];
     sgn = __funnelshift_l(__float_as_uint(y[i]), sgn, 4);  // top nibble of y (sign and three exponent bits) shifted in
   }
@@ -111,14 +112,24 @@ __device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_
   return ((mag & 0x77777777u) ^ 0x44444444u) | (sgn & 0x88888888u);
 }
 
+// largest magnitude of a block: eight three-input maxima
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float amax16(const float (&v)[16]) {
+  float m[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) m[i] = max3(fabsf(v[3 * i]), fabsf(v[3 * i + 1]), fabsf(v[3 * i + 2]));
+  return fmaxf(max3(m[0], m[1], m[2]), max3(m[3], m[4], fabsf(v[15])));
+}
+
 // encode_block with the multiplier looked up in a table filled by fill_r_table (same bytes as encode_block).
 // add[i] = sr_addend of draw i (only read with stochastic rounding).
 __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&add)[16], bool sr, float six_s_T,
                                                      const float* r_tab, uint32_t (&packed)[2]) {
-  float m8[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) m8[i] = fmaxf(fabsf(v[i]), fabsf(v[i + 8]));
-  const float amax = fmaxf(fmaxf(fmaxf(m8[0], m8[4]), fmaxf(m8[1], m8[5])), fmaxf(fmaxf(m8[2], m8[6]), fmaxf(m8[3], m8[7])));
+  const float amax = amax16(v);
   const float t = fminf(__fdiv_rn(amax, six_s_T), 448.0f);
   float sb_unused;
   const uint32_t byte = metis_e4m3_ceil(t, &sb_unused);
@@ -133,6 +144,12 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
     uint32_t t0[8], t1[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) { y0[i] = __fmul_rn(v[i], r); y1[i] = __fmul_rn(v[8 + i], r); t0[i] = add[i]; t1[i] = add[8 + i]; }
+    // values beyond 6 saturate.  They only occur where the block scale itself is saturated or the product of the block maximum
+    // rounds up, and the block maximum shows it, so the other blocks are spared a minimum per element.
+    if (!(__fmul_rn(amax, r) <= 6.0f)) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { y0[i] = copysignf(fminf(fabsf(y0[i]), 6.0f), y0[i]); y1[i] = copysignf(fminf(fabsf(y1[i]), 6.0f), y1[i]); }
+    }
     packed[0] = e2m1x8_sr(y0, t0);
     packed[1] = e2m1x8_sr(y1, t1);
   }

@@ -174,3 +174,22 @@ def test_tensor_amax_sees_every_element(ctx, dtype, rows, cols, pad):
     h.quantize_nvfp4(x)
     torch.cuda.synchronize()
     assert h.device_status() != 0
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_stochastic_rounding_of_saturated_and_exact_blocks(ctx, dtype):
+    """Blocks whose scale is clamped at 448 (a tensor scale far too small: most elements saturate at 6), blocks whose maximum
+    falls exactly on an E4M3 scale, values on the E2M1 grid (never rounded up, whatever the draw) and just above it, and
+    tiny ones: byte for byte the oracle's codes."""
+    B, h = ctx
+    rng = np.random.default_rng(77)
+    x = rng.standard_normal((192, 320)).astype(np.float32)
+    x[:32] *= 1e4
+    x[32:48] = np.tile(np.array([0, 0.5, 1, 1.5, 2, 3, 4, 6], dtype=np.float32), 40)
+    x[48:64] = np.tile(np.array([0.5, 1, 1.5, 2, 3, 4, 5.96875, 6], dtype=np.float32) * np.float32(1.0078125), 40)
+    x[64:80] *= 1e-6
+    x[::3] *= -1
+    x = synth.to_bf16_values(x)
+    xd = torch.from_numpy(x).to(dtype).cuda()
+    for ts in (None, 1.0 / 448, 1.0):
+        _compare(B, h, x, xd, B.BLOCKS_BOTH, onv.ROUND_SR, B.SF_TILED, tensor_scale=ts)
