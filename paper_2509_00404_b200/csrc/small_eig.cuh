@@ -126,6 +126,47 @@ __device__ __forceinline__ void cta_cholesky(double* Y, int n, double tol, doubl
   __syncthreads();
 }
 
+// X = L^-1 (nothing is written above the diagonal blocks) for the factor of cta_cholesky, by all nthr threads: the 8 x 8 diagonal
+// blocks first (lane = column), then a warp per block column, X_ib = -X_ii sum_k L_ik X_kb on the FP64 tensor cores
+// without a barrier.  inv: reciprocal pivots (zero for a dependent column, whose row of X is then zero).
+template <int P>
+__device__ __forceinline__ void cta_invert_lower(const double* L, const double* inv, int n, double* X, int xp, int nthr) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3, nb = (n + 7) / 8;
+  for (int b = warp; b < nb; b += nthr >> 5) {
+    if (lane < 8) {
+      double x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < i; ++k) s = fma(L[(8 * b + i) * P + 8 * b + k], x[k], s);
+        const double r = 8 * b + i < n ? inv[8 * b + i] : 0.0;
+        x[i] = i == lane ? r : (i > lane ? -r * s : 0.0);
+        X[(8 * b + i) * xp + 8 * b + lane] = x[i];
+      }
+    }
+  }
+  __syncthreads();
+  for (int b = warp; b < nb; b += nthr >> 5) {
+    for (int i = b + 1; i < nb; ++i) {
+      double t[2][2] = {};
+      for (int k = b; k < i; ++k)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) dmma(t[h], L[(8 * i + g) * P + 8 * k + 4 * h + q], X[(8 * k + 4 * h + q) * xp + 8 * b + g]);
+      double* out = X + (8 * i + g) * xp + 8 * b + 2 * q;
+      out[0] = t[0][0] + t[1][0]; out[1] = t[0][1] + t[1][1];
+      __syncwarp();
+      double d[2] = {0.0, 0.0};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) dmma(d, -X[(8 * i + g) * xp + 8 * i + 4 * h + q], X[(8 * i + 4 * h + q) * xp + 8 * b + g]);
+      __syncwarp();
+      out[0] = d[0]; out[1] = d[1];
+      __syncwarp();
+    }
+  }
+  __syncthreads();
+}
+
 // ------------------------------------------------------------------------------------------------
 // Symmetric positive semi-definite eigen-decomposition in one CTA.
 //   1. the matrix, sorted by descending diagonal, is factorised G = L L^T (FP64; dependent columns zeroed);

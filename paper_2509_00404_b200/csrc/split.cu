@@ -138,21 +138,21 @@ gram_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t stride_r
 }
 
 // ------------------------------------------------------------------------------------------------
-// One CholeskyQR pass, step 1 (one CTA): G (one Gram partial) = L L^T in FP64; writes L (q x q, row-major,
-// upper part unused) and the reciprocal pivots.  A pivot below 1e-13 of the largest diagonal marks a
-// dependent sketch column: its reciprocal is stored as zero, so the corresponding column of H = Z L^-T
-// becomes zero instead of amplified noise.
-__global__ void __launch_bounds__(256)
-chol_kernel(const double* __restrict__ g, int q, double* __restrict__ l_out, double* __restrict__ invd_out,
-            const int* __restrict__ skip, int* __restrict__ well_conditioned) {
+// One CholeskyQR pass, step 1 (one CTA): G = L L^T in FP64; writes L^-T (q x q, row-major, zero below the diagonal), so that step 2
+// is a product on many CTAs instead of a triangular solve per row.  A pivot below 1e-13 of the largest diagonal marks a
+// dependent sketch column: the corresponding column of H = Z L^-T becomes zero instead of amplified noise.
+constexpr size_t CHOL_SMEM = sizeof(double) * MAXQ * LP;
+__global__ void __launch_bounds__(512)
+chol_kernel(const double* __restrict__ g, int q, double* __restrict__ linvt_out, const int* __restrict__ skip, int* __restrict__ well_conditioned) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;
+  extern __shared__ __align__(16) double xs[];
   __shared__ double L[MAXQ][LP];
   __shared__ double gmax_s;
   __shared__ double dmin_s;
-  const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-  const int q8 = (q + 7) & ~7;
-  for (int o = tid; o < q8 * q8; o += 256) {
+  __shared__ double inv_s[MAXQ];
+  const int tid = threadIdx.x, q8 = (q + 7) & ~7;
+  for (int o = tid; o < q8 * q8; o += 512) {
     const int i = o / q8, j = o % q8;
     L[i][j] = i < q && j < q ? g[i * q + j] : 0.0;
   }
@@ -166,13 +166,12 @@ chol_kernel(const double* __restrict__ g, int q, double* __restrict__ l_out, dou
   }
   __syncthreads();
   const double tol = 1e-13 * gmax_s;
-  __shared__ double inv_s[MAXQ];
-  metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, 256);
-  if (tid < q) invd_out[tid] = inv_s[tid];
+  metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, 512);
   // With every pivot above 1e-8 of the largest diagonal the FP64 factorisation leaves Z L^-T orthonormal to
   // ~1e-8 already, below the FP32 rounding of its storage: the caller's second pass is then skipped.
   if (tid == 0 && well_conditioned != nullptr) *well_conditioned = (dmin_s > 1e-8 * gmax_s) ? 1 : 0;
-  for (int o = tid; o < q * q; o += 256) l_out[o] = L[o / q][o % q];
+  metis_small::cta_invert_lower<LP>(&L[0][0], inv_s, q, xs, LP, 512);
+  for (int o = tid; o < q * q; o += 512) { const int i = o / q, j = o % q; linvt_out[o] = i <= j ? xs[j * LP + i] : 0.0; }
 }
 
 // One CholeskyQR pass, steps 0 and 1 in one CTA, for a sketch short enough to sit in shared memory as FP64 (the
@@ -184,13 +183,11 @@ constexpr size_t GC_MAX_SMEM = 176 * 1024;              // beside ~45 KiB of sta
 __host__ __device__ inline int gram_chol_pitch(int q) { return ((q + 7) & ~7) + 4; }   // 4 or 12 mod 16: conflict-free fragment loads
 __host__ inline size_t gram_chol_smem(int64_t n_s, int q) { return (size_t)n_s * gram_chol_pitch(q) * sizeof(double); }
 // Well-conditioned sketch (every pivot above 1e-8 of the largest diagonal: Z L^-T is orthonormal to ~1e-8 already):
-// the kernel writes L and the reciprocal pivots and clears *applied; apply_chol_kernel, on many CTAs, does the
-// triangular solves.  Otherwise (rare) the whole CholeskyQR2 runs here on the FP64 copy - solve, second Gram
+// the kernel writes L^-T and clears *applied; orth_apply_kernel, on many CTAs, multiplies by it.  Otherwise (rare) the whole CholeskyQR2 runs here on the FP64 copy - solve, second Gram
 // matrix, second factor, second solve - H is written over z and *applied is set, which makes the apply kernel
 // behind this one return at once.
 __global__ void __launch_bounds__(GC_THREADS, 1)
-gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ l_out, double* __restrict__ invd_out,
-                 int* __restrict__ applied) {
+gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ linvt_out, int* __restrict__ applied) {
   metis_pdl_wait();
   extern __shared__ __align__(16) double zs[];
   __shared__ double L[MAXQ][LP];
@@ -233,7 +230,8 @@ gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ l_o
     const double tol = 1e-13 * gmax_s;
     metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, GC_THREADS);
     if (pass == 0 && dmin_s > 1e-8 * gmax_s) break;
-    // z_row <- z_row L^-T in shared memory, one warp per row (the recurrence of apply_chol_kernel)
+    // z_row <- z_row L^-T in shared memory by forward substitution, one warp per row, column-oriented: lane i % 32 keeps z_i; step j
+    // broadcasts h_j = z_j / L[j][j] from its owner and every lane subtracts h_j L[i][j] from its own later entries
     solved_here = true;
     for (int r = warp; r < n_s; r += GC_THREADS / 32) {
       double* zr = zs + r * zp;
@@ -259,45 +257,71 @@ gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ l_o
   if (solved_here) {
     for (int e = tid; e < n_s * q; e += GC_THREADS) z[e] = (float)zs[(e / q) * zp + e % q];
   } else {
-    if (tid < q) invd_out[tid] = inv_s[tid];
-    for (int e = tid; e < q * q; e += GC_THREADS) l_out[e] = L[e / q][e % q];
+    // the FP64 copy of z is not needed any more: n_s >= q rows of the same pitch hold the inverse
+    metis_small::cta_invert_lower<LP>(&L[0][0], inv_s, q, zs, zp, GC_THREADS);
+    for (int e = tid; e < q * q; e += GC_THREADS) { const int i = e / q, j = e % q; linvt_out[e] = i <= j ? zs[j * zp + i] : 0.0; }
   }
 }
 
-// One CholeskyQR pass, step 2: z_row <- z_row L^-T by forward substitution, one warp per row, column-oriented:
-// lane i%32 keeps z_i; step j broadcasts h_j = z_j / L[j][j] from its owner and every lane subtracts h_j L[i][j]
-// from its own later entries, so a step is one shuffle and one multiply-add deep (no reduction across lanes).
+// One CholeskyQR pass, step 2: Z <- Z L^-T in place, 64 rows per CTA, on the FP64 tensor cores (a warp per eight rows), and optionally
+// the transposed BF16 splits of the result for the tensor-core projection (the layout of h_splits_kernel).  A triangular solve
+// per row, one column after the other, took 15 us for 4096 x 40, 47 us for 16384 x 40 and 186 us for 28672 x 72.
+constexpr int OA_ROWS = 64, OA_P = OA_ROWS + 4, OA_OP = OA_ROWS + 1;
+__host__ __device__ constexpr size_t oa_smem(int kt) { return sizeof(double) * (size_t)(8 * kt) * (OA_P + 8 * kt + 4) + sizeof(float) * 8 * OA_OP; }
+template <int KT>                                       // ceil(q / 8)
 __global__ void __launch_bounds__(256)
-apply_chol_kernel(float* __restrict__ z, int64_t n_rows, int q, const double* __restrict__ l, const double* __restrict__ invd,
-                  const int* __restrict__ skip) {
+orth_apply_kernel(float* __restrict__ z, int64_t n_rows, int q, const double* __restrict__ linvt, const int* __restrict__ skip,
+                  __nv_bfloat16* __restrict__ hsp, int jp, int64_t ldh) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;
-  __shared__ double L[MAXQ][LP];
-  __shared__ double inv_s[MAXQ];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int o = tid; o < q * q; o += 256) L[o / q][o % q] = l[o];
-  if (tid < q) inv_s[tid] = invd[tid];
-  __syncthreads();
-  const int64_t r = (int64_t)blockIdx.x * 8 + warp;
-  if (r >= n_rows) return;
-  static_assert(MAXQ <= 96, "three values per lane");
-  double z0 = lane < q ? (double)z[r * q + lane] : 0.0;               // entries lane, lane + 32, lane + 64
-  double z1 = lane + 32 < q ? (double)z[r * q + lane + 32] : 0.0;
-  double z2 = lane + 64 < q ? (double)z[r * q + lane + 64] : 0.0;
-  for (int j = 0; j < q; ++j) {
-    const double lj0 = lane < q ? L[lane][j] : 0.0;                    // column j of L (zero above the diagonal is not
-    const double lj1 = lane + 32 < q ? L[lane + 32][j] : 0.0;          // stored: masked by the index tests below)
-    const double lj2 = lane + 64 < q ? L[lane + 64][j] : 0.0;
-    const double zj = __shfl_sync(0xFFFFFFFFu, j < 32 ? z0 : (j < 64 ? z1 : z2), j & 31);
-    const double hj = zj * inv_s[j];
-    if (lane == (j & 31)) { if (j < 32) z0 = hj; else if (j < 64) z1 = hj; else z2 = hj; }
-    if (lane > j) z0 -= hj * lj0;
-    if (lane + 32 > j) z1 -= hj * lj1;
-    if (lane + 64 > j) z2 -= hj * lj2;
+  constexpr int Q8 = 8 * KT, WP = Q8 + 4;
+  extern __shared__ __align__(16) double oa_sm[];
+  double *As = oa_sm, *Ws = oa_sm + Q8 * OA_P;
+  float* Os = reinterpret_cast<float*>(oa_sm);          // [Q8 + 8][OA_OP], over As and Ws once they have been read
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, qq = lane & 3;
+  const int64_t p0 = (int64_t)blockIdx.x * OA_ROWS;
+#pragma unroll 4
+  for (int o = tid; o < OA_ROWS * Q8; o += 256) {
+    const int r = o / Q8, i = o % Q8;
+    As[i * OA_P + r] = i < q && p0 + r < n_rows ? (double)z[(p0 + r) * q + i] : 0.0;
   }
-  if (lane < q) z[r * q + lane] = (float)z0;
-  if (lane + 32 < q) z[r * q + lane + 32] = (float)z1;
-  if (lane + 64 < q) z[r * q + lane + 64] = (float)z2;
+#pragma unroll 4
+  for (int o = tid; o < Q8 * Q8; o += 256) {
+    const int i = o / Q8, j = o % Q8;
+    Ws[i * WP + j] = i < q && j < q ? linvt[i * q + j] : 0.0;
+  }
+  __syncthreads();
+  double acc[KT][2] = {};
+#pragma unroll
+  for (int kk = 0; kk < Q8; kk += 4) {
+    const double a = As[(kk + qq) * OA_P + 8 * warp + g];
+#pragma unroll
+    for (int t = kk / 8; t < KT; ++t) metis_small::dmma(acc[t], a, Ws[(kk + qq) * WP + 8 * t + g]);              // L^-T is upper triangular
+  }
+  __syncthreads();
+#pragma unroll
+  for (int t = 0; t < KT; ++t)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) Os[(8 * t + 2 * qq + e) * OA_OP + 8 * warp + g] = (float)acc[t][e];
+  for (int o = tid; o < 8 * OA_OP; o += 256) Os[Q8 * OA_OP + o] = 0.0f;
+  __syncthreads();
+  for (int o = tid; o < OA_ROWS * q; o += 256) {
+    const int r = o / q, j = o - r * q;
+    if (p0 + r < n_rows) z[(p0 + r) * q + j] = Os[j * OA_OP + r];
+  }
+  if (hsp == nullptr) return;
+  for (int o = tid; o < jp * (OA_ROWS / 2); o += 256) { // rows beyond n_rows and vectors beyond q are zeros
+    const int j = o / (OA_ROWS / 2), r = o % (OA_ROWS / 2) * 2;
+    float x = Os[j * OA_OP + r], y = Os[j * OA_OP + r + 1];
+    uint32_t w[3];
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+      w[t] = *reinterpret_cast<const uint32_t*>(&h);
+      x -= __uint_as_float(w[t] << 16); y -= __uint_as_float(w[t] & 0xFFFF0000u);
+      *reinterpret_cast<uint32_t*>(hsp + ((int64_t)t * jp + j) * ldh + p0 + r) = w[t];
+    }
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1256,6 +1280,17 @@ void launch_project(dim3 grid, cudaStream_t s, const __nv_bfloat16* x, int64_t c
   (void)(metis_launch_pdl((project_kernel<NJ4>), dim3(grid), dim3(256), (size_t)(0), s, x, cols, idx, n_s, q, h, rpp, mp)); METIS_COUNT_LAUNCH();
 }
 
+metis_status_t launch_orth_apply(cudaStream_t s, float* z, int64_t n_s, int q, const double* linvt, const int* skip, __nv_bfloat16* hsp, int jp, int64_t ldh) {
+  const dim3 grid((unsigned)metis_ceil_div(n_s, OA_ROWS));
+#define METIS_OA(KT) METIS_CUDA_TRY(metis_launch_pdl((orth_apply_kernel<KT>), grid, dim3(256), oa_smem(KT), s, z, n_s, q, linvt, skip, hsp, jp, ldh)); break
+  switch ((q + 7) / 8) {
+    case 1: METIS_OA(1); case 2: METIS_OA(2); case 3: METIS_OA(3); case 4: METIS_OA(4); case 5: METIS_OA(5); case 6: METIS_OA(6); case 7: METIS_OA(7); case 8: METIS_OA(8);
+    default: METIS_OA(9);
+  }
+#undef METIS_OA
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
 template <int KT>
 metis_status_t launch_basis_kt(cudaStream_t s, int ctas, size_t smem, const float* m, int64_t cols, int q, int k, int kp, const double* evals, const double* evecs, float* basis,
                                __nv_bfloat16* bs, __nv_bfloat16* bt, __nv_bfloat16* b6, int kx, float* sigma_out, unsigned long long* keys, float* amax_out) {
@@ -1596,6 +1631,10 @@ int64_t metis_default_sample_count(int64_t rows, int32_t q) {
 
 metis_status_t metis_split_set_attrs() {
   using namespace metis_qt;
+#define METIS_OA_ATTR(KT) METIS_CUDA_TRY(cudaFuncSetAttribute(orth_apply_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oa_smem(KT)))
+  METIS_OA_ATTR(1); METIS_OA_ATTR(2); METIS_OA_ATTR(3); METIS_OA_ATTR(4); METIS_OA_ATTR(5); METIS_OA_ATTR(6); METIS_OA_ATTR(7); METIS_OA_ATTR(8); METIS_OA_ATTR(9);
+#undef METIS_OA_ATTR
+  METIS_CUDA_TRY(cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHOL_SMEM));
 #define METIS_FR_ATTR(KT) METIS_CUDA_TRY(cudaFuncSetAttribute(basis_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fr_smem(MAXQ))); \
   METIS_CUDA_TRY(cudaFuncSetAttribute(factors_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fr_smem(MAXQ)))
   METIS_FR_ATTR(1); METIS_FR_ATTR(2); METIS_FR_ATTR(3); METIS_FR_ATTR(4); METIS_FR_ATTR(5); METIS_FR_ATTR(6); METIS_FR_ATTR(7); METIS_FR_ATTR(8);
@@ -1752,8 +1791,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   float* zp = reinterpret_cast<float*>(wsb + L.zp);
   float* z = reinterpret_cast<float*>(wsb + L.z);
   double* gram = reinterpret_cast<double*>(wsb + L.gram);
-  double* linv = reinterpret_cast<double*>(wsb + L.linv);
-  double* invd = linv + MAXQ * MAXQ;
+  double* linvt = reinterpret_cast<double*>(wsb + L.linv);
   int* cond_flag = reinterpret_cast<int*>(amax + 8);
   double* gram1 = reinterpret_cast<double*>(wsb + L.gram1);
   double* evals = reinterpret_cast<double*>(wsb + L.evals);
@@ -1818,32 +1856,37 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     METIS_CUDA_TRY(metis_launch_pdl((reduce_partials_kernel), dim3((unsigned)metis_ceil_div(n_s * q, 256)), dim3(256), (size_t)(0), s, zp, chunks, n_s * q, z)); METIS_COUNT_LAUNCH();
   }
   // (3) CholeskyQR2: orthonormal basis H of range(Z), in place
-  if (gram_chol_smem(n_s, q) <= GC_MAX_SMEM) {
-    // a short sketch: Gram matrix and factorisation in one CTA; the triangular solves on many CTAs unless the sketch
+  // the projection on tensor cores wants the BF16 splits of H as well (n_s >= 1024)
+  const bool split_h = n_s >= 1024 && cols % 8 == 0, one_cta = gram_chol_smem(n_s, q) <= GC_MAX_SMEM;
+  const int jp = (q + 15) / 16 * 16, ldh = (int)((n_s + 63) / 64 * 64);
+  if (one_cta) {
+    // a short sketch: Gram matrix and factorisation in one CTA; the product with L^-T on many CTAs unless the sketch
     // was ill-conditioned, in which case the first kernel has done both passes itself and the second returns at once
-    METIS_CUDA_TRY(metis_launch_pdl((gram_chol_kernel), dim3(1), dim3(GC_THREADS), gram_chol_smem(n_s, q), s, z, (int)n_s, q, linv, invd, cond_flag)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((apply_chol_kernel), dim3((unsigned)metis_ceil_div(n_s, 8)), dim3(256), (size_t)(0), s, z, n_s, q, linv, invd, (const int*)cond_flag)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((gram_chol_kernel), dim3(1), dim3(GC_THREADS), gram_chol_smem(n_s, q), s, z, (int)n_s, q, linvt, cond_flag)); METIS_COUNT_LAUNCH();
+    METIS_TRY(launch_orth_apply(s, z, n_s, q, linvt, cond_flag, nullptr, jp, ldh));
   } else {
-  for (int pass = 0; pass < 2; ++pass) {
-    int64_t rpp; const int parts = gram_parts(n_s, &rpp);
-    const int* skip = pass == 0 ? nullptr : cond_flag;
-    METIS_CUDA_TRY(metis_launch_pdl((gram_kernel), dim3(parts), dim3(256), (size_t)(0), s, z, n_s, q, q, 1, rpp, gram, skip)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(q * q, 32)), dim3(128), (size_t)(0), s, gram, parts, q * q, gram1, skip)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((chol_kernel), dim3(1), dim3(256), (size_t)(0), s, gram1, q, linv, invd, skip, pass == 0 ? cond_flag : nullptr)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((apply_chol_kernel), dim3((unsigned)metis_ceil_div(n_s, 8)), dim3(256), (size_t)(0), s, z, n_s, q, linv, invd, skip)); METIS_COUNT_LAUNCH();
-  }
+    for (int pass = 0; pass < 2; ++pass) {
+      int64_t rpp; const int parts = gram_parts(n_s, &rpp);
+      const int* skip = pass == 0 ? nullptr : cond_flag;
+      METIS_CUDA_TRY(metis_launch_pdl((gram_kernel), dim3(parts), dim3(256), (size_t)(0), s, z, n_s, q, q, 1, rpp, gram, skip)); METIS_COUNT_LAUNCH();
+      METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(q * q, 32)), dim3(128), (size_t)(0), s, gram, parts, q * q, gram1, skip)); METIS_COUNT_LAUNCH();
+      METIS_CUDA_TRY(metis_launch_pdl((chol_kernel), dim3(1), dim3(512), CHOL_SMEM, s, gram1, q, linvt, skip, pass == 0 ? cond_flag : nullptr)); METIS_COUNT_LAUNCH();
+      METIS_TRY(launch_orth_apply(s, z, n_s, q, linvt, skip, split_h ? hsp : nullptr, jp, ldh));
+    }
   }
   // (4) M = H^T x[S,:], eigen-decomposition of M M^T, right basis
   {
     int rpp; int parts;
     bool project_tc = false;
-    if (n_s >= 1024 && cols % 8 == 0) {
+    if (split_h) {
+      if (one_cta) {                                    // that factorisation leaves the splits to a kernel of their own
+        METIS_CUDA_TRY(metis_launch_pdl(h_splits_kernel, dim3((unsigned)metis_ceil_div(ldh, 256), (unsigned)jp), dim3(256), (size_t)0, s, z, (int)n_s, q, jp, ldh, hsp, q)); METIS_COUNT_LAUNCH();
+      }
       parts = (int)metis_ceil_div(n_s, 512);
       if (parts > PJ_MAX_PARTS) parts = PJ_MAX_PARTS;
       rpp = (int)(metis_ceil_div(metis_ceil_div(n_s, parts), PP_K) * PP_K);
       parts = (int)metis_ceil_div(n_s, rpp);
-      const int mt = (q + 15) / 16, jp = mt * 16, ldh = (int)((n_s + 63) / 64 * 64);
-      METIS_CUDA_TRY(metis_launch_pdl(h_splits_kernel, dim3((unsigned)metis_ceil_div(ldh, 256), (unsigned)jp), dim3(256), (size_t)0, s, z, (int)n_s, q, jp, ldh, hsp, q)); METIS_COUNT_LAUNCH();
+      const int mt = jp / 16;
       project_tc = full && metis_project_tc_usable(x, hsp, cols, jp);
       if (project_tc) {
         // every row, in order: M^T = x^T H on the tcgen05 kernel of the broadcast pass (x as an MN-major operand)
