@@ -296,13 +296,19 @@ chol_mid_kernel(const double* __restrict__ g, int n, double tol_rel, double* __r
   for (int i = tid; i < n; i += CW_THREADS) { diag[i] = g[(int64_t)i * n + i]; perm[i] = i; }
   if (tid == 0) gmax_s = 0.0;
   __syncthreads();
-  for (int i = tid >> 1; i < n; i += CW_THREADS / 2) {     // two lanes per entry
-    const double d = diag[i];
+  static_assert(CM_MAX <= CW_THREADS / 2, "two lanes per diagonal entry in one pass");
+  {
+    // two lanes per entry, in whole warps: for an odd n the lanes of a pair count different numbers of entries, so the sum is
+    // taken behind the loop by every thread (joined inside it, a lane's partner may not have arrived)
+    const int i = tid >> 1;
+    const double d = i < n ? diag[i] : 0.0;
     int rank = 0;
+    if (i < n) {
 #pragma unroll 8
-    for (int j = tid & 1; j < n; j += 2) rank += (diag[j] > d) || (diag[j] == d && j < i);
-    rank += __shfl_xor_sync(__activemask(), rank, 1);
-    if ((tid & 1) == 0) {
+      for (int j = tid & 1; j < n; j += 2) rank += (diag[j] > d) || (diag[j] == d && j < i);
+    }
+    rank += __shfl_xor_sync(0xFFFFFFFFu, rank, 1);
+    if (i < n && (tid & 1) == 0) {
       if (rank == 0) gmax_s = d;
       if (perm_out != nullptr) perm[rank] = i;             // NaNs may collide; every entry stays a valid index
     }

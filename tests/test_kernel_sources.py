@@ -1,0 +1,22 @@
+"""Rules of the CUDA sources that no run can show, because the compiler may happen to hide their violation: checked on the text."""
+import glob
+import os
+import re
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2509_00404_b200", "csrc")
+
+
+def _sources():
+    """(file, line number, code) of every line, comments removed."""
+    out = []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        with open(path) as f:
+            for i, line in enumerate(f, 1):
+                out.append((os.path.basename(path), i, line.split("//")[0]))
+    assert len(out) > 1000
+    return out
+
+
+def test_no_exchange_takes_its_mask_from_the_lanes_that_happen_to_be_active():
+    """__activemask() does not bring a warp together: a lane whose partner has not arrived yet would exchange with nothing."""
+    assert [(f, i) for f, i, code in _sources() if "__activemask" in code] == []
