@@ -491,14 +491,17 @@ __global__ void rot_scales_kernel(const double* __restrict__ evals, const float*
 constexpr int ER_STEPS = 3;                               // refinement steps (two are enough unless eigenvalues are close)
 struct EigState {
   unsigned int emax[ER_STEPS];                            // largest |E_ij| of a step (bits)
-  float norm2[ER_STEPS];                                  // squared norm of E
+  // squared norm of E in units of 2^-40: a sum of integers is the same in every order of arrival, and it chooses the solver
+  unsigned long long norm2[ER_STEPS];
   int open[ER_STEPS];                                     // some pair could not be separated
 };
 __device__ __forceinline__ void eig_state_reset(EigState* st, int tid) {
-  if (tid < ER_STEPS) { st->emax[tid] = 0u; st->norm2[tid] = 0.0f; st->open[tid] = 0; }
+  if (tid < ER_STEPS) { st->emax[tid] = 0u; st->norm2[tid] = 0ull; st->open[tid] = 0; }
 }
+constexpr float EIG_NORM2_UNITS = 1099511627776.0f;       // 2^40
+__device__ __forceinline__ unsigned long long eig_norm2_units(float x) { return x < 1024.0f ? __float2ull_rz(x * EIG_NORM2_UNITS) : 1ull << 50; }   // (a NaN is a large one)
 enum { EIG_RUNNING = 0, EIG_DONE = 1, EIG_FAILED = 2 };
-__device__ __forceinline__ bool eig_step_bad(const EigState* st, int t) { return __ldcg(&st->open[t]) != 0 || !(__ldcg(&st->norm2[t]) < 0.0625f); }
+__device__ __forceinline__ bool eig_step_bad(const EigState* st, int t) { return __ldcg(&st->open[t]) != 0 || __ldcg(&st->norm2[t]) >= eig_norm2_units(0.0625f); }
 // what the steps before `step` have come to; *last: the last step that was applied
 __device__ __forceinline__ int eig_status(const EigState* st, int step, int* last) {
   *last = -1;
@@ -747,7 +750,7 @@ refine_correction_kernel(const double* __restrict__ s, const double* __restrict_
   const bool any = __any_sync(0xFFFFFFFFu, open);
   if ((threadIdx.x & 31) == 0) {
     atomicMax(&st->emax[step], __float_as_uint(em));
-    atomicAdd(&st->norm2[step], en);                      // only compared with a bound
+    atomicAdd(&st->norm2[step], eig_norm2_units(en));
     if (any) st->open[step] = 1;
   }
 }

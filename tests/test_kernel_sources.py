@@ -20,3 +20,11 @@ def _sources():
 def test_no_exchange_takes_its_mask_from_the_lanes_that_happen_to_be_active():
     """__activemask() does not bring a warp together: a lane whose partner has not arrived yet would exchange with nothing."""
     assert [(f, i) for f, i, code in _sources() if "__activemask" in code] == []
+
+
+def test_nothing_is_summed_in_the_order_of_arrival():
+    """The library repeats itself bit for bit, so its atomic additions are on integers."""
+    adds = [(f, i, code.strip()) for f, i, code in _sources() if re.search(r"\batomicAdd\b|\bred\.[a-z.]*add", code)]
+    assert [a for a in adds if "eig_norm2_units(" not in a[2]] == []
+    decl = [code for _, _, code in _sources() if re.search(r"\bnorm2\[ER_STEPS\]", code)]
+    assert len(decl) == 1 and "unsigned long long" in decl[0]
