@@ -112,47 +112,63 @@ __device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_
   return ((mag & 0x77777777u) ^ 0x44444444u) | (sgn & 0x88888888u);
 }
 
-// largest magnitude of a block: eight three-input maxima
+// largest magnitude of a block: eight three-input maxima, which pass a NaN over or (KEEP_NAN) on
+template <bool KEEP_NAN>
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
-  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  if (KEEP_NAN) asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  else asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+template <bool KEEP_NAN>
 __device__ __forceinline__ float amax16(const float (&v)[16]) {
   float m[5];
 #pragma unroll
-  for (int i = 0; i < 5; ++i) m[i] = max3(fabsf(v[3 * i]), fabsf(v[3 * i + 1]), fabsf(v[3 * i + 2]));
-  return fmaxf(max3(m[0], m[1], m[2]), max3(m[3], m[4], fabsf(v[15])));
+  for (int i = 0; i < 5; ++i) m[i] = max3<KEEP_NAN>(fabsf(v[3 * i]), fabsf(v[3 * i + 1]), fabsf(v[3 * i + 2]));
+  const float lo = max3<KEEP_NAN>(m[0], m[1], m[2]), hi = max3<KEEP_NAN>(m[3], m[4], fabsf(v[15]));
+  return max3<KEEP_NAN>(lo, hi, hi);
 }
 
 // encode_block with the multiplier looked up in a table filled by fill_r_table (same bytes as encode_block).
 // add[i] = sr_addend of draw i (only read with stochastic rounding).
 __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&add)[16], bool sr, float six_s_T,
                                                      const float* r_tab, uint32_t (&packed)[2]) {
-  const float amax = amax16(v);
-  const float t = fminf(__fdiv_rn(amax, six_s_T), 448.0f);
   float sb_unused;
-  const uint32_t byte = metis_e4m3_ceil(t, &sb_unused);
-  const float r = r_tab[byte];
   if (!sr) {
+    const uint32_t byte = metis_e4m3_ceil(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f), &sb_unused);
+    const float r = r_tab[byte];
     packed[0] = e2m1x8_rne(__fmul_rn(v[0], r), __fmul_rn(v[1], r), __fmul_rn(v[2], r), __fmul_rn(v[3], r),
                            __fmul_rn(v[4], r), __fmul_rn(v[5], r), __fmul_rn(v[6], r), __fmul_rn(v[7], r));
     packed[1] = e2m1x8_rne(__fmul_rn(v[8], r), __fmul_rn(v[9], r), __fmul_rn(v[10], r), __fmul_rn(v[11], r),
                            __fmul_rn(v[12], r), __fmul_rn(v[13], r), __fmul_rn(v[14], r), __fmul_rn(v[15], r));
-  } else {
-    float y0[8], y1[8];
-    uint32_t t0[8], t1[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { y0[i] = __fmul_rn(v[i], r); y1[i] = __fmul_rn(v[8 + i], r); t0[i] = add[i]; t1[i] = add[8 + i]; }
-    // values beyond 6 saturate.  They only occur where the block scale itself is saturated or the product of the block maximum
-    // rounds up, and the block maximum shows it, so the other blocks are spared a minimum per element.
-    if (!(__fmul_rn(amax, r) <= 6.0f)) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) { y0[i] = copysignf(fminf(fabsf(y0[i]), 6.0f), y0[i]); y1[i] = copysignf(fminf(fabsf(y1[i]), 6.0f), y1[i]); }
-    }
-    packed[0] = e2m1x8_sr(y0, t0);
-    packed[1] = e2m1x8_sr(y1, t1);
+    return byte;
   }
+  float y0[8], y1[8];
+  uint32_t t0[8], t1[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { t0[i] = add[i]; t1[i] = add[8 + i]; }
+  const float amax = amax16<true>(v);
+  uint32_t byte = metis_e4m3_ceil(fminf(__fdiv_rn(amax, six_s_T), 448.0f), &sb_unused);
+  float r = r_tab[byte];
+  // values beyond 6 saturate, and a NaN is stored as 6.  They only occur where the block scale itself is saturated, the product
+  // of the block maximum rounds up, or an element is a NaN, and the block maximum shows it, so the other blocks are spared a
+  // minimum per element.  The scale of a block is that of its other elements (448 where there are none).
+  if (__fmul_rn(amax, r) <= 6.0f) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { y0[i] = __fmul_rn(v[i], r); y1[i] = __fmul_rn(v[8 + i], r); }
+  } else {
+    if (isnan(amax)) {
+      byte = metis_e4m3_ceil(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f), &sb_unused);
+      r = r_tab[byte];
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float a = __fmul_rn(v[i], r), b = __fmul_rn(v[8 + i], r);
+      y0[i] = copysignf(fminf(fabsf(a), 6.0f), a); y1[i] = copysignf(fminf(fabsf(b), 6.0f), b);
+    }
+  }
+  packed[0] = e2m1x8_sr(y0, t0);
+  packed[1] = e2m1x8_sr(y1, t1);
   return byte;
 }
 

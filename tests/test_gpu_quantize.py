@@ -193,3 +193,36 @@ def test_stochastic_rounding_of_saturated_and_exact_blocks(ctx, dtype):
     xd = torch.from_numpy(x).to(dtype).cuda()
     for ts in (None, 1.0 / 448, 1.0):
         _compare(B, h, x, xd, B.BLOCKS_BOTH, onv.ROUND_SR, B.SF_TILED, tensor_scale=ts)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("rounding", [onv.ROUND_RNE, onv.ROUND_SR])
+def test_a_nan_is_stored_as_six_and_its_block_is_scaled_by_the_others(ctx, dtype, rounding):
+    """With a caller's tensor scale no amax check sees a NaN: it becomes +6 times the block scale, in ordinary, saturated and zero
+    blocks and beside an infinity, and every other element keeps the code that it has with a zero in the NaN's place.  A block
+    of nothing else gets the largest scale."""
+    from gpu_util import nv_to_numpy
+    B, h = ctx
+    rng = np.random.default_rng(78)
+    x = synth.to_bf16_values(rng.standard_normal((192, 192)).astype(np.float32))
+    x[16:32] *= 4096.0
+    x[32:48] = 0.0
+    nan = np.zeros(x.shape, dtype=bool)
+    nan[::5, ::7] = True                             # several in a block and one, in either orientation
+    nan[48:96] = False
+    nan[50, 3] = nan[70, 100] = True
+    nan[112:128] = False
+    nan[112:128, 64:80] = True
+    x[nan] = 0.0
+    x[80, 40] = np.inf
+    xn = np.where(nan, np.float32("nan"), x).astype(np.float32)
+    ts = np.float32(1.0 / 448)
+    bc, br = h.quantize_nvfp4(torch.from_numpy(xn).to(dtype).cuda(), B.BLOCKS_BOTH, rounding, seed=5, layout=B.SF_TILED, tensor_scale=ts)
+    torch.cuda.synchronize()
+    for t, axis, at in ((bc, onv.AXIS_COLS, nan), (br, onv.AXIS_ROWS, nan.T)):
+        c, s, _ = nv_to_numpy(t)
+        with np.errstate(invalid="ignore", over="ignore"):
+            oc, os_, _ = onv.quantize(np.where(np.isinf(x), np.float32(3e38), x), axis, rounding, seed=5, tensor_scale=ts)
+        os_ = np.where(at.reshape(at.shape[0], -1, 16).all(axis=2), np.uint8(126), os_)
+        assert np.array_equal(s, os_)
+        assert np.array_equal(c[~at], oc[~at]) and bool((c[at] == 7).all())
