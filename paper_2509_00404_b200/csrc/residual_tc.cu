@@ -342,8 +342,11 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         __syncwarp();
         if (lane == 0) {
           const uint32_t src = base + (uint32_t)patch_off + (uint32_t)ew * (PATCH_F * 4);
-          if (p.c_codes != nullptr) tma_store_2d(&map_cc, src, (int)(c0 / 2), (int)slab_row0);
-          if (p.r_codes != nullptr) tma_store_2d(&map_rc, src + 512u, (int)(slab_row0 / 2), (int)c0);
+          // (a copy that left its matrix would be clipped without a word: the debug build checks its 16 bytes and its 32 rows)
+          if (p.c_codes != nullptr) METIS_DBG_GUARD(g.dev_status, c0 / 2, 16, c_kbytes) METIS_DBG_GUARD(g.dev_status, slab_row0, 32, p.rows)
+            tma_store_2d(&map_cc, src, (int)(c0 / 2), (int)slab_row0);
+          if (p.r_codes != nullptr) METIS_DBG_GUARD(g.dev_status, slab_row0 / 2, 16, r_kbytes) METIS_DBG_GUARD(g.dev_status, c0, 32, p.cols)
+            tma_store_2d(&map_rc, src + 512u, (int)(slab_row0 / 2), (int)c0);
           bulk_commit();
         }
       }

@@ -28,3 +28,15 @@ def test_nothing_is_summed_in_the_order_of_arrival():
     assert [a for a in adds if "eig_norm2_units(" not in a[2]] == []
     decl = [code for _, _, code in _sources() if re.search(r"\bnorm2\[ER_STEPS\]", code)]
     assert len(decl) == 1 and "unsigned long long" in decl[0]
+
+
+def test_tensor_copies_of_codes_are_checked_in_the_debug_build():
+    """A tensor copy that leaves its matrix is clipped by the hardware, so nothing else would show it: both of its ranges stand behind
+    the debug build's check."""
+    with open(os.path.join(CSRC, "residual_tc.cu")) as f:
+        code = re.sub(r"//[^\n]*", "", f.read())
+    copies = [m.start() for m in re.finditer(r"\btma_store_2d\(", code)]
+    assert len(copies) == 2
+    for at in copies:
+        statement = code[code.rfind(";", 0, at):at]
+        assert re.findall(r"METIS_DBG_GUARD\([^,]*, [^,]*, (\d+), ", statement) == ["16", "32"], statement
