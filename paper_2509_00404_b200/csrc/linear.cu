@@ -391,6 +391,17 @@ __device__ __forceinline__ __half2 e2m1x2_to_half2(uint32_t byte) {
   return *reinterpret_cast<const __half2*>(&w);
 }
 
+// One entry of the contraction as FP32 multiply-adds in order.  An FP32 gradient that is infinite or rounds to infinity in BF16
+// leaves a NaN as its remainder, and sums that overflow may meet with opposite signs: an entry that came out as a NaN is
+// settled here, so that the gradients are infinite where FP32 products make them so and a NaN stands for a real one.  Never
+// entered for finite gradients; a NaN ends the sum.
+template <typename T>
+__device__ __noinline__ float fg_plain_sum(const T* g, int64_t stride, int64_t n_c, const uint8_t* f_codes, const uint8_t* f_sf, int f_layout, int64_t t) {
+  float acc = 0.0f;
+  for (int64_t c = 0; c < n_c && !isnan(acc); ++c) acc = fmaf((float)g[c * stride], deq_at(f_codes, f_sf, f_layout, n_c, t, c), acc);
+  return acc;
+}
+
 template <int NT, bool TRANS, typename T, bool VEC>     // NT = ceil(k / 8) groups of eight factor vectors, at most 8
 __global__ void __launch_bounds__(FG_THREADS, NT <= 4 ? 3 : 2)
 factor_grad_kernel(const T* __restrict__ gsrc, int64_t ldg, int64_t n_r, int64_t n_c, int k, int t0, int k_all,
@@ -560,6 +571,7 @@ factor_grad_kernel(const T* __restrict__ gsrc, int64_t ldg, int64_t n_r, int64_t
         asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(x) : "r"(peer));
         v += x;
       }
+      if (isnan(v) && r < n_r) v = fg_plain_sum<T>(gsrc + (TRANS ? r : r * ldg), c_stride, n_c, f_codes, f_sf, f_layout, t0 + t);
       v *= fts;
       if (r < n_r) {
         out[(int64_t)(t0 + t) * n_r + r] = v * sigma[t0 + t];

@@ -183,6 +183,55 @@ def test_factor_gradient_strips_and_chunks(ctx, l, n, m, k, dtype, pad):
     assert rel_fro(fg[1].cpu().numpy(), np.einsum("jt,ji,it->t", lq, dwn, rq)) < 1e-5
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("peak", [3.4e38, 1e39])
+def test_factor_gradients_of_an_overflowing_weight_gradient(ctx, dtype, peak):
+    """Entries of dW that are infinite, or finite in FP32 and infinite in BF16: alone in a row or column, two of the same and two of
+    opposite sign in one, in the first and the last chunk.  The gradients are what FP32 products and sums give: infinite, a NaN
+    only for 0 * inf and inf - inf, finite where the factor's entry keeps them so, and untouched elsewhere."""
+    from gpu_util import rel_fro, nv_to_numpy, nv_dequant
+    B, h = ctx
+    l, n, m, k = 128, 320, 448, 20
+    rng = np.random.default_rng(5)
+    spots = [(3, 5, 1), (64, 200, -1), (64, 447, -1), (130, 17, 1), (130, 260, -1), (319, 128, 1), (200, 300, 1), (210, 300, 1), (220, 310, -1), (221, 310, 1)]
+    dy, x = np.zeros((l, n), dtype=np.float32), np.zeros((l, m), dtype=np.float32)
+    dy[len(spots):] = 1e-4 * rng.standard_normal((l - len(spots), n)); x[len(spots):] = 1e-4 * rng.standard_normal((l - len(spots), m))
+    for t, (r, c, sgn) in enumerate(spots):
+        dy[t, r], x[t, c] = sgn, 1.0
+    do, xo = (h.split(torch.from_numpy(a).cuda().to(torch.bfloat16), 0, 0) for a in (dy, x))
+    xo.res_by_rows.tensor_scale.fill_(1.0)
+    do.res_by_rows.tensor_scale.fill_(peak / 2688.0 ** 2)          # both maxima are stored as 448 * 6
+    torch.manual_seed(3)
+    wo = B.Operand(n, m, k)
+    wo.left_q, wo.right_q = h.quantize_nvfp4(torch.randn(k, n, device="cuda"))[0], h.quantize_nvfp4(torch.randn(k, m, device="cuda"))[0]
+    wo.sigma.copy_(torch.rand(k, device="cuda") + 0.5)
+    fg = (torch.empty((k, n), device="cuda"), torch.empty(k, device="cuda"), torch.empty((k, m), device="cuda"))
+    dw = torch.empty((n, m), dtype=dtype, device="cuda")
+    h.linear_bwd(do, xo, wo, need_dx=False, out=(None, dw), factor_grads=fg)
+    torch.cuda.synchronize()
+    dwn = dw.float().cpu().numpy().astype(np.float64)
+    big = np.abs(dwn) > 3.39e38
+    assert int(big.sum()) == len(spots) and bool(np.isinf(dwn[big]).all()) == (peak > 3.4e38 or dtype == torch.bfloat16)
+    sig = wo.sigma.cpu().numpy().astype(np.float64)
+    for got, fac, mat in ((fg[0], wo.right_q, dwn), (fg[2], wo.left_q, dwn.T)):
+        codes, _, ts = nv_to_numpy(fac)
+        unscaled = (nv_dequant(fac)[:k] / float(ts)).T              # the sums are over E2M1 * E4M3 values, the FP32 scales come last
+        with np.errstate(invalid="ignore", over="ignore"):
+            sums = np.zeros((mat.shape[0], k))
+            for c in range(mat.shape[1]):                           # an FP32 sum that has overflowed stays infinite
+                sums += mat[:, c:c + 1] * unscaled[c]
+                sums = np.where(np.abs(sums) > 3.4028236e38, np.copysign(np.inf, sums), sums)
+            want = sums * float(ts) * sig
+            want = np.where(np.abs(want) > 3.4028236e38, np.copysign(np.inf, want), want)
+        got = got.cpu().numpy().T.astype(np.float64)
+        assert np.array_equal(np.isnan(got), np.isnan(want)) and np.array_equal(np.isposinf(got), np.isposinf(want)) and np.array_equal(np.isneginf(got), np.isneginf(want))
+        rows = np.abs(mat).max(axis=1) > 3.39e38
+        fin = np.isfinite(want)
+        assert np.isinf(want[rows]).any() and fin[~rows].all()
+        assert rel_fro(got[~rows], want[~rows]) < 2e-6
+        assert np.allclose(got[rows][fin[rows]], want[rows][fin[rows]], rtol=1e-5, atol=2e-6 * np.abs(want[~rows]).max())
+
+
 def test_factor_gradients_need_the_weight_gradient(ctx):
     from gpu_util import to_dev_bf16
     B, h = ctx
