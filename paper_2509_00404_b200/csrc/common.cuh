@@ -271,7 +271,6 @@ int metis_project_slices(int64_t rows, int64_t cols);
 metis_status_t metis_launch_project_tc(metis_context* ctx, const void* x, int64_t rows, int64_t cols, const void* hsp, int jp,
                                        int64_t ldh, float* part, cudaStream_t s);
 int metis_residual_kx(int kp);
-bool metis_residual_tc_usable(const void* x, int64_t cols);
 metis_status_t metis_launch_gemm_check(const metis_nvfp4_t* a, const metis_nvfp4_t* b, void* d, int d_dtype,
                                        int64_t ldd, cudaStream_t s);
 metis_status_t metis_launch_gemm_tc(metis_context* ctx, const metis_nvfp4_t* a, const metis_nvfp4_t* b, void* d,

@@ -1,5 +1,4 @@
-// NVFP4 quantization of a 128 x 128 FP32 tile held in shared memory, in one or both block
-// orientations (Section 2.3).  Used by the stand-alone quantizer and by the fused
+// NVFP4 encoding of blocks of 16 values in registers (Section 2.3).  Used by the stand-alone quantizer and by the fused
 // residual -> quantizer kernel of the split, so both produce identical codes for identical values.
 #pragma once
 #include "common.cuh"
@@ -7,7 +6,6 @@
 namespace metis_qt {
 
 constexpr int TILE = 128;
-constexpr int PITCH = 132;            // floats per shared-memory tile row (conflict-free float4 access by row)
 constexpr int THREADS = 256;
 
 struct QuantParams {
@@ -23,11 +21,6 @@ struct QuantParams {
   int64_t c_sf_bytes, r_sf_bytes;
   uint32_t* dbg;
   PhiloxKeys keys;                    // round keys of `seed` (filled where the element draws are made in bulk)
-};
-
-struct __align__(16) Stage {
-  uint8_t codes[TILE][TILE / 2];      // 8 KiB: [stored row in tile][packed k]
-  uint8_t sf[TILE][TILE / 16];        // 1 KiB: [stored row in tile][block]
 };
 
 // Encodes one block of 16 values; returns the scale byte, writes 8 code bytes.
@@ -83,7 +76,6 @@ __device__ __forceinline__ uint32_t e2m1x8_rne(float a0, float a1, float a2, flo
 // What a 16-bit draw u contributes to the rounding of its element: (65535 - u) * 256 + 255, one byte permutation of the
 // COMPLEMENTED Philox word that holds the draw in its low (hi = false) or high half.
 __device__ __forceinline__ uint32_t sr_addend(uint32_t not_word, bool hi) { return __byte_perm(not_word, 0xFFu, hi ? 0x5324u : 0x5104u); }
-__device__ __forceinline__ uint32_t sr_addend16(uint32_t u16) { return ((~u16 & 0xFFFFu) << 8) | 0xFFu; }
 
 // Eight stochastically rounded codes in one word; add[i] = sr_addend of draw i.  The same decision as metis_e2m1_sr,
 // arranged for the instruction mix of the SM (integer logic, shifts and compares issue at half the FP32 / IMAD rate, and bound
@@ -170,138 +162,6 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
   packed[0] = e2m1x8_sr(y0, t0);
   packed[1] = e2m1x8_sr(y1, t1);
   return byte;
-}
-
-// tile:  [TILE][PITCH] floats, rows/cols outside the matrix already zero-filled
-// rnd:   [TILE][TILE] 16-bit draws (only read when rounding == SR)
-// stage: scratch
-// All THREADS threads of the block must call this; contains __syncthreads().
-__device__ __forceinline__ void quantize_tile(const float* tile, const uint16_t* rnd, Stage* stage,
-                                              const QuantParams& p, int64_t row0, int64_t col0, float s_T) {
-  const int tid = threadIdx.x;
-  const bool sr = p.rounding == METIS_ROUND_SR;
-  const float six_s_T = __fmul_rn(6.0f, s_T);
-  const int vrows = (int)min((int64_t)TILE, p.rows - row0);
-  const int vcols = (int)min((int64_t)TILE, p.cols - col0);
-
-  if (p.c_codes != nullptr) {
-    // blocks along columns: thread -> (row = tid % 128, blocks b = tid/128 + 2*it)
-#pragma unroll 1
-    for (int it = 0; it < 4; ++it) {
-      const int r = tid & 127, b = (tid >> 7) + 2 * it;
-      float v[16];
-      uint32_t u[16];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float4 q = *reinterpret_cast<const float4*>(tile + r * PITCH + b * 16 + i * 4);
-        v[4 * i] = q.x; v[4 * i + 1] = q.y; v[4 * i + 2] = q.z; v[4 * i + 3] = q.w;
-      }
-      if (sr) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) u[i] = rnd[r * TILE + b * 16 + i];
-      }
-      uint32_t packed[2];
-      const uint32_t byte = encode_block(v, u, sr, s_T, six_s_T, packed);
-      *reinterpret_cast<uint2*>(&stage->codes[r][b * 8]) = make_uint2(packed[0], packed[1]);
-      stage->sf[r][b] = (uint8_t)byte;
-    }
-    __syncthreads();
-    // coalesced write-out
-    const int64_t kbytes = p.cols / 2;
-    for (int i = tid; i < TILE * 8; i += THREADS) {      // 8-byte units: one block of 16 codes each
-      const int r = i >> 3, seg = i & 7;
-      if (r < vrows && seg * 16 < vcols) {
-        *reinterpret_cast<uint2*>(p.c_codes + (row0 + r) * kbytes + col0 / 2 + seg * 8) =
-            *reinterpret_cast<const uint2*>(&stage->codes[r][seg * 8]);
-      }
-    }
-    const int64_t bpr = p.cols / 16;
-    for (int i = tid; i < TILE * 8; i += THREADS) {
-      int r, b;
-      if (p.c_layout == METIS_SF_TILED) {   // walk the two 512-byte atoms in storage order
-        const int atom = i >> 9, w = i & 511;
-        r = (w >> 4) + 32 * ((w >> 2) & 3);
-        b = atom * 4 + (w & 3);
-      } else {
-        r = i >> 3; b = i & 7;
-      }
-      if (b * 16 < vcols && (r < vrows || p.c_layout == METIS_SF_TILED)) {
-        const uint8_t val = r < vrows ? stage->sf[r][b] : (uint8_t)0;
-        p.c_scales[metis_sf_offset(row0 + r, col0 / 16 + b, bpr, p.c_layout)] = val;
-      }
-    }
-    __syncthreads();
-  }
-
-  if (p.r_codes != nullptr) {
-    // blocks along rows: stored row = source column.  thread -> (col = tid % 128, row-blocks b = tid/128 + 2*it)
-#pragma unroll 1
-    for (int it = 0; it < 4; ++it) {
-      const int c = tid & 127, b = (tid >> 7) + 2 * it;
-      float v[16];
-      uint32_t u[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) v[i] = tile[(b * 16 + i) * PITCH + c];
-      if (sr) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) u[i] = rnd[(b * 16 + i) * TILE + c];
-      }
-      uint32_t packed[2];
-      const uint32_t byte = encode_block(v, u, sr, s_T, six_s_T, packed);
-      *reinterpret_cast<uint2*>(&stage->codes[c][b * 8]) = make_uint2(packed[0], packed[1]);
-      stage->sf[c][b] = (uint8_t)byte;
-    }
-    __syncthreads();
-    const int64_t kbytes = p.rows / 2;
-    for (int i = tid; i < TILE * 8; i += THREADS) {
-      const int c = i >> 3, seg = i & 7;
-      if (c < vcols && seg * 16 < vrows) {
-        *reinterpret_cast<uint2*>(p.r_codes + (col0 + c) * kbytes + row0 / 2 + seg * 8) =
-            *reinterpret_cast<const uint2*>(&stage->codes[c][seg * 8]);
-      }
-    }
-    const int64_t bpr = p.rows / 16;
-    for (int i = tid; i < TILE * 8; i += THREADS) {
-      int c, b;
-      if (p.r_layout == METIS_SF_TILED) {
-        const int atom = i >> 9, w = i & 511;
-        c = (w >> 4) + 32 * ((w >> 2) & 3);
-        b = atom * 4 + (w & 3);
-      } else {
-        c = i >> 3; b = i & 7;
-      }
-      if (b * 16 < vrows && (c < vcols || p.r_layout == METIS_SF_TILED)) {
-        const uint8_t val = c < vcols ? stage->sf[c][b] : (uint8_t)0;
-        p.r_scales[metis_sf_offset(col0 + c, row0 / 16 + b, bpr, p.r_layout)] = val;
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Fills the tile's 16-bit draws.  Fast path: elements consecutive along a row share Philox counters.
-__device__ __forceinline__ void fill_draws(uint16_t* rnd, const QuantParams& p, int64_t row0, int64_t col0) {
-  const int tid = threadIdx.x;
-  if (p.e_stride_c == 1 && (p.e_stride_r & 7) == 0 && (col0 & 7) == 0) {
-    for (int i = tid; i < TILE * (TILE / 8); i += THREADS) {
-      const int r = i >> 4, g = i & 15;
-      const uint64_t e = (uint64_t)(row0 + r) * (uint64_t)p.e_stride_r + (uint64_t)(col0 + g * 8);
-      const uint4 w = metis_philox_block(e >> 3, p.seed, p.stream_id);
-      uint4 out;
-      out.x = w.x; out.y = w.y; out.z = w.z; out.w = w.w;   // halves in order: low half of word 0 first
-      *reinterpret_cast<uint4*>(rnd + r * TILE + g * 8) = out;
-    }
-  } else {
-    for (int i = tid; i < TILE * TILE; i += THREADS) {
-      const int r = i >> 7, c = i & 127;
-      const uint64_t e = (uint64_t)(row0 + r) * (uint64_t)p.e_stride_r + (uint64_t)(col0 + c) * (uint64_t)p.e_stride_c;
-      rnd[i] = (uint16_t)metis_draw_u16(e, p.seed, p.stream_id);
-    }
-  }
-}
-
-constexpr size_t smem_bytes(bool sr) {
-  return sizeof(float) * TILE * PITCH + sizeof(Stage) + (sr ? sizeof(uint16_t) * TILE * TILE : 0);
 }
 
 }  // namespace metis_qt

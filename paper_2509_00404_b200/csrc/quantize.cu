@@ -8,13 +8,13 @@ namespace {
 // so that narrow rows do not idle the block, and one 32-bit division per unit finds the unit's place (a 64-bit division per
 // vector and scalar FP32 loads held the kernel at 3.3 TB/s for BF16 and 1.1 TB/s for FP32).  Units are walked
 // from the end of the tensor to its start: the quantizer that follows reads from the start, which is then what L2 holds.
-template <int DTYPE, bool VEC>
+template <int DTYPE>
 __global__ void __launch_bounds__(256)
 amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, int tpr, int narrow, uint32_t segs, uint32_t units, float* __restrict__ out) {
   // |x| as a bit pattern: non-negative floats order like their bit patterns, infinity above every number and a
   // NaN above infinity, so a non-finite element survives the reduction (fmaxf would drop a NaN)
   constexpr int UNROLL = 8;
-  constexpr int E = VEC ? (DTYPE == METIS_BF16 ? 8 : 4) : 1;                   // elements per load
+  constexpr int E = DTYPE == METIS_BF16 ? 8 : 4;           // elements per load
   uint32_t m = 0u;
   const int tx = threadIdx.x & (tpr - 1), ty = threadIdx.x / tpr, rpp = 256 / tpr;
   const int64_t vecs = cols / E;
@@ -27,17 +27,14 @@ amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, 
       // rows of at most tpr vectors: the unit is UNROLL row groups; longer rows: UNROLL steps along the row
       const int64_t r = narrow ? r0 + (int64_t)j * rpp : r0, c = narrow ? c0 : c0 + (int64_t)j * tpr;
       q[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (r < rows && c < vecs) {
-        if (VEC) q[j] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(x) + (r * ld + c * E) * (DTYPE == METIS_BF16 ? 2 : 4)));
-        else q[j].x = __float_as_uint(metis_ld_as_float(x, DTYPE, r * ld + c));
-      }
+      if (r < rows && c < vecs) q[j] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(x) + (r * ld + c * E) * (16 / E)));
     }
 #pragma unroll
     for (int j = 0; j < UNROLL; ++j) {
       const uint32_t w[4] = {q[j].x, q[j].y, q[j].z, q[j].w};
 #pragma unroll
-      for (int e = 0; e < (VEC ? 4 : 1); ++e) {
-        if (VEC && DTYPE == METIS_BF16) { m = max(m, (w[e] << 16) & 0x7FFFFFFFu); m = max(m, w[e] & 0x7FFF0000u); }
+      for (int e = 0; e < 4; ++e) {
+        if (DTYPE == METIS_BF16) { m = max(m, (w[e] << 16) & 0x7FFFFFFFu); m = max(m, w[e] & 0x7FFF0000u); }
         else m = max(m, w[e] & 0x7FFFFFFFu);
       }
     }
@@ -311,13 +308,14 @@ metis_status_t metis_quantize_set_attrs() {
 
 metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* amax_out,
                                  cudaStream_t s) {
-  METIS_CUDA_TRY(cudaMemsetAsync(amax_out, 0, sizeof(float), s));
-  if (rows * cols == 0) return METIS_OK;
   const bool bf = dtype == METIS_BF16;
   const int64_t e = bf ? 8 : 4;
-  const bool vec = cols % e == 0 && ld % e == 0 && metis_aligned16(x);
+  // the quantizer behind it wants the same of the operand: whole 16-byte loads
+  if (cols % e || ld % e || !metis_aligned16(x)) return METIS_ERR_ALIGNMENT;
+  METIS_CUDA_TRY(cudaMemsetAsync(amax_out, 0, sizeof(float), s));
+  if (rows * cols == 0) return METIS_OK;
   if (ld == cols) { cols = rows * cols; rows = 1; ld = cols; }                  // contiguous: one long row
-  const int64_t vecs = vec ? cols / e : cols;
+  const int64_t vecs = cols / e;
   int tpr = 256;
   while (tpr > 1 && tpr / 2 >= vecs) tpr /= 2;
   const bool narrow = vecs <= tpr;                                              // rows of at most one step of the block
@@ -326,10 +324,8 @@ metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t
   const int64_t units = groups * segs;
   if (units > 0xFFFFFFFFll) return METIS_ERR_SHAPE;
   const unsigned grid = (unsigned)(units < 148 * 8 ? units : 148 * 8);
-#define METIS_AMAX(DT, V) amax_kernel<DT, V><<<grid, 256, 0, s>>>(x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out)
-  if (bf) { if (vec) METIS_AMAX(METIS_BF16, true); else METIS_AMAX(METIS_BF16, false); }
-  else { if (vec) METIS_AMAX(METIS_FP32, true); else METIS_AMAX(METIS_FP32, false); }
-#undef METIS_AMAX
+  if (bf) amax_kernel<METIS_BF16><<<grid, 256, 0, s>>>(x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out);
+  else amax_kernel<METIS_FP32><<<grid, 256, 0, s>>>(x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out);
   METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
   return METIS_OK;

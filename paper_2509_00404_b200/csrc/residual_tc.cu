@@ -384,8 +384,6 @@ static metis_status_t make_map_codes(metis_context* ctx, CUtensorMap* map, const
 
 int metis_residual_kx(int kp) { return (6 * kp + 63) / 64 * 64; }
 
-bool metis_residual_tc_usable(const void* x, int64_t cols) { return metis_aligned16(x) && cols % 8 == 0; }
-
 // a6: [rows][kx] = per row [Ch|Ch|Cl|Ch|Cl2|Cl], b6: [cols][kx] = per column [Bh|Bl|Bh|Bl2|Bh|Bl] (BF16,
 // kx = metis_residual_kx(kp)).  b6 is filled by the caller; a6 too unless `coef` ([rows][kp] FP32) is given,
 // in which case it is written here first.

@@ -406,18 +406,17 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t&
   lo2 = pack_bf16(xr2, yr2);
 }
 
-// BF16 splits of the right basis in both operand orientations:
+// BF16 splits of the right basis:
 //   bs[t][j][col]  (col contiguous; B operand of C = x B, contraction over col); with more than 64 vectors the
 //                  layout is by groups of 64 vectors, bs[group][t][j in group][col], so that the three terms of a
 //                  group are one contiguous matrix (one launch of the coefficient kernel per group)
-//   bt[t][col][j]  (j contiguous, padded to kp; B operand of C B^T, contraction over j; optional)
+//   b6[col][kx]    (optional) per column the six K blocks [Bh | Bl | Bh | Bl2 | Bh | Bl] of the residual product
 __global__ void __launch_bounds__(128)
 basis_splits_kernel(const float* __restrict__ basis, int64_t cols, int k, int kp, __nv_bfloat16* __restrict__ bs,
-                    __nv_bfloat16* __restrict__ bt, __nv_bfloat16* __restrict__ b6, int kx) {
+                    __nv_bfloat16* __restrict__ b6, int kx) {
   metis_pdl_wait();
   const int64_t col = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (col >= cols) return;
-  // b6 (optional): [cols][kx], per column the six K blocks [Bh | Bl | Bh | Bl2 | Bh | Bl] of the residual product
   if (b6 != nullptr && blockIdx.y == 0)
     for (int z = 6 * kp; z < kx; z += 8) *reinterpret_cast<uint4*>(b6 + col * kx + z) = make_uint4(0u, 0u, 0u, 0u);
   {
@@ -436,108 +435,12 @@ basis_splits_kernel(const float* __restrict__ basis, int64_t cols, int k, int kp
 #pragma unroll
       for (int jj = 0; jj < 8; ++jj)
         bs[(row0 + jj) * cols + col] = __ushort_as_bfloat16((unsigned short)((w[t][jj >> 1] >> (16 * (jj & 1))) & 0xFFFFu));
-      if (bt != nullptr) *reinterpret_cast<uint4*>(bt + ((int64_t)t * cols + col) * kp + j0) = make_uint4(w[t][0], w[t][1], w[t][2], w[t][3]);
     }
     if (b6 != nullptr) {
       const int sel[6] = {0, 1, 0, 2, 0, 1};
 #pragma unroll
       for (int term = 0; term < 6; ++term)
         *reinterpret_cast<uint4*>(b6 + col * kx + term * kp + j0) = make_uint4(w[sel[term]][0], w[sel[term]][1], w[sel[term]][2], w[sel[term]][3]);
-    }
-  }
-}
-
-// Broadcast of the sampled subspace to every row (Section 3.1): C[r][j] = sum_col x[r, col] * B[j][col],
-// stored row-major with kp columns (zero padded).  One CTA = 32 rows; its 8 warps split the columns and
-// their partial tiles are added in fixed order.  Fused by-products of the same pass over x: amax|x|
-// (atomic max, order independent) and the FP64 Gram partial of the CTA's rows of C (for Rayleigh-Ritz).
-template <int KP>
-__global__ void __launch_bounds__(256)
-coeff_mma_kernel(const __nv_bfloat16* __restrict__ x, int64_t rows, int64_t cols, const __nv_bfloat16* __restrict__ bs,
-                 float* __restrict__ coef, float* __restrict__ amax_out, double* __restrict__ gram_part) {
-  metis_pdl_wait();
-  constexpr int NT = KP / 8;
-  extern __shared__ __align__(16) unsigned char smem[];
-  float* red = reinterpret_cast<float*>(smem);                 // [8 warps][32 rows][KP]
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int64_t row0 = (int64_t)blockIdx.x * 32;
-  const int ksteps = (int)(cols / 16);
-  const int ks_begin = (int)((int64_t)ksteps * warp / 8), ks_end = (int)((int64_t)ksteps * (warp + 1) / 8);
-  float acc[2][NT][4];
-#pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int n = 0; n < NT; ++n)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.0f;
-  uint32_t amax2 = 0u;                                         // two running |.| maxima, BF16 pair
-  const bool v0 = row0 + g < rows, v1 = row0 + g + 8 < rows, v2 = row0 + g + 16 < rows, v3 = row0 + g + 24 < rows;
-  const __nv_bfloat16* xr0 = x + (row0 + g) * cols;
-#pragma unroll 2
-  for (int ks = ks_begin; ks < ks_end; ++ks) {
-    const int kk = ks * 16 + 2 * t;
-    uint32_t a[2][4];
-    a[0][0] = v0 ? *reinterpret_cast<const uint32_t*>(xr0 + kk) : 0u;
-    a[0][1] = v1 ? *reinterpret_cast<const uint32_t*>(xr0 + 8 * cols + kk) : 0u;
-    a[0][2] = v0 ? *reinterpret_cast<const uint32_t*>(xr0 + kk + 8) : 0u;
-    a[0][3] = v1 ? *reinterpret_cast<const uint32_t*>(xr0 + 8 * cols + kk + 8) : 0u;
-    a[1][0] = v2 ? *reinterpret_cast<const uint32_t*>(xr0 + 16 * cols + kk) : 0u;
-    a[1][1] = v3 ? *reinterpret_cast<const uint32_t*>(xr0 + 24 * cols + kk) : 0u;
-    a[1][2] = v2 ? *reinterpret_cast<const uint32_t*>(xr0 + 16 * cols + kk + 8) : 0u;
-    a[1][3] = v3 ? *reinterpret_cast<const uint32_t*>(xr0 + 24 * cols + kk + 8) : 0u;
-#pragma unroll
-    for (int m = 0; m < 2; ++m)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const uint32_t ab = a[m][e] & 0x7FFF7FFFu;             // |.| of both halves; BF16 magnitudes order like integers
-        const uint32_t lo = max(ab & 0xFFFFu, amax2 & 0xFFFFu), hi = max(ab >> 16, amax2 >> 16);
-        amax2 = lo | (hi << 16);
-      }
-#pragma unroll
-    for (int sp = 0; sp < 3; ++sp) {
-      const __nv_bfloat16* bsp = bs + (int64_t)sp * KP * cols;
-#pragma unroll
-      for (int n = 0; n < NT; ++n) {
-        const __nv_bfloat16* bp = bsp + (int64_t)(n * 8 + g) * cols + kk;
-        const uint32_t b0 = *reinterpret_cast<const uint32_t*>(bp), b1 = *reinterpret_cast<const uint32_t*>(bp + 8);
-        mma_bf16(acc[0][n], a[0], b0, b1);
-        mma_bf16(acc[1][n], a[1], b0, b1);
-      }
-    }
-  }
-  // per-warp partial tile -> shared memory
-#pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      float* r0p = red + ((warp * 32) + m * 16 + g) * KP + n * 8 + 2 * t;
-      r0p[0] = acc[m][n][0]; r0p[1] = acc[m][n][1];
-      r0p[8 * KP] = acc[m][n][2]; r0p[8 * KP + 1] = acc[m][n][3];
-    }
-  {
-    uint32_t am = max((amax2 & 0xFFFFu) << 16, amax2 & 0xFFFF0000u);      // ordered bit patterns: a NaN survives
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xFFFFFFFFu, am, o));
-    if (lane == 0 && amax_out) atomicMax(reinterpret_cast<unsigned int*>(amax_out), am);
-  }
-  __syncthreads();
-  float* cfin = red + 8 * 32 * KP;                             // [32][KP] final tile
-  for (int o = tid; o < 32 * KP; o += 256) {
-    float sacc = 0.0f;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) sacc += red[w * 32 * KP + o];
-    cfin[o] = sacc;
-    const int64_t r = row0 + o / KP;
-    if (r < rows) coef[r * KP + (o % KP)] = sacc;
-  }
-  __syncthreads();
-  if (gram_part) {
-    for (int o = tid; o < KP * KP; o += 256) {
-      const int i = o / KP, j = o % KP;
-      double a = 0.0;
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) a += (double)cfin[r * KP + i] * (double)cfin[r * KP + j];
-      gram_part[(int64_t)blockIdx.x * KP * KP + o] = a;
     }
   }
 }
@@ -623,95 +526,6 @@ coef_finish_kernel(const float* __restrict__ part, int slices, int64_t rows, flo
       gram_part[(int64_t)blockIdx.x * KP * KP + o] = a;
     }
   }
-}
-
-// ------------------------------------------------------------------------------------------------
-// Fused residual + quantizer: R = x - C B^T on a 128 x 128 tile (tensor cores, three-term BF16 splits of
-// both FP32 operands), then NVFP4 in one or both block orientations straight from shared memory (the
-// residual never goes to HBM unless `dense` is given).  coef: [rows][KP] row-major, bt: [3][cols][KP].
-template <int KP>
-__global__ void __launch_bounds__(metis_qt::THREADS, 2)
-residual_quant_kernel(const __nv_bfloat16* __restrict__ x, const float* __restrict__ coef,
-                      const __nv_bfloat16* __restrict__ bt, metis_qt::QuantParams p,
-                      const float* __restrict__ amax_src, float* ts_out0, float* ts_out1, float* __restrict__ dense) {
-  metis_pdl_wait();
-  using namespace metis_qt;
-  extern __shared__ __align__(16) unsigned char smem[];
-  float* tile = reinterpret_cast<float*>(smem);
-  Stage* stage = reinterpret_cast<Stage*>(smem + sizeof(float) * TILE * PITCH);
-  uint16_t* rnd = reinterpret_cast<uint16_t*>(smem + sizeof(float) * TILE * PITCH + sizeof(Stage));
-  const bool sr = p.rounding == METIS_ROUND_SR;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int64_t row0 = (int64_t)blockIdx.y * TILE, col0 = (int64_t)blockIdx.x * TILE;
-  const float s_T = metis_tensor_scale(*amax_src);
-  if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
-    if (ts_out0) *ts_out0 = s_T;
-    if (ts_out1) *ts_out1 = s_T;
-  }
-  if (sr) fill_draws(rnd, p, row0, col0);
-  // this warp: rows row0 + 16*warp .. +15, all 128 columns
-  const int64_t ra = row0 + warp * 16 + g, rb = ra + 8;
-  const bool va = ra < p.rows, vb = rb < p.rows;
-  float acc[16][4];
-#pragma unroll
-  for (int n = 0; n < 16; ++n)
-#pragma unroll
-    for (int e = 0; e < 4; ++e) acc[n][e] = 0.0f;
-#pragma unroll
-  for (int ks = 0; ks < KP / 16; ++ks) {
-    const int kk = ks * 16 + 2 * t;
-    uint32_t ah[4], al[4], al2[4];
-    {
-      const float2 z = make_float2(0.0f, 0.0f);
-      const float2 c0 = va ? *reinterpret_cast<const float2*>(coef + ra * KP + kk) : z;
-      const float2 c1 = vb ? *reinterpret_cast<const float2*>(coef + rb * KP + kk) : z;
-      const float2 c2 = va ? *reinterpret_cast<const float2*>(coef + ra * KP + kk + 8) : z;
-      const float2 c3 = vb ? *reinterpret_cast<const float2*>(coef + rb * KP + kk + 8) : z;
-      split3(c0.x, c0.y, ah[0], al[0], al2[0]);
-      split3(c1.x, c1.y, ah[1], al[1], al2[1]);
-      split3(c2.x, c2.y, ah[2], al[2], al2[2]);
-      split3(c3.x, c3.y, ah[3], al[3], al2[3]);
-    }
-#pragma unroll
-    for (int n = 0; n < 16; ++n) {
-      const int64_t col = col0 + n * 8 + g;
-      uint32_t bh0 = 0, bh1 = 0, bl0 = 0, bl1 = 0, bm0 = 0, bm1 = 0;
-      if (col < p.cols) {
-        const __nv_bfloat16* bp = bt + col * KP + kk;
-        bh0 = *reinterpret_cast<const uint32_t*>(bp); bh1 = *reinterpret_cast<const uint32_t*>(bp + 8);
-        bl0 = *reinterpret_cast<const uint32_t*>(bp + p.cols * KP); bl1 = *reinterpret_cast<const uint32_t*>(bp + p.cols * KP + 8);
-        bm0 = *reinterpret_cast<const uint32_t*>(bp + 2 * p.cols * KP); bm1 = *reinterpret_cast<const uint32_t*>(bp + 2 * p.cols * KP + 8);
-      }
-      // smallest terms first
-      mma_bf16(acc[n], al, bl0, bl1);
-      mma_bf16(acc[n], al2, bh0, bh1);
-      mma_bf16(acc[n], ah, bm0, bm1);
-      mma_bf16(acc[n], al, bh0, bh1);
-      mma_bf16(acc[n], ah, bl0, bl1);
-      mma_bf16(acc[n], ah, bh0, bh1);
-    }
-  }
-  // R = x - acc into the shared tile (and to `dense` when asked)
-#pragma unroll
-  for (int n = 0; n < 16; ++n) {
-    const int64_t col = col0 + n * 8 + 2 * t;
-    const int lc = n * 8 + 2 * t;
-    float x00 = 0.0f, x01 = 0.0f, x10 = 0.0f, x11 = 0.0f;
-    if (col < p.cols) {
-      if (va) { const uint32_t w = *reinterpret_cast<const uint32_t*>(x + ra * p.cols + col); x00 = __uint_as_float(w << 16); x01 = __uint_as_float(w & 0xFFFF0000u); }
-      if (vb) { const uint32_t w = *reinterpret_cast<const uint32_t*>(x + rb * p.cols + col); x10 = __uint_as_float(w << 16); x11 = __uint_as_float(w & 0xFFFF0000u); }
-    }
-    const float2 r0v = make_float2(x00 - acc[n][0], x01 - acc[n][1]);
-    const float2 r1v = make_float2(x10 - acc[n][2], x11 - acc[n][3]);
-    *reinterpret_cast<float2*>(tile + (warp * 16 + g) * PITCH + lc) = (va && col < p.cols) ? r0v : make_float2(0.0f, 0.0f);
-    *reinterpret_cast<float2*>(tile + (warp * 16 + g + 8) * PITCH + lc) = (vb && col < p.cols) ? r1v : make_float2(0.0f, 0.0f);
-    if (dense != nullptr && col < p.cols) {
-      if (va) *reinterpret_cast<float2*>(dense + ra * p.cols + col) = r0v;
-      if (vb) *reinterpret_cast<float2*>(dense + rb * p.cols + col) = r1v;
-    }
-  }
-  __syncthreads();
-  quantize_tile(tile, rnd, stage, p, row0, col0, s_T);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1058,12 +872,12 @@ __device__ __forceinline__ void sign_contest(const float* Os, int k, int64_t p0,
   if (lane == 0 && top != 0u) atomicMax(reinterpret_cast<unsigned int*>(amax), top);
 }
 
-// Right basis B[j][col] = sum_i evecs[i][j] M[i][col] / s_j, s_j = sqrt(eval_j), and its BF16 splits (see basis_splits_kernel; bs,
-// bt and b6 are optional).  keys (FULL mode, where this is the right factor itself): the sign contest.
+// Right basis B[j][col] = sum_i evecs[i][j] M[i][col] / s_j, s_j = sqrt(eval_j), and its BF16 splits (see basis_splits_kernel; bs
+// is optional).  keys (FULL mode, where this is the right factor itself): the sign contest.
 template <int KT>
 __global__ void __launch_bounds__(256)
 basis_kernel(const float* __restrict__ m, int64_t cols, int q, int k, int kp, const double* __restrict__ evals, const double* __restrict__ evecs,
-             float* __restrict__ basis, __nv_bfloat16* __restrict__ bs, __nv_bfloat16* __restrict__ bt, __nv_bfloat16* __restrict__ b6, int kx,
+             float* __restrict__ basis, __nv_bfloat16* __restrict__ bs, __nv_bfloat16* __restrict__ b6, int kx,
              float* __restrict__ sigma_out, unsigned long long* __restrict__ keys, float* __restrict__ amax_out) {
   metis_pdl_wait();
   extern __shared__ __align__(16) double fr_sm[];
@@ -1101,30 +915,23 @@ basis_kernel(const float* __restrict__ m, int64_t cols, int q, int k, int kp, co
     for (int e = 0; e < 8; ++e) v[e] = Os[(j0 + e) * FR_OP + c];
     uint4 h, l, l2;
     metis_split3x8(v, h, l, l2);
-    if (bt != nullptr) {
-      *reinterpret_cast<uint4*>(bt + col * kp + j0) = h;
-      *reinterpret_cast<uint4*>(bt + (cols + col) * kp + j0) = l;
-      *reinterpret_cast<uint4*>(bt + (2 * cols + col) * kp + j0) = l2;
-    }
-    if (b6 != nullptr) {
-      __nv_bfloat16* dst = b6 + col * kx + j0;
-      *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + kp) = l; *reinterpret_cast<uint4*>(dst + 2 * kp) = h;
-      *reinterpret_cast<uint4*>(dst + 3 * kp) = l2; *reinterpret_cast<uint4*>(dst + 4 * kp) = h; *reinterpret_cast<uint4*>(dst + 5 * kp) = l;
-      if (j0 == 0)
-        for (int z = 6 * kp; z < kx; z += 8) *reinterpret_cast<uint4*>(b6 + col * kx + z) = make_uint4(0u, 0u, 0u, 0u);
-    }
+    __nv_bfloat16* dst = b6 + col * kx + j0;
+    *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + kp) = l; *reinterpret_cast<uint4*>(dst + 2 * kp) = h;
+    *reinterpret_cast<uint4*>(dst + 3 * kp) = l2; *reinterpret_cast<uint4*>(dst + 4 * kp) = h; *reinterpret_cast<uint4*>(dst + 5 * kp) = l;
+    if (j0 == 0)
+      for (int z = 6 * kp; z < kx; z += 8) *reinterpret_cast<uint4*>(b6 + col * kx + z) = make_uint4(0u, 0u, 0u, 0u);
   }
   if (keys != nullptr) sign_contest(Os, k, p0, cols, keys, amax_out);
 }
 
 // The factors of a decomposition, unsigned.  Blocks below n_right: right[j][col] = sum_i basis[i][col] W[i][j] and the sign contest;
 // the others: left[j][r] = s_j sum_i src[r * ld + i] W[i][j] with s_j = 1 / sqrt(eval_j) when evals is given (Rayleigh-Ritz; sigma_out = sqrt(eval_j)),
-// and from it the coefficients left * sigma of the residual product (FULL mode): as its BF16 operand a6, or as coef [r][kp].
+// and from it the coefficients left * sigma of the residual product (FULL mode) as its BF16 operand a6.
 struct FactorsArgs {
   const double* w; int ldw, n_in, k, kp;
   const float* basis; int64_t cols; float* right; unsigned long long* keys; float* amax_right;
   const float* src; int64_t ld, rows; const double* evals; float* left; float* sigma_out; float* amax_left;
-  const float* sigma_for_coef; float* coef; __nv_bfloat16* a6; int kx;
+  const float* sigma_for_coef; __nv_bfloat16* a6; int kx;
 };
 template <int KT>
 __global__ void __launch_bounds__(256)
@@ -1170,18 +977,13 @@ factors_kernel(FactorsArgs f, int n_right) {
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = j0 + e < k ? Os[(j0 + e) * FR_OP + c] * f.sigma_for_coef[j0 + e] : 0.0f;
-    if (f.a6 != nullptr) {
-      uint4 h, l, l2;
-      metis_split3x8(v, h, l, l2);
-      __nv_bfloat16* dst = f.a6 + r * f.kx + j0;
-      *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + kp) = h; *reinterpret_cast<uint4*>(dst + 2 * kp) = l;
-      *reinterpret_cast<uint4*>(dst + 3 * kp) = h; *reinterpret_cast<uint4*>(dst + 4 * kp) = l2; *reinterpret_cast<uint4*>(dst + 5 * kp) = l;
-      if (j0 == 0)
-        for (int z = 6 * kp; z < f.kx; z += 8) *reinterpret_cast<uint4*>(f.a6 + r * f.kx + z) = make_uint4(0u, 0u, 0u, 0u);
-    } else {
-#pragma unroll
-      for (int e = 0; e < 8; ++e) f.coef[r * kp + j0 + e] = v[e];
-    }
+    uint4 h, l, l2;
+    metis_split3x8(v, h, l, l2);
+    __nv_bfloat16* dst = f.a6 + r * f.kx + j0;
+    *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + kp) = h; *reinterpret_cast<uint4*>(dst + 2 * kp) = l;
+    *reinterpret_cast<uint4*>(dst + 3 * kp) = h; *reinterpret_cast<uint4*>(dst + 4 * kp) = l2; *reinterpret_cast<uint4*>(dst + 5 * kp) = l;
+    if (j0 == 0)
+      for (int z = 6 * kp; z < f.kx; z += 8) *reinterpret_cast<uint4*>(f.a6 + r * f.kx + z) = make_uint4(0u, 0u, 0u, 0u);
   }
 }
 
@@ -1193,7 +995,7 @@ int sketch_tc_cols(int q) { return q <= 48 ? 48 : 96; }
 int sketch_chunk_cols(int64_t n_s) { return n_s <= 512 ? 64 : SKM_COLS; }
 
 struct SplitWs {
-  size_t amax, idx, zp, omt, z, gram, gram1, linv, evals, evecs, mp, m, basis, coef, keys, evals2, evecs2, bs, bt,
+  size_t amax, idx, zp, omt, z, gram, gram1, linv, evals, evecs, mp, m, basis, coef, keys, evals2, evecs2, bs,
       gram_c, part, a6, b6, hsp, total;
 };
 
@@ -1243,7 +1045,6 @@ SplitWs split_ws_layout(int64_t rows, int64_t cols, int k, int p, int64_t n_s) {
   w.b6 = take(sizeof(__nv_bfloat16) * (size_t)metis_residual_kx(kp) * cols);
   w.hsp = take(n_s >= 1024 ? sizeof(__nv_bfloat16) * 3 * (size_t)((q + 15) / 16 * 16) * (size_t)((n_s + 63) / 64 * 64) : 0);
   w.bs = take(sizeof(__nv_bfloat16) * 3 * (size_t)kp * cols);
-  w.bt = take(sizeof(__nv_bfloat16) * 3 * (size_t)kp * cols);
   w.gram_c = take(sizeof(double) * (size_t)metis_ceil_div(rows, 32) * kp * kp);
   w.keys = take(sizeof(unsigned long long) * MAXQ);
   w.evals2 = take(sizeof(double) * MAXQ);
@@ -1293,8 +1094,8 @@ metis_status_t launch_orth_apply(cudaStream_t s, float* z, int64_t n_s, int q, c
 }
 template <int KT>
 metis_status_t launch_basis_kt(cudaStream_t s, int ctas, size_t smem, const float* m, int64_t cols, int q, int k, int kp, const double* evals, const double* evecs, float* basis,
-                               __nv_bfloat16* bs, __nv_bfloat16* bt, __nv_bfloat16* b6, int kx, float* sigma_out, unsigned long long* keys, float* amax_out) {
-  METIS_CUDA_TRY(metis_launch_pdl((basis_kernel<KT>), dim3((unsigned)ctas), dim3(256), smem, s, m, cols, q, k, kp, evals, evecs, basis, bs, bt, b6, kx, sigma_out, keys, amax_out));
+                               __nv_bfloat16* bs, __nv_bfloat16* b6, int kx, float* sigma_out, unsigned long long* keys, float* amax_out) {
+  METIS_CUDA_TRY(metis_launch_pdl((basis_kernel<KT>), dim3((unsigned)ctas), dim3(256), smem, s, m, cols, q, k, kp, evals, evecs, basis, bs, b6, kx, sigma_out, keys, amax_out));
   METIS_COUNT_LAUNCH();
   return METIS_OK;
 }
@@ -1571,7 +1372,7 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
   if (full) {
     // right = basis with the sign convention, left = H U~_k (same flips), coefficients = left * sigma
     METIS_CUDA_TRY(metis_launch_pdl(metis_wide::sign_rows_kernel, dim3((unsigned)k), dim3(256), (size_t)0, s, out->right, cols, sign, amax + 2)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((basis_splits_kernel), bs_grid, dim3(128), (size_t)(0), s, (const float*)out->right, cols, k, kp, bs, (__nv_bfloat16*)nullptr, b6, kx6)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((basis_splits_kernel), bs_grid, dim3(128), (size_t)(0), s, (const float*)out->right, cols, k, kp, bs, b6, kx6)); METIS_COUNT_LAUNCH();
     METIS_CUDA_TRY(metis_launch_pdl(metis_wide::rot_scales_kernel, dim3((unsigned)metis_ceil_div(k, 128)), dim3(128), (size_t)0, s, (const double*)evals, (const float*)sign, k, 2,
                                     scale, (float*)nullptr)); METIS_COUNT_LAUNCH();
     if (kp > k) METIS_CUDA_TRY(cudaMemsetAsync(coef, 0, sizeof(float) * (size_t)kp * rows, s));
@@ -1582,7 +1383,7 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
     METIS_TRY(metis_fork(ctx, s, 1));
     METIS_TRY(metis_launch_residual_tc(ctx, x, coef, k, kp, qp, amax, t0, t1, residual_dense, a6, b6, s));
   } else {
-    METIS_CUDA_TRY(metis_launch_pdl((basis_splits_kernel), bs_grid, dim3(128), (size_t)(0), s, (const float*)basis, cols, k, kp, bs, (__nv_bfloat16*)nullptr, b6, kx6)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((basis_splits_kernel), bs_grid, dim3(128), (size_t)(0), s, (const float*)basis, cols, k, kp, bs, b6, kx6)); METIS_COUNT_LAUNCH();
     // (5) broadcast C = x B, WIDE_CG basis vectors per pass over x
     const int slices = metis_coeff_slices(rows, cols, nullptr);
     for (int j0 = 0; j0 < kp; j0 += WIDE_CG) {
@@ -1630,7 +1431,6 @@ int64_t metis_default_sample_count(int64_t rows, int32_t q) {
 }
 
 metis_status_t metis_split_set_attrs() {
-  using namespace metis_qt;
 #define METIS_OA_ATTR(KT) METIS_CUDA_TRY(cudaFuncSetAttribute(orth_apply_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oa_smem(KT)))
   METIS_OA_ATTR(1); METIS_OA_ATTR(2); METIS_OA_ATTR(3); METIS_OA_ATTR(4); METIS_OA_ATTR(5); METIS_OA_ATTR(6); METIS_OA_ATTR(7); METIS_OA_ATTR(8); METIS_OA_ATTR(9);
 #undef METIS_OA_ATTR
@@ -1642,12 +1442,6 @@ metis_status_t metis_split_set_attrs() {
 #define METIS_EIG_ATTR(NT8) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_small::eig_kernel<NT8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_small::eig_smem(8 * NT8)))
   METIS_EIG_ATTR(1); METIS_EIG_ATTR(2); METIS_EIG_ATTR(3); METIS_EIG_ATTR(4); METIS_EIG_ATTR(5); METIS_EIG_ATTR(6); METIS_EIG_ATTR(7); METIS_EIG_ATTR(8); METIS_EIG_ATTR(9);
 #undef METIS_EIG_ATTR
-  METIS_CUDA_TRY(cudaFuncSetAttribute(coeff_mma_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * 9 * 32 * 64)));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(coeff_mma_kernel<48>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * 9 * 32 * 48)));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(residual_quant_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true)));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(residual_quant_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true)));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(residual_quant_kernel<48>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true)));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(residual_quant_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes(true)));
   METIS_CUDA_TRY(cudaFuncSetAttribute(gram_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GC_MAX_SMEM));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::JC_SMEM));
 #define METIS_JF_ATTR(LN, R) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_fp32_kernel<LN, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::jf_smem(LN, R)))
@@ -1744,7 +1538,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   if (k == 0) n_s = 16;
   if (wide) {
     // the tensor-core passes carry the wide path: 16-byte aligned rows of x, whole 64-column chunks
-    if (cols % 64 || rows % 64 || (!packed && !metis_residual_tc_usable(xv, cols))) return METIS_ERR_SHAPE;
+    if (cols % 64 || rows % 64) return METIS_ERR_SHAPE;
     const WideWs W = wide_ws_layout(rows, cols, k, p, n_s, full);
     if (ws_bytes < W.total + pack_bytes) return METIS_ERR_WORKSPACE;
     if (!out->left || !out->sigma || !out->right || !out->left_q.codes || !out->right_q.codes || !out->left_q.scales ||
@@ -1804,18 +1598,13 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   double* evals2 = reinterpret_cast<double*>(wsb + L.evals2);
   double* evecs2 = reinterpret_cast<double*>(wsb + L.evecs2);
   __nv_bfloat16* bs = reinterpret_cast<__nv_bfloat16*>(wsb + L.bs);
-  __nv_bfloat16* bt = reinterpret_cast<__nv_bfloat16*>(wsb + L.bt);
   double* gram_c = reinterpret_cast<double*>(wsb + L.gram_c);
   float* part = reinterpret_cast<float*>(wsb + L.part);
   __nv_bfloat16* hsp = reinterpret_cast<__nv_bfloat16*>(wsb + L.hsp);
-  void* a6 = wsb + L.a6;
-  void* b6 = wsb + L.b6;
+  __nv_bfloat16* a6 = reinterpret_cast<__nv_bfloat16*>(wsb + L.a6);
+  __nv_bfloat16* b6 = reinterpret_cast<__nv_bfloat16*>(wsb + L.b6);
   // the residual kernel's K-concatenated BF16 operands are written by the kernels that produce coefficients and basis
-  const bool resid_tc = metis_residual_tc_usable(x, cols);
   const int kx6 = metis_residual_kx((k + 15) / 16 * 16);
-  __nv_bfloat16* a6p = resid_tc ? reinterpret_cast<__nv_bfloat16*>(a6) : nullptr;
-  __nv_bfloat16* b6p = resid_tc ? reinterpret_cast<__nv_bfloat16*>(b6) : nullptr;
-  bool a6_ready = false;
   metis_context* ctx = h;
   const int kp = (k + 15) / 16 * 16;
   // (1) row sample (clears the amax slots of x, left and right, the condition flag and the sign keys), (2) sketch (tensor cores; Omega
@@ -1938,36 +1727,23 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   const int n_cta_c = (int)metis_ceil_div(rows, 32);
   const int n_cta_cols = (int)metis_ceil_div(cols, FR_POS), n_cta_rows = (int)metis_ceil_div(rows, FR_POS);
   float* rb = full ? out->right : basis;
-  __nv_bfloat16* btp = resid_tc ? nullptr : bt;
-  METIS_TRY(launch_basis(s, n_cta_cols, fr_smem(q), m, cols, q, k, kp, evals, evecs, rb, full ? (__nv_bfloat16*)nullptr : bs, btp, b6p, kx6, full ? out->sigma : nullptr, full ? keys : nullptr, amax + 2));
+  METIS_TRY(launch_basis(s, n_cta_cols, fr_smem(q), m, cols, q, k, kp, evals, evecs, rb, full ? (__nv_bfloat16*)nullptr : bs, b6, kx6, full ? out->sigma : nullptr, full ? keys : nullptr, amax + 2));
   if (full) {
-    // left = H U~_k; coefficients = left * sigma, as the residual product's operand where the tensor-core pass runs
+    // left = H U~_k; coefficients = left * sigma, as the residual product's operand
     FactorsArgs f{};
     f.w = evecs; f.ldw = q; f.n_in = q; f.k = k; f.kp = kp;
     f.src = z; f.ld = q; f.rows = rows; f.left = out->left; f.amax_left = amax + 1;
-    f.sigma_for_coef = out->sigma; f.coef = coef; f.a6 = a6p; f.kx = kx6;
+    f.sigma_for_coef = out->sigma; f.a6 = a6; f.kx = kx6;
     METIS_TRY(launch_factors(s, f, 0, n_cta_rows));
-    a6_ready = resid_tc;
   } else {
-    if (metis_coeff_tc_usable(x, bs, cols, kp)) {
-      // tensor-core pass over x (column slices), then the slices are summed and the Gram partials formed
-      METIS_TRY(metis_launch_coeff_tc(ctx, x, rows, cols, bs, kp, part, amax, 0, s));
-      a6_ready = resid_tc;
-      const int slices = metis_coeff_slices(rows, cols, nullptr);
-      switch (kp) {
-        case 16: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<16>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6p, kx6)); break;
-        case 32: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<32>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6p, kx6)); break;
-        case 48: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<48>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6p, kx6)); break;
-        default: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<64>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6p, kx6)); break;
-      }
-    } else {
-      const size_t smem = sizeof(float) * 9 * 32 * kp;
-      switch (kp) {
-        case 16: METIS_CUDA_TRY(metis_launch_pdl((coeff_mma_kernel<16>), dim3(n_cta_c), dim3(256), (size_t)(smem), s, x, rows, cols, bs, coef, amax, gram_c)); break;
-        case 32: METIS_CUDA_TRY(metis_launch_pdl((coeff_mma_kernel<32>), dim3(n_cta_c), dim3(256), (size_t)(smem), s, x, rows, cols, bs, coef, amax, gram_c)); break;
-        case 48: METIS_CUDA_TRY(metis_launch_pdl((coeff_mma_kernel<48>), dim3(n_cta_c), dim3(256), (size_t)(smem), s, x, rows, cols, bs, coef, amax, gram_c)); break;
-        default: METIS_CUDA_TRY(metis_launch_pdl((coeff_mma_kernel<64>), dim3(n_cta_c), dim3(256), (size_t)(smem), s, x, rows, cols, bs, coef, amax, gram_c)); break;
-      }
+    // tensor-core pass over x (column slices), then the slices are summed and the Gram partials formed
+    METIS_TRY(metis_launch_coeff_tc(ctx, x, rows, cols, bs, kp, part, amax, 0, s));
+    const int slices = metis_coeff_slices(rows, cols, nullptr);
+    switch (kp) {
+      case 16: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<16>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
+      case 32: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<32>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
+      case 48: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<48>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
+      default: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<64>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
     }
     METIS_COUNT_LAUNCH();
   }
@@ -1977,25 +1753,12 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     qp.e_stride_r = cols; qp.e_stride_c = 1;
     if (want_c) { qp.c_codes = rc.codes; qp.c_scales = rc.scales; qp.c_layout = rc.sf_layout; }
     if (want_r) { qp.r_codes = rr.codes; qp.r_scales = rr.scales; qp.r_layout = rr.sf_layout; }
-    const size_t smem = smem_bytes(rounding == METIS_ROUND_SR);
-    dim3 grid((unsigned)metis_ceil_div(cols, TILE), (unsigned)metis_ceil_div(rows, TILE));
     float* t0 = want_c ? rc.tensor_scale : nullptr; float* t1 = want_r ? rr.tensor_scale : nullptr;
     // the big residual pass and the small factor chain below are independent from here on: the factor chain
     // goes to a (high-priority) side stream and is joined back at the end of the call
     METIS_TRY(metis_fork(ctx, s, 1));
-    cudaStream_t sr = s;
-    if (resid_tc) {
-      METIS_TRY(metis_launch_residual_tc(ctx, x, a6_ready ? nullptr : coef, k, kp, qp, amax, t0, t1, residual_dense, a6, b6, sr));
-    } else {
-      switch (kp) {
-        case 16: METIS_CUDA_TRY(metis_launch_pdl((residual_quant_kernel<16>), dim3(grid), dim3(THREADS), (size_t)(smem), sr, x, coef, bt, qp, amax, t0, t1, residual_dense)); break;
-        case 32: METIS_CUDA_TRY(metis_launch_pdl((residual_quant_kernel<32>), dim3(grid), dim3(THREADS), (size_t)(smem), sr, x, coef, bt, qp, amax, t0, t1, residual_dense)); break;
-        case 48: METIS_CUDA_TRY(metis_launch_pdl((residual_quant_kernel<48>), dim3(grid), dim3(THREADS), (size_t)(smem), sr, x, coef, bt, qp, amax, t0, t1, residual_dense)); break;
-        default: METIS_CUDA_TRY(metis_launch_pdl((residual_quant_kernel<64>), dim3(grid), dim3(THREADS), (size_t)(smem), sr, x, coef, bt, qp, amax, t0, t1, residual_dense)); break;
-      }
-      METIS_COUNT_LAUNCH();
-    }
-    METIS_CUDA_TRY(metis_launch_pdl((split_status_kernel), dim3(1), dim3(32), (size_t)(0), sr, amax, evals, k, ctx->dev_status)); METIS_COUNT_LAUNCH();
+    METIS_TRY(metis_launch_residual_tc(ctx, x, nullptr, k, kp, qp, amax, t0, t1, residual_dense, a6, b6, s));
+    METIS_CUDA_TRY(metis_launch_pdl((split_status_kernel), dim3(1), dim3(32), (size_t)(0), s, amax, evals, k, ctx->dev_status)); METIS_COUNT_LAUNCH();
   }
   cudaStream_t sf = ctx->side[0];
   if (!full) {
