@@ -1,5 +1,5 @@
-"""GPU: the debug build of the library (METIS_DEBUG=1) - every store of codes and scales of the quantizing kernels is
-checked against the extent of its buffer; a store that would fall outside is skipped and reported through the device
+"""GPU: the debug build of the library (METIS_DEBUG=1) - every store of codes and scales of the tile quantizer and the
+residual pass is checked against the extent of its buffer; a store that would fall outside is skipped and reported through the device
 status word.  compute-sanitizer is not available, so this build is what stands in for it.  The library is loaded once
 per process, so the debug library runs in a child process."""
 import os

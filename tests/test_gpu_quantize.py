@@ -155,8 +155,8 @@ def test_random_hadamard_recipe_matches_the_oracle_byte_for_byte(case):
 @pytest.mark.parametrize("rows,cols,pad", [(16, 64, 0), (16, 64, 8), (33, 64, 4), (130, 1088, 64), (70, 2112, 16), (64, 16448, 4), (3, 16448, 64), (4096, 2112, 0)])
 def test_tensor_amax_sees_every_element(ctx, dtype, rows, cols, pad):
     """The tensor scale is amax / 2688 whichever element is the largest: corners, the ends of a row, a middle row, and every
-    column of one row (operands of one short row group, rows of several segments, strided rows whose starts do or do not
-    allow 16-byte loads).  The columns beyond the operand hold larger values and must not count."""
+    column of one row (operands of one short row group, rows of several segments, contiguous ones and strided ones, whose rows
+    always start on 16-byte boundaries).  The columns beyond the operand hold larger values and must not count."""
     B, h = ctx
     if dtype == torch.bfloat16 and pad % 8:
         pad += 4                                     # the library wants rows on 16-byte boundaries

@@ -429,3 +429,56 @@ def test_wide_eigen_solver_sizes_and_spectra(ctx, k, p, spectrum):
     core = left @ xd @ right.T
     assert (core - torch.diag(torch.diagonal(core))).abs().max() < 1e-6 * sig[0]
     assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
+
+
+def _planted(rows, cols, k, spectrum, seed):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    u = torch.linalg.qr(torch.randn((rows, k), generator=g, device="cuda", dtype=torch.float64))[0]
+    v = torch.linalg.qr(torch.randn((cols, k), generator=g, device="cuda", dtype=torch.float64))[0]
+    i = torch.arange(k, device="cuda", dtype=torch.float64)
+    s = {"geometric": 3000.0 * 10 ** (-i / k), "equal": 1000.0 + 0 * i, "half": torch.where(i < k // 2, 1000.0 + 0 * i, 900.0 - 2 * i),
+         "close": 1000.0 * (1 + 1e-6 * i), "apart": 1000.0 * (1 + 1e-4 * i), "decades": 3000.0 * 10 ** (-3 * i / k)}[spectrum]
+    return ((u * s) @ v.T + 0.05 * torch.randn((rows, cols), generator=g, device="cuda", dtype=torch.float64)).to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("k,p", [(4, 4), (12, 0), (36, 7), (64, 8), (68, 4), (96, 1), (136, 24), (160, 3), (220, 5), (256, 16)])
+@pytest.mark.parametrize("spectrum", ["half", "close", "apart", "decades"])
+def test_eigen_solvers_of_graded_and_nearly_equal_spectra(ctx, k, p, spectrum):
+    """What the number of refinement steps and the choice of the solver that finishes a matrix are decided on: singular values of which
+    half agree, that agree to 1e-6 and to 1e-4, and that fall by three decades.  A right vector is a combination of FP32 rows (2^-24
+    each) of the largest singular value's size divided by its own singular value, so its errors carry their ratio."""
+    B, h = ctx
+    x = _planted(768, 640, k, spectrum, 100 * k + p)
+    op = h.split(x, k, p, sketch=B.SKETCH_FULL, seed=11)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    left, right, sig, xd = op.left.double(), op.right.double(), op.sigma.double(), x.double()
+    eye = torch.eye(k, device="cuda", dtype=torch.float64)
+    tol = 1e-6 + 2.0 ** -23 * float(sig[0] / sig[-1])
+    assert (left @ left.T - eye).abs().max() < 1e-6 and (right @ right.T - eye).abs().max() < tol
+    core = left @ xd @ right.T
+    assert (core - torch.diag(torch.diagonal(core))).abs().max() < tol * sig[0]
+    assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
+    assert bool((sig[:-1] >= sig[1:]).all())
+
+
+@pytest.mark.parametrize("k,p", [(4, 4), (20, 5), (32, 8), (64, 8), (96, 9), (128, 8), (256, 16)])
+@pytest.mark.parametrize("spectrum", ["geometric", "equal", "half", "close", "decades"])
+def test_eigen_solvers_of_sampled_splits(ctx, k, p, spectrum):
+    """The two solves of a SAMPLED split (sampled rows, Rayleigh-Ritz): whatever rows were drawn, the right factor is orthonormal and so is
+    X R / sigma.  Bounds as above, for the basis and the coefficients and with the accumulation of the coefficients over 640 columns
+    (2^-21 times the ratio of the singular values)."""
+    B, h = ctx
+    x = _planted(1536, 640, k, spectrum, 100 * k + p)
+    op = h.split(x, k, p, sketch=B.SKETCH_SAMPLED, seed=11)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    left, right, sig, xd = op.left.double(), op.right.double(), op.sigma.double(), x.double()
+    eye = torch.eye(k, device="cuda", dtype=torch.float64)
+    tol = 1e-6 + 2.0 ** -21 * float(sig[0] / sig[-1])
+    assert (left @ left.T - eye).abs().max() < tol and (right @ right.T - eye).abs().max() < tol
+    core = left @ xd @ right.T
+    assert (core - torch.diag(torch.diagonal(core))).abs().max() < tol * sig[0]
+    assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
+    assert bool((sig[:-1] >= sig[1:]).all())
