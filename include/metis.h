@@ -142,9 +142,9 @@ metis_status_t metis_debug_timestamp(metis_handle_t h, uint64_t* device_slot, me
  * returns normally; the context stays usable. */
 metis_status_t metis_debug_wait_timeout(metis_handle_t h, uint32_t polls, uint32_t* device_seen, metis_stream_t stream);
 
-/* Debug build (compiled with METIS_DEBUG_BUILD; the Python binding loads it when METIS_DEBUG=1): the quantizing kernels
- * check every global store of codes and scales against the extent of its output buffer and, instead of storing out
- * of range, skip the store and set METIS_DEV_INDEX in the device status word.  metis_debug_build() tells which
+/* Debug build (compiled with METIS_DEBUG_BUILD; the Python binding loads it when METIS_DEBUG=1): the tile quantizer and
+ * the residual pass of a split check every global store of codes and scales (tensor copies by their column and row
+ * ranges) against the extent of its output buffer and, instead of storing out of range, skip the store and set METIS_DEV_INDEX in the device status word.  metis_debug_build() tells which
  * library this is (1 = debug).  metis_debug_index_check runs the same check in a one-thread kernel on a made-up
  * store of nbytes at `offset` into a buffer of `extent` bytes (nothing is accessed): the self-test of the mechanism. */
 int32_t metis_debug_build(void);

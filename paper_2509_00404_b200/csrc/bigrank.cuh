@@ -3,12 +3,13 @@
 // (Section 3.1: thin QR of the sketch, small SVD of the projected operand), as kernels that tile over the rank:
 //
 //   gram64_kernel            G = V^T V in FP64, 64 x 64 output tiles over slabs of rows (partials, summed in order)
-//   chol_wide_kernel         blocked Cholesky factor of a q x q Gram matrix (panels of 32 columns in shared memory,
-//                            the matrix in L2) and the inverses of its diagonal blocks, one CTA
+//   chol_mid_kernel          Cholesky factor of a q x q Gram matrix and the inverses of its diagonal blocks, one CTA: q up to
+//                            160, the matrix in shared memory
+//   chol_wide_kernel         the same above that: panels of 32 columns in shared memory, the matrix in L2
 //   trsm_wide_kernel         H = Z L^-T by blocked forward substitution (32 rows of Z per CTA)
 //   gemm64_kernel            C = A B with FP32 A, FP64 B and FP64 accumulation, arbitrary strides (right basis,
 //                            factor rotations)
-//   jacobi_fp32_kernel       FP32 one-sided block Jacobi on a cluster of up to eight CTAs: the columns live in the cluster's
+//   jacobi_fp32_kernel       FP32 one-sided block Jacobi on a cluster of two to six CTAs: the columns live in the cluster's
 //                            distributed shared memory, column blocks travel between CTAs by DSMEM stores
 //   refine_*_kernel          FP64 refinement of the eigenvectors it found (steps of matrix products), eigen_finish_kernel
 //   jacobi_cluster_kernel    the FP64 form of the sweeps, and jacobi_collect_kernel: only run for matrices the refinement
@@ -31,7 +32,7 @@ constexpr int MAXK_WIDE = 256;
 
 // ------------------------------------------------------------------------------------------------
 // part[p][i][j] = sum over the p-th slab of rows r of v(r, i) v(r, j),  v(r, i) = V[r * sr + i * sv], FP64.
-// grid (tiles_j, tiles_i, slabs); the 16 x 16 threads of a CTA own 4 x 4 outputs each.
+// grid (tiles_j, tiles_i, slabs).
 // On the FP64 tensor cores: a warp owns 16 x 32 of the tile; tiles above the diagonal are the mirror image of those below it
 // (as FP64 multiply-adds from shared memory over all tiles a rank-128 step spent 305 us on it, 190 us so).
 constexpr int G64_T = 64, G64_R = 32, G64_P = G64_T + 4;
@@ -90,12 +91,8 @@ gram64_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t sr, in
 }
 
 // ------------------------------------------------------------------------------------------------
-// Cholesky factor of the n x n Gram matrix g (n <= MAXQ_WIDE), one CTA of 1024 threads, blocked by panels of
-// CW_NB columns (left-looking): a panel is the Gram panel minus the product of the finished columns of its rows
-// with those of its own CW_NB rows - staged through shared memory in chunks of CW_NB columns, so the finished
-// part of L is read once per panel - and is then factorised inside shared memory.  The matrix itself (half a
-// megabyte in FP64) stays in global memory.  A pivot not above tol_rel * (largest diagonal entry) marks a
-// dependent sketch column: its column of L and its row and column of the diagonal-block inverse are zero.
+// Cholesky factor of the n x n Gram matrix g (symmetric to the bit, n <= MAXQ_WIDE).  A pivot not above tol_rel * (largest
+// diagonal entry) marks a dependent sketch column: its column of L and its row and column of the diagonal-block inverse are zero.
 //   l_out     n x n row-major lower factor (strict upper part zero)
 //   dinv_out  (optional) inverses of the CW_NB x CW_NB diagonal blocks of L, [panel][CW_NB][CW_NB] row-major lower:
 //             what the triangular solve H = Z L^-T needs besides L itself (trsm_wide_kernel)
@@ -108,7 +105,7 @@ constexpr int CW_ROWS = (MAXQ_WIDE + 31) / 32 * 32;
 constexpr int CW_RT = (CW_ROWS / 8 + CW_WARPS - 1) / CW_WARPS;                 // row tiles per warp
 constexpr size_t CW_SMEM = sizeof(double) * ((size_t)2 * CW_ROWS * CW_P + CW_NB * CW_P);
 
-// Blocked (left-looking) Cholesky factor of the n x n matrix g (symmetrised on the fly), one CTA, panels of 32 columns:
+// One CTA, left-looking, panels of 32 columns; the matrix itself (half a megabyte in FP64) stays in global memory:
 //   1. the panel (rows j0 .. n-1) minus the products with the finished columns on the FP64 tensor cores, the finished columns
 //      streamed from global memory (L2) in chunks of 32, the next chunk on its way while one is multiplied;
 //   2. the 32 x 32 diagonal block factorised by one warp in registers (lane = row; a column step is one pivot broadcast, one
@@ -117,8 +114,6 @@ constexpr size_t CW_SMEM = sizeof(double) * ((size_t)2 * CW_ROWS * CW_P + CW_NB 
 //   4. the rows below the block:  L = A X^T  with X the inverse, on the tensor cores.
 // With FP64 multiply-adds from shared memory and a column of the diagonal block per shared-memory round trip the
 // factorisation took 138 us at n = 136; this form takes 104 us, and 286 us at n = 264.
-// A pivot at or below tol_rel * max diag gives a zero column.  l_out: the factor (lower triangle, zeros above);
-// dinv_out: the inverses of the diagonal blocks (32 x 32 each) for the blocked triangular solve.
 struct EigState;
 __device__ __forceinline__ void eig_state_reset(EigState* st, int tid);
 __global__ void __launch_bounds__(CW_THREADS, 1)
@@ -487,7 +482,8 @@ __global__ void rot_scales_kernel(const double* __restrict__ evals, const float*
 // finish (pairs of eigenvalues too close, or no convergence) is done by the FP64 Jacobi kernels, which otherwise return at
 // once.  The decisions are made on the device, in EigState, so that a call needs no host synchronisation.
 // Measured inside a layer step, n = 136: factorisation, solver and collection 138 + 1590 + 21 us before (FP64 sweeps on the cluster), now
-// 45 + 338 + 60 us.
+// 45 + 338 + 60 us.  Repeated eigenvalues pay for both solvers: a decomposition of 1024 x 768 from every row, k = 128, all
+// planted values equal, 2187 -> 2583 us.
 constexpr int ER_STEPS = 3;                               // refinement steps (two are enough unless eigenvalues are close)
 struct EigState {
   unsigned int emax[ER_STEPS];                            // largest |E_ij| of a step (bits)

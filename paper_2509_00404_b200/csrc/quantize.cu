@@ -6,7 +6,7 @@ namespace {
 // amax|x| of a strided matrix: one read of the tensor, bound by HBM.  A unit of work is UNROLL 16-byte vectors per
 // thread, all requested before the first is looked at; `tpr` threads (a power of two, at most 256) stand side by side on a row,
 // so that narrow rows do not idle the block, and one 32-bit division per unit finds the unit's place (a 64-bit division per
-// vector and scalar FP32 loads held the kernel at 3.3 TB/s for BF16 and 1.1 TB/s for FP32).  Units are walked
+// vector and scalar FP32 loads held the kernel at 3.6 TB/s for BF16 and 1.1 TB/s for FP32).  Units are walked
 // from the end of the tensor to its start: the quantizer that follows reads from the start, which is then what L2 holds.
 template <int DTYPE>
 __global__ void __launch_bounds__(256)
@@ -70,7 +70,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
   //     pass 2 reads 32 consecutive words of a row, a permutation of the chunks inside one 128-byte window.
   //   FP32 tile: rows of 512 bytes = 32 chunks of 16 bytes, chunk ch stored at ch ^ (ch >> 3): the eight lanes of a quarter warp store
   //     every fourth chunk of a row onto all banks; pass 2 reads 32 consecutive columns, a permutation inside one 128-byte window.
-  //     (Element stores into rows of 129 words met four to a bank; with them and unpipelined loads: 100 us at 14336 x 4096, 71 us now.)
+  //     (Element stores into rows of 129 words met four to a bank; with them and unpipelined loads: 100 us at 14336 x 4096, 73 us so.)
   //   staged row-block codes: 72-byte rows; a BF16 thread owns two adjacent columns, so column c is staged in row
   //     (c >> 1) + 64 (c & 1) and the 32 lanes of a store write 32 consecutive rows (18 words apart: 16 lanes cover
   //     the 32 banks with their 8 bytes each).

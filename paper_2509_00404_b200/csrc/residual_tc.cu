@@ -254,7 +254,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       }
       // FAST: a warp's codes - 32 rows of 16 bytes in either orientation - are staged in its patch and stored by tensor copies.  A
       // lane's store goes to a row of its own, so as ordinary stores they cost the load / store pipe a wavefront per lane
-      // and were 40 % of what bounds the round-to-nearest kernel (77 - 85 % of the pipe's wavefronts).
+      // (4096 x 4096, round to nearest, counted: 46 % of the pipe's wavefront slots over all SMs, 32 % with the copies; 29.5 -> 24.5 us).
       uint32_t pk0[2] = {0u, 0u}, pk1[2] = {0u, 0u}, pkr[2][2];
       if (p.c_codes != nullptr && step_ok) {
         // blocks along the columns: two blocks of this row, from registers

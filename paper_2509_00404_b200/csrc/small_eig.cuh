@@ -42,7 +42,7 @@ __device__ __forceinline__ void lower_tile(int o, int& ti, int& tj) {
 }
 
 // In-place Cholesky factorisation of the lower triangle of Y (n x n, n8 = n rounded up to a multiple of eight, row pitch P doubles,
-// rows and columns up to n8 must exist and be zero beyond n), called by all nthr threads of the CTA, 32 nthr / 32 >= n8 - 8.
+// rows and columns up to n8 must exist and be zero beyond n), called by all nthr >= n8 - 8 threads of the CTA.
 // Panels of eight columns: every warp factorises the panel's diagonal block in registers (lane = row; a column step is one
 // pivot broadcast, one reciprocal and one multiply-add deep, without a barrier) and carries 32 rows below it along; then all warps subtract
 // the panel's rank-8 product from the trailing tiles on the FP64 tensor cores, two tiles at a time.  (One barrier per
@@ -186,10 +186,11 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 // with the exit test cos^2 < 1e-8, which this replaces, left 1e-9 ... 1e-12); FP32 only decides how good the start is.
 // Input: Gram matrix (ld x ld, leading n x n block used).  Output: eigenvalues descending, eigenvectors as columns of
 // evecs[n][n].
-// Measured alone (full spectra, seven sweeps): n = 40 74 us - factorisation 6.5, Jacobi 55, refinement 7 - and n = 72 228 us; the
-// FP64 one-sided Jacobi before it took 113 - 126 us (n = 40), 52 us (n = 32), 250 us (n = 64) and 440 us (n = 72) inside a
-// layer step, against 56 - 64, 31, 122 and 239 us.  Half of the eigenvalues equal to the last digit, the worst case of step 4:
-// 190 us at n = 40.
+// Measured alone: n = 40 63 us for a sampled operand and 70 us for one decomposed from every row (seven sweeps), n = 32 32 us; about three
+// quarters of it is the Jacobi phase.  The FP64 one-sided Jacobi before it took 113 - 126 us (n = 40), 52 us (n = 32), 250 us
+// (n = 64) and 440 us (n = 72) inside a layer step, against 56 - 64, 31, 122 and 239 us.  Repeated eigenvalues, the worst case of
+// step 4, are the one spectrum that got slower: 190 us at n = 40, half of them equal to the last digit; a decomposition of 1024 x 768,
+// k = 32, all planted values equal, 333 -> 407 us.  (FP64 sweeps at once instead of the second attempt: 392 -> 494 us sampled.)
 constexpr int EIG_THREADS = 512;
 constexpr int EIG_MAX_SWEEPS = 16, EIG_MAX_REFINE = 6, EIG_ORTH_FROM = 4;   // the last two refinement steps only orthonormalise
 constexpr float EIG_EXIT_COS2 = 1e-4f;                  // last FP32 sweep: its rotations and two refinement steps square this three times

@@ -2,8 +2,8 @@
 //
 // Steps (FULL = on all rows, SAMPLED = subspace from a sparse row sample, "broadcast" to all rows):
 //   amax(x) -> row sample -> sketch Z = x[S,:] Omega (Omega from Philox + quantile table, never stored)
-//   -> CholeskyQR2 (FP64 Gram + Cholesky) -> M = H^T x[S,:] -> eigen-decomposition of M M^T (Jacobi,
-//   FP64) -> right basis B -> [SAMPLED: C = x B, Rayleigh-Ritz on C^T C] -> residual R = x - C B^T fused
+//   -> CholeskyQR2 (FP64 Gram + Cholesky) -> M = H^T x[S,:] -> eigen-decomposition of M M^T (Jacobi
+//   sweeps in FP32, refined in FP64) -> right basis B -> [SAMPLED: C = x B, Rayleigh-Ritz on C^T C] -> residual R = x - C B^T fused
 //   with the NVFP4 quantizer in both block orientations -> factor rotation, sign fix, factor quantization.
 #include "quant_tile.cuh"
 #include "bigrank.cuh"
