@@ -189,8 +189,8 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 // Measured alone: n = 40 63 us for a sampled operand and 70 us for one decomposed from every row (seven sweeps), n = 32 32 us; about three
 // quarters of it is the Jacobi phase.  The FP64 one-sided Jacobi before it took 113 - 126 us (n = 40), 52 us (n = 32), 250 us
 // (n = 64) and 440 us (n = 72) inside a layer step, against 56 - 64, 31, 122 and 239 us.  Repeated eigenvalues, the worst case of
-// step 4, are the one spectrum that got slower: 190 us at n = 40, half of them equal to the last digit; a decomposition of 1024 x 768,
-// k = 32, all planted values equal, 333 -> 407 us.  (FP64 sweeps at once instead of the second attempt: 392 -> 494 us sampled.)
+// step 4, are what got slower: 190 us at n = 40, half of them equal to the last digit; a decomposition of 1024 x 768 from every
+// row, k = 32, all planted values equal, 333 -> 407 us.  (FP64 sweeps at once instead of the second attempt: 392 -> 494 us sampled.)
 constexpr int EIG_THREADS = 512;
 constexpr int EIG_MAX_SWEEPS = 16, EIG_MAX_REFINE = 6, EIG_ORTH_FROM = 4;   // the last two refinement steps only orthonormalise
 constexpr float EIG_EXIT_COS2 = 1e-4f;                  // last FP32 sweep: its rotations and two refinement steps square this three times
