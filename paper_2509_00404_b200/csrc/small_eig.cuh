@@ -2,6 +2,7 @@
 // eigen-decomposition.  Both are latency chains on one SM, so what counts is the number of dependent steps and how long one is.
 #pragma once
 #include "common.cuh"
+#include "tridiag.cuh"
 
 namespace metis_small {
 
@@ -48,10 +49,10 @@ __device__ __forceinline__ void lower_tile(int o, int& ti, int& tj) {
 // the panel's rank-8 product from the trailing tiles on the FP64 tensor cores, two tiles at a time.  (One barrier per
 // column with the matrix spread over 256 threads' registers took 800 cycles a column.)  A pivot not above `tol` marks a dependent column:
 // it takes no part in the updates and ends as a zero column with inv_out[j] = 0; otherwise inv_out[j] = 1 / L[j][j].
-// *dmin_out (optional): the smallest accepted pivot.
-template <int P>
-__device__ __forceinline__ void cta_cholesky(double* Y, int n, double tol, double* inv_out, double* dmin_out, int nthr) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_warps = nthr >> 5;
+// *dmin_out (optional): the smallest accepted pivot.  tid, bar: index within the group of nthr threads and the group's barrier.
+template <int P, class Bar>
+__device__ __forceinline__ void group_cholesky(double* Y, int n, double tol, double* inv_out, double* dmin_out, int tid, int nthr, Bar bar) {
+  const int lane = tid & 31, warp = tid >> 5, n_warps = nthr >> 5;
   const int n8 = (n + 7) & ~7, g = lane >> 2, q = lane & 3;
   double dmin = 1e300;
   for (int c0 = 0; c0 < n8; c0 += 8) {
@@ -86,7 +87,7 @@ __device__ __forceinline__ void cta_cholesky(double* Y, int n, double tol, doubl
         if (r < n8) Y[r * P + c0 + c] = v[c] * ic;
       }
     }
-    __syncthreads();                                    // the block has been read by every warp: its factor may be stored
+    bar();                                    // the block has been read by every warp: its factor may be stored
     if (warp == 0 && lane < 8) {
       if (c0 + lane < n) inv_out[c0 + lane] = inv;
 #pragma unroll
@@ -116,14 +117,19 @@ __device__ __forceinline__ void cta_cholesky(double* Y, int n, double tol, doubl
       for (int u = 0; u < 2; ++u)
         if (u == 0 || two) { out[u][0] = acc[u][0]; out[u][1] = acc[u][1]; }
     }
-    __syncthreads();
+    bar();
   }
   if (dmin_out != nullptr && warp == 0) {
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_xor_sync(0xFFFFFFFFu, dmin, o));
     if (lane == 0) *dmin_out = dmin;
   }
-  __syncthreads();
+  bar();
+}
+
+template <int P>
+__device__ __forceinline__ void cta_cholesky(double* Y, int n, double tol, double* inv_out, double* dmin_out, int nthr) {
+  group_cholesky<P>(Y, n, tol, inv_out, dmin_out, (int)threadIdx.x, nthr, [] { __syncthreads(); });
 }
 
 // X = L^-1 (nothing is written above the diagonal blocks) for the factor of cta_cholesky, by all nthr threads: the 8 x 8 diagonal
@@ -169,31 +175,36 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 
 // ------------------------------------------------------------------------------------------------
 // Symmetric positive semi-definite eigen-decomposition in one CTA.
-//   1. the matrix, sorted by descending diagonal, is factorised G = L L^T (FP64; dependent columns zeroed);
-//   2. one-sided Jacobi on the columns of L in FP32: Y = L J with orthogonal columns, so the normalised columns approximate the
-//      eigenvectors.  Eight lanes own two blocks of two columns: one round loads four columns, forms their six inner
-//      products at once, works out the four rotations between the blocks on the 4 x 4 Gram matrix in registers and
-//      applies them - one barrier and one reduction for what takes two of each when single couples are rotated.  A round
-//      is bound by latency and by its warps' own instruction streams (n = 40: 784 cycles; sixteen lanes a group: 990);
+//   1. Householder reduction to a tridiagonal matrix T in FP64 (tridiag.cuh), the matrix in the registers of four threads per row.
+//      A step is a chain of two reductions over eight lanes, a reciprocal square root, a reciprocal and three barriers, 750 - 870
+//      cycles at n = 40; what counts is the number of instructions a warp has to issue in it, so one more warp works out the
+//      scalars and the two vectors of the update, which every thread doing that for itself made 1250 - 1400 cycles.
+//      Meanwhile six warps sort the matrix by descending diagonal and factorise it, G = L L^T (dependent columns zeroed);
+//   2. eigenvalues of T by multisection on Sturm counts to a relative 2^-30 of themselves, eigenvectors by twisted factorisations
+//      (Dhillon and Parlett, "Orthogonal eigenvectors and relative gaps", 2003, without their representation tree), taken back through
+//      the reflectors in panels of eight (compact WY) on the FP64 tensor cores;
 //   3. FP64 refinement of the eigenvectors U (Ogita and Aishima, "Iterative refinement for symmetric eigenvalue
 //      decomposition", 2018): with R = I - U^T U and S = U^T G U, U += U E, E_ij = (S_ij + s_j R_ij) / (s_j - s_i), E_ii = R_ii / 2,
 //      s_i = S_ii / (1 - R_ii); the error is squared by each step.  S is formed as W^T W with W = L^T U, which keeps the
-//      relative accuracy of small eigenvalues.  The products run on the FP64 tensor cores;
-//   4. eigenvalues too close to be separated this way (|E_ij| above 1/16, or E as a whole not small) send the matrix back to
-//      step 2 with a tight exit test; if pairs are still open after that, they are only orthonormalised in step 3 and FP64
+//      relative accuracy of small eigenvalues, of which T keeps only the absolute one.  The products run on the FP64 tensor cores.
+//      One step is enough unless eigenvalues lie closer than a hundredth of a per cent or so;
+//   4. eigenvalues that agree to about 1e-9 come out of step 2 with dependent vectors (|E_ij| above 1/16, or E as a whole not
+//      small): then one-sided Jacobi on the columns of L in FP32 makes the start instead (Y = L J with orthogonal columns; eight lanes
+//      own two blocks of two columns: one round loads four columns, forms their six inner products at once, works out the
+//      four rotations between the blocks on the 4 x 4 Gram matrix in registers and applies them, 784 cycles at n = 40) and
+//      step 3 is repeated; if pairs are still open after that, they are only orthonormalised in step 3 and FP64
 //      one-sided Jacobi sweeps on the columns of W = L^T U, U rotated along, finish the work (repeated eigenvalues).
-// Precision: the columns of U leave the loop orthonormal, and the pairs of W orthogonal, to about 1e-12 (FP64 rotations
-// with the exit test cos^2 < 1e-8, which this replaces, left 1e-9 ... 1e-12); FP32 only decides how good the start is.
+// Precision: the columns of U leave the loop orthonormal, and the pairs of W orthogonal, to 1e-10 or better.
 // Input: Gram matrix (ld x ld, leading n x n block used).  Output: eigenvalues descending, eigenvectors as columns of
 // evecs[n][n].
-// Measured alone: n = 40 63 us for a sampled operand and 70 us for one decomposed from every row (seven sweeps), n = 32 32 us; about three
-// quarters of it is the Jacobi phase.  The FP64 one-sided Jacobi before it took 113 - 126 us (n = 40), 52 us (n = 32), 250 us
-// (n = 64) and 440 us (n = 72) inside a layer step, against 56 - 64, 31, 122 and 239 us.  Repeated eigenvalues, the worst case of
-// step 4, are what got slower: 190 us at n = 40, half of them equal to the last digit; a decomposition of 1024 x 768 from every
-// row, k = 32, all planted values equal, 333 -> 407 us.  (FP64 sweeps at once instead of the second attempt: 392 -> 494 us sampled.)
-constexpr int EIG_THREADS = 512;
+// Measured alone, planted spectrum (before: the Jacobi sweeps of step 4 as the start of every matrix): n = 8 10.4 us (12.5), n = 32 33 (42),
+// n = 40 43 (66), n = 64 88 (128), n = 72 115 (228); eigenvalues within 4e-5 of each other n = 40 47 (158), n = 72 128 (719); nearly diagonal
+// matrices are the ones the sweeps finished sooner: n = 32 33 (25), n = 40 43 (35).  Repeated eigenvalues pay for both starts:
+// half of them equal to the last digit n = 40 176 (152), n = 72 919 (861).  The reduction takes 18 of the 43 us at n = 40, the multisection 6.
+// Four threads per row reduce the matrix while six warps factorise it; the products and the multisection use all of them.
+constexpr int EIG_CHOL_THREADS = 192;
+__host__ __device__ constexpr int eig_threads(int nt8) { return nt8 <= 1 ? 256 : 512; }
 constexpr int EIG_MAX_SWEEPS = 16, EIG_MAX_REFINE = 6, EIG_ORTH_FROM = 4;   // the last two refinement steps only orthonormalise
-constexpr float EIG_EXIT_COS2 = 1e-4f;                  // last FP32 sweep: its rotations and two refinement steps square this three times
 constexpr float EIG_TIGHT_COS2 = 1e-11f;                // as orthogonal as FP32 columns get
 __host__ __device__ constexpr size_t eig_smem(int n) {  // L, U, W, E in FP64, Y in FP32
   const int n8 = (n + 7) & ~7;
@@ -288,10 +299,11 @@ __device__ __forceinline__ void block_rotate(float2 (&a)[R], float2 (&b)[R], flo
 }
 
 template <int NT8>                                      // n rounded up to a multiple of eight, over eight
-__global__ void __launch_bounds__(EIG_THREADS, 1)
+__global__ void __launch_bounds__(eig_threads(NT8), 1)
 eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ evals, double* __restrict__ evecs) {
   metis_pdl_wait();
-  constexpr int N8 = 8 * NT8, P = N8 + 4;
+  constexpr int N8 = 8 * NT8, P = N8 + 4, EIG_THREADS = eig_threads(NT8);
+  constexpr int TD = 4 * N8, TS = TD + 32;              // threads of the reduction: four per row, and the warp that works out its scalars
   constexpr int R = NT8, RP = N8;                       // rows per lane, rows of a column in Y
   constexpr int NB = N8 / 2;                            // column blocks of two (an even number)
   constexpr int GROUPS = NB / 2, JT = (8 * GROUPS + 31) / 32 * 32;             // groups of eight lanes, threads of the Jacobi phase
@@ -305,62 +317,375 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   __shared__ __align__(8) float nrm[N8];
   __shared__ int perm[N8], order[N8];
   __shared__ double gmax_s;
-  __shared__ int flags[2][EIG_MAX_SWEEPS], flags64[EIG_MAX_SWEEPS];
+  __shared__ int flags[EIG_MAX_SWEEPS], flags64[EIG_MAX_SWEEPS];
+  __shared__ __align__(16) double2 te[N8 + 1];          // diagonal and squared subdiagonal of the tridiagonal matrix
+  __shared__ __align__(16) double ys[N8], rs[2][N8], us[N8];
+  __shared__ __align__(16) double2 pq[N8];
+  __shared__ double eo[N8 + 1], beta_s[N8], v1_s[N8];
+  __shared__ int pos[N8];
+  __shared__ unsigned char grid_count[EIG_THREADS];
+  __shared__ __align__(16) double Tp[64 * NT8], Pt[64 * NT8];
   __shared__ unsigned int emax_s[2][EIG_MAX_REFINE];
   __shared__ float en_w[EIG_THREADS / 32];
   __shared__ uint8_t pairs[NB][GROUPS][2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
 
-  // ---- sort by the diagonal, factorise ----
+  // ---- the matrix; tables ----
   for (int o = tid; o < N8 * N8; o += EIG_THREADS) {
     const int i = o / N8, j = o % N8;
     E[i * P + j] = (i < n && j < n) ? gm[i * ld + j] : (i == j ? -1.0 : 0.0);
   }
   if (tid < N8) perm[tid] = tid;
-  if (tid < EIG_MAX_SWEEPS) flags[0][tid] = flags[1][tid] = flags64[tid] = 0;
-  if (tid < EIG_MAX_REFINE) emax_s[0][tid] = emax_s[1][tid] = 0u;
   for (int o = tid; o < (NB - 1) * GROUPS; o += EIG_THREADS) {                  // round-robin tournament of the blocks
     const int step = o / GROUPS, m = o % GROUPS;
     const int a = m == 0 ? 0 : (step + m) % (NB - 1) + 1, b = m == 0 ? step % (NB - 1) + 1 : (step + NB - 1 - m) % (NB - 1) + 1;
     pairs[step][m][0] = (uint8_t)min(a, b); pairs[step][m][1] = (uint8_t)max(a, b);
   }
+  if (tid < EIG_MAX_SWEEPS) flags[tid] = flags64[tid] = 0;
+  if (tid < EIG_MAX_REFINE) emax_s[0][tid] = emax_s[1][tid] = 0u;
   __syncthreads();
-  if (tid < 4 * N8) {                                   // rank of the diagonal entries, four lanes per entry
-    const int e = tid >> 2;
-    const double d = E[e * P + e];
-    int rank = 0;
-    for (int j = tid & 3; j < N8; j += 4) { const double x = E[j * P + j]; rank += (x > d) || (x == d && j < e); }
-    rank += __shfl_xor_sync(0xFFFFFFFFu, rank, 1);
-    rank += __shfl_xor_sync(0xFFFFFFFFu, rank, 2);
-    if ((tid & 3) == 0) {
+  // an even power of two brings the largest entry near one; its root does for the FP32 copy of the factor
+  int top = 0;
+  for (int i = lane; i < n; i += 32) top = max(top, __double2hiint(E[i * P + i]));
+  top = __reduce_max_sync(0xFFFFFFFFu, top) >> 20;
+  const int ex = top > 0 && top < 2046 ? (top - 1022 + 1) >> 1 : 0;
+  const double y_scale = __hiloint2double((1023 - ex) << 20, 0);
+  double* V = W;                                        // row j: column j of the trailing matrix when it is reduced (reflector j)
+  const int s8 = tid & 7;
+  auto bar_r = [] { asm volatile("bar.sync 2, %0;" ::"n"(TS) : "memory"); };
+  if (tid < TD) {
+    auto bar = bar_r;
+    // ---- Householder reduction: eight lanes hold rows i0 and i0 + 1 in registers (columns s8, s8 + 8, ...) ----
+    const int i0 = 2 * (tid >> 3), last_row = (tid | 31) >> 2 | 1;
+    double row[2][NT8];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+      for (int t = 0; t < NT8; ++t) {
+        const int c = s8 + 8 * t, i = i0 + h;
+        row[h][t] = i < n && c < n ? 0.5 * (E[i * P + c] + E[c * P + i]) * (y_scale * y_scale) : 0.0;
+      }
+    // row j (if this thread holds part of it) becomes the next column to be reduced, row j + 1 goes beside it
+    auto publish = [&](int j) {
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if ((j + u) >> 1 == i0 >> 1) {
+          double* out = u == 0 ? V + j * P : rs[j & 1];
+          const bool odd = (j + u) & 1;
+#pragma unroll
+          for (int t = 0; t < NT8; ++t) out[s8 + 8 * t] = s8 + 8 * t > j ? (odd ? row[1][t] : row[0][t]) : 0.0;
+        }
+    };
+    publish(0);
+    if (tid == 0) te[0].x = row[0][0];
+    bar();
+#pragma unroll 1
+    for (int j = 0; j + 2 < n; ++j) {
+      const bool live = last_row > j;                   // the warp has a row below j
+      double x[NT8];
+      if (live) {
+        double y0 = 0.0, y1 = 0.0;
+#pragma unroll
+        for (int t = 0; t < NT8; ++t) {
+          x[t] = V[j * P + s8 + 8 * t];
+          y0 = fma(row[0][t], x[t], y0); y1 = fma(row[1][t], x[t], y1);
+        }
+        const bool hi = s8 & 4;                         // lanes 0 - 3 end with the sum of row i0, lanes 4 - 7 with that of i0 + 1
+        double y = (hi ? y1 : y0) + __shfl_xor_sync(0xFFFFFFFFu, hi ? y0 : y1, 4);
+        y += __shfl_xor_sync(0xFFFFFFFFu, y, 2);
+        y += __shfl_xor_sync(0xFFFFFFFFu, y, 1);
+        if ((s8 & 3) == 0) ys[i0 + (s8 >> 2)] = y;
+      }
+      bar();
+      bar();
+      if (live) {
+        const double2 c0 = pq[i0], c1 = pq[i0 + 1];
+#pragma unroll
+        for (int t = 0; t < NT8; ++t) {
+          const double u = us[s8 + 8 * t];
+          row[0][t] = fma(c0.x, u, fma(c0.y, x[t], row[0][t]));
+          row[1][t] = fma(c1.x, u, fma(c1.y, x[t], row[1][t]));
+        }
+        publish(j + 1);
+      }
+      bar();
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)                         // what is left of the last two rows
+#pragma unroll
+      for (int t = 0; t < NT8; ++t)
+        if (s8 + 8 * t == n - 1) {
+          if (i0 + h == n - 2) eo[n - 2] = row[h][t];
+          if (i0 + h == n - 1) te[n - 1].x = row[h][t];
+        }
+  } else if (tid < TS) {
+    auto bar = bar_r;
+    // ---- the warp of the scalars (its four groups of eight lanes do the same): with y = A x and r = A e_1 it is
+    // A v = u = y - alpha r,  v^T A v = x^T y - 2 alpha y_1 + alpha^2 r_1;  w = beta u - K v,  A -= v w^T + w v^T = p u^T + q v^T.
+    // Column j + 1 of the product is not read again except for its first entry, so x stands for v in the last term ----
+    bar();
+#pragma unroll 1
+    for (int j = 0; j + 2 < n; ++j) {
+      const double* r = rs[j & 1];
+      double x[NT8], rc[NT8], sq[2] = {0.0, 0.0}, xy[2] = {0.0, 0.0}, alpha, beta;
+#pragma unroll
+      for (int t = 0; t < NT8; ++t) { x[t] = V[j * P + s8 + 8 * t]; rc[t] = r[s8 + 8 * t]; }
+      const double x0 = V[j * P + j + 1], ra = r[j + 1];
+#pragma unroll
+      for (int t = 0; t < NT8; ++t) sq[t & 1] = fma(x[t], x[t], sq[t & 1]);
+      sq[0] += sq[1];
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) sq[0] += __shfl_xor_sync(0xFFFFFFFFu, sq[0], o);
+      metis_tri::reflector(x0, sq[0], alpha, beta);
+      const double b2 = beta * beta, v1 = x0 - alpha, a2 = alpha * alpha * ra;
+      bar();                                            // the product is there
+      double y[NT8];
+#pragma unroll
+      for (int t = 0; t < NT8; ++t) { y[t] = ys[s8 + 8 * t]; xy[t & 1] = fma(x[t], y[t], xy[t & 1]); }
+      const double ya = ys[j + 1], k0 = fma(-2.0 * alpha, ya, a2);
+      xy[0] += xy[1];
+#pragma unroll
+      for (int t = 0; t < NT8; ++t) {
+        y[t] = fma(-alpha, rc[t], y[t]);
+        us[s8 + 8 * t] = y[t];
+      }
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) xy[0] += __shfl_xor_sync(0xFFFFFFFFu, xy[0], o);
+      const double K2 = b2 * (xy[0] + k0);
+#pragma unroll
+      for (int t = 0; t < NT8; ++t) {
+        const double v = s8 + 8 * t == j + 1 ? v1 : x[t];
+        pq[s8 + 8 * t] = make_double2(-beta * v, fma(-beta, y[t], K2 * v));
+      }
+      bar();                                            // the update may go on
+      if (lane == 0) {
+        eo[j] = alpha; beta_s[j] = beta; v1_s[j] = v1;
+        te[j + 1].x = fma(-v1, fma(2.0 * beta, fma(-alpha, ra, ya), -K2 * v1), ra);
+      }
+      bar();                                            // the next column is there
+    }
+  } else if (tid < TS + EIG_CHOL_THREADS) {
+    // ---- meanwhile: sorted by the diagonal and factorised ----
+    auto bar = [] { asm volatile("bar.sync 3, %0;" ::"n"(EIG_CHOL_THREADS) : "memory"); };
+    const int ct = tid - TS;
+    for (int e = ct; e < N8; e += EIG_CHOL_THREADS) {
+      const double d = E[e * P + e];
+      int rank = 0;
+#pragma unroll 8
+      for (int j = 0; j < N8; ++j) { const double x = E[j * P + j]; rank += (x > d) || (x == d && j < e); }
+      pos[e] = rank;
       if (e < n) perm[rank] = e;                        // NaNs may collide; every entry stays a valid index
       if (rank == 0) gmax_s = d;
     }
-  }
-  __syncthreads();
-  for (int o = tid; o < N8 * N8; o += EIG_THREADS) {
-    const int i = o / N8, j = o % N8;
-    Lm[i * P + j] = (i < n && j < n) ? 0.5 * (E[perm[i] * P + perm[j]] + E[perm[j] * P + perm[i]]) : 0.0;
-  }
-  const double gmax = gmax_s;
-  __syncthreads();
-  cta_cholesky<P>(Lm, n, 1e-14 * gmax, inv_s, nullptr, EIG_THREADS);
-  // FP32 copy, scaled to a largest entry near one
-  int ex = 0;
-  if (gmax > 0.0 && gmax < 1e300) { (void)frexp(gmax, &ex); ex = (ex + 1) / 2; }
-  const double y_scale = ldexp(1.0, -ex);
-  for (int o = tid; o < NB * RP; o += EIG_THREADS) {
-    const int b = o / RP, r = o % RP;
-    float2 y = make_float2(0.0f, 0.0f);
-    if (r < n) {
-      if (r >= 2 * b) y.x = (float)(Lm[r * P + 2 * b] * y_scale);
-      if (r >= 2 * b + 1) y.y = (float)(Lm[r * P + 2 * b + 1] * y_scale);
+    bar();
+    for (int o = ct; o < N8 * N8; o += EIG_CHOL_THREADS) {
+      const int i = o / N8, j = o % N8;
+      Lm[i * P + j] = (i < n && j < n) ? 0.5 * (E[perm[i] * P + perm[j]] + E[perm[j] * P + perm[i]]) : 0.0;
     }
-    Yb[o] = y;
+    bar();
+    group_cholesky<P>(Lm, n, 1e-14 * gmax_s, inv_s, nullptr, ct, EIG_CHOL_THREADS, bar);
   }
+  __syncthreads();
+  const double gmax = gmax_s;
+  if (tid <= N8) {
+    te[tid].y = tid > 0 && tid < n ? fmax(eo[tid - 1] * eo[tid - 1], 1e-60) : 0.0;
+    if (tid >= n) te[tid].x = 4.0 * N8;
+  }
+  if (tid + 2 < n) V[tid * P + tid + 1] = v1_s[tid];
   for (int o = tid; o < N8 * N8; o += EIG_THREADS) {   // the factor's upper triangle (the factorisation leaves the input there)
     const int i = o / N8, j = o % N8;
     if (j > i) Lm[i * P + j] = 0.0;
+  }
+  const int rank = __syncthreads_count(tid < n && inv_s[tid < n ? tid : 0] > 0.0);
+  // ---- eigenvalues and eigenvectors of the tridiagonal matrix, descending ----
+  const long long grid_lo = __double_as_longlong(0x1p-56), grid_w = (__double_as_longlong(2.0 * N8) - grid_lo) / EIG_THREADS + 1;
+  {
+    const double x[1] = {__longlong_as_double(grid_lo + grid_w * (tid + 1))};  // brings every eigenvalue to about a tenth of an octave
+    int c[1];
+    metis_tri::sturm_counts<1>(te, NT8, x, c);
+    grid_count[tid] = (unsigned char)c[0];
+  }
+  __syncthreads();
+  double *Dp = E, *Z = U;                               // column e of each: vector e
+  constexpr int TV = 4 * N8;                            // four threads per vector
+  // Lanes per eigenvalue in the multisection, so that a warp (or two) runs on each of the four schedulers: a round costs 25 cycles per
+  // row and warp there.
+  constexpr int LE = N8 <= 32 ? 4 : (N8 <= 40 || N8 > 64 ? 3 : 2), PW = 32 / LE, TE = (N8 + PW - 1) / PW * 32;
+  {
+    if (tid < TE) {
+      const int e = PW * warp + min(lane / LE, PW - 1), below = max(n - 1 - e, 0);
+      int at = 0;                                       // the first point with more than `below` eigenvalues under it
+#pragma unroll
+      for (int step = EIG_THREADS / 2; step > 0; step >>= 1) if (grid_count[at + step - 1] <= below) at += step;
+      const double v = metis_tri::multisect<LE>(te, NT8, grid_lo + grid_w * at, grid_lo + grid_w * (at + 1), below,
+                                                LE == 4 ? 9 : (LE == 3 ? 10 : 12));
+      if (lane % LE == 0 && lane / LE < PW && e < N8) lam[e] = v;
+    }
+  }
+  __syncthreads();
+  if (tid < TV) {
+    auto bar = [] { asm volatile("bar.sync 2, %0;" ::"n"(TV) : "memory"); };
+    if (tid < 2 * n) {                                  // pivots from the top and from the bottom
+      const int e = tid >> 1, down = tid & 1;
+      const double lm = lam[e];
+      double* D = (down ? Z : Dp) + e;
+      double pm = 0.0, p = 1.0;
+#pragma unroll 1
+      for (int b = 0; b < NT8; ++b) {
+        double d[8], e2[8];                             // (rows beyond the matrix read padding, forwards, or row 0, backwards; nothing is kept)
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = 8 * b + u;
+          d[u] = te[down ? max(n - 1 - i, 0) : i].x - lm;
+          e2[u] = te[down ? max(n - i, 0) : i].y;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const double pn = fma(d[u], p, -e2[u] * pm);
+          d[u] = pn * metis_tri::rcp_mid(p + 1e-290);
+          pm = p; p = pn;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int i = 8 * b + u;
+          if (i < n) D[(down ? n - 1 - i : i) * P] = d[u];
+        }
+        const int big = max(__double2hiint(p) & 0x7FF00000, __double2hiint(pm) & 0x7FF00000);
+        const double sc = __hiloint2double(0x7FE00000 - big, 0);
+        p *= sc; pm *= sc;
+      }
+    }
+    bar();
+    {
+      // twist where |gamma| is least: z = 1 there, the other entries are products of e / pivot outwards from it
+      const int e = tid >> 2, s = tid & 3;
+      const double lm = lam[e];
+      double best = 1e300, du[2 * NT8], dd[2 * NT8];
+      int at = 0;
+#pragma unroll
+      for (int t = 0; t < 2 * NT8; ++t) { du[t] = Dp[(s + 4 * t) * P + e]; dd[t] = Z[(s + 4 * t) * P + e]; }
+#pragma unroll
+      for (int t = 0; t < 2 * NT8; ++t) {
+        const int i = s + 4 * t;
+        const double gamma = fabs(du[t] + dd[t] - (te[i].x - lm));
+        if (i < n && gamma < best) { best = gamma; at = i; }
+      }
+#pragma unroll
+      for (int o = 2; o > 0; o >>= 1) {
+        const double other = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+        const int oi = __shfl_xor_sync(0xFFFFFFFFu, at, o);
+        if (other < best || (other == best && oi < at)) { best = other; at = oi; }
+      }
+      if (s == 0) order[e] = at;
+#pragma unroll
+      for (int t = 0; t < 2 * NT8; ++t) {
+        const int i = s + 4 * t;
+        const double f = eo[i < at ? i : max(i - 1, 0)] * metis_tri::rcp_mid((i < at ? du[t] : dd[t]) + 1e-60);
+        Z[i * P + e] = i < n ? (i == at ? 1.0 : -f) : 0.0;
+      }
+    }
+    bar();
+    {                                                   // two threads per vector, by whole warps
+      const int e = tid >> 1, step = tid & 1 ? 1 : -1;
+      double f = 1.0, zz = tid & 1 ? 0.0 : 1.0;
+      int i = e < n ? order[e] + step : -1;
+      while (i >= 0 && i < n) {                         // four at a time, the loads ahead of the products
+        double m[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) { const int at = i + u * step; m[u] = at >= 0 && at < n ? Z[at * P + e] : 0.0; }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int at = i + u * step;
+          f *= m[u];
+          zz = fma(f, f, zz);
+          if (at >= 0 && at < n) Z[at * P + e] = f;
+        }
+        i += 4 * step;
+      }
+      zz += __shfl_xor_sync(0xFFFFFFFFu, zz, 1);
+      if (step > 0 && e < N8) ys[e] = e < rank ? metis_tri::rsqrt_mid(zz) : 0.0;         // a dependent column of the factor: no vector
+    }
+  } else {
+    // ---- meanwhile: the reflectors in panels of eight, H_8b ... H_8b+7 = I - V_b^T T_b V_b (T_b: inverse of diag(1 / beta) + the
+    // upper triangle of V_b V_b^T), a warp per panel ----
+    for (int b = warp - TV / 32; b < NT8; b += (EIG_THREADS - TV) / 32) {
+      double acc[2][2] = {};
+#pragma unroll
+      for (int kk = 0; kk < N8; kk += 4) {
+        const bool on = 8 * b + g + 2 < n;
+        const double a = on ? V[(8 * b + g) * P + kk + q] : 0.0;
+        dmma(acc[(kk >> 2) & 1], a, a);                 // the fragments of V_b and of its transpose hold the same entries
+      }
+      double* t = Tp + 64 * b;
+      t[8 * g + 2 * q] = acc[0][0] + acc[1][0]; t[8 * g + 2 * q + 1] = acc[0][1] + acc[1][1];
+      __syncwarp();
+      double xcol[8];                                   // column `lane` of the lower triangular inverse: T_b transposed
+      if (lane < 8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          double sum = 0.0;
+#pragma unroll
+          for (int k = 0; k < i; ++k) sum = fma(t[8 * i + k], xcol[k], sum);
+          const double bt = 8 * b + i + 2 < n ? beta_s[8 * b + i] : 0.0;
+          xcol[i] = i == lane ? bt : (i > lane ? -bt * sum : 0.0);
+        }
+      }
+      __syncwarp();
+      if (lane < 8)
+#pragma unroll
+        for (int i = 0; i < 8; ++i) t[8 * lane + i] = xcol[i];                 // T_b[lane][i]
+    }
+  }
+  __syncthreads();
+  // ---- back through the panels: a warp per eight vectors, without a barrier ----
+  for (int tj = warp; tj < NT8; tj += EIG_THREADS / 32) {
+    double* Zc = Z + 8 * tj;
+    double* patch = Pt + 64 * tj;
+    if (8 * tj + 8 > n)                                 // vectors beyond the matrix
+      for (int i = lane; i < 8 * N8; i += 32) if (8 * tj + (i & 7) >= n) Zc[(i >> 3) * P + (i & 7)] = 0.0;
+    __syncwarp();
+#pragma unroll 1
+    for (int b = (n - 3) >> 3; b >= 0; --b) {
+      const bool on_g = 8 * b + g + 2 < n;
+      double acc[2][2] = {};
+#pragma unroll
+      for (int kk = 0; kk < N8; kk += 4)
+        dmma(acc[(kk >> 2) & 1], on_g ? V[(8 * b + g) * P + kk + q] : 0.0, Zc[(kk + q) * P + g]);
+      *reinterpret_cast<double2*>(patch + 8 * g + 2 * q) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+      __syncwarp();
+      double y[2] = {0.0, 0.0};
+#pragma unroll
+      for (int kk = 0; kk < 8; kk += 4) dmma(y, Tp[64 * b + 8 * g + kk + q], patch[8 * (kk + q) + g]);
+      __syncwarp();
+      *reinterpret_cast<double2*>(patch + 8 * g + 2 * q) = make_double2(-y[0], -y[1]);
+      __syncwarp();
+      const double y0 = patch[8 * q + g], y1 = patch[8 * (q + 4) + g];
+      const bool on0 = 8 * b + q + 2 < n, on1 = 8 * b + 4 + q + 2 < n;
+      double d[NT8][2], a0[NT8], a1[NT8];
+#pragma unroll
+      for (int ti = 0; ti < NT8; ++ti) {
+        const double2 z = *reinterpret_cast<const double2*>(Zc + (8 * ti + g) * P + 2 * q);
+        d[ti][0] = z.x; d[ti][1] = z.y;
+        a0[ti] = on0 ? V[(8 * b + q) * P + 8 * ti + g] : 0.0;
+        a1[ti] = on1 ? V[(8 * b + 4 + q) * P + 8 * ti + g] : 0.0;
+      }
+#pragma unroll
+      for (int ti = 0; ti < NT8; ++ti) dmma(d[ti], a0[ti], y0);
+#pragma unroll
+      for (int ti = 0; ti < NT8; ++ti) {
+        dmma(d[ti], a1[ti], y1);
+        *reinterpret_cast<double2*>(Zc + (8 * ti + g) * P + 2 * q) = make_double2(d[ti][0], d[ti][1]);
+      }
+      __syncwarp();
+    }
+    // normalised, in the order of the factor's rows
+    double z[2 * NT8];
+    const double rz = ys[8 * tj + (lane & 7)];
+#pragma unroll
+    for (int t = 0; t < 2 * NT8; ++t) z[t] = Zc[((lane >> 3) + 4 * t) * P + (lane & 7)];
+    __syncwarp();
+#pragma unroll
+    for (int t = 0; t < 2 * NT8; ++t) Zc[pos[(lane >> 3) + 4 * t] * P + (lane & 7)] = z[t] * rz;
   }
   __syncthreads();
 
@@ -377,81 +702,88 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   int still_open = 0;                                   // pairs left to the FP64 sweeps
   bool orth_only = false;
   for (int attempt = 0; attempt < 2; ++attempt) {
-    const float exit_cos2 = attempt == 0 ? EIG_EXIT_COS2 : EIG_TIGHT_COS2;
     bool again = false;
     X = U; Wb = W;
-    // ---- one-sided block Jacobi in FP32 on JT threads ----
-    if (tid < JT) {
-      auto bar = [] { asm volatile("bar.sync 1, %0;" ::"n"(JT) : "memory"); };
-      const int m = tid >> 3, sub = tid & 7;
-      const bool active = m < GROUPS;
-      const int mc = min(m, GROUPS - 1);                // groups beyond the last one repeat its work and store nothing
-      float2* nrm2 = reinterpret_cast<float2*>(nrm);
-      // A group's access is 64 of a 128-byte line.  With an even number of chunks of eight rows, odd groups walk them in the
-      // order 1, 0, 3, 2, ..., so that the two groups of a half warp never meet in the same banks (n = 64: a sixth off a
-      // round); an odd number would need a padding chunk, which costs more than the conflicts.
-      const int odd = R % 2 == 0 ? m & 1 : 0;
-      auto row_of = [&](int t) { return sub + 8 * (t ^ odd); };
-      for (int sweep = 0; sweep < EIG_MAX_SWEEPS; ++sweep) {
-        // squared column norms: a group takes blocks 2m and 2m + 1
+    if (attempt == 1) {                                 // the start by way of T had dependent vectors
+      constexpr float exit_cos2 = EIG_TIGHT_COS2;
+      for (int o = tid; o < NB * RP; o += EIG_THREADS) {
+        const int b = o / RP, r = o % RP;
+        Yb[o] = make_float2((float)(Lm[r * P + 2 * b] * y_scale), (float)(Lm[r * P + 2 * b + 1] * y_scale));
+      }
+      __syncthreads();
+      // ---- one-sided block Jacobi in FP32 on JT threads ----
+      if (tid < JT) {
+        auto bar = [] { asm volatile("bar.sync 1, %0;" ::"n"(JT) : "memory"); };
+        const int m = tid >> 3, sub = tid & 7;
+        const bool active = m < GROUPS;
+        const int mc = min(m, GROUPS - 1);                // groups beyond the last one repeat its work and store nothing
+        float2* nrm2 = reinterpret_cast<float2*>(nrm);
+        // A group's access is 64 of a 128-byte line.  With an even number of chunks of eight rows, odd groups walk them in the
+        // order 1, 0, 3, 2, ..., so that the two groups of a half warp never meet in the same banks (n = 64: a sixth off a
+        // round); an odd number would need a padding chunk, which costs more than the conflicts.
+        const int odd = R % 2 == 0 ? m & 1 : 0;
+        auto row_of = [&](int t) { return sub + 8 * (t ^ odd); };
+        for (int sweep = 0; sweep < EIG_MAX_SWEEPS; ++sweep) {
+          // squared column norms: a group takes blocks 2m and 2m + 1
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float2 sq = make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int t = 0; t < R; ++t) { const float2 y = Yb[(2 * mc + h) * RP + sub + 8 * t]; sq = fma2(y, y, sq); }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) { sq.x += __shfl_xor_sync(0xFFFFFFFFu, sq.x, o); sq.y += __shfl_xor_sync(0xFFFFFFFFu, sq.y, o); }
+            if (active && sub == 0) nrm2[2 * m + h] = sq;
+          }
+          int p = pairs[0][mc][0], r = pairs[0][mc][1];
+          bar();
+          bool above = false;
+          for (int step = 0; step < NB - 1; ++step) {
+            float2* yp = Yb + p * RP;
+            float2* yr = Yb + r * RP;
+            float2 a[R], b[R];                              // columns (0, 1) and (2, 3)
+#pragma unroll
+            for (int t = 0; t < R; ++t) { a[t] = yp[row_of(t)]; b[t] = yr[row_of(t)]; }
+            const int pn = pairs[step + 1][mc][0], rn = pairs[step + 1][mc][1];  // (the table has a row more than it fills)
+            float2 n01 = nrm2[p], n23 = nrm2[r];
+            block_rotate<R, 8>(a, b, n01, n23, step == 0, exit_cos2, above);
+            if (active) {
+#pragma unroll
+              for (int t = 0; t < R; ++t) { yp[row_of(t)] = a[t]; yr[row_of(t)] = b[t]; }
+              if (sub == 0) { nrm2[p] = n01; nrm2[r] = n23; }
+            }
+            p = pn; r = rn;
+            bar();
+          }
+          if (__any_sync(0xFFFFFFFFu, above && active) && lane == 0) flags[sweep] = 1;
+          bar();
+          if (!flags[sweep]) break;
+        }
+        // reciprocal column lengths in FP64 (0 for a zero column)
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          float2 sq = make_float2(0.0f, 0.0f);
+          double sx = 0.0, sy = 0.0;
 #pragma unroll
-          for (int t = 0; t < R; ++t) { const float2 y = Yb[(2 * mc + h) * RP + sub + 8 * t]; sq = fma2(y, y, sq); }
-#pragma unroll
-          for (int o = 4; o > 0; o >>= 1) { sq.x += __shfl_xor_sync(0xFFFFFFFFu, sq.x, o); sq.y += __shfl_xor_sync(0xFFFFFFFFu, sq.y, o); }
-          if (active && sub == 0) nrm2[2 * m + h] = sq;
-        }
-        int p = pairs[0][mc][0], r = pairs[0][mc][1];
-        bar();
-        bool above = false;
-        for (int step = 0; step < NB - 1; ++step) {
-          float2* yp = Yb + p * RP;
-          float2* yr = Yb + r * RP;
-          float2 a[R], b[R];                              // columns (0, 1) and (2, 3)
-#pragma unroll
-          for (int t = 0; t < R; ++t) { a[t] = yp[row_of(t)]; b[t] = yr[row_of(t)]; }
-          const int pn = pairs[step + 1][mc][0], rn = pairs[step + 1][mc][1];  // (the table has a row more than it fills)
-          float2 n01 = nrm2[p], n23 = nrm2[r];
-          block_rotate<R, 8>(a, b, n01, n23, step == 0, exit_cos2, above);
-          if (active) {
-#pragma unroll
-            for (int t = 0; t < R; ++t) { yp[row_of(t)] = a[t]; yr[row_of(t)] = b[t]; }
-            if (sub == 0) { nrm2[p] = n01; nrm2[r] = n23; }
+          for (int t = 0; t < R; ++t) {
+            const float2 y = Yb[(2 * mc + h) * RP + sub + 8 * t];
+            sx = fma((double)y.x, (double)y.x, sx); sy = fma((double)y.y, (double)y.y, sy);
           }
-          p = pn; r = rn;
-          bar();
-        }
-        if (__any_sync(0xFFFFFFFFu, above && active) && lane == 0) flags[attempt][sweep] = 1;
-        bar();
-        if (!flags[attempt][sweep]) break;
-      }
-      // reciprocal column lengths in FP64 (0 for a zero column)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        double sx = 0.0, sy = 0.0;
-#pragma unroll
-        for (int t = 0; t < R; ++t) {
-          const float2 y = Yb[(2 * mc + h) * RP + sub + 8 * t];
-          sx = fma((double)y.x, (double)y.x, sx); sy = fma((double)y.y, (double)y.y, sy);
-        }
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) { sx += __shfl_xor_sync(0xFFFFFFFFu, sx, o); sy += __shfl_xor_sync(0xFFFFFFFFu, sy, o); }
-        if (active && sub < 2) {
-          const double v = sub == 0 ? sx : sy;
-          inv_s[2 * (2 * m + h) + sub] = v > 0.0 ? rsqrt64(v) : 0.0;
+          for (int o = 4; o > 0; o >>= 1) { sx += __shfl_xor_sync(0xFFFFFFFFu, sx, o); sy += __shfl_xor_sync(0xFFFFFFFFu, sy, o); }
+          if (active && sub < 2) {
+            const double v = sub == 0 ? sx : sy;
+            inv_s[2 * (2 * m + h) + sub] = v > 0.0 ? rsqrt64(v) : 0.0;
+          }
         }
       }
-    }
-    __syncthreads();
+      __syncthreads();
 
-    // ---- U = normalised columns (zero columns stay zero) ----
-    for (int o = tid; o < N8 * N8; o += EIG_THREADS) {
-      const int i = o / N8, j = o % N8;
-      U[i * P + j] = (double)(reinterpret_cast<const float*>(Yb + (j >> 1) * RP + i)[j & 1]) * inv_s[j];
+      // ---- U = normalised columns (zero columns stay zero) ----
+      for (int o = tid; o < N8 * N8; o += EIG_THREADS) {
+        const int i = o / N8, j = o % N8;
+        U[i * P + j] = (double)(reinterpret_cast<const float*>(Yb + (j >> 1) * RP + i)[j & 1]) * inv_s[j];
+      }
+      __syncthreads();
     }
-    __syncthreads();
 
     // ---- FP64 refinement ----
     for (int it = 0; it < EIG_MAX_REFINE; ++it) {
@@ -529,7 +861,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
 #pragma unroll
       for (int w = 0; w < N_WARPS; ++w) norm2 += en_w[w];
       if (still_open || !(norm2 < 0.0625f)) {
-        if (attempt == 0) { again = true; break; }        // back to the FP32 sweeps, with the tight exit test
+        if (attempt == 0) { again = true; break; }        // the FP32 sweeps make another start
         still_open = 1;
         if (!(norm2 < 0.0625f)) { orth_only = true; continue; }                    // the same step once more, pairs only orthonormalised
       }

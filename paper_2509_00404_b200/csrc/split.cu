@@ -1065,7 +1065,7 @@ int gram_parts(int64_t n_rows, int64_t* rows_per_part) {
 
 metis_status_t launch_eig(cudaStream_t s, const double* g, int n, int ld, double* evals, double* evecs) {
   const size_t smem = metis_small::eig_smem(n);
-#define METIS_EIG(NT8) case NT8: METIS_CUDA_TRY(metis_launch_pdl((metis_small::eig_kernel<NT8>), dim3(1), dim3(metis_small::EIG_THREADS), smem, s, g, n, ld, evals, evecs)); break
+#define METIS_EIG(NT8) case NT8: METIS_CUDA_TRY(metis_launch_pdl((metis_small::eig_kernel<NT8>), dim3(1), dim3(metis_small::eig_threads(NT8)), smem, s, g, n, ld, evals, evecs)); break
   switch ((n + 7) / 8) {
     METIS_EIG(1); METIS_EIG(2); METIS_EIG(3); METIS_EIG(4); METIS_EIG(5); METIS_EIG(6); METIS_EIG(7); METIS_EIG(8); METIS_EIG(9);
     default: return METIS_ERR_SHAPE;

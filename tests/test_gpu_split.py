@@ -482,3 +482,29 @@ def test_eigen_solvers_of_sampled_splits(ctx, k, p, spectrum):
     assert (core - torch.diag(torch.diagonal(core))).abs().max() < tol * sig[0]
     assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
     assert bool((sig[:-1] >= sig[1:]).all())
+
+
+@pytest.mark.parametrize("k,p", [(4, 3), (32, 0), (28, 5), (32, 8), (40, 1), (56, 8), (60, 5), (64, 7)])
+@pytest.mark.parametrize("spectrum", ["geometric", "pairs", "apart"])
+def test_eigen_solver_size_classes_and_exact_pairs(ctx, k, p, spectrum):
+    """The sizes at which the multisection changes its lanes per eigenvalue (n = 32 / 33, 40 / 41, 64 / 65) and orders that are no
+    multiple of eight; "pairs": an operand of two equal diagonal blocks, every singular value of which is there twice to the last digit (the
+    tridiagonal start has dependent vectors, or parts that do not couple).  Bounds as above."""
+    B, h = ctx
+    if spectrum == "pairs":
+        x = torch.zeros((1536, 640), dtype=torch.bfloat16, device="cuda")
+        x[:768, :320] = _planted(768, 640, k // 2, "geometric", 7 * k + p)[:, :320]
+        x[768:, 320:] = x[:768, :320]
+    else:
+        x = _planted(1536, 640, k, spectrum, 100 * k + p)
+    op = h.split(x, k, p, sketch=B.SKETCH_FULL, seed=11)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    left, right, sig, xd = op.left.double(), op.right.double(), op.sigma.double(), x.double()
+    eye = torch.eye(k, device="cuda", dtype=torch.float64)
+    tol = 1e-6 + 2.0 ** -23 * float(sig[0] / sig[-1])
+    assert (left @ left.T - eye).abs().max() < 1e-6 and (right @ right.T - eye).abs().max() < tol
+    core = left @ xd @ right.T
+    assert (core - torch.diag(torch.diagonal(core))).abs().max() < tol * sig[0]
+    assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
+    assert bool((sig[:-1] >= sig[1:]).all())
