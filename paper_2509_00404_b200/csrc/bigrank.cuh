@@ -9,9 +9,11 @@
 //   trsm_wide_kernel         H = Z L^-T by blocked forward substitution (32 rows of Z per CTA)
 //   gemm64_kernel            C = A B with FP32 A, FP64 B and FP64 accumulation, arbitrary strides (right basis,
 //                            factor rotations)
-//   jacobi_fp32_kernel       FP32 one-sided block Jacobi on a cluster of two to six CTAs: the columns live in the cluster's
-//                            distributed shared memory, column blocks travel between CTAs by DSMEM stores
-//   refine_*_kernel          FP64 refinement of the eigenvectors it found (steps of matrix products), eigen_finish_kernel
+//   tridiag_chol_kernel      up to 144: Householder reduction in one CTA's registers beside the factorisation in another's shared
+//                            memory; tridiag_vectors_kernel, tridiag_back_kernel: eigenvectors of the tridiagonal matrix, taken back
+//   jacobi_fp32_kernel       above that, FP32 one-sided block Jacobi on a cluster of four to six CTAs: the columns live in the
+//                            cluster's distributed shared memory, column blocks travel between CTAs by DSMEM stores
+//   refine_*_kernel          FP64 refinement of the eigenvectors they found (steps of matrix products), eigen_finish_kernel
 //   jacobi_cluster_kernel    the FP64 form of the sweeps, and jacobi_collect_kernel: only run for matrices the refinement
 //                            cannot finish (eigenvalues that agree to working precision)
 //   sign_rows_kernel         sign convention of the factor pairs
@@ -19,6 +21,8 @@
 // Included by split.cu only.
 #pragma once
 #include <cooperative_groups.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 #include "small_eig.cuh"
@@ -276,11 +280,8 @@ chol_wide_kernel(const double* __restrict__ g, int n, double tol_rel, double* l_
 // diagonal blocks, one warp each.
 constexpr int CM_MAX = 160, CM_P = CM_MAX + 4;
 __host__ __device__ constexpr size_t cm_smem(int n) { return sizeof(double) * (size_t)((n + 7) / 8 * 8) * CM_P; }
-__global__ void __launch_bounds__(CW_THREADS, 1)
-chol_mid_kernel(const double* __restrict__ g, int n, double tol_rel, double* __restrict__ l_out, double* dinv_out, int* perm_out, EigState* state,
-                const int* __restrict__ skip, int* __restrict__ well_conditioned) {
-  metis_pdl_wait();
-  if (skip != nullptr && *skip) return;
+__device__ __forceinline__ void chol_mid(const double* __restrict__ g, int n, double tol_rel, double* __restrict__ l_out, double* dinv_out, int* perm_out,
+                                         EigState* state, int* __restrict__ well_conditioned) {
   extern __shared__ __align__(16) unsigned char cm_sm[];
   double* Y = reinterpret_cast<double*>(cm_sm);
   __shared__ double diag[CM_MAX], inv_s[CM_MAX];
@@ -341,6 +342,14 @@ chol_mid_kernel(const double* __restrict__ g, int n, double tol_rel, double* __r
       dinv_out[(int64_t)warp * CW_NB * CW_NB + i * CW_NB + lane] = x[i];
     }
   }
+}
+
+__global__ void __launch_bounds__(CW_THREADS, 1)
+chol_mid_kernel(const double* __restrict__ g, int n, double tol_rel, double* __restrict__ l_out, double* dinv_out, int* perm_out, EigState* state,
+                const int* __restrict__ skip, int* __restrict__ well_conditioned) {
+  metis_pdl_wait();
+  if (skip != nullptr && *skip) return;
+  chol_mid(g, n, tol_rel, l_out, dinv_out, perm_out, state, well_conditioned);
 }
 
 // H = Z L^-T by blocked forward substitution, in place: for panel J of CW_NB columns
@@ -478,12 +487,13 @@ __global__ void rot_scales_kernel(const double* __restrict__ evals, const float*
 
 // ------------------------------------------------------------------------------------------------
 // Symmetric eigen-decomposition of a Gram matrix of n up to MAXQ_WIDE, in the steps of the one-CTA solver (small_eig.cuh):
-// sorted Cholesky factor, FP32 block Jacobi, FP64 refinement with matrix products over many CTAs; a matrix the refinement cannot
-// finish (pairs of eigenvalues too close, or no convergence) is done by the FP64 Jacobi kernels, which otherwise return at
-// once.  The decisions are made on the device, in EigState, so that a call needs no host synchronisation.
-// Measured inside a layer step, n = 136: factorisation, solver and collection 138 + 1590 + 21 us before (FP64 sweeps on the cluster), now
-// 45 + 338 + 60 us.  Repeated eigenvalues pay for both solvers: a decomposition of 1024 x 768 from every row, k = 128, all
-// planted values equal, 2187 -> 2583 us.
+// sorted Cholesky factor, a start (tridiagonal matrix up to n = 144, FP32 block Jacobi above), FP64 refinement with matrix products over
+// many CTAs; a matrix the refinement cannot finish (pairs of eigenvalues too close, or no convergence) is done by the FP64 Jacobi
+// kernels, which otherwise return at once.  The decisions are made on the device, in EigState, so that a call needs no host
+// synchronisation.
+// Measured inside a layer step, factorisation and start: n = 136 243 us (reduction 202, vectors 20, back 20; factorisation and FP32
+// Jacobi before: 43 + 338), n = 128 190 us (37 + 276), n = 104 165 us; refinement, finish and collection 60 us.  Repeated eigenvalues pay
+// for both solvers.
 constexpr int ER_STEPS = 3;                               // refinement steps (two are enough unless eigenvalues are close)
 struct EigState {
   unsigned int emax[ER_STEPS];                            // largest |E_ij| of a step (bits)
@@ -663,6 +673,436 @@ jacobi_fp32_kernel(const double* __restrict__ l, int n, double* __restrict__ x) 
       if (i < n && c < n) x[(int64_t)i * n + c] = (double)v.x * rx;
       if (i < n && c + 1 < n) x[(int64_t)i * n + c + 1] = (double)v.y * ry;
     }
+  }
+}
+
+// The start of the refinement up to n = WT_MAX, as in the one-CTA solver: Householder reduction to a tridiagonal matrix (CTA 0)
+// beside the sorted factorisation (CTA 1).  Fifteen warps hold the matrix in registers, warp w the rows w, w + 15, ..., a lane the
+// columns n - 1 - lane, n - 1 - lane - 32, ...: a column of the vectors is loaded once for all of a warp's rows (shared-memory delivery,
+// 128 bytes a cycle, is what a squarer tile of four lanes a row waits for), and what is finished drops out, three rows at a time.
+// Above n = 128 the first columns, finished first, live in shared memory: five per lane do not fit the registers.
+// The sixteenth warp works out the scalars, the vectors of the update and the next column, so that a step has two barriers.  A step takes
+// 2300 cycles at n = 128, 3300 over the first quarter: the shared-memory pipe (52 cycles a warp for the factors of 36 elements a lane,
+// 24 for the exchanges) and the FP64 pipe (54) share it with the scalars' 1050; one warp per row and lane would need the
+// products summed through shared memory, five columns per lane spilled (n = 136: 309 us).
+// Outputs: v[j][.] the reflectors (zero up to column j), tri = d, e, beta (n each).
+constexpr int WT_WARPS = 15, WT_THREADS = 32 * (WT_WARPS + 1), WT_MAX = 144, WT_TAIL = 16, WT_ROWS = 3;
+static_assert(WT_MAX <= CM_MAX && WT_THREADS >= CW_THREADS, "the factorisation runs in the same launch");
+template <int R, int C, bool TAIL>                        // rows per warp (15 R >= n), columns per lane (32 C + TAIL * WT_TAIL >= n)
+__global__ void __launch_bounds__(WT_THREADS, 1)
+tridiag_chol_kernel(const double* __restrict__ gm, int n, double* __restrict__ l_out, int* __restrict__ perm_out, EigState* __restrict__ state,
+                    double* __restrict__ v_out, double* __restrict__ tri) {
+  metis_pdl_wait();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (blockIdx.x == 1) {
+    if (tid < CW_THREADS) chol_mid(gm, n, 1e-14, l_out, nullptr, perm_out, state, nullptr);
+    return;
+  }
+  constexpr int CS = TAIL ? C + 1 : C, NP = 32 * CS;      // columns per lane of the scalars' warp
+  __shared__ double xs_[32 + NP], rs_[32 + NP], us_[32 + NP], ys[NP];          // the first 32 stay zero: columns below the first
+  __shared__ __align__(16) double2 pq[NP];
+  __shared__ double tail[TAIL ? WT_MAX + WT_WARPS : 1][WT_TAIL];               // columns 0 ... n - 32 C - 1
+  double *xs = xs_ + 32, *rs = rs_ + 32, *us = us_ + 32;
+  for (int i = tid; i < 32 + NP; i += WT_THREADS) { xs_[i] = 0.0; rs_[i] = 0.0; us_[i] = 0.0; if (i < NP) { ys[i] = 0.0; pq[i] = make_double2(0.0, 0.0); } }
+  int top = 0;                                            // an even power of two brings the largest entry near one
+  for (int i = lane; i < n; i += 32) top = max(top, __double2hiint(gm[(int64_t)i * n + i]));
+  top = __reduce_max_sync(0xFFFFFFFFu, top) >> 20;
+  const int ex = top > 0 && top < 2046 ? (top - 1022 + 1) >> 1 : 0;
+  const double scale = __hiloint2double((1023 - 2 * ex) << 20, 0);
+  double *d_out = tri, *e_out = tri + n, *b_out = tri + 2 * n;
+  const int n_tail = TAIL ? n - 32 * C : 0;
+  __syncthreads();
+  if (warp < WT_WARPS) {
+    const int c0 = n - 1 - lane;                          // column of t = 0
+    double row[R][C];
+#pragma unroll
+    for (int a = 0; a < R; ++a) {
+      const int i = warp + WT_WARPS * a;
+#pragma unroll
+      for (int t = 0; t < C; ++t) row[a][t] = i < n && c0 - 32 * t >= 0 ? gm[(int64_t)i * n + c0 - 32 * t] * scale : 0.0;
+      if (TAIL && i < WT_MAX + WT_WARPS && lane < WT_TAIL) tail[i][lane] = i < n && lane < n_tail ? gm[(int64_t)i * n + lane] * scale : 0.0;
+    }
+    // row i, columns from `from` on
+    auto publish = [&](double* out, int i, int from) {
+      const int a_own = i / WT_WARPS;
+      if (i - a_own * WT_WARPS == warp) {
+        if (TAIL && lane < n_tail) out[lane] = lane >= from ? tail[i][lane] : 0.0;
+#pragma unroll
+        for (int a = 0; a < R; ++a)
+          if (a == a_own) {
+#pragma unroll
+            for (int t = 0; t < C; ++t) if (c0 - 32 * t >= 0) out[c0 - 32 * t] = c0 - 32 * t >= from ? row[a][t] : 0.0;
+          }
+      }
+    };
+    __syncwarp();
+    publish(xs, 0, 1);
+    if (tid == 0) d_out[0] = gm[0] * scale;
+    __syncthreads();
+    double x[C];                                          // the vector of the last product
+#pragma unroll
+    for (int t = 0; t < C; ++t) x[t] = 0.0;
+    double x_tail = 0.0;
+    // the update of step j - 1 and the product of step j on the last rl rows and the last 32 cl columns, which are all that is left
+    auto work = [&](auto cl, auto rl, int j) {
+      constexpr int CL = decltype(cl)::value, RL = decltype(rl)::value, A0 = R - RL;
+      double u[CL], xn[CL], y[RL];
+#pragma unroll
+      for (int t = 0; t < CL; ++t) { u[t] = us[c0 - 32 * t]; xn[t] = xs[c0 - 32 * t]; }
+#pragma unroll
+      for (int b = 0; b < RL; b += WT_ROWS) {
+#pragma unroll
+        for (int a = b; a < b + WT_ROWS && a < RL; ++a) y[a] = 0.0;
+        if (warp + WT_WARPS * (A0 + b + WT_ROWS - 1) >= j) {
+          double2 c[WT_ROWS];
+#pragma unroll
+          for (int h = 0; h < WT_ROWS; ++h) if (b + h < RL) c[h] = pq[warp + WT_WARPS * (A0 + b + h)];
+#pragma unroll
+          for (int h = 0; h < WT_ROWS; ++h)               // (a factor that stays from one multiply-add to the next is read once)
+            if (b + h < RL) {
+#pragma unroll
+              for (int t = 0; t < CL; ++t) row[A0 + b + h][t] = fma(c[h].y, x[t], row[A0 + b + h][t]);
+#pragma unroll
+              for (int t = 0; t < CL; ++t) row[A0 + b + h][t] = fma(c[h].x, u[t], row[A0 + b + h][t]);
+            }
+#pragma unroll
+          for (int t = 0; t < CL; ++t)
+#pragma unroll
+            for (int h = 0; h < WT_ROWS; ++h)
+              if (b + h < RL) y[b + h] = fma(row[A0 + b + h][t], xn[t], y[b + h]);
+        }
+      }
+      if (TAIL && CL == C && j <= n_tail && lane < n_tail) {
+        const double ut = us[lane], xt = xs[lane];
+#pragma unroll
+        for (int a = 0; a < RL; ++a) {
+          const double2 c = pq[warp + WT_WARPS * (A0 + a)];
+          double* at = &tail[warp + WT_WARPS * (A0 + a)][lane];
+          const double v = fma(c.x, ut, fma(c.y, x_tail, *at));
+          *at = v;
+          y[a] = fma(v, xt, y[a]);
+        }
+        x_tail = xt;
+      }
+#pragma unroll
+      for (int t = 0; t < CL; ++t) x[t] = xn[t];
+      // sums over the lanes: at each exchange half of the values go to the other half of the lanes; a lane ends with row `mine`
+      int m = RL, mine = 0, half_at[5];
+#pragma unroll
+      for (int k = 0; k < 5; ++k) {
+        const int o = 16 >> k, half = (m + 1) / 2;
+        const bool hi = lane & o;
+#pragma unroll
+        for (int h = 0; h < half; ++h) {
+          if (h + half < m) {
+            const double give = hi ? y[h] : y[h + half], keep = hi ? y[h + half] : y[h];
+            y[h] = keep + __shfl_xor_sync(0xFFFFFFFFu, give, o);
+          } else {
+            y[h] += __shfl_xor_sync(0xFFFFFFFFu, y[h], o);
+          }
+        }
+        half_at[k] = half;
+        m = half;
+      }
+#pragma unroll
+      for (int k = 4; k >= 0; --k)
+        if (mine + half_at[k] < (k == 0 ? RL : half_at[k > 0 ? k - 1 : 0]) && (lane & (16 >> k))) mine += half_at[k];
+      ys[warp + WT_WARPS * (A0 + mine)] = y[0];
+      __syncwarp();
+      publish(rs, j + 1, j + 1);
+    };
+    constexpr int N_MAX = 32 * C + (TAIL ? WT_TAIL : 0), R2 = C > 2 ? R - (N_MAX - 64) / WT_WARPS : R, R1 = R - (N_MAX - 32) / WT_WARPS;
+    const int from2 = max(n - 64, WT_WARPS * (R - R2)), from1 = max(n - 32, WT_WARPS * (R - R1));   // what the later forms leave out is finished
+#pragma unroll 1
+    for (int j = 0; j + 2 < n; ++j) {
+      if (warp + WT_WARPS * (R - 1) >= j) {
+        if (j >= from1) work(std::integral_constant<int, 1>(), std::integral_constant<int, R1>(), j);
+        else if (j >= from2) work(std::integral_constant<int, 2>(), std::integral_constant<int, R2>(), j);
+        else work(std::integral_constant<int, C>(), std::integral_constant<int, R>(), j);
+      }
+      __syncthreads();                                    // the product is there
+      __syncthreads();                                    // the next update and the next column are there
+    }
+    // the last diagonal entry, with the last update
+    if (lane == 0) {
+#pragma unroll
+      for (int a = 0; a < R; ++a) {
+        const int i = warp + WT_WARPS * a;
+        if (i == n - 1) d_out[n - 1] = fma(pq[i].x, us[n - 1], fma(pq[i].y, x[0], row[a][0]));
+      }
+    }
+  } else {
+    // with y = A x and r = A e_1 it is A v = u = y - alpha r,  v^T A v = x^T y - 2 alpha y_1 + alpha^2 r_1;  w = beta u - K v,
+    // A -= v w^T + w v^T = p u^T + q v^T.  Column j + 1 of the product is not read again except for its first entry, so x
+    // stands for v in the last term.  The next column, r + u_1 p + v_1 q, needs no row of the updated matrix: this warp goes on with its
+    // length and its reflector while the others update and multiply.
+    __syncthreads();
+    double x[CS];
+#pragma unroll
+    for (int t = 0; t < CS; ++t) x[t] = xs[lane + 32 * t];
+#pragma unroll 1
+    for (int j = 0; j + 2 < n; ++j) {
+      double r[CS], y[CS], sq = 0.0, xy = 0.0, alpha, beta;
+      const double x0 = xs[j + 1];
+#pragma unroll
+      for (int t = 0; t < CS; ++t) sq = fma(x[t], x[t], sq);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xFFFFFFFFu, sq, o);
+      metis_tri::reflector(x0, sq, alpha, beta);
+      const double b2 = beta * beta, v1 = x0 - alpha;
+#pragma unroll
+      for (int t = 0; t < CS; ++t)
+        if (lane + 32 * t < n) v_out[(int64_t)j * n + lane + 32 * t] = lane + 32 * t == j + 1 ? v1 : x[t];
+      if (lane == 0) { e_out[j] = alpha; b_out[j] = beta; }
+      __syncthreads();                                    // the product is there
+#pragma unroll
+      for (int t = 0; t < CS; ++t) { y[t] = ys[lane + 32 * t]; r[t] = rs[lane + 32 * t]; xy = fma(x[t], y[t], xy); }
+      const double ya = ys[j + 1], ra = rs[j + 1], k0 = fma(alpha, fma(alpha, ra, -2.0 * ya), 0.0), u1 = fma(-alpha, ra, ya);
+#pragma unroll
+      for (int t = 0; t < CS; ++t) { y[t] = fma(-alpha, r[t], y[t]); us[lane + 32 * t] = y[t]; }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) xy += __shfl_xor_sync(0xFFFFFFFFu, xy, o);
+      const double K2 = b2 * (xy + k0);
+#pragma unroll
+      for (int t = 0; t < CS; ++t) {
+        const int c = lane + 32 * t;
+        const double v = c == j + 1 ? v1 : x[t], p = -beta * v, qv = fma(-beta, y[t], K2 * v);
+        pq[c] = make_double2(p, qv);
+        x[t] = c > j + 1 ? fma(v1, qv, fma(u1, p, r[t])) : 0.0;
+        xs[c] = x[t];
+      }
+      if (lane == 0) d_out[j + 1] = fma(-v1, fma(2.0 * beta, u1, -K2 * v1), ra);
+      __syncthreads();                                    // the next update and the next column are there
+    }
+    if (lane == 0) e_out[n - 2] = xs[n - 1];
+  }
+}
+
+// Eigenvalue and eigenvector number e (descending) of the tridiagonal matrix, one warp each (zt[e][.], normalised): multisection into 33 parts,
+// a round costs 13 cycles per row (two points per lane: 24), twisted factorisation.  Behind them, one warp per panel of eight
+// reflectors: H_8b ... H_8b+7 = I - V_b^T T_b V_b (T_b: inverse of diag(1 / beta) + the upper triangle of V_b V_b^T).
+constexpr int WV_WARPS = 4, WV_ROUNDS = 7;                // of the multisection: relative width 2^-29
+__global__ void __launch_bounds__(32 * WV_WARPS)
+tridiag_vectors_kernel(const double* __restrict__ tri, const double* __restrict__ v, int n, double* __restrict__ zt, double* __restrict__ panels) {
+  metis_pdl_wait();
+  __shared__ __align__(16) double2 te[WT_MAX + 1];
+  __shared__ double eo[WT_MAX + 1], dn[WV_WARPS][WT_MAX], up[WV_WARPS][WT_MAX];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
+  const int n8 = (n + 7) & ~7, groups = (n + WV_WARPS - 1) / WV_WARPS;
+  if ((int)blockIdx.x >= groups) {
+    const int b = ((int)blockIdx.x - groups) * WV_WARPS + warp;
+    if (8 * b + 2 >= n) return;
+    double acc[2][2] = {};
+    const bool on = 8 * b + g + 2 < n;
+    const double* row = v + (int64_t)(on ? 8 * b + g : 0) * n;
+#pragma unroll 4
+    for (int kk = 0; kk < n8; kk += 8)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = kk + 4 * h + q;
+        const double a = on && c < n ? row[c] : 0.0;
+        metis_small::dmma(acc[h], a, a);                  // the fragments of V_b and of its transpose hold the same entries
+      }
+    double* t = dn[warp];
+    t[8 * g + 2 * q] = acc[0][0] + acc[1][0]; t[8 * g + 2 * q + 1] = acc[0][1] + acc[1][1];
+    __syncwarp();
+    if (lane < 8) {
+      double x[8];                                        // column `lane` of the lower triangular inverse: T_b transposed
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        double sum = 0.0;
+#pragma unroll
+        for (int k = 0; k < i; ++k) sum = fma(t[8 * i + k], x[k], sum);
+        const double bt = 8 * b + i + 2 < n ? tri[2 * n + 8 * b + i] : 0.0;
+        x[i] = i == lane ? bt : (i > lane ? -bt * sum : 0.0);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) panels[64 * b + 8 * lane + i] = x[i];        // T_b[lane][i]
+    }
+    return;
+  }
+  for (int i = tid; i <= n8; i += 32 * WV_WARPS) {
+    const double e = i > 0 && i < n ? tri[n + i - 1] : 0.0;
+    te[i] = i < n ? make_double2(tri[i], i > 0 ? fmax(e * e, 1e-60) : 0.0) : make_double2(4.0 * WT_MAX, 0.0);
+    if (i > 0) eo[i - 1] = e;
+  }
+  __syncthreads();
+  const int e = (int)blockIdx.x * WV_WARPS + warp;
+  if (e >= n) return;
+  double lm;
+  {
+    long long lo = __double_as_longlong(0x1p-56), hi = __double_as_longlong(2.0 * WT_MAX);
+#pragma unroll 1
+    for (int r = 0; r < WV_ROUNDS; ++r) {
+      const long long w = (long long)((unsigned long long)(hi - lo + 32) / 33);
+      const double x[1] = {__longlong_as_double(lo + w * (lane + 1))};
+      int c[1];
+      metis_tri::sturm_counts<1>(te, n8 >> 3, x, c);
+      const unsigned int over = __ballot_sync(0xFFFFFFFFu, c[0] > n - 1 - e);
+      const int f = over != 0u ? __ffs((int)over) - 1 : 32;
+      hi = lo + w * (f + 1);
+      lo += w * f;
+    }
+    lm = __longlong_as_double(lo + ((hi - lo) >> 1));
+  }
+  double *Dp = dn[warp], *Dm = up[warp];
+  if (lane < 2) {                                         // pivots from the top and from the bottom
+    double* D = lane ? Dm : Dp;
+    double pm = 0.0, p = 1.0;
+#pragma unroll 1
+    for (int b = 0; b < n8; b += 8) {
+      double d[8], e2[8];                                 // (rows beyond the matrix read padding, forwards, or row 0, backwards; nothing is kept)
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = b + u;
+        d[u] = te[lane ? max(n - 1 - i, 0) : i].x - lm;
+        e2[u] = te[lane ? max(n - i, 0) : i].y;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const double pn = fma(d[u], p, -e2[u] * pm);
+        d[u] = pn * metis_tri::rcp_mid(p + 1e-290);
+        pm = p; p = pn;
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = b + u;
+        if (i < n) D[lane ? n - 1 - i : i] = d[u];
+      }
+      const int big = max(__double2hiint(p) & 0x7FF00000, __double2hiint(pm) & 0x7FF00000);
+      const double sc = __hiloint2double(0x7FE00000 - big, 0);
+      p *= sc; pm *= sc;
+    }
+  }
+  __syncwarp();
+  // twist where |gamma| is least: z = 1 there, the other entries are products of e / pivot outwards from it
+  double best = 1e300;
+  int at = 0;
+  for (int i = lane; i < n; i += 32) {
+    const double gamma = fabs(Dp[i] + Dm[i] - (te[i].x - lm));
+    if (gamma < best) { best = gamma; at = i; }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double other = __shfl_xor_sync(0xFFFFFFFFu, best, o);
+    const int oi = __shfl_xor_sync(0xFFFFFFFFu, at, o);
+    if (other < best || (other == best && oi < at)) { best = other; at = oi; }
+  }
+  for (int i = lane; i < n; i += 32) {
+    const double f = eo[i < at ? i : max(i - 1, 0)] * metis_tri::rcp_mid((i < at ? Dp[i] : Dm[i]) + 1e-60);
+    Dm[i] = i == at ? 1.0 : -f;
+  }
+  __syncwarp();
+  double zz = lane == 0 ? 1.0 : 0.0;
+  if (lane < 2) {
+    const int step = lane ? 1 : -1;
+    double f = 1.0;
+    for (int i = at + step; i >= 0 && i < n; i += 8 * step) {                  // eight at a time, the loads ahead of the products
+      double m[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) { const int k = i + u * step; m[u] = k >= 0 && k < n ? Dm[k] : 0.0; }
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int k = i + u * step;
+        f *= m[u];
+        zz = fma(f, f, zz);
+        if (k >= 0 && k < n) Dm[k] = f;
+      }
+    }
+  }
+  __syncwarp();
+  zz += __shfl_xor_sync(0xFFFFFFFFu, zz, 1);
+  const double rz = metis_tri::rsqrt_mid(__shfl_sync(0xFFFFFFFFu, zz, 0));
+  for (int i = lane; i < n; i += 32) zt[(int64_t)e * n + i] = Dm[i] * rz;
+}
+
+// x (n x n, column e: vector e, rows in the order of the factor's) = H_0 H_1 ... zt^T: eight vectors per CTA, panel by panel from the
+// last, the sums over rows and then the rows dealt out to eight warps; the reflectors in shared memory.  Vectors beyond the
+// factor's rank are zero.
+constexpr int WB_WARPS = 8, WB_THREADS = 32 * WB_WARPS, WB_ZP = 12, WB_TILES = (WT_MAX / 8 + WB_WARPS - 1) / WB_WARPS;
+__host__ __device__ constexpr size_t wb_smem(int n) { return sizeof(double) * (size_t)((n + 7) / 8 * 8) * ((n + 7) / 8 * 8 + 4 + WB_ZP); }
+__global__ void __launch_bounds__(WB_THREADS)
+tridiag_back_kernel(const double* __restrict__ zt, const double* __restrict__ v, const double* __restrict__ panels, const double* __restrict__ l,
+                    const int* __restrict__ perm, int n, double* __restrict__ x) {
+  metis_pdl_wait();
+  extern __shared__ __align__(16) unsigned char wb_sm[];
+  const int n8 = (n + 7) & ~7, P = n8 + 4;
+  double* V = reinterpret_cast<double*>(wb_sm);           // [n8][P]
+  double* Z = V + (size_t)n8 * P;                         // [n8][WB_ZP]: eight vectors as columns
+  __shared__ double Ts[8 * WT_MAX], part[WB_WARPS][64], patch[64];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3, e0 = 8 * (int)blockIdx.x;
+  const int n_panels = (n - 2 + 7) / 8;
+  constexpr int CT = (WT_MAX + 31) / 32;
+#pragma unroll 4
+  for (int j = warp; j < n8; j += WB_WARPS) {
+    double r[CT];
+#pragma unroll
+    for (int t = 0; t < CT; ++t) r[t] = j + 2 < n && lane + 32 * t < n ? v[(int64_t)j * n + lane + 32 * t] : 0.0;
+#pragma unroll
+    for (int t = 0; t < CT; ++t) if (lane + 32 * t < n8) V[j * P + lane + 32 * t] = r[t];
+  }
+  for (int o = tid; o < 64 * n_panels; o += WB_THREADS) Ts[o] = panels[o];
+#pragma unroll
+  for (int t = 0; t < CT; ++t) {                          // a warp per vector
+    const int i = lane + 32 * t;
+    if (i < n8) Z[i * WB_ZP + warp] = e0 + warp < n && i < n ? zt[(int64_t)(e0 + warp) * n + i] : 0.0;
+  }
+  const int rank = __syncthreads_count(tid < n && l[(int64_t)min(tid, n - 1) * (n + 1)] > 0.0);
+  const int tiles = n8 / 8;
+  for (int b = n_panels - 1; b >= 0; --b) {
+    double acc[2][2] = {}, fa[WB_TILES][2], fb[WB_TILES][2];
+#pragma unroll
+    for (int u = 0; u < WB_TILES; ++u) {
+      const int t = warp + WB_WARPS * u;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        fa[u][h] = t < tiles ? V[(8 * b + g) * P + 8 * t + 4 * h + q] : 0.0;
+        fb[u][h] = t < tiles ? Z[(8 * t + 4 * h + q) * WB_ZP + g] : 0.0;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < WB_TILES; ++u)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) metis_small::dmma(acc[h], fa[u][h], fb[u][h]);
+    *reinterpret_cast<double2*>(&part[warp][8 * g + 2 * q]) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+    // the update's operands, on the way meanwhile
+    double d[WB_TILES][2];
+#pragma unroll
+    for (int u = 0; u < WB_TILES; ++u) {
+      const int t = warp + WB_WARPS * u;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        fa[u][h] = t < tiles ? V[(8 * b + 4 * h + q) * P + 8 * t + g] : 0.0;
+        d[u][h] = t < tiles ? Z[(8 * t + g) * WB_ZP + 2 * q + h] : 0.0;
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {                                      // -T_b (V_b Z)
+      double y[2] = {0.0, 0.0};
+#pragma unroll
+      for (int kk = 0; kk < 8; kk += 4) {
+        const int at = 8 * (kk + q) + g;
+        double sum = 0.0;
+#pragma unroll
+        for (int w = 0; w < WB_WARPS; ++w) sum += part[w][at];
+        metis_small::dmma(y, Ts[64 * b + 8 * g + kk + q], sum);
+      }
+      *reinterpret_cast<double2*>(patch + 8 * g + 2 * q) = make_double2(-y[0], -y[1]);
+    }
+    __syncthreads();
+    const double y0 = patch[8 * q + g], y1 = patch[8 * (q + 4) + g];
+#pragma unroll
+    for (int u = 0; u < WB_TILES; ++u) {
+      const int t = warp + WB_WARPS * u;
+      metis_small::dmma(d[u], fa[u][0], y0);
+      metis_small::dmma(d[u], fa[u][1], y1);
+      if (t < tiles) { Z[(8 * t + g) * WB_ZP + 2 * q] = d[u][0]; Z[(8 * t + g) * WB_ZP + 2 * q + 1] = d[u][1]; }
+    }
+    __syncthreads();
+  }
+  for (int o = tid; o < 8 * n; o += WB_THREADS) {
+    const int i = o >> 3, e = o & 7;
+    if (e0 + e < n) x[(int64_t)i * n + e0 + e] = e0 + e < rank ? Z[perm[i] * WB_ZP + e] : 0.0;
   }
 }
 

@@ -1224,6 +1224,19 @@ metis_status_t launch_jacobi_fp32(cudaStream_t s, const double* l, int n, double
   return METIS_OK;
 }
 
+// factor and starting vectors of a matrix of up to WT_MAX: v, zt, tri are scratch of n x n and (tri: 3 n and the panels' 8 n)
+template <int R, int C, bool TAIL>
+metis_status_t launch_tridiag(cudaStream_t s, const double* gram1, int n, double* l, int* perm, metis_wide::EigState* st, double* v, double* zt, double* tri, double* x) {
+  using namespace metis_wide;
+  double* panels = tri + 3 * n;
+  const unsigned vec = (unsigned)metis_ceil_div(n, WV_WARPS), pan = (unsigned)metis_ceil_div(metis_ceil_div(n - 2, 8), WV_WARPS);
+  METIS_CUDA_TRY(metis_launch_pdl((tridiag_chol_kernel<R, C, TAIL>), dim3(2), dim3(WT_THREADS), cm_smem(n), s, gram1, n, l, perm, st, v, tri)); METIS_COUNT_LAUNCH();
+  METIS_CUDA_TRY(metis_launch_pdl(tridiag_vectors_kernel, dim3(vec + pan), dim3(32 * WV_WARPS), (size_t)0, s, (const double*)tri, (const double*)v, n, zt, panels)); METIS_COUNT_LAUNCH();
+  METIS_CUDA_TRY(metis_launch_pdl(tridiag_back_kernel, dim3((unsigned)metis_ceil_div(n, 8)), dim3(WB_THREADS), wb_smem(n), s, (const double*)zt, (const double*)v,
+                                  (const double*)panels, (const double*)l, (const int*)perm, n, x)); METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+
 metis_status_t launch_eig_wide(cudaStream_t s, const double* gram1, int n, double* scratch, double* l, double* ycm, double* evals, double* evecs) {
   if (n <= MAXQ) return launch_eig(s, gram1, n, n, evals, evecs);               // a small rank with a large oversampling
   using namespace metis_wide;
@@ -1232,11 +1245,12 @@ metis_status_t launch_eig_wide(cudaStream_t s, const double* gram1, int n, doubl
   EigState* st = reinterpret_cast<EigState*>(scratch + 6 * nn);
   int* failed = reinterpret_cast<int*>(st + 1);
   int* perm = failed + 1;
-  METIS_TRY(launch_chol_wide(s, gram1, n, 1e-14, l, nullptr, perm, st, nullptr, nullptr));
-  if (n <= 96) METIS_TRY((launch_jacobi_fp32<8, 12>(s, l, n, x[0])));
-  else if (n <= 112) METIS_TRY((launch_jacobi_fp32<8, 14>(s, l, n, x[0])));
-  else if (n <= 128) METIS_TRY((launch_jacobi_fp32<8, 16>(s, l, n, x[0])));
-  else if (n <= 144) METIS_TRY((launch_jacobi_fp32<8, 18>(s, l, n, x[0])));
+  if (n <= 90) METIS_TRY((launch_tridiag<6, 3, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  else if (n <= 96) METIS_TRY((launch_tridiag<9, 3, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  else if (n <= 128) METIS_TRY((launch_tridiag<9, 4, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  else if (n <= WT_MAX) METIS_TRY((launch_tridiag<10, 4, true>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  else METIS_TRY(launch_chol_wide(s, gram1, n, 1e-14, l, nullptr, perm, st, nullptr, nullptr));
+  if (n <= WT_MAX) {}
   else if (n <= 176) METIS_TRY((launch_jacobi_fp32<8, 22>(s, l, n, x[0])));
   else if (n <= 192) METIS_TRY((launch_jacobi_fp32<16, 12>(s, l, n, x[0])));
   else if (n <= 224) METIS_TRY((launch_jacobi_fp32<16, 14>(s, l, n, x[0])));
@@ -1444,8 +1458,12 @@ metis_status_t metis_split_set_attrs() {
 #undef METIS_EIG_ATTR
   METIS_CUDA_TRY(cudaFuncSetAttribute(gram_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GC_MAX_SMEM));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::JC_SMEM));
+#define METIS_WT_ATTR(R, C, T) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::tridiag_chol_kernel<R, C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::cm_smem(metis_wide::WT_MAX)))
+  METIS_WT_ATTR(6, 3, false); METIS_WT_ATTR(9, 3, false); METIS_WT_ATTR(9, 4, false); METIS_WT_ATTR(10, 4, true);
+#undef METIS_WT_ATTR
+  METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::tridiag_back_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::wb_smem(metis_wide::WT_MAX)));
 #define METIS_JF_ATTR(LN, R) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_fp32_kernel<LN, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::jf_smem(LN, R)))
-  METIS_JF_ATTR(8, 12); METIS_JF_ATTR(8, 14); METIS_JF_ATTR(8, 16); METIS_JF_ATTR(8, 18); METIS_JF_ATTR(8, 22);
+  METIS_JF_ATTR(8, 22);
   METIS_JF_ATTR(16, 12); METIS_JF_ATTR(16, 14); METIS_JF_ATTR(16, 16); METIS_JF_ATTR(16, 18);
 #undef METIS_JF_ATTR
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::chol_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::cm_smem(metis_wide::CM_MAX)));

@@ -508,3 +508,29 @@ def test_eigen_solver_size_classes_and_exact_pairs(ctx, k, p, spectrum):
     assert (core - torch.diag(torch.diagonal(core))).abs().max() < tol * sig[0]
     assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
     assert bool((sig[:-1] >= sig[1:]).all())
+
+
+@pytest.mark.parametrize("k,p", [(84, 6), (84, 7), (88, 8), (92, 5), (124, 4), (128, 1), (136, 8), (144, 1)])
+@pytest.mark.parametrize("spectrum", ["geometric", "close", "pairs"])
+def test_wide_eigen_solver_at_the_edges_of_the_reduction(ctx, k, p, spectrum):
+    """Rows and columns per thread of the reduction change at n = 90 / 91, 96 / 97 and 128 / 129, the other start begins above n = 144; both
+    solves of a sampled split (n = k + p and n = k), and exact pairs of singular values (see the small solver's test).  Bounds as
+    for sampled splits."""
+    B, h = ctx
+    if spectrum == "pairs":
+        x = torch.zeros((1536, 640), dtype=torch.bfloat16, device="cuda")
+        x[:768, :320] = _planted(768, 640, k // 2, "geometric", 7 * k + p)[:, :320]
+        x[768:, 320:] = x[:768, :320]
+    else:
+        x = _planted(1536, 640, k, spectrum, 100 * k + p)
+    op = h.split(x, k, p, sketch=B.SKETCH_FULL if spectrum == "pairs" else B.SKETCH_SAMPLED, seed=11)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    left, right, sig, xd = op.left.double(), op.right.double(), op.sigma.double(), x.double()
+    eye = torch.eye(k, device="cuda", dtype=torch.float64)
+    tol = 1e-6 + 2.0 ** -21 * float(sig[0] / sig[-1])
+    assert (left @ left.T - eye).abs().max() < tol and (right @ right.T - eye).abs().max() < tol
+    core = left @ xd @ right.T
+    assert (core - torch.diag(torch.diagonal(core))).abs().max() < tol * sig[0]
+    assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
+    assert bool((sig[:-1] >= sig[1:]).all())
