@@ -339,17 +339,20 @@ rank_update_kernel(const float* __restrict__ y0, int64_t M, int64_t N, int kc, c
 //
 // A contraction whose large operand is read once: bound by the bytes of G.  A factor entry without its tensor scale
 // is an E2M1 x E4M3 product and exact in BF16, an FP32 gradient is three BF16 terms, so the products of mma.sync are
-// exact and only the FP32 sums round.  The tensor core truncates its sums, so an accumulator runs over one chunk (12 adds)
-// and is then added to an FP32 total.  A CTA owns a strip of 64 values of r; its four warps are 2 (r) x 2 (halves of a
-// chunk of 128 values of c), and the CTAs of a cluster divide the chunks; the 2 * cluster totals of a strip are added in a
+// exact and only the FP32 sums round.  The tensor core truncates its sums, so an accumulator runs over a quarter of a chunk (6 adds)
+// and is then added to an FP32 total.  A CTA owns a strip of 64 values of r; its eight warps are 2 (r) x 4 (quarters of a
+// chunk of 128 values of c), and the CTAs of a cluster divide the chunks; the 4 * cluster totals of a strip are added in a
 // fixed order at the end (shared memory, then distributed shared memory).
-// G goes from global memory straight into fragment registers - every element is used by exactly one thread; the
-// contraction index (and, for TRANS, r) is permuted so that each load is 16 bytes and a warp's loads cover whole
-// 64 / 128-byte runs - and the factor chunk is dequantized into shared memory, double-buffered.
-constexpr int FG_ROWS = 64, FG_CHUNK = 128, FG_KW = FG_CHUNK / 64, FG_THREADS = 64 * FG_KW, FG_PITCH = FG_CHUNK + 16;    // pitch: 8 words mod 32, conflict-free 64-bit fragment loads
-constexpr int fg_smem(int nt) {
-  const int stage = 2 * 8 * nt * FG_PITCH * 2, red = FG_KW * FG_ROWS * (8 * nt + 1) * 4;
-  return stage > red ? stage : red;
+// G comes through a ring of asynchronous copies (three FP32 chunks, five BF16 ones, in flight: 96 and 80 KB per SM; loads straight into
+// fragment registers, two steps ahead of twelve warps, left every warp waiting for memory four cycles in seven), the factor
+// chunk through registers a chunk ahead and, dequantized, through a double buffer; the contraction index (and, for TRANS, r) is permuted so that
+// a fragment load is four neighbours.  14336 x 4096 FP32, k = 32: 140 -> 102 us (TRANS = 0), 154 -> 76 us; a chunk of 32 KB takes
+// 1.45 us of an SM with two warps per scheduler, twice what its bytes take.
+constexpr int FG_ROWS = 64, FG_CHUNK = 128, FG_KW = FG_CHUNK / 32, FG_THREADS = 64 * FG_KW, FG_PITCH = FG_CHUNK + 16;    // pitch: 8 words mod 32, conflict-free 64-bit fragment loads
+constexpr int FG_QUADS = FG_ROWS * FG_CHUNK / 4 / FG_THREADS;                    // groups of four elements per thread and chunk
+__host__ __device__ constexpr int fg_stages(int es) { return es == 4 ? 4 : 6; }                      // chunks of G in flight or in use: 128 KB (FP32), 96 KB
+constexpr int fg_smem(int nt, int es) {                                          // (the sums at the end, 66 KB at most, take the ring's place)
+  return 2 * 8 * nt * FG_PITCH * 2 + fg_stages(es) * FG_ROWS * FG_CHUNK * es;
 }
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -365,23 +368,21 @@ __device__ __forceinline__ uint32_t take_bf16x2(float& x, float& y) {
   y -= __uint_as_float(w & 0xFFFF0000u);
   return w;
 }
-// four consecutive elements of G from index `off` on (VEC: 16-byte aligned FP32, 8-byte aligned BF16)
+// four consecutive elements of G into shared memory, zeros unless `in` (src is a valid address all the same; VEC: 16-byte aligned FP32, 8-byte aligned BF16, asynchronous)
 template <typename T, bool VEC>
-__device__ __forceinline__ float4 fg_load4(const T* g, int64_t off, bool in) {
-  float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  if (!in) return v;
-  if (sizeof(T) == 4) {
-    const float* f = reinterpret_cast<const float*>(g) + off;
-    if (VEC) v = __ldg(reinterpret_cast<const float4*>(f));
-    else v = make_float4(f[0], f[1], f[2], f[3]);
+__device__ __forceinline__ void fg_fetch4(uint32_t dst, const T* src, bool in) {
+  if (VEC) {
+    if (sizeof(T) == 4) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(dst), "l"(src), "r"(in ? 8 : 0) : "memory");
   } else {
-    const uint16_t* f = reinterpret_cast<const uint16_t*>(g) + off;
-    uint2 w;
-    if (VEC) w = __ldg(reinterpret_cast<const uint2*>(f));
-    else w = make_uint2((uint32_t)f[0] | ((uint32_t)f[1] << 16), (uint32_t)f[2] | ((uint32_t)f[3] << 16));
-    v = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
+    uint32_t w[4] = {0u, 0u, 0u, 0u};
+    if (in) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) w[e] = sizeof(T) == 4 ? reinterpret_cast<const uint32_t*>(src)[e] : (uint32_t)reinterpret_cast<const uint16_t*>(src)[e];
+    }
+    if (sizeof(T) == 4) asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]) : "memory");
+    else asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(dst), "r"(w[0] | (w[1] << 16)), "r"(w[2] | (w[3] << 16)) : "memory");
   }
-  return v;
 }
 
 // the two E2M1 codes of the low byte as FP16 (exact)
@@ -403,14 +404,16 @@ __device__ __noinline__ float fg_plain_sum(const T* g, int64_t stride, int64_t n
 }
 
 template <int NT, bool TRANS, typename T, bool VEC>     // NT = ceil(k / 8) groups of eight factor vectors, at most 8
-__global__ void __launch_bounds__(FG_THREADS, NT <= 4 ? 3 : 2)
+__global__ void __launch_bounds__(FG_THREADS, 1)
 factor_grad_kernel(const T* __restrict__ gsrc, int64_t ldg, int64_t n_r, int64_t n_c, int k, int t0, int k_all,
                    const uint8_t* f_codes, const uint8_t* f_sf, int f_layout, const float* f_ts,
                    const uint8_t* o_codes, const uint8_t* o_sf, int o_layout, const float* o_ts,
                    const float* __restrict__ sigma, float* __restrict__ out, float* __restrict__ ds_part) {
   // factor vectors t0 .. t0 + k - 1 of k_all (a launch handles at most 64 of them)
   extern __shared__ __align__(16) unsigned char fg_sm[];
-  __nv_bfloat16* fs = reinterpret_cast<__nv_bfloat16*>(fg_sm);                   // [2][8 NT][FG_PITCH]
+  constexpr int QB = 4 * (int)sizeof(T), STAGES = fg_stages(sizeof(T)), STAGE = FG_ROWS * FG_CHUNK * (int)sizeof(T);
+  unsigned char* ring = fg_sm;                                                   // [STAGES][FG_ROWS x FG_CHUNK of G]
+  __nv_bfloat16* fs = reinterpret_cast<__nv_bfloat16*>(fg_sm + STAGES * STAGE);  // [2][8 NT][FG_PITCH]
   float* red = reinterpret_cast<float*>(fg_sm);                                  // [FG_KW][FG_ROWS][8 NT + 1], after the loop
   constexpr int RP = 8 * NT + 1;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
@@ -418,51 +421,81 @@ factor_grad_kernel(const T* __restrict__ gsrc, int64_t ldg, int64_t n_r, int64_t
   uint32_t rank, csize;
   asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
   asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(csize));
-  const int64_t strip = blockIdx.x / csize, r0 = strip * FG_ROWS + 32 * mw;
+  const int64_t strip = blockIdx.x / csize;
   const int chunks = (int)((n_c + FG_CHUNK - 1) / FG_CHUNK), per = (chunks + (int)csize - 1) / (int)csize;
   const int ch0 = (int)rank * per, ch1 = min(chunks, ch0 + per);
-
-  // A step is 16 values of c: slots {2q, 2q+1, 2q+8, 2q+9} of a fragment hold c = base + 4q .. 4q + 3.
-  //   TRANS = 0: one load is four values of c of row r0 + 16 i + g (+ 8)
-  //   TRANS = 1: one load is r0 + 4g .. 4g + 3 of one c; rows g / g + 8 of fragment i are r0 + 4g + 2i / + 1
-  // Offsets of the four loads at c = 0, and what one value of c adds.
-  int64_t off[4];
-  bool row_in[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int64_t r = TRANS ? r0 + 4 * g : r0 + 16 * (u >> 1) + 8 * (u & 1) + g;
-    row_in[u] = r < n_r;
-    off[u] = TRANS ? (4 * q + u) * ldg + r : r * ldg + 4 * q;
-  }
   const int64_t c_stride = TRANS ? ldg : 1;
-  auto load_step = [&](float4 (&v)[4], int64_t c0) {
-    const int64_t base = c0 * c_stride;
-    const int64_t c_left = n_c - c0 - 4 * q;             // n_c is a multiple of 16: a load is inside or outside as a whole
+
+  // A chunk lies in the ring as it lies in memory: FG_ROWS rows of 32 quads of c, or (TRANS) FG_CHUNK rows of 16 quads of r.  Quad i of
+  // row j is stored at i ^ 4 (j & 3), or i ^ SW ((j >> 2) & 3): the 128 bytes that a fragment load of eight (FP32) or sixteen lanes
+  // collects from two or four rows then lie in different banks.
+  constexpr int SW = sizeof(T) == 4 ? 2 : 4;
+  // This thread's quads: column i of rows j0, j0 + FJ, ...  (FJ is a multiple of what the swizzle looks at.)
+  constexpr int FJ = TRANS ? FG_THREADS / 16 : FG_THREADS / 32;
+  const int fj = TRANS ? tid >> 4 : tid >> 5, fi = TRANS ? tid & 15 : tid & 31;
+  const uint32_t f_dst = (uint32_t)__cvta_generic_to_shared(ring) + (uint32_t)(TRANS ? fj * 16 + (fi ^ (SW * ((fj >> 2) & 3))) : fj * 32 + (fi ^ (4 * (fj & 3)))) * QB;
+  const int64_t f_r = strip * FG_ROWS + (TRANS ? 4 * fi : fj);                   // first r of the first quad
+  const int f_rows = (int)min((int64_t)FG_ROWS, n_r - f_r), f_c = TRANS ? fj : 4 * fi;
+  auto fetch = [&](int ch) {
+    const uint32_t dst = f_dst + (uint32_t)((ch - ch0) % STAGES) * STAGE;
+    const int64_t c0 = (int64_t)ch * FG_CHUNK + f_c;
+    const T* src = gsrc + f_r * (TRANS ? 1 : ldg) + c0 * c_stride;
+    const int c_left = (int)min((int64_t)FG_CHUNK, n_c - c0);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) v[u] = fg_load4<T, VEC>(gsrc, base + off[u], row_in[u] && c_left > (TRANS ? u : 0));
+    for (int u = 0; u < FG_QUADS; ++u) {
+      const bool in = TRANS ? f_rows > 0 && FJ * u < c_left : FJ * u < f_rows && c_left > 0;
+      fg_fetch4<T, VEC>(dst + u * FJ * (TRANS ? 16 : 32) * QB, in ? src + (int64_t)(FJ * u) * ldg : gsrc, in);
+    }
+  };
+  // A step is 16 values of c: slots {2q, 2q+1, 2q+8, 2q+9} of a fragment hold c = base + 4q .. 4q + 3.
+  //   TRANS = 0: one load is four values of c of row 32 mw + 16 i + g (+ 8)
+  //   TRANS = 1: one load is rows 32 mw + 4g .. 4g + 3 of one c; rows g / g + 8 of fragment i are 4g + 2i / + 1
+  auto load_step = [&](const unsigned char* st, float4 (&v)[4], int c0) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = TRANS ? c0 + 4 * q + u : 32 * mw + 16 * (u >> 1) + 8 * (u & 1) + g;
+      const int at = TRANS ? j * 16 + ((8 * mw + g) ^ (SW * q)) : j * 32 + (((c0 >> 2) + q) ^ (4 * (j & 3)));
+      if (sizeof(T) == 4) v[u] = *reinterpret_cast<const float4*>(st + at * QB);
+      else {
+        const uint2 w = *reinterpret_cast<const uint2*>(st + at * QB);
+        v[u] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xFFFF0000u), __uint_as_float(w.y << 16), __uint_as_float(w.y & 0xFFFF0000u));
+      }
+    }
   };
   const bool wide_codes = (reinterpret_cast<uintptr_t>(f_codes) & 7u) == 0;      // n_c is a multiple of 16: every block is then aligned
-  // factor chunk ch, dequantized without the tensor scale; rows beyond k and values of c beyond n_c are zero
-  auto stage = [&](int ch, int buf) {
-    const int64_t c_base = (int64_t)ch * FG_CHUNK;
-    for (int o = tid; o < 8 * NT * (FG_CHUNK / 16); o += FG_THREADS) {
-      const int t = o / (FG_CHUNK / 16), b = o % (FG_CHUNK / 16);
-      const int64_t c = c_base + 16 * b;
-      uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+  // Factor chunk: codes and scales travel in registers for a chunk (8 NT x 8 blocks, one or two per thread) and are dequantized without the
+  // tensor scale on the way into shared memory; rows beyond k and values of c beyond n_c are zero.
+  constexpr int FB = (8 * NT * (FG_CHUNK / 16) + FG_THREADS - 1) / FG_THREADS;
+  uint2 code[FB];
+  uint32_t scale[FB];
+  auto fetch_factor = [&](int ch) {
+#pragma unroll
+    for (int u = 0; u < FB; ++u) {
+      const int o = tid + FG_THREADS * u, t = o / (FG_CHUNK / 16);
+      const int64_t c = (int64_t)ch * FG_CHUNK + 16 * (o % (FG_CHUNK / 16));
+      code[u] = make_uint2(0u, 0u); scale[u] = 0u;
       if (t < k && c < n_c) {
         const uint8_t* src = f_codes + (int64_t)(t0 + t) * (n_c / 2) + c / 2;
-        uint2 code;
-        if (wide_codes) code = *reinterpret_cast<const uint2*>(src);
-        else code = make_uint2(src[0] | (src[1] << 8) | (src[2] << 16) | ((uint32_t)src[3] << 24), src[4] | (src[5] << 8) | (src[6] << 16) | ((uint32_t)src[7] << 24));
-        // E2M1 pairs to FP16 in one conversion; the products with the block scale have six significant bits and lie
-        // between 2^-10 and 2688, so they are exact in FP16 and in BF16
-        const __half2 sc = __float2half2_rn(metis_e4m3_value(f_sf[metis_sf_offset(t0 + t, c / 16, n_c / 16, f_layout)]));
+        if (wide_codes) code[u] = *reinterpret_cast<const uint2*>(src);
+        else code[u] = make_uint2(src[0] | (src[1] << 8) | (src[2] << 16) | ((uint32_t)src[3] << 24), src[4] | (src[5] << 8) | (src[6] << 16) | ((uint32_t)src[7] << 24));
+        scale[u] = f_sf[metis_sf_offset(t0 + t, c / 16, n_c / 16, f_layout)];
+      }
+    }
+  };
+  auto store_factor = [&](int buf) {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float2 v = __half22float2(__hmul2(e2m1x2_to_half2((j < 4 ? code.x : code.y) >> (8 * (j & 3))), sc));
-          const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
-          w[j] = *reinterpret_cast<const uint32_t*>(&h);
-        }
+    for (int u = 0; u < FB; ++u) {
+      const int o = tid + FG_THREADS * u, t = o / (FG_CHUNK / 16), b = o % (FG_CHUNK / 16);
+      if (8 * NT * (FG_CHUNK / 16) % FG_THREADS != 0 && t >= 8 * NT) continue;
+      uint32_t w[8];
+      // E2M1 pairs to FP16 in one conversion; the products with the block scale have six significant bits and lie
+      // between 2^-10 and 2688, so they are exact in FP16 and in BF16
+      const __half2 sc = __float2half2_rn(metis_e4m3_value(scale[u]));
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const float2 v = __half22float2(__hmul2(e2m1x2_to_half2((j < 4 ? code[u].x : code[u].y) >> (8 * (j & 3))), sc));
+        const __nv_bfloat162 h = __floats2bfloat162_rn(v.x, v.y);
+        w[j] = *reinterpret_cast<const uint32_t*>(&h);
       }
       uint4* dst = reinterpret_cast<uint4*>(fs + (buf * 8 * NT + t) * FG_PITCH + 16 * b);
       dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
@@ -476,54 +509,60 @@ factor_grad_kernel(const T* __restrict__ gsrc, int64_t ldg, int64_t n_r, int64_t
     for (int j = 0; j < NT; ++j)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[i][j][e] = total[i][j][e] = 0.0f;
-  // two steps of G are on their way while the two before them are multiplied
-  float4 v_buf[2][2][4];
-  if (ch0 < ch1) {
-    const int64_t c_first = (int64_t)ch0 * FG_CHUNK + 64 * kw;
-    load_step(v_buf[0][0], c_first); load_step(v_buf[0][1], c_first + 16);
-    stage(ch0, 0);
+#pragma unroll
+  for (int p = 0; p < STAGES - 1; ++p) {
+    if (ch0 + p < ch1) fetch(ch0 + p);
+    asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  __syncthreads();
+  if (ch0 < ch1) {
+    fetch_factor(ch0);
+    store_factor(0);
+    if (ch0 + 1 < ch1) fetch_factor(ch0 + 1);
+  }
   for (int ch = ch0; ch < ch1; ++ch) {
     const int buf = (ch - ch0) & 1;
-    const int64_t c_w = (int64_t)ch * FG_CHUNK + 64 * kw;
+    asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+    __syncthreads();                                       // chunk ch is there; what held chunk ch - 1 may be overwritten
+    if (ch + STAGES - 1 < ch1) fetch(ch + STAGES - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (ch + 1 < ch1) store_factor(buf ^ 1);
+    if (ch + 2 < ch1) fetch_factor(ch + 2);
+    const unsigned char* st_g = ring + ((ch - ch0) % STAGES) * STAGE;
+    float4 vv[2][4];
+    load_step(st_g, vv[0], 32 * kw);
+    load_step(st_g, vv[1], 32 * kw + 16);
 #pragma unroll
-    for (int hs = 0; hs < 2; ++hs) {
-      const int64_t c_next = hs == 0 ? c_w + 32 : c_w + FG_CHUNK;               // beyond n_c the loads return zeros
-      if (hs == 0 || ch + 1 < ch1) { load_step(v_buf[hs ^ 1][0], c_next); load_step(v_buf[hs ^ 1][1], c_next + 16); }
-      if (hs == 0 && ch + 1 < ch1) stage(ch + 1, buf ^ 1);
+    for (int st = 0; st < 2; ++st) {
+      const int c_w = 32 * kw + 16 * st;
+      const float4 (&v)[4] = vv[st];
+      float ax[2][4][2];                                                         // [fragment][register][pair]
 #pragma unroll
-      for (int st = 0; st < 2; ++st) {
-        const float4 (&v)[4] = v_buf[hs][st];
-        float ax[2][4][2];                                                       // [fragment][register][pair]
+      for (int i = 0; i < 2; ++i) {
+        if (TRANS) {
+          const float* e0 = reinterpret_cast<const float*>(&v[0]) + 2 * i; const float* e1 = reinterpret_cast<const float*>(&v[1]) + 2 * i;
+          const float* e2 = reinterpret_cast<const float*>(&v[2]) + 2 * i; const float* e3 = reinterpret_cast<const float*>(&v[3]) + 2 * i;
+          ax[i][0][0] = e0[0]; ax[i][0][1] = e1[0]; ax[i][1][0] = e0[1]; ax[i][1][1] = e1[1];
+          ax[i][2][0] = e2[0]; ax[i][2][1] = e3[0]; ax[i][3][0] = e2[1]; ax[i][3][1] = e3[1];
+        } else {
+          ax[i][0][0] = v[2 * i].x; ax[i][0][1] = v[2 * i].y; ax[i][1][0] = v[2 * i + 1].x; ax[i][1][1] = v[2 * i + 1].y;
+          ax[i][2][0] = v[2 * i].z; ax[i][2][1] = v[2 * i].w; ax[i][3][0] = v[2 * i + 1].z; ax[i][3][1] = v[2 * i + 1].w;
+        }
+      }
+      uint32_t bf[NT][2];
+#pragma unroll
+      for (int j = 0; j < NT; ++j) {
+        const uint2 w = *reinterpret_cast<const uint2*>(fs + (buf * 8 * NT + 8 * j + g) * FG_PITCH + c_w + 4 * q);
+        bf[j][0] = w.x; bf[j][1] = w.y;
+      }
+#pragma unroll
+      for (int term = 0; term < (sizeof(T) == 4 ? 3 : 1); ++term) {
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-          if (TRANS) {
-            const float* e0 = reinterpret_cast<const float*>(&v[0]) + 2 * i; const float* e1 = reinterpret_cast<const float*>(&v[1]) + 2 * i;
-            const float* e2 = reinterpret_cast<const float*>(&v[2]) + 2 * i; const float* e3 = reinterpret_cast<const float*>(&v[3]) + 2 * i;
-            ax[i][0][0] = e0[0]; ax[i][0][1] = e1[0]; ax[i][1][0] = e0[1]; ax[i][1][1] = e1[1];
-            ax[i][2][0] = e2[0]; ax[i][2][1] = e3[0]; ax[i][3][0] = e2[1]; ax[i][3][1] = e3[1];
-          } else {
-            ax[i][0][0] = v[2 * i].x; ax[i][0][1] = v[2 * i].y; ax[i][1][0] = v[2 * i + 1].x; ax[i][1][1] = v[2 * i + 1].y;
-            ax[i][2][0] = v[2 * i].z; ax[i][2][1] = v[2 * i].w; ax[i][3][0] = v[2 * i + 1].z; ax[i][3][1] = v[2 * i + 1].w;
-          }
-        }
-        uint32_t bf[NT][2];
+          uint32_t a[4];
 #pragma unroll
-        for (int j = 0; j < NT; ++j) {
-          const uint2 w = *reinterpret_cast<const uint2*>(fs + (buf * 8 * NT + 8 * j + g) * FG_PITCH + 64 * kw + 32 * hs + 16 * st + 4 * q);
-          bf[j][0] = w.x; bf[j][1] = w.y;
-        }
+          for (int e = 0; e < 4; ++e) a[e] = take_bf16x2(ax[i][e][0], ax[i][e][1]);
 #pragma unroll
-        for (int term = 0; term < (sizeof(T) == 4 ? 3 : 1); ++term) {
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            uint32_t a[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) a[e] = take_bf16x2(ax[i][e][0], ax[i][e][1]);
-#pragma unroll
-            for (int j = 0; j < NT; ++j) mma_16816(acc[i][j], a, bf[j][0], bf[j][1]);
-          }
+          for (int j = 0; j < NT; ++j) mma_16816(acc[i][j], a, bf[j][0], bf[j][1]);
         }
       }
     }
@@ -533,9 +572,10 @@ factor_grad_kernel(const T* __restrict__ gsrc, int64_t ldg, int64_t n_r, int64_t
       for (int j = 0; j < NT; ++j)
 #pragma unroll
         for (int e = 0; e < 4; ++e) { total[i][j][e] += acc[i][j][e]; acc[i][j][e] = 0.0f; }
-    __syncthreads();
   }
-  // ---- sums of the halves, then of the cluster's CTAs ----
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  __syncthreads();                                         // the ring has been read
+  // ---- sums of the quarters of a chunk, then of the cluster's CTAs ----
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -602,13 +642,13 @@ factor_grad_sigma_kernel(const float* __restrict__ part, int n_part, int k, floa
 template <int NT, bool TRANS, typename T, bool VEC>
 metis_status_t launch_factor_grad_nt(cudaStream_t s, const T* g, int64_t ldg, int64_t n_r, int64_t n_c, int kg, int t0, int k, const metis_nvfp4_t* f,
                                      const metis_nvfp4_t* o, const float* sigma, float* out, float* ds_part) {
-  // CTAs of a cluster divide the contraction until the grid holds the chip's resident CTAs (a strip's work is the whole
-  // contraction: without the split 64 strips of a 4096-wide operand would leave more than half of the SMs idle)
+  // CTAs of a cluster divide the contraction until three quarters of the SMs have one (a strip's work is the whole contraction; an SM
+  // alone fetches about twice its share of the memory's bandwidth, so that a partly filled wave costs little)
   const int64_t strips = metis_ceil_div(n_r, FG_ROWS), chunks = metis_ceil_div(n_c, FG_CHUNK);
   unsigned csize = 1;
-  while (csize < 8 && strips * csize < 3 * 148 && 2 * csize <= chunks) csize *= 2;
+  while (csize < 8 && strips * csize < 111 && 2 * csize <= chunks) csize *= 2;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(strips * csize)); cfg.blockDim = dim3(FG_THREADS); cfg.dynamicSmemBytes = (size_t)fg_smem(NT); cfg.stream = s;
+  cfg.gridDim = dim3((unsigned)(strips * csize)); cfg.blockDim = dim3(FG_THREADS); cfg.dynamicSmemBytes = (size_t)fg_smem(NT, sizeof(T)); cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = csize; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
@@ -815,7 +855,7 @@ metis_status_t split_gemm(metis_context* ctx, const Side& a, const Side& b, void
 
 metis_status_t metis_linear_set_attrs() {
   METIS_CUDA_TRY(cudaFuncSetAttribute(rank_update_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(float) * 2 * 128 * 68)));
-#define METIS_FG_ATTR(NT, TR, T, V) METIS_CUDA_TRY(cudaFuncSetAttribute(factor_grad_kernel<NT, TR, T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, fg_smem(NT)))
+#define METIS_FG_ATTR(NT, TR, T, V) METIS_CUDA_TRY(cudaFuncSetAttribute(factor_grad_kernel<NT, TR, T, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, fg_smem(NT, sizeof(T))))
 #define METIS_FG_ATTRS(NT) \
   METIS_FG_ATTR(NT, false, float, true); METIS_FG_ATTR(NT, false, float, false); METIS_FG_ATTR(NT, true, float, true); METIS_FG_ATTR(NT, true, float, false); \
   METIS_FG_ATTR(NT, false, __nv_bfloat16, true); METIS_FG_ATTR(NT, false, __nv_bfloat16, false); METIS_FG_ATTR(NT, true, __nv_bfloat16, true); \

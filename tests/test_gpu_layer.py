@@ -183,6 +183,16 @@ def test_factor_gradient_strips_and_chunks(ctx, l, n, m, k, dtype, pad):
     assert rel_fro(fg[1].cpu().numpy(), np.einsum("jt,ji,it->t", lq, dwn, rq)) < 1e-5
 
 
+@pytest.mark.parametrize("l,n,m,k,dtype,pad", [
+    (64, 64, 9280, 8, torch.float32, 0),           # ten chunks per CTA, the last one half: the ring goes round twice
+    (64, 9280, 128, 24, torch.bfloat16, 0),
+    (64, 192, 9280, 48, torch.float32, 2),
+])
+def test_factor_gradients_of_a_long_contraction(ctx, l, n, m, k, dtype, pad):
+    """More chunks per CTA than the ring holds, in both directions; the bounds of the test above."""
+    test_factor_gradient_strips_and_chunks(ctx, l, n, m, k, dtype, pad)
+
+
 @pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
 @pytest.mark.parametrize("peak", [3.4e38, 1e39])
 def test_factor_gradients_of_an_overflowing_weight_gradient(ctx, dtype, peak):
