@@ -73,35 +73,38 @@ __device__ __forceinline__ uint32_t e2m1x8_rne(float a0, float a1, float a2, flo
   return w;
 }
 
-// What a 16-bit draw u contributes to the rounding of its element: (65535 - u) * 256 + 255, one byte permutation of the
-// COMPLEMENTED Philox word that holds the draw in its low (hi = false) or high half.
-__device__ __forceinline__ uint32_t sr_addend(uint32_t not_word, bool hi) { return __byte_perm(not_word, 0xFFu, hi ? 0x5324u : 0x5104u); }
+// What a 16-bit draw u contributes to the rounding of its element: 256 u - 2^24, one byte permutation of the Philox word that holds
+// the draw in its low (hi = false) or high half.
+constexpr uint32_t SR_SEL_LO = 0x4105u, SR_SEL_HI = 0x4325u;                    // byte selectors, against 0xFF
+__device__ __forceinline__ uint32_t sr_term(uint32_t word, bool hi) { return __byte_perm(word, 0xFFu, hi ? SR_SEL_HI : SR_SEL_LO); }
 
-// Eight stochastically rounded codes in one word; add[i] = sr_addend of draw i.  The same decision as metis_e2m1_sr,
+// Eight stochastically rounded codes in one word; term[i] = sr_term of draw i.  The same decision as metis_e2m1_sr,
 // arranged for the instruction mix of the SM (integer logic, shifts and compares issue at half the FP32 / IMAD rate, and bound
 // this code):
 //   b = max(a, RU(a/2 + 1/2)) maps a < 1 onto [1/2, 1] (the E2M1 grid {0, 1/2, 1} becomes {1/2, 3/4, 1}: one
 //       mantissa bit per binade like the values from 1 up) and leaves a >= 1 alone, without a select;
-//   4 bits(b) + add: the 22 mantissa bits below the grid bit carry into it exactly when  frac * 65536 > u  (4 frac22 + (65535 - u) 256 +
-//       255 >= 2^24  <=>  frac22 > 64 u): comparison, selection and increment in one multiply-add;
-//   the magnitude code is then bits 24 .. 26, minus 4 modulo 8: the top bytes of four elements are gathered by byte permutations, the
-//       two words of even and odd elements are merged and the eight "- 4" taken off together;
+//   with S = 4 bits(b) + (65535 - u) 256 + 255 the 22 mantissa bits below the grid bit carry into it exactly when  frac * 65536 > u
+//       (4 frac22 + (65535 - u) 256 + 255 >= 2^24  <=>  frac22 > 64 u): comparison, selection and increment in one multiply-add.  What is
+//       formed is the complement, ~S = term - 4 bits(b): the draw then enters as it is (complementing the Philox words first
+//       cost half an instruction per element);
+//   the magnitude code is bits 24 .. 26 of S, minus 4 modulo 8: the top bytes of four elements are gathered by byte permutations, the
+//       two words of even and odd elements are merged and the complement and the eight "- 4" taken off together;
 //   the sign nibbles are gathered with one funnel shift per element and masked once per word.
 // (Against a compare per element with the draw shifted up and codes packed one by one: residual_tc_kernel 236 -> 204 us at 8192 x 14336, k = 32, the
 // minimum per element below included; quantize_kernel 472 -> 371 us at 16384 x 14336 with both orientations, its third CTA per SM
-// included.)
-__device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_t (&add)[8]) {
+// included; 340 us with the complement formed here, the scale byte without branches and one block of code per loop.)
+__device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_t (&term)[8]) {
   uint32_t s[8], sgn = 0u;
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
     const float a = fabsf(y[i]);                           // at most 6 (the caller has seen to it)
-    s[i] = __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f))) * 4u + add[i];
+    s[i] = term[i] - __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f))) * 4u;
     sgn = __funnelshift_l(__float_as_uint(y[i]), sgn, 4);  // top nibble of y (sign and three exponent bits) shifted in
   }
   const uint32_t even = __byte_perm(__byte_perm(s[0], s[2], 0x0073u), __byte_perm(s[4], s[6], 0x7300u), 0x7610u);
   const uint32_t odd = __byte_perm(__byte_perm(s[1], s[3], 0x0073u), __byte_perm(s[5], s[7], 0x7300u), 0x7610u);
   const uint32_t mag = ((even & 0x0F0F0F0Fu) | ((odd * 16u) & 0xF0F0F0F0u));
-  return ((mag & 0x77777777u) ^ 0x44444444u) | (sgn & 0x88888888u);
+  return ((mag & 0x77777777u) ^ 0x33333333u) | (sgn & 0x88888888u);
 }
 
 // largest magnitude of a block: eight three-input maxima, which pass a NaN over or (KEEP_NAN) on
@@ -121,13 +124,18 @@ __device__ __forceinline__ float amax16(const float (&v)[16]) {
   return max3<KEEP_NAN>(lo, hi, hi);
 }
 
+// the byte of metis_e4m3_ceil without its branches: 0 for zero and a NaN
+__device__ __forceinline__ uint32_t e4m3_ceil_byte(float t) {
+  const uint32_t normal = ((__float_as_uint(t) + 0xFFFFFu) >> 20) - (120u << 3), subnormal = __float2uint_ru(__fmul_rn(t, 512.0f));
+  return t > 0.015625f ? normal : subnormal;
+}
+
 // encode_block with the multiplier looked up in a table filled by fill_r_table (same bytes as encode_block).
-// add[i] = sr_addend of draw i (only read with stochastic rounding).
-__device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&add)[16], bool sr, float six_s_T,
+// term[i] = sr_term of draw i (only read with stochastic rounding).
+__device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&term)[16], bool sr, float six_s_T,
                                                      const float* r_tab, uint32_t (&packed)[2]) {
-  float sb_unused;
   if (!sr) {
-    const uint32_t byte = metis_e4m3_ceil(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f), &sb_unused);
+    const uint32_t byte = e4m3_ceil_byte(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f));
     const float r = r_tab[byte];
     packed[0] = e2m1x8_rne(__fmul_rn(v[0], r), __fmul_rn(v[1], r), __fmul_rn(v[2], r), __fmul_rn(v[3], r),
                            __fmul_rn(v[4], r), __fmul_rn(v[5], r), __fmul_rn(v[6], r), __fmul_rn(v[7], r));
@@ -138,9 +146,9 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
   float y0[8], y1[8];
   uint32_t t0[8], t1[8];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) { t0[i] = add[i]; t1[i] = add[8 + i]; }
+  for (int i = 0; i < 8; ++i) { t0[i] = term[i]; t1[i] = term[8 + i]; }
   const float amax = amax16<true>(v);
-  uint32_t byte = metis_e4m3_ceil(fminf(__fdiv_rn(amax, six_s_T), 448.0f), &sb_unused);
+  uint32_t byte = e4m3_ceil_byte(fminf(__fdiv_rn(amax, six_s_T), 448.0f));
   float r = r_tab[byte];
   // values beyond 6 saturate, and a NaN is stored as 6.  They only occur where the block scale itself is saturated, the product
   // of the block maximum rounds up, or an element is a NaN, and the block maximum shows it, so the other blocks are spared a
@@ -150,7 +158,7 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
     for (int i = 0; i < 8; ++i) { y0[i] = __fmul_rn(v[i], r); y1[i] = __fmul_rn(v[8 + i], r); }
   } else {
     if (isnan(amax)) {
-      byte = metis_e4m3_ceil(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f), &sb_unused);
+      byte = e4m3_ceil_byte(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f));
       r = r_tab[byte];
     }
 #pragma unroll

@@ -51,6 +51,11 @@ amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, 
   }
 }
 
+// two draws in a word: those of elements e and e + step
+__device__ __noinline__ uint32_t draw_pair(uint64_t e, uint64_t step, uint64_t seed, uint32_t stream) {
+  return metis_draw_u16(e, seed, stream) | (metis_draw_u16(e + step, seed, stream) << 16);
+}
+
 // Stand-alone quantizer, 128 x 128 elements per CTA.
 //  pass 1  every thread loads 16 consecutive elements of a row (32 bytes of BF16) - exactly one block along the
 //          columns - and, if that orientation is wanted, encodes it in registers and writes its 8 code bytes
@@ -83,7 +88,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
   uint8_t* sfc = codes_s + TILE * QK_CP;
   uint8_t* sfr = sfc;
   float* r_tab = reinterpret_cast<float*>(sfc + TILE * 8);                     // multiplier per scale byte
-  uint16_t* rnd = reinterpret_cast<uint16_t*>(r_tab + R_TABLE);                // [TILE][TILE] complemented draws (SR only)
+  uint16_t* rnd = reinterpret_cast<uint16_t*>(r_tab + R_TABLE);                // [TILE][TILE] draws (SR only)
 
   auto staged_row = [](int c) { return sizeof(T) == 2 ? (c >> 1) + 64 * (c & 1) : c; };
   // Scale bytes of the tile, from their staging area [stored row][8] to global memory.  The four blocks of a 64-element
@@ -128,46 +133,54 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
   const bool wide_ld = sizeof(T) == 2 && (ld & 15) == 0 && (reinterpret_cast<uintptr_t>(x) & 31) == 0;   // 32-byte aligned blocks
 
   // ---- pass 1 ----
-  // all global loads of the tile are issued before the first block is encoded: 128 bytes per thread in flight
-  uint4 raw[sizeof(T) == 2 ? 8 : 1];
-  if (sizeof(T) == 2) {
-#pragma unroll
-    for (int it = 0; it < 4; ++it) {
-      const int b = tid & 7, r = (tid >> 3) + 32 * it;
-      raw[2 * it] = raw[2 * it + 1] = make_uint4(0u, 0u, 0u, 0u);
-      if (r < vrows && b * 16 < vcols) {
-        const uint4* src = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(x) + (row0 + r) * ld + col0 + b * 16);
-        if (wide_ld) {                                     // one 32-byte load per block: consecutive lanes, consecutive 32 bytes
-          asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                       : "=r"(raw[2 * it].x), "=r"(raw[2 * it].y), "=r"(raw[2 * it].z), "=r"(raw[2 * it].w),
-                         "=r"(raw[2 * it + 1].x), "=r"(raw[2 * it + 1].y), "=r"(raw[2 * it + 1].z), "=r"(raw[2 * it + 1].w)
-                       : "l"(src));
-        } else {
-          raw[2 * it] = src[0]; raw[2 * it + 1] = src[1];
-        }
+  // BF16, round to nearest: all global loads of the tile are issued before the first block is encoded, 128 bytes per thread in flight.
+  // BF16, stochastic: bound by instructions, a block ahead is enough, and a loop of one block instead of four side by side keeps the code in
+  // the instruction cache (0.8 of 4.6 stall cycles per instruction were fetches)
+  constexpr int AHEAD = SR ? 1 : 4;
+  uint4 raw[sizeof(T) == 2 ? 2 * AHEAD : 1];
+  const int b = tid & 7, r0 = tid >> 3;                    // this thread's blocks: (r0 + 32 it, b)
+  const T* src0 = x + (row0 + r0) * ld + col0 + b * 16;
+  auto load_bf16 = [&](int it) {
+    uint4& lo = raw[sizeof(T) == 2 ? 2 * (it % AHEAD) : 0];
+    uint4& hi = raw[sizeof(T) == 2 ? 2 * (it % AHEAD) + 1 : 0];
+    lo = hi = make_uint4(0u, 0u, 0u, 0u);
+    if (r0 + 32 * it < vrows && b * 16 < vcols) {
+      const uint4* src = reinterpret_cast<const uint4*>(src0 + (int64_t)(32 * it) * ld);
+      if (wide_ld) {                                       // one 32-byte load per block: consecutive lanes, consecutive 32 bytes
+        asm volatile("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(lo.x), "=r"(lo.y), "=r"(lo.z), "=r"(lo.w), "=r"(hi.x), "=r"(hi.y), "=r"(hi.z), "=r"(hi.w)
+                     : "l"(src));
+      } else {
+        lo = src[0]; hi = src[1];
       }
     }
+  };
+  if (sizeof(T) == 2) {
+#pragma unroll
+    for (int it = 0; it < AHEAD; ++it) load_bf16(it);
   }
   // FP32: the block of the next round is loaded while this round's is encoded
   float4 nxt[sizeof(T) == 4 ? 4 : 1];
   auto load_fp32 = [&](int it) {
-    const int b = tid & 7, r = (tid >> 3) + 32 * it;
-    const bool in = r < vrows && b * 16 < vcols;
-    const float4* src = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(x) + (row0 + r) * ld + col0 + b * 16);
+    const bool in = r0 + 32 * it < vrows && b * 16 < vcols;
+    const float4* src = reinterpret_cast<const float4*>(src0 + (int64_t)(32 * it) * ld);
 #pragma unroll
     for (int j = 0; j < 4; ++j) nxt[sizeof(T) == 4 ? j : 0] = in ? src[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   };
   if (sizeof(T) == 4) load_fp32(0);
   __syncthreads();                                         // multiplier table complete (the tile loads are in flight)
-#pragma unroll
+  const int64_t gc = col0 + b * 16;
+  int64_t code_at = (row0 + r0) * (p.cols / 2) + gc / 2;   // of the block's codes; the next block is 32 rows on
+  uint64_t draw_at = ((uint64_t)(row0 + r0) * (uint64_t)p.e_stride_r + (uint64_t)gc) >> 3;
+#pragma unroll (SR ? 1 : 4)
   for (int it = 0; it < 4; ++it) {
-    const int b = tid & 7, r = (tid >> 3) + 32 * it;
-    const int64_t gr = row0 + r, gc = col0 + b * 16;
+    const int r = r0 + 32 * it;
     const bool in = r < vrows && b * 16 < vcols;
     float v[16];
     uint32_t u[16];
     if (sizeof(T) == 2) {
-      const uint4 q0 = raw[sizeof(T) == 2 ? 2 * it : 0], q1 = raw[sizeof(T) == 2 ? 2 * it + 1 : 0];
+      const uint4 q0 = raw[sizeof(T) == 2 ? 2 * (it % AHEAD) : 0], q1 = raw[sizeof(T) == 2 ? 2 * (it % AHEAD) + 1 : 0];
+      if (SR && it < 3) load_bf16(it + 1);
       const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
       for (int j = 0; j < 8; ++j) { v[2 * j] = __uint_as_float(w[j] << 16); v[2 * j + 1] = __uint_as_float(w[j] & 0xFFFF0000u); }
@@ -188,25 +201,18 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       }
     }
     if (sr) {
-      uint32_t nw[8];                                      // complemented draws, two per word
-      if (fast_draws && in) {
-        const uint64_t e = (uint64_t)gr * (uint64_t)p.e_stride_r + (uint64_t)gc;
-        const uint4 w0 = metis_philox_block_keys(e >> 3, p.keys, p.stream_id), w1 = metis_philox_block_keys((e >> 3) + 1, p.keys, p.stream_id);
-        const uint32_t ww[8] = {~w0.x, ~w0.y, ~w0.z, ~w0.w, ~w1.x, ~w1.y, ~w1.z, ~w1.w};
-#pragma unroll
-        for (int j = 0; j < 8; ++j) nw[j] = ww[j];
+      uint32_t nw[8];                                      // draws, two per word
+      if (fast_draws) {
+        const uint4 w0 = metis_philox_block_keys(draw_at, p.keys, p.stream_id), w1 = metis_philox_block_keys(draw_at + 1, p.keys, p.stream_id);
+        nw[0] = w0.x; nw[1] = w0.y; nw[2] = w0.z; nw[3] = w0.w; nw[4] = w1.x; nw[5] = w1.y; nw[6] = w1.z; nw[7] = w1.w;
       } else {
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          uint32_t d[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h)
-            d[h] = in ? metis_draw_u16((uint64_t)gr * (uint64_t)p.e_stride_r + (uint64_t)(gc + 2 * j + h) * (uint64_t)p.e_stride_c, p.seed, p.stream_id) : 0u;
-          nw[j] = ~(d[0] | (d[1] << 16));
-        }
+        for (int j = 0; j < 8; ++j)
+          nw[j] = draw_pair((uint64_t)(row0 + r) * (uint64_t)p.e_stride_r + (uint64_t)(gc + 2 * j) * (uint64_t)p.e_stride_c, (uint64_t)p.e_stride_c, p.seed, p.stream_id);
       }
+      draw_at += 4 * (uint64_t)p.e_stride_r;               // 32 rows, eight draws to a Philox block
 #pragma unroll
-      for (int j = 0; j < 8; ++j) { u[2 * j] = sr_addend(nw[j], false); u[2 * j + 1] = sr_addend(nw[j], true); }
+      for (int j = 0; j < 8; ++j) { u[2 * j] = sr_term(nw[j], false); u[2 * j + 1] = sr_term(nw[j], true); }
       if (want_r) {
         if (sizeof(T) == 2) {
           uint4* drow = reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(rnd) + r * 256);
@@ -222,7 +228,8 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
     if (want_c) {
       uint32_t packed[2];
       const uint32_t byte = encode_block_tab(v, u, sr, six_s_T, r_tab, packed);
-      if (in) METIS_DBG_GUARD(p.dbg, gr * (p.cols / 2) + gc / 2, 8, p.rows * p.cols / 2) *reinterpret_cast<uint2*>(p.c_codes + gr * (p.cols / 2) + gc / 2) = make_uint2(packed[0], packed[1]);
+      if (in) METIS_DBG_GUARD(p.dbg, code_at, 8, p.rows * p.cols / 2) *reinterpret_cast<uint2*>(p.c_codes + code_at) = make_uint2(packed[0], packed[1]);
+      code_at += 16 * p.cols;
       sfc[r * 8 + b] = in ? (uint8_t)byte : (uint8_t)0;
     }
   }
@@ -249,7 +256,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const uint32_t w = reinterpret_cast<const uint32_t*>(rnd)[(b * 16 + i) * 64 + pw];
-            u0[i] = sr_addend(w, false); u1[i] = sr_addend(w, true);
+            u0[i] = sr_term(w, false); u1[i] = sr_term(w, true);
           }
         }
         uint32_t packed[2];
@@ -270,7 +277,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       for (int i = 0; i < 16; ++i) v[i] = reinterpret_cast<const float*>(tile)[(b * 16 + i) * TP + (((c >> 2) ^ (c >> 5)) << 2 | (c & 3))];
       if (sr) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) u[i] = sr_addend((uint32_t)rnd[(b * 16 + i) * TILE + c], false);
+        for (int i = 0; i < 16; ++i) u[i] = sr_term((uint32_t)rnd[(b * 16 + i) * TILE + c], false);
       }
       uint32_t packed[2];
       const uint32_t byte = encode_block_tab(v, u, sr, six_s_T, r_tab, packed);
@@ -279,11 +286,13 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
     }
     }
     __syncthreads();
-    const int64_t kbytes = p.rows / 2;
-    for (int i = tid; i < TILE * 8; i += THREADS) {
-      const int c = i >> 3, seg = i & 7;
-      if (c < vcols && seg * 16 < vrows)
-        METIS_DBG_GUARD(p.dbg, (col0 + c) * kbytes + row0 / 2 + seg * 8, 8, p.rows * p.cols / 2) *reinterpret_cast<uint2*>(p.r_codes + (col0 + c) * kbytes + row0 / 2 + seg * 8) = *reinterpret_cast<const uint2*>(codes_s + staged_row(c) * QK_CP + seg * 8);
+    int64_t at = (col0 + r0) * (p.rows / 2) + row0 / 2 + b * 8;               // columns r0, r0 + 32, ...
+    const uint8_t* from = codes_s + staged_row(r0) * QK_CP + b * 8;
+#pragma unroll
+    for (int it = 0; it < 4; ++it) {
+      if (r0 + 32 * it < vcols && b * 16 < vrows)
+        METIS_DBG_GUARD(p.dbg, at, 8, p.rows * p.cols / 2) *reinterpret_cast<uint2*>(p.r_codes + at) = *reinterpret_cast<const uint2*>(from + (sizeof(T) == 2 ? 16 : 32) * it * QK_CP);
+      at += 16 * p.rows;
     }
     write_scales(p.r_scales, p.r_sf_bytes, p.r_layout, p.rows / 16, sfr, true, vcols, vrows, col0, row0 / 16);
   }

@@ -234,7 +234,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       if (lane == 0) { mbar_arrive(tempty_bar(acc)); mbar_arrive(xempty_bar(xb)); }
       const bool step_ok = FAST || c0 < p.cols;                                      // false: the warp's columns lie outside the matrix
       const bool blk1_ok = FAST || c0 + 16 < p.cols;
-      uint32_t nw[16];                                      // complemented draws, two per word
+      uint32_t nw[16];                                      // draws, two per word
       if (sr) {
         const uint64_t e0 = (uint64_t)row * (uint64_t)p.e_stride_r + (uint64_t)c0;        // multiple of 8
 #pragma unroll
@@ -242,7 +242,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           const uint4 w = metis_philox_block_keys((e0 >> 3) + q4, p.keys, p.stream_id);
           const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) nw[4 * q4 + j] = ~ww[j];
+          for (int j = 0; j < 4; ++j) nw[4 * q4 + j] = ww[j];
         }
       }
       if (!FAST && g.dense != nullptr && row_ok && step_ok) {
@@ -261,7 +261,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         float v0[16], v1[16];
         uint32_t u0[16], u1[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? metis_qt::sr_addend(nw[i >> 1], i & 1) : 0u; u1[i] = sr ? metis_qt::sr_addend(nw[8 + (i >> 1)], i & 1) : 0u; }
+        for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? metis_qt::sr_term(nw[i >> 1], i & 1) : 0u; u1[i] = sr ? metis_qt::sr_term(nw[8 + (i >> 1)], i & 1) : 0u; }
         const uint32_t sb0 = encode_block_tab(v0, u0, sr, six_s_T, r_tab, pk0);
         const uint32_t sb1 = encode_block_tab(v1, u1, sr, six_s_T, r_tab, pk1);
         if (!FAST && row_ok) {
@@ -286,7 +286,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         // blocks along the rows: the warp transposes its 32 x 32 values 16 columns at a time through its patch;
         // in each half lane l encodes the block of column l % 16, rows 16 * (l / 16) .. +15
         const int cb = lane & 15, rb = lane >> 4;
-        const uint32_t add_sel = (cb & 1) ? 0x5324u : 0x5104u;
+        const uint32_t term_sel = (cb & 1) ? metis_qt::SR_SEL_HI : metis_qt::SR_SEL_LO;
         const bool rb_ok = FAST || slab_row0 + 16 * rb < p.rows;
         if (FAST) {                                                          // the patch still feeds the last tile's copies until here
           if (lane == 0) bulk_wait_read_all();
@@ -313,7 +313,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             t[i] = patch[rb * PATCH_HALF + i * 20 + cb];
-            d[i] = sr ? __byte_perm(upatch[rb * 176 + i * 10 + (cb >> 1)], 0xFFu, add_sel) : 0u;   // sr_addend of this column's half
+            d[i] = sr ? __byte_perm(upatch[rb * 176 + i * 10 + (cb >> 1)], 0xFFu, term_sel) : 0u;   // sr_term of this column's half
           }
           uint32_t pk[2];
           const uint32_t sb = encode_block_tab(t, d, sr, six_s_T, r_tab, pk);
