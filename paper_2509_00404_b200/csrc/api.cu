@@ -231,7 +231,6 @@ metis_status_t metis_quantize_nvfp4(metis_handle_t h, const void* x, int32_t dty
     if (!ws || ws_bytes < 256) return METIS_ERR_WORKSPACE;
     float* amax = static_cast<float*>(ws);
     METIS_TRY(metis_launch_amax(x, dtype, rows, cols, ld, amax, s));
-    METIS_TRY(metis_launch_amax_check(h, amax, s));
     ts_src = amax;
     is_amax = 1;
   } else {
@@ -268,7 +267,7 @@ metis_status_t metis_requantize_operand(metis_handle_t h, const void* residual, 
   const int64_t rows = op->rows, cols = op->cols;
   const int k = op->k;
   if (rows <= 0 || cols <= 0 || rows % 16 || cols % 16 || k < 0 || k > 256 || ld_res < cols) return METIS_ERR_SHAPE;
-  if (!metis_aligned16(residual)) return METIS_ERR_ALIGNMENT;
+  if (!metis_aligned16(residual) || ld_res % (res_dtype == METIS_BF16 ? 8 : 4)) return METIS_ERR_ALIGNMENT;
   const bool want_c = (residual_axes & METIS_BLOCKS_ALONG_COLS) != 0, want_r = (residual_axes & METIS_BLOCKS_ALONG_ROWS) != 0;
   if (!want_c && !want_r) return METIS_ERR_INVALID_ARG;
   metis_nvfp4_t rc = op->res_by_cols, rr = op->res_by_rows;
@@ -280,6 +279,7 @@ metis_status_t metis_requantize_operand(metis_handle_t h, const void* residual, 
     if (!op->left || !op->right || !op->sigma || !lq.codes || !lq.scales || !lq.tensor_scale || !rq.codes || !rq.scales || !rq.tensor_scale)
       return METIS_ERR_INVALID_ARG;
     if ((lq.sf_layout == METIS_SF_TILED && rows % 64) || (rq.sf_layout == METIS_SF_TILED && cols % 64)) return METIS_ERR_SHAPE;
+    if (!metis_aligned16(op->left) || !metis_aligned16(op->right)) return METIS_ERR_ALIGNMENT;
     lq.rows = k; lq.k_len = rows; rq.rows = k; rq.k_len = cols;
   }
   if (!ws || ws_bytes < 256 || !metis_aligned16(ws)) return METIS_ERR_WORKSPACE;
@@ -287,9 +287,9 @@ metis_status_t metis_requantize_operand(metis_handle_t h, const void* residual, 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const float* ts_src;
   int is_amax = 0;
+  METIS_CUDA_TRY(cudaMemsetAsync(amax, 0, 3 * sizeof(float), s));
   if (res_tscale == METIS_TSCALE_AMAX_SELF) {
-    METIS_TRY(metis_launch_amax(residual, res_dtype, rows, cols, ld_res, amax, s));
-    METIS_TRY(metis_launch_amax_check(h, amax, s));
+    METIS_TRY(metis_launch_amax(residual, res_dtype, rows, cols, ld_res, amax, s, true));
     ts_src = amax; is_amax = 1;
   } else {
     ts_src = want_c ? rc.tensor_scale : rr.tensor_scale;
@@ -297,8 +297,8 @@ metis_status_t metis_requantize_operand(metis_handle_t h, const void* residual, 
   METIS_TRY(metis_launch_quantize(residual, res_dtype, rows, cols, ld_res, rounding, seed, METIS_STREAM_RESIDUAL, cols, 1, ts_src, is_amax,
                                   want_c ? &rc : nullptr, want_r ? &rr : nullptr, s, h->dev_status));
   if (k > 0) {
-    METIS_TRY(metis_launch_amax(op->left, METIS_FP32, k, rows, rows, amax + 1, s));
-    METIS_TRY(metis_launch_amax(op->right, METIS_FP32, k, cols, cols, amax + 2, s));
+    METIS_TRY(metis_launch_amax(op->left, METIS_FP32, k, rows, rows, amax + 1, s, true));
+    METIS_TRY(metis_launch_amax(op->right, METIS_FP32, k, cols, cols, amax + 2, s, true));
     METIS_TRY(metis_launch_quantize_factors(op->left, rows, op->right, cols, k, rounding, seed, amax + 1, amax + 2, &lq, &rq, s));
   }
   return METIS_OK;

@@ -249,7 +249,7 @@ __device__ __forceinline__ bool metis_dbg_ok(uint32_t* status, int64_t off, int6
 
 // ---- internal entry points shared between translation units --------------------------------
 metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* amax_out,
-                                 cudaStream_t s);
+                                 cudaStream_t s, bool zeroed = false);           // zeroed: *amax_out is zero already
 metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, int rounding,
                                      uint64_t seed, uint32_t stream_id, int64_t e_stride_r, int64_t e_stride_c,
                                      const float* tscale_src, int tscale_is_amax, const metis_nvfp4_t* by_cols,

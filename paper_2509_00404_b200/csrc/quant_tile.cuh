@@ -20,8 +20,14 @@ struct QuantParams {
   // debug build: extents of the scale buffers (the code buffers hold rows * cols / 2 bytes) and the status word
   int64_t c_sf_bytes, r_sf_bytes;
   uint32_t* dbg;
+  uint32_t* status;                   // set to METIS_DEV_NONFINITE where the tensor scale's amax is not finite (may be nullptr)
   PhiloxKeys keys;                    // round keys of `seed` (filled where the element draws are made in bulk)
 };
+
+// amax of the tensor about to be quantized is not a finite number (one thread of a launch calls)
+__device__ __forceinline__ void check_amax(const QuantParams& p, const float* amax) {
+  if (p.status != nullptr && !(fabsf(*amax) <= 3.0e38f)) atomicOr(p.status, METIS_DEV_NONFINITE);
+}
 
 // Encodes one block of 16 values; returns the scale byte, writes 8 code bytes.
 __device__ __forceinline__ uint32_t encode_block(const float (&v)[16], const uint32_t (&u)[16], bool sr, float s_T,

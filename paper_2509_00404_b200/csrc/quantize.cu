@@ -13,6 +13,8 @@ __global__ void __launch_bounds__(256)
 amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, int tpr, int narrow, uint32_t segs, uint32_t units, float* __restrict__ out) {
   // |x| as a bit pattern: non-negative floats order like their bit patterns, infinity above every number and a
   // NaN above infinity, so a non-finite element survives the reduction (fmaxf would drop a NaN)
+  metis_pdl_wait();
+  metis_pdl_trigger();                                     // the quantizer behind this kernel sets itself up meanwhile
   constexpr int UNROLL = 8;
   constexpr int E = DTYPE == METIS_BF16 ? 8 : 4;           // elements per load
   uint32_t m = 0u;
@@ -118,12 +120,14 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
     }
   };
   const int tid = threadIdx.x;
+  metis_pdl_wait();
   const int64_t row0 = (int64_t)blockIdx.y * TILE, col0 = (int64_t)blockIdx.x * TILE;
   const float s_T = tscale_is_amax ? metis_tensor_scale(*tscale_src) : *tscale_src;
   const float six_s_T = __fmul_rn(6.0f, s_T);
   if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) {
     if (ts_out0 != nullptr && ts_out0 != tscale_src) *ts_out0 = s_T;
     if (ts_out1 != nullptr && ts_out1 != tscale_src) *ts_out1 = s_T;
+    if (tscale_is_amax) check_amax(p, tscale_src);
   }
   constexpr bool sr = SR;
   fill_r_table(r_tab, s_T, tid, THREADS);
@@ -316,12 +320,12 @@ metis_status_t metis_quantize_set_attrs() {
 }
 
 metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* amax_out,
-                                 cudaStream_t s) {
+                                 cudaStream_t s, bool zeroed) {
   const bool bf = dtype == METIS_BF16;
   const int64_t e = bf ? 8 : 4;
   // the quantizer behind it wants the same of the operand: whole 16-byte loads
   if (cols % e || ld % e || !metis_aligned16(x)) return METIS_ERR_ALIGNMENT;
-  METIS_CUDA_TRY(cudaMemsetAsync(amax_out, 0, sizeof(float), s));
+  if (!zeroed) METIS_CUDA_TRY(cudaMemsetAsync(amax_out, 0, sizeof(float), s));
   if (rows * cols == 0) return METIS_OK;
   if (ld == cols) { cols = rows * cols; rows = 1; ld = cols; }                  // contiguous: one long row
   const int64_t vecs = cols / e;
@@ -333,8 +337,8 @@ metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t
   const int64_t units = groups * segs;
   if (units > 0xFFFFFFFFll) return METIS_ERR_SHAPE;
   const unsigned grid = (unsigned)(units < 148 * 8 ? units : 148 * 8);
-  if (bf) amax_kernel<METIS_BF16><<<grid, 256, 0, s>>>(x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out);
-  else amax_kernel<METIS_FP32><<<grid, 256, 0, s>>>(x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out);
+  if (bf) METIS_CUDA_TRY(metis_launch_pdl((amax_kernel<METIS_BF16>), dim3(grid), dim3(256), (size_t)0, s, x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out));
+  else METIS_CUDA_TRY(metis_launch_pdl((amax_kernel<METIS_FP32>), dim3(grid), dim3(256), (size_t)0, s, x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out));
   METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
   return METIS_OK;
@@ -396,6 +400,8 @@ __device__ __forceinline__ void rowblocks_body(const float* x, int64_t ld, const
 __global__ void __launch_bounds__(256)
 quantize_rowblocks_kernel(const float* __restrict__ x, int64_t ld, metis_qt::QuantParams p, const float* __restrict__ tscale_src,
                           int tscale_is_amax, float* ts_out) {
+  metis_pdl_wait();
+  if (tscale_is_amax && blockIdx.x == 0 && threadIdx.x == 0) metis_qt::check_amax(p, tscale_src);
   rowblocks_body(x, ld, p, tscale_src, tscale_is_amax, ts_out, nullptr, nullptr);
 }
 
@@ -499,6 +505,7 @@ metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int
                                      const float* tscale_src, int tscale_is_amax, const metis_nvfp4_t* by_cols,
                                      const metis_nvfp4_t* by_rows, cudaStream_t s, uint32_t* dbg_status) {
   using namespace metis_qt;
+  // (dbg_status: also told of an amax that is not finite)
   if (rows == 0 || cols == 0) return METIS_OK;
   // vector loads of 16 elements per thread: the rows must start on 16-byte boundaries
   if (cols % 16 || (dtype == METIS_BF16 ? ld % 8 : ld % 4)) return METIS_ERR_ALIGNMENT;
@@ -508,12 +515,11 @@ metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int
   p.keys = metis_philox_keys(seed);
   if (by_cols) { p.c_codes = by_cols->codes; p.c_scales = by_cols->scales; p.c_layout = by_cols->sf_layout; p.c_sf_bytes = (int64_t)metis_sf_bytes(rows, cols, p.c_layout); }
   if (by_rows) { p.r_codes = by_rows->codes; p.r_scales = by_rows->scales; p.r_layout = by_rows->sf_layout; p.r_sf_bytes = (int64_t)metis_sf_bytes(cols, rows, p.r_layout); }
-  p.dbg = dbg_status;
+  p.dbg = p.status = dbg_status;
   if (dtype == METIS_FP32 && by_cols && !by_rows && rows <= 64) {
     const int64_t rows_pad = p.c_layout == METIS_SF_TILED ? (rows + 127) / 128 * 128 : rows;
-    quantize_rowblocks_kernel<<<(unsigned)metis_ceil_div(rows_pad * (cols / 16), 256), 256, 0, s>>>(
-        reinterpret_cast<const float*>(x), ld, p, tscale_src, tscale_is_amax, by_cols->tensor_scale); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(cudaGetLastError());
+    METIS_CUDA_TRY(metis_launch_pdl(quantize_rowblocks_kernel, dim3((unsigned)metis_ceil_div(rows_pad * (cols / 16), 256)), dim3(256), (size_t)0, s,
+                                    reinterpret_cast<const float*>(x), ld, p, tscale_src, tscale_is_amax, by_cols->tensor_scale)); METIS_COUNT_LAUNCH();
     return METIS_OK;
   }
   const bool sr = rounding == METIS_ROUND_SR;
@@ -521,12 +527,12 @@ metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int
   float* t0 = by_cols ? by_cols->tensor_scale : nullptr; float* t1 = by_rows ? by_rows->tensor_scale : nullptr;
   if (dtype == METIS_BF16) {
     const __nv_bfloat16* xb = reinterpret_cast<const __nv_bfloat16*>(x);
-    if (sr) quantize_kernel<__nv_bfloat16, true><<<grid, THREADS, quantize_smem<__nv_bfloat16>(true), s>>>(xb, ld, p, tscale_src, tscale_is_amax, t0, t1);
-    else quantize_kernel<__nv_bfloat16, false><<<grid, THREADS, quantize_smem<__nv_bfloat16>(false), s>>>(xb, ld, p, tscale_src, tscale_is_amax, t0, t1);
+    if (sr) METIS_CUDA_TRY(metis_launch_pdl((quantize_kernel<__nv_bfloat16, true>), grid, dim3(THREADS), quantize_smem<__nv_bfloat16>(true), s, xb, ld, p, tscale_src, tscale_is_amax, t0, t1));
+    else METIS_CUDA_TRY(metis_launch_pdl((quantize_kernel<__nv_bfloat16, false>), grid, dim3(THREADS), quantize_smem<__nv_bfloat16>(false), s, xb, ld, p, tscale_src, tscale_is_amax, t0, t1));
   } else {
     const float* xf = reinterpret_cast<const float*>(x);
-    if (sr) quantize_kernel<float, true><<<grid, THREADS, quantize_smem<float>(true), s>>>(xf, ld, p, tscale_src, tscale_is_amax, t0, t1);
-    else quantize_kernel<float, false><<<grid, THREADS, quantize_smem<float>(false), s>>>(xf, ld, p, tscale_src, tscale_is_amax, t0, t1);
+    if (sr) METIS_CUDA_TRY(metis_launch_pdl((quantize_kernel<float, true>), grid, dim3(THREADS), quantize_smem<float>(true), s, xf, ld, p, tscale_src, tscale_is_amax, t0, t1));
+    else METIS_CUDA_TRY(metis_launch_pdl((quantize_kernel<float, false>), grid, dim3(THREADS), quantize_smem<float>(false), s, xf, ld, p, tscale_src, tscale_is_amax, t0, t1));
   }
   METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
