@@ -58,7 +58,7 @@ __device__ __forceinline__ void tile64_mac(const double (*as)[G64_P], const doub
 __global__ void __launch_bounds__(256)
 gram64_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t sr, int64_t sv, int64_t rows_per_part,
               double* __restrict__ part, const int* __restrict__ skip) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   if (skip != nullptr && *skip) return;
   if (blockIdx.x > blockIdx.y) return;
   __shared__ double as[G64_R][G64_P], bs[G64_R][G64_P];
@@ -361,7 +361,7 @@ constexpr size_t TW_SMEM = sizeof(double) * ((size_t)TW_ROWS * TW_HP + 3 * CW_NB
 __global__ void __launch_bounds__(256)
 trsm_wide_kernel(float* __restrict__ z, int64_t n_rows, int n, const double* __restrict__ l, const double* __restrict__ dinv,
                  const int* __restrict__ skip) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char tw_sm[];
   double (*Hs)[TW_HP] = reinterpret_cast<double (*)[TW_HP]>(tw_sm);
@@ -423,7 +423,7 @@ struct Gemm64Args {
 };
 __global__ void __launch_bounds__(256)
 gemm64_kernel(Gemm64Args g) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   if (g.skip != nullptr && *g.skip) return;
   constexpr int T = G64_T, KT = G64_R;
   __shared__ double as[KT][G64_P], bs[KT][G64_P];
@@ -472,7 +472,7 @@ gemm64_kernel(Gemm64Args g) {
 // mode 1: sign_j / sqrt(eval_j) (Rayleigh-Ritz left factor; sigma_out likewise), mode 2: sign_j
 __global__ void rot_scales_kernel(const double* __restrict__ evals, const float* __restrict__ sign, int k, int mode,
                                   double* __restrict__ scale, float* __restrict__ sigma_out) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= k) return;
   double s = 1.0;
@@ -884,7 +884,7 @@ tridiag_chol_kernel(const double* __restrict__ gm, int n, double* __restrict__ l
 constexpr int WV_WARPS = 4, WV_ROUNDS = 7;                // of the multisection: relative width 2^-29
 __global__ void __launch_bounds__(32 * WV_WARPS)
 tridiag_vectors_kernel(const double* __restrict__ tri, const double* __restrict__ v, int n, double* __restrict__ zt, double* __restrict__ panels) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   __shared__ __align__(16) double2 te[WT_MAX + 1];
   __shared__ double eo[WT_MAX + 1], dn[WV_WARPS][WT_MAX], up[WV_WARPS][WT_MAX];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
@@ -1024,7 +1024,7 @@ __host__ __device__ constexpr size_t wb_smem(int n) { return sizeof(double) * (s
 __global__ void __launch_bounds__(WB_THREADS)
 tridiag_back_kernel(const double* __restrict__ zt, const double* __restrict__ v, const double* __restrict__ panels, const double* __restrict__ l,
                     const int* __restrict__ perm, int n, double* __restrict__ x) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   extern __shared__ __align__(16) unsigned char wb_sm[];
   const int n8 = (n + 7) & ~7, P = n8 + 4;
   double* V = reinterpret_cast<double*>(wb_sm);           // [n8][P]
@@ -1113,7 +1113,7 @@ template <int OP>
 __global__ void __launch_bounds__(128)
 refine_product_kernel(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ c, const double* __restrict__ a1,
                       double* __restrict__ c1, int n, const EigState* __restrict__ st, int step) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   int last;
   if (eig_status(st, step, &last) != EIG_RUNNING) return;
   if (OP == 2 && eig_step_bad(st, step)) return;
@@ -1155,7 +1155,7 @@ refine_product_kernel(const double* __restrict__ a, const double* __restrict__ b
 // E of a step from S and G1 = X^T X, and what the status is made of
 __global__ void __launch_bounds__(256)
 refine_correction_kernel(const double* __restrict__ s, const double* __restrict__ g1, double* __restrict__ e_out, int n, EigState* __restrict__ st, int step) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   int last;
   if (eig_status(st, step, &last) != EIG_RUNNING) return;
   const int o = blockIdx.x * 256 + threadIdx.x;
@@ -1196,7 +1196,7 @@ __global__ void __launch_bounds__(1024, 1)
 eigen_finish_kernel(const double* __restrict__ x0, const double* __restrict__ x1, const double* __restrict__ s, const double* __restrict__ g1,
                     const int* __restrict__ perm, int n, const EigState* __restrict__ st, double* __restrict__ evals, double* __restrict__ evecs,
                     int* __restrict__ failed) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   __shared__ double lam[MAXQ_WIDE];
   __shared__ int order[MAXQ_WIDE];
   int last;
@@ -1434,7 +1434,7 @@ jacobi_collect_kernel(const double* __restrict__ ycm, int n, const int* __restri
 // is made positive; sign[j] records the flip for the left factor; amax|right| into *amax_out.
 __global__ void __launch_bounds__(256)
 sign_rows_kernel(float* __restrict__ right, int64_t cols, float* __restrict__ sign_out, float* __restrict__ amax_out) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   __shared__ float bv[8], bs_[8];
   __shared__ int bi[8];
   __shared__ float sg_s;
@@ -1474,7 +1474,7 @@ sign_rows_kernel(float* __restrict__ right, int64_t cols, float* __restrict__ si
 __global__ void __launch_bounds__(256)
 coef_sum_kernel(const float* __restrict__ part, int slices, int64_t rows, int gw, int j0, int kp, float* __restrict__ coef,
                 __nv_bfloat16* __restrict__ a6, int kx) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int g8 = gw / 8;
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (idx >= rows * g8) return;
@@ -1505,7 +1505,7 @@ coef_sum_kernel(const float* __restrict__ part, int slices, int64_t rows, int gw
 // gathers the sampled rows of x into a contiguous matrix: xs[j][:] = x[idx[j]][:]   (16 bytes per thread)
 __global__ void __launch_bounds__(256)
 gather_rows_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __restrict__ idx, int n_s, __nv_bfloat16* __restrict__ xs) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int64_t per_row = cols / 8;
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= (int64_t)n_s * per_row) return;

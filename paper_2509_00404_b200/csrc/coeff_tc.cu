@@ -69,6 +69,7 @@ coeff_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  metis_pdl_wait_trigger();                                 // the set-up above overlaps the kernel before this one
 
   if (warp == 0) {
     // ------------------------------- producer -------------------------------
@@ -208,8 +209,7 @@ cudaError_t set_attr() { return cudaFuncSetAttribute(coeff_tc_kernel<NB>, cudaFu
 template <int NB>
 metis_status_t launch(const CUtensorMap& mx, const CUtensorMap& mb, const CoeffArgs& g, dim3 grid, cudaStream_t s) {
   constexpr size_t smem = coeff_smem<NB>();
-  coeff_tc_kernel<NB><<<grid, NUM_THREADS, smem, s>>>(mx, mb, g); METIS_COUNT_LAUNCH();
-  METIS_CUDA_TRY(cudaGetLastError());
+  METIS_CUDA_TRY(metis_launch_pdl((coeff_tc_kernel<NB>), grid, dim3(NUM_THREADS), smem, s, mx, mb, g)); METIS_COUNT_LAUNCH();
   return METIS_OK;
 }
 

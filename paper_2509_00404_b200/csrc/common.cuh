@@ -61,6 +61,9 @@ __device__ __forceinline__ void metis_pdl_wait() { asm volatile("griddepcontrol.
 // Lets the next kernel of the stream (if it was launched with the helper below) be scheduled as soon as SMs have
 // room, before this kernel has finished; it still waits for this kernel's completion in its own metis_pdl_wait().
 __device__ __forceinline__ void metis_pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Both, at the head of a short kernel of a chain: the launch of the next kernel then overlaps this one instead of following it.
+// Kernels of one CTA that run long give the signal near their end, so that what follows does not hold SMs meanwhile.
+__device__ __forceinline__ void metis_pdl_wait_trigger() { metis_pdl_wait(); metis_pdl_trigger(); }
 
 template <typename... KArgs, typename... Args>
 static inline cudaError_t metis_launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {

@@ -51,6 +51,7 @@ struct ResidArgs {
 __global__ void __launch_bounds__(256)
 splits6_kernel(const float* __restrict__ src, int64_t n, int k, int kp, int kx, int64_t stride_i, int64_t stride_j, int pattern_b,
                __nv_bfloat16* __restrict__ out) {
+  metis_pdl_wait_trigger();
   const int groups = kx / 8;
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (idx >= n * groups) return;
@@ -119,6 +120,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  metis_pdl_wait();                                         // the set-up above overlaps the kernel before this one
 
   if (warp == 0) {
     // ------------------------------- producer -------------------------------
@@ -401,8 +403,8 @@ metis_status_t metis_launch_residual_tc(metis_context* ctx, const void* x, const
   const int kx = metis_residual_kx(kp);
   const int64_t rows = qp.rows, cols = qp.cols;
   if (coef != nullptr) {
-    splits6_kernel<<<(unsigned)metis_ceil_div(rows * (kx / 8), 256), 256, 0, s>>>(coef, rows, k, kp, kx, kp, 1, 0,
-                                                                                  reinterpret_cast<__nv_bfloat16*>(a6)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl(splits6_kernel, dim3((unsigned)metis_ceil_div(rows * (kx / 8), 256)), dim3(256), (size_t)0, s, coef, rows, k, kp, kx, kp, 1, 0,
+                                    reinterpret_cast<__nv_bfloat16*>(a6))); METIS_COUNT_LAUNCH();
   }
   CUtensorMap mx, ma, mb;
   METIS_TRY(make_map_bf16(ctx, &mx, x, rows, cols, cols, TM));
@@ -435,13 +437,12 @@ metis_status_t metis_launch_residual_tc(metis_context* ctx, const void* x, const
   const int usable = ctx->sm_count > 2 * reserve ? ctx->sm_count - reserve : ctx->sm_count;
   const int grid = (int)(tiles < usable ? tiles : usable);
   if (sr) {
-    if (fast) residual_tc_kernel<true, true><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
-    else residual_tc_kernel<true, false><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
+    if (fast) METIS_CUDA_TRY(metis_launch_pdl((residual_tc_kernel<true, true>), dim3((unsigned)grid), dim3(NUM_THREADS), SMEM_BYTES, s, mx, ma, mb, mcc, mrc, g));
+    else METIS_CUDA_TRY(metis_launch_pdl((residual_tc_kernel<true, false>), dim3((unsigned)grid), dim3(NUM_THREADS), SMEM_BYTES, s, mx, ma, mb, mcc, mrc, g));
   } else {
-    if (fast) residual_tc_kernel<false, true><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
-    else residual_tc_kernel<false, false><<<grid, NUM_THREADS, SMEM_BYTES, s>>>(mx, ma, mb, mcc, mrc, g);
+    if (fast) METIS_CUDA_TRY(metis_launch_pdl((residual_tc_kernel<false, true>), dim3((unsigned)grid), dim3(NUM_THREADS), SMEM_BYTES, s, mx, ma, mb, mcc, mrc, g));
+    else METIS_CUDA_TRY(metis_launch_pdl((residual_tc_kernel<false, false>), dim3((unsigned)grid), dim3(NUM_THREADS), SMEM_BYTES, s, mx, ma, mb, mcc, mrc, g));
   }
   METIS_COUNT_LAUNCH();
-  METIS_CUDA_TRY(cudaGetLastError());
   return METIS_OK;
 }

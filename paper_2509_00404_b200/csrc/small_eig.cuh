@@ -689,6 +689,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   }
   __syncthreads();
 
+  metis_pdl_trigger();                                  // what is left is short, or rare
   double *X = U, *Wb = W;                               // the current vectors; the next ones overwrite W
   constexpr int N_WARPS = EIG_THREADS / 32, TRI = NT8 * (NT8 + 1) / 2, TPW = (TRI + N_WARPS - 1) / N_WARPS;
   int t_i[TPW], t_j[TPW];                               // this warp's lower tiles of S and R

@@ -22,7 +22,7 @@ constexpr int LP = metis_small::PITCH;                 // row pitch of a factor 
 // The sampled rows; the first block of the one-CTA chain's call also clears what its later kernels accumulate into (a memset of
 // its own was a launch in front of every decomposition).
 __global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, int64_t rows, uint64_t seed, int full, float* __restrict__ amax, unsigned long long* __restrict__ keys) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   if (blockIdx.x == 0 && amax != nullptr && threadIdx.x < 64) {
     if (threadIdx.x < 16) amax[threadIdx.x] = 0.0f;
     keys[threadIdx.x] = 0ull;
@@ -39,7 +39,7 @@ __global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, int64_t rows,
 // Device-detected conditions of a split: amax|x| not finite (a NaN or an infinity in the operand: amax is kept as
 // an ordered bit pattern, so a NaN ranks above every number), a non-finite eigenvalue.  One warp.
 __global__ void split_status_kernel(const float* __restrict__ amax, const double* __restrict__ evals, int k, uint32_t* dev_status) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   uint32_t bits = 0u;
   if (threadIdx.x == 0 && !(fabsf(*amax) <= 3.0e38f)) bits |= METIS_DEV_NONFINITE;
   for (int j = threadIdx.x; j < k; j += 32)
@@ -48,7 +48,7 @@ __global__ void split_status_kernel(const float* __restrict__ amax, const double
 }
 
 __global__ void reduce_partials_kernel(const float* __restrict__ zp, int n_chunks, int64_t n, float* __restrict__ z) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n) return;
   float acc = 0.0f;
@@ -75,7 +75,7 @@ constexpr int GR_TPW = 6;                               // tiles per warp: 45 lo
 __global__ void __launch_bounds__(256)
 gram_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t stride_row, int64_t stride_vec,
             int64_t rows_per_part, double* __restrict__ part, const int* __restrict__ skip) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   if (skip != nullptr && *skip) return;                 // second CholeskyQR pass not needed (see chol_kernel)
   __shared__ double tile[GR_TILE][LP];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q4 = lane & 3;
@@ -169,6 +169,7 @@ chol_kernel(const double* __restrict__ g, int q, double* __restrict__ linvt_out,
   metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, 512);
   // With every pivot above 1e-8 of the largest diagonal the FP64 factorisation leaves Z L^-T orthonormal to
   // ~1e-8 already, below the FP32 rounding of its storage: the caller's second pass is then skipped.
+  metis_pdl_trigger();
   if (tid == 0 && well_conditioned != nullptr) *well_conditioned = (dmin_s > 1e-8 * gmax_s) ? 1 : 0;
   metis_small::cta_invert_lower<LP>(&L[0][0], inv_s, q, xs, LP, 512);
   for (int o = tid; o < q * q; o += 512) { const int i = o / q, j = o % q; linvt_out[o] = i <= j ? xs[j * LP + i] : 0.0; }
@@ -229,6 +230,7 @@ gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ lin
     __syncthreads();
     const double tol = 1e-13 * gmax_s;
     metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, GC_THREADS);
+    metis_pdl_trigger();
     if (pass == 0 && dmin_s > 1e-8 * gmax_s) break;
     // z_row <- z_row L^-T in shared memory by forward substitution, one warp per row, column-oriented: lane i % 32 keeps z_i; step j
     // broadcasts h_j = z_j / L[j][j] from its owner and every lane subtracts h_j L[i][j] from its own later entries
@@ -272,7 +274,7 @@ template <int KT>                                       // ceil(q / 8)
 __global__ void __launch_bounds__(256)
 orth_apply_kernel(float* __restrict__ z, int64_t n_rows, int q, const double* __restrict__ linvt, const int* __restrict__ skip,
                   __nv_bfloat16* __restrict__ hsp, int jp, int64_t ldh) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   if (skip != nullptr && *skip) return;
   constexpr int Q8 = 8 * KT, WP = Q8 + 4;
   extern __shared__ __align__(16) double oa_sm[];
@@ -332,7 +334,7 @@ template <int NJ4>                                                  // float4 gr
 __global__ void __launch_bounds__(256)
 project_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __restrict__ idx, int n_s, int q,
                const float* __restrict__ h, int rows_per_part, float* __restrict__ mp) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   __shared__ __align__(16) float hs[2][PJ_ROWS][MAXQ / 2];
   __shared__ int ids[PJ_ROWS];
   const int tid = threadIdx.x, c2 = tid & 127, jg = tid >> 7;       // jg: sketch columns 2*j + jg
@@ -414,7 +416,7 @@ __device__ __forceinline__ void split3(float x, float y, uint32_t& hi, uint32_t&
 __global__ void __launch_bounds__(128)
 basis_splits_kernel(const float* __restrict__ basis, int64_t cols, int k, int kp, __nv_bfloat16* __restrict__ bs,
                     __nv_bfloat16* __restrict__ b6, int kx) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int64_t col = (int64_t)blockIdx.x * 128 + threadIdx.x;
   if (col >= cols) return;
   if (b6 != nullptr && blockIdx.y == 0)
@@ -450,7 +452,7 @@ basis_splits_kernel(const float* __restrict__ basis, int64_t cols, int k, int kp
 __global__ void __launch_bounds__(128)
 reduce_gram_kernel(const double* __restrict__ in, int n_in, int nn, double* __restrict__ out,
                    const int* __restrict__ skip) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   if (skip != nullptr && *skip) return;
   __shared__ double part[4][32];
   const int lane = threadIdx.x & 31, sl = threadIdx.x >> 5;
@@ -478,7 +480,7 @@ template <int KP>
 __global__ void __launch_bounds__(256)
 coef_finish_kernel(const float* __restrict__ part, int slices, int64_t rows, float* __restrict__ coef,
                    double* __restrict__ gram_part, __nv_bfloat16* __restrict__ a6, int kx) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   __shared__ float cfin[32 * KP];
   const int tid = threadIdx.x;
   const int64_t row0 = (int64_t)blockIdx.x * 32;
@@ -541,7 +543,7 @@ __global__ void __launch_bounds__(256)
 sketch_mma_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __restrict__ idx, int n_s, int q,
                   uint64_t seed, const __nv_bfloat16* __restrict__ lut, float* __restrict__ zp, float* __restrict__ amax_out,
                   int ccols) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   extern __shared__ __align__(16) unsigned char smem[];
   __nv_bfloat16* om = reinterpret_cast<__nv_bfloat16*>(smem);          // [NT*8][SKM_PITCH]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
@@ -627,7 +629,7 @@ sketch_mma_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* 
 // coefficient pass.  One thread per Philox block of eight consecutive elements e = col * q + j.
 __global__ void __launch_bounds__(256)
 omega_rows_kernel(int64_t cols, int q, int nb, uint64_t seed, const __nv_bfloat16* __restrict__ lut, __nv_bfloat16* __restrict__ omt) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const uint64_t total = (uint64_t)cols * (uint64_t)q;
   const uint64_t blk = (uint64_t)blockIdx.x * 256 + threadIdx.x;
   if (blk < (total + 7) / 8) {
@@ -647,7 +649,7 @@ omega_rows_kernel(int64_t cols, int q, int nb, uint64_t seed, const __nv_bfloat1
 // m[j][col] = sum over slices s of part[s][col][j], j < q (the tensor-core projection writes M transposed, jp wide)
 __global__ void __launch_bounds__(256)
 reduce_proj_kernel(const float* __restrict__ part, int slices, int64_t cols, int jp, int q, float* __restrict__ m) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   __shared__ float t[32][33];
   const int64_t c0 = (int64_t)blockIdx.x * 32;
   const int j0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -670,7 +672,7 @@ reduce_proj_kernel(const float* __restrict__ part, int slices, int64_t cols, int
 // z[r * ldz + j] = sum over slices s of part[s][r][j], j < q (part rows are nb wide); fixed order
 __global__ void __launch_bounds__(256)
 reduce_sketch_kernel(const float* __restrict__ part, int slices, int64_t rows, int nb, int q, float* __restrict__ z, int ldz) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= rows * q) return;
   const int64_t r = i / q;
@@ -696,7 +698,7 @@ constexpr int PP_COLS = 128, PP_K = 64, PP_STAGES = 3, PP_XP = PP_COLS + 8, PP_H
 // hsp[sp][j][r] (r contiguous, ldh >= rows rounded up to 64, zero padded): three-term BF16 split of H[r][j]
 __global__ void __launch_bounds__(256)
 h_splits_kernel(const float* __restrict__ h, int n_s, int q, int jp, int ldh, __nv_bfloat16* __restrict__ hsp, int pitch_h) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int r = blockIdx.x * 256 + threadIdx.x, j = blockIdx.y;
   if (r >= ldh) return;
   const float v = (r < n_s && j < q) ? h[(int64_t)r * pitch_h + j] : 0.0f;
@@ -717,7 +719,7 @@ template <int MT>                                      // sketch columns / 16, r
 __global__ void __launch_bounds__(256)
 project_pipe_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __restrict__ idx, int n_s, int q,
                     const __nv_bfloat16* __restrict__ hsp, int ldh, int rows_per_part, float* __restrict__ mp) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   extern __shared__ __align__(16) unsigned char psm[];
   constexpr int XS_BYTES = PP_K * PP_XP * 2, HS_BYTES = 3 * MT * 16 * PP_HP * 2, STAGE = XS_BYTES + HS_BYTES;
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(psm);
@@ -879,7 +881,7 @@ __global__ void __launch_bounds__(256)
 basis_kernel(const float* __restrict__ m, int64_t cols, int q, int k, int kp, const double* __restrict__ evals, const double* __restrict__ evecs,
              float* __restrict__ basis, __nv_bfloat16* __restrict__ bs, __nv_bfloat16* __restrict__ b6, int kx,
              float* __restrict__ sigma_out, unsigned long long* __restrict__ keys, float* __restrict__ amax_out) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   extern __shared__ __align__(16) double fr_sm[];
   __shared__ double scale[FR_POS];
   double *As = fr_sm, *Ws = fr_sm + ((q + 7) / 8 * 8 < 40 ? 40 : (q + 7) / 8 * 8) * FR_P;
@@ -936,7 +938,7 @@ struct FactorsArgs {
 template <int KT>
 __global__ void __launch_bounds__(256)
 factors_kernel(FactorsArgs f, int n_right) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   extern __shared__ __align__(16) double fr_sm[];
   __shared__ double scale[FR_POS];
   double *As = fr_sm, *Ws = fr_sm + ((f.n_in + 7) / 8 * 8 < 40 ? 40 : (f.n_in + 7) / 8 * 8) * FR_P;
@@ -1487,7 +1489,7 @@ namespace {
 // contiguous BF16 copy of a strided BF16 or FP32 operand (FP32 rounded to nearest even), eight elements per thread
 __global__ void __launch_bounds__(256)
 pack_bf16_kernel(const void* __restrict__ x, int dtype, int64_t rows, int64_t cols, int64_t ld, __nv_bfloat16* __restrict__ out) {
-  metis_pdl_wait();
+  metis_pdl_wait_trigger();
   const int64_t g = (int64_t)blockIdx.x * 256 + threadIdx.x, per_row = cols / 8;
   if (g >= rows * per_row) return;
   const int64_t r = g / per_row, c = (g - r * per_row) * 8;
