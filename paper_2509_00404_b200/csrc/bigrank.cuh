@@ -6,7 +6,7 @@
 //   chol_mid_kernel          Cholesky factor of a q x q Gram matrix and the inverses of its diagonal blocks, one CTA: q up to
 //                            160, the matrix in shared memory
 //   chol_wide_kernel         the same above that: panels of 32 columns in shared memory, the matrix in L2
-//   trsm_wide_kernel         H = Z L^-T by blocked forward substitution (32 rows of Z per CTA)
+//   trsm_wide_kernel         H = Z L^-T by blocked forward substitution (32 rows of Z per CTA, FP64 tensor cores)
 //   gemm64_kernel            C = A B with FP32 A, FP64 B and FP64 accumulation, arbitrary strides (right basis,
 //                            factor rotations)
 //   tridiag_chol_kernel      up to 144: Householder reduction in one CTA's registers beside the factorisation in another's shared
@@ -66,16 +66,27 @@ gram64_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t sr, in
   const int i0 = blockIdx.y * G64_T, j0 = blockIdx.x * G64_T;
   const int64_t r_begin = (int64_t)blockIdx.z * rows_per_part, r_end = min(n_rows, r_begin + rows_per_part);
   double acc[2][4][2] = {};
+  constexpr int PER = G64_R * G64_T / 256;                // values of either operand per thread and step; the next step's are on
+  float va[PER], vb[PER];                                 // their way while this one is multiplied
+  auto fetch = [&](int64_t r0) {
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int o = tid + 256 * u, rr = sr == 1 ? o % G64_R : o / G64_T, ii = sr == 1 ? o / G64_R : o % G64_T;
+      const float* src = v + (r0 + rr) * sr;
+      va[u] = r0 + rr < r_end && i0 + ii < n ? src[(int64_t)(i0 + ii) * sv] : 0.0f;
+      vb[u] = r0 + rr < r_end && j0 + ii < n ? src[(int64_t)(j0 + ii) * sv] : 0.0f;
+    }
+  };
+  fetch(r_begin);
   for (int64_t r0 = r_begin; r0 < r_end; r0 += G64_R) {
 #pragma unroll
-    for (int o = tid; o < G64_R * G64_T; o += 256) {
-      int rr, ii;
-      if (sr == 1) { rr = o % G64_R; ii = o / G64_R; } else { ii = o % G64_T; rr = o / G64_T; }
-      const bool okr = r0 + rr < r_end;
-      as[rr][ii] = (okr && i0 + ii < n) ? (double)v[(r0 + rr) * sr + (int64_t)(i0 + ii) * sv] : 0.0;
-      bs[rr][ii] = (okr && j0 + ii < n) ? (double)v[(r0 + rr) * sr + (int64_t)(j0 + ii) * sv] : 0.0;
+    for (int u = 0; u < PER; ++u) {
+      const int o = tid + 256 * u, rr = sr == 1 ? o % G64_R : o / G64_T, ii = sr == 1 ? o / G64_R : o % G64_T;
+      as[rr][ii] = (double)va[u];
+      bs[rr][ii] = (double)vb[u];
     }
     __syncthreads();
+    if (r0 + G64_R < r_end) fetch(r0 + G64_R);
     tile64_mac(as, bs, wm, wn, g, q, acc);
     __syncthreads();
   }
@@ -354,10 +365,13 @@ chol_mid_kernel(const double* __restrict__ g, int n, double tol_rel, double* __r
 
 // H = Z L^-T by blocked forward substitution, in place: for panel J of CW_NB columns
 //   h_J = (z_J - sum_{K < J} h_K L[J][K]^T) Dinv_J^T.
-// A CTA owns 32 rows of Z and keeps their finished part of H in shared memory (FP64); L is read in CW_NB x CW_NB
-// chunks.  l, dinv: outputs of chol_wide_kernel.  FP32 in, FP64 arithmetic, FP32 out.
-constexpr int TW_ROWS = 32, TW_HP = MAXQ_WIDE + 1;
-constexpr size_t TW_SMEM = sizeof(double) * ((size_t)TW_ROWS * TW_HP + 3 * CW_NB * CW_P);
+// A CTA owns 32 rows of Z and keeps their finished part of H in shared memory (FP64).  The products run on the FP64 tensor cores, a warp
+// two 8 x 8 tiles of the panel; the factor's and the inverse's entries go from L2 into fragment registers, a panel of 32 columns ahead
+// (544 x 136 46 -> 15.5 us, 7168 x 136 61 -> 22.6 us; before: multiply-adds from shared memory, loads behind barriers).
+// l, dinv: outputs of the wide Cholesky kernels.  FP32 in, FP64 arithmetic, FP32 out.
+constexpr int TW_ROWS = 32, TW_HP = MAXQ_WIDE + 4, TW_TP = CW_NB + 4;          // pitches 4 mod 16: conflict-free fragments
+constexpr size_t TW_SMEM = sizeof(double) * TW_ROWS * (TW_HP + TW_TP);
+static_assert(CW_NB == 32 && TW_HP % 16 == 4 && TW_TP % 16 == 4, "fragment layout");
 __global__ void __launch_bounds__(256)
 trsm_wide_kernel(float* __restrict__ z, int64_t n_rows, int n, const double* __restrict__ l, const double* __restrict__ dinv,
                  const int* __restrict__ skip) {
@@ -365,45 +379,69 @@ trsm_wide_kernel(float* __restrict__ z, int64_t n_rows, int n, const double* __r
   if (skip != nullptr && *skip) return;
   extern __shared__ __align__(16) unsigned char tw_sm[];
   double (*Hs)[TW_HP] = reinterpret_cast<double (*)[TW_HP]>(tw_sm);
-  double (*Ls)[CW_P] = reinterpret_cast<double (*)[CW_P]>(tw_sm + sizeof(double) * TW_ROWS * TW_HP);
-  double (*Ds)[CW_P] = Ls + CW_NB;
-  double (*Ts)[CW_P] = Ls + 2 * CW_NB;
-  const int tid = threadIdx.x, tr = tid >> 5, tc = tid & 31;       // rows tr + 8 m, column tc of the panel
-  const int64_t r0 = (int64_t)blockIdx.x * TW_ROWS;
+  double (*Ts)[TW_TP] = reinterpret_cast<double (*)[TW_TP]>(tw_sm + sizeof(double) * TW_ROWS * TW_HP);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
+  const int row = 8 * (warp & 3) + g;                     // row of the fragments this lane holds
+  const int64_t r = (int64_t)blockIdx.x * TW_ROWS + row;
   for (int j0 = 0; j0 < n; j0 += CW_NB) {
-    const int w = min(CW_NB, n - j0);
-    double acc[4];
+    const int jt[2] = {j0 + 8 * (warp >> 2), j0 + 8 * (warp >> 2) + 16};       // first columns of the warp's tiles
+    double acc[2][2][2] = {}, f[2][8];
+    // entries of the factor (k0 < j0) or of the inverse of its diagonal block (k0 = j0) that multiply columns k0 ... k0 + 31
+    auto fetch = [&](int k0) {
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      const int64_t r = r0 + tr + 8 * m;
-      acc[m] = (r < n_rows && tc < w) ? (double)z[r * n + j0 + tc] : 0.0;
-    }
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          const int c = jt[u] + g;
+          f[u][s] = c >= n ? 0.0 : (k0 < j0 ? __ldg(l + (int64_t)c * n + k0 + 4 * s + q) : __ldg(dinv + (int64_t)(j0 / CW_NB) * CW_NB * CW_NB + (c - j0) * CW_NB + 4 * s + q));
+        }
+    };
+    fetch(0);
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int c = jt[u] + 2 * q + e;
+        acc[u][0][e] = r < n_rows && c < n ? (double)z[r * n + c] : 0.0;
+      }
     for (int k0 = 0; k0 < j0; k0 += CW_NB) {
-      __syncthreads();
-      for (int o = tid; o < CW_NB * CW_NB; o += 256) { const int c = o / CW_NB, kk = o % CW_NB; Ls[c][kk] = c < w ? l[(int64_t)(j0 + c) * n + k0 + kk] : 0.0; }
-      __syncthreads();
-#pragma unroll 8
-      for (int kk = 0; kk < CW_NB; ++kk) {
-        const double lv = Ls[tc][kk];
+      double b[2][8];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) acc[m] -= Hs[tr + 8 * m][k0 + kk] * lv;
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int s = 0; s < 8; ++s) b[u][s] = f[u][s];
+      fetch(k0 + CW_NB);
+#pragma unroll
+      for (int s = 0; s < 8; ++s) {
+        const double a = -Hs[row][k0 + 4 * s + q];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) metis_small::dmma(acc[u][s & 1], a, b[u][s]);
       }
     }
-    __syncthreads();
-    for (int o = tid; o < CW_NB * CW_NB; o += 256) Ds[o / CW_NB][o % CW_NB] = dinv[(int64_t)(j0 / CW_NB) * CW_NB * CW_NB + o];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) Ts[tr + 8 * m][tc] = acc[m];
-    __syncthreads();
+    for (int u = 0; u < 2; ++u)
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      double sacc = 0.0;
-      for (int cp = 0; cp <= tc; ++cp) sacc += Ts[tr + 8 * m][cp] * Ds[tc][cp];
-      const int64_t r = r0 + tr + 8 * m;
-      if (tc < w) {
-        Hs[tr + 8 * m][j0 + tc] = sacc;
-        if (r < n_rows) z[r * n + j0 + tc] = (float)sacc;
-      }
+      for (int e = 0; e < 2; ++e) Ts[row][jt[u] - j0 + 2 * q + e] = acc[u][0][e] + acc[u][1][e];
+    __syncthreads();
+    double h[2][2][2] = {};
+#pragma unroll
+    for (int s = 0; s < 8; ++s) {
+      const double a = Ts[row][4 * s + q];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) metis_small::dmma(h[u][s & 1], a, f[u][s]);
     }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int c = jt[u] + 2 * q + e;
+        const double v = h[u][0][e] + h[u][1][e];
+        if (c < n) {
+          Hs[row][c] = v;
+          if (r < n_rows) z[r * n + c] = (float)v;
+        }
+      }
+    __syncthreads();                                      // the panel's columns are there; Ts has been read
   }
 }
 
@@ -431,17 +469,29 @@ gemm64_kernel(Gemm64Args g) {
   const int64_t m0 = (int64_t)blockIdx.y * T;
   const int n0 = blockIdx.x * T;
   double acc[2][4][2] = {};
+  constexpr int PER = KT * T / 256;                       // values of either operand per thread and step; the next step's are on
+  float va[PER];                                          // their way while this one is multiplied
+  double vb[PER];
+  const bool a_rows = g.a_k == 1, b_cols = g.b_k == 1;
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int o = tid + 256 * u;
+      const int kk = a_rows ? o % KT : o / T, mm = a_rows ? o / KT : o % T, kb = b_cols ? o % KT : o / T, nn = b_cols ? o / KT : o % T;
+      va[u] = m0 + mm < g.M && k0 + kk < g.K ? g.a[(m0 + mm) * g.a_m + (int64_t)(k0 + kk) * g.a_k] : 0.0f;
+      vb[u] = n0 + nn < g.N && k0 + kb < g.K ? g.b[(int64_t)(k0 + kb) * g.b_k + (int64_t)(n0 + nn) * g.b_n] : 0.0;
+    }
+  };
+  fetch(0);
   for (int k0 = 0; k0 < g.K; k0 += KT) {
 #pragma unroll
-    for (int o = tid; o < KT * T; o += 256) {
-      int kk, mm;
-      if (g.a_k == 1) { kk = o % KT; mm = o / KT; } else { mm = o % T; kk = o / T; }
-      as[kk][mm] = (m0 + mm < g.M && k0 + kk < g.K) ? (double)g.a[(m0 + mm) * g.a_m + (int64_t)(k0 + kk) * g.a_k] : 0.0;
-      int kb, nn;
-      if (g.b_k == 1) { kb = o % KT; nn = o / KT; } else { nn = o % T; kb = o / T; }
-      bs[kb][nn] = (n0 + nn < g.N && k0 + kb < g.K) ? g.b[(int64_t)(k0 + kb) * g.b_k + (int64_t)(n0 + nn) * g.b_n] : 0.0;
+    for (int u = 0; u < PER; ++u) {
+      const int o = tid + 256 * u;
+      as[a_rows ? o % KT : o / T][a_rows ? o / KT : o % T] = (double)va[u];
+      bs[b_cols ? o % KT : o / T][b_cols ? o / KT : o % T] = vb[u];
     }
     __syncthreads();
+    if (k0 + KT < g.K) fetch(k0 + KT);
     tile64_mac(as, bs, wm, wn, gq, q, acc);
     __syncthreads();
   }
