@@ -733,8 +733,8 @@ jacobi_fp32_kernel(const double* __restrict__ l, int n, double* __restrict__ x) 
 // Above n = 128 the first columns, finished first, live in shared memory: five per lane do not fit the registers.
 // The sixteenth warp works out the scalars, the vectors of the update and the next column, so that a step has two barriers.  A step takes
 // 2300 cycles at n = 128, 3300 over the first quarter: the shared-memory pipe (52 cycles a warp for the factors of 36 elements a lane,
-// 24 for the exchanges) and the FP64 pipe (54) share it with the scalars' 1050; one warp per row and lane would need the
-// products summed through shared memory, five columns per lane spilled (n = 136: 309 us).
+// 24 for the exchanges) and the FP64 pipe (54) share it with the scalars' 1050 (rows along the lanes instead would
+// need the products of fifteen warps summed through shared memory; five columns per lane in registers spilled, n = 136: 309 us).
 // Outputs: v[j][.] the reflectors (zero up to column j), tri = d, e, beta (n each).
 constexpr int WT_WARPS = 15, WT_THREADS = 32 * (WT_WARPS + 1), WT_MAX = 144, WT_TAIL = 16, WT_ROWS = 3;
 static_assert(WT_MAX <= CM_MAX && WT_THREADS >= CW_THREADS, "the factorisation runs in the same launch");
