@@ -738,7 +738,16 @@ jacobi_fp32_kernel(const double* __restrict__ l, int n, double* __restrict__ x) 
 // Outputs: v[j][.] the reflectors (zero up to column j), tri = d, e, beta (n each).
 constexpr int WT_WARPS = 15, WT_THREADS = 32 * (WT_WARPS + 1), WT_MAX = 144, WT_TAIL = 16, WT_ROWS = 3;
 static_assert(WT_MAX <= CM_MAX && WT_THREADS >= CW_THREADS, "the factorisation runs in the same launch");
-template <int R, int C, bool TAIL>                        // rows per warp (15 R >= n), columns per lane (32 C + TAIL * WT_TAIL >= n)
+// An instance of R rows per warp and C columns per lane holds orders up to N_MAX.  Rows it has beyond the matrix are worked on like the
+// others (they stay zero), so what is indexed by a row has an entry for each of its WT_WARPS * R.
+template <int R, int C, bool TAIL>
+struct WtShape {
+  static constexpr int ROWS = WT_WARPS * R, COLS = 32 * C + (TAIL ? WT_TAIL : 0), N_MAX = ROWS < COLS ? ROWS : COLS;
+  static constexpr int LANE_COLS = TAIL ? C + 1 : C, PADDED = 32 * LANE_COLS;   // columns per lane of the scalars' warp, and of all its lanes
+  static constexpr int ENTRIES = ROWS > PADDED ? ROWS : PADDED;
+  static_assert(COLS <= PADDED && (!TAIL || ROWS <= WT_MAX + WT_WARPS), "columns of the vectors, rows of the tail");
+};
+template <int R, int C, bool TAIL>
 __global__ void __launch_bounds__(WT_THREADS, 1)
 tridiag_chol_kernel(const double* __restrict__ gm, int n, double* __restrict__ l_out, int* __restrict__ perm_out, EigState* __restrict__ state,
                     double* __restrict__ v_out, double* __restrict__ tri) {
@@ -748,12 +757,15 @@ tridiag_chol_kernel(const double* __restrict__ gm, int n, double* __restrict__ l
     if (tid < CW_THREADS) chol_mid(gm, n, 1e-14, l_out, nullptr, perm_out, state, nullptr);
     return;
   }
-  constexpr int CS = TAIL ? C + 1 : C, NP = 32 * CS;      // columns per lane of the scalars' warp
-  __shared__ double xs_[32 + NP], rs_[32 + NP], us_[32 + NP], ys[NP];          // the first 32 stay zero: columns below the first
-  __shared__ __align__(16) double2 pq[NP];
+  using Shape = WtShape<R, C, TAIL>;
+  constexpr int CS = Shape::LANE_COLS, NP = Shape::PADDED;
+  __shared__ double xs_[32 + NP], rs_[32 + NP], us_[32 + NP];                  // the first 32 stay zero: columns below the first
+  __shared__ double ys[Shape::ENTRIES];                   // by row, as is pq; what lies beyond the matrix stays zero
+  __shared__ __align__(16) double2 pq[Shape::ENTRIES];
   __shared__ double tail[TAIL ? WT_MAX + WT_WARPS : 1][WT_TAIL];               // columns 0 ... n - 32 C - 1
   double *xs = xs_ + 32, *rs = rs_ + 32, *us = us_ + 32;
-  for (int i = tid; i < 32 + NP; i += WT_THREADS) { xs_[i] = 0.0; rs_[i] = 0.0; us_[i] = 0.0; if (i < NP) { ys[i] = 0.0; pq[i] = make_double2(0.0, 0.0); } }
+  for (int i = tid; i < 32 + NP; i += WT_THREADS) { xs_[i] = 0.0; rs_[i] = 0.0; us_[i] = 0.0; }
+  for (int i = tid; i < Shape::ENTRIES; i += WT_THREADS) { ys[i] = 0.0; pq[i] = make_double2(0.0, 0.0); }
   int top = 0;                                            // an even power of two brings the largest entry near one
   for (int i = lane; i < n; i += 32) top = max(top, __double2hiint(gm[(int64_t)i * n + i]));
   top = __reduce_max_sync(0xFFFFFFFFu, top) >> 20;

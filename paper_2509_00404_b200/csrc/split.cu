@@ -1226,10 +1226,12 @@ metis_status_t launch_jacobi_fp32(cudaStream_t s, const double* l, int n, double
   return METIS_OK;
 }
 
-// factor and starting vectors of a matrix of up to WT_MAX: v, zt, tri are scratch of n x n and (tri: 3 n and the panels' 8 n)
-template <int R, int C, bool TAIL>
+// factor and starting vectors of a matrix of order N_FROM ... N_TO: v, zt, tri are scratch of n x n and (tri: 3 n and the panels' 8 n)
+template <int N_FROM, int N_TO, int R, int C, bool TAIL>
 metis_status_t launch_tridiag(cudaStream_t s, const double* gram1, int n, double* l, int* perm, metis_wide::EigState* st, double* v, double* zt, double* tri, double* x) {
   using namespace metis_wide;
+  static_assert(N_TO <= WtShape<R, C, TAIL>::N_MAX && N_TO <= WT_MAX, "rows and columns of the instance");
+  static_assert(N_FROM >= 32 * (TAIL ? C : C - 1), "a lane's last column is at most 32 below the first");
   double* panels = tri + 3 * n;
   const unsigned vec = (unsigned)metis_ceil_div(n, WV_WARPS), pan = (unsigned)metis_ceil_div(metis_ceil_div(n - 2, 8), WV_WARPS);
   METIS_CUDA_TRY(metis_launch_pdl((tridiag_chol_kernel<R, C, TAIL>), dim3(2), dim3(WT_THREADS), cm_smem(n), s, gram1, n, l, perm, st, v, tri)); METIS_COUNT_LAUNCH();
@@ -1247,10 +1249,10 @@ metis_status_t launch_eig_wide(cudaStream_t s, const double* gram1, int n, doubl
   EigState* st = reinterpret_cast<EigState*>(scratch + 6 * nn);
   int* failed = reinterpret_cast<int*>(st + 1);
   int* perm = failed + 1;
-  if (n <= 90) METIS_TRY((launch_tridiag<6, 3, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
-  else if (n <= 96) METIS_TRY((launch_tridiag<9, 3, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
-  else if (n <= 128) METIS_TRY((launch_tridiag<9, 4, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
-  else if (n <= WT_MAX) METIS_TRY((launch_tridiag<10, 4, true>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  if (n <= 90) METIS_TRY((launch_tridiag<MAXQ + 1, 90, 6, 3, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  else if (n <= 96) METIS_TRY((launch_tridiag<91, 96, 9, 3, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  else if (n <= 128) METIS_TRY((launch_tridiag<97, 128, 9, 4, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
+  else if (n <= WT_MAX) METIS_TRY((launch_tridiag<129, WT_MAX, 10, 4, true>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
   else METIS_TRY(launch_chol_wide(s, gram1, n, 1e-14, l, nullptr, perm, st, nullptr, nullptr));
   if (n <= WT_MAX) {}
   else if (n <= 176) METIS_TRY((launch_jacobi_fp32<8, 22>(s, l, n, x[0])));

@@ -534,3 +534,20 @@ def test_wide_eigen_solver_at_the_edges_of_the_reduction(ctx, k, p, spectrum):
     assert (core - torch.diag(torch.diagonal(core))).abs().max() < tol * sig[0]
     assert (torch.diagonal(core) - sig).abs().max() < 1e-5 * sig[0]
     assert bool((sig[:-1] >= sig[1:]).all())
+
+
+@pytest.mark.parametrize("k,p", [(84, 7), (88, 8), (96, 8), (120, 8), (128, 8)])
+def test_a_wide_split_repeats_itself(ctx, k, p):
+    """Orders (k + p and k) at which the reduction works on more rows than the matrix has: what lies beyond it is never read, so every
+    call gives the same bytes, whatever ran on the SM before."""
+    B, h = ctx
+    x, other = _planted(1536, 640, k, "geometric", k), _planted(1536, 640, k, "close", k + 1)
+    first = None
+    for i in range(6):
+        if i % 2:
+            h.split(other, 128, 8, sketch=B.SKETCH_SAMPLED, seed=3)
+        op = h.split(x, k, p, sketch=B.SKETCH_SAMPLED, seed=11)
+        got = [t.clone() for t in (op.left, op.sigma, op.right, op.left_q.codes, op.right_q.codes, op.res_by_cols.codes, op.res_by_cols.scales)]
+        if first is None:
+            first = got
+        assert all(torch.equal(a, b) for a, b in zip(first, got))

@@ -40,3 +40,44 @@ def test_tensor_copies_of_codes_are_checked_in_the_debug_build():
     for at in copies:
         statement = code[code.rfind(";", 0, at):at]
         assert re.findall(r"METIS_DBG_GUARD\([^,]*, [^,]*, (\d+), ", statement) == ["16", "32"], statement
+
+
+def _constants(text, known):
+    """Values of the `constexpr int` names that `text` declares, `known` given (conditional expressions become Python's)."""
+    out = dict(known)
+    for statement in re.findall(r"constexpr int ([^;(]*(?:\([^;]*\))?[^;]*);", text):
+        for name, expr in re.findall(r"(\w+) = ([^,]+)", statement):
+            expr = re.sub(r"\w+::", "", expr.replace("&&", " and ").replace("||", " or ")).strip()
+            expr = re.sub(r"^(.+?) \? (.+) : (.+)$", r"(\2) if (\1) else (\3)", expr.replace("(TAIL ? WT_TAIL : 0)", "(WT_TAIL if TAIL else 0)"))
+            try:
+                out[name] = int(eval(expr.replace("/", "//"), {}, out))
+            except (NameError, SyntaxError):
+                pass                                       # made of something else than integers known here
+    return out
+
+
+def test_arrays_of_the_reduction_hold_an_entry_for_every_row_of_an_instance():
+    """tridiag_chol_kernel works on WT_WARPS * R rows, whether or not they belong to the matrix, and indexes two shared arrays with
+    them.  Out of range, an access falls into a neighbouring array, which no run shows."""
+    with open(os.path.join(CSRC, "bigrank.cuh")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    with open(os.path.join(CSRC, "split.cu")) as f:
+        launches = re.sub(r"//[^\n]*", "", f.read())
+    kernel = text[text.index("tridiag_chol_kernel(const"):]
+    kernel = kernel[:kernel.index("\n}\n")]
+    shape = re.search(r"struct WtShape \{(.*?)\n\};", text, re.S)
+    for name in ("ys", "pq"):
+        assert re.findall(r"\b%s\[([^\]]*WT_WARPS[^\]]*)\]" % name, kernel)
+    instances = re.findall(r"launch_tridiag<(?:[^<>]*, )??(\d+), (\d+), (true|false)>\(s,", launches)
+    assert len(instances) == 4
+    for r, c, tail in instances:
+        known = _constants(text[text.index("constexpr int WT_WARPS"):text.index("struct WtShape" if shape else "template <int R, int C, bool TAIL>")],
+                           {"R": int(r), "C": int(c), "TAIL": tail == "true"})
+        known = _constants((shape.group(1) if shape else "") + kernel, known)
+        rows = 15 * int(r)                                 # warp + WT_WARPS * a, a < R
+        assert known["WT_WARPS"] == 15
+        for name in ("ys", "pq"):
+            extent = re.search(r"__shared__[^;]*\b%s\[([^\]]+)\]" % name, kernel).group(1)
+            assert eval(re.sub(r"\w+::", "", extent), {}, known) >= rows, (name, r, c, tail)
+        if tail == "true":
+            assert rows <= known["WT_MAX"] + known["WT_WARPS"]                 # rows of `tail`
