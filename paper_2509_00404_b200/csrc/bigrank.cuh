@@ -1091,7 +1091,8 @@ tridiag_back_kernel(const double* __restrict__ zt, const double* __restrict__ v,
   const int n8 = (n + 7) & ~7, P = n8 + 4;
   double* V = reinterpret_cast<double*>(wb_sm);           // [n8][P]
   double* Z = V + (size_t)n8 * P;                         // [n8][WB_ZP]: eight vectors as columns
-  __shared__ double Ts[8 * WT_MAX], part[WB_WARPS][64], patch[64];
+  __shared__ double Ts[8 * WT_MAX];
+  __shared__ __align__(16) double part[WB_WARPS][64], patch[64];               // stored in pairs
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3, e0 = 8 * (int)blockIdx.x;
   const int n_panels = (n - 2 + 7) / 8;
   constexpr int CT = (WT_MAX + 31) / 32;

@@ -293,7 +293,7 @@ lowrank_bf16_kernel(int64_t M, int64_t N, int ka, int kb, int kx, const float* _
 __global__ void __launch_bounds__(256)
 rank_update_kernel(const float* __restrict__ y0, int64_t M, int64_t N, int kc, const float* __restrict__ lcat,
                    const float* __restrict__ rcat, void* __restrict__ out, int out_dtype, int64_t ldo) {
-  extern __shared__ float sm[];
+  extern __shared__ __align__(16) float sm[];
   float* ls = sm;                       // [kc][64 + 4]
   float* rs = sm + kc * 68;
   const int tid = threadIdx.x;

@@ -81,3 +81,32 @@ def test_arrays_of_the_reduction_hold_an_entry_for_every_row_of_an_instance():
             assert eval(re.sub(r"\w+::", "", extent), {}, known) >= rows, (name, r, c, tail)
         if tail == "true":
             assert rows <= known["WT_MAX"] + known["WT_WARPS"]                 # rows of `tail`
+
+
+def test_shared_arrays_accessed_in_vectors_are_declared_aligned():
+    """A 16- (8-) byte access to a shared array of smaller elements needs the declaration to say so: without it the array lies where
+    the others leave room."""
+    size = {"double2": 16, "float4": 16, "uint4": 16, "int4": 16, "float2": 8, "uint2": 8, "int2": 8}
+    wanted, found = 0, []
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        with open(path) as f:
+            text = re.sub(r"//[^\n]*", "", f.read())
+        for kernel in re.split(r"\b__global__\b", text)[1:]:
+            align = {"smem_raw": 1024} if "(raw + 1023u) & ~1023u" in kernel else {}   # rounded up by the kernel itself
+            for decl in re.findall(r"__shared__[^;]*;", kernel):
+                a = re.search(r"__align__\((\d+)\)", decl)
+                base = 8 if re.search(r"\b(double|float2|uint2|uint64_t)\b", decl) else (16 if re.search(r"\b(double2|float4|uint4)\b", decl) else 4)
+                for name in re.findall(r"\b(\w+)\[", decl):
+                    align.setdefault(name, max(base, int(a.group(1)) if a else 0))
+            source = dict(re.findall(r"\*\s*(?:__restrict__ )?(\w+) = (?:reinterpret_cast<[^;=]*>\()?&?(\w+)\b(?![(])", kernel))
+            for type_, name in re.findall(r"reinterpret_cast<(?:const )?(\w+)\s*\*>\(\s*&?(\w+)", kernel):
+                for _ in range(4):
+                    if name in align or name not in source:
+                        break
+                    name = source[name]
+                if type_ in size and name in align:
+                    wanted += 1
+                    if align[name] < size[type_]:
+                        found.append((os.path.basename(path), type_, name))
+    assert wanted >= 10
+    assert found == []
