@@ -150,6 +150,10 @@ metis_status_t metis_debug_wait_timeout(metis_handle_t h, uint32_t polls, uint32
 int32_t metis_debug_build(void);
 metis_status_t metis_debug_index_check(metis_handle_t h, int64_t offset, int64_t nbytes, int64_t extent, metis_stream_t stream);
 
+/* Test hook: rcp[i] and rsqrt[i] (device, n values each) are the FP64 reciprocal and reciprocal square root of x[i] as the dense kernels of
+ * a decomposition form them (Newton-Raphson; for normal values whose results are normal). */
+metis_status_t metis_debug_reciprocals(metis_handle_t h, const double* x, int64_t n, double* rcp, double* rsqrt, metis_stream_t stream);
+
 /* Test / benchmark hook: kernels launched by the library in this process so far (host counter, atomic). */
 uint64_t metis_debug_launch_count(void);
 

@@ -27,6 +27,7 @@ STATUS_NAMES = {0: "OK", 1: "INVALID_ARG", 2: "SHAPE", 3: "ALIGNMENT", 4: "WORKS
 
 EXPORTED = ["metis_create", "metis_destroy", "metis_last_device_status", "metis_debug_quantile_table",
             "metis_debug_launch_count", "metis_debug_timestamp", "metis_debug_wait_timeout", "metis_debug_build", "metis_debug_index_check",
+            "metis_debug_reciprocals",
             "metis_sf_bytes", "metis_workspace_bytes", "metis_default_sample_count", "metis_quantize_nvfp4", "metis_quantize_rht_nvfp4",
             "metis_split", "metis_requantize_operand", "metis_linear_fwd", "metis_linear_fwd_static_ws", "metis_linear_bwd", "metis_gemm_nvfp4"]
 
@@ -75,6 +76,7 @@ def lib():
     l.metis_debug_build.argtypes = []
     l.metis_debug_build.restype = i32
     l.metis_debug_index_check.argtypes = [vp, i64, i64, i64, vp]
+    l.metis_debug_reciprocals.argtypes = [vp, vp, i64, vp, vp, vp]
     l.metis_sf_bytes.argtypes = [i64, i64, i32]
     l.metis_sf_bytes.restype = sz
     l.metis_workspace_bytes.argtypes = [i32, i64, i64, i32, i32, P(sz)]
@@ -352,6 +354,12 @@ class Handle:
     def index_check(self, offset, nbytes, extent, stream=None):
         """metis_debug_index_check: the debug build's store check on a made-up store (nothing is accessed)."""
         _check("metis_debug_index_check", lib().metis_debug_index_check(self._h, offset, nbytes, extent, _stream_ptr(stream)))
+
+    def reciprocals(self, x, stream=None):
+        """metis_debug_reciprocals: (1 / x, 1 / sqrt(x)) of a contiguous float64 CUDA tensor, as the decomposition's kernels form them."""
+        rcp, rsq = torch.empty_like(x), torch.empty_like(x)
+        _check("metis_debug_reciprocals", lib().metis_debug_reciprocals(self._h, _ptr(x), x.numel(), _ptr(rcp), _ptr(rsq), _stream_ptr(stream)))
+        return rcp, rsq
 
     def wait_timeout(self, polls=256, stream=None):
         """metis_debug_wait_timeout: runs the bounded-wait hook; returns the two per-warp words as a CUDA int32 tensor."""

@@ -5,6 +5,7 @@
 
 #include <atomic>
 
+#include "reciprocal.cuh"
 #include "tc_ptx.cuh"
 
 size_t metis_split_ws_bytes(int64_t rows, int64_t cols, int k, int p);
@@ -132,6 +133,22 @@ int32_t metis_debug_build(void) {
 metis_status_t metis_debug_index_check(metis_handle_t h, int64_t offset, int64_t nbytes, int64_t extent, metis_stream_t stream) {
   if (!h || nbytes <= 0 || extent < 0) return METIS_ERR_INVALID_ARG;
   index_check_kernel<<<1, 1, 0, reinterpret_cast<cudaStream_t>(stream)>>>(h->dev_status, offset, nbytes, extent); METIS_COUNT_LAUNCH();
+  METIS_CUDA_TRY(cudaGetLastError());
+  return METIS_OK;
+}
+
+namespace {
+__global__ void reciprocals_kernel(const double* __restrict__ x, int64_t n, double* __restrict__ rcp, double* __restrict__ rsq) {
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= n) return;
+  rcp[i] = metis_small::rcp_newton(x[i]);
+  rsq[i] = metis_small::rsqrt_newton(x[i]);
+}
+}  // namespace
+
+metis_status_t metis_debug_reciprocals(metis_handle_t h, const double* x, int64_t n, double* rcp, double* rsqrt, metis_stream_t stream) {
+  if (!h || !x || !rcp || !rsqrt || n <= 0 || n > (int64_t)1 << 30) return METIS_ERR_INVALID_ARG;
+  reciprocals_kernel<<<(unsigned)metis_ceil_div(n, 256), 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(x, n, rcp, rsqrt); METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
   return METIS_OK;
 }

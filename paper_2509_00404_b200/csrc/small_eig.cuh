@@ -2,33 +2,13 @@
 // eigen-decomposition.  Both are latency chains on one SM, so what counts is the number of dependent steps and how long one is.
 #pragma once
 #include "common.cuh"
+#include "reciprocal.cuh"
 #include "tridiag.cuh"
 
 namespace metis_small {
 
 constexpr int MAXQ = 72;                                // k + p at most (k = 64 with p = 8)
 constexpr int PITCH = MAXQ + 4;                         // doubles; 4 or 12 mod 16: every fragment access below is conflict-free
-
-// 1/sqrt(x) in FP64: scaled into the FP32 range by an even power of two, FP32 seed, two Newton steps
-__device__ __forceinline__ double rsqrt64(double x) {
-  int e;
-  const double mant = frexp(x, &e);                     // x = mant * 2^e, mant in [0.5, 1)
-  const int e2 = e & ~1;
-  const double xs = ldexp(mant, e - e2);                // in [0.5, 2)
-  double y = (double)rsqrtf((float)xs);
-  y = y * (1.5 - 0.5 * xs * y * y);
-  y = y * (1.5 - 0.5 * xs * y * y);
-  return ldexp(y, -(e2 / 2));
-}
-
-// 1/x in FP64: the hardware's FP64 reciprocal seed (error below 2^-20) and two Newton steps
-__device__ __forceinline__ double rcp64(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  y = fma(y, fma(-x, y, 1.0), y);
-  y = fma(y, fma(-x, y, 1.0), y);
-  return y;
-}
 
 // FP64 tensor-core tile: d (8 x 8) += a (8 x 4) b (4 x 8).  Lane (g = lane / 4, q = lane % 4) holds a[g][q], b[q][g] and
 // d[g][2q], d[g][2q + 1].
@@ -67,7 +47,7 @@ __device__ __forceinline__ void group_cholesky(double* Y, int n, double tol, dou
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const double d = __shfl_sync(0xFFFFFFFFu, vd[j], j);
-        const double rd = d > tol ? rcp64(d) : 0.0;
+        const double rd = d > tol ? rcp_newton(d) : 0.0;
         if ((lane & 7) == j) my_pivot = d;
         const double ld = vd[j] * rd, l = v[j] * rd;
 #pragma unroll
@@ -78,7 +58,7 @@ __device__ __forceinline__ void group_cholesky(double* Y, int n, double tol, dou
         }
       }
       const bool ok = my_pivot > tol;
-      inv = ok ? rsqrt64(my_pivot) : 0.0;
+      inv = ok ? rsqrt_newton(my_pivot) : 0.0;
       if (ok) dmin = fmin(dmin, my_pivot);
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
@@ -542,7 +522,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const double pn = fma(d[u], p, -e2[u] * pm);
-          d[u] = pn * metis_tri::rcp_mid(p + 1e-290);
+          d[u] = pn * rcp_newton(p + 1e-290);
           pm = p; p = pn;
         }
 #pragma unroll
@@ -580,7 +560,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
 #pragma unroll
       for (int t = 0; t < 2 * NT8; ++t) {
         const int i = s + 4 * t;
-        const double f = eo[i < at ? i : max(i - 1, 0)] * metis_tri::rcp_mid((i < at ? du[t] : dd[t]) + 1e-60);
+        const double f = eo[i < at ? i : max(i - 1, 0)] * rcp_newton((i < at ? du[t] : dd[t]) + 1e-60);
         Z[i * P + e] = i < n ? (i == at ? 1.0 : -f) : 0.0;
       }
     }
@@ -603,7 +583,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
         i += 4 * step;
       }
       zz += __shfl_xor_sync(0xFFFFFFFFu, zz, 1);
-      if (step > 0 && e < N8) ys[e] = e < rank ? metis_tri::rsqrt_mid(zz) : 0.0;         // a dependent column of the factor: no vector
+      if (step > 0 && e < N8) ys[e] = e < rank ? rsqrt_newton(zz) : 0.0;         // a dependent column of the factor: no vector
     }
   } else {
     // ---- meanwhile: the reflectors in panels of eight, H_8b ... H_8b+7 = I - V_b^T T_b V_b (T_b: inverse of diag(1 / beta) + the
@@ -772,7 +752,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
           for (int o = 4; o > 0; o >>= 1) { sx += __shfl_xor_sync(0xFFFFFFFFu, sx, o); sy += __shfl_xor_sync(0xFFFFFFFFu, sy, o); }
           if (active && sub < 2) {
             const double v = sub == 0 ? sx : sy;
-            inv_s[2 * (2 * m + h) + sub] = v > 0.0 ? rsqrt64(v) : 0.0;
+            inv_s[2 * (2 * m + h) + sub] = v > 0.0 ? rsqrt_newton(v) : 0.0;
           }
         }
       }
@@ -918,8 +898,8 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
         __syncwarp();
         if (active && c * c > 1e-30 * (a * b)) {
           above |= c * c > 1e-13 * (a * b);
-          const double d = b - a, rh = rsqrt64(fma(4.0 * c, c, d * d));
-          const double cc = fma(0.5 * fabs(d), rh, 0.5), rs = rsqrt64(cc);
+          const double d = b - a, rh = rsqrt_newton(fma(4.0 * c, c, d * d));
+          const double cc = fma(0.5 * fabs(d), rh, 0.5), rs = rsqrt_newton(cc);
           const double cs = cc * rs, sn = (d < 0.0 ? -c : c) * rh * rs;
 #pragma unroll
           for (int t = 0; t < NT8; ++t) {

@@ -3,30 +3,17 @@
 // and not a result: vectors of eigenvalues that agree to 1e-9 or so come out linearly dependent, and the caller has to look.
 #pragma once
 #include "common.cuh"
+#include "reciprocal.cuh"
 
 namespace metis_tri {
-
-// 1/sqrt(x) and 1/x for x well inside the FP64 range: the hardware's seed (error below 2^-20) and one step of third order
-__device__ __forceinline__ double rsqrt_mid(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(0.375, e, 0.5), y);
-}
-__device__ __forceinline__ double rcp_mid(double x) {
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x, y, 1.0);
-  return fma(y, fma(e, e, e), y);
-}
 
 // The reflector that takes x (first entry x0, squared length sq) to alpha e_1: H = I - beta v v^T, v = x - alpha e_1.
 // x whose square is below rounding of a matrix with entries near one is left alone (beta = 0).
 __device__ __forceinline__ void reflector(double x0, double sq, double& alpha, double& beta) {
-  const double len = sq * rsqrt_mid(sq);
+  const double len = sq * metis_small::rsqrt_newton(sq);
   const bool on = sq > 1e-60;
   alpha = on ? -copysign(len, x0) : x0;
-  beta = on ? rcp_mid(fma(fabs(x0), len, sq)) : 0.0;
+  beta = on ? metis_small::rcp_newton(fma(fabs(x0), len, sq)) : 0.0;
 }
 
 // Sturm sequences of T - x over 8 * blocks rows for M points x: the numbers of eigenvalues below them.  te[i] = (d_i, e_{i-1}^2),

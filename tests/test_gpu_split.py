@@ -551,3 +551,24 @@ def test_a_wide_split_repeats_itself(ctx, k, p):
         if first is None:
             first = got
         assert all(torch.equal(a, b) for a, b in zip(first, got))
+
+
+def test_reciprocals_against_cuda_and_extended_precision(ctx):
+    """The FP64 reciprocal and reciprocal square root of the dense kernels, from 2^-1000 to 2^1000 with 1e-290 and 1e-60 (what keeps a
+    pivot from zero) among them.  Error bounds: one rounding for the reciprocal, three halves of one for the root (its product is rounded
+    before it is subtracted), against 80-bit arithmetic; CUDA's own results are within one rounding (division) and two (root)."""
+    B, h = ctx
+    rng = np.random.default_rng(17)
+    x = np.ldexp(rng.uniform(1.0, 2.0, 1 << 20), rng.integers(-1000, 1000, 1 << 20))
+    x[:6] = [1e-290, 1e-60, 1.0, 2.0, 4.0, 1.0 - 2.0 ** -53]
+    x[6:1024] = np.ldexp(1.0 + rng.integers(0, 64, 1018) * 2.0 ** -52, rng.integers(-600, 600, 1018))       # just above powers of two
+    dx = torch.from_numpy(x).cuda()
+    rcp, rsq = h.reciprocals(dx)
+    wide = x.astype(np.longdouble)
+    for got, ref, bound in ((rcp, 1.0 / wide, 1.0), (rsq, 1.0 / np.sqrt(wide), 1.5)):
+        err = np.max(np.abs(got.cpu().numpy().astype(np.longdouble) - ref) / ref)
+        assert err <= bound * 2.0 ** -53 * (1.0 + 2.0 ** -10), float(err * 2.0 ** 53)
+    for got, ref, bound in ((rcp, 1.0 / dx, 2.0), (rsq, torch.rsqrt(dx), 3.5)):
+        assert ((got - ref).abs() / ref).max() <= bound * 2.0 ** -53 * (1.0 + 2.0 ** -10)
+    neg = h.reciprocals(-dx)[0]
+    assert torch.equal(neg, -rcp)
