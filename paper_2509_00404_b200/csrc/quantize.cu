@@ -14,7 +14,6 @@ amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, 
   // |x| as a bit pattern: non-negative floats order like their bit patterns, infinity above every number and a
   // NaN above infinity, so a non-finite element survives the reduction (fmaxf would drop a NaN)
   metis_pdl_wait();
-  metis_pdl_trigger();                                     // the quantizer behind this kernel sets itself up meanwhile
   constexpr int UNROLL = 8;
   constexpr int E = DTYPE == METIS_BF16 ? 8 : 4;           // elements per load
   uint32_t m = 0u;
@@ -41,6 +40,9 @@ amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, 
       }
     }
   }
+  // The launch of the quantizer behind this kernel overlaps its end.  (At the head, the quantizer's CTAs, which need the result for
+  // all they do, would stand on SMs for as long as this kernel runs: up to 81 us, out of the reach of other streams.)
+  metis_pdl_trigger();
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
   __shared__ uint32_t wmax[8];
