@@ -665,7 +665,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
     for (int t = 0; t < 2 * NT8; ++t) z[t] = Zc[((lane >> 3) + 4 * t) * P + (lane & 7)];
     __syncwarp();
 #pragma unroll
-    for (int t = 0; t < 2 * NT8; ++t) Zc[pos[(lane >> 3) + 4 * t] * P + (lane & 7)] = z[t] * rz;
+    for (int t = 0; t < 2 * NT8; ++t) Zc[pos[(lane >> 3) + 4 * t] * P + (lane & 7)] = rz != 0.0 ? z[t] * rz : 0.0;   // (z may have overflowed)
   }
   __syncthreads();
 
@@ -686,6 +686,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
     bool again = false;
     X = U; Wb = W;
     if (attempt == 1) {                                 // the start by way of T had dependent vectors
+      orth_only = false;
       constexpr float exit_cos2 = EIG_TIGHT_COS2;
       for (int o = tid; o < NB * RP; o += EIG_THREADS) {
         const int b = o / RP, r = o % RP;
