@@ -1253,13 +1253,14 @@ metis_status_t launch_eig_wide(cudaStream_t s, const double* gram1, int n, doubl
   else if (n <= 96) METIS_TRY((launch_tridiag<91, 96, 9, 3, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
   else if (n <= 128) METIS_TRY((launch_tridiag<97, 128, 9, 4, false>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
   else if (n <= WT_MAX) METIS_TRY((launch_tridiag<129, WT_MAX, 10, 4, true>(s, gram1, n, l, perm, st, w, sm, g1, x[0])));
-  else METIS_TRY(launch_chol_wide(s, gram1, n, 1e-14, l, nullptr, perm, st, nullptr, nullptr));
-  if (n <= WT_MAX) {}
-  else if (n <= 176) METIS_TRY((launch_jacobi_fp32<8, 22>(s, l, n, x[0])));
-  else if (n <= 192) METIS_TRY((launch_jacobi_fp32<16, 12>(s, l, n, x[0])));
-  else if (n <= 224) METIS_TRY((launch_jacobi_fp32<16, 14>(s, l, n, x[0])));
-  else if (n <= 256) METIS_TRY((launch_jacobi_fp32<16, 16>(s, l, n, x[0])));
-  else METIS_TRY((launch_jacobi_fp32<16, 18>(s, l, n, x[0])));
+  else {
+    METIS_TRY(launch_chol_wide(s, gram1, n, 1e-14, l, nullptr, perm, st, nullptr, nullptr));
+    if (n <= 176) METIS_TRY((launch_jacobi_fp32<8, 22>(s, l, n, x[0])));
+    else if (n <= 192) METIS_TRY((launch_jacobi_fp32<16, 12>(s, l, n, x[0])));
+    else if (n <= 224) METIS_TRY((launch_jacobi_fp32<16, 14>(s, l, n, x[0])));
+    else if (n <= 256) METIS_TRY((launch_jacobi_fp32<16, 16>(s, l, n, x[0])));
+    else METIS_TRY((launch_jacobi_fp32<16, 18>(s, l, n, x[0])));
+  }
   const unsigned t = (unsigned)((n + 31) / 32);
   for (int step = 0; step < ER_STEPS; ++step) {
     double *xc = x[step & 1], *xn = x[(step & 1) ^ 1];
