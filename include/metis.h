@@ -154,6 +154,11 @@ metis_status_t metis_debug_index_check(metis_handle_t h, int64_t offset, int64_t
  * a decomposition form them (Newton-Raphson; for normal values whose results are normal). */
 metis_status_t metis_debug_reciprocals(metis_handle_t h, const double* x, int64_t n, double* rcp, double* rsqrt, metis_stream_t stream);
 
+/* Test hook: eigenvalues (n, descending) and eigenvectors (columns of the n x n evecs) of a symmetric positive semi-definite matrix of order
+ * n <= 272, row-major FP64 on the device, by the solver of a decomposition.  Workspace for n > 72: 8 n (n + 34) doubles. */
+metis_status_t metis_debug_eigen(metis_handle_t h, const double* gram, int32_t n, double* evals, double* evecs, void* ws, size_t ws_bytes,
+                                 metis_stream_t stream);
+
 /* Test / benchmark hook: kernels launched by the library in this process so far (host counter, atomic). */
 uint64_t metis_debug_launch_count(void);
 

@@ -27,7 +27,7 @@ STATUS_NAMES = {0: "OK", 1: "INVALID_ARG", 2: "SHAPE", 3: "ALIGNMENT", 4: "WORKS
 
 EXPORTED = ["metis_create", "metis_destroy", "metis_last_device_status", "metis_debug_quantile_table",
             "metis_debug_launch_count", "metis_debug_timestamp", "metis_debug_wait_timeout", "metis_debug_build", "metis_debug_index_check",
-            "metis_debug_reciprocals",
+            "metis_debug_reciprocals", "metis_debug_eigen",
             "metis_sf_bytes", "metis_workspace_bytes", "metis_default_sample_count", "metis_quantize_nvfp4", "metis_quantize_rht_nvfp4",
             "metis_split", "metis_requantize_operand", "metis_linear_fwd", "metis_linear_fwd_static_ws", "metis_linear_bwd", "metis_gemm_nvfp4"]
 
@@ -77,6 +77,7 @@ def lib():
     l.metis_debug_build.restype = i32
     l.metis_debug_index_check.argtypes = [vp, i64, i64, i64, vp]
     l.metis_debug_reciprocals.argtypes = [vp, vp, i64, vp, vp, vp]
+    l.metis_debug_eigen.argtypes = [vp, vp, i32, vp, vp, vp, sz, vp]
     l.metis_sf_bytes.argtypes = [i64, i64, i32]
     l.metis_sf_bytes.restype = sz
     l.metis_workspace_bytes.argtypes = [i32, i64, i64, i32, i32, P(sz)]
@@ -360,6 +361,15 @@ class Handle:
         rcp, rsq = torch.empty_like(x), torch.empty_like(x)
         _check("metis_debug_reciprocals", lib().metis_debug_reciprocals(self._h, _ptr(x), x.numel(), _ptr(rcp), _ptr(rsq), _stream_ptr(stream)))
         return rcp, rsq
+
+    def eigen(self, gram, stream=None):
+        """metis_debug_eigen: (eigenvalues descending, eigenvectors as columns) of a symmetric positive semi-definite float64 CUDA matrix."""
+        n = gram.shape[0]
+        evals, evecs = torch.zeros(n, dtype=torch.float64, device="cuda"), torch.zeros((n, n), dtype=torch.float64, device="cuda")
+        ws = torch.empty(8 * n * (n + 34), dtype=torch.float64, device="cuda")
+        _check("metis_debug_eigen", lib().metis_debug_eigen(self._h, _ptr(gram.contiguous()), n, _ptr(evals), _ptr(evecs), _ptr(ws), 8 * ws.numel(),
+                                                            _stream_ptr(stream)))
+        return evals, evecs
 
     def wait_timeout(self, polls=256, stream=None):
         """metis_debug_wait_timeout: runs the bounded-wait hook; returns the two per-warp words as a CUDA int32 tensor."""

@@ -1233,7 +1233,8 @@ refine_correction_kernel(const double* __restrict__ s, const double* __restrict_
       e = 0.5 * r;
       if (i != j) {
         const double sv = s[o], li = s[(int64_t)i * n + i] / gi, lj = s[(int64_t)j * n + j] / gj;
-        if (sv * sv > 1e-28 * fabs(li * lj)) {            // orthogonal to FP64 rounding otherwise
+        const double ro = 0.5 * r * (li + lj);            // what orthonormalising alone adds to S_ij
+        if (fmax(sv * sv, ro * ro) > 1e-28 * fabs(li * lj)) {                      // orthogonal to FP64 rounding otherwise, and stays so
           const double gap = lj - li, a = sv + lj * r, b = sv + li * r;
           if (fabs(a) < 0.0625 * fabs(gap) && fabs(b) < 0.0625 * fabs(gap)) e = a / gap;
           else if (sv * sv > 1e-24 * fabs(li * lj)) open = true;

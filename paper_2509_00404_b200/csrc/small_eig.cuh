@@ -174,13 +174,18 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 //      four rotations between the blocks on the 4 x 4 Gram matrix in registers and applies them, 784 cycles at n = 40) and
 //      step 3 is repeated; if pairs are still open after that, they are only orthonormalised in step 3 and FP64
 //      one-sided Jacobi sweeps on the columns of W = L^T U, U rotated along, finish the work (repeated eigenvalues).
-// Precision: the columns of U leave the loop orthonormal, and the pairs of W orthogonal, to 1e-10 or better.
+// Precision, n = 8 ... 72, in 80 bits (in brackets: with the FP32 sweeps as every start): U^T G U diagonal to 2e-15 (2e-12) of its largest
+// entry, and to 1e-14, 1e-13 and 4e-12 (6e-12, 3e-11 and 9e-10) of sqrt(lambda_i lambda_j) where the eigenvalues span two, four and six decades (the factor's
+// rounding), U orthonormal to 1e-15 (1e-13); eigenvalues within 4e-5 of each other 3e-14 and 1e-13 (6e-8 and 1e-14); half of them repeated
+// 1e-8 and 3e-9 (7e-8 and 2e-8).  A pair of W that is orthogonal already is left to the orthonormalisation alone, half of R_ij to either column, only
+// if that does not tilt it: between eigenvalues of different size it does, by half of R_ij times the root of their ratio.
 // Input: Gram matrix (ld x ld, leading n x n block used).  Output: eigenvalues descending, eigenvectors as columns of
 // evecs[n][n].
-// Measured alone, planted spectrum (before: the Jacobi sweeps of step 4 as the start of every matrix): n = 8 10.4 us (12.5), n = 32 33 (42),
-// n = 40 43 (66), n = 64 88 (128), n = 72 115 (228); eigenvalues within 4e-5 of each other n = 40 47 (158), n = 72 128 (719); nearly diagonal
-// matrices are the ones the sweeps finished sooner: n = 32 33 (25), n = 40 43 (35).  Repeated eigenvalues pay for both starts:
-// half of them equal to the last digit n = 40 176 (152), n = 72 919 (861).  The reduction takes 18 of the 43 us at n = 40, the multisection 6.
+// Measured alone, planted spectrum (before: the Jacobi sweeps of step 4 as the start of every matrix): n = 8 10.4 us (12.5), n = 32 33 (43),
+// n = 40 43 (64), n = 64 88 (127), n = 72 115 (242); eigenvalues within 4e-5 of each other n = 40 47 (151), n = 72 129 (840).  Nearly diagonal
+// matrices are the ones the sweeps finished sooner: off the diagonal 1e-4 of it n = 32 33 (21), n = 40 43 (29), n = 72 115 (80), a multiple of the
+// identity n = 40 54 (25), n = 72 150 (66).  Repeated eigenvalues pay for both starts: half of them n = 40 161 (142), n = 72 882 (877).
+// The reduction takes 18 of the 43 us at n = 40, the multisection 6.
 // Four threads per row reduce the matrix while six warps factorise it; the products and the multisection use all of them.
 constexpr int EIG_CHOL_THREADS = 192;
 __host__ __device__ constexpr int eig_threads(int nt8) { return nt8 <= 1 ? 256 : 512; }
@@ -820,7 +825,8 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
               if (inv_s[i] == 0.0 || inv_s[j] == 0.0) { e_ij = 0.0; e_ji = 0.0; }
               else if (!orth_only) {
                 const double gap = lam[j] - lam[i], a = sv[u][e] + lam[j] * r, b = sv[u][e] + lam[i] * r;
-                if (sv[u][e] * sv[u][e] > 1e-28 * fabs(lam[i] * lam[j])) {         // orthogonal to FP64 rounding: nothing to rotate
+                const double ro = 0.5 * r * (lam[i] + lam[j]);                     // what orthonormalising alone adds to S_ij
+                if (fmax(sv[u][e] * sv[u][e], ro * ro) > 1e-28 * fabs(lam[i] * lam[j])) {    // else orthogonal to FP64 rounding, and stays so
                   if (fabs(a) < 0.0625 * fabs(gap) && fabs(b) < 0.0625 * fabs(gap)) {
                     const double rg = 1.0 / gap;
                     e_ij = a * rg; e_ji = -b * rg;

@@ -1441,6 +1441,15 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
 
 }  // namespace
 
+metis_status_t metis_debug_eigen(metis_handle_t h, const double* gram, int32_t n, double* evals, double* evecs, void* ws, size_t ws_bytes, metis_stream_t stream) {
+  if (!h || !gram || !evals || !evecs) return METIS_ERR_INVALID_ARG;
+  if (n < 1 || n > metis_wide::MAXQ_WIDE) return METIS_ERR_SHAPE;
+  const size_t nn = (size_t)n * n;
+  if (n > MAXQ && (!ws || !metis_aligned16(ws) || ws_bytes < sizeof(double) * (8 * nn + (size_t)metis_wide::MAXQ_WIDE * n))) return METIS_ERR_WORKSPACE;
+  double* scratch = reinterpret_cast<double*>(ws);        // seven matrices, then the factor and the columns of the FP64 sweeps
+  return launch_eig_wide(reinterpret_cast<cudaStream_t>(stream), gram, n, scratch, scratch + 7 * nn, scratch + 8 * nn, evals, evecs);
+}
+
 int64_t metis_default_sample_count(int64_t rows, int32_t q) {
   int64_t want = 4 * (int64_t)q;
   const int64_t pct = (rows + 99) / 100;
