@@ -79,10 +79,12 @@ __device__ __forceinline__ uint32_t e2m1x8_rne(float a0, float a1, float a2, flo
   return w;
 }
 
-// What a 16-bit draw u contributes to the rounding of its element: 256 u - 2^24, one byte permutation of the Philox word that holds
-// the draw in its low (hi = false) or high half.
-constexpr uint32_t SR_SEL_LO = 0x4105u, SR_SEL_HI = 0x4325u;                    // byte selectors, against 0xFF
-__device__ __forceinline__ uint32_t sr_term(uint32_t word, bool hi) { return __byte_perm(word, 0xFFu, hi ? SR_SEL_HI : SR_SEL_LO); }
+// What a 16-bit draw u contributes to the rounding of its element, one byte permutation of a Philox word that holds the draw in its
+// low (hi = false) or high half:  256 u - 2^24 of the word as it is, or (COMPL) (65535 - u) 256 + 255 of its complement.
+template <bool COMPL> constexpr uint32_t SR_SEL_LO = COMPL ? 0x5104u : 0x4105u;  // byte selectors, against 0xFF
+template <bool COMPL> constexpr uint32_t SR_SEL_HI = COMPL ? 0x5324u : 0x4325u;
+template <bool COMPL>
+__device__ __forceinline__ uint32_t sr_term(uint32_t word, bool hi) { return __byte_perm(word, 0xFFu, hi ? SR_SEL_HI<COMPL> : SR_SEL_LO<COMPL>); }
 
 // Eight stochastically rounded codes in one word; term[i] = sr_term of draw i.  The same decision as metis_e2m1_sr,
 // arranged for the instruction mix of the SM (integer logic, shifts and compares issue at half the FP32 / IMAD rate, and bound
@@ -90,27 +92,30 @@ __device__ __forceinline__ uint32_t sr_term(uint32_t word, bool hi) { return __b
 //   b = max(a, RU(a/2 + 1/2)) maps a < 1 onto [1/2, 1] (the E2M1 grid {0, 1/2, 1} becomes {1/2, 3/4, 1}: one
 //       mantissa bit per binade like the values from 1 up) and leaves a >= 1 alone, without a select;
 //   with S = 4 bits(b) + (65535 - u) 256 + 255 the 22 mantissa bits below the grid bit carry into it exactly when  frac * 65536 > u
-//       (4 frac22 + (65535 - u) 256 + 255 >= 2^24  <=>  frac22 > 64 u): comparison, selection and increment in one multiply-add.  What is
-//       formed is the complement, ~S = term - 4 bits(b): the draw then enters as it is (complementing the Philox words first
-//       cost half an instruction per element);
+//       (4 frac22 + (65535 - u) 256 + 255 >= 2^24  <=>  frac22 > 64 u): comparison, selection and increment in one multiply-add.  Either S is
+//       formed (COMPL) or its complement, ~S = term - 4 bits(b), where the draw enters as it is: complementing the Philox words costs half an
+//       instruction per element, which the quantizer saves; the residual pass, at its 96 registers a thread, spills then
+//       (8192 x 14336, k = 32, on a slower part: 214 us with S, 227 with ~S);
 //   the magnitude code is bits 24 .. 26 of S, minus 4 modulo 8: the top bytes of four elements are gathered by byte permutations, the
 //       two words of even and odd elements are merged and the complement and the eight "- 4" taken off together;
 //   the sign nibbles are gathered with one funnel shift per element and masked once per word.
 // (Against a compare per element with the draw shifted up and codes packed one by one: residual_tc_kernel 236 -> 204 us at 8192 x 14336, k = 32, the
-// minimum per element below included; quantize_kernel 472 -> 371 us at 16384 x 14336 with both orientations, its third CTA per SM
-// included; 340 us with the complement formed here, the scale byte without branches and one block of code per loop.)
+// minimum per element below included, 199 us with the scale byte without branches; quantize_kernel 472 -> 371 us at 16384 x 14336 with
+// both orientations, its third CTA per SM included, 340 us with the complement formed here, that scale byte and one block of code per loop.)
+template <bool COMPL>
 __device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_t (&term)[8]) {
   uint32_t s[8], sgn = 0u;
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
     const float a = fabsf(y[i]);                           // at most 6 (the caller has seen to it)
-    s[i] = term[i] - __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f))) * 4u;
+    const uint32_t b4 = __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f))) * 4u;
+    s[i] = COMPL ? b4 + term[i] : term[i] - b4;
     sgn = __funnelshift_l(__float_as_uint(y[i]), sgn, 4);  // top nibble of y (sign and three exponent bits) shifted in
   }
   const uint32_t even = __byte_perm(__byte_perm(s[0], s[2], 0x0073u), __byte_perm(s[4], s[6], 0x7300u), 0x7610u);
   const uint32_t odd = __byte_perm(__byte_perm(s[1], s[3], 0x0073u), __byte_perm(s[5], s[7], 0x7300u), 0x7610u);
   const uint32_t mag = ((even & 0x0F0F0F0Fu) | ((odd * 16u) & 0xF0F0F0F0u));
-  return ((mag & 0x77777777u) ^ 0x33333333u) | (sgn & 0x88888888u);
+  return ((mag & 0x77777777u) ^ (COMPL ? 0x44444444u : 0x33333333u)) | (sgn & 0x88888888u);
 }
 
 // largest magnitude of a block: eight three-input maxima, which pass a NaN over or (KEEP_NAN) on
@@ -137,7 +142,8 @@ __device__ __forceinline__ uint32_t e4m3_ceil_byte(float t) {
 }
 
 // encode_block with the multiplier looked up in a table filled by fill_r_table (same bytes as encode_block).
-// term[i] = sr_term of draw i (only read with stochastic rounding).
+// term[i] = sr_term<COMPL> of draw i (only read with stochastic rounding).
+template <bool COMPL>
 __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&term)[16], bool sr, float six_s_T,
                                                      const float* r_tab, uint32_t (&packed)[2]) {
   if (!sr) {
@@ -173,8 +179,8 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
       y0[i] = copysignf(fminf(fabsf(a), 6.0f), a); y1[i] = copysignf(fminf(fabsf(b), 6.0f), b);
     }
   }
-  packed[0] = e2m1x8_sr(y0, t0);
-  packed[1] = e2m1x8_sr(y1, t1);
+  packed[0] = e2m1x8_sr<COMPL>(y0, t0);
+  packed[1] = e2m1x8_sr<COMPL>(y1, t1);
   return byte;
 }
 

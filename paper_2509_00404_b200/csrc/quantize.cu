@@ -218,7 +218,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       }
       draw_at += 4 * (uint64_t)p.e_stride_r;               // 32 rows, eight draws to a Philox block
 #pragma unroll
-      for (int j = 0; j < 8; ++j) { u[2 * j] = sr_term(nw[j], false); u[2 * j + 1] = sr_term(nw[j], true); }
+      for (int j = 0; j < 8; ++j) { u[2 * j] = sr_term<false>(nw[j], false); u[2 * j + 1] = sr_term<false>(nw[j], true); }
       if (want_r) {
         if (sizeof(T) == 2) {
           uint4* drow = reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(rnd) + r * 256);
@@ -233,7 +233,7 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
     }
     if (want_c) {
       uint32_t packed[2];
-      const uint32_t byte = encode_block_tab(v, u, sr, six_s_T, r_tab, packed);
+      const uint32_t byte = encode_block_tab<false>(v, u, sr, six_s_T, r_tab, packed);
       if (in) METIS_DBG_GUARD(p.dbg, code_at, 8, p.rows * p.cols / 2) *reinterpret_cast<uint2*>(p.c_codes + code_at) = make_uint2(packed[0], packed[1]);
       code_at += 16 * p.cols;
       sfc[r * 8 + b] = in ? (uint8_t)byte : (uint8_t)0;
@@ -262,14 +262,14 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
             const uint32_t w = reinterpret_cast<const uint32_t*>(rnd)[(b * 16 + i) * 64 + pw];
-            u0[i] = sr_term(w, false); u1[i] = sr_term(w, true);
+            u0[i] = sr_term<false>(w, false); u1[i] = sr_term<false>(w, true);
           }
         }
         uint32_t packed[2];
-        uint32_t byte = encode_block_tab(v0, u0, sr, six_s_T, r_tab, packed);
+        uint32_t byte = encode_block_tab<false>(v0, u0, sr, six_s_T, r_tab, packed);
         *reinterpret_cast<uint2*>(codes_s + wd * QK_CP + b * 8) = make_uint2(packed[0], packed[1]);
         sfr[wd * 8 + b] = (uint8_t)byte;
-        byte = encode_block_tab(v1, u1, sr, six_s_T, r_tab, packed);
+        byte = encode_block_tab<false>(v1, u1, sr, six_s_T, r_tab, packed);
         *reinterpret_cast<uint2*>(codes_s + (64 + wd) * QK_CP + b * 8) = make_uint2(packed[0], packed[1]);
         sfr[(64 + wd) * 8 + b] = (uint8_t)byte;
       }
@@ -283,10 +283,10 @@ quantize_kernel(const T* __restrict__ x, int64_t ld, metis_qt::QuantParams p, co
       for (int i = 0; i < 16; ++i) v[i] = reinterpret_cast<const float*>(tile)[(b * 16 + i) * TP + (((c >> 2) ^ (c >> 5)) << 2 | (c & 3))];
       if (sr) {
 #pragma unroll
-        for (int i = 0; i < 16; ++i) u[i] = sr_term((uint32_t)rnd[(b * 16 + i) * TILE + c], false);
+        for (int i = 0; i < 16; ++i) u[i] = sr_term<false>((uint32_t)rnd[(b * 16 + i) * TILE + c], false);
       }
       uint32_t packed[2];
-      const uint32_t byte = encode_block_tab(v, u, sr, six_s_T, r_tab, packed);
+      const uint32_t byte = encode_block_tab<false>(v, u, sr, six_s_T, r_tab, packed);
       *reinterpret_cast<uint2*>(codes_s + c * QK_CP + b * 8) = make_uint2(packed[0], packed[1]);
       sfr[c * 8 + b] = (uint8_t)byte;
     }

@@ -38,13 +38,15 @@ constexpr int NUM_THREADS = 64 + 32 * N_EW;               // producer, MMA issue
 constexpr size_t SMEM_BYTES = (size_t)RING * SLOT_BYTES + 2 * X_BYTES + N_EW * (PATCH_F * 4 + PATCH_U * 2) + 1024 + 256 + metis_qt::R_TABLE * 4;
 
 struct ResidArgs {
-  QuantParams p;
   const float* amax_src;
+  QuantParams p;
   float* ts_out0; float* ts_out1;
   float* dense;
   int k_chunks;             // 64-wide K chunks of A6 / B6
   uint32_t* dev_status;
 };
+// (8192 x 14336, stochastic rounding, the branching scale byte: 218 us so, 228 with the round keys eight bytes off; the quantizer does not mind)
+static_assert((offsetof(ResidArgs, p) + offsetof(QuantParams, keys)) % 16 == 0, "the round keys lie on 16 bytes among the kernel's parameters");
 
 // out[i][6*kp padded to kx] for vector i: pattern A = [h|h|l|h|l2|l] (coefficients), pattern B = [h|l|h|l2|h|l] (basis).
 // src element (i, j): src[i*stride_i + j*stride_j], j < k (zero beyond).  One thread per (i, group of 8 j).
@@ -236,7 +238,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
       if (lane == 0) { mbar_arrive(tempty_bar(acc)); mbar_arrive(xempty_bar(xb)); }
       const bool step_ok = FAST || c0 < p.cols;                                      // false: the warp's columns lie outside the matrix
       const bool blk1_ok = FAST || c0 + 16 < p.cols;
-      uint32_t nw[16];                                      // draws, two per word
+      uint32_t nw[16];                                      // complemented draws, two per word
       if (sr) {
         const uint64_t e0 = (uint64_t)row * (uint64_t)p.e_stride_r + (uint64_t)c0;        // multiple of 8
 #pragma unroll
@@ -244,7 +246,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           const uint4 w = metis_philox_block_keys((e0 >> 3) + q4, p.keys, p.stream_id);
           const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) nw[4 * q4 + j] = ww[j];
+          for (int j = 0; j < 4; ++j) nw[4 * q4 + j] = ~ww[j];
         }
       }
       if (!FAST && g.dense != nullptr && row_ok && step_ok) {
@@ -263,9 +265,9 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         float v0[16], v1[16];
         uint32_t u0[16], u1[16];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? metis_qt::sr_term(nw[i >> 1], i & 1) : 0u; u1[i] = sr ? metis_qt::sr_term(nw[8 + (i >> 1)], i & 1) : 0u; }
-        const uint32_t sb0 = encode_block_tab(v0, u0, sr, six_s_T, r_tab, pk0);
-        const uint32_t sb1 = encode_block_tab(v1, u1, sr, six_s_T, r_tab, pk1);
+        for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? metis_qt::sr_term<true>(nw[i >> 1], i & 1) : 0u; u1[i] = sr ? metis_qt::sr_term<true>(nw[8 + (i >> 1)], i & 1) : 0u; }
+        const uint32_t sb0 = encode_block_tab<true>(v0, u0, sr, six_s_T, r_tab, pk0);
+        const uint32_t sb1 = encode_block_tab<true>(v1, u1, sr, six_s_T, r_tab, pk1);
         if (!FAST && row_ok) {
           uint8_t* cp = p.c_codes + row * c_kbytes + c0 / 2;
           METIS_DBG_GUARD(g.dev_status, row * c_kbytes + c0 / 2, blk1_ok ? 16 : 8, p.rows * c_kbytes) {
@@ -288,7 +290,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         // blocks along the rows: the warp transposes its 32 x 32 values 16 columns at a time through its patch;
         // in each half lane l encodes the block of column l % 16, rows 16 * (l / 16) .. +15
         const int cb = lane & 15, rb = lane >> 4;
-        const uint32_t term_sel = (cb & 1) ? metis_qt::SR_SEL_HI : metis_qt::SR_SEL_LO;
+        const uint32_t term_sel = (cb & 1) ? metis_qt::SR_SEL_HI<true> : metis_qt::SR_SEL_LO<true>;
         const bool rb_ok = FAST || slab_row0 + 16 * rb < p.rows;
         if (FAST) {                                                          // the patch still feeds the last tile's copies until here
           if (lane == 0) bulk_wait_read_all();
@@ -318,7 +320,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             d[i] = sr ? __byte_perm(upatch[rb * 176 + i * 10 + (cb >> 1)], 0xFFu, term_sel) : 0u;   // sr_term of this column's half
           }
           uint32_t pk[2];
-          const uint32_t sb = encode_block_tab(t, d, sr, six_s_T, r_tab, pk);
+          const uint32_t sb = encode_block_tab<true>(t, d, sr, six_s_T, r_tab, pk);
           pkr[hf][0] = pk[0]; pkr[hf][1] = pk[1];
           if (!FAST && col_ok && rb_ok) METIS_DBG_GUARD(g.dev_status, col * r_kbytes + (slab_row0 + 16 * rb) / 2, 8, p.cols * r_kbytes)
             *reinterpret_cast<uint2*>(p.r_codes + col * r_kbytes + (slab_row0 + 16 * rb) / 2) = make_uint2(pk[0], pk[1]);

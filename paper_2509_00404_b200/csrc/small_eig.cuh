@@ -175,7 +175,7 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 //      step 3 is repeated; if pairs are still open after that, they are only orthonormalised in step 3 and FP64
 //      one-sided Jacobi sweeps on the columns of W = L^T U, U rotated along, finish the work (repeated eigenvalues).
 // Precision, n = 8 ... 72, in 80 bits (in brackets: with the FP32 sweeps as every start): U^T G U diagonal to 2e-15 (2e-12) of its largest
-// entry, and to 1e-14, 1e-13 and 4e-12 (6e-12, 3e-11 and 9e-10) of sqrt(lambda_i lambda_j) where the eigenvalues span two, four and six decades (the factor's
+// entry, and to 1e-14, 1e-13 and 4e-12 (4e-12, 3e-11 and 9e-10) of sqrt(lambda_i lambda_j) where the eigenvalues span two, four and six decades (the factor's
 // rounding), U orthonormal to 1e-15 (1e-13); eigenvalues within 4e-5 of each other 3e-14 and 1e-13 (6e-8 and 1e-14); half of them repeated
 // 1e-8 and 3e-9 (7e-8 and 2e-8).  A pair of W that is orthogonal already is left to the orthonormalisation alone, half of R_ij to either column, only
 // if that does not tilt it: between eigenvalues of different size it does, by half of R_ij times the root of their ratio.
