@@ -947,7 +947,7 @@ constexpr int WV_WARPS = 4, WV_ROUNDS = 7;                // of the multisection
 __global__ void __launch_bounds__(32 * WV_WARPS)
 tridiag_vectors_kernel(const double* __restrict__ tri, const double* __restrict__ v, int n, double* __restrict__ zt, double* __restrict__ panels) {
   metis_pdl_wait_trigger();
-  __shared__ __align__(16) double2 te[WT_MAX + 1];
+  __shared__ __align__(16) double2 te[WT_MAX + 8];          // (a block beyond the matrix is read ahead)
   __shared__ double eo[WT_MAX + 1], dn[WV_WARPS][WT_MAX], up[WV_WARPS][WT_MAX];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
   const int n8 = (n + 7) & ~7, groups = (n + WV_WARPS - 1) / WV_WARPS;
@@ -985,7 +985,7 @@ tridiag_vectors_kernel(const double* __restrict__ tri, const double* __restrict_
   }
   for (int i = tid; i <= n8; i += 32 * WV_WARPS) {
     const double e = i > 0 && i < n ? tri[n + i - 1] : 0.0;
-    te[i] = i < n ? make_double2(tri[i], i > 0 ? fmax(e * e, 1e-60) : 0.0) : make_double2(4.0 * WT_MAX, 0.0);
+    te[i] = i < n ? make_double2(tri[i], i > 0 ? fmax(e * e, metis_tri::TINY_SQUARE) : 0.0) : make_double2(4.0 * WT_MAX, 0.0);
     if (i > 0) eo[i - 1] = e;
   }
   __syncthreads();

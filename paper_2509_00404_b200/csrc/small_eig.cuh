@@ -1,6 +1,8 @@
 // One-CTA dense linear algebra of a decomposition (n <= 72): FP64 Cholesky factorisation and the symmetric
 // eigen-decomposition.  Both are latency chains on one SM, so what counts is the number of dependent steps and how long one is.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 #include "reciprocal.cuh"
 #include "tridiag.cuh"
@@ -156,9 +158,11 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 // ------------------------------------------------------------------------------------------------
 // Symmetric positive semi-definite eigen-decomposition in one CTA.
 //   1. Householder reduction to a tridiagonal matrix T in FP64 (tridiag.cuh), the matrix in the registers of four threads per row.
-//      A step is a chain of two reductions over eight lanes, a reciprocal square root, a reciprocal and three barriers, 750 - 870
-//      cycles at n = 40; what counts is the number of instructions a warp has to issue in it, so one more warp works out the
-//      scalars and the two vectors of the update, which every thread doing that for itself made 1250 - 1400 cycles.
+//      A step is a chain through one more warp, which works out the scalars, the vectors of the update and the next column: product, its sum with x,
+//      the update, the next product, 640 cycles at n = 40 (FP64 operation 8, matrix instruction 26, 64-bit shuffle with addition 35, shared-memory
+//      round trip 29, barrier 20 to 40).  What counts is how long the two chains are - the other warps' from the vectors to the next product and the
+//      scalars' warp's through the next reflector - and the bytes that the vectors bring into registers (128 a cycle: at n = 72 half of a step).
+//      Every thread working out the scalars for itself made it 1000 cycles, three barriers with the column published by its owner 1050.
 //      Meanwhile six warps sort the matrix by descending diagonal and factorise it, G = L L^T (dependent columns zeroed);
 //   2. eigenvalues of T by multisection on Sturm counts to a relative 2^-30 of themselves, eigenvectors by twisted factorisations
 //      (Dhillon and Parlett, "Orthogonal eigenvectors and relative gaps", 2003, without their representation tree), taken back through
@@ -181,11 +185,10 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 // if that does not tilt it: between eigenvalues of different size it does, by half of R_ij times the root of their ratio.
 // Input: Gram matrix (ld x ld, leading n x n block used).  Output: eigenvalues descending, eigenvectors as columns of
 // evecs[n][n].
-// Measured alone, planted spectrum (before: the Jacobi sweeps of step 4 as the start of every matrix): n = 8 10.4 us (12.5), n = 32 33 (43),
-// n = 40 43 (64), n = 64 88 (127), n = 72 115 (242); eigenvalues within 4e-5 of each other n = 40 47 (151), n = 72 129 (840).  Nearly diagonal
-// matrices are the ones the sweeps finished sooner: off the diagonal 1e-4 of it n = 32 33 (21), n = 40 43 (29), n = 72 115 (80), a multiple of the
-// identity n = 40 54 (25), n = 72 150 (66).  Repeated eigenvalues pay for both starts: half of them n = 40 161 (142), n = 72 882 (877).
-// The reduction takes 18 of the 43 us at n = 40, the multisection 6.
+// Measured alone, planted spectrum (in brackets: the reduction with three barriers a step, and the Jacobi sweeps of step 4 as the start of every
+// matrix): n = 8 10.3 us (10.3, 12.5), n = 32 25.8 (32.8, 43), n = 40 34.9 (43.1, 64), n = 64 68 (88, 127), n = 72 93 (115, 242).  Nearly diagonal
+// matrices are the ones the sweeps alone finish sooner (off the diagonal 1e-4 of it n = 32 21, n = 40 29, n = 72 80), and repeated eigenvalues pay for both starts.
+// Cycles at n = 40: load 2.5 k, reduction 25 k, multisection 13 k + 2 k, vectors 5.6 k + 4.9 k, refinement 7.4 k, output 2.3 k.
 // Four threads per row reduce the matrix while six warps factorise it; the products and the multisection use all of them.
 constexpr int EIG_CHOL_THREADS = 192;
 __host__ __device__ constexpr int eig_threads(int nt8) { return nt8 <= 1 ? 256 : 512; }
@@ -303,29 +306,23 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   __shared__ int perm[N8], order[N8];
   __shared__ double gmax_s;
   __shared__ int flags[EIG_MAX_SWEEPS], flags64[EIG_MAX_SWEEPS];
-  __shared__ __align__(16) double2 te[N8 + 1];          // diagonal and squared subdiagonal of the tridiagonal matrix
-  __shared__ __align__(16) double ys[N8], rs[2][N8], us[N8];
-  __shared__ __align__(16) double2 pq[N8];
+  __shared__ __align__(16) double2 te[N8 + 8];          // diagonal and squared subdiagonal of the tridiagonal matrix (a block beyond it is read ahead)
+  __shared__ __align__(16) double ys[N8], rs[2][N8], us[N8], ps[N8], qs[N8];
   __shared__ double eo[N8 + 1], beta_s[N8], v1_s[N8];
   __shared__ int pos[N8];
-  __shared__ unsigned char grid_count[EIG_THREADS];
-  __shared__ __align__(16) double Tp[64 * NT8], Pt[64 * NT8];
+  __shared__ unsigned char grid_count[EIG_THREADS / 2];
+  __shared__ __align__(16) double Tp[64 * NT8];
   __shared__ unsigned int emax_s[2][EIG_MAX_REFINE];
   __shared__ float en_w[EIG_THREADS / 32];
   __shared__ uint8_t pairs[NB][GROUPS][2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q = lane & 3;
 
-  // ---- the matrix; tables ----
+  // ---- the matrix ----
   for (int o = tid; o < N8 * N8; o += EIG_THREADS) {
     const int i = o / N8, j = o % N8;
     E[i * P + j] = (i < n && j < n) ? gm[i * ld + j] : (i == j ? -1.0 : 0.0);
   }
   if (tid < N8) perm[tid] = tid;
-  for (int o = tid; o < (NB - 1) * GROUPS; o += EIG_THREADS) {                  // round-robin tournament of the blocks
-    const int step = o / GROUPS, m = o % GROUPS;
-    const int a = m == 0 ? 0 : (step + m) % (NB - 1) + 1, b = m == 0 ? step % (NB - 1) + 1 : (step + NB - 1 - m) % (NB - 1) + 1;
-    pairs[step][m][0] = (uint8_t)min(a, b); pairs[step][m][1] = (uint8_t)max(a, b);
-  }
   if (tid < EIG_MAX_SWEEPS) flags[tid] = flags64[tid] = 0;
   if (tid < EIG_MAX_REFINE) emax_s[0][tid] = emax_s[1][tid] = 0u;
   __syncthreads();
@@ -336,13 +333,13 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   const int ex = top > 0 && top < 2046 ? (top - 1022 + 1) >> 1 : 0;
   const double y_scale = __hiloint2double((1023 - ex) << 20, 0);
   double* V = W;                                        // row j: column j of the trailing matrix when it is reduced (reflector j)
-  const int s8 = tid & 7;
-  auto bar_r = [] { asm volatile("bar.sync 2, %0;" ::"n"(TS) : "memory"); };
+  auto arrive = [](int id) { asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(TS) : "memory"); };
+  auto await = [](int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(TS) : "memory"); };
+  constexpr int Y_READY = 2, U_READY = 4, X_READY = 5;
   if (tid < TD) {
-    auto bar = bar_r;
     // ---- Householder reduction: eight lanes hold rows i0 and i0 + 1 in registers (columns s8, s8 + 8, ...) ----
-    const int i0 = 2 * (tid >> 3), last_row = (tid | 31) >> 2 | 1;
-    double row[2][NT8];
+    const int s8 = tid & 7, i0 = 2 * (tid >> 3), last_row = (tid | 31) >> 2 | 1;
+    double row[2][NT8], x[NT8];
 #pragma unroll
     for (int h = 0; h < 2; ++h)
 #pragma unroll
@@ -350,51 +347,64 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
         const int c = s8 + 8 * t, i = i0 + h;
         row[h][t] = i < n && c < n ? 0.5 * (E[i * P + c] + E[c * P + i]) * (y_scale * y_scale) : 0.0;
       }
-    // row j (if this thread holds part of it) becomes the next column to be reduced, row j + 1 goes beside it
-    auto publish = [&](int j) {
+    if (tid < 8) {                                      // column 0; row 1
+      if (tid == 0) te[0].x = row[0][0];
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
-        if ((j + u) >> 1 == i0 >> 1) {
-          double* out = u == 0 ? V + j * P : rs[j & 1];
-          const bool odd = (j + u) & 1;
-#pragma unroll
-          for (int t = 0; t < NT8; ++t) out[s8 + 8 * t] = s8 + 8 * t > j ? (odd ? row[1][t] : row[0][t]) : 0.0;
-        }
-    };
-    publish(0);
-    if (tid == 0) te[0].x = row[0][0];
-    bar();
-#pragma unroll 1
-    for (int j = 0; j + 2 < n; ++j) {
-      const bool live = last_row > j;                   // the warp has a row below j
-      double x[NT8];
-      if (live) {
-        double y0 = 0.0, y1 = 0.0;
-#pragma unroll
-        for (int t = 0; t < NT8; ++t) {
-          x[t] = V[j * P + s8 + 8 * t];
-          y0 = fma(row[0][t], x[t], y0); y1 = fma(row[1][t], x[t], y1);
-        }
-        const bool hi = s8 & 4;                         // lanes 0 - 3 end with the sum of row i0, lanes 4 - 7 with that of i0 + 1
-        double y = (hi ? y1 : y0) + __shfl_xor_sync(0xFFFFFFFFu, hi ? y0 : y1, 4);
-        y += __shfl_xor_sync(0xFFFFFFFFu, y, 2);
-        y += __shfl_xor_sync(0xFFFFFFFFu, y, 1);
-        if ((s8 & 3) == 0) ys[i0 + (s8 >> 2)] = y;
-      }
-      bar();
-      bar();
-      if (live) {
-        const double2 c0 = pq[i0], c1 = pq[i0 + 1];
-#pragma unroll
-        for (int t = 0; t < NT8; ++t) {
-          const double u = us[s8 + 8 * t];
-          row[0][t] = fma(c0.x, u, fma(c0.y, x[t], row[0][t]));
-          row[1][t] = fma(c1.x, u, fma(c1.y, x[t], row[1][t]));
-        }
-        publish(j + 1);
-      }
-      bar();
+      for (int t = 0; t < NT8; ++t) { V[s8 + 8 * t] = s8 + 8 * t > 0 ? row[0][t] : 0.0; rs[0][s8 + 8 * t] = row[1][t]; }
     }
+    await(X_READY);
+#pragma unroll
+    for (int t = 0; t < NT8; ++t) x[t] = V[s8 + 8 * t];
+    // steps `from` ... `to` - 1, columns from 8 T0 on (those before are done)
+    auto steps = [&](auto t0, int from, int to) {
+      constexpr int T0 = decltype(t0)::value;
+#pragma unroll 1
+      for (int j = from; j < to; ++j) {
+        const bool live = last_row > j;                   // the warp has a row below j
+        if (live) {
+          // the sums of eight lanes are those of two columns of a matrix product that each lane q, q + 4, ... gets, for rows 2 q and 2 q + 1
+          // of the warp's eight: two matrix instructions and an addition (50 cycles; by shuffles 105)
+          double y0 = 0.0, y1 = 0.0, d0[2] = {0.0, 0.0}, d1[2] = {0.0, 0.0};
+#pragma unroll
+          for (int t = T0; t < NT8; ++t) { y0 = fma(row[0][t], x[t], y0); y1 = fma(row[1][t], x[t], y1); }
+          dmma(d0, 1.0, y0);
+          dmma(d1, 1.0, y1);
+          if (lane < 4) *reinterpret_cast<double2*>(ys + 8 * warp + 2 * lane) = make_double2(d0[0] + d0[1], d1[0] + d1[1]);
+        }
+        arrive(Y_READY);
+        await(U_READY);
+        if (live) {
+          const double2 c = *reinterpret_cast<const double2*>(ps + i0);
+#pragma unroll
+          for (int t = T0; t < NT8; ++t) {
+            const double u = us[s8 + 8 * t];
+            row[0][t] = fma(c.x, u, row[0][t]);
+            row[1][t] = fma(c.y, u, row[1][t]);
+          }
+        }
+        await(X_READY);
+        if (live) {
+          const double2 c = *reinterpret_cast<const double2*>(qs + i0);
+#pragma unroll
+          for (int t = T0; t < NT8; ++t) {
+            row[0][t] = fma(c.x, x[t], row[0][t]);
+            row[1][t] = fma(c.y, x[t], row[1][t]);
+            x[t] = V[(j + 1) * P + s8 + 8 * t];
+          }
+          double* out = rs[(j + 1) & 1] + s8;             // row j + 2 for the next step
+          const bool even = i0 == j + 2, odd = i0 + 1 == j + 2;
+#pragma unroll
+          for (int t = T0; t < NT8; ++t) {
+            if (even) out[8 * t] = row[0][t];
+            if (odd) out[8 * t] = row[1][t];
+          }
+        }
+      }
+    };
+    constexpr int SEG = NT8 >= 7 ? 3 : (NT8 >= 4 ? (NT8 + 1) / 2 : NT8);         // blocks of eight columns to a loop
+    steps(std::integral_constant<int, 0>{}, 0, min(8 * SEG, n - 2));
+    if (SEG < NT8) steps(std::integral_constant<int, SEG < NT8 ? SEG : 0>{}, 8 * SEG, min(16 * SEG, n - 2));
+    if (2 * SEG < NT8) steps(std::integral_constant<int, 2 * SEG < NT8 ? 2 * SEG : 0>{}, 16 * SEG, n - 2);
 #pragma unroll
     for (int h = 0; h < 2; ++h)                         // what is left of the last two rows
 #pragma unroll
@@ -404,50 +414,77 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
           if (i0 + h == n - 1) te[n - 1].x = row[h][t];
         }
   } else if (tid < TS) {
-    auto bar = bar_r;
-    // ---- the warp of the scalars (its four groups of eight lanes do the same): with y = A x and r = A e_1 it is
+    // ---- the warp of the scalars, entries lane, lane + 32, ... of the vectors: with y = A x and r = A e_1 it is
     // A v = u = y - alpha r,  v^T A v = x^T y - 2 alpha y_1 + alpha^2 r_1;  w = beta u - K v,  A -= v w^T + w v^T = p u^T + q v^T.
-    // Column j + 1 of the product is not read again except for its first entry, so x stands for v in the last term ----
-    bar();
+    // p and u, which do not depend on K, go ahead of q; the next column it updates by itself, so that the others go from the update
+    // to the next product without a barrier, and works out that column's reflector meanwhile.  Column j + 1 is not read again
+    // except for its first entry, so x stands for v in the others' last term ----
+    constexpr int OWN = (N8 + 31) / 32;
+    // the sum of a warp, in each lane: sums of four lanes first as columns (each lane gets two of the eight), then as rows
+    auto sum32 = [](double v) {
+      double d[2] = {0.0, 0.0}, f[2] = {0.0, 0.0};
+      dmma(d, 1.0, v);
+      dmma(f, d[0] + d[1], 1.0);
+      return f[0];
+    };
+    double x[OWN];
+    await(X_READY);
+#pragma unroll
+    for (int k = 0; k < OWN; ++k) x[k] = lane + 32 * k < N8 ? V[lane + 32 * k] : 0.0;
+    double x0 = V[1];
 #pragma unroll 1
     for (int j = 0; j + 2 < n; ++j) {
-      const double* r = rs[j & 1];
-      double x[NT8], rc[NT8], sq[2] = {0.0, 0.0}, xy[2] = {0.0, 0.0}, alpha, beta;
+      const double *rj = rs[j & 1], xb = V[j * P + j + 2];
+      double sq = 0.0, xy = 0.0, y[OWN], v[OWN], r[OWN], alpha, beta;
 #pragma unroll
-      for (int t = 0; t < NT8; ++t) { x[t] = V[j * P + s8 + 8 * t]; rc[t] = r[s8 + 8 * t]; }
-      const double x0 = V[j * P + j + 1], ra = r[j + 1];
+      for (int k = 0; k < OWN; ++k) sq = fma(x[k], x[k], sq);
+      metis_tri::reflector(x0, sum32(sq), alpha, beta);
+      const double v1 = x0 - alpha, pa = -beta * v1;
 #pragma unroll
-      for (int t = 0; t < NT8; ++t) sq[t & 1] = fma(x[t], x[t], sq[t & 1]);
-      sq[0] += sq[1];
-#pragma unroll
-      for (int o = 4; o > 0; o >>= 1) sq[0] += __shfl_xor_sync(0xFFFFFFFFu, sq[0], o);
-      metis_tri::reflector(x0, sq[0], alpha, beta);
-      const double b2 = beta * beta, v1 = x0 - alpha, a2 = alpha * alpha * ra;
-      bar();                                            // the product is there
-      double y[NT8];
-#pragma unroll
-      for (int t = 0; t < NT8; ++t) { y[t] = ys[s8 + 8 * t]; xy[t & 1] = fma(x[t], y[t], xy[t & 1]); }
-      const double ya = ys[j + 1], k0 = fma(-2.0 * alpha, ya, a2);
-      xy[0] += xy[1];
-#pragma unroll
-      for (int t = 0; t < NT8; ++t) {
-        y[t] = fma(-alpha, rc[t], y[t]);
-        us[s8 + 8 * t] = y[t];
+      for (int k = 0; k < OWN; ++k) {
+        const int e = lane + 32 * k;
+        v[k] = e == j + 1 ? v1 : x[k];
+        if (e < N8) ps[e] = -beta * v[k];
       }
+      eo[j] = alpha; beta_s[j] = beta; v1_s[j] = v1;
+      await(Y_READY);                                   // the product and row j + 1 are there
 #pragma unroll
-      for (int o = 4; o > 0; o >>= 1) xy[0] += __shfl_xor_sync(0xFFFFFFFFu, xy[0], o);
-      const double K2 = b2 * (xy[0] + k0);
+      for (int k = 0; k < OWN; ++k) {
+        const int e = min(lane + 32 * k, N8 - 1);
+        y[k] = ys[e]; r[k] = rj[e];
+      }
+      const double ya = ys[j + 1], ra = rj[j + 1], yb = ys[j + 2], rb = rj[j + 2];
 #pragma unroll
-      for (int t = 0; t < NT8; ++t) {
-        const double v = s8 + 8 * t == j + 1 ? v1 : x[t];
-        pq[s8 + 8 * t] = make_double2(-beta * v, fma(-beta, y[t], K2 * v));
+      for (int k = 0; k < OWN; ++k) {
+        const int e = lane + 32 * k;
+        xy = fma(x[k], y[k], xy);
+        y[k] = e > j ? fma(-alpha, r[k], y[k]) : 0.0;   // now u
+        if (e < N8) us[e] = y[k];
       }
-      bar();                                            // the update may go on
-      if (lane == 0) {
-        eo[j] = alpha; beta_s[j] = beta; v1_s[j] = v1;
-        te[j + 1].x = fma(-v1, fma(2.0 * beta, fma(-alpha, ra, ya), -K2 * v1), ra);
+      arrive(U_READY);
+      xy = sum32(xy);
+      const double ua = fma(-alpha, ra, ya), ba = -beta * ua, b2 = beta * beta, k0 = b2 * (alpha * fma(alpha, ra, -2.0 * ya));
+      double xv[OWN];
+#pragma unroll
+      for (int k = 0; k < OWN; ++k) {                   // all of the next column but the term with K
+        const int e = lane + 32 * k;
+        const bool in = e > j + 1 && e < N8;
+        r[k] = in ? fma(pa, y[k], fma(ba, v[k], r[k])) : 0.0;
+        xv[k] = in ? v1 * v[k] : 0.0;
+        y[k] *= -beta;
       }
-      bar();                                            // the next column is there
+      const double x0a = fma(pa, fma(-alpha, rb, yb), fma(ba, xb, rb)), x0b = v1 * xb;
+      const double K2 = fma(b2, xy, k0);
+#pragma unroll
+      for (int k = 0; k < OWN; ++k) {
+        const int e = lane + 32 * k;
+        x[k] = fma(K2, xv[k], r[k]);
+        if (e < N8) { qs[e] = fma(K2, v[k], y[k]); V[(j + 1) * P + e] = x[k]; }
+      }
+      arrive(X_READY);
+      x0 = fma(K2, x0b, x0a);
+      te[j + 1].x = fma(pa, ua, fma(fma(K2, v1, ba), v1, ra));
+      __syncwarp();
     }
   } else if (tid < TS + EIG_CHOL_THREADS) {
     // ---- meanwhile: sorted by the diagonal and factorised ----
@@ -473,7 +510,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   __syncthreads();
   const double gmax = gmax_s;
   if (tid <= N8) {
-    te[tid].y = tid > 0 && tid < n ? fmax(eo[tid - 1] * eo[tid - 1], 1e-60) : 0.0;
+    te[tid].y = tid > 0 && tid < n ? fmax(eo[tid - 1] * eo[tid - 1], metis_tri::TINY_SQUARE) : 0.0;
     if (tid >= n) te[tid].x = 4.0 * N8;
   }
   if (tid + 2 < n) V[tid * P + tid + 1] = v1_s[tid];
@@ -483,9 +520,10 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   }
   const int rank = __syncthreads_count(tid < n && inv_s[tid < n ? tid : 0] > 0.0);
   // ---- eigenvalues and eigenvectors of the tridiagonal matrix, descending ----
-  const long long grid_lo = __double_as_longlong(0x1p-56), grid_w = (__double_as_longlong(2.0 * N8) - grid_lo) / EIG_THREADS + 1;
-  {
-    const double x[1] = {__longlong_as_double(grid_lo + grid_w * (tid + 1))};  // brings every eigenvalue to about a tenth of an octave
+  constexpr int GRID = EIG_THREADS / 2;                  // points that bring every eigenvalue to about a sixth of an octave
+  const long long grid_lo = __double_as_longlong(0x1p-56), grid_w = (__double_as_longlong(2.0 * N8) - grid_lo) / GRID + 1;
+  if (tid < GRID) {
+    const double x[1] = {__longlong_as_double(grid_lo + grid_w * (tid + 1))};
     int c[1];
     metis_tri::sturm_counts<1>(te, NT8, x, c);
     grid_count[tid] = (unsigned char)c[0];
@@ -493,17 +531,17 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   __syncthreads();
   double *Dp = E, *Z = U;                               // column e of each: vector e
   constexpr int TV = 4 * N8;                            // four threads per vector
-  // Lanes per eigenvalue in the multisection, so that a warp (or two) runs on each of the four schedulers: a round costs 25 cycles per
-  // row and warp there.
+  // Lanes per eigenvalue in the multisection, two points each, so that a warp (or two) runs on each of the four schedulers: a round costs 25 cycles per
+  // row and warp there (three points on fewer warps: n = 40 1290 -> 1650 cycles a round).
   constexpr int LE = N8 <= 32 ? 4 : (N8 <= 40 || N8 > 64 ? 3 : 2), PW = 32 / LE, TE = (N8 + PW - 1) / PW * 32;
   {
     if (tid < TE) {
       const int e = PW * warp + min(lane / LE, PW - 1), below = max(n - 1 - e, 0);
       int at = 0;                                       // the first point with more than `below` eigenvalues under it
 #pragma unroll
-      for (int step = EIG_THREADS / 2; step > 0; step >>= 1) if (grid_count[at + step - 1] <= below) at += step;
-      const double v = metis_tri::multisect<LE>(te, NT8, grid_lo + grid_w * at, grid_lo + grid_w * (at + 1), below,
-                                                LE == 4 ? 9 : (LE == 3 ? 10 : 12));
+      for (int step = GRID / 2; step > 0; step >>= 1) if (grid_count[at + step - 1] <= below) at += step;
+      const double v = metis_tri::multisect<LE, 2>(te, NT8, grid_lo + grid_w * at, grid_lo + grid_w * (at + 1), below,
+                                                   LE == 4 ? 9 : (LE == 3 ? 10 : 12));
       if (lane % LE == 0 && lane / LE < PW && e < N8) lam[e] = v;
     }
   }
@@ -622,55 +660,41 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
     }
   }
   __syncthreads();
-  // ---- back through the panels: a warp per eight vectors, without a barrier ----
+  // ---- back through the panels: a warp per eight vectors, which it holds transposed, Z^T -= (Z^T V_b^T) T_b^T V_b: an accumulator tile
+  // (lane: row g, columns 2 q and 2 q + 1) is the left operand of the next product as it stands, its columns taken in the order 2 q, then
+  // 2 q + 1, so that nothing but V and T comes from shared memory (with Z there, n = 40: 6300 -> 3000 cycles) ----
   for (int tj = warp; tj < NT8; tj += EIG_THREADS / 32) {
-    double* Zc = Z + 8 * tj;
-    double* patch = Pt + 64 * tj;
-    if (8 * tj + 8 > n)                                 // vectors beyond the matrix
-      for (int i = lane; i < 8 * N8; i += 32) if (8 * tj + (i & 7) >= n) Zc[(i >> 3) * P + (i & 7)] = 0.0;
+    double z[NT8][2];
+#pragma unroll
+    for (int t = 0; t < NT8; ++t)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) z[t][h] = 8 * tj + g < n ? Z[(8 * t + 2 * q + h) * P + 8 * tj + g] : 0.0;     // (vectors beyond the matrix)
+    const double rz = ys[8 * tj + g];
     __syncwarp();
 #pragma unroll 1
     for (int b = (n - 3) >> 3; b >= 0; --b) {
-      const bool on_g = 8 * b + g + 2 < n;
-      double acc[2][2] = {};
+      const bool on = 8 * b + g + 2 < n, on0 = 8 * b + 2 * q + 2 < n, on1 = 8 * b + 2 * q + 3 < n;
+      const double *vr = V + (8 * b + g) * P + 2 * q, *v0 = V + (8 * b + 2 * q) * P + g;
+      double acc[2][2] = {}, y[2] = {0.0, 0.0};
 #pragma unroll
-      for (int kk = 0; kk < N8; kk += 4)
-        dmma(acc[(kk >> 2) & 1], on_g ? V[(8 * b + g) * P + kk + q] : 0.0, Zc[(kk + q) * P + g]);
-      *reinterpret_cast<double2*>(patch + 8 * g + 2 * q) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
-      __syncwarp();
-      double y[2] = {0.0, 0.0};
-#pragma unroll
-      for (int kk = 0; kk < 8; kk += 4) dmma(y, Tp[64 * b + 8 * g + kk + q], patch[8 * (kk + q) + g]);
-      __syncwarp();
-      *reinterpret_cast<double2*>(patch + 8 * g + 2 * q) = make_double2(-y[0], -y[1]);
-      __syncwarp();
-      const double y0 = patch[8 * q + g], y1 = patch[8 * (q + 4) + g];
-      const bool on0 = 8 * b + q + 2 < n, on1 = 8 * b + 4 + q + 2 < n;
-      double d[NT8][2], a0[NT8], a1[NT8];
-#pragma unroll
-      for (int ti = 0; ti < NT8; ++ti) {
-        const double2 z = *reinterpret_cast<const double2*>(Zc + (8 * ti + g) * P + 2 * q);
-        d[ti][0] = z.x; d[ti][1] = z.y;
-        a0[ti] = on0 ? V[(8 * b + q) * P + 8 * ti + g] : 0.0;
-        a1[ti] = on1 ? V[(8 * b + 4 + q) * P + 8 * ti + g] : 0.0;
+      for (int t = 0; t < NT8; ++t) {
+        const double2 v = on ? *reinterpret_cast<const double2*>(vr + 8 * t) : make_double2(0.0, 0.0);
+        dmma(acc[0], z[t][0], v.x);
+        dmma(acc[1], z[t][1], v.y);
       }
+      const double2 tb = *reinterpret_cast<const double2*>(Tp + 64 * b + 8 * g + 2 * q);
+      dmma(y, -(acc[0][0] + acc[1][0]), tb.x);
+      dmma(y, -(acc[0][1] + acc[1][1]), tb.y);
 #pragma unroll
-      for (int ti = 0; ti < NT8; ++ti) dmma(d[ti], a0[ti], y0);
+      for (int t = 0; t < NT8; ++t) dmma(z[t], y[0], on0 ? v0[8 * t] : 0.0);
 #pragma unroll
-      for (int ti = 0; ti < NT8; ++ti) {
-        dmma(d[ti], a1[ti], y1);
-        *reinterpret_cast<double2*>(Zc + (8 * ti + g) * P + 2 * q) = make_double2(d[ti][0], d[ti][1]);
-      }
-      __syncwarp();
+      for (int t = 0; t < NT8; ++t) dmma(z[t], y[1], on1 ? v0[P + 8 * t] : 0.0);
     }
     // normalised, in the order of the factor's rows
-    double z[2 * NT8];
-    const double rz = ys[8 * tj + (lane & 7)];
 #pragma unroll
-    for (int t = 0; t < 2 * NT8; ++t) z[t] = Zc[((lane >> 3) + 4 * t) * P + (lane & 7)];
-    __syncwarp();
+    for (int t = 0; t < NT8; ++t)
 #pragma unroll
-    for (int t = 0; t < 2 * NT8; ++t) Zc[pos[(lane >> 3) + 4 * t] * P + (lane & 7)] = rz != 0.0 ? z[t] * rz : 0.0;   // (z may have overflowed)
+      for (int h = 0; h < 2; ++h) Z[pos[8 * t + 2 * q + h] * P + 8 * tj + g] = rz != 0.0 ? z[t][h] * rz : 0.0;  // (z may have overflowed)
   }
   __syncthreads();
 
@@ -693,6 +717,11 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
     if (attempt == 1) {                                 // the start by way of T had dependent vectors
       orth_only = false;
       constexpr float exit_cos2 = EIG_TIGHT_COS2;
+      for (int o = tid; o < (NB - 1) * GROUPS; o += EIG_THREADS) {                  // round-robin tournament of the blocks
+        const int step = o / GROUPS, m = o % GROUPS;
+        const int a = m == 0 ? 0 : (step + m) % (NB - 1) + 1, b = m == 0 ? step % (NB - 1) + 1 : (step + NB - 1 - m) % (NB - 1) + 1;
+        pairs[step][m][0] = (uint8_t)min(a, b); pairs[step][m][1] = (uint8_t)max(a, b);
+      }
       for (int o = tid; o < NB * RP; o += EIG_THREADS) {
         const int b = o / RP, r = o % RP;
         Yb[o] = make_float2((float)(Lm[r * P + 2 * b] * y_scale), (float)(Lm[r * P + 2 * b + 1] * y_scale));
@@ -828,7 +857,7 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
                 const double ro = 0.5 * r * (lam[i] + lam[j]);                     // what orthonormalising alone adds to S_ij
                 if (fmax(sv[u][e] * sv[u][e], ro * ro) > 1e-28 * fabs(lam[i] * lam[j])) {    // else orthogonal to FP64 rounding, and stays so
                   if (fabs(a) < 0.0625 * fabs(gap) && fabs(b) < 0.0625 * fabs(gap)) {
-                    const double rg = 1.0 / gap;
+                    const double rg = rcp_newton(gap);
                     e_ij = a * rg; e_ji = -b * rg;
                   } else if (sv[u][e] * sv[u][e] > 1e-24 * fabs(lam[i] * lam[j])) open = true;
                 }
@@ -941,10 +970,8 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   }
   __syncthreads();
   if (tid < n) evals[tid] = lam[order[tid]] + 0.0 * gmax;                      // a non-finite matrix is seen by the status check
-  for (int o = tid; o < n * n; o += EIG_THREADS) {
-    const int i = o / n, j = o % n;
-    evecs[perm[i] * n + j] = X[i * P + order[j]];
-  }
+  for (int i = warp; i < n; i += EIG_THREADS / 32)
+    for (int j = lane; j < n; j += 32) evecs[perm[i] * n + j] = X[i * P + order[j]];
 }
 
 }  // namespace metis_small
