@@ -15,7 +15,7 @@ struct metis_nvtx_range {
 };
 #define METIS_NVTX(name) metis_nvtx_range nvtx_range_(name)
 
-constexpr int METIS_N_SIDE = 5;                        // side streams per handle (the backward pass uses all five)
+constexpr int METIS_N_SIDE = 1;                        // side streams per handle (the factor chain of a split)
 struct metis_context {
   int device;
   int sm_count;
@@ -278,3 +278,6 @@ metis_status_t metis_launch_gemm_check(const metis_nvfp4_t* a, const metis_nvfp4
                                        int64_t ldd, cudaStream_t s);
 metis_status_t metis_launch_gemm_tc(metis_context* ctx, const metis_nvfp4_t* a, const metis_nvfp4_t* b, void* d,
                                     int d_dtype, int64_t ldd, cudaStream_t s);
+// d (a->rows x b->rows, FP32) = a b^T for up to eight small products in one launch; widens: more than 64 rows of b make the tile wider
+struct metis_gemm_job { const metis_nvfp4_t *a, *b; float* d; int64_t ldd; bool widens; };
+metis_status_t metis_launch_gemm_group(metis_context* ctx, const metis_gemm_job* jobs, int n, cudaStream_t s);

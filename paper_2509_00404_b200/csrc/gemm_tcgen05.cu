@@ -7,10 +7,11 @@
 // These matrix products are where nearly all of the training arithmetic goes (Section 3): the
 // residual x residual term of Eq. 2 / Eq. 3 / the weight gradient, and the skinny factor products.
 //
-// Two kernels, both persistent over output tiles and warp-specialised (TMA producer warp, MMA issuer warp,
-// epilogue warps; shared-memory ring with mbarriers; FP32 accumulators in tensor memory):
-//   gemm_nvfp4_kernel<BLOCK_N>       one CTA per 128 x BLOCK_N tile (skinny products)
-//   two_cta::gemm_nvfp4_2cta_kernel  a CTA pair (cta_group::2) per 256 x 256 tile, optionally followed by BF16
+// Three kernels, all warp-specialised (TMA producer warp, MMA issuer warp, epilogue warps; shared-memory ring with
+// mbarriers; FP32 accumulators in tensor memory):
+//   gemm_nvfp4_kernel<BLOCK_N>       one CTA per 128 x BLOCK_N tile (an output dimension below 256), persistent
+//   gemm_nvfp4_group_kernel          the skinny products of a layer in one launch, contractions divided inside clusters
+//   two_cta::gemm_nvfp4_2cta_kernel  a CTA pair (cta_group::2) per 256 x 256 tile, persistent, optionally followed by BF16
 //                                    K boxes that add a low-rank correction into the same accumulator
 // The producer and issuer loops are walked by whole warps with one elected lane issuing, so that descriptors
 // and addresses stay in uniform registers.  Every mbarrier wait is bounded; on expiry the kernel records
@@ -260,6 +261,227 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   }
 }
 
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// shared::cluster address of the same shared-memory offset in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t local_addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
+  return r;
+}
+
+// =================================================================================================
+// The skinny products of one or two split products (rank x rank, residual x factor) in one launch: FP32 results of at most a few hundred
+// columns whose time is the latency of a CTA's K loop and of the launches.  A CTA takes one 128 x BLOCK_N tile and
+// 1 / 2^log_split of its contraction; the CTAs of a tile are neighbours in a cluster and add their accumulators in a fixed order through
+// distributed shared memory.  Every problem has its own split, chosen by the launcher so that no CTA's share is long and the SMs are filled.
+// As up to six launches of whole contractions on five streams, with the events between them, the products of a backward pass and what waits for
+// them took 17 us at 4096 x 4096 x 4096, k = 32, 11 us at 1088 x 2112 x 1472 and 29 us at 16384 tokens, 4096 -> 1024 (K = 16384 in 8 to 41 CTAs); now 12, 7 and 19 us.
+// =================================================================================================
+constexpr int GROUP_MAX = 8;
+struct alignas(64) GroupProblem {
+  CUtensorMap map_a, map_b;
+  const uint8_t *a_sf, *b_sf;
+  const float *a_ts, *b_ts;
+  float* d;
+  int64_t ldd;
+  int M, N, K, tiles_m, tiles, first_cluster, log_split;
+};
+struct GroupArgs {
+  GroupProblem p[GROUP_MAX];
+  int n;
+  uint32_t* dev_status;
+};
+
+template <int BLOCK_N, int STAGES>
+struct GroupCfg {
+  static constexpr int A_BYTES = BLOCK_M * BLOCK_K / 2, B_BYTES = BLOCK_N * BLOCK_K / 2, SF_BYTES = K_STEPS * 512;     // scales: 128 rows of either operand
+  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES + 2 * SF_BYTES;
+  static constexpr int SF_COLS = 2 * 4 * K_STEPS;          // scale columns of a ring stage
+  static constexpr int TMEM_COLS = BLOCK_N + STAGES * SF_COLS <= 256 ? 256 : 512;
+  static constexpr int PITCH = BLOCK_N + 4;                // floats; of the accumulator in shared memory
+  static constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 8 * (2 * STAGES + 1) + 8 + 896;                  // (the base is aligned to 128)
+  static_assert(BLOCK_N + STAGES * SF_COLS <= 512, "tensor memory budget");
+  static_assert(BLOCK_M * PITCH * 4 <= STAGES * STAGE_BYTES, "the accumulator takes the ring's place");
+};
+
+template <int BLOCK_N, int STAGES>
+__global__ void __launch_bounds__(NUM_THREADS)
+gemm_nvfp4_group_kernel(const __grid_constant__ GroupArgs args) {
+  using C = GroupCfg<BLOCK_N, STAGES>;
+  metis_pdl_trigger();
+  extern __shared__ __align__(1024) unsigned char group_smem[];
+  const uint32_t raw = smem_u32(group_smem), base = (raw + 1023u) & ~1023u;
+  unsigned char* gen_base = group_smem + (base - raw);
+  auto a_addr = [&](int s) { return base + (uint32_t)s * C::STAGE_BYTES; };
+  auto b_addr = [&](int s) { return a_addr(s) + C::A_BYTES; };
+  auto sfa_addr = [&](int s) { return b_addr(s) + C::B_BYTES; };
+  auto sfb_addr = [&](int s) { return sfa_addr(s) + C::SF_BYTES; };
+  const uint32_t bar_base = base + (uint32_t)STAGES * C::STAGE_BYTES;
+  auto full_bar = [&](int s) { return bar_base + 8u * s; };
+  auto empty_bar = [&](int s) { return bar_base + 8u * (STAGES + s); };
+  const uint32_t tfull_bar = bar_base + 8u * (2 * STAGES);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gen_base + (size_t)STAGES * C::STAGE_BYTES + 8 * (2 * STAGES + 1));
+  volatile int* dead = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  uint32_t csize;
+  asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(csize));
+  const int rank = (int)cluster_rank(), cluster = (int)(blockIdx.x / csize);
+  int which = 0;
+  while (which + 1 < args.n && cluster >= args.p[which + 1].first_cluster) ++which;
+  const GroupProblem& g = args.p[which];
+  const int split = 1 << g.log_split, part = rank & (split - 1);
+  const int tile = (cluster - g.first_cluster) * ((int)csize >> g.log_split) + (rank >> g.log_split);
+  const bool active = tile < g.tiles;
+  const int mb = tile % g.tiles_m, nb = tile / g.tiles_m;
+  const int num_kb = (g.K + BLOCK_K - 1) / BLOCK_K, kb0 = num_kb * part >> g.log_split, kb1 = active ? num_kb * (part + 1) >> g.log_split : kb0;
+  const int sf_k_atoms = g.K / MMA_K;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
+    mbar_init(tfull_bar, 1);
+    *dead = 0;
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc(smem_u32(tmem_slot), C::TMEM_COLS);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  metis_pdl_wait();                                          // the set-up above touched this CTA's shared and tensor memory only
+
+  const int quarter = warp & 3, row = quarter * 32 + lane;   // of the tile, warps 2 ... 5
+  bool done = false;                                         // this CTA's part of the accumulator is complete
+  if (warp == 0) {
+    int s = 0; uint32_t ph = 0;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait(empty_bar(s), ph ^ 1u, args.dev_status, dead)) break;
+      if (elect_one()) {
+        const int atoms = min(K_STEPS, sf_k_atoms - kb * K_STEPS);
+        mbar_expect_tx(full_bar(s), (uint32_t)(C::A_BYTES + C::B_BYTES) + (uint32_t)atoms * 1024u);
+        tma_load_2d(a_addr(s), &g.map_a, kb * (BLOCK_K / 2), mb * BLOCK_M, full_bar(s));
+        tma_load_2d(b_addr(s), &g.map_b, kb * (BLOCK_K / 2), nb * BLOCK_N, full_bar(s));
+        bulk_load(sfa_addr(s), g.a_sf + ((size_t)mb * sf_k_atoms + (size_t)kb * K_STEPS) * 512, atoms * 512, full_bar(s));
+        bulk_load(sfb_addr(s), g.b_sf + ((size_t)(nb * BLOCK_N / 128) * sf_k_atoms + (size_t)kb * K_STEPS) * 512, atoms * 512, full_bar(s));
+      }
+      __syncwarp();
+      if (++s == STAGES) { s = 0; ph ^= 1u; }
+    }
+  } else if (warp == 1) {
+    constexpr uint32_t idesc = make_idesc(BLOCK_M, BLOCK_N);
+    const uint32_t half = BLOCK_N < 128 ? (uint32_t)(nb * BLOCK_N % 128) / 32u : 0u;       // scale columns of the tile's rows inside their slab of 128
+    int s = 0; uint32_t ph = 0;
+    bool ok = true;
+    for (int kb = kb0; kb < kb1; ++kb) {
+      if (!mbar_wait(full_bar(s), ph, args.dev_status, dead)) { ok = false; break; }
+      tc_fence_after();
+      if (elect_one()) {
+        const int atoms = min(K_STEPS, sf_k_atoms - kb * K_STEPS);
+        const uint32_t sfa_t = tmem_base + BLOCK_N + s * C::SF_COLS, sfb_t = sfa_t + 4 * K_STEPS;
+        const uint64_t sfa_d = make_smem_desc(sfa_addr(s), 128, SWIZZLE_NONE), sfb_d = make_smem_desc(sfb_addr(s), 128, SWIZZLE_NONE);
+        const uint64_t a_d = make_smem_desc(a_addr(s), 1024, SWIZZLE_128B), b_d = make_smem_desc(b_addr(s), 1024, SWIZZLE_128B);
+        for (int k = 0; k < atoms; ++k) {
+          tc_cp_sf(sfa_t + 4 * k, sfa_d + (uint64_t)(k * 32));
+          tc_cp_sf(sfb_t + 4 * k, sfb_d + (uint64_t)(k * 32));
+        }
+        for (int k = 0; k < atoms; ++k)
+          tc_mma_nvf4(tmem_base, a_d + (uint64_t)(k * 2), b_d + (uint64_t)(k * 2), idesc, sfa_t + 4 * k, sfb_t + 4 * k + half, kb > kb0 || k > 0 ? 1u : 0u);
+        tc_commit(empty_bar(s));
+      }
+      __syncwarp();
+      if (++s == STAGES) { s = 0; ph ^= 1u; }
+    }
+    if (ok && kb1 > kb0 && elect_one()) tc_commit(tfull_bar);
+    __syncwarp();
+  } else if (kb1 > kb0 && mbar_wait(tfull_bar, 0u, args.dev_status, dead)) {
+    tc_fence_after();
+    done = true;
+  }
+  const float alpha = active && warp >= 2 ? (*g.a_ts) * (*g.b_ts) : 0.0f;
+  const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16);
+  const int64_t grow = (int64_t)mb * BLOCK_M + row;
+  float* acc_s = reinterpret_cast<float*>(gen_base);         // [BLOCK_M][PITCH], over the ring, which has been read
+  if (warp >= 2 && active) {
+#pragma unroll 1
+    for (int c0 = 0; c0 < BLOCK_N; c0 += 32) {
+      const int col = nb * BLOCK_N + c0;
+      if (col >= g.N) break;
+      uint32_t r[32];
+      if (done) tc_ld32(t_row + c0, r);
+      else {                                                 // a wait expired, or a share of no blocks
+#pragma unroll
+        for (int j = 0; j < 32; ++j) r[j] = 0u;
+      }
+      if (split > 1) {
+#pragma unroll
+        for (int j = 0; j < 32; j += 4)
+          *reinterpret_cast<float4*>(acc_s + row * C::PITCH + c0 + j) =
+              make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]), __uint_as_float(r[j + 3]));
+      } else if (grow < g.M) {
+        float* dst = g.d + grow * g.ldd + col;
+        if (col + 32 <= g.N && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+#pragma unroll
+          for (int j = 0; j < 32; j += 4)
+            *reinterpret_cast<float4*>(dst + j) = make_float4(__uint_as_float(r[j]) * alpha, __uint_as_float(r[j + 1]) * alpha,
+                                                              __uint_as_float(r[j + 2]) * alpha, __uint_as_float(r[j + 3]) * alpha);
+        } else {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) if (col + j < g.N) dst[j] = __uint_as_float(r[j]) * alpha;
+        }
+      }
+    }
+  }
+  if (csize > 1) {                                           // (the same for every CTA of the grid)
+    __syncwarp();
+    cluster_sync();
+    if (split > 1 && active && warp >= 2) {
+      // rows part * 128 / split ... of the tile, the parts added in their order; consecutive threads: consecutive columns
+      const int rows = BLOCK_M >> g.log_split, ncols = min(BLOCK_N, g.N - nb * BLOCK_N), per_row = (ncols + 3) / 4;
+      const uint32_t src = smem_u32(acc_s);
+      const uint32_t first = (uint32_t)(rank - part);
+      for (int o = threadIdx.x - 64; o < rows * per_row; o += 128) {
+        const int rr = part * rows + o / per_row, c = o % per_row * 4;
+        if (mb * BLOCK_M + rr >= g.M) break;
+        const uint32_t at = src + (uint32_t)(rr * C::PITCH + c) * 4u;
+        float4 x[8];                                         // all loads in flight
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          x[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (u < split)
+            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[u].x), "=f"(x[u].y), "=f"(x[u].z), "=f"(x[u].w) : "r"(map_to_rank(at, first + (uint32_t)u)));
+        }
+        float4 v = x[0];
+#pragma unroll
+        for (int u = 1; u < 8; ++u) { v.x += x[u].x; v.y += x[u].y; v.z += x[u].z; v.w += x[u].w; }
+        float* dst = g.d + (int64_t)(mb * BLOCK_M + rr) * g.ldd + nb * BLOCK_N + c;
+        const float e[4] = {v.x * alpha, v.y * alpha, v.z * alpha, v.w * alpha};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) if (c + j < ncols) dst[j] = e[j];
+      }
+    }
+    __syncwarp();
+    cluster_sync();                                          // the others may still be reading
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (*dead) {
+    // a wait expired: give copies already in flight time to land before the shared memory is released
+    for (int i = 0; i < 2000; ++i) __nanosleep(1000);
+    __syncthreads();
+  }
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, C::TMEM_COLS);
+  }
+}
+
 // =================================================================================================
 // Two-CTA variant (cta_group::2): a cluster of two CTAs on neighbouring SMs computes one 256 x 256 tile.
 // Each CTA loads 128 rows of A and 128 rows of B per K block (the pair's MMA reads both halves of B),
@@ -289,26 +511,12 @@ constexpr int NUM_THREADS = 384;                            // producer, MMA iss
 constexpr int OUT_STAGE_BYTES = 8 * 4096;                   // per epilogue warp: 32 rows x 128 bytes of converted output
 constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + OUT_STAGE_BYTES + 1024 + 256;
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // arrive on the barrier at the same shared-memory offset in CTA `rank` of the cluster
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t local_bar, uint32_t rank) {
   asm volatile(
       "{ .reg .b32 ra; mapa.shared::cluster.u32 ra, %0, %1;\n"
       "  mbarrier.arrive.release.cluster.shared::cluster.b64 _, [ra]; }"
       ::"r"(local_bar), "r"(rank) : "memory");
-}
-// shared::cluster address of the same shared-memory offset in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t local_addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
-  return r;
 }
 // Tensor load into THIS CTA's shared memory whose byte count is credited to a barrier that may live in the
 // pair's other CTA (cta_group::2 form; no multicast): both CTAs of a pair report to the leader's barrier.
@@ -699,6 +907,20 @@ metis_status_t launch(metis_context* ctx, const metis_nvfp4_t* a, const metis_nv
   return METIS_OK;
 }
 
+template <int BLOCK_N, int STAGES>
+metis_status_t launch_group(metis_context* ctx, const GroupArgs& args, int clusters, int csize, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(clusters * csize)); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = GroupCfg<BLOCK_N, STAGES>::SMEM_BYTES; cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)csize; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  METIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_nvfp4_group_kernel<BLOCK_N, STAGES>, args)); METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+
 // 2-D map over a row-major BF16 matrix rows x kx (kx a multiple of 64), box 64 elements x 128 rows, 128-byte swizzle
 metis_status_t make_bf16_map(metis_context* ctx, CUtensorMap* map, const void* ptr, int64_t rows, int64_t kx) {
   const cuuint64_t dims[2] = {(cuuint64_t)kx, (cuuint64_t)rows};
@@ -759,6 +981,9 @@ metis_status_t launch_2cta(metis_context* ctx, const metis_nvfp4_t* a, const met
 
 metis_status_t metis_gemm_set_attrs(metis_context* ctx) {
   METIS_CUDA_TRY(cudaFuncSetAttribute(gemm_nvfp4_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg<128>::SMEM_BYTES));
+  METIS_CUDA_TRY(cudaFuncSetAttribute(gemm_nvfp4_group_kernel<64, 7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GroupCfg<64, 7>::SMEM_BYTES));
+  METIS_CUDA_TRY(cudaFuncSetAttribute(gemm_nvfp4_group_kernel<64, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GroupCfg<64, 4>::SMEM_BYTES));
+  METIS_CUDA_TRY(cudaFuncSetAttribute(gemm_nvfp4_group_kernel<128, 6>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GroupCfg<128, 6>::SMEM_BYTES));
   METIS_CUDA_TRY(cudaFuncSetAttribute(two_cta::gemm_nvfp4_2cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)two_cta::SMEM_BYTES));
   // how many 2-CTA clusters can be resident at once (an odd SM count inside a GPC leaves an SM unpaired)
   cudaLaunchConfig_t cfg = {};
@@ -798,4 +1023,65 @@ metis_status_t metis_launch_gemm_tc_fused(metis_context* ctx, const metis_nvfp4_
       !metis_aligned16(lx) || !metis_aligned16(rx))
     return METIS_ERR_ALIGNMENT;
   return launch_2cta(ctx, a, b, d, d_dtype, ldd, lx, rx, kx, s);
+}
+
+// FP32 products of one launch (see gemm_nvfp4_group_kernel).  Split of the contractions: the problem whose CTAs have the most K blocks is halved again while
+// that fills SMs that have nothing, or while those CTAs alone would run a quarter longer than an
+// even share of all the work.
+metis_status_t metis_launch_gemm_group(metis_context* ctx, const metis_gemm_job* jobs, int n, cudaStream_t s) {
+  if (n <= 0) return METIS_OK;
+  if (n > GROUP_MAX) return METIS_ERR_INVALID_ARG;
+  int64_t widest = 0;
+  for (int i = 0; i < n; ++i) {
+    const metis_nvfp4_t *a = jobs[i].a, *b = jobs[i].b;
+    if (a->rows <= 0 || b->rows <= 0 || a->k_len != b->k_len || a->k_len % 64 != 0 || a->k_len <= 0) return METIS_ERR_SHAPE;
+    if (a->sf_layout != METIS_SF_TILED || b->sf_layout != METIS_SF_TILED) return METIS_ERR_INVALID_ARG;
+    if (!metis_aligned16(a->codes) || !metis_aligned16(b->codes) || !metis_aligned16(a->scales) || !metis_aligned16(b->scales)) return METIS_ERR_ALIGNMENT;
+    if (a->rows > INT32_MAX || b->rows > INT32_MAX || a->k_len > INT32_MAX) return METIS_ERR_SHAPE;
+    if (jobs[i].widens && b->rows > widest) widest = b->rows;
+  }
+  const int block_n = widest > 64 ? 128 : 64;
+  int64_t tiles[GROUP_MAX], kb[GROUP_MAX], total = 0, ctas = 0;
+  int split[GROUP_MAX], order[GROUP_MAX];
+  for (int i = 0; i < n; ++i) {
+    tiles[i] = metis_ceil_div(jobs[i].a->rows, BLOCK_M) * metis_ceil_div(jobs[i].b->rows, block_n);
+    kb[i] = metis_ceil_div(jobs[i].a->k_len, BLOCK_K);
+    split[i] = 0; order[i] = i;
+    total += tiles[i] * kb[i]; ctas += tiles[i];
+  }
+  for (;;) {
+    int top = -1;
+    for (int i = 0; i < n; ++i)
+      if (split[i] < 3 && kb[i] >> split[i] >= 4 && (top < 0 || kb[i] >> split[i] > kb[top] >> split[top])) top = i;
+    if (top < 0) break;
+    const int64_t more = tiles[top] << split[top], share = kb[top] >> split[top];
+    // (GPCs hold clusters of four and eight on 128 SMs)
+    if (ctas + more > (split[top] >= 1 ? 128 : ctx->sm_count) && 4 * share * ctx->sm_count <= 5 * total) break;
+    ctas += more; ++split[top];
+  }
+  int log_c = 0;
+  for (int i = 0; i < n; ++i) if (split[i] > log_c) log_c = split[i];
+  for (int i = 1; i < n; ++i)                              // the longest shares first
+    for (int j = i; j > 0 && kb[order[j]] >> split[order[j]] > kb[order[j - 1]] >> split[order[j - 1]]; --j) { const int t = order[j]; order[j] = order[j - 1]; order[j - 1] = t; }
+  GroupArgs args;
+  args.n = n; args.dev_status = ctx->dev_status;
+  int64_t clusters = 0;
+  for (int o = 0; o < n; ++o) {
+    const int i = order[o];
+    const metis_nvfp4_t *a = jobs[i].a, *b = jobs[i].b;
+    GroupProblem& g = args.p[o];
+    METIS_TRY(make_codes_map(ctx, &g.map_a, a, BLOCK_M));
+    METIS_TRY(make_codes_map(ctx, &g.map_b, b, block_n));
+    g.a_sf = a->scales; g.b_sf = b->scales; g.a_ts = a->tensor_scale; g.b_ts = b->tensor_scale;
+    g.d = jobs[i].d; g.ldd = jobs[i].ldd;
+    g.M = (int)a->rows; g.N = (int)b->rows; g.K = (int)a->k_len;
+    g.tiles_m = (int)metis_ceil_div(a->rows, BLOCK_M); g.tiles = (int)tiles[i];
+    g.first_cluster = (int)clusters; g.log_split = split[i];
+    clusters += metis_ceil_div(tiles[i], (int64_t)1 << (log_c - split[i]));
+  }
+  const int64_t grid = clusters << log_c;
+  if (grid > INT32_MAX) return METIS_ERR_SHAPE;
+  if (block_n == 128) return launch_group<128, 6>(ctx, args, (int)clusters, 1 << log_c, s);
+  // two CTAs to an SM where there is more than one for each
+  return grid > ctx->sm_count ? launch_group<64, 4>(ctx, args, (int)clusters, 1 << log_c, s) : launch_group<64, 7>(ctx, args, (int)clusters, 1 << log_c, s);
 }

@@ -27,129 +27,165 @@ __device__ __forceinline__ float deq_at(const uint8_t* codes, const uint8_t* sf,
   return metis_e2m1_value(code) * metis_e4m3_value(sf[metis_sf_offset(r, c / 16, k_len / 16, layout)]);
 }
 
-// Finishes the two skinny operands of the rank-(ka+kb) update, in place.  Layout: Lcat [M][kb + ka],
-// Rcat [N][kb + ka].  On entry Lcat[:, :kb] holds G1 and Rcat[:, kb:] holds Wt (written there by the skinny
-// GEMMs).  On exit  Lcat[:, :kb] = (G1 + Fo_a sa P) sb,  Lcat[:, kb:] = Fo_a sa,  Rcat[:, :kb] = Fo_b.
-// One warp per row.  Every global load of a row is issued before the first value is used (the loads are one
-// round trip instead of a chain of them), and the finished rows stay in shared memory for the BF16 pass.
-__device__ __forceinline__ float deq_of(uint32_t byte, uint32_t sf_byte, int64_t c) {
-  const uint32_t code = (c & 1) ? (byte >> 4) : (byte & 15u);
-  return metis_e2m1_value(code) * metis_e4m3_value((uint8_t)sf_byte);
+// Finishes the two skinny operands of the rank-(ka+kb) update.  Layout: Lcat [M][kb + ka], Rcat [N][kb + ka].  On entry Lcat[:, :kb] holds
+// G1 and Rcat[:, kb:] holds Wt (written there by the skinny GEMMs).  With A = (G1 + Fo_a sa P) sb the result is
+//   lx == nullptr:  in place, Lcat = [A | Fo_a sa], Rcat = [Fo_b | Wt]
+//   else:           the BF16 operands of the in-accumulator correction, zero padded to kx columns.  A dequantized factor entry is an
+//                   E2M1 x E4M3 product (six significant bits): with its FP32 scales moved to the other operand it is exact in BF16
+//                   and needs no low part, so each of the two rank-k terms costs two column groups instead of three:
+//                     Lx = [ A' hi | A' lo | Fa | Fa ],  A' = A ts_b / alpha        (k_b columns), Fa = Fo_a / ts_a (k_a)
+//                     Rx = [ Fb   | Fb   | B hi | B lo ],  Fb = Fo_b / ts_b (k_b),  B = Wt sa ts_a / alpha          (k_a columns)
+// A warp takes R rows (lane: vectors lane and lane + 32): every global load is issued before the first value is used, and a row of P in shared memory serves R rows.
+// Latency is what it costs (some 1.6 k instructions of a warp at nine cycles each with R = 4, J = 2 and two warps to a scheduler: 13 us for 4096 rows), so R is 1
+// until every scheduler has some eight warps, and ranks up to 32 have an instance of their own.  One row per warp for any number of rows, the finished rows
+// through shared memory and FP32 operands written beside the BF16 ones: 17.8 us for 16384 + 4096 rows at k = 32, 8 for 4096; now 9 - 10 and 6.
+// the two E2M1 codes of the low byte as FP16 (exact)
+__device__ __forceinline__ __half2 e2m1x2_to_half2(uint32_t byte) {
+  uint32_t w;
+  asm("{ .reg .b8 t; cvt.u8.u32 t, %1; cvt.rn.f16x2.e2m1x2 %0, t; }" : "=r"(w) : "r"(byte));
+  return *reinterpret_cast<const __half2*>(&w);
 }
-__global__ void __launch_bounds__(256)
-lowrank_finish_kernel(int64_t M, int64_t N, int ka, int kb,
-                      const uint8_t* foa_codes, const uint8_t* foa_sf, int foa_layout, const float* foa_ts,
-                      const float* sa,
-                      const uint8_t* fob_codes, const uint8_t* fob_sf, int fob_layout, const float* fob_ts,
-                      const float* sb, const float* __restrict__ pm, float* __restrict__ lcat, float* __restrict__ rcat,
-                      __nv_bfloat16* __restrict__ lx, __nv_bfloat16* __restrict__ rx, int kx,
-                      const float* res_a_ts, const float* res_b_ts) {
-  __shared__ float ps[64][65];
-  __shared__ float fa[8][64];
-  __shared__ float lrow[8][128];
-  __shared__ float rrow[8][128];
-  __shared__ float lraw[8][64], rraw[8][64];                // the factors as E2M1 x E4M3 products, before any FP32 scale
+struct FinishArgs {
+  int64_t M, N;
+  int ka, kb, kx, foa_layout, fob_layout;
+  const uint8_t *foa_codes, *foa_sf, *fob_codes, *fob_sf;
+  const float *foa_ts, *sa, *fob_ts, *sb, *pm;
+  float *lcat, *rcat;
+  __nv_bfloat16 *lx, *rx;
+  const float *res_a_ts, *res_b_ts;
+};
+// Two products' operands in one launch: blocks below n_first belong to the first.
+template <int R, int J>                                     // rows per warp: 1, 2 or 4; 32-vector groups of the ranks: 1 or 2
+__global__ void __launch_bounds__(256, J == 1 ? (R == 1 ? 6 : (R == 2 ? 5 : 4)) : (R == 4 ? 3 : 4))          // one wave where the rows allow it
+lowrank_finish_kernel(const __grid_constant__ FinishArgs first, const __grid_constant__ FinishArgs second, int n_first) {
+  const bool is_first = (int)blockIdx.x < n_first;
+  const FinishArgs& f = is_first ? first : second;
+  const int64_t M = f.M, N = f.N;
+  const int ka = f.ka, kb = f.kb, kx = f.kx, foa_layout = f.foa_layout, fob_layout = f.fob_layout;
+  const uint8_t *foa_codes = f.foa_codes, *foa_sf = f.foa_sf, *fob_codes = f.fob_codes, *fob_sf = f.fob_sf;
+  const float *foa_ts = f.foa_ts, *sa = f.sa, *fob_ts = f.fob_ts, *sb = f.sb, *__restrict__ pm = f.pm, *res_a_ts = f.res_a_ts, *res_b_ts = f.res_b_ts;
+  float *__restrict__ lcat = f.lcat, *__restrict__ rcat = f.rcat;
+  __nv_bfloat16 *__restrict__ lx = f.lx, *__restrict__ rx = f.rx;
+  __shared__ float ps[32 * J][32 * J];
+  __shared__ float fa[8][32 * J][R];                            // Fo_a sa of a warp's rows
   metis_pdl_wait();
   metis_pdl_trigger();                                      // the large GEMM behind this kernel sets itself up meanwhile
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int kc = ka + kb;
-  const int64_t i = (int64_t)blockIdx.x * 8 + warp;
-  // ---- loads (ka, kb <= 64: two values per lane and operand) ----
-  uint32_t a_byte[2] = {0u, 0u}, a_sfb[2] = {0u, 0u}, b_byte[2] = {0u, 0u}, b_sfb[2] = {0u, 0u};
-  float sa_v[2] = {0.0f, 0.0f}, sb_v[2] = {0.0f, 0.0f}, g1[2] = {0.0f, 0.0f}, wt[2] = {0.0f, 0.0f};
+  const int64_t i0 = ((int64_t)((int)blockIdx.x - (is_first ? 0 : n_first)) * 8 + warp) * R;     // (M and N are multiples of 16)
+  const bool in_m = i0 < M, in_n = i0 < N;
+  // ---- loads (ka, kb <= 64: two vectors per lane and operand) ----
+  uint32_t a_code[J] = {}, a_sfb[J] = {}, b_code[J] = {}, b_sfb[J] = {};
+  float sa_v[J] = {}, sb_v[J] = {}, g1[J][R] = {}, wt[J][R] = {};
 #pragma unroll
-  for (int j = 0; j < 2; ++j) {
+  for (int j = 0; j < J; ++j) {
     const int u = lane + 32 * j;
     if (u < ka) {
       sa_v[j] = sa[u];
-      if (i < M) {
-        a_byte[j] = foa_codes[(int64_t)u * (M / 2) + i / 2];
-        a_sfb[j] = foa_sf[metis_sf_offset(u, i / 16, M / 16, foa_layout)];
+      if (in_m) {
+        const uint8_t* src = foa_codes + (int64_t)u * (M / 2) + i0 / 2;
+        a_code[j] = R == 4 ? src[0] | (uint32_t)src[1] << 8 : (R == 2 ? src[0] : src[0] >> (4 * (int)(i0 & 1)));
+        a_sfb[j] = foa_sf[metis_sf_offset(u, i0 / 16, M / 16, foa_layout)];
       }
-      if (i < N) wt[j] = rcat[i * kc + kb + u];
+      if (in_n)
+#pragma unroll
+        for (int r = 0; r < R; ++r) wt[j][r] = rcat[(i0 + r) * kc + kb + u];
     }
     if (u < kb) {
       sb_v[j] = sb[u];
-      if (i < M) g1[j] = lcat[i * kc + u];
-      if (i < N) {
-        b_byte[j] = fob_codes[(int64_t)u * (N / 2) + i / 2];
-        b_sfb[j] = fob_sf[metis_sf_offset(u, i / 16, N / 16, fob_layout)];
+      if (in_m)
+#pragma unroll
+        for (int r = 0; r < R; ++r) g1[j][r] = lcat[(i0 + r) * kc + u];
+      if (in_n) {
+        const uint8_t* src = fob_codes + (int64_t)u * (N / 2) + i0 / 2;
+        b_code[j] = R == 4 ? src[0] | (uint32_t)src[1] << 8 : (R == 2 ? src[0] : src[0] >> (4 * (int)(i0 & 1)));
+        b_sfb[j] = fob_sf[metis_sf_offset(u, i0 / 16, N / 16, fob_layout)];
       }
     }
   }
   const float tsa = ka ? *foa_ts : 0.0f, tsb = kb ? *fob_ts : 0.0f;
   const float inv_alpha = lx != nullptr ? 1.0f / ((*res_a_ts) * (*res_b_ts)) : 0.0f;
-  for (int o = tid; o < ka * kb; o += 256) ps[o / kb][o % kb] = pm[o];
+  for (int o = warp; o < ka; o += 32) {                     // four rows of P in flight
+    float v[4][J];
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int j = 0; j < J; ++j) v[b][j] = o + 8 * b < ka && lane + 32 * j < kb ? pm[(o + 8 * b) * kb + lane + 32 * j] : 0.0f;
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int j = 0; j < J; ++j) if (o + 8 * b < ka) ps[o + 8 * b][lane + 32 * j] = v[b][j];
+  }
+  float raw_a[J][R], raw_b[J][R];                           // the factors as E2M1 x E4M3 products (exact in FP16), before any FP32 scale
+  auto dequantize = [](uint32_t code, uint32_t sf, float (&out)[R]) {
+    const __half2 sc = __float2half2_rn(metis_e4m3_value(sf));
+#pragma unroll
+    for (int r = 0; r < R; r += 2) {
+      const float2 v = __half22float2(__hmul2(e2m1x2_to_half2(code >> (4 * r)), sc));
+      out[r] = v.x;
+      if (r + 1 < R) out[r + 1] = v.y;
+    }
+  };
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    dequantize(a_code[j], a_sfb[j], raw_a[j]);
+    dequantize(b_code[j], b_sfb[j], raw_b[j]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) fa[warp][lane + 32 * j][r] = raw_a[j][r] * tsa * sa_v[j];
+  }
   __syncthreads();
-  if (i < M) {
+  if (in_m) {
+#pragma unroll 4
+    for (int u = 0; u < ka; ++u) {
+      float fr[R];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int u = lane + 32 * j;
-      if (u < ka) {
-        const float raw = deq_of(a_byte[j], a_sfb[j], i);
-        const float v = raw * tsa * sa_v[j];
-        lraw[warp][u] = raw;
-        fa[warp][u] = v;
-        lrow[warp][kb + u] = v;
-        lcat[i * kc + kb + u] = v;
-      }
-    }
-    __syncwarp();
+      for (int r = 0; r < R; ++r) fr[r] = fa[warp][u][r];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int t = lane + 32 * j;
-      if (t < kb) {
-        float v = g1[j];
-        for (int u = 0; u < ka; ++u) v = fmaf(fa[warp][u], ps[u][t], v);
-        v *= sb_v[j];
-        lrow[warp][t] = v;
-        lcat[i * kc + t] = v;
-      }
+      for (int j = 0; j < J; ++j)
+        {
+          const float p = ps[u][lane + 32 * j];
+#pragma unroll
+          for (int r = 0; r < R; ++r) g1[j][r] = fmaf(fr[r], p, g1[j][r]);
+        }
     }
   }
-  if (i < N) {
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int t = lane + 32 * j;
-      if (t < kb) {
-        const float raw = deq_of(b_byte[j], b_sfb[j], i);
-        const float v = raw * tsb;
-        rraw[warp][t] = raw;
-        rrow[warp][t] = v;
-        rcat[i * kc + t] = v;
-      }
-      if (t < ka) rrow[warp][kb + t] = wt[j];
-    }
-  }
-  if (lx == nullptr) return;
-  // BF16 operands of the in-accumulator correction, zero padded to kx columns.  A dequantized factor entry is an
-  // E2M1 x E4M3 product (six significant bits): with its FP32 scales moved to the other operand it is exact in BF16
-  // and needs no low part, so each of the two rank-k terms costs two column groups instead of three:
-  //   Lx = [ A hi | A lo | Fa | Fa ],  A  = (G1 + Fo_a sa P) sb ts_b / alpha     (k_b columns), Fa = Fo_a / ts_a (k_a)
-  //   Rx = [ Fb   | Fb   | B hi | B lo ],  Fb = Fo_b / ts_b (k_b),  B = Wt sa ts_a / alpha          (k_a columns)
-  __syncwarp();
   const float l_scale = tsb * inv_alpha, r_scale = tsa * inv_alpha;
-  for (int c = lane; c < kx; c += 32) {
-    float lo_ = 0.0f, ro_ = 0.0f;
-    if (c < 2 * kb) {
-      const int t = c < kb ? c : c - kb;
-      if (i < M) {
-        const float v = lrow[warp][t] * l_scale;
-        const float h = __bfloat162float(__float2bfloat16_rn(v));
-        lo_ = c < kb ? h : v - h;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int64_t i = i0 + r;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const int u = lane + 32 * j;
+      const float a = g1[j][r] * sb_v[j];
+      if (lx == nullptr) {
+        if (in_m && u < kb) lcat[i * kc + u] = a;
+        if (in_m && u < ka) lcat[i * kc + kb + u] = raw_a[j][r] * tsa * sa_v[j];
+        if (in_n && u < kb) rcat[i * kc + u] = raw_b[j][r] * tsb;
+        continue;
       }
-      if (i < N) ro_ = rraw[warp][t];
-    } else if (c < 2 * kc) {
-      const int u0 = c - 2 * kb, u = u0 < ka ? u0 : u0 - ka;
-      if (i < M) lo_ = lraw[warp][u];
-      if (i < N) {
-        const float v = rrow[warp][kb + u] * sa[u] * r_scale;
-        const float h = __bfloat162float(__float2bfloat16_rn(v));
-        ro_ = u0 < ka ? h : v - h;
+      if (u < kb) {
+        if (in_m) {
+          const float v = a * l_scale;
+          const __nv_bfloat16 h = __float2bfloat16_rn(v);
+          lx[i * kx + u] = h;
+          lx[i * kx + kb + u] = __float2bfloat16_rn(v - __bfloat162float(h));
+        }
+        if (in_n) rx[i * kx + u] = rx[i * kx + kb + u] = __float2bfloat16_rn(raw_b[j][r]);
+      }
+      if (u < ka) {
+        if (in_m) lx[i * kx + 2 * kb + u] = lx[i * kx + 2 * kb + ka + u] = __float2bfloat16_rn(raw_a[j][r]);
+        if (in_n) {
+          const float v = wt[j][r] * sa_v[j] * r_scale;
+          const __nv_bfloat16 h = __float2bfloat16_rn(v);
+          rx[i * kx + 2 * kb + u] = h;
+          rx[i * kx + 2 * kb + ka + u] = __float2bfloat16_rn(v - __bfloat162float(h));
+        }
       }
     }
-    if (i < M) lx[i * kx + c] = __float2bfloat16_rn(lo_);
-    if (i < N) rx[i * kx + c] = __float2bfloat16_rn(ro_);
+    for (int c = 2 * kc + lane; c < kx && lx != nullptr; c += 32) {
+      if (in_m) lx[i * kx + c] = __float2bfloat16_rn(0.0f);
+      if (in_n) rx[i * kx + c] = __float2bfloat16_rn(0.0f);
+    }
   }
 }
 
@@ -160,12 +196,15 @@ lowrank_finish_kernel(int64_t M, int64_t N, int ka, int kb,
 //   lowrank_bf16_kernel        the BF16 correction operands, eight columns per thread
 constexpr int LW_MAXK = 256;
 __global__ void __launch_bounds__(256)
-lowrank_deq_wide_kernel(int64_t M, int64_t N, int ka, int kb,
-                        const uint8_t* foa_codes, const uint8_t* foa_sf, int foa_layout, const float* foa_ts, const float* sa,
-                        const uint8_t* fob_codes, const uint8_t* fob_sf, int fob_layout, const float* fob_ts,
-                        float* __restrict__ lcat, float* __restrict__ rcat,
-                        __nv_bfloat16* __restrict__ lx, __nv_bfloat16* __restrict__ rx, int kx) {
+lowrank_deq_wide_kernel(const __grid_constant__ FinishArgs first, const __grid_constant__ FinishArgs second) {
   metis_pdl_wait();
+  const FinishArgs& f = blockIdx.y == 0 ? first : second;
+  const int64_t M = f.M, N = f.N;
+  const int ka = f.ka, kb = f.kb, kx = f.kx, foa_layout = f.foa_layout, fob_layout = f.fob_layout;
+  const uint8_t *foa_codes = f.foa_codes, *foa_sf = f.foa_sf, *fob_codes = f.fob_codes, *fob_sf = f.fob_sf;
+  const float *foa_ts = f.foa_ts, *sa = f.sa, *fob_ts = f.fob_ts;
+  float *__restrict__ lcat = f.lcat, *__restrict__ rcat = f.rcat;
+  __nv_bfloat16 *__restrict__ lx = f.lx, *__restrict__ rx = f.rx;
   const int tid = threadIdx.x, kc = ka + kb;
   const int64_t i0 = (int64_t)blockIdx.x * 32 + 8 * (tid & 3);      // this thread's eight rows (M, N are multiples of 16)
   const float tsa = ka ? *foa_ts : 0.0f, tsb = kb ? *fob_ts : 0.0f;
@@ -202,8 +241,14 @@ lowrank_deq_wide_kernel(int64_t M, int64_t N, int ka, int kb,
 }
 
 __global__ void __launch_bounds__(256)
-lowrank_gemm_wide_kernel(int64_t M, int ka, int kb, const float* __restrict__ sb, const float* __restrict__ pm, float* __restrict__ lcat) {
+lowrank_gemm_wide_kernel(const __grid_constant__ FinishArgs first, const __grid_constant__ FinishArgs second) {
   metis_pdl_wait();
+  const FinishArgs& f = blockIdx.z == 0 ? first : second;
+  const int64_t M = f.M;
+  const int ka = f.ka, kb = f.kb;
+  const float *__restrict__ sb = f.sb, *__restrict__ pm = f.pm;
+  float* __restrict__ lcat = f.lcat;
+  if ((int)blockIdx.x * 64 >= kb || (int64_t)blockIdx.y * 64 >= M) return;
   constexpr int KT = 16;
   __shared__ __align__(16) float as[KT][68], bs[KT][68];   // [u][row], [u][column]
   const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, kc = ka + kb;
@@ -247,10 +292,14 @@ lowrank_gemm_wide_kernel(int64_t M, int ka, int kb, const float* __restrict__ sb
 // were written by lowrank_deq_wide_kernel.  One thread per row and eight columns (the group boundaries 2 k_b and
 // 2 (k_a + k_b) are multiples of eight).
 __global__ void __launch_bounds__(256)
-lowrank_bf16_kernel(int64_t M, int64_t N, int ka, int kb, int kx, const float* __restrict__ lcat, const float* __restrict__ rcat,
-                    const float* foa_ts, const float* __restrict__ sa, const float* fob_ts,
-                    __nv_bfloat16* __restrict__ lx, __nv_bfloat16* __restrict__ rx, const float* res_a_ts, const float* res_b_ts) {
+lowrank_bf16_kernel(const __grid_constant__ FinishArgs first, const __grid_constant__ FinishArgs second) {
   metis_pdl_wait();
+  const FinishArgs& f = blockIdx.y == 0 ? first : second;
+  const int64_t M = f.M, N = f.N;
+  const int ka = f.ka, kb = f.kb, kx = f.kx;
+  const float *__restrict__ lcat = f.lcat, *__restrict__ rcat = f.rcat, *foa_ts = f.foa_ts, *__restrict__ sa = f.sa, *fob_ts = f.fob_ts, *res_a_ts = f.res_a_ts, *res_b_ts = f.res_b_ts;
+  __nv_bfloat16 *__restrict__ lx = f.lx, *__restrict__ rx = f.rx;
+  if (lx == nullptr) return;                                // a layer of fewer than 256 rows beside one that has them
   const int64_t idx = (int64_t)blockIdx.x * 256 + threadIdx.x;
   const int64_t mx = M > N ? M : N;
   const int per_row = kx / 8, kc = ka + kb;
@@ -293,6 +342,7 @@ lowrank_bf16_kernel(int64_t M, int64_t N, int ka, int kb, int kx, const float* _
 __global__ void __launch_bounds__(256)
 rank_update_kernel(const float* __restrict__ y0, int64_t M, int64_t N, int kc, const float* __restrict__ lcat,
                    const float* __restrict__ rcat, void* __restrict__ out, int out_dtype, int64_t ldo) {
+  metis_pdl_wait();
   extern __shared__ __align__(16) float sm[];
   float* ls = sm;                       // [kc][64 + 4]
   float* rs = sm + kc * 68;
@@ -389,12 +439,6 @@ __device__ __forceinline__ void fg_fetch4(uint32_t dst, const T* src, bool in) {
   }
 }
 
-// the two E2M1 codes of the low byte as FP16 (exact)
-__device__ __forceinline__ __half2 e2m1x2_to_half2(uint32_t byte) {
-  uint32_t w;
-  asm("{ .reg .b8 t; cvt.u8.u32 t, %1; cvt.rn.f16x2.e2m1x2 %0, t; }" : "=r"(w) : "r"(byte));
-  return *reinterpret_cast<const __half2*>(&w);
-}
 
 // One entry of the contraction as FP32 multiply-adds in order.  An FP32 gradient that is infinite or rounds to infinity in BF16
 // leaves a NaN as its remainder, and sums that overflow may meet with opposite signs: an entry that came out as a NaN is
@@ -790,46 +834,63 @@ metis_status_t make_plan(const Side& a, const Side& b, void* ws, size_t ws_bytes
   return METIS_OK;
 }
 
-// Everything of a product that comes before its large GEMM: the three skinny products (straight into their
-// slots of the concatenated operands) and the finishing kernel.  The skinny products run on the handle's side
-// streams `side0` and `side0 + 1` beside `s` (the caller has made those streams wait for `s`'s past already).
-metis_status_t split_gemm_prologue(metis_context* ctx, const Side& a, const Side& b, const Plan& pl, int side0,
-                                   cudaStream_t s) {
-  if (pl.kc == 0) return METIS_OK;
-  const int64_t M = pl.M, N = pl.N;
-  const int ka = pl.ka, kb = pl.kb, kc = pl.kc;
-  if (!pl.fuse) METIS_TRY(metis_launch_gemm_tc(ctx, a.res, b.res, pl.y0, METIS_FP32, N, s));
-  cudaStream_t s1 = ctx->side[side0], s2 = ctx->side[side0 + 1];
-  if (kb) METIS_TRY(metis_launch_gemm_tc(ctx, a.res, b.fc, pl.lcat, METIS_FP32, kc, s));
-  if (ka) METIS_TRY(metis_launch_gemm_tc(ctx, b.res, a.fc, pl.rcat + kb, METIS_FP32, kc, s1));
-  if (ka && kb) METIS_TRY(metis_launch_gemm_tc(ctx, a.fc, b.fc, pl.pm, METIS_FP32, kb, s2));
-  METIS_TRY(metis_join(ctx, s, side0));
-  METIS_TRY(metis_join(ctx, s, side0 + 1));
-  const int64_t mx = M > N ? M : N;
-  if (ka > 64 || kb > 64) {
-    METIS_CUDA_TRY(metis_launch_pdl(lowrank_deq_wide_kernel, dim3((unsigned)metis_ceil_div(mx, 32)), dim3(256), 0, s,
-        M, N, ka, kb, ka ? a.fo->codes : nullptr, ka ? a.fo->scales : nullptr, ka ? a.fo->sf_layout : 0,
-        ka ? a.fo->tensor_scale : nullptr, a.sigma, kb ? b.fo->codes : nullptr, kb ? b.fo->scales : nullptr,
-        kb ? b.fo->sf_layout : 0, kb ? b.fo->tensor_scale : nullptr, pl.lcat, pl.rcat, pl.lx, pl.rx, pl.kx)); METIS_COUNT_LAUNCH();
-    if (kb) {
-      METIS_CUDA_TRY(metis_launch_pdl(lowrank_gemm_wide_kernel, dim3((unsigned)metis_ceil_div(kb, 64), (unsigned)metis_ceil_div(M, 64)), dim3(256), 0, s,
-          M, ka, kb, b.sigma, (const float*)pl.pm, pl.lcat)); METIS_COUNT_LAUNCH();
+// Everything of one or two products that comes before their large GEMMs: the skinny products (straight into their slots of the concatenated
+// operands; of a layer with fewer than 256 rows the residual product too) in one launch and the finishing kernels.
+metis_status_t split_gemm_prologue(metis_context* ctx, const Side* const* a, const Side* const* b, const Plan* const* pl, int n, cudaStream_t s) {
+  metis_gemm_job jobs[8];
+  FinishArgs f[2] = {};
+  int n_jobs = 0, n_f = 0;
+  bool wide = false, fused = false;
+  int64_t mx[2] = {0, 0};
+  int kx = 0, kb_max = 0, k_max = 0;
+  for (int i = 0; i < n; ++i) {
+    if (pl[i]->kc == 0) continue;
+    const Side &sa = *a[i], &sb = *b[i];
+    const Plan& p = *pl[i];
+    const int ka = p.ka, kb = p.kb, kc = p.kc;
+    if (!p.fuse) {
+      if (metis_ceil_div(p.M, 128) * metis_ceil_div(p.N, 64) <= ctx->sm_count) jobs[n_jobs++] = {sa.res, sb.res, p.y0, p.N, false};
+      else METIS_TRY(metis_launch_gemm_tc(ctx, sa.res, sb.res, p.y0, METIS_FP32, p.N, s));
     }
-    if (pl.lx != nullptr) {
-      METIS_CUDA_TRY(metis_launch_pdl(lowrank_bf16_kernel, dim3((unsigned)metis_ceil_div(mx * (pl.kx / 8), 256)), dim3(256), 0, s, M, N, ka, kb, pl.kx,
-          (const float*)pl.lcat, (const float*)pl.rcat, (const float*)(ka ? a.fo->tensor_scale : nullptr), (const float*)a.sigma,
-          (const float*)(kb ? b.fo->tensor_scale : nullptr),
-          pl.lx, pl.rx, (const float*)a.res->tensor_scale, (const float*)b.res->tensor_scale)); METIS_COUNT_LAUNCH();
+    if (kb) jobs[n_jobs++] = {sa.res, sb.fc, p.lcat, kc, true};
+    if (ka) jobs[n_jobs++] = {sb.res, sa.fc, p.rcat + kb, kc, true};
+    if (ka && kb) jobs[n_jobs++] = {sa.fc, sb.fc, p.pm, kb, true};
+    FinishArgs& o = f[n_f];
+    o.M = p.M; o.N = p.N; o.ka = ka; o.kb = kb; o.kx = p.kx;
+    if (ka) { o.foa_codes = sa.fo->codes; o.foa_sf = sa.fo->scales; o.foa_layout = sa.fo->sf_layout; o.foa_ts = sa.fo->tensor_scale; }
+    if (kb) { o.fob_codes = sb.fo->codes; o.fob_sf = sb.fo->scales; o.fob_layout = sb.fo->sf_layout; o.fob_ts = sb.fo->tensor_scale; }
+    o.sa = sa.sigma; o.sb = sb.sigma; o.pm = p.pm; o.lcat = p.lcat; o.rcat = p.rcat; o.lx = p.lx; o.rx = p.rx;
+    o.res_a_ts = sa.res->tensor_scale; o.res_b_ts = sb.res->tensor_scale;
+    mx[n_f] = p.M > p.N ? p.M : p.N;
+    wide |= ka > 64 || kb > 64; fused |= p.lx != nullptr;
+    if (p.kx > kx) kx = p.kx;
+    if (kb > kb_max) kb_max = kb;
+    k_max = ka > k_max ? ka : k_max; k_max = kb > k_max ? kb : k_max;
+    ++n_f;
+  }
+  if (n_f == 0) return METIS_OK;
+  METIS_TRY(metis_launch_gemm_group(ctx, jobs, n_jobs, s));
+  const int64_t longest = mx[0] > mx[1] ? mx[0] : mx[1];
+  if (wide) {
+    METIS_CUDA_TRY(metis_launch_pdl(lowrank_deq_wide_kernel, dim3((unsigned)metis_ceil_div(longest, 32), (unsigned)n_f), dim3(256), 0, s, f[0], f[1])); METIS_COUNT_LAUNCH();
+    if (kb_max) {
+      METIS_CUDA_TRY(metis_launch_pdl(lowrank_gemm_wide_kernel, dim3((unsigned)metis_ceil_div(kb_max, 64), (unsigned)metis_ceil_div(longest, 64), (unsigned)n_f), dim3(256), 0, s,
+                                      f[0], f[1])); METIS_COUNT_LAUNCH();
     }
-    METIS_CUDA_TRY(cudaGetLastError());
+    if (fused) {
+      METIS_CUDA_TRY(metis_launch_pdl(lowrank_bf16_kernel, dim3((unsigned)metis_ceil_div(longest * (kx / 8), 256), (unsigned)n_f), dim3(256), 0, s, f[0], f[1])); METIS_COUNT_LAUNCH();
+    }
     return METIS_OK;
   }
-  METIS_CUDA_TRY(metis_launch_pdl(lowrank_finish_kernel, dim3((unsigned)metis_ceil_div(mx, 8)), dim3(256), 0, s,
-      M, N, ka, kb, ka ? a.fo->codes : nullptr, ka ? a.fo->scales : nullptr, ka ? a.fo->sf_layout : 0,
-      ka ? a.fo->tensor_scale : nullptr, a.sigma, kb ? b.fo->codes : nullptr, kb ? b.fo->scales : nullptr,
-      kb ? b.fo->sf_layout : 0, kb ? b.fo->tensor_scale : nullptr, b.sigma, pl.pm, pl.lcat, pl.rcat, pl.lx, pl.rx, pl.kx,
-      a.res->tensor_scale, b.res->tensor_scale)); METIS_COUNT_LAUNCH();
-  METIS_CUDA_TRY(cudaGetLastError());
+  // rows per warp: one while all rows together are not more than eight warps for every scheduler
+  const int64_t rows = mx[0] + mx[1], per = 32ll * ctx->sm_count;
+#define METIS_FINISH_J(R, J) METIS_CUDA_TRY(metis_launch_pdl((lowrank_finish_kernel<R, J>), dim3((unsigned)(n_first + metis_ceil_div(mx[1], 8 * (R)))), dim3(256), 0, s, f[0], f[1], (int)n_first))
+#define METIS_FINISH(R) { const int64_t n_first = metis_ceil_div(mx[0], 8 * (R)); if (k_max <= 32) METIS_FINISH_J(R, 1); else METIS_FINISH_J(R, 2); METIS_COUNT_LAUNCH(); }
+  if (rows <= per + per / 2) METIS_FINISH(1)
+  else if (rows <= 3 * per) METIS_FINISH(2)
+  else METIS_FINISH(4)
+#undef METIS_FINISH_J
+#undef METIS_FINISH
   return METIS_OK;
 }
 
@@ -842,8 +903,7 @@ metis_status_t split_gemm_main(metis_context* ctx, const Side& a, const Side& b,
   }
   dim3 grid((unsigned)metis_ceil_div(pl.N, 64), (unsigned)metis_ceil_div(pl.M, 64));
   const size_t smem = sizeof(float) * 2 * pl.kc * 68;
-  rank_update_kernel<<<grid, 256, smem, s>>>(pl.y0, pl.M, pl.N, pl.kc, pl.lcat, pl.rcat, d, d_dtype, ldd); METIS_COUNT_LAUNCH();
-  METIS_CUDA_TRY(cudaGetLastError());
+  METIS_CUDA_TRY(metis_launch_pdl(rank_update_kernel, grid, dim3(256), smem, s, (const float*)pl.y0, pl.M, pl.N, pl.kc, (const float*)pl.lcat, (const float*)pl.rcat, d, d_dtype, ldd)); METIS_COUNT_LAUNCH();
   return METIS_OK;
 }
 
@@ -851,8 +911,9 @@ metis_status_t split_gemm(metis_context* ctx, const Side& a, const Side& b, void
                           size_t ws_bytes, cudaStream_t s) {
   Plan pl;
   METIS_TRY(make_plan(a, b, ws, ws_bytes, &pl));
-  METIS_TRY(metis_fork(ctx, s, 2));
-  METIS_TRY(split_gemm_prologue(ctx, a, b, pl, 0, s));
+  const Side *pa = &a, *pb = &b;
+  const Plan* pp = &pl;
+  METIS_TRY(split_gemm_prologue(ctx, &pa, &pb, &pp, 1, s));
   return split_gemm_main(ctx, a, b, pl, d, d_dtype, ldd, s);
 }
 
@@ -920,20 +981,17 @@ metis_status_t metis_linear_bwd(metis_handle_t h, const metis_operand_t* dy, con
   Side wa{&dy->res_by_rows, &dy->left_q, &dy->right_q, dy->sigma, dy->k};
   Side wb = x ? Side{&x->res_by_rows, &x->left_q, &x->right_q, x->sigma, x->k} : Side{};
   if (dx && dw) {
-    // Both products: with room for two sets of intermediates, everything that precedes the weight gradient's
-    // large GEMM runs on a side stream underneath the input gradient.
+    // Both products: with room for two sets of intermediates, everything that precedes the large GEMMs goes together.
     Plan pd, pw;
     METIS_TRY(make_plan(da, db, ws, ws_bytes, &pd));
     const size_t off = pd.bytes;
     const metis_status_t st = make_plan(wa, wb, ws ? reinterpret_cast<unsigned char*>(ws) + off : nullptr,
                                         ws_bytes > off ? ws_bytes - off : 0, &pw);
     if (st == METIS_OK) {
-      // all six skinny products at once (a large GEMM, once resident, leaves no SM to a kernel that comes later)
-      METIS_TRY(metis_fork(h, s, METIS_N_SIDE));
-      METIS_TRY(split_gemm_prologue(h, wa, wb, pw, 3, h->side[2]));
-      METIS_TRY(split_gemm_prologue(h, da, db, pd, 0, s));
+      const Side *as[2] = {&da, &wa}, *bs[2] = {&db, &wb};
+      const Plan* ps[2] = {&pd, &pw};
+      METIS_TRY(split_gemm_prologue(h, as, bs, ps, 2, s));
       METIS_TRY(split_gemm_main(h, da, db, pd, dx, dx_dtype, lddx, s));
-      METIS_TRY(metis_join(h, s, 2));
       METIS_TRY(split_gemm_main(h, wa, wb, pw, dw, dw_dtype, lddw, s));
     } else if (st == METIS_ERR_WORKSPACE) {
       METIS_TRY(split_gemm(h, da, db, dx, dx_dtype, lddx, ws, ws_bytes, s));

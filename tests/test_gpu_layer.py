@@ -311,6 +311,34 @@ def test_ragged_layer_through_the_two_cta_gemm(ctx):
                 "dw": rel_fro(dw.cpu().numpy(), olay.linear_wgrad(dq, xq))}, (xo, xq), (wo, wq), (do, dq))
 
 
+@pytest.mark.parametrize("l,n,m,kd,kx,kw", [
+    (64, 192, 64, 4, 4, 4),               # one K block of each product, a residual product with an odd number of 64-column tiles
+    (128, 448, 192, 8, 12, 4),            # residual product in the group, unequal ranks
+    (320, 2112, 576, 36, 32, 40),         # 33-vector remainders of the finishing kernel, ragged K
+    (512, 256, 4160, 16, 16, 16),         # contractions of 17 K blocks divided by eight, of one and of two beside them
+    (4096, 256, 320, 64, 48, 64),         # more than one CTA per SM, two rows per warp of the finishing kernel
+    (9216, 256, 256, 16, 20, 12),         # four rows per warp
+    (256, 512, 768, 72, 64, 64),          # a rank above 64 beside ranks below it
+])
+def test_skinny_products_in_one_launch(ctx, l, n, m, kd, kx, kw):
+    """Forward and both gradients against float64 products of the library's own codes (exact codes, FP32 sums: 2e-5)."""
+    from gpu_util import to_dev_bf16, rel_fro
+    B, h = ctx
+    t = [synth.planted(r, c, 8, 100 * s * (np.sqrt(r) + np.sqrt(c)), 10 * s * (np.sqrt(r) + np.sqrt(c)), s, sd)[0]
+         for r, c, s, sd in ((l, m, 1.0, 71), (n, m, 0.02, 72), (l, n, 1e-4, 73))]
+    xo, wo, do = (h.split(to_dev_bf16(a), k, 4, sketch=B.SKETCH_FULL, seed=i) for i, (a, k) in enumerate(zip(t, (kx, kw, kd))))
+    y = h.linear_fwd(xo, wo)
+    dx, dw = h.linear_bwd(do, xo, wo)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    lx, rxc, rxr = _oracle_from_gpu_operand(xo, kx)
+    lw, rwc, rwr = _oracle_from_gpu_operand(wo, kw)
+    ld, rdc, rdr = _oracle_from_gpu_operand(do, kd)
+    assert rel_fro(y.cpu().numpy(), (lx + rxc) @ (lw + rwc).T) < 2e-5
+    assert rel_fro(dx.cpu().numpy(), (ld + rdc) @ (lw + rwr)) < 2e-5
+    assert rel_fro(dw.cpu().numpy(), (ld + rdr).T @ (lx + rxr)) < 2e-5
+
+
 def test_bf16_output(ctx):
     from gpu_util import to_dev_bf16, rel_fro
     B, h = ctx
