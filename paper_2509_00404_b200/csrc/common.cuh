@@ -76,6 +76,41 @@ static inline cudaError_t metis_launch_pdl(void (*kernel)(KArgs...), dim3 grid, 
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// The same for clusters of `csize` consecutive CTAs along one axis of the grid (0: x, 1: y).
+template <typename... KArgs, typename... Args>
+static inline cudaError_t metis_launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int axis, int csize, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = axis == 0 ? (unsigned)csize : 1u; at[1].val.clusterDim.y = axis == 1 ? (unsigned)csize : 1u; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Rank of this CTA in its cluster and the cluster's size; the cluster's barrier (every thread of every CTA); the shared::cluster address of the
+// same shared-memory offset in another CTA.
+__device__ __forceinline__ uint32_t metis_cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t metis_cluster_size() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void metis_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t metis_map_to_rank(uint32_t local_addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
+  return r;
+}
+
 #define METIS_CUDA_TRY(expr)                         \
   do {                                               \
     cudaError_t e__ = (expr);                        \
@@ -261,11 +296,13 @@ int metis_coeff_slices(int64_t rows, int64_t cols, int* chunks_per_slice);
 bool metis_coeff_tc_usable(const void* x, const void* bs, int64_t cols, int kp);
 metis_status_t metis_launch_coeff_tc(metis_context* ctx, const void* x, int64_t rows, int64_t cols, const void* bs, int kp,
                                      float* part, float* amax, int raw, cudaStream_t s);
+// what a split reports in the status word: an amax that is not finite, an eigenvalue that is not finite
+struct metis_split_checks { const float* amax; const double* evals; int k; uint32_t* status; };
 // keys (optional): one key per vector, bit 0 set where the pair has to be flipped (left and right in place) before it is quantized
 metis_status_t metis_launch_quantize_factors(float* left, int64_t rows, float* right, int64_t cols, int k, int rounding,
                                              uint64_t seed, const float* amax_left, const float* amax_right,
                                              const metis_nvfp4_t* lq, const metis_nvfp4_t* rq, cudaStream_t s,
-                                             const unsigned long long* keys = nullptr);
+                                             const unsigned long long* keys = nullptr, const metis_split_checks* checks = nullptr);
 metis_status_t metis_launch_amax_check(metis_context* ctx, const float* amax, cudaStream_t s);
 metis_status_t metis_launch_quantize_rht(metis_context* ctx, const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, int rounding, uint64_t seed,
                                          uint32_t stream_id, const metis_nvfp4_t* out, float* amax_ws, cudaStream_t s);

@@ -261,21 +261,6 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_consta
   }
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// shared::cluster address of the same shared-memory offset in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t local_addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_addr), "r"(rank));
-  return r;
-}
-
 // =================================================================================================
 // The skinny products of one or two split products (rank x rank, residual x factor) in one launch: FP32 results of at most a few hundred
 // columns whose time is the latency of a CTA's K loop and of the launches.  A CTA takes one 128 x BLOCK_N tile and
@@ -333,7 +318,7 @@ gemm_nvfp4_group_kernel(const __grid_constant__ GroupArgs args) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   uint32_t csize;
   asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(csize));
-  const int rank = (int)cluster_rank(), cluster = (int)(blockIdx.x / csize);
+  const int rank = (int)metis_cluster_rank(), cluster = (int)(blockIdx.x / csize);
   int which = 0;
   while (which + 1 < args.n && cluster >= args.p[which + 1].first_cluster) ++which;
   const GroupProblem& g = args.p[which];
@@ -440,7 +425,7 @@ gemm_nvfp4_group_kernel(const __grid_constant__ GroupArgs args) {
   }
   if (csize > 1) {                                           // (the same for every CTA of the grid)
     __syncwarp();
-    cluster_sync();
+    metis_cluster_sync();
     if (split > 1 && active && warp >= 2) {
       // rows part * 128 / split ... of the tile, the parts added in their order; consecutive threads: consecutive columns
       const int rows = BLOCK_M >> g.log_split, ncols = min(BLOCK_N, g.N - nb * BLOCK_N), per_row = (ncols + 3) / 4;
@@ -455,7 +440,7 @@ gemm_nvfp4_group_kernel(const __grid_constant__ GroupArgs args) {
         for (int u = 0; u < 8; ++u) {
           x[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
           if (u < split)
-            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[u].x), "=f"(x[u].y), "=f"(x[u].z), "=f"(x[u].w) : "r"(map_to_rank(at, first + (uint32_t)u)));
+            asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[u].x), "=f"(x[u].y), "=f"(x[u].z), "=f"(x[u].w) : "r"(metis_map_to_rank(at, first + (uint32_t)u)));
         }
         float4 v = x[0];
 #pragma unroll
@@ -467,7 +452,7 @@ gemm_nvfp4_group_kernel(const __grid_constant__ GroupArgs args) {
       }
     }
     __syncwarp();
-    cluster_sync();                                          // the others may still be reading
+    metis_cluster_sync();                                          // the others may still be reading
   }
   tc_fence_before();
   __syncthreads();
@@ -599,7 +584,7 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   volatile int* dead = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_rank();
+  const uint32_t rank = metis_cluster_rank();
   const bool leader = rank == 0;
   const int pair = blockIdx.x >> 1, num_pairs = gridDim.x >> 1;
   const int num_m = (g.M + TILE_M - 1) / TILE_M, num_n = (g.N + TILE_N - 1) / TILE_N;
@@ -635,10 +620,10 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
     *dead = 0;
     fence_barrier_init();
   }
-  cluster_sync();
+  metis_cluster_sync();
   if (warp == 1) tmem_alloc2(smem_u32(tmem_slot), TMEM_COLS);
   tc_fence_before();
-  cluster_sync();
+  metis_cluster_sync();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   // everything above touched only this CTA's shared and tensor memory: it may overlap the previous kernel's tail
@@ -668,7 +653,7 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
         for (int kb = 0; kb < num_kb; ++kb) {
           if (!mbar_wait(empty_bar(s), ph ^ 1u, g.dev_status, dead)) { ok = false; break; }
           if (elect_one()) {
-            const uint32_t bar = map_to_rank(full_bar(s), 0u);
+            const uint32_t bar = metis_map_to_rank(full_bar(s), 0u);
             if (kb >= num_fp4_kb) {                           // BF16 correction box: 128 rows x 64 elements each
               if (leader) mbar_expect_tx(full_bar(s), 2u * (uint32_t)(A_BYTES + B_BYTES));
               tma_load_2d_pair(a_addr(s), &map_l, (kb - num_fp4_kb) * 64, a_row, bar);
@@ -854,7 +839,7 @@ gemm_nvfp4_2cta_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_c
   if (*dead) {
     for (int i = 0; i < 2000; ++i) __nanosleep(1000);
   }
-  cluster_sync();                                             // the peer may still read this CTA's shared memory until here
+  metis_cluster_sync();                                             // the peer may still read this CTA's shared memory until here
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc2(tmem_base, TMEM_COLS);
@@ -909,15 +894,8 @@ metis_status_t launch(metis_context* ctx, const metis_nvfp4_t* a, const metis_nv
 
 template <int BLOCK_N, int STAGES>
 metis_status_t launch_group(metis_context* ctx, const GroupArgs& args, int clusters, int csize, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(clusters * csize)); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = GroupCfg<BLOCK_N, STAGES>::SMEM_BYTES; cfg.stream = s;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = (unsigned)csize; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 2;
-  METIS_CUDA_TRY(cudaLaunchKernelEx(&cfg, gemm_nvfp4_group_kernel<BLOCK_N, STAGES>, args)); METIS_COUNT_LAUNCH();
+  METIS_CUDA_TRY(metis_launch_pdl_cluster(gemm_nvfp4_group_kernel<BLOCK_N, STAGES>, dim3((unsigned)(clusters * csize)), dim3(NUM_THREADS),
+                                          GroupCfg<BLOCK_N, STAGES>::SMEM_BYTES, s, 0, csize, args)); METIS_COUNT_LAUNCH();
   return METIS_OK;
 }
 

@@ -496,9 +496,17 @@ metis_status_t metis_launch_quantize_rht(metis_context* ctx, const void* x, int 
 // (keys: the sign keys of the vectors, or nullptr; x is then flipped where the key says so)
 struct RowblocksJob { float* x; int64_t ld; metis_qt::QuantParams p; const float* tscale_src; float* ts_out; const unsigned long long* keys; };
 __global__ void __launch_bounds__(256)
-quantize_rowblocks_pair_kernel(RowblocksJob a, RowblocksJob b) {
+quantize_rowblocks_pair_kernel(RowblocksJob a, RowblocksJob b, metis_split_checks checks) {
   const RowblocksJob& j = blockIdx.y == 0 ? a : b;
   metis_pdl_wait();
+  if (checks.status != nullptr && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 32) {
+    // device-detected conditions of the split that these factors belong to (amax is kept as an ordered bit pattern, so a NaN ranks above every number)
+    uint32_t bits = 0u;
+    if (threadIdx.x == 0 && !(fabsf(*checks.amax) <= 3.0e38f)) bits |= METIS_DEV_NONFINITE;
+    for (int i = threadIdx.x; i < checks.k; i += 32)
+      if (!(fabs(checks.evals[i]) <= 1.0e300)) bits |= METIS_DEV_NUMERIC;
+    if (bits) atomicOr(checks.status, bits);
+  }
   rowblocks_body(j.x, j.ld, j.p, j.tscale_src, 1, j.ts_out, j.keys, j.x);
 }
 
@@ -545,7 +553,8 @@ metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int
 // tensor scale from each tensor's own amax) in one launch.
 metis_status_t metis_launch_quantize_factors(float* left, int64_t rows, float* right, int64_t cols, int k, int rounding,
                                              uint64_t seed, const float* amax_left, const float* amax_right,
-                                             const metis_nvfp4_t* lq, const metis_nvfp4_t* rq, cudaStream_t s, const unsigned long long* keys) {
+                                             const metis_nvfp4_t* lq, const metis_nvfp4_t* rq, cudaStream_t s, const unsigned long long* keys,
+                                             const metis_split_checks* checks) {
   using namespace metis_qt;
   if (k <= 0 || k > 256 || rows % 16 || cols % 16) return METIS_ERR_SHAPE;
   RowblocksJob a{}, b{};
@@ -559,6 +568,6 @@ metis_status_t metis_launch_quantize_factors(float* left, int64_t rows, float* r
   const int64_t pad_a = a.p.c_layout == METIS_SF_TILED ? (k + 127) / 128 * 128 : k, pad_b = b.p.c_layout == METIS_SF_TILED ? (k + 127) / 128 * 128 : k;
   const int64_t work_a = pad_a * (rows / 16), work_b = pad_b * (cols / 16);
   const unsigned gx = (unsigned)metis_ceil_div(work_a > work_b ? work_a : work_b, 256);
-  METIS_CUDA_TRY(metis_launch_pdl(quantize_rowblocks_pair_kernel, dim3(gx, 2), dim3(256), (size_t)0, s, a, b)); METIS_COUNT_LAUNCH();
+  METIS_CUDA_TRY(metis_launch_pdl(quantize_rowblocks_pair_kernel, dim3(gx, 2), dim3(256), (size_t)0, s, a, b, checks != nullptr ? *checks : metis_split_checks{})); METIS_COUNT_LAUNCH();
   return METIS_OK;
 }

@@ -24,67 +24,75 @@ __device__ __forceinline__ void lower_tile(int o, int& ti, int& tj) {
   tj = o - ti * (ti + 1) / 2;
 }
 
-// In-place Cholesky factorisation of the lower triangle of Y (n x n, n8 = n rounded up to a multiple of eight, row pitch P doubles,
-// rows and columns up to n8 must exist and be zero beyond n), called by all nthr >= n8 - 8 threads of the CTA.
-// Panels of eight columns: every warp factorises the panel's diagonal block in registers (lane = row; a column step is one
-// pivot broadcast, one reciprocal and one multiply-add deep, without a barrier) and carries 32 rows below it along; then all warps subtract
-// the panel's rank-8 product from the trailing tiles on the FP64 tensor cores, two tiles at a time.  (One barrier per
-// column with the matrix spread over 256 threads' registers took 800 cycles a column.)  A pivot not above `tol` marks a dependent column:
-// it takes no part in the updates and ends as a zero column with inv_out[j] = 0; otherwise inv_out[j] = 1 / L[j][j].
-// *dmin_out (optional): the smallest accepted pivot.  tid, bar: index within the group of nthr threads and the group's barrier.
+// In-place Cholesky factorisation of the lower triangle of Y (n x n, n8 = n rounded up to a multiple of eight, row pitch P doubles (even),
+// rows and columns up to n8 must exist and be zero beyond n), called by all nthr threads (at least two warps and n8 - 8 threads).
+// Panels of eight columns: every thread factorises the panel's diagonal block for itself in registers (a column is a reciprocal root and two operations
+// deep, without an exchange: with a row of the block per lane it was a broadcast of the pivot deeper and 36 double shuffles a panel, 2200 cycles with the
+// trailing update against 1500) and carries one row below it along; then all warps but the last, which stores the block, subtract the panel's rank-8 product from the trailing tiles
+// on the FP64 tensor cores, two tiles at a time.  (One barrier per column with the matrix spread over 256 threads' registers took 800 cycles a
+// column.)  A pivot not above `tol` marks a dependent column: it takes no part in the updates and ends as a zero column with
+// inv_out[j] = 0; otherwise inv_out[j] = 1 / L[j][j].  *dmin_out (optional): the smallest accepted pivot, to 20 bits from below.  tid, bar: index within the group of nthr
+// threads and the group's barrier.
 template <int P, class Bar>
 __device__ __forceinline__ void group_cholesky(double* Y, int n, double tol, double* inv_out, double* dmin_out, int tid, int nthr, Bar bar) {
   const int lane = tid & 31, warp = tid >> 5, n_warps = nthr >> 5;
   const int n8 = (n + 7) & ~7, g = lane >> 2, q = lane & 3;
-  double dmin = 1e300;
+  int dmin = 0x7FE00000;                                // of the smallest accepted pivot, its high word
   for (int c0 = 0; c0 < n8; c0 += 8) {
-    const int r = c0 + 8 + 32 * warp + lane, rd_ = c0 + (lane & 7);             // a row below the block, a row of the block
-    double vd[8], inv = 0.0;
-    const bool busy = warp == 0 || c0 + 8 + 32 * warp < n8;
+    const int r = c0 + 8 + 32 * warp + lane;            // a row below the block
+    const bool busy = warp == n_warps - 1 || c0 + 8 + 32 * warp < n8;
+    double a[8][8], inv[8];                             // the block's lower triangle
     if (busy) {
       double v[8];
 #pragma unroll
-      for (int c = 0; c < 8; ++c) { vd[c] = Y[rd_ * P + c0 + c]; v[c] = r < n8 ? Y[r * P + c0 + c] : 0.0; }
-      double my_pivot = 0.0;                            // lane j < 8: pivot of column c0 + j
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int c = 0; c <= i; c += 2) {
+          const double2 x = *reinterpret_cast<const double2*>(Y + (c0 + i) * P + c0 + c);
+          a[i][c] = x.x;
+          if (c < i) a[i][c + 1] = x.y;
+        }
+#pragma unroll
+      for (int c = 0; c < 8; ++c) v[c] = r < n8 ? Y[r * P + c0 + c] : 0.0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const double d = __shfl_sync(0xFFFFFFFFu, vd[j], j);
-        const double rd = d > tol ? rcp_newton(d) : 0.0;
-        if ((lane & 7) == j) my_pivot = d;
-        const double ld = vd[j] * rd, l = v[j] * rd;
+        const double d = a[j][j], rs = rsqrt_newton(d);  // (selected, not branched around)
+        const bool on = d > tol;
+        inv[j] = on ? rs : 0.0;
+        dmin = min(dmin, on ? __double2hiint(d) : 0x7FE00000);
+#pragma unroll
+        for (int i = j; i < 8; ++i) a[i][j] *= inv[j];
+        v[j] *= inv[j];
 #pragma unroll
         for (int c = j + 1; c < 8; ++c) {
-          const double u = __shfl_sync(0xFFFFFFFFu, vd[j], c);
-          vd[c] = fma(-ld, u, vd[c]);
-          v[c] = fma(-l, u, v[c]);
+#pragma unroll
+          for (int i = c; i < 8; ++i) a[i][c] = fma(-a[i][j], a[c][j], a[i][c]);
+          v[c] = fma(-v[j], a[c][j], v[c]);
         }
       }
-      const bool ok = my_pivot > tol;
-      inv = ok ? rsqrt_newton(my_pivot) : 0.0;
-      if (ok) dmin = fmin(dmin, my_pivot);
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const double ic = __shfl_sync(0xFFFFFFFFu, inv, c);
-        vd[c] *= ic;
-        if (r < n8) Y[r * P + c0 + c] = v[c] * ic;
-      }
+      for (int c = 0; c < 8; ++c) if (r < n8) Y[r * P + c0 + c] = v[c];
     }
     bar();                                    // the block has been read by every warp: its factor may be stored
-    if (warp == 0 && lane < 8) {
-      if (c0 + lane < n) inv_out[c0 + lane] = inv;
+    if (warp == n_warps - 1) {                          // while the others go on; every lane stores all of it (a row per lane: a branch of 200 cycles for each)
 #pragma unroll
-      for (int c = 0; c < 8; ++c) Y[rd_ * P + c0 + c] = c <= lane ? vd[c] : 0.0;
+      for (int i = 0; i < 8; ++i) {
+        if (c0 + i < n) inv_out[c0 + i] = inv[i];
+#pragma unroll
+        for (int c = 0; c < 8; c += 2)
+          *reinterpret_cast<double2*>(Y + (c0 + i) * P + c0 + c) = make_double2(c <= i ? a[i][c] : 0.0, c < i ? a[i][c + 1] : 0.0);
+      }
     }
     // trailing tiles (ti >= tj > panel): Y -= L_panel L_panel^T
     const int first = c0 / 8 + 1, nt = n8 / 8 - first, tiles = nt * (nt + 1) / 2;
-    for (int o = warp; o < tiles; o += 2 * n_warps) {
+    for (int o = warp; o < tiles && warp < n_warps - 1; o += 2 * (n_warps - 1)) {
       double acc[2][2], a[2][2], b[2][2];
       double* out[2];
-      const bool two = o + n_warps < tiles;
+      const bool two = o + n_warps - 1 < tiles;
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         int ti, tj;
-        lower_tile(u == 0 || !two ? o : o + n_warps, ti, tj);
+        lower_tile(u == 0 || !two ? o : o + n_warps - 1, ti, tj);
         const int ri = 8 * (first + ti) + g, rj = 8 * (first + tj) + g;
         out[u] = Y + ri * P + 8 * (first + tj) + 2 * q;
         acc[u][0] = out[u][0]; acc[u][1] = out[u][1];
@@ -101,11 +109,7 @@ __device__ __forceinline__ void group_cholesky(double* Y, int n, double tol, dou
     }
     bar();
   }
-  if (dmin_out != nullptr && warp == 0) {
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) dmin = fmin(dmin, __shfl_xor_sync(0xFFFFFFFFu, dmin, o));
-    if (lane == 0) *dmin_out = dmin;
-  }
+  if (dmin_out != nullptr && tid == nthr - 1) *dmin_out = __hiloint2double(dmin, 0);
   bar();
 }
 
@@ -114,45 +118,23 @@ __device__ __forceinline__ void cta_cholesky(double* Y, int n, double tol, doubl
   group_cholesky<P>(Y, n, tol, inv_out, dmin_out, (int)threadIdx.x, nthr, [] { __syncthreads(); });
 }
 
-// X = L^-1 (nothing is written above the diagonal blocks) for the factor of cta_cholesky, by all nthr threads: the 8 x 8 diagonal
-// blocks first (lane = column), then a warp per block column, X_ib = -X_ii sum_k L_ik X_kb on the FP64 tensor cores
-// without a barrier.  inv: reciprocal pivots (zero for a dependent column, whose row of X is then zero).
+// The inverse of diagonal block b of the factor of cta_cholesky (8 x 8, into X with row pitch xp), by one warp (lane = column).  inv: reciprocal
+// pivots (zero for a dependent column, whose row of the inverse is then zero).
 template <int P>
-__device__ __forceinline__ void cta_invert_lower(const double* L, const double* inv, int n, double* X, int xp, int nthr) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q = lane & 3, nb = (n + 7) / 8;
-  for (int b = warp; b < nb; b += nthr >> 5) {
-    if (lane < 8) {
-      double x[8];
+__device__ __forceinline__ void invert_diagonal_block(const double* L, const double* inv, int n, int b, double* X, int xp) {
+  const int lane = threadIdx.x & 31;
+  if (lane < 8) {
+    double x[8];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        double s = 0.0;
+    for (int i = 0; i < 8; ++i) {
+      double s = 0.0;
 #pragma unroll
-        for (int k = 0; k < i; ++k) s = fma(L[(8 * b + i) * P + 8 * b + k], x[k], s);
-        const double r = 8 * b + i < n ? inv[8 * b + i] : 0.0;
-        x[i] = i == lane ? r : (i > lane ? -r * s : 0.0);
-        X[(8 * b + i) * xp + 8 * b + lane] = x[i];
-      }
+      for (int k = 0; k < i; ++k) s = fma(L[(8 * b + i) * P + 8 * b + k], x[k], s);
+      const double r = 8 * b + i < n ? inv[8 * b + i] : 0.0;
+      x[i] = i == lane ? r : (i > lane ? -r * s : 0.0);
+      X[i * xp + lane] = x[i];
     }
   }
-  __syncthreads();
-  for (int b = warp; b < nb; b += nthr >> 5) {
-    for (int i = b + 1; i < nb; ++i) {
-      double t[2][2] = {};
-      for (int k = b; k < i; ++k)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) dmma(t[h], L[(8 * i + g) * P + 8 * k + 4 * h + q], X[(8 * k + 4 * h + q) * xp + 8 * b + g]);
-      double* out = X + (8 * i + g) * xp + 8 * b + 2 * q;
-      out[0] = t[0][0] + t[1][0]; out[1] = t[0][1] + t[1][1];
-      __syncwarp();
-      double d[2] = {0.0, 0.0};
-#pragma unroll
-      for (int h = 0; h < 2; ++h) dmma(d, -X[(8 * i + g) * xp + 8 * i + 4 * h + q], X[(8 * i + 4 * h + q) * xp + 8 * b + g]);
-      __syncwarp();
-      out[0] = d[0]; out[1] = d[1];
-      __syncwarp();
-    }
-  }
-  __syncthreads();
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -183,7 +165,7 @@ __device__ __forceinline__ void cta_invert_lower(const double* L, const double* 
 // rounding), U orthonormal to 1e-15 (1e-13); eigenvalues within 4e-5 of each other 3e-14 and 1e-13 (6e-8 and 1e-14); half of them repeated
 // 1e-8 and 3e-9 (7e-8 and 2e-8).  A pair of W that is orthogonal already is left to the orthonormalisation alone, half of R_ij to either column, only
 // if that does not tilt it: between eigenvalues of different size it does, by half of R_ij times the root of their ratio.
-// Input: Gram matrix (ld x ld, leading n x n block used).  Output: eigenvalues descending, eigenvectors as columns of
+// Input: `parts` partials of the Gram matrix (ld x ld each, leading n x n block used).  Output: eigenvalues descending, eigenvectors as columns of
 // evecs[n][n].
 // Measured alone, planted spectrum (in brackets: the reduction with three barriers a step, and the Jacobi sweeps of step 4 as the start of every
 // matrix): n = 8 10.3 us (10.3, 12.5), n = 32 25.8 (32.8, 43), n = 40 34.9 (43.1, 64), n = 64 68 (88, 127), n = 72 93 (115, 242).  Nearly diagonal
@@ -288,7 +270,7 @@ __device__ __forceinline__ void block_rotate(float2 (&a)[R], float2 (&b)[R], flo
 
 template <int NT8>                                      // n rounded up to a multiple of eight, over eight
 __global__ void __launch_bounds__(eig_threads(NT8), 1)
-eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ evals, double* __restrict__ evecs) {
+eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __restrict__ evals, double* __restrict__ evecs) {
   metis_pdl_wait();
   constexpr int N8 = 8 * NT8, P = N8 + 4, EIG_THREADS = eig_threads(NT8);
   constexpr int TD = 4 * N8, TS = TD + 32;              // threads of the reduction: four per row, and the warp that works out its scalars
@@ -320,7 +302,19 @@ eig_kernel(const double* __restrict__ gm, int n, int ld, double* __restrict__ ev
   // ---- the matrix ----
   for (int o = tid; o < N8 * N8; o += EIG_THREADS) {
     const int i = o / N8, j = o % N8;
-    E[i * P + j] = (i < n && j < n) ? gm[i * ld + j] : (i == j ? -1.0 : 0.0);
+    double a = i == j ? -1.0 : 0.0;
+    if (i < n && j < n) {
+      const double* src = gm + i * ld + j;
+      a = src[0];
+      for (int p = 1; p < parts; p += 8) {              // the other partials, in their order, loads in flight
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = p + u < parts ? src[(p + u) * ld * ld] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) a += v[u];
+      }
+    }
+    E[i * P + j] = a;
   }
   if (tid < N8) perm[tid] = tid;
   if (tid < EIG_MAX_SWEEPS) flags[tid] = flags64[tid] = 0;

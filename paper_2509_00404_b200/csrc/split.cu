@@ -19,20 +19,25 @@ constexpr int MAXQ = metis_small::MAXQ;                // k + p at most (k = 64 
 constexpr int LP = metis_small::PITCH;                 // row pitch of a factor in shared memory
 
 // ------------------------------------------------------------------------------------------------
-// The sampled rows; the first block of the one-CTA chain's call also clears what its later kernels accumulate into (a memset of
-// its own was a launch in front of every decomposition).
-__global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, int64_t rows, uint64_t seed, int full, float* __restrict__ amax, unsigned long long* __restrict__ keys) {
+// The j-th sampled row: one row per stratum of g consecutive rows, offset from Philox (g = 0: every row)
+struct RowSample { uint32_t g; uint64_t seed; };
+__device__ __forceinline__ int sample_row(const RowSample& rs, int j) {
+  if (rs.g == 0u) return j;
+  const uint4 w = metis_philox((uint32_t)j, 0u, METIS_STREAM_SAMPLING, 0u, (uint32_t)rs.seed, (uint32_t)(rs.seed >> 32));
+  return (int)((uint32_t)j * rs.g + w.x % rs.g);
+}
+// What the later kernels of a decomposition accumulate into, cleared by its first kernel (a memset of its own was a launch in front of
+// every decomposition): amax slots, condition flag, sign keys.
+__device__ __forceinline__ void clear_accumulators(float* amax, unsigned long long* keys) {
+  if (threadIdx.x < 16) amax[threadIdx.x] = 0.0f;
+  if (threadIdx.x < 64) keys[threadIdx.x] = 0ull;
+}
+
+// the sampled rows as indices (wide chain)
+__global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, RowSample rs) {
   metis_pdl_wait_trigger();
-  if (blockIdx.x == 0 && amax != nullptr && threadIdx.x < 64) {
-    if (threadIdx.x < 16) amax[threadIdx.x] = 0.0f;
-    keys[threadIdx.x] = 0ull;
-  }
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n_s) return;
-  if (full) { idx[j] = j; return; }
-  const uint32_t g = (uint32_t)(rows / n_s);
-  const uint4 w = metis_philox((uint32_t)j, 0u, METIS_STREAM_SAMPLING, 0u, (uint32_t)seed, (uint32_t)(seed >> 32));
-  idx[j] = (int)((uint32_t)j * g + w.x % g);          // one row per stratum of g consecutive rows
+  if (j < n_s) idx[j] = sample_row(rs, j);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -47,342 +52,400 @@ __global__ void split_status_kernel(const float* __restrict__ amax, const double
   if (bits) atomicOr(dev_status, bits);
 }
 
-__global__ void reduce_partials_kernel(const float* __restrict__ zp, int n_chunks, int64_t n, float* __restrict__ z) {
-  metis_pdl_wait_trigger();
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float acc = 0.0f;
-  int c = 0;
-  for (; c + 8 <= n_chunks; c += 8) {                                    // eight loads in flight; fixed order: reproducible
-    float t[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) t[u] = zp[(int64_t)(c + u) * n + i];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) acc += t[u];
-  }
-  for (; c < n_chunks; ++c) acc += zp[(int64_t)c * n + i];
-  z[i] = acc;
-}
-
 // ------------------------------------------------------------------------------------------------
-// Gram partials in FP64: part[p][i][j] = sum over the p-th slab of rows r of v(r,i) v(r,j),
-// v(r,i) = V[r*stride_row + i*stride_vec].
-// On the FP64 tensor cores: 64 rows at a time are converted to FP64 in shared memory (FP32 -> FP64 conversions are a slow-rate
-// instruction: once per element), a warp owns up to six lower 8 x 8 tiles of the result.  As FP64 multiply-adds
-// from shared memory the same slabs took 8.4 us (4096 x 40) and 24 us (16384 x 40).
+// Gram matrices in FP64 on the FP64 tensor cores: positions are taken 64 at a time, converted to FP64 in shared memory (FP32 -> FP64 conversions are a
+// slow-rate instruction: once per element), a warp owns up to six lower 8 x 8 tiles of the result.  The CTAs of a cluster add their tiles through
+// distributed shared memory in a fixed order, so that the kernel that needs the matrix (one CTA) adds at most GR_PARTS partials as it loads
+// them; a reduction of its own behind 64 partials was a launch of 3 - 4 us in the chain.
 constexpr int GR_TILE = 64;
 constexpr int GR_TPW = 6;                               // tiles per warp: 45 lower tiles at n = 72 over eight warps
-__global__ void __launch_bounds__(256)
-gram_kernel(const float* __restrict__ v, int64_t n_rows, int n, int64_t stride_row, int64_t stride_vec,
-            int64_t rows_per_part, double* __restrict__ part, const int* __restrict__ skip) {
-  metis_pdl_wait_trigger();
-  if (skip != nullptr && *skip) return;                 // second CholeskyQR pass not needed (see chol_kernel)
-  __shared__ double tile[GR_TILE][LP];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q4 = lane & 3;
-  const int64_t r_begin = (int64_t)blockIdx.x * rows_per_part;
-  const int64_t r_end = min(n_rows, r_begin + rows_per_part);
-  const int n8 = (n + 7) & ~7, tiles = (n8 / 8) * (n8 / 8 + 1) / 2;
-  int t_i[GR_TPW], t_j[GR_TPW];
+constexpr int GR_PARTS = 16, GR_CLUSTER = 8;
+struct GramTiles {
+  int t_i[GR_TPW], t_j[GR_TPW], tiles;
   double acc[GR_TPW][2][2];                             // even and odd steps: two chains in flight
+};
+__device__ __forceinline__ void gram_begin(GramTiles& t, int n8) {
+  t.tiles = (n8 / 8) * (n8 / 8 + 1) / 2;
 #pragma unroll
   for (int u = 0; u < GR_TPW; ++u) {
-    const int o = warp + 8 * u;
-    int ti = 0;
-    while ((ti + 1) * (ti + 2) / 2 <= o) ++ti;
-    t_i[u] = ti; t_j[u] = o - ti * (ti + 1) / 2;
-    acc[u][0][0] = acc[u][0][1] = acc[u][1][0] = acc[u][1][1] = 0.0;
+    metis_small::lower_tile((int)(threadIdx.x >> 5) + 8 * u, t.t_i[u], t.t_j[u]);
+    t.acc[u][0][0] = t.acc[u][0][1] = t.acc[u][1][0] = t.acc[u][1][1] = 0.0;
   }
-  for (int i = tid; i < GR_TILE * (n8 - n); i += 256) tile[i / (n8 - n)][n + i % (n8 - n)] = 0.0;
-  for (int64_t r0 = r_begin; r0 < r_end; r0 += GR_TILE) {
-    if (stride_row == 1) {
-      for (int i = tid; i < GR_TILE * n; i += 256) {
-        const int rr = i % GR_TILE, ii = i / GR_TILE;
-        tile[rr][ii] = r0 + rr < r_end ? (double)v[r0 + rr + ii * stride_vec] : 0.0;
-      }
-    } else {
-      for (int i = tid; i < GR_TILE * n; i += 256) {
-        const int ii = i % n, rr = i / n;
-        tile[rr][ii] = r0 + rr < r_end ? (double)v[(r0 + rr) * stride_row + ii * stride_vec] : 0.0;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < GR_TPW; ++u) {
-      if (warp + 8 * u < tiles) {
-        const double* pa = &tile[q4][8 * t_i[u] + g];
-        const double* pb = &tile[q4][8 * t_j[u] + g];
-#pragma unroll
-        for (int kk = 0; kk < GR_TILE; kk += 8) {
-          metis_small::dmma(acc[u][0], pa[kk * LP], pb[kk * LP]);
-          metis_small::dmma(acc[u][1], pa[(kk + 4) * LP], pb[(kk + 4) * LP]);
-        }
-      }
-    }
-    __syncthreads();
-  }
-  double* out = part + (int64_t)blockIdx.x * n * n;
+}
+// acc += the product of ROWS positions, tile[position][index] (PITCH 4 or 12 mod 16: conflict-free)
+template <int ROWS, int PITCH>
+__device__ __forceinline__ void gram_add(GramTiles& t, const double* tile) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, q4 = lane & 3;
 #pragma unroll
   for (int u = 0; u < GR_TPW; ++u) {
-    if (warp + 8 * u < tiles) {
+    if (warp + 8 * u < t.tiles) {
+      const double* pa = tile + q4 * PITCH + 8 * t.t_i[u] + g;
+      const double* pb = tile + q4 * PITCH + 8 * t.t_j[u] + g;
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int i = 8 * t_i[u] + g, j = 8 * t_j[u] + 2 * q4 + e;
-        const double x = acc[u][0][e] + acc[u][1][e];
-        if (i < n && j < n) {
-          out[i * n + j] = x;
-          if (t_i[u] != t_j[u]) out[j * n + i] = x;
-        }
+      for (int kk = 0; kk < ROWS; kk += 8) {
+        metis_small::dmma(t.acc[u][0], pa[kk * PITCH], pb[kk * PITCH]);
+        metis_small::dmma(t.acc[u][1], pa[(kk + 4) * PITCH], pb[(kk + 4) * PITCH]);
       }
     }
   }
 }
+// the cluster's sum into out (n x n); gp: shared memory for 64 doubles per tile, written by nobody else meanwhile; by all 256 threads of every CTA
+__device__ __forceinline__ void gram_end(const GramTiles& t, double* gp, int n, double* __restrict__ out) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q4 = lane & 3;
+#pragma unroll
+  for (int u = 0; u < GR_TPW; ++u)
+    if (warp + 8 * u < t.tiles)
+      *reinterpret_cast<double2*>(gp + 64 * (warp + 8 * u) + 8 * g + 2 * q4) = make_double2(t.acc[u][0][0] + t.acc[u][1][0], t.acc[u][0][1] + t.acc[u][1][1]);
+  const uint32_t csize = metis_cluster_size(), rank = metis_cluster_rank(), src = (uint32_t)__cvta_generic_to_shared(gp);
+  __syncthreads();
+  metis_cluster_sync();
+  for (int o = 4 * (int)rank + (tid >> 6); o < t.tiles; o += 4 * (int)csize) {     // four tiles at a time, an entry per thread
+    const int e = tid & 63;
+    double v[GR_CLUSTER], x = 0.0;
+#pragma unroll
+    for (uint32_t c = 0; c < GR_CLUSTER; ++c) {
+      v[c] = 0.0;
+      if (c < csize) asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v[c]) : "r"(metis_map_to_rank(src + (uint32_t)(64 * o + e) * 8u, c)));
+    }
+#pragma unroll
+    for (uint32_t c = 0; c < GR_CLUSTER; ++c) x += v[c];
+    int ti, tj;
+    metis_small::lower_tile(o, ti, tj);
+    const int i = 8 * ti + (e >> 3), j = 8 * tj + (e & 7);
+    if (i < n && j < n) {
+      out[i * n + j] = x;
+      if (ti != tj) out[j * n + i] = x;
+    }
+  }
+  metis_cluster_sync();                                 // the others may still be reading
+}
+// the sum of `parts` partials of an entry (at most GR_PARTS), loads in flight
+__device__ __forceinline__ double sum_parts(const double* __restrict__ in, int parts, int64_t stride) {
+  double a = 0.0;
+#pragma unroll
+  for (int p0 = 0; p0 < GR_PARTS; p0 += 8) {
+    if (p0 >= parts) break;
+    double v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) v[u] = p0 + u < parts ? in[(int64_t)(p0 + u) * stride] : 0.0;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) a += v[u];
+  }
+  return a;
+}
+// cluster and grid of a Gram kernel over `tiles` tiles of positions: at most GR_PARTS clusters, a CTA takes every grid-th tile
+inline void gram_grid(int64_t tiles, int* ctas, int* csize) {
+  int c = 1;
+  while (c < GR_CLUSTER && c < tiles) c *= 2;
+  const int64_t n = (tiles + c - 1) / c;
+  *csize = c; *ctas = (int)(n < GR_PARTS ? n : GR_PARTS) * c;
+}
+
+// Sums column slices of a tensor-core pass in a fixed order, v[position][i] = sum over s of part[s][position][i] (rows `width` wide, i < q), stores them
+// row by row (TRANS = 0: out[position][i]) or vector by vector (TRANS = 1: out[i][position]) and forms the Gram matrix of the q vectors.
+// out may be null (the slices are then the vectors themselves).
+constexpr size_t SG_SMEM = sizeof(double) * (GR_TILE * LP + 64 * 45);
+template <bool TRANS>
+__global__ void __launch_bounds__(256)
+sum_gram_kernel(const float* __restrict__ part, int slices, int64_t n_pos, int width, int q, float* __restrict__ out, double* __restrict__ gram_part,
+                const int* __restrict__ skip) {
+  metis_pdl_wait_trigger();
+  if (skip != nullptr && *skip) return;                 // second CholeskyQR pass not needed (see chol_kernel)
+  extern __shared__ __align__(16) double sg_sm[];
+  double *tile = sg_sm, *gp = sg_sm + GR_TILE * LP;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n8 = (q + 7) & ~7;
+  GramTiles t;
+  gram_begin(t, n8);
+  const int64_t tiles = (n_pos + GR_TILE - 1) / GR_TILE;
+  for (int64_t ti = blockIdx.x; ti < tiles; ti += gridDim.x) {
+    const int64_t p0 = ti * GR_TILE;
+    if ((width & 3) == 0) {
+      // the tile is one run of 64 * width floats per slice: groups of four, two groups' slices in flight (columns from q on are zeros)
+      const int w4 = width >> 2, n_o = (int)min((int64_t)GR_TILE, n_pos - p0) * w4;
+      const float4* src = reinterpret_cast<const float4*>(part) + p0 * w4;
+      const int64_t stride = n_pos * w4;
+      for (int o0 = tid; o0 < GR_TILE * w4; o0 += 512) {
+        float4 v[2][8];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int sl = 0; sl < 8; ++sl) v[u][sl] = sl < slices && o0 + 256 * u < n_o ? src[sl * stride + o0 + 256 * u] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          const int o = o0 + 256 * u, p = o / w4, j = 4 * (o - p * w4);
+          if (o >= GR_TILE * w4) break;
+          float4 x = v[u][0];
+#pragma unroll
+          for (int sl = 1; sl < 8; ++sl) { x.x += v[u][sl].x; x.y += v[u][sl].y; x.z += v[u][sl].z; x.w += v[u][sl].w; }
+          for (int sl = 8; sl < slices && o < n_o; ++sl) { const float4 y = src[sl * stride + o]; x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w; }
+          if (j < n8) {
+            *reinterpret_cast<double2*>(tile + p * LP + j) = make_double2((double)x.x, (double)x.y);
+            *reinterpret_cast<double2*>(tile + p * LP + j + 2) = make_double2((double)x.z, (double)x.w);
+          }
+          if (!TRANS && out != nullptr && o < n_o) {
+            float* dst = out + (p0 + p) * q + j;
+            if ((q & 3) == 0) { if (j < q) *reinterpret_cast<float4*>(dst) = x; }
+            else {
+              const float e[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+              for (int k = 0; k < 4; ++k) if (j + k < q) dst[k] = e[k];
+            }
+          }
+        }
+      }
+    } else {
+      for (int o = tid; o < GR_TILE * n8; o += 256) {
+        const int p = o / n8, j = o - p * n8;
+        float x = 0.0f;
+        if (p0 + p < n_pos && j < q) {
+          for (int sl = 0; sl < slices; ++sl) x += part[(sl * n_pos + p0 + p) * width + j];
+          if (!TRANS && out != nullptr) out[(p0 + p) * q + j] = x;
+        }
+        tile[p * LP + j] = (double)x;
+      }
+    }
+    __syncthreads();
+    if (TRANS)
+      for (int i = warp; i < q; i += 8)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          if (p0 + lane + 32 * h < n_pos) out[(int64_t)i * n_pos + p0 + lane + 32 * h] = (float)tile[(lane + 32 * h) * LP + i];
+    gram_add<GR_TILE, LP>(t, tile);
+    __syncthreads();
+  }
+  gram_end(t, gp, q, gram_part + (int64_t)(blockIdx.x / metis_cluster_size()) * q * q);
+}
 
 // ------------------------------------------------------------------------------------------------
-// One CholeskyQR pass, step 1 (one CTA): G = L L^T in FP64; writes L^-T (q x q, row-major, zero below the diagonal), so that step 2
-// is a product on many CTAs instead of a triangular solve per row.  A pivot below 1e-13 of the largest diagonal marks a
+// largest diagonal entry of a Gram matrix, to 20 bits from below (the high words order like the values); every warp by itself
+__device__ __forceinline__ double gram_scale(const double* L, int q) {
+  int top = 0;
+  for (int i = threadIdx.x & 31; i < q; i += 32) top = max(top, __double2hiint(L[i * LP + i]));
+  return __hiloint2double(__reduce_max_sync(0xFFFFFFFFu, top), 0);
+}
+
+// H = Z L^-T for eight rows by one warp, in registers: block column b is (Z_b - sum_k H_k L_bk^T) X_b^T with X_b the inverse of the factor's
+// 8 x 8 diagonal block.  h: accumulator tiles (lane: row lane / 4, columns 2 (lane % 4) and the next); a tile is the left operand of the next
+// product as it stands, its columns taken in the order 2 q, then 2 q + 1.
+template <int KT>
+__device__ __forceinline__ void solve_rows(double (&h)[KT][2], const double* L, const double (*Xd)[64]) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, q4 = lane & 3;
+#pragma unroll
+  for (int b = 0; b < KT; ++b) {
+    double acc2[2] = {0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < b; ++k) {
+      const double2 l = *reinterpret_cast<const double2*>(L + (8 * b + g) * LP + 8 * k + 2 * q4);
+      metis_small::dmma(h[b], -h[k][0], l.x);
+      metis_small::dmma(acc2, -h[k][1], l.y);
+    }
+    const double2 x = *reinterpret_cast<const double2*>(Xd[b] + 8 * g + 2 * q4);
+    const double a0 = h[b][0] + acc2[0], a1 = h[b][1] + acc2[1];
+    h[b][0] = h[b][1] = 0.0;
+    metis_small::dmma(h[b], a0, x.x);
+    metis_small::dmma(h[b], a1, x.y);
+  }
+}
+// Stores eight rows of H: FP32 rows of z, and the three-term BF16 splits, transposed (hsp[term][vector][row]: pairs of neighbouring rows, an even
+// row's lane keeps column j, an odd row's column j + 1).  r: this lane's row.
+template <int KT>
+__device__ __forceinline__ void store_rows(const double (&h)[KT][2], int64_t r, int64_t n_rows, int q, float* __restrict__ z, __nv_bfloat16* __restrict__ hsp, int jp, int64_t ldh) {
+  const int lane = threadIdx.x & 31, q4 = lane & 3;
+  const bool odd = lane & 4, in = r < n_rows;
+#pragma unroll
+  for (int b = 0; b < KT; ++b) {
+    const int j = 8 * b + 2 * q4;
+    const float v0 = in ? (float)h[b][0] : 0.0f, v1 = in ? (float)h[b][1] : 0.0f;
+    if (in) {
+      if ((q & 1) == 0) { if (j < q) *reinterpret_cast<float2*>(z + r * q + j) = make_float2(v0, v1); }
+      else { if (j < q) z[r * q + j] = v0; if (j + 1 < q) z[r * q + j + 1] = v1; }
+    }
+    const float other = __shfl_xor_sync(0xFFFFFFFFu, odd ? v0 : v1, 4);
+    float x = odd ? other : v0, y = odd ? v1 : other;
+    __nv_bfloat16* dst = hsp + (int64_t)(j + (odd ? 1 : 0)) * ldh + (r & ~(int64_t)1);
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const __nv_bfloat162 hb = __floats2bfloat162_rn(x, y);
+      const uint32_t w = *reinterpret_cast<const uint32_t*>(&hb);
+      x -= __uint_as_float(w << 16); y -= __uint_as_float(w & 0xFFFF0000u);
+      *reinterpret_cast<uint32_t*>(dst + (int64_t)t * jp * ldh) = w;
+    }
+  }
+}
+// One CholeskyQR pass of many rows, step 1 (one CTA): G = L L^T in FP64 from its partials; writes L and the inverses of its 8 x 8 diagonal blocks
+// (l_out: MAXQ x LP, then a block's 64 entries each), so that step 2 is a product on many CTAs.  A pivot below 1e-13 of the largest diagonal marks a
 // dependent sketch column: the corresponding column of H = Z L^-T becomes zero instead of amplified noise.
-constexpr size_t CHOL_SMEM = sizeof(double) * MAXQ * LP;
-__global__ void __launch_bounds__(512)
-chol_kernel(const double* __restrict__ g, int q, double* __restrict__ linvt_out, const int* __restrict__ skip, int* __restrict__ well_conditioned) {
+constexpr int CHOL_THREADS = 256, L_DOUBLES = MAXQ * LP + 64 * (MAXQ / 8);
+__global__ void __launch_bounds__(CHOL_THREADS)
+chol_kernel(const double* __restrict__ gm, int parts, int q, double* __restrict__ l_out, const int* __restrict__ skip, int* __restrict__ well_conditioned) {
   metis_pdl_wait();
   if (skip != nullptr && *skip) return;
-  extern __shared__ __align__(16) double xs[];
-  __shared__ double L[MAXQ][LP];
-  __shared__ double gmax_s;
-  __shared__ double dmin_s;
-  __shared__ double inv_s[MAXQ];
-  const int tid = threadIdx.x, q8 = (q + 7) & ~7;
-  for (int o = tid; o < q8 * q8; o += 512) {
-    const int i = o / q8, j = o % q8;
-    L[i][j] = i < q && j < q ? g[i * q + j] : 0.0;
-  }
+  __shared__ __align__(16) double L[MAXQ][LP];
+  __shared__ double dmin_s, inv_s[MAXQ];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q8 = (q + 7) & ~7;
+  for (int i = warp; i < q8; i += CHOL_THREADS / 32)
+    for (int j = lane; j < q8; j += 32) L[i][j] = i < q && j <= i ? sum_parts(gm + i * q + j, parts, (int64_t)q * q) : 0.0;
   __syncthreads();
-  if (tid < 32) {
-    double gm = 0.0;
-    for (int i = tid; i < q; i += 32) gm = fmax(gm, L[i][i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) gm = fmax(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, o));
-    if (tid == 0) gmax_s = gm;
-  }
-  __syncthreads();
-  const double tol = 1e-13 * gmax_s;
-  metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, 512);
+  const double gmax = gram_scale(&L[0][0], q);
+  metis_small::cta_cholesky<LP>(&L[0][0], q, 1e-13 * gmax, inv_s, &dmin_s, CHOL_THREADS);
   // With every pivot above 1e-8 of the largest diagonal the FP64 factorisation leaves Z L^-T orthonormal to
   // ~1e-8 already, below the FP32 rounding of its storage: the caller's second pass is then skipped.
   metis_pdl_trigger();
-  if (tid == 0 && well_conditioned != nullptr) *well_conditioned = (dmin_s > 1e-8 * gmax_s) ? 1 : 0;
-  metis_small::cta_invert_lower<LP>(&L[0][0], inv_s, q, xs, LP, 512);
-  for (int o = tid; o < q * q; o += 512) { const int i = o / q, j = o % q; linvt_out[o] = i <= j ? xs[j * LP + i] : 0.0; }
+  if (tid == 0 && well_conditioned != nullptr) *well_conditioned = (dmin_s > 1e-8 * gmax) ? 1 : 0;
+  for (int b = warp; b < q8 / 8; b += CHOL_THREADS / 32) metis_small::invert_diagonal_block<LP>(&L[0][0], inv_s, q, b, l_out + MAXQ * LP + 64 * b, 8);
+  for (int o = tid; o < q8 * LP / 2; o += CHOL_THREADS) reinterpret_cast<double2*>(l_out)[o] = reinterpret_cast<const double2*>(&L[0][0])[o];
 }
 
-// One CholeskyQR pass, steps 0 and 1 in one CTA, for a sketch short enough to sit in shared memory as FP64 (the
-// row-sampled case: a few hundred rows): G = Z^T Z and its Cholesky factor without a trip through global memory.
-// The Gram matrix is formed on the FP64 tensor cores, a warp per lower 8 x 8 tile (as FP64 multiply-adds from shared memory
-// it took half of the kernel: 22 -> 9 us at 160 x 40 with the panel factorisation).
-constexpr int GC_THREADS = 512;
-constexpr size_t GC_MAX_SMEM = 176 * 1024;              // beside ~45 KiB of static shared memory: 288 sampled rows at q = 72
-__host__ __device__ inline int gram_chol_pitch(int q) { return ((q + 7) & ~7) + 4; }   // 4 or 12 mod 16: conflict-free fragment loads
-__host__ inline size_t gram_chol_smem(int64_t n_s, int q) { return (size_t)n_s * gram_chol_pitch(q) * sizeof(double); }
-// Well-conditioned sketch (every pivot above 1e-8 of the largest diagonal: Z L^-T is orthonormal to ~1e-8 already):
-// the kernel writes L^-T and clears *applied; orth_apply_kernel, on many CTAs, multiplies by it.  Otherwise (rare) the whole CholeskyQR2 runs here on the FP64 copy - solve, second Gram
-// matrix, second factor, second solve - H is written over z and *applied is set, which makes the apply kernel
-// behind this one return at once.
-__global__ void __launch_bounds__(GC_THREADS, 1)
-gram_chol_kernel(float* __restrict__ z, int n_s, int q, double* __restrict__ linvt_out, int* __restrict__ applied) {
-  metis_pdl_wait();
-  extern __shared__ __align__(16) double zs[];
-  __shared__ double L[MAXQ][LP];
-  __shared__ double gmax_s;
-  __shared__ double dmin_s;
-  __shared__ double inv_s[MAXQ];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int q8 = (q + 7) & ~7, zp = gram_chol_pitch(q);
-  for (int o = tid; o < n_s * zp; o += GC_THREADS) {
-    const int r = o / zp, c = o - r * zp;
-    zs[o] = c < q ? (double)z[(int64_t)r * q + c] : 0.0;
-  }
-  const int g = lane >> 2, q4 = lane & 3, tiles = (q8 / 8) * (q8 / 8 + 1) / 2;
-  bool solved_here = false;
-  __syncthreads();
-  for (int pass = 0; pass < 2; ++pass) {
-    for (int o = warp; o < tiles; o += GC_THREADS / 32) {
-      int ti = 0;
-      while ((ti + 1) * (ti + 2) / 2 <= o) ++ti;
-      const int tj = o - ti * (ti + 1) / 2;
-      double acc[4][2] = {};
-      const double* pa = zs + q4 * zp + 8 * ti + g;
-      const double* pb = zs + q4 * zp + 8 * tj + g;
-      for (int r0 = 0; r0 < n_s; r0 += 16) {               // n_s is a multiple of 16
-#pragma unroll
-        for (int u = 0; u < 4; ++u) metis_small::dmma(acc[u], pa[(r0 + 4 * u) * zp], pb[(r0 + 4 * u) * zp]);
-      }
-#pragma unroll
-      for (int e = 0; e < 2; ++e) L[8 * ti + g][8 * tj + 2 * q4 + e] = (acc[0][e] + acc[1][e]) + (acc[2][e] + acc[3][e]);
-    }
-    __syncthreads();
-    if (tid < 32) {
-      double gm = 0.0;
-      for (int i = tid; i < q; i += 32) gm = fmax(gm, L[i][i]);
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) gm = fmax(gm, __shfl_xor_sync(0xFFFFFFFFu, gm, off));
-      if (tid == 0) gmax_s = gm;
-    }
-    __syncthreads();
-    const double tol = 1e-13 * gmax_s;
-    metis_small::cta_cholesky<LP>(&L[0][0], q, tol, inv_s, &dmin_s, GC_THREADS);
-    metis_pdl_trigger();
-    if (pass == 0 && dmin_s > 1e-8 * gmax_s) break;
-    // z_row <- z_row L^-T in shared memory by forward substitution, one warp per row, column-oriented: lane i % 32 keeps z_i; step j
-    // broadcasts h_j = z_j / L[j][j] from its owner and every lane subtracts h_j L[i][j] from its own later entries
-    solved_here = true;
-    for (int r = warp; r < n_s; r += GC_THREADS / 32) {
-      double* zr = zs + r * zp;
-      double z0 = lane < q ? zr[lane] : 0.0, z1 = lane + 32 < q ? zr[lane + 32] : 0.0, z2 = lane + 64 < q ? zr[lane + 64] : 0.0;
-      for (int j = 0; j < q; ++j) {
-        const double lj0 = lane < q ? L[lane][j] : 0.0;
-        const double lj1 = lane + 32 < q ? L[lane + 32][j] : 0.0;
-        const double lj2 = lane + 64 < q ? L[lane + 64][j] : 0.0;
-        const double zj = __shfl_sync(0xFFFFFFFFu, j < 32 ? z0 : (j < 64 ? z1 : z2), j & 31);
-        const double hj = zj * inv_s[j];
-        if (lane == (j & 31)) { if (j < 32) z0 = hj; else if (j < 64) z1 = hj; else z2 = hj; }
-        if (lane > j) z0 -= hj * lj0;
-        if (lane + 32 > j) z1 -= hj * lj1;
-        if (lane + 64 > j) z2 -= hj * lj2;
-      }
-      if (lane < q) zr[lane] = z0;
-      if (lane + 32 < q) zr[lane + 32] = z1;
-      if (lane + 64 < q) zr[lane + 64] = z2;
-    }
-    __syncthreads();
-  }
-  if (tid == 0) *applied = solved_here ? 1 : 0;
-  if (solved_here) {
-    for (int e = tid; e < n_s * q; e += GC_THREADS) z[e] = (float)zs[(e / q) * zp + e % q];
-  } else {
-    // the FP64 copy of z is not needed any more: n_s >= q rows of the same pitch hold the inverse
-    metis_small::cta_invert_lower<LP>(&L[0][0], inv_s, q, zs, zp, GC_THREADS);
-    for (int e = tid; e < q * q; e += GC_THREADS) { const int i = e / q, j = e % q; linvt_out[e] = i <= j ? zs[j * zp + i] : 0.0; }
-  }
-}
-
-// One CholeskyQR pass, step 2: Z <- Z L^-T in place, 64 rows per CTA, on the FP64 tensor cores (a warp per eight rows), and optionally
-// the transposed BF16 splits of the result for the tensor-core projection (the layout of h_splits_kernel).  A triangular solve
-// per row, one column after the other, took 15 us for 4096 x 40, 47 us for 16384 x 40 and 186 us for 28672 x 72.
-constexpr int OA_ROWS = 64, OA_P = OA_ROWS + 4, OA_OP = OA_ROWS + 1;
-__host__ __device__ constexpr size_t oa_smem(int kt) { return sizeof(double) * (size_t)(8 * kt) * (OA_P + 8 * kt + 4) + sizeof(float) * 8 * OA_OP; }
+// One CholeskyQR pass of many rows, step 2: Z <- Z L^-T in place, 64 rows per CTA, a warp per eight rows, and the splits of the result.  (As a product with
+// the explicit inverse from shared memory, with FP64 copies of Z and the inverse: 1570 instructions a warp, 8 us of a chain.  A triangular solve per
+// row, one column after the other, took 15 us for 4096 x 40, 47 us for 16384 x 40 and 186 us for 28672 x 72.)
+constexpr int OA_ROWS = 64;
 template <int KT>                                       // ceil(q / 8)
 __global__ void __launch_bounds__(256)
-orth_apply_kernel(float* __restrict__ z, int64_t n_rows, int q, const double* __restrict__ linvt, const int* __restrict__ skip,
+orth_apply_kernel(float* __restrict__ z, int64_t n_rows, int q, const double* __restrict__ l, const int* __restrict__ skip,
                   __nv_bfloat16* __restrict__ hsp, int jp, int64_t ldh) {
   metis_pdl_wait_trigger();
   if (skip != nullptr && *skip) return;
-  constexpr int Q8 = 8 * KT, WP = Q8 + 4;
-  extern __shared__ __align__(16) double oa_sm[];
-  double *As = oa_sm, *Ws = oa_sm + Q8 * OA_P;
-  float* Os = reinterpret_cast<float*>(oa_sm);          // [Q8 + 8][OA_OP], over As and Ws once they have been read
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, qq = lane & 3;
-  const int64_t p0 = (int64_t)blockIdx.x * OA_ROWS;
-#pragma unroll 4
-  for (int o = tid; o < OA_ROWS * Q8; o += 256) {
-    const int r = o / Q8, i = o % Q8;
-    As[i * OA_P + r] = i < q && p0 + r < n_rows ? (double)z[(p0 + r) * q + i] : 0.0;
+  __shared__ __align__(16) double L[8 * KT][LP];
+  __shared__ __align__(16) double Xd[KT][64];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q4 = lane & 3;
+  const int64_t r0 = (int64_t)blockIdx.x * OA_ROWS, r = r0 + 8 * warp + g;
+  double h[KT][2];
+#pragma unroll
+  for (int b = 0; b < KT; ++b) {
+    const int j = 8 * b + 2 * q4;
+    float2 v = make_float2(0.0f, 0.0f);
+    if (r < n_rows && (q & 1) == 0 && j < q) v = *reinterpret_cast<const float2*>(z + r * q + j);
+    else if (r < n_rows && (q & 1) != 0) { if (j < q) v.x = z[r * q + j]; if (j + 1 < q) v.y = z[r * q + j + 1]; }
+    h[b][0] = (double)v.x; h[b][1] = (double)v.y;
   }
 #pragma unroll 4
-  for (int o = tid; o < Q8 * Q8; o += 256) {
-    const int i = o / Q8, j = o % Q8;
-    Ws[i * WP + j] = i < q && j < q ? linvt[i * q + j] : 0.0;
-  }
+  for (int o = tid; o < 8 * KT * LP / 2; o += 256) reinterpret_cast<double2*>(&L[0][0])[o] = reinterpret_cast<const double2*>(l)[o];
+  for (int o = tid; o < 64 * KT / 2; o += 256) reinterpret_cast<double2*>(&Xd[0][0])[o] = reinterpret_cast<const double2*>(l + MAXQ * LP)[o];
   __syncthreads();
-  double acc[KT][2] = {};
-#pragma unroll
-  for (int kk = 0; kk < Q8; kk += 4) {
-    const double a = As[(kk + qq) * OA_P + 8 * warp + g];
-#pragma unroll
-    for (int t = kk / 8; t < KT; ++t) metis_small::dmma(acc[t], a, Ws[(kk + qq) * WP + 8 * t + g]);              // L^-T is upper triangular
-  }
-  __syncthreads();
-#pragma unroll
-  for (int t = 0; t < KT; ++t)
-#pragma unroll
-    for (int e = 0; e < 2; ++e) Os[(8 * t + 2 * qq + e) * OA_OP + 8 * warp + g] = (float)acc[t][e];
-  for (int o = tid; o < 8 * OA_OP; o += 256) Os[Q8 * OA_OP + o] = 0.0f;
-  __syncthreads();
-  for (int o = tid; o < OA_ROWS * q; o += 256) {
-    const int r = o / q, j = o - r * q;
-    if (p0 + r < n_rows) z[(p0 + r) * q + j] = Os[j * OA_OP + r];
-  }
-  if (hsp == nullptr) return;
-  for (int o = tid; o < jp * (OA_ROWS / 2); o += 256) { // rows beyond n_rows and vectors beyond q are zeros
-    const int j = o / (OA_ROWS / 2), r = o % (OA_ROWS / 2) * 2;
-    float x = Os[j * OA_OP + r], y = Os[j * OA_OP + r + 1];
-    uint32_t w[3];
-#pragma unroll
-    for (int t = 0; t < 3; ++t) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
-      w[t] = *reinterpret_cast<const uint32_t*>(&h);
-      x -= __uint_as_float(w[t] << 16); y -= __uint_as_float(w[t] & 0xFFFF0000u);
-      *reinterpret_cast<uint32_t*>(hsp + ((int64_t)t * jp + j) * ldh + p0 + r) = w[t];
-    }
-  }
+  solve_rows<KT>(h, &L[0][0], Xd);
+  store_rows<KT>(h, r, n_rows, q, z, hsp, jp, ldh);     // (rows up to the next multiple of 64 are zeros of the splits)
+  if (jp > 8 * KT && tid < 24 * OA_ROWS / 8)            // vectors beyond 8 KT (eight of each term)
+    *reinterpret_cast<uint4*>(hsp + ((int64_t)(tid >> 6) * jp + 8 * KT + (tid & 7)) * ldh + r0 + 8 * ((tid >> 3) & 7)) = make_uint4(0u, 0u, 0u, 0u);
 }
 
-// ------------------------------------------------------------------------------------------------
-// Projection partials: Mp[part][j][col] = sum over the part's sampled rows r of H[r][j] * x[idx[r], col]
-// (q x cols per part, row j contiguous).  Thread: two adjacent columns, every second sketch column.
-constexpr int PJ_COLS = 256, PJ_ROWS = 32;
-template <int NJ4>                                                  // float4 groups of sketch columns per thread
-__global__ void __launch_bounds__(256)
-project_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __restrict__ idx, int n_s, int q,
-               const float* __restrict__ h, int rows_per_part, float* __restrict__ mp) {
-  metis_pdl_wait_trigger();
-  __shared__ __align__(16) float hs[2][PJ_ROWS][MAXQ / 2];
-  __shared__ int ids[PJ_ROWS];
-  const int tid = threadIdx.x, c2 = tid & 127, jg = tid >> 7;       // jg: sketch columns 2*j + jg
-  const int64_t col = (int64_t)blockIdx.x * PJ_COLS + c2 * 2;
-  const int r_begin = blockIdx.y * rows_per_part, r_end = min(n_s, r_begin + rows_per_part);
-  float acc0[NJ4 * 4], acc1[NJ4 * 4];
+// Orthonormalisation of a short sketch (the row-sampled case: a few hundred rows) by one cluster: a CTA takes every eighth group of eight rows - the sum of the
+// sketch's partials, its part of G = Z^T Z on the FP64 tensor cores, later its rows of H = Z L^-T - and all of them factorise G, whose sum they
+// exchange through distributed shared memory, for themselves.  With a pivot below 1e-8 of the largest diagonal a second pass runs on
+// the FP64 rows (above that Z L^-T is orthonormal to ~1e-8 already, below the FP32 rounding of its storage); a pivot below 1e-13 marks a
+// dependent column, whose column of H is zero.  In one CTA of sixteen warps 17.7 us at 160 x 40 (sum 4.6 k cycles, Gram matrix 4.4 k,
+// factor 10.9 k, H 8.5 k) and 52 us at 288 x 72; now 11.2 us (1.4 k, 1.1 k and 3.1 k for the exchange, 8.4 k, 1.9 k) and 22.6 us.
+constexpr int GC_THREADS = 256, GC_CLUSTER = 8;
+constexpr int64_t GC_MAX_ROWS = 1024;                   // longer sketches: sum_gram_kernel, chol_kernel, orth_apply_kernel
+__host__ __device__ constexpr int gram_chol_pitch(int kt) { return 8 * kt + 4; }        // 4 or 12 mod 16: conflict-free fragment loads
+__host__ __device__ constexpr int64_t gram_chol_rows(int64_t n_s) { return (n_s / 8 + GC_CLUSTER - 1) / GC_CLUSTER * 8; }      // of a CTA
+__host__ __device__ constexpr size_t gram_chol_smem(int64_t n_s, int kt) {
+  return sizeof(double) * (size_t)(8 * kt * LP + 64 * (kt * (kt + 1) / 2) + gram_chol_rows(n_s) * gram_chol_pitch(kt));
+}
+template <int KT>                                       // ceil(q / 8)
+__global__ void __launch_bounds__(GC_THREADS, 1)
+gram_chol_kernel(const float* __restrict__ zp, int parts, int width, int n_s, int q, float* __restrict__ z, __nv_bfloat16* __restrict__ hsp, int jp, int64_t ldh) {
+  metis_pdl_wait();
+  constexpr int Q8 = 8 * KT, ZP = gram_chol_pitch(KT), TILES = KT * (KT + 1) / 2, TPW = (TILES + 7) / 8;
+  extern __shared__ __align__(16) double gc_sm[];
+  double (*L)[LP] = reinterpret_cast<double (*)[LP]>(gc_sm);                     // [Q8][LP]
+  double *gp = gc_sm + Q8 * LP, *zs = gp + 64 * TILES;  // [TILES][64], [own rows][ZP]
+  __shared__ __align__(16) double Xd[KT][64];
+  __shared__ double dmin_s, inv_s[MAXQ];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, q4 = lane & 3;
+  const int rank = (int)metis_cluster_rank(), groups = (n_s / 8 - rank + GC_CLUSTER - 1) / GC_CLUSTER;         // own groups of eight rows: rank, rank + 8, ...
+  // ---- the sketch: eight columns of a row per thread, all partials in flight ----
+  for (int o = tid; o < groups * 8 * KT; o += GC_THREADS) {
+    const int lr = o / KT, c0 = 8 * (o - lr * KT), r = 8 * (rank + GC_CLUSTER * (lr >> 3)) + (lr & 7);
+    const float* src = zp + (int64_t)r * width + c0;        // (a partial's columns beyond q, if it has them, are zeros)
+    const int64_t stride = (int64_t)n_s * width;
+    float a[8] = {};
+    if ((width & 3) == 0) {                              // whole groups of four
 #pragma unroll
-  for (int j = 0; j < NJ4 * 4; ++j) { acc0[j] = 0.0f; acc1[j] = 0.0f; }
-  for (int r0 = r_begin; r0 < r_end; r0 += PJ_ROWS) {
-    for (int i = tid; i < PJ_ROWS * MAXQ; i += 256) {
-      const int rr = i / MAXQ, jj = i % MAXQ;
-      hs[jj & 1][rr][jj >> 1] = (r0 + rr < r_end && jj < q) ? h[(int64_t)(r0 + rr) * q + jj] : 0.0f;
+      for (int p0 = 0; p0 < GR_PARTS; p0 += 8) {
+        if (p0 >= parts) break;
+        float4 u[8], v[8];
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          u[p] = v[p] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (p0 + p < parts) {
+            u[p] = *reinterpret_cast<const float4*>(src + (p0 + p) * stride);
+            if (c0 + 4 < width) v[p] = *reinterpret_cast<const float4*>(src + (p0 + p) * stride + 4);
+          }
+        }
+#pragma unroll
+        for (int p = 0; p < 8; ++p) { a[0] += u[p].x; a[1] += u[p].y; a[2] += u[p].z; a[3] += u[p].w; a[4] += v[p].x; a[5] += v[p].y; a[6] += v[p].z; a[7] += v[p].w; }
+      }
+    } else {
+#pragma unroll 4
+      for (int p = 0; p < parts; ++p)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) a[e] += c0 + e < q ? src[p * stride + e] : 0.0f;
     }
-    if (tid < PJ_ROWS) ids[tid] = (r0 + tid < r_end) ? idx[r0 + tid] : 0;
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) *reinterpret_cast<double2*>(zs + lr * ZP + c0 + e) = make_double2((double)a[e], (double)a[e + 1]);
+  }
+  __syncthreads();
+  for (int pass = 0; pass < 2; ++pass) {
+#pragma unroll
+    for (int u = 0; u < TPW; ++u) {
+      const int o = warp + 8 * u;
+      if (o < TILES) {
+        int ti, tj;
+        metis_small::lower_tile(o, ti, tj);
+        double acc[2][2] = {};
+        for (int r0 = 0; r0 < 8 * groups; r0 += 8)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) metis_small::dmma(acc[h], zs[(r0 + 4 * h + q4) * ZP + 8 * ti + g], zs[(r0 + 4 * h + q4) * ZP + 8 * tj + g]);
+        *reinterpret_cast<double2*>(gp + 64 * o + 8 * g + 2 * q4) = make_double2(acc[0][0] + acc[1][0], acc[0][1] + acc[1][1]);
+      }
+    }
     __syncthreads();
-    const int nr = min(PJ_ROWS, r_end - r0);
-    // the tile's x values first, all loads in flight (inside the loop below each was an L2 round trip per row)
-    uint32_t xw[PJ_ROWS];
+    metis_cluster_sync();                                // (also: every CTA has finished with its L of the pass before)
+    // tile o is summed by CTA o % 8, in the order of the ranks, and handed to all
+    for (int o = rank + GC_CLUSTER * (tid >> 6); o < TILES; o += GC_CLUSTER * (GC_THREADS / 64)) {
+      const int e = tid & 63;
+      int ti, tj;
+      metis_small::lower_tile(o, ti, tj);
+      const uint32_t src = (uint32_t)__cvta_generic_to_shared(gp + 64 * o + e), dst = (uint32_t)__cvta_generic_to_shared(&L[8 * ti + (e >> 3)][8 * tj + (e & 7)]);
+      double v[GC_CLUSTER], x = 0.0;
 #pragma unroll
-    for (int rr = 0; rr < PJ_ROWS; ++rr) {
-      xw[rr] = 0u;
-      if (rr < nr) {
-        if (col + 1 < cols) xw[rr] = *reinterpret_cast<const uint32_t*>(x + (int64_t)ids[rr] * cols + col);
-        else if (col < cols) xw[rr] = (uint32_t)__bfloat16_as_ushort(x[(int64_t)ids[rr] * cols + col]);
+      for (uint32_t c = 0; c < GC_CLUSTER; ++c) asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v[c]) : "r"(metis_map_to_rank(src, c)));
+#pragma unroll
+      for (uint32_t c = 0; c < GC_CLUSTER; ++c) x += v[c];
+#pragma unroll
+      for (uint32_t c = 0; c < GC_CLUSTER; ++c) asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(metis_map_to_rank(dst, c)), "d"(x) : "memory");
+    }
+    __syncthreads();
+    metis_cluster_sync();
+    const double gmax = gram_scale(&L[0][0], q);
+    metis_small::cta_cholesky<LP>(&L[0][0], q, 1e-13 * gmax, inv_s, &dmin_s, GC_THREADS);
+    metis_pdl_trigger();
+    const bool last = pass == 1 || dmin_s > 1e-8 * gmax;
+    for (int b = warp; b < KT; b += GC_THREADS / 32) metis_small::invert_diagonal_block<LP>(&L[0][0], inv_s, q, b, Xd[b], 8);
+    __syncthreads();
+    for (int gr = warp; gr < groups; gr += GC_THREADS / 32) {
+      double h[KT][2];
+      double* row = zs + (8 * gr + g) * ZP + 2 * q4;
+#pragma unroll
+      for (int b = 0; b < KT; ++b) { const double2 v = *reinterpret_cast<const double2*>(row + 8 * b); h[b][0] = v.x; h[b][1] = v.y; }
+      solve_rows<KT>(h, &L[0][0], Xd);
+      if (last) store_rows<KT>(h, 8 * (rank + GC_CLUSTER * gr) + g, n_s, q, z, hsp, jp, ldh);
+      else {
+#pragma unroll
+        for (int b = 0; b < KT; ++b) *reinterpret_cast<double2*>(row + 8 * b) = make_double2(h[b][0], h[b][1]);
       }
     }
-#pragma unroll
-    for (int rr = 0; rr < PJ_ROWS; ++rr) {
-      if (rr >= nr) break;
-      const float x0 = __uint_as_float(xw[rr] << 16), x1 = __uint_as_float(xw[rr] & 0xFFFF0000u);
-#pragma unroll
-      for (int j4 = 0; j4 < NJ4; ++j4) {
-        const float4 hv = *reinterpret_cast<const float4*>(&hs[jg][rr][j4 * 4]);
-        acc0[j4 * 4 + 0] = fmaf(hv.x, x0, acc0[j4 * 4 + 0]); acc1[j4 * 4 + 0] = fmaf(hv.x, x1, acc1[j4 * 4 + 0]);
-        acc0[j4 * 4 + 1] = fmaf(hv.y, x0, acc0[j4 * 4 + 1]); acc1[j4 * 4 + 1] = fmaf(hv.y, x1, acc1[j4 * 4 + 1]);
-        acc0[j4 * 4 + 2] = fmaf(hv.z, x0, acc0[j4 * 4 + 2]); acc1[j4 * 4 + 2] = fmaf(hv.z, x1, acc1[j4 * 4 + 2]);
-        acc0[j4 * 4 + 3] = fmaf(hv.w, x0, acc0[j4 * 4 + 3]); acc1[j4 * 4 + 3] = fmaf(hv.w, x1, acc1[j4 * 4 + 3]);
-      }
-    }
+    if (last) break;
     __syncthreads();
   }
-  float* dst = mp + (int64_t)blockIdx.y * q * cols;
-#pragma unroll
-  for (int j = 0; j < NJ4 * 4; ++j)
-    if (2 * j + jg < q) {
-      if (col < cols) dst[(int64_t)(2 * j + jg) * cols + col] = acc0[j];
-      if (col + 1 < cols) dst[(int64_t)(2 * j + jg) * cols + col + 1] = acc1[j];
-    }
+  // the splits' padding: vectors beyond Q8, rows beyond n_s
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  if (jp > Q8 && tid < 24)
+    for (int gr = 0; gr < groups; ++gr) *reinterpret_cast<uint4*>(hsp + ((int64_t)(tid >> 3) * jp + Q8 + (tid & 7)) * ldh + 8 * (rank + GC_CLUSTER * gr)) = zero;
+  if (rank * GC_THREADS + tid < 3 * jp)
+    for (int64_t r = n_s; r < ldh; r += 8) *reinterpret_cast<uint4*>(hsp + (int64_t)(rank * GC_THREADS + tid) * ldh + r) = zero;
+  metis_cluster_sync();                                  // (nobody reads another's shared memory any more)
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -474,17 +537,24 @@ reduce_gram_kernel(const double* __restrict__ in, int n_in, int nn, double* __re
   if (sl == 0 && e < nn) out[e] = ((part[0][lane] + part[1][lane]) + part[2][lane]) + part[3][lane];
 }
 
-// Sums the column slices of the tensor-core broadcast pass in a fixed order: coef[r][j] = sum_s part[s][r][j],
-// and writes the FP64 Gram partial of the CTA's 32 rows of C (for Rayleigh-Ritz).
+// Sums the column slices of the tensor-core broadcast pass in a fixed order: coef[r][j] = sum_s part[s][r][j], writes the residual
+// product's operand a6 and, per cluster of CTAs of 32 rows each, the Gram partial of their rows of C (for Rayleigh-Ritz).
 template <int KP>
 __global__ void __launch_bounds__(256)
 coef_finish_kernel(const float* __restrict__ part, int slices, int64_t rows, float* __restrict__ coef,
                    double* __restrict__ gram_part, __nv_bfloat16* __restrict__ a6, int kx) {
-  metis_pdl_wait_trigger();
+  constexpr int CP = KP + 4;                            // 4 mod 16: conflict-free fragment loads
   __shared__ float cfin[32 * KP];
+  __shared__ __align__(16) double cd[32 * CP];          // converted once: FP32 -> FP64 is a slow-rate instruction
+  __shared__ __align__(16) double gp[64 * (KP / 8) * (KP / 8 + 1) / 2];
+  GramTiles gt;
+  gram_begin(gt, KP);
+  metis_pdl_wait_trigger();
   const int tid = threadIdx.x;
   const int64_t row0 = (int64_t)blockIdx.x * 32;
-  for (int o = tid; o < 32 * KP; o += 256) {
+#pragma unroll
+  for (int u = 0; u < 32 * KP / 256; ++u) {
+    const int o = tid + 256 * u;
     const int64_t r = row0 + o / KP;
     float v = 0.0f;
     if (r < rows) {
@@ -496,75 +566,56 @@ coef_finish_kernel(const float* __restrict__ part, int slices, int64_t rows, flo
       coef[r * KP + (o % KP)] = v;
     }
     cfin[o] = v;
+    cd[o / KP * CP + o % KP] = (double)v;
   }
   __syncthreads();
-  if (a6 != nullptr) {
-    // a6: [rows][kx], per row the six K blocks [Ch | Ch | Cl | Ch | Cl2 | Cl] of the residual product (zero padded)
-    for (int o = tid; o < 32 * (KP / 8); o += 256) {
-      const int rr = o / (KP / 8), j0 = (o % (KP / 8)) * 8;
-      const int64_t r = row0 + rr;
-      if (r >= rows) continue;
-      float v[8];
+  // a6: [rows][kx], per row the six K blocks [Ch | Ch | Cl | Ch | Cl2 | Cl] of the residual product (zero padded)
+  for (int o = tid; o < 32 * (KP / 8); o += 256) {
+    const int rr = o / (KP / 8), j0 = (o % (KP / 8)) * 8;
+    const int64_t r = row0 + rr;
+    if (r >= rows) continue;
+    float v[8];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = cfin[rr * KP + j0 + e];
-      uint4 h, l, l2;
-      metis_split3x8(v, h, l, l2);
-      __nv_bfloat16* dst = a6 + r * kx + j0;
-      *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + KP) = h; *reinterpret_cast<uint4*>(dst + 2 * KP) = l;
-      *reinterpret_cast<uint4*>(dst + 3 * KP) = h; *reinterpret_cast<uint4*>(dst + 4 * KP) = l2; *reinterpret_cast<uint4*>(dst + 5 * KP) = l;
-      if (j0 == 0)
-        for (int z = 6 * KP; z < kx; z += 8) *reinterpret_cast<uint4*>(a6 + r * kx + z) = make_uint4(0u, 0u, 0u, 0u);
-    }
+    for (int e = 0; e < 8; ++e) v[e] = cfin[rr * KP + j0 + e];
+    uint4 h, l, l2;
+    metis_split3x8(v, h, l, l2);
+    __nv_bfloat16* dst = a6 + r * kx + j0;
+    *reinterpret_cast<uint4*>(dst) = h; *reinterpret_cast<uint4*>(dst + KP) = h; *reinterpret_cast<uint4*>(dst + 2 * KP) = l;
+    *reinterpret_cast<uint4*>(dst + 3 * KP) = h; *reinterpret_cast<uint4*>(dst + 4 * KP) = l2; *reinterpret_cast<uint4*>(dst + 5 * KP) = l;
+    if (j0 == 0)
+      for (int z = 6 * KP; z < kx; z += 8) *reinterpret_cast<uint4*>(a6 + r * kx + z) = make_uint4(0u, 0u, 0u, 0u);
   }
-  if (gram_part) {
-    __shared__ double cd[32 * KP];                      // converted once: FP32 -> FP64 is a slow-rate instruction
-    for (int o = tid; o < 32 * KP; o += 256) cd[o] = (double)cfin[o];
-    __syncthreads();
-    for (int o = tid; o < KP * KP; o += 256) {
-      const int i = o / KP, j = o % KP;
-      double a = 0.0;
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) a += cd[r * KP + i] * cd[r * KP + j];
-      gram_part[(int64_t)blockIdx.x * KP * KP + o] = a;
-    }
-  }
+  gram_add<32, CP>(gt, cd);
+  gram_end(gt, gp, KP, gram_part + (int64_t)(blockIdx.x / metis_cluster_size()) * KP * KP);
 }
 
 // ------------------------------------------------------------------------------------------------
-// Sketch of gathered rows (mma.sync): Zp[chunk][row][j] = sum over the chunk's columns of x[idx[row], col] * Omega[col, j].
-// One CTA = 256 sampled rows x one column chunk (`ccols` = 64 or 256 columns, see sketch_chunk_cols); Omega's slice
-// is generated once per CTA (Philox + quantile table) straight into shared memory, transposed to [j][col] BF16 (its
-// values are BF16 by construction, so the products are exact and only the FP32 accumulation rounds).  Optionally also
-// reduces amax|x| over the rows it reads.  A full sketch of an aligned operand does not come here: it runs on the
-// tcgen05 kernel of the broadcast pass (omega_rows_kernel + metis_launch_coeff_tc in its raw mode).
-constexpr int SKM_ROWS = 256, SKM_COLS = 256, SKM_PITCH = SKM_COLS + 8;
+// Sketch of sampled rows (mma.sync): zp[part][row][j] = sum over the columns of a cluster's CTAs of x[row of the sample, col] * Omega[col, j].
+// One CTA = 256 sampled rows x chunks of `ccols` columns (every gridDim.y-th); Omega's slice is generated per chunk (Philox + quantile table)
+// straight into shared memory, transposed to [j][col] BF16 (its values are BF16 by construction, so the products are exact and only
+// the FP32 accumulation rounds), the first one before the wait for the kernels in front.  The CTAs of a cluster add their sums through
+// distributed shared memory in a fixed order, which leaves at most GR_PARTS partials for the kernel that needs Z (64 of them were added
+// by a launch of its own).  A full sketch does not come here: it runs on the tcgen05 kernel of the broadcast pass (omega_rows_kernel +
+// metis_launch_coeff_tc in its raw mode).
+constexpr int SKM_ROWS = 256, SKM_COLS = 256;
+__host__ __device__ constexpr int skm_pitch(int nt) { return 8 * nt + 4; }             // floats, of the sums in shared memory
+__host__ __device__ constexpr size_t skm_smem(int nt, int ccols) {
+  const size_t om = sizeof(__nv_bfloat16) * nt * 8 * (size_t)(ccols + 8), sums = sizeof(float) * SKM_ROWS * skm_pitch(nt);
+  return om > sums ? om : sums;
+}
 template <int NT>                                      // sketch columns / 8, rounded up
 __global__ void __launch_bounds__(256)
-sketch_mma_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __restrict__ idx, int n_s, int q,
-                  uint64_t seed, const __nv_bfloat16* __restrict__ lut, float* __restrict__ zp, float* __restrict__ amax_out,
-                  int ccols) {
-  metis_pdl_wait_trigger();
+sketch_mma_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, RowSample rs, int n_s, int q, uint64_t seed, const __nv_bfloat16* __restrict__ lut,
+                  float* __restrict__ zp, int ccols, int chunks, float* __restrict__ amax, unsigned long long* __restrict__ keys) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __nv_bfloat16* om = reinterpret_cast<__nv_bfloat16*>(smem);          // [NT*8][SKM_PITCH]
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int64_t col0 = (int64_t)blockIdx.y * ccols;        // ccols <= SKM_COLS columns per CTA
-  const int row0 = blockIdx.x * SKM_ROWS + warp * 32;
-  const int ncols = (int)min((int64_t)ccols, cols - col0);
-  for (int i = tid; i < NT * 8 * SKM_PITCH; i += 256) om[i] = __float2bfloat16_rn(0.0f);
-  __syncthreads();
-  const uint64_t e_lo = (uint64_t)col0 * q, e_hi = (uint64_t)(col0 + ncols) * q;
-  for (uint64_t blk = (e_lo >> 3) + tid; blk <= ((e_hi - 1) >> 3); blk += 256) {
-    const uint4 w = metis_philox_block(blk, seed, METIS_STREAM_OMEGA);
-#pragma unroll
-    for (uint32_t h = 0; h < 8; ++h) {
-      const uint64_t e = (blk << 3) + h;
-      if (e >= e_lo && e < e_hi) {
-        const uint32_t rel = (uint32_t)(e - e_lo);
-        om[(rel % q) * SKM_PITCH + rel / q] = lut[metis_u16_of(w, h)];
-      }
-    }
-  }
-  __syncthreads();
+  __shared__ int ids[SKM_ROWS];
+  __nv_bfloat16* om = reinterpret_cast<__nv_bfloat16*>(smem);          // [NT*8][pitch]
+  float* sums = reinterpret_cast<float*>(smem);                        // [SKM_ROWS][SP], afterwards
+  constexpr int SP = skm_pitch(NT);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, pitch = ccols + 8;
+  const int row0 = blockIdx.x * SKM_ROWS, rw = warp * 32;  // this CTA's rows, this warp's among them
+  ids[tid] = row0 + tid < n_s ? sample_row(rs, row0 + tid) : 0;
+  const bool busy = row0 + rw < n_s;
   float acc[2][NT][4];
 #pragma unroll
   for (int m = 0; m < 2; ++m)
@@ -572,64 +623,110 @@ sketch_mma_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* 
     for (int n = 0; n < NT; ++n)
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.0f;
-  const bool v0 = row0 + g < n_s, v1 = row0 + g + 8 < n_s, v2 = row0 + g + 16 < n_s, v3 = row0 + g + 24 < n_s;
-  const __nv_bfloat16* p0 = x + (int64_t)(v0 ? idx[row0 + g] : 0) * cols + col0;
-  const __nv_bfloat16* p1 = x + (int64_t)(v1 ? idx[row0 + g + 8] : 0) * cols + col0;
-  const __nv_bfloat16* p2 = x + (int64_t)(v2 ? idx[row0 + g + 16] : 0) * cols + col0;
-  const __nv_bfloat16* p3 = x + (int64_t)(v3 ? idx[row0 + g + 24] : 0) * cols + col0;
-  uint32_t amax2 = 0u;
-#pragma unroll 2
-  for (int ks = 0; ks < ncols / 16; ++ks) {
-    const int kk = ks * 16 + 2 * t;
-    uint32_t a[2][4];
-    a[0][0] = v0 ? *reinterpret_cast<const uint32_t*>(p0 + kk) : 0u;
-    a[0][1] = v1 ? *reinterpret_cast<const uint32_t*>(p1 + kk) : 0u;
-    a[0][2] = v0 ? *reinterpret_cast<const uint32_t*>(p0 + kk + 8) : 0u;
-    a[0][3] = v1 ? *reinterpret_cast<const uint32_t*>(p1 + kk + 8) : 0u;
-    a[1][0] = v2 ? *reinterpret_cast<const uint32_t*>(p2 + kk) : 0u;
-    a[1][1] = v3 ? *reinterpret_cast<const uint32_t*>(p3 + kk) : 0u;
-    a[1][2] = v2 ? *reinterpret_cast<const uint32_t*>(p2 + kk + 8) : 0u;
-    a[1][3] = v3 ? *reinterpret_cast<const uint32_t*>(p3 + kk + 8) : 0u;
-    if (amax_out) {
+  for (int i = tid; i < (8 * NT - q) * pitch; i += 256) om[q * pitch + i] = __float2bfloat16_rn(0.0f);         // vectors beyond q
+  bool first = true;
+  for (int ch = blockIdx.y; ch < chunks; ch += gridDim.y) {
+    const int64_t col0 = (int64_t)ch * ccols;              // ccols <= SKM_COLS columns per chunk
+    const int ncols = (int)min((int64_t)ccols, cols - col0);
+    const uint64_t e_lo = (uint64_t)col0 * q, e_hi = (uint64_t)(col0 + ncols) * q;
+    for (uint64_t blk = (e_lo >> 3) + tid; blk <= ((e_hi - 1) >> 3); blk += 256) {
+      const uint4 w = metis_philox_block(blk, seed, METIS_STREAM_OMEGA);
+      const int rel = (int)((int64_t)(blk << 3) - (int64_t)e_lo);      // element of the chunk; the first block may begin before it
+      int c = rel >= 0 ? rel / q : -1, j = rel - c * q;
+      if (rel < 0) { c = -((q - 1 - rel) / q); j = rel - c * q; }
 #pragma unroll
-      for (int m = 0; m < 2; ++m)
+      for (uint32_t h = 0; h < 8; ++h) {
+        if (c >= 0 && c < ncols) om[j * pitch + c] = lut[metis_u16_of(w, h)];
+        if (++j == q) { j = 0; ++c; }
+      }
+    }
+    if (first) {
+      metis_pdl_wait_trigger();
+      if (blockIdx.x == 0 && blockIdx.y == 0) clear_accumulators(amax, keys);
+      first = false;
+    }
+    __syncthreads();
+    if (busy) {
+      const bool v0 = row0 + rw + g < n_s, v1 = row0 + rw + g + 8 < n_s, v2 = row0 + rw + g + 16 < n_s, v3 = row0 + rw + g + 24 < n_s;
+      const __nv_bfloat16 *p0 = x + (int64_t)ids[rw + g] * cols + col0, *p1 = x + (int64_t)ids[rw + g + 8] * cols + col0;
+      const __nv_bfloat16 *p2 = x + (int64_t)ids[rw + g + 16] * cols + col0, *p3 = x + (int64_t)ids[rw + g + 24] * cols + col0;
+      for (int k0 = 0; k0 < ncols; k0 += 64) {             // four steps' loads in flight
+        uint32_t a[4][2][4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const uint32_t ab = a[m][e] & 0x7FFF7FFFu;
-          amax2 = max(ab & 0xFFFFu, amax2 & 0xFFFFu) | (max(ab >> 16, amax2 >> 16) << 16);
+        for (int u = 0; u < 4; ++u) {
+          const int kk = k0 + 16 * u + 2 * t;
+          const bool in = k0 + 16 * u < ncols;
+          a[u][0][0] = in && v0 ? *reinterpret_cast<const uint32_t*>(p0 + kk) : 0u;
+          a[u][0][1] = in && v1 ? *reinterpret_cast<const uint32_t*>(p1 + kk) : 0u;
+          a[u][0][2] = in && v0 ? *reinterpret_cast<const uint32_t*>(p0 + kk + 8) : 0u;
+          a[u][0][3] = in && v1 ? *reinterpret_cast<const uint32_t*>(p1 + kk + 8) : 0u;
+          a[u][1][0] = in && v2 ? *reinterpret_cast<const uint32_t*>(p2 + kk) : 0u;
+          a[u][1][1] = in && v3 ? *reinterpret_cast<const uint32_t*>(p3 + kk) : 0u;
+          a[u][1][2] = in && v2 ? *reinterpret_cast<const uint32_t*>(p2 + kk + 8) : 0u;
+          a[u][1][3] = in && v3 ? *reinterpret_cast<const uint32_t*>(p3 + kk + 8) : 0u;
         }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (k0 + 16 * u >= ncols) break;
+#pragma unroll
+          for (int n = 0; n < NT; ++n) {
+            const __nv_bfloat16* bp = om + (n * 8 + g) * pitch + k0 + 16 * u + 2 * t;
+            const uint32_t b0 = *reinterpret_cast<const uint32_t*>(bp), b1 = *reinterpret_cast<const uint32_t*>(bp + 8);
+            mma_bf16(acc[0][n], a[u][0], b0, b1);
+            mma_bf16(acc[1][n], a[u][1], b0, b1);
+          }
+        }
+      }
+    }
+    __syncthreads();                                       // the next chunk's Omega, or the sums, take its place
+  }
+  if (first) metis_pdl_wait_trigger();                     // a CTA without columns, at the end of a cluster
+  if (busy) {
+#pragma unroll
+    for (int m = 0; m < 2; ++m)
+#pragma unroll
+      for (int n = 0; n < NT; ++n) {
+        float* dst = sums + (rw + m * 16 + g) * SP + n * 8 + 2 * t;
+        *reinterpret_cast<float2*>(dst) = make_float2(acc[m][n][0], acc[m][n][1]);
+        *reinterpret_cast<float2*>(dst + 8 * SP) = make_float2(acc[m][n][2], acc[m][n][3]);
+      }
+  }
+  const uint32_t csize = metis_cluster_size(), rank = metis_cluster_rank(), src = (uint32_t)__cvta_generic_to_shared(sums);
+  __syncthreads();
+  metis_cluster_sync();
+  const int nr = min(SKM_ROWS, n_s - row0);
+  float* out = zp + (int64_t)(blockIdx.y / csize) * n_s * q;
+  for (int o = (int)rank * 256 + tid; o < nr * 2 * NT; o += (int)csize * 256) {  // groups of four entries of a row
+    const int r = o / (2 * NT), c = 4 * (o % (2 * NT));
+    float4 v[GR_CLUSTER];
+#pragma unroll
+    for (uint32_t u = 0; u < GR_CLUSTER; ++u) {
+      v[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (u < csize)
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[u].x), "=f"(v[u].y), "=f"(v[u].z), "=f"(v[u].w)
+                     : "r"(metis_map_to_rank(src + (uint32_t)(r * SP + c) * 4u, u)));
     }
 #pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      const __nv_bfloat16* bp = om + (n * 8 + g) * SKM_PITCH + kk;
-      const uint32_t b0 = *reinterpret_cast<const uint32_t*>(bp), b1 = *reinterpret_cast<const uint32_t*>(bp + 8);
-      mma_bf16(acc[0][n], a[0], b0, b1);
-      mma_bf16(acc[1][n], a[1], b0, b1);
+    for (int u = 1; u < GR_CLUSTER; ++u) { v[0].x += v[u].x; v[0].y += v[u].y; v[0].z += v[u].z; v[0].w += v[u].w; }
+    float* dst = out + (int64_t)(row0 + r) * q + c;
+    if ((q & 3) == 0) { if (c < q) *reinterpret_cast<float4*>(dst) = v[0]; }
+    else {
+      const float e[4] = {v[0].x, v[0].y, v[0].z, v[0].w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) if (c + u < q) dst[u] = e[u];
     }
   }
-  float* dst = zp + (int64_t)blockIdx.y * n_s * q;
-#pragma unroll
-  for (int m = 0; m < 2; ++m)
-#pragma unroll
-    for (int n = 0; n < NT; ++n) {
-      const int r = row0 + m * 16 + g, j = n * 8 + 2 * t;
-      if (r < n_s) { if (j < q) dst[(int64_t)r * q + j] = acc[m][n][0]; if (j + 1 < q) dst[(int64_t)r * q + j + 1] = acc[m][n][1]; }
-      if (r + 8 < n_s) { if (j < q) dst[(int64_t)(r + 8) * q + j] = acc[m][n][2]; if (j + 1 < q) dst[(int64_t)(r + 8) * q + j + 1] = acc[m][n][3]; }
-    }
-  if (amax_out) {
-    uint32_t am = max((amax2 & 0xFFFFu) << 16, amax2 & 0xFFFF0000u);      // ordered bit patterns: a NaN survives
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) am = max(am, __shfl_xor_sync(0xFFFFFFFFu, am, o));
-    if (lane == 0) atomicMax(reinterpret_cast<unsigned int*>(amax_out), am);
-  }
+  metis_cluster_sync();                                    // the others may still be reading
 }
 
 // Full-mode sketch on the tcgen05 path: Omega is written once, transposed and zero-padded to nb rows
 // (omt[j][col], BF16: its values are BF16 by construction), and Z = X Omega runs on the same kernel as the
 // coefficient pass.  One thread per Philox block of eight consecutive elements e = col * q + j.
 __global__ void __launch_bounds__(256)
-omega_rows_kernel(int64_t cols, int q, int nb, uint64_t seed, const __nv_bfloat16* __restrict__ lut, __nv_bfloat16* __restrict__ omt) {
+omega_rows_kernel(int64_t cols, int q, int nb, uint64_t seed, const __nv_bfloat16* __restrict__ lut, __nv_bfloat16* __restrict__ omt, float* __restrict__ amax,
+                  unsigned long long* __restrict__ keys) {
   metis_pdl_wait_trigger();
+  if (keys != nullptr && blockIdx.x == 0) clear_accumulators(amax, keys);
   const uint64_t total = (uint64_t)cols * (uint64_t)q;
   const uint64_t blk = (uint64_t)blockIdx.x * 256 + threadIdx.x;
   if (blk < (total + 7) / 8) {
@@ -685,16 +782,6 @@ reduce_sketch_kernel(const float* __restrict__ part, int slices, int64_t rows, i
   z[r * ldz + j] = acc;
 }
 
-// Tensor-core projection: Mp[part][j][col] = sum over the part's sampled rows r of H[r][j] * x[idx[r], col].
-// The contraction runs over rows of the row-major x, so x tiles are staged in shared memory and read back
-// transposed with ldmatrix; H (FP32) is fed as three BF16 terms.  CTA = 128 columns x one slab of rows.
-// ------------------------------------------------------------------------------------------------
-// Projection M = H^T x over many rows (every row in FULL mode), software-pipelined: the CTA owns 128 columns and
-// a slab of rows, and walks the slab in chunks of 64 rows through a three-stage cp.async ring (x rows gathered
-// by idx, the three BF16 terms of H pre-split and transposed by h_splits_kernel), so the loads of chunk c + 2
-// overlap the MMAs of chunk c.  Same partial layout as project_kernel: Mp[part][j][col].
-constexpr int PP_COLS = 128, PP_K = 64, PP_STAGES = 3, PP_XP = PP_COLS + 8, PP_HP = PP_K + 8;
-
 // hsp[sp][j][r] (r contiguous, ldh >= rows rounded up to 64, zero padded): three-term BF16 split of H[r][j]
 __global__ void __launch_bounds__(256)
 h_splits_kernel(const float* __restrict__ h, int n_s, int q, int jp, int ldh, __nv_bfloat16* __restrict__ hsp, int pitch_h) {
@@ -715,88 +802,148 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
 
-template <int MT>                                      // sketch columns / 16, rounded up
+// ------------------------------------------------------------------------------------------------
+// Projection of sampled rows, M[j][col] = sum over r of H[r][j] x[row r, col], and the Gram matrix M M^T (mma.sync; the contraction runs over rows of the
+// row-major x, so that x tiles are staged in shared memory and read back transposed with ldmatrix; H is fed as three BF16 terms).
+// A CTA owns 64 columns and walks all rows in chunks of 64 through a ring of asynchronous copies (x gathered by row; it does not depend on
+// the kernels before, so its first chunks are on their way before the wait for them); four warps across the columns, two halves
+// of a chunk.  The tensor core truncates its sums: that of the leading terms of 16 rows goes into an FP32 total at once, and what it lost, the same
+// products less the sum, is an accumulator of its own with the smaller terms.
+// With M whole in the CTA its Gram matrix follows from shared memory (see gram_add).  As FP32 multiply-adds over ten slabs of rows, their sum, a
+// Gram kernel and its reduction this was four launches, 21 us at 160 x 4096 with q = 40; now 7.
+constexpr int PG_COLS = 64, PG_K = 64, PG_STAGES = 4, PG_XP = PG_COLS + 8, PG_HP = PG_K + 8;
+__host__ __device__ constexpr size_t pg_smem(int mt) {
+  const size_t ring = (size_t)PG_STAGES * (PG_K * PG_XP * 2 + 3 * mt * 16 * PG_HP * 2), post = sizeof(float) * mt * 16 * (PG_COLS + 4) + SG_SMEM;
+  return ring > post ? ring : post;
+}
+template <int MT>                                       // sketch columns / 16, rounded up
 __global__ void __launch_bounds__(256)
-project_pipe_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, const int* __restrict__ idx, int n_s, int q,
-                    const __nv_bfloat16* __restrict__ hsp, int ldh, int rows_per_part, float* __restrict__ mp) {
-  metis_pdl_wait_trigger();
+project_gram_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, RowSample rs, int n_s, int q, const __nv_bfloat16* __restrict__ hsp, int ldh,
+                    float* __restrict__ m, double* __restrict__ gram_part) {
   extern __shared__ __align__(16) unsigned char psm[];
-  constexpr int XS_BYTES = PP_K * PP_XP * 2, HS_BYTES = 3 * MT * 16 * PP_HP * 2, STAGE = XS_BYTES + HS_BYTES;
+  constexpr int XS_BYTES = PG_K * PG_XP * 2, HS_BYTES = 3 * MT * 16 * PG_HP * 2, STAGE = XS_BYTES + HS_BYTES, MP = PG_COLS + 4;
+  float* Ms = reinterpret_cast<float*>(psm);            // [MT * 16][MP], over the ring, which has been read by then
+  double *tile = reinterpret_cast<double*>(psm + sizeof(float) * MT * 16 * MP), *gp = tile + GR_TILE * LP;
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(psm);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int64_t col0 = (int64_t)blockIdx.x * PP_COLS;
-  const int r_begin = blockIdx.y * rows_per_part, r_end = min(n_s, r_begin + rows_per_part);
-  const int n_chunks = (r_end - r_begin + PP_K - 1) / PP_K;
-  float acc[MT][2][4];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, wn = warp & 3, kh = warp >> 2, n8 = (q + 7) & ~7;
+  const int n_chunks = (n_s + PG_K - 1) / PG_K;
+  const int64_t tiles = (cols + PG_COLS - 1) / PG_COLS;
+  __shared__ int ids[256];                              // the first rows of the sample (beyond them each copy works its row out)
+  ids[tid] = tid < n_s ? sample_row(rs, tid) : 0;
+  auto load_x = [&](int64_t col0, int c) {
+    const uint32_t xs = sbase + (uint32_t)(c % PG_STAGES) * STAGE;
 #pragma unroll
-  for (int m = 0; m < MT; ++m)
-#pragma unroll
-    for (int n = 0; n < 2; ++n)
-#pragma unroll
-      for (int e = 0; e < 4; ++e) acc[m][n][e] = 0.0f;
-
-  auto load_chunk = [&](int c) {
-    const int st = c % PP_STAGES;
-    const int r0 = r_begin + c * PP_K;
-    const uint32_t xs = sbase + (uint32_t)st * STAGE, hs = xs + XS_BYTES;
-    for (int i = tid; i < PP_K * (PP_COLS / 8); i += 256) {
-      const int rr = i >> 4, c8 = (i & 15) * 8;
-      const bool ok = r0 + rr < r_end && col0 + c8 + 8 <= cols;
-      const __nv_bfloat16* src = ok ? x + (int64_t)idx[r0 + rr] * cols + col0 + c8 : x;
-      cp_async16(xs + (uint32_t)(rr * PP_XP + c8) * 2u, src, ok);
-    }
-    for (int i = tid; i < 3 * MT * 16 * (PP_K / 8); i += 256) {
-      const int row = i >> 3, k8 = (i & 7) * 8;          // row = sp * MT*16 + j
-      cp_async16(hs + (uint32_t)(row * PP_HP + k8) * 2u, hsp + (int64_t)row * ldh + r0 + k8, true);
+    for (int u = 0; u < 2; ++u) {
+      const int rr = (tid >> 3) + 32 * u, c8 = (tid & 7) * 8, r = c * PG_K + rr;
+      const bool ok = r < n_s && col0 + c8 + 8 <= cols;
+      cp_async16(xs + (uint32_t)(rr * PG_XP + c8) * 2u, ok ? x + (int64_t)(r < 256 ? ids[r] : sample_row(rs, r)) * cols + col0 + c8 : x, ok);
     }
   };
-
-  for (int c = 0; c < PP_STAGES - 1; ++c) {
-    if (c < n_chunks) load_chunk(c);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
-  for (int c = 0; c < n_chunks; ++c) {
-    asm volatile("cp.async.wait_group %0;" ::"n"(PP_STAGES - 2) : "memory");
-    __syncthreads();                                     // chunk c has landed; everyone is done with chunk c - 1
-    if (c + PP_STAGES - 1 < n_chunks) load_chunk(c + PP_STAGES - 1);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    const int st = c % PP_STAGES;
-    const uint32_t xs = sbase + (uint32_t)st * STAGE, hs = xs + XS_BYTES;
-#pragma unroll
-    for (int ks = 0; ks < PP_K / 16; ++ks) {
-      uint32_t b[2][2];
-#pragma unroll
-      for (int n = 0; n < 2; ++n) {
-        const uint32_t addr = xs + (uint32_t)((ks * 16 + (lane & 15)) * PP_XP + (warp * 2 + n) * 8) * 2u;
-        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(b[n][0]), "=r"(b[n][1]) : "r"(addr));
-      }
-#pragma unroll
-      for (int sp = 0; sp < 3; ++sp)
-#pragma unroll
-        for (int m = 0; m < MT; ++m) {
-          uint32_t a[4];
-          const uint32_t addr = hs + (uint32_t)(((sp * MT + m) * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * PP_HP + ks * 16 + (lane >> 4) * 8) * 2u;
-          asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                       : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(addr));
-          mma_bf16(acc[m][0], a, b[0][0], b[0][1]);
-          mma_bf16(acc[m][1], a, b[1][0], b[1][1]);
-        }
+  auto load_h = [&](int c) {
+    const uint32_t hs = sbase + (uint32_t)(c % PG_STAGES) * STAGE + XS_BYTES;
+    for (int i = tid; i < 3 * MT * 16 * (PG_K / 8); i += 256) {
+      const int row = i >> 3, k8 = (i & 7) * 8;          // row = term * MT * 16 + j
+      cp_async16(hs + (uint32_t)(row * PG_HP + k8) * 2u, hsp + (int64_t)row * ldh + c * PG_K + k8, true);
     }
-  }
-  float* dst = mp + (int64_t)blockIdx.y * q * cols;
+  };
+  GramTiles gt;
+  gram_begin(gt, n8);
+  __syncthreads();
+  bool first = true;
+  for (int64_t ti = blockIdx.x; ti < tiles; ti += gridDim.x) {
+    const int64_t col0 = ti * PG_COLS;
 #pragma unroll
-  for (int m = 0; m < MT; ++m)
+    for (int c = 0; c < PG_STAGES - 1; ++c) if (c < n_chunks) load_x(col0, c);
+    if (first) { metis_pdl_wait_trigger(); first = false; }
 #pragma unroll
-    for (int n = 0; n < 2; ++n) {
-      const int j = m * 16 + g;
-      const int64_t col = col0 + (warp * 2 + n) * 8 + 2 * t;
-      if (col + 1 < cols) {
-        if (j < q) *reinterpret_cast<float2*>(dst + (int64_t)j * cols + col) = make_float2(acc[m][n][0], acc[m][n][1]);
-        if (j + 8 < q) *reinterpret_cast<float2*>(dst + (int64_t)(j + 8) * cols + col) = make_float2(acc[m][n][2], acc[m][n][3]);
+    for (int c = 0; c < PG_STAGES - 1; ++c) {            // (the x copies belong to the first group)
+      if (c < n_chunks) load_h(c);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    float acc[MT][2][4], total[MT][2][4];
+#pragma unroll
+    for (int a = 0; a < MT; ++a)
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) total[a][n][e] = 0.0f;
+    for (int c = 0; c < n_chunks; ++c) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(PG_STAGES - 2) : "memory");
+      __syncthreads();                                     // chunk c has landed; everyone is done with chunk c - 1
+      if (c + PG_STAGES - 1 < n_chunks) { load_x(col0, c + PG_STAGES - 1); load_h(c + PG_STAGES - 1); }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+      const uint32_t xs = sbase + (uint32_t)(c % PG_STAGES) * STAGE, hs = xs + XS_BYTES;
+#pragma unroll
+      for (int k2 = 0; k2 < 2; ++k2) {
+        const int ks = 2 * kh + k2;
+#pragma unroll
+        for (int a = 0; a < MT; ++a)
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[a][n][e] = 0.0f;
+        uint32_t b[4];
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+                     : "r"(xs + (uint32_t)((ks * 16 + (lane & 15)) * PG_XP + wn * 16 + (lane >> 4) * 8) * 2u));
+#pragma unroll
+        for (int a = 0; a < MT; ++a)
+#pragma unroll
+          for (int sp = 0; sp < 3; ++sp) {
+            uint32_t af[4];
+            const uint32_t addr = hs + (uint32_t)(((sp * MT + a) * 16 + (lane & 7) + ((lane >> 3) & 1) * 8) * PG_HP + ks * 16 + (lane >> 4) * 8) * 2u;
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(af[0]), "=r"(af[1]), "=r"(af[2]), "=r"(af[3]) : "r"(addr));
+            mma_bf16(acc[a][0], af, b[0], b[1]);
+            mma_bf16(acc[a][1], af, b[2], b[3]);
+            if (sp == 0) {                                 // what the sum lost: the same products less what it kept
+#pragma unroll
+              for (int n = 0; n < 2; ++n)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { total[a][n][e] += acc[a][n][e]; acc[a][n][e] = -acc[a][n][e]; }
+              mma_bf16(acc[a][0], af, b[0], b[1]);
+              mma_bf16(acc[a][1], af, b[2], b[3]);
+            }
+          }
+#pragma unroll
+        for (int a = 0; a < MT; ++a)
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) total[a][n][e] += acc[a][n][e];
       }
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();                                       // the ring has been read
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {                 // the second half of the chunks is added to the first
+      if (kh == half)
+#pragma unroll
+        for (int a = 0; a < MT; ++a)
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              float& o = Ms[(a * 16 + g + 8 * (e >> 1)) * MP + wn * 16 + n * 8 + 2 * t + (e & 1)];
+              o = half ? o + total[a][n][e] : total[a][n][e];
+            }
+      __syncthreads();
+    }
+    for (int o = tid; o < q * (PG_COLS / 4); o += 256) {
+      const int j = o >> 4, c4 = (o & 15) * 4;
+      if (col0 + c4 < cols) *reinterpret_cast<float4*>(m + (int64_t)j * cols + col0 + c4) = *reinterpret_cast<const float4*>(Ms + j * MP + c4);
+    }
+    for (int o = tid; o < n8 * GR_TILE; o += 256) {        // (vectors q ... n8 - 1 and columns beyond the matrix are zeros)
+      const int j = o >> 6, c = o & 63;
+      tile[c * LP + j] = (double)Ms[j * MP + c];
+    }
+    __syncthreads();
+    gram_add<GR_TILE, LP>(gt, tile);
+    __syncthreads();                                       // the next tile's ring lies over it
+  }
+  if (first) metis_pdl_wait_trigger();                     // a CTA without columns, at the end of a cluster
+  gram_end(gt, gp, q, gram_part + (int64_t)(blockIdx.x / metis_cluster_size()) * q * q);
 }
-
 
 // ------------------------------------------------------------------------------------------------
 // Factors from eigenvectors:  out[j][p] = scale_j sum_i src(i, p) W[i][j]  for a tile of 64 positions p (columns or rows of the
@@ -994,50 +1141,41 @@ factors_kernel(FactorsArgs f, int n_right) {
 // accumulator columns of the tensor-core sketch: k + p rounded up to what the coefficient kernel is built for
 int sketch_tc_cols(int q) { return q <= 48 ? 48 : 96; }
 
-int sketch_chunk_cols(int64_t n_s) { return n_s <= 512 ? 64 : SKM_COLS; }
+// Column chunks of a sampled sketch: 64 columns each (a 160-row sketch has one row block, so narrow chunks are what gives it CTAs), wider ones or more than
+// one to a CTA beyond 128 CTAs, so that the clusters leave at most GR_PARTS partials.
+struct SketchGrid { int ccols, chunks, ctas, csize, parts; };
+SketchGrid sketch_grid(int64_t cols) {
+  SketchGrid s{};
+  s.ccols = cols <= 64 * 128 ? 64 : (cols <= 128 * 128 ? 128 : SKM_COLS);
+  s.chunks = (int)metis_ceil_div(cols, s.ccols);
+  gram_grid(s.chunks, &s.ctas, &s.csize);
+  s.parts = s.ctas / s.csize;
+  return s;
+}
 
 struct SplitWs {
-  size_t amax, idx, zp, omt, z, gram, gram1, linv, evals, evecs, mp, m, basis, coef, keys, evals2, evecs2, bs,
+  size_t amax, zp, omt, z, gram, gram1, linv, evals, evecs, mp, m, basis, coef, keys, evals2, evecs2, bs,
       gram_c, part, a6, b6, hsp, total;
 };
-
-constexpr int PJ_MAX_PARTS = 16;
-
-int project_parts(int64_t n_s, int64_t cols, int* rows_per_part) {
-  const int64_t col_chunks = metis_ceil_div(cols, PJ_COLS);
-  int64_t parts = metis_ceil_div(2 * 148, col_chunks);          // aim at two CTAs per SM
-  if (parts > PJ_MAX_PARTS) parts = PJ_MAX_PARTS;
-  if (parts > metis_ceil_div(n_s, 16)) parts = metis_ceil_div(n_s, 16);
-  if (parts < 1) parts = 1;
-  int64_t rpp = metis_ceil_div(n_s, parts);
-  rpp = metis_ceil_div(rpp, 16) * 16;
-  *rows_per_part = (int)rpp;
-  return (int)metis_ceil_div(n_s, rpp);
-}
 
 SplitWs split_ws_layout(int64_t rows, int64_t cols, int k, int p, int64_t n_s) {
   SplitWs w{};
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
   const int q = k + p;
-  const int64_t chunks = metis_ceil_div(cols, sketch_chunk_cols(n_s));
   w.amax = take(256);
-  w.idx = take(sizeof(int) * (size_t)n_s);
-  // the full-mode tensor-core sketch writes slices x rows x nb partials into the same buffer
+  // the full-mode tensor-core sketch writes slices x rows x nb partials into the buffer of the sampled one's
   const int nb_sk = sketch_tc_cols(q);
-  const size_t zp_mma = (size_t)chunks * n_s * q, zp_tc = (size_t)metis_coeff_slices(rows, cols, nullptr) * rows * nb_sk;
+  const size_t zp_mma = (size_t)GR_PARTS * n_s * q, zp_tc = (size_t)metis_coeff_slices(rows, cols, nullptr) * rows * nb_sk;
   w.zp = take(sizeof(float) * (zp_mma > zp_tc ? zp_mma : zp_tc));
   w.omt = take(sizeof(__nv_bfloat16) * (size_t)nb_sk * cols);
   w.z = take(sizeof(float) * (size_t)n_s * q);
-  w.gram = take(sizeof(double) * 64 * MAXQ * MAXQ);
-  w.linv = take(sizeof(double) * (MAXQ * MAXQ + MAXQ));
+  w.gram = take(sizeof(double) * GR_PARTS * MAXQ * MAXQ);
+  w.linv = take(sizeof(double) * L_DOUBLES);
   w.gram1 = take(sizeof(double) * MAXQ * MAXQ);
   w.evals = take(sizeof(double) * MAXQ);
   w.evecs = take(sizeof(double) * MAXQ * MAXQ);
-  {
-    const size_t per_col_mma = (size_t)PJ_MAX_PARTS * q, per_col_tc = (size_t)8 * ((q + 15) / 16 * 16);   // tensor-core projection: <= 8 slices x jp
-    w.mp = take(sizeof(float) * (per_col_mma > per_col_tc ? per_col_mma : per_col_tc) * cols);
-  }
+  w.mp = take(sizeof(float) * (size_t)8 * ((q + 15) / 16 * 16) * cols);                 // tensor-core projection: at most eight slices
   w.m = take(sizeof(float) * (size_t)q * cols);
   w.basis = take(sizeof(float) * (size_t)k * cols);
   const int kp = (k + 15) / 16 * 16;
@@ -1045,7 +1183,7 @@ SplitWs split_ws_layout(int64_t rows, int64_t cols, int k, int p, int64_t n_s) {
   w.part = take(sizeof(float) * (size_t)metis_coeff_slices(rows, cols, nullptr) * kp * rows);
   w.a6 = take(sizeof(__nv_bfloat16) * (size_t)metis_residual_kx(kp) * rows);
   w.b6 = take(sizeof(__nv_bfloat16) * (size_t)metis_residual_kx(kp) * cols);
-  w.hsp = take(n_s >= 1024 ? sizeof(__nv_bfloat16) * 3 * (size_t)((q + 15) / 16 * 16) * (size_t)((n_s + 63) / 64 * 64) : 0);
+  w.hsp = take(sizeof(__nv_bfloat16) * 3 * (size_t)((q + 15) / 16 * 16) * (size_t)((n_s + 63) / 64 * 64));
   w.bs = take(sizeof(__nv_bfloat16) * 3 * (size_t)kp * cols);
   w.gram_c = take(sizeof(double) * (size_t)metis_ceil_div(rows, 32) * kp * kp);
   w.keys = take(sizeof(unsigned long long) * MAXQ);
@@ -1055,19 +1193,9 @@ SplitWs split_ws_layout(int64_t rows, int64_t cols, int k, int p, int64_t n_s) {
   return w;
 }
 
-int gram_parts(int64_t n_rows, int64_t* rows_per_part) {
-  int parts = (int)metis_ceil_div(n_rows, 64);
-  if (parts > 64) parts = 64;
-  if (parts < 1) parts = 1;
-  int64_t rpp = metis_ceil_div(n_rows, parts);
-  rpp = metis_ceil_div(rpp, GR_TILE) * GR_TILE;
-  *rows_per_part = rpp;
-  return (int)metis_ceil_div(n_rows, rpp);
-}
-
-metis_status_t launch_eig(cudaStream_t s, const double* g, int n, int ld, double* evals, double* evecs) {
+metis_status_t launch_eig(cudaStream_t s, const double* g, int parts, int n, int ld, double* evals, double* evecs) {
   const size_t smem = metis_small::eig_smem(n);
-#define METIS_EIG(NT8) case NT8: METIS_CUDA_TRY(metis_launch_pdl((metis_small::eig_kernel<NT8>), dim3(1), dim3(metis_small::eig_threads(NT8)), smem, s, g, n, ld, evals, evecs)); break
+#define METIS_EIG(NT8) case NT8: METIS_CUDA_TRY(metis_launch_pdl((metis_small::eig_kernel<NT8>), dim3(1), dim3(metis_small::eig_threads(NT8)), smem, s, g, parts, n, ld, evals, evecs)); break
   switch ((n + 7) / 8) {
     METIS_EIG(1); METIS_EIG(2); METIS_EIG(3); METIS_EIG(4); METIS_EIG(5); METIS_EIG(6); METIS_EIG(7); METIS_EIG(8); METIS_EIG(9);
     default: return METIS_ERR_SHAPE;
@@ -1077,15 +1205,55 @@ metis_status_t launch_eig(cudaStream_t s, const double* g, int n, int ld, double
   return METIS_OK;
 }
 
-template <int NJ4>
-void launch_project(dim3 grid, cudaStream_t s, const __nv_bfloat16* x, int64_t cols, const int* idx, int n_s, int q,
-                    const float* h, int rpp, float* mp) {
-  (void)(metis_launch_pdl((project_kernel<NJ4>), dim3(grid), dim3(256), (size_t)(0), s, x, cols, idx, n_s, q, h, rpp, mp)); METIS_COUNT_LAUNCH();
+// Gram partials of vectors given as column slices of a tensor-core pass (see sum_gram_kernel); returns the number of partials
+template <bool TRANS>
+metis_status_t launch_sum_gram(cudaStream_t s, const float* part, int slices, int64_t n_pos, int width, int q, float* out, double* gram, const int* skip, int* parts) {
+  int ctas, csize;
+  gram_grid(metis_ceil_div(n_pos, GR_TILE), &ctas, &csize);
+  *parts = ctas / csize;
+  METIS_CUDA_TRY(metis_launch_pdl_cluster(sum_gram_kernel<TRANS>, dim3((unsigned)ctas), dim3(256), SG_SMEM, s, 0, csize, part, slices, n_pos, width, q, out, gram, skip)); METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+metis_status_t launch_project_gram(cudaStream_t s, const __nv_bfloat16* x, int64_t cols, const RowSample& rs, int n_s, int q, const __nv_bfloat16* hsp, int ldh, float* m, double* gram, int* parts) {
+  int ctas, csize;
+  gram_grid(metis_ceil_div(cols, PG_COLS), &ctas, &csize);
+  *parts = ctas / csize;
+#define METIS_PG(MT) case MT: METIS_CUDA_TRY(metis_launch_pdl_cluster(project_gram_kernel<MT>, dim3((unsigned)ctas), dim3(256), pg_smem(MT), s, 0, csize, x, cols, rs, n_s, q, hsp, ldh, m, gram)); break
+  switch ((q + 15) / 16) {
+    METIS_PG(1); METIS_PG(2); METIS_PG(3); METIS_PG(4); METIS_PG(5);
+    default: return METIS_ERR_SHAPE;
+  }
+#undef METIS_PG
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+metis_status_t launch_sketch(cudaStream_t s, const SketchGrid& sk, const __nv_bfloat16* x, int64_t cols, const RowSample& rs, int n_s, int q, uint64_t seed, const __nv_bfloat16* lut, float* zp,
+                             float* amax, unsigned long long* keys) {
+  const dim3 grid((unsigned)metis_ceil_div(n_s, SKM_ROWS), (unsigned)sk.ctas);
+#define METIS_SK(NT) case NT: METIS_CUDA_TRY(metis_launch_pdl_cluster(sketch_mma_kernel<NT>, grid, dim3(256), skm_smem(NT, sk.ccols), s, 1, sk.csize, x, cols, rs, n_s, q, seed, lut, zp, \
+                                                                       sk.ccols, sk.chunks, amax, keys)); break
+  switch ((q + 7) / 8) {
+    METIS_SK(1); METIS_SK(2); METIS_SK(3); METIS_SK(4); METIS_SK(5); METIS_SK(6); METIS_SK(7); METIS_SK(8); METIS_SK(9);
+    default: return METIS_ERR_SHAPE;
+  }
+#undef METIS_SK
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
+}
+metis_status_t launch_gram_chol(cudaStream_t s, const float* zp, int parts, int width, int n_s, int q, float* z, __nv_bfloat16* hsp, int jp, int64_t ldh) {
+#define METIS_GC(KT) case KT: METIS_CUDA_TRY(metis_launch_pdl_cluster(gram_chol_kernel<KT>, dim3(GC_CLUSTER), dim3(GC_THREADS), gram_chol_smem(n_s, KT), s, 0, GC_CLUSTER, zp, parts, width, n_s, q, z, hsp, jp, ldh)); break
+  switch ((q + 7) / 8) {
+    METIS_GC(1); METIS_GC(2); METIS_GC(3); METIS_GC(4); METIS_GC(5); METIS_GC(6); METIS_GC(7); METIS_GC(8); METIS_GC(9);
+    default: return METIS_ERR_SHAPE;
+  }
+#undef METIS_GC
+  METIS_COUNT_LAUNCH();
+  return METIS_OK;
 }
 
 metis_status_t launch_orth_apply(cudaStream_t s, float* z, int64_t n_s, int q, const double* linvt, const int* skip, __nv_bfloat16* hsp, int jp, int64_t ldh) {
   const dim3 grid((unsigned)metis_ceil_div(n_s, OA_ROWS));
-#define METIS_OA(KT) METIS_CUDA_TRY(metis_launch_pdl((orth_apply_kernel<KT>), grid, dim3(256), oa_smem(KT), s, z, n_s, q, linvt, skip, hsp, jp, ldh)); break
+#define METIS_OA(KT) METIS_CUDA_TRY(metis_launch_pdl((orth_apply_kernel<KT>), grid, dim3(256), (size_t)0, s, z, n_s, q, linvt, skip, hsp, jp, ldh)); break
   switch ((q + 7) / 8) {
     case 1: METIS_OA(1); case 2: METIS_OA(2); case 3: METIS_OA(3); case 4: METIS_OA(4); case 5: METIS_OA(5); case 6: METIS_OA(6); case 7: METIS_OA(7); case 8: METIS_OA(8);
     default: METIS_OA(9);
@@ -1242,7 +1410,7 @@ metis_status_t launch_tridiag(cudaStream_t s, const double* gram1, int n, double
 }
 
 metis_status_t launch_eig_wide(cudaStream_t s, const double* gram1, int n, double* scratch, double* l, double* ycm, double* evals, double* evecs) {
-  if (n <= MAXQ) return launch_eig(s, gram1, n, n, evals, evecs);               // a small rank with a large oversampling
+  if (n <= MAXQ) return launch_eig(s, gram1, 1, n, n, evals, evecs);               // a small rank with a large oversampling
   using namespace metis_wide;
   const size_t nn = (size_t)n * n;
   double *x[2] = {scratch, scratch + nn}, *w = scratch + 2 * nn, *sm = scratch + 3 * nn, *g1 = scratch + 4 * nn, *e = scratch + 5 * nn;
@@ -1321,8 +1489,8 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
   if (src_amax != nullptr) METIS_CUDA_TRY(cudaMemcpyAsync(amax, src_amax, sizeof(float), cudaMemcpyDeviceToDevice, s));
   const __nv_bfloat16* xr = x;
   if (!full) {
-    METIS_CUDA_TRY(metis_launch_pdl((sample_rows_kernel), dim3((unsigned)metis_ceil_div(n_s, 256)), dim3(256), (size_t)(0), s, idx, (int)n_s, rows, seed, 0,
-                                    (float*)nullptr, (unsigned long long*)nullptr)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((sample_rows_kernel), dim3((unsigned)metis_ceil_div(n_s, 256)), dim3(256), (size_t)(0), s, idx, (int)n_s,
+                                    RowSample{(uint32_t)(rows / n_s), seed})); METIS_COUNT_LAUNCH();
     METIS_CUDA_TRY(metis_launch_pdl(metis_wide::gather_rows_kernel, dim3((unsigned)metis_ceil_div(n_s * (cols / 8), 256)), dim3(256), (size_t)0, s, x, cols,
                                     (const int*)idx, (int)n_s, xs)); METIS_COUNT_LAUNCH();
     xr = xs;
@@ -1331,7 +1499,8 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
   const int nbq = (q + WIDE_SK - 1) / WIDE_SK * WIDE_SK;
   {
     const uint64_t blocks = ((uint64_t)cols * q + 7) / 8;
-    METIS_CUDA_TRY(metis_launch_pdl((omega_rows_kernel), dim3((unsigned)metis_ceil_div((int64_t)blocks, 256)), dim3(256), (size_t)(0), s, cols, q, nbq, seed, ctx->quantile_lut, omt)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((omega_rows_kernel), dim3((unsigned)metis_ceil_div((int64_t)blocks, 256)), dim3(256), (size_t)(0), s, cols, q, nbq, seed, ctx->quantile_lut, omt,
+                                    (float*)nullptr, (unsigned long long*)nullptr)); METIS_COUNT_LAUNCH();
     const int slices = metis_coeff_slices(n_r, cols, nullptr);
     for (int j0 = 0; j0 < q; j0 += WIDE_SK) {
       const int qg = q - j0 < WIDE_SK ? q - j0 : WIDE_SK;
@@ -1431,11 +1600,11 @@ metis_status_t split_wide(metis_context* ctx, const __nv_bfloat16* x, int64_t ro
       METIS_TRY(launch_gemm64(sf, g));
     }
   }
-  METIS_CUDA_TRY(metis_launch_pdl((split_status_kernel), dim3(1), dim3(32), (size_t)(0), s, (const float*)amax, (const double*)evals, k, ctx->dev_status)); METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
+  const metis_split_checks checks{amax, evals, k, ctx->dev_status};
   metis_nvfp4_t lq = out->left_q, rq = out->right_q;
   lq.rows = k; lq.k_len = rows; rq.rows = k; rq.k_len = cols;
-  METIS_TRY(metis_launch_quantize_factors(out->left, rows, out->right, cols, k, rounding, seed, amax + 1, amax + 2, &lq, &rq, sf));
+  METIS_TRY(metis_launch_quantize_factors(out->left, rows, out->right, cols, k, rounding, seed, amax + 1, amax + 2, &lq, &rq, sf, nullptr, &checks));
   return metis_join(ctx, s, 0);
 }
 
@@ -1459,10 +1628,6 @@ int64_t metis_default_sample_count(int64_t rows, int32_t q) {
 }
 
 metis_status_t metis_split_set_attrs() {
-#define METIS_OA_ATTR(KT) METIS_CUDA_TRY(cudaFuncSetAttribute(orth_apply_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)oa_smem(KT)))
-  METIS_OA_ATTR(1); METIS_OA_ATTR(2); METIS_OA_ATTR(3); METIS_OA_ATTR(4); METIS_OA_ATTR(5); METIS_OA_ATTR(6); METIS_OA_ATTR(7); METIS_OA_ATTR(8); METIS_OA_ATTR(9);
-#undef METIS_OA_ATTR
-  METIS_CUDA_TRY(cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CHOL_SMEM));
 #define METIS_FR_ATTR(KT) METIS_CUDA_TRY(cudaFuncSetAttribute(basis_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fr_smem(MAXQ))); \
   METIS_CUDA_TRY(cudaFuncSetAttribute(factors_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fr_smem(MAXQ)))
   METIS_FR_ATTR(1); METIS_FR_ATTR(2); METIS_FR_ATTR(3); METIS_FR_ATTR(4); METIS_FR_ATTR(5); METIS_FR_ATTR(6); METIS_FR_ATTR(7); METIS_FR_ATTR(8);
@@ -1470,7 +1635,12 @@ metis_status_t metis_split_set_attrs() {
 #define METIS_EIG_ATTR(NT8) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_small::eig_kernel<NT8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_small::eig_smem(8 * NT8)))
   METIS_EIG_ATTR(1); METIS_EIG_ATTR(2); METIS_EIG_ATTR(3); METIS_EIG_ATTR(4); METIS_EIG_ATTR(5); METIS_EIG_ATTR(6); METIS_EIG_ATTR(7); METIS_EIG_ATTR(8); METIS_EIG_ATTR(9);
 #undef METIS_EIG_ATTR
-  METIS_CUDA_TRY(cudaFuncSetAttribute(gram_chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GC_MAX_SMEM));
+#define METIS_GC_ATTR(KT) METIS_CUDA_TRY(cudaFuncSetAttribute(gram_chol_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gram_chol_smem(GC_MAX_ROWS, KT))); \
+  METIS_CUDA_TRY(cudaFuncSetAttribute(sketch_mma_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)skm_smem(KT, SKM_COLS)))
+  METIS_GC_ATTR(1); METIS_GC_ATTR(2); METIS_GC_ATTR(3); METIS_GC_ATTR(4); METIS_GC_ATTR(5); METIS_GC_ATTR(6); METIS_GC_ATTR(7); METIS_GC_ATTR(8); METIS_GC_ATTR(9);
+#undef METIS_GC_ATTR
+  METIS_CUDA_TRY(cudaFuncSetAttribute(sum_gram_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SG_SMEM));
+  METIS_CUDA_TRY(cudaFuncSetAttribute(sum_gram_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SG_SMEM));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::JC_SMEM));
 #define METIS_WT_ATTR(R, C, T) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::tridiag_chol_kernel<R, C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::cm_smem(metis_wide::WT_MAX)))
   METIS_WT_ATTR(6, 3, false); METIS_WT_ATTR(9, 3, false); METIS_WT_ATTR(9, 4, false); METIS_WT_ATTR(10, 4, true);
@@ -1483,8 +1653,7 @@ metis_status_t metis_split_set_attrs() {
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::chol_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::cm_smem(metis_wide::CM_MAX)));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::chol_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::CW_SMEM));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::trsm_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::TW_SMEM));
-#define METIS_PP_ATTR(MTV) METIS_CUDA_TRY(cudaFuncSetAttribute(project_pipe_kernel<MTV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-      (int)((size_t)PP_STAGES * (PP_K * PP_XP * 2 + 3 * (MTV) * 16 * PP_HP * 2))))
+#define METIS_PP_ATTR(MT) METIS_CUDA_TRY(cudaFuncSetAttribute(project_gram_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pg_smem(MT)))
   METIS_PP_ATTR(1); METIS_PP_ATTR(2); METIS_PP_ATTR(3); METIS_PP_ATTR(4); METIS_PP_ATTR(5);
 #undef METIS_PP_ATTR
   return METIS_OK;
@@ -1532,11 +1701,8 @@ size_t metis_split_ws_bytes(int64_t rows, int64_t cols, int k, int p) {
     const size_t b = wide_ws_layout(rows, cols, k, p, metis_default_sample_count(rows, k + p), false).total;
     return a > b ? a : b;
   }
-  // Every buffer grows with the sample count except the sketch partials, whose chunk width steps from 64 to 256
-  // columns above 512 sampled rows: the FULL sketch (n_s = rows) and a 512-row sample bound every other case.
-  const size_t full = split_ws_layout(rows, cols, k, p, rows).total;
-  const size_t narrow = split_ws_layout(rows, cols, k, p, rows < 512 ? rows : 512).total;
-  return full > narrow ? full : narrow;
+  // every buffer grows with the sample count: the FULL sketch (n_s = rows) bounds every other case
+  return split_ws_layout(rows, cols, k, p, rows).total;
 }
 
 metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int64_t rows, int64_t cols, int64_t ld, int32_t k, int32_t p,
@@ -1612,7 +1778,6 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   if (out->left_q.sf_layout == METIS_SF_TILED && rows % 64) return METIS_ERR_SHAPE;
   if (out->right_q.sf_layout == METIS_SF_TILED && cols % 64) return METIS_ERR_SHAPE;
 
-  int* idx = reinterpret_cast<int*>(wsb + L.idx);
   float* zp = reinterpret_cast<float*>(wsb + L.zp);
   float* z = reinterpret_cast<float*>(wsb + L.z);
   double* gram = reinterpret_cast<double*>(wsb + L.gram);
@@ -1638,124 +1803,50 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   const int kx6 = metis_residual_kx((k + 15) / 16 * 16);
   metis_context* ctx = h;
   const int kp = (k + 15) / 16 * 16;
-  // (1) row sample (clears the amax slots of x, left and right, the condition flag and the sign keys), (2) sketch (tensor cores; Omega
-  // generated per CTA into shared memory).  amax|x| for the residual's tensor scale: fused into the sketch pass (FULL) or
-  // the broadcast pass (SAMPLED).
-  METIS_CUDA_TRY(metis_launch_pdl((sample_rows_kernel), dim3((unsigned)metis_ceil_div(n_s, 256)), dim3(256), (size_t)(0), s, idx, (int)n_s, rows, seed, full ? 1 : 0, amax, keys)); METIS_COUNT_LAUNCH();
-  if (src_amax != nullptr) METIS_CUDA_TRY(cudaMemcpyAsync(amax, src_amax, sizeof(float), cudaMemcpyDeviceToDevice, s));
-  const int ccols = sketch_chunk_cols(n_s);
-  const int chunks = (int)metis_ceil_div(cols, ccols);
+  // (1) row sample and (2) sketch on the tensor cores; the first kernel also clears the amax slots of x, left and right, the condition flag and the
+  // sign keys.  amax|x| for the residual's tensor scale: fused into the sketch pass (FULL) or the broadcast pass (SAMPLED).
+  const RowSample rs{full ? 0u : (uint32_t)(rows / n_s), seed};
   __nv_bfloat16* omt = reinterpret_cast<__nv_bfloat16*>(wsb + L.omt);
-  const int nb_sk = sketch_tc_cols(q);
-  const bool sketch_tc = full && q <= 96 && metis_coeff_tc_usable(x, omt, cols, nb_sk / 3);
-  if (sketch_tc) {
+  const int nb_sk = sketch_tc_cols(q), jp = (q + 15) / 16 * 16, ldh = (int)((n_s + 63) / 64 * 64);
+  const bool one_cluster = n_s <= GC_MAX_ROWS;
+  int parts = 0, slices_z = 0, width_z = q;             // the sketch's partials: zp[slices_z][n_s][width_z]
+  if (full) {
     const uint64_t blocks = ((uint64_t)cols * q + 7) / 8;
-    METIS_CUDA_TRY(metis_launch_pdl((omega_rows_kernel), dim3((unsigned)metis_ceil_div((int64_t)blocks, 256)), dim3(256), (size_t)(0), s, cols, q, nb_sk, seed, ctx->quantile_lut, omt)); METIS_COUNT_LAUNCH();
+    METIS_CUDA_TRY(metis_launch_pdl((omega_rows_kernel), dim3((unsigned)metis_ceil_div((int64_t)blocks, 256)), dim3(256), (size_t)(0), s, cols, q, nb_sk, seed, ctx->quantile_lut, omt,
+                                    amax, keys)); METIS_COUNT_LAUNCH();
+    if (src_amax != nullptr) METIS_CUDA_TRY(cudaMemcpyAsync(amax, src_amax, sizeof(float), cudaMemcpyDeviceToDevice, s));
     METIS_TRY(metis_launch_coeff_tc(ctx, x, rows, cols, omt, nb_sk / 3, zp, amax, 1, s));
-    const int slices = metis_coeff_slices(rows, cols, nullptr);
-    METIS_CUDA_TRY(metis_launch_pdl((reduce_sketch_kernel), dim3((unsigned)metis_ceil_div(rows * q, 256)), dim3(256), (size_t)(0), s, zp, slices, rows, nb_sk, q, z, q)); METIS_COUNT_LAUNCH();
+    slices_z = metis_coeff_slices(rows, cols, nullptr); width_z = nb_sk;
   } else {
-    const int nt = (q + 7) / 8;
-    const size_t smem = sizeof(__nv_bfloat16) * nt * 8 * SKM_PITCH;
-    dim3 grid((unsigned)metis_ceil_div(n_s, SKM_ROWS), (unsigned)chunks);
-    float* am = full ? amax : nullptr;                  // FULL mode: amax|x| comes out of this pass
-    switch (nt) {
-      case 1: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<1>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      case 2: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<2>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      case 3: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<3>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      case 4: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<4>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      case 5: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<5>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      case 6: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<6>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      case 7: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<7>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      case 8: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<8>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-      default: METIS_CUDA_TRY(metis_launch_pdl((sketch_mma_kernel<9>), dim3(grid), dim3(256), (size_t)(smem), s, x, cols, idx, (int)n_s, q, seed, ctx->quantile_lut, zp, am, ccols)); break;
-    }
-    METIS_COUNT_LAUNCH();
+    const SketchGrid sk = sketch_grid(cols);
+    METIS_TRY(launch_sketch(s, sk, x, cols, rs, (int)n_s, q, seed, ctx->quantile_lut, zp, amax, keys));
+    if (src_amax != nullptr) METIS_CUDA_TRY(cudaMemcpyAsync(amax, src_amax, sizeof(float), cudaMemcpyDeviceToDevice, s));
+    slices_z = sk.parts;
   }
-  if (!sketch_tc) {
-    METIS_CUDA_TRY(metis_launch_pdl((reduce_partials_kernel), dim3((unsigned)metis_ceil_div(n_s * q, 256)), dim3(256), (size_t)(0), s, zp, chunks, n_s * q, z)); METIS_COUNT_LAUNCH();
-  }
-  // (3) CholeskyQR2: orthonormal basis H of range(Z), in place
-  // the projection on tensor cores wants the BF16 splits of H as well (n_s >= 1024)
-  const bool split_h = n_s >= 1024 && cols % 8 == 0, one_cta = gram_chol_smem(n_s, q) <= GC_MAX_SMEM;
-  const int jp = (q + 15) / 16 * 16, ldh = (int)((n_s + 63) / 64 * 64);
-  if (one_cta) {
-    // a short sketch: Gram matrix and factorisation in one CTA; the product with L^-T on many CTAs unless the sketch
-    // was ill-conditioned, in which case the first kernel has done both passes itself and the second returns at once
-    METIS_CUDA_TRY(metis_launch_pdl((gram_chol_kernel), dim3(1), dim3(GC_THREADS), gram_chol_smem(n_s, q), s, z, (int)n_s, q, linvt, cond_flag)); METIS_COUNT_LAUNCH();
-    METIS_TRY(launch_orth_apply(s, z, n_s, q, linvt, cond_flag, nullptr, jp, ldh));
+  // (3) CholeskyQR2: orthonormal basis H of range(Z), its BF16 splits for the projection
+  if (one_cluster) {
+    METIS_TRY(launch_gram_chol(s, zp, slices_z, width_z, (int)n_s, q, z, hsp, jp, ldh));
   } else {
     for (int pass = 0; pass < 2; ++pass) {
-      int64_t rpp; const int parts = gram_parts(n_s, &rpp);
       const int* skip = pass == 0 ? nullptr : cond_flag;
-      METIS_CUDA_TRY(metis_launch_pdl((gram_kernel), dim3(parts), dim3(256), (size_t)(0), s, z, n_s, q, q, 1, rpp, gram, skip)); METIS_COUNT_LAUNCH();
-      METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(q * q, 32)), dim3(128), (size_t)(0), s, gram, parts, q * q, gram1, skip)); METIS_COUNT_LAUNCH();
-      METIS_CUDA_TRY(metis_launch_pdl((chol_kernel), dim3(1), dim3(512), CHOL_SMEM, s, gram1, q, linvt, skip, pass == 0 ? cond_flag : nullptr)); METIS_COUNT_LAUNCH();
-      METIS_TRY(launch_orth_apply(s, z, n_s, q, linvt, skip, split_h ? hsp : nullptr, jp, ldh));
+      if (pass == 0) METIS_TRY(launch_sum_gram<false>(s, zp, slices_z, n_s, width_z, q, z, gram, skip, &parts));
+      else METIS_TRY(launch_sum_gram<false>(s, z, 1, n_s, q, q, nullptr, gram, skip, &parts));
+      METIS_CUDA_TRY(metis_launch_pdl((chol_kernel), dim3(1), dim3(CHOL_THREADS), (size_t)0, s, (const double*)gram, parts, q, linvt, skip, pass == 0 ? cond_flag : (int*)nullptr)); METIS_COUNT_LAUNCH();
+      METIS_TRY(launch_orth_apply(s, z, n_s, q, linvt, skip, hsp, jp, ldh));
     }
   }
-  // (4) M = H^T x[S,:], eigen-decomposition of M M^T, right basis
-  {
-    int rpp; int parts;
-    bool project_tc = false;
-    if (split_h) {
-      if (one_cta) {                                    // that factorisation leaves the splits to a kernel of their own
-        METIS_CUDA_TRY(metis_launch_pdl(h_splits_kernel, dim3((unsigned)metis_ceil_div(ldh, 256), (unsigned)jp), dim3(256), (size_t)0, s, z, (int)n_s, q, jp, ldh, hsp, q)); METIS_COUNT_LAUNCH();
-      }
-      parts = (int)metis_ceil_div(n_s, 512);
-      if (parts > PJ_MAX_PARTS) parts = PJ_MAX_PARTS;
-      rpp = (int)(metis_ceil_div(metis_ceil_div(n_s, parts), PP_K) * PP_K);
-      parts = (int)metis_ceil_div(n_s, rpp);
-      const int mt = jp / 16;
-      project_tc = full && metis_project_tc_usable(x, hsp, cols, jp);
-      if (project_tc) {
-        // every row, in order: M^T = x^T H on the tcgen05 kernel of the broadcast pass (x as an MN-major operand)
-        METIS_TRY(metis_launch_project_tc(ctx, x, rows, cols, hsp, jp, ldh, mp, s));
-        dim3 rgrid((unsigned)metis_ceil_div(cols, 32), (unsigned)metis_ceil_div(q, 32));
-        METIS_CUDA_TRY(metis_launch_pdl((reduce_proj_kernel), rgrid, dim3(256), (size_t)(0), s, mp, metis_project_slices(rows, cols), cols, jp, q, m)); METIS_COUNT_LAUNCH();
-      } else {
-      dim3 grid((unsigned)metis_ceil_div(cols, PP_COLS), (unsigned)parts);
-      const size_t psmem = (size_t)PP_STAGES * (PP_K * PP_XP * 2 + 3 * jp * PP_HP * 2);
-#define METIS_PP(MTV) { \
-        METIS_CUDA_TRY(metis_launch_pdl((project_pipe_kernel<MTV>), grid, dim3(256), psmem, s, x, cols, idx, (int)n_s, q, hsp, ldh, rpp, mp)); }
-      switch (mt) {
-        case 1: METIS_PP(1); break;
-        case 2: METIS_PP(2); break;
-        case 3: METIS_PP(3); break;
-        case 4: METIS_PP(4); break;
-        default: METIS_PP(5); break;
-      }
-#undef METIS_PP
-      METIS_COUNT_LAUNCH();
-      }
-    } else {
-    parts = project_parts(n_s, cols, &rpp);
-    dim3 grid((unsigned)metis_ceil_div(cols, PJ_COLS), (unsigned)parts);
-    const int nj4 = (q + 7) / 8;
-    switch (nj4) {
-      case 1: launch_project<1>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      case 2: launch_project<2>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      case 3: launch_project<3>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      case 4: launch_project<4>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      case 5: launch_project<5>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      case 6: launch_project<6>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      case 7: launch_project<7>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      case 8: launch_project<8>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-      default: launch_project<9>(grid, s, x, cols, idx, (int)n_s, q, z, rpp, mp); break;
-    }
-    }
-    if (!project_tc) {
-      METIS_CUDA_TRY(metis_launch_pdl((reduce_partials_kernel), dim3((unsigned)metis_ceil_div((int64_t)q * cols, 256)), dim3(256), (size_t)(0), s, mp, parts, (int64_t)q * cols, m)); METIS_COUNT_LAUNCH();
-    }
+  // (4) M = H^T x[S,:] and M M^T, eigen-decomposition, right basis
+  if (full && n_s >= 1024 && metis_project_tc_usable(x, hsp, cols, jp)) {
+    // every row, in order: M^T = x^T H on the tcgen05 kernel of the broadcast pass (x as an MN-major operand)
+    METIS_TRY(metis_launch_project_tc(ctx, x, rows, cols, hsp, jp, ldh, mp, s));
+    METIS_TRY(launch_sum_gram<true>(s, mp, metis_project_slices(rows, cols), cols, jp, q, m, gram, nullptr, &parts));
+  } else {
+    METIS_TRY(launch_project_gram(s, x, cols, rs, (int)n_s, q, hsp, ldh, m, gram, &parts));
   }
-  {
-    int64_t rpp; const int parts = gram_parts(cols, &rpp);
-    METIS_CUDA_TRY(metis_launch_pdl((gram_kernel), dim3(parts), dim3(256), (size_t)(0), s, m, cols, q, 1, cols, rpp, gram, nullptr)); METIS_COUNT_LAUNCH();
-    METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(q * q, 32)), dim3(128), (size_t)(0), s, gram, parts, q * q, gram1, nullptr)); METIS_COUNT_LAUNCH();
-    METIS_TRY(launch_eig(s, gram1, q, q, evals, evecs));
-  }
+  METIS_TRY(launch_eig(s, gram, parts, q, q, evals, evecs));
   // (5) right basis and its splits; coefficients of every row in the basis, (6) fused residual + quantizer
   const int n_cta_c = (int)metis_ceil_div(rows, 32);
+  int csize_c = 1;                                        // CTAs of the coefficients' last kernel to a Gram partial
   const int n_cta_cols = (int)metis_ceil_div(cols, FR_POS), n_cta_rows = (int)metis_ceil_div(rows, FR_POS);
   float* rb = full ? out->right : basis;
   METIS_TRY(launch_basis(s, n_cta_cols, fr_smem(q), m, cols, q, k, kp, evals, evecs, rb, full ? (__nv_bfloat16*)nullptr : bs, b6, kx6, full ? out->sigma : nullptr, full ? keys : nullptr, amax + 2));
@@ -1770,12 +1861,16 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     // tensor-core pass over x (column slices), then the slices are summed and the Gram partials formed
     METIS_TRY(metis_launch_coeff_tc(ctx, x, rows, cols, bs, kp, part, amax, 0, s));
     const int slices = metis_coeff_slices(rows, cols, nullptr);
+    while (csize_c < GR_CLUSTER && csize_c < n_cta_c) csize_c *= 2;
+    const dim3 grid_c((unsigned)metis_ceil_div(n_cta_c, csize_c) * (unsigned)csize_c);
+#define METIS_CF(KP) METIS_CUDA_TRY(metis_launch_pdl_cluster((coef_finish_kernel<KP>), grid_c, dim3(256), (size_t)(0), s, 0, csize_c, (const float*)part, slices, rows, coef, gram_c, a6, kx6)); break
     switch (kp) {
-      case 16: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<16>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
-      case 32: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<32>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
-      case 48: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<48>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
-      default: METIS_CUDA_TRY(metis_launch_pdl((coef_finish_kernel<64>), dim3(n_cta_c), dim3(256), (size_t)(0), s, part, slices, rows, coef, gram_c, a6, kx6)); break;
+      case 16: METIS_CF(16);
+      case 32: METIS_CF(32);
+      case 48: METIS_CF(48);
+      default: METIS_CF(64);
     }
+#undef METIS_CF
     METIS_COUNT_LAUNCH();
   }
   {
@@ -1789,13 +1884,17 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     // goes to a (high-priority) side stream and is joined back at the end of the call
     METIS_TRY(metis_fork(ctx, s, 1));
     METIS_TRY(metis_launch_residual_tc(ctx, x, nullptr, k, kp, qp, amax, t0, t1, residual_dense, a6, b6, s));
-    METIS_CUDA_TRY(metis_launch_pdl((split_status_kernel), dim3(1), dim3(32), (size_t)(0), s, amax, evals, k, ctx->dev_status)); METIS_COUNT_LAUNCH();
   }
   cudaStream_t sf = ctx->side[0];
   if (!full) {
     // (7) Rayleigh-Ritz on C^T C (Gram partials came out of the broadcast pass), rotate both factors
-    METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(kp * kp, 32)), dim3(128), (size_t)(0), sf, gram_c, n_cta_c, kp * kp, gram1, nullptr)); METIS_COUNT_LAUNCH();
-    METIS_TRY(launch_eig(sf, gram1, k, kp, evals2, evecs2));
+    int parts_c = (int)metis_ceil_div(n_cta_c, csize_c);
+    const double* g2 = gram_c;
+    if (parts_c > GR_PARTS) {                             // more than 4096 rows: summed on many CTAs first
+      METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(kp * kp, 32)), dim3(128), (size_t)(0), sf, (const double*)gram_c, parts_c, kp * kp, gram1, (const int*)nullptr)); METIS_COUNT_LAUNCH();
+      g2 = gram1; parts_c = 1;
+    }
+    METIS_TRY(launch_eig(sf, g2, parts_c, k, kp, evals2, evecs2));
     FactorsArgs f{};
     f.w = evecs2; f.ldw = k; f.n_in = k; f.k = k; f.kp = kp;
     f.basis = basis; f.cols = cols; f.right = out->right; f.keys = keys; f.amax_right = amax + 2;
@@ -1803,9 +1902,10 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     METIS_TRY(launch_factors(sf, f, n_cta_cols, n_cta_rows));
   }
   METIS_CUDA_TRY(cudaGetLastError());
-  // (8) apply the sign convention and quantize the factors (stored transposed: k x rows, k x cols; blocks along the long dimension)
+  // (8) apply the sign convention and quantize the factors (stored transposed: k x rows, k x cols; blocks along the long dimension), status of the split
   metis_nvfp4_t lq = out->left_q, rq = out->right_q;
   lq.rows = k; lq.k_len = rows; rq.rows = k; rq.k_len = cols;
-  METIS_TRY(metis_launch_quantize_factors(out->left, rows, out->right, cols, k, rounding, seed, amax + 1, amax + 2, &lq, &rq, sf, keys));
+  const metis_split_checks checks{amax, evals, k, ctx->dev_status};
+  METIS_TRY(metis_launch_quantize_factors(out->left, rows, out->right, cols, k, rounding, seed, amax + 1, amax + 2, &lq, &rq, sf, keys, &checks));
   return metis_join(ctx, s, 0);
 }

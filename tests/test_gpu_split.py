@@ -108,6 +108,33 @@ def test_wide_ranks_on_the_cluster_solver(ctx, case, mode_name):
     _check_against_oracle(B, h, x, k, p, mode, seed=5, rounding=1 if rank == 64 else 0)
 
 
+@pytest.mark.parametrize("rows,cols,k,p,mode_name,n_sample", [
+    (64, 256, 4, 1, "full", 0),               # odd sketch width, fewer rows than the cluster has CTAs for
+    (192, 8256, 8, 3, "sampled", 0),          # 128-column chunks of the sketch, the last one ragged
+    (256, 16448, 8, 4, "sampled", 0),         # 256-column chunks, more than one tile of columns per CTA of the projection
+    (960, 448, 12, 4, "full", 0),             # projection of all rows without the tcgen05 pass
+    (1024, 448, 8, 8, "full", 0), (1088, 448, 4, 3, "full", 0),           # last length of the cluster's orthonormalisation, first of the long one
+    (2048, 512, 20, 5, "sampled", 1040),      # a long sample: partials of a width that is no multiple of four
+    (4160, 320, 16, 8, "sampled", 0),         # more Gram partials of the coefficients than the eigen-solver adds
+    (1088, 576, 64, 8, "sampled", 304),       # 38 groups of rows for eight CTAs
+])
+def test_chain_kernels_at_their_edges(ctx, rows, cols, k, p, mode_name, n_sample):
+    B, h = ctx
+    x, _ = synth.planted(rows, cols, k, 100 * (np.sqrt(rows) + np.sqrt(cols)), 10 * (np.sqrt(rows) + np.sqrt(cols)), 1.0, 91 + rows + k)
+    from gpu_util import to_dev_bf16, rel_fro
+    mode = B.SKETCH_FULL if mode_name == "full" else B.SKETCH_SAMPLED
+    op, dense = h.split(to_dev_bf16(x), k, p, sketch=mode, n_sample=n_sample, seed=5, want_residual=True)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    sp = osp.split(x.astype(np.float64), k, p, osp.MODE_FULL if mode_name == "full" else osp.MODE_SAMPLED, seed=5, n_sample=n_sample)
+    assert np.max(np.abs(op.sigma.cpu().numpy() - sp.sigma) / sp.sigma) < 1e-5
+    # FP32 residual of X-sized terms, as in _check_against_oracle; the coefficients are FP32 sums over the columns on the tensor core, which truncates
+    # them: up to 2^-24 of the sum for each of cols / 64 / 8 boxes of a slice, so that the noise grows with the columns beyond 8192
+    growth = 4.0 * np.sqrt(max(k, 64)) * max(1.0, cols / 8192)
+    assert rel_fro(dense.cpu().numpy(), sp.residual) < max(1e-6, growth * 2.0 ** -24 * np.linalg.norm(x) / np.linalg.norm(sp.residual))
+    assert rel_fro(op.right.cpu().numpy().T, sp.right) < 1e-3 and rel_fro(op.left.cpu().numpy().T, sp.left) < 1e-3
+
+
 def test_planted_noise_free_spectrum_is_recovered(ctx):
     """Closed form: with no bulk and rank <= k+p the sketch captures the whole matrix and Lambda is the planted
     spectrum.  The library only takes bfloat16 input, whose rounding adds a full-rank perturbation of relative size
