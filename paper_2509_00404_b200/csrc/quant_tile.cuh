@@ -66,6 +66,45 @@ __device__ __forceinline__ void fill_r_table(float* tab, float s_T, int tid, int
     tab[b] = (b == 0 || b == 127) ? 0.0f : __fdiv_rn(1.0f, __fmul_rn(metis_e4m3_value((uint32_t)b), s_T));
 }
 
+// The scale byte of a block: the smallest E4M3 value not below t = min(amax / six, 448), the quotient rounded to nearest.
+// six is the same for all blocks, so its reciprocal is taken once and the quotient corrected twice with its exact remainder.  The first
+// correction leaves it within one unit in the last place, the second, with a correctly rounded reciprocal, rounds it as a division does
+// (Markstein, IBM J. Res. Dev. 34, 1990).  That holds while no remainder is subnormal: amax >= lo with 2^-70 <= six <= 2^100 and lo = six 2^-30
+// keeps the last bit of every product above 2^-149.  Other blocks are divided (zero, a NaN, one far below the tensor's maximum); an infinity
+// gives a NaN here, and the largest scale like there.
+struct BlockScaler { float six, inv, lo; };
+__device__ __forceinline__ BlockScaler block_scaler(float s_T) {
+  BlockScaler q;
+  q.six = __fmul_rn(6.0f, s_T);
+  const bool usable = q.six >= 0x1p-70f && q.six <= 0x1p100f;
+  q.inv = usable ? __frcp_rn(q.six) : 0.0f;
+  q.lo = usable ? q.six * 0x1p-30f : __int_as_float(0x7F800000);
+  return q;
+}
+// t 2^-120, rounded up, has E4M3's exponents as an FP32 number, its subnormals among FP32's: one addition rounds either kind up to E4M3
+__device__ __forceinline__ uint32_t e4m3_ceil_byte(float t) { return (__float_as_uint(__fmul_ru(t, 0x1p-120f)) + 0xFFFFFu) >> 20; }
+__device__ __forceinline__ uint32_t scale_byte(float amax, const BlockScaler& q) {
+  float t;
+  if (amax >= q.lo && q.inv != 0.0f) {
+    t = __fmul_rn(amax, q.inv);
+    t = __fmaf_rn(__fmaf_rn(-t, q.six, amax), q.inv, t);
+    t = __fmaf_rn(__fmaf_rn(-t, q.six, amax), q.inv, t);
+  } else {
+    t = __fdiv_rn(amax, q.six);
+  }
+  return e4m3_ceil_byte(fminf(t, 448.0f));
+}
+
+// two products at once
+__device__ __forceinline__ void mul2(float& d0, float& d1, float a0, float a1, float b0, float b1) {
+  asm("{ .reg .b64 a, b, d;\n"
+      "mov.b64 a, {%2, %3};\n"
+      "mov.b64 b, {%4, %5};\n"
+      "mul.rn.f32x2 d, a, b;\n"
+      "mov.b64 {%0, %1}, d; }"
+      : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+
 // four round-to-nearest-even code bytes (eight values) packed into one word
 __device__ __forceinline__ uint32_t e2m1x8_rne(float a0, float a1, float a2, float a3, float a4, float a5, float a6, float a7) {
   uint32_t w;
@@ -86,36 +125,43 @@ template <bool COMPL> constexpr uint32_t SR_SEL_HI = COMPL ? 0x5324u : 0x4325u;
 template <bool COMPL>
 __device__ __forceinline__ uint32_t sr_term(uint32_t word, bool hi) { return __byte_perm(word, 0xFFu, hi ? SR_SEL_HI<COMPL> : SR_SEL_LO<COMPL>); }
 
-// Eight stochastically rounded codes in one word; term[i] = sr_term of draw i.  The same decision as metis_e2m1_sr,
-// arranged for the instruction mix of the SM (integer logic, shifts and compares issue at half the FP32 / IMAD rate, and bound
-// this code):
-//   b = max(a, RU(a/2 + 1/2)) maps a < 1 onto [1/2, 1] (the E2M1 grid {0, 1/2, 1} becomes {1/2, 3/4, 1}: one
-//       mantissa bit per binade like the values from 1 up) and leaves a >= 1 alone, without a select;
-//   with S = 4 bits(b) + (65535 - u) 256 + 255 the 22 mantissa bits below the grid bit carry into it exactly when  frac * 65536 > u
-//       (4 frac22 + (65535 - u) 256 + 255 >= 2^24  <=>  frac22 > 64 u): comparison, selection and increment in one multiply-add.  Either S is
-//       formed (COMPL) or its complement, ~S = term - 4 bits(b), where the draw enters as it is: complementing the Philox words costs half an
-//       instruction per element, which the quantizer saves; the residual pass, at its 96 registers a thread, spills then
-//       (8192 x 14336, k = 32, on a slower part: 214 us with S, 227 with ~S);
-//   the magnitude code is bits 24 .. 26 of S, minus 4 modulo 8: the top bytes of four elements are gathered by byte permutations, the
-//       two words of even and odd elements are merged and the complement and the eight "- 4" taken off together;
-//   the sign nibbles are gathered with one funnel shift per element and masked once per word.
-// (Against a compare per element with the draw shifted up and codes packed one by one: residual_tc_kernel 236 -> 204 us at 8192 x 14336, k = 32, the
-// minimum per element below included, 199 us with the scale byte without branches; quantize_kernel 472 -> 371 us at 16384 x 14336 with
-// both orientations, its third CTA per SM included, 340 us with the complement formed here, that scale byte and one block of code per loop.)
+// Stochastically rounded codes.  The same decision as metis_e2m1_sr, arranged for the instruction mix of the SM (integer logic, shifts and
+// compares issue at half the FP32 / IMAD rate, and bound this code):
+//   z = RU(a 2^-126), a = |y| <= 6, is an FP32 number with E2M1's exponents: a < 1 becomes subnormal, rounded up to 22 bits below
+//       the grid's spacing of 1/2, and a >= 1 is only scaled.  The bits of z are then the code in units of 2^22, for every binade
+//       alike: no select, no offset;
+//   with S = 4 bits(z) + (65535 - u) 256 + 255 the 22 bits below the grid carry into the code exactly when  frac * 65536 > u
+//       (4 frac22 + (65535 - u) 256 + 255 >= 2^24  <=>  frac22 > 64 u): comparison, selection and increment in one multiply-add, and the
+//       top byte of S is the code.  Either S is formed (COMPL) or its complement, ~S = term - 4 bits(z), where the draw enters as it is:
+//       complementing the Philox words costs half an instruction per element, which the quantizer saves (the residual pass, at its 96 registers
+//       a thread, spills then);
+//   the codes of eight elements are gathered by byte permutations, those of even and of odd elements, and merged in one multiply-add;
+//   the sign nibbles are gathered with one funnel shift per element, or, from BF16 pairs, with half a permutation.
+// 16384 x 14336 BF16 in both orientations: 472 us with a compare per element; 341 us with a < 1 mapped onto
+// [1/2, 1] by max(a, RU(a/2 + 1/2)), four masks and shifts per word of codes and a division per block; 317 us so, 309 us with the maxima
+// on BF16 pairs, 276 us (30.4 instructions) with whole tiles in a kernel of their own (quantize_kernel).
+// Residual pass, 8192 x 14336, k = 32: 231 -> 219 us (226 uncomplemented); 16384 x 4096, k = 64: 149 -> 139 us.
+constexpr float SR_SCALE = 0x1p-126f;
+template <bool COMPL>
+__device__ __forceinline__ uint32_t sr_sum(float z, uint32_t term) { return COMPL ? __float_as_uint(z) * 4u + term : term - __float_as_uint(z) * 4u; }
+// s: sums of eight elements; sgn: their signs on the top bits of the nibbles, other bits are ignored
+template <bool COMPL>
+__device__ __forceinline__ uint32_t e2m1x8_gather(const uint32_t (&s)[8], uint32_t sgn) {
+  const uint32_t even = __byte_perm(__byte_perm(s[0], s[2], 0x0073u), __byte_perm(s[4], s[6], 0x7300u), 0x7610u);
+  const uint32_t odd = __byte_perm(__byte_perm(s[1], s[3], 0x0073u), __byte_perm(s[5], s[7], 0x7300u), 0x7610u);
+  // bytes 0 .. 7, or 255 less that: F0 | 15 - c and, with the four ones shifted in, 16 (15 - c) | 15
+  const uint32_t mag = COMPL ? even + odd * 16u : ~(even & (odd * 16u + 15u));
+  return mag | (sgn & 0x88888888u);
+}
 template <bool COMPL>
 __device__ __forceinline__ uint32_t e2m1x8_sr(const float (&y)[8], const uint32_t (&term)[8]) {
   uint32_t s[8], sgn = 0u;
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
-    const float a = fabsf(y[i]);                           // at most 6 (the caller has seen to it)
-    const uint32_t b4 = __float_as_uint(fmaxf(a, __fmaf_ru(a, 0.5f, 0.5f))) * 4u;
-    s[i] = COMPL ? b4 + term[i] : term[i] - b4;
+    s[i] = sr_sum<COMPL>(__fmul_ru(fabsf(y[i]), SR_SCALE), term[i]);
     sgn = __funnelshift_l(__float_as_uint(y[i]), sgn, 4);  // top nibble of y (sign and three exponent bits) shifted in
   }
-  const uint32_t even = __byte_perm(__byte_perm(s[0], s[2], 0x0073u), __byte_perm(s[4], s[6], 0x7300u), 0x7610u);
-  const uint32_t odd = __byte_perm(__byte_perm(s[1], s[3], 0x0073u), __byte_perm(s[5], s[7], 0x7300u), 0x7610u);
-  const uint32_t mag = ((even & 0x0F0F0F0Fu) | ((odd * 16u) & 0xF0F0F0F0u));
-  return ((mag & 0x77777777u) ^ (COMPL ? 0x44444444u : 0x33333333u)) | (sgn & 0x88888888u);
+  return e2m1x8_gather<COMPL>(s, sgn);
 }
 
 // largest magnitude of a block: eight three-input maxima, which pass a NaN over or (KEEP_NAN) on
@@ -135,24 +181,19 @@ __device__ __forceinline__ float amax16(const float (&v)[16]) {
   return max3<KEEP_NAN>(lo, hi, hi);
 }
 
-// the byte of metis_e4m3_ceil without its branches: 0 for zero and a NaN
-__device__ __forceinline__ uint32_t e4m3_ceil_byte(float t) {
-  const uint32_t normal = ((__float_as_uint(t) + 0xFFFFFu) >> 20) - (120u << 3), subnormal = __float2uint_ru(__fmul_rn(t, 512.0f));
-  return t > 0.015625f ? normal : subnormal;
-}
-
 // encode_block with the multiplier looked up in a table filled by fill_r_table (same bytes as encode_block).
 // term[i] = sr_term<COMPL> of draw i (only read with stochastic rounding).
 template <bool COMPL>
-__device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&term)[16], bool sr, float six_s_T,
+__device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const uint32_t (&term)[16], bool sr, const BlockScaler& q,
                                                      const float* r_tab, uint32_t (&packed)[2]) {
   if (!sr) {
-    const uint32_t byte = e4m3_ceil_byte(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f));
+    const uint32_t byte = scale_byte(amax16<false>(v), q);
     const float r = r_tab[byte];
-    packed[0] = e2m1x8_rne(__fmul_rn(v[0], r), __fmul_rn(v[1], r), __fmul_rn(v[2], r), __fmul_rn(v[3], r),
-                           __fmul_rn(v[4], r), __fmul_rn(v[5], r), __fmul_rn(v[6], r), __fmul_rn(v[7], r));
-    packed[1] = e2m1x8_rne(__fmul_rn(v[8], r), __fmul_rn(v[9], r), __fmul_rn(v[10], r), __fmul_rn(v[11], r),
-                           __fmul_rn(v[12], r), __fmul_rn(v[13], r), __fmul_rn(v[14], r), __fmul_rn(v[15], r));
+    float y[16];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mul2(y[2 * i], y[2 * i + 1], v[2 * i], v[2 * i + 1], r, r);
+    packed[0] = e2m1x8_rne(y[0], y[1], y[2], y[3], y[4], y[5], y[6], y[7]);
+    packed[1] = e2m1x8_rne(y[8], y[9], y[10], y[11], y[12], y[13], y[14], y[15]);
     return byte;
   }
   float y0[8], y1[8];
@@ -160,17 +201,17 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
 #pragma unroll
   for (int i = 0; i < 8; ++i) { t0[i] = term[i]; t1[i] = term[8 + i]; }
   const float amax = amax16<true>(v);
-  uint32_t byte = e4m3_ceil_byte(fminf(__fdiv_rn(amax, six_s_T), 448.0f));
+  uint32_t byte = scale_byte(amax, q);
   float r = r_tab[byte];
   // values beyond 6 saturate, and a NaN is stored as 6.  They only occur where the block scale itself is saturated, the product
   // of the block maximum rounds up, or an element is a NaN, and the block maximum shows it, so the other blocks are spared a
   // minimum per element.  The scale of a block is that of its other elements (448 where there are none).
   if (__fmul_rn(amax, r) <= 6.0f) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { y0[i] = __fmul_rn(v[i], r); y1[i] = __fmul_rn(v[8 + i], r); }
+    for (int i = 0; i < 4; ++i) { mul2(y0[2 * i], y0[2 * i + 1], v[2 * i], v[2 * i + 1], r, r); mul2(y1[2 * i], y1[2 * i + 1], v[8 + 2 * i], v[9 + 2 * i], r, r); }
   } else {
     if (isnan(amax)) {
-      byte = e4m3_ceil_byte(fminf(__fdiv_rn(amax16<false>(v), six_s_T), 448.0f));
+      byte = scale_byte(amax16<false>(v), q);
       r = r_tab[byte];
     }
 #pragma unroll
@@ -182,6 +223,108 @@ __device__ __forceinline__ uint32_t encode_block_tab(const float (&v)[16], const
   packed[0] = e2m1x8_sr<COMPL>(y0, t0);
   packed[1] = e2m1x8_sr<COMPL>(y1, t1);
   return byte;
+}
+
+// ---- the same for BF16 values in packed words, two elements each (lo, hi) ----
+// Against the form on single values: the sign is masked once per word, both multiplications are two at a time, the maximum is taken on the bit
+// patterns of a pair (a NaN is above every number) and the signs come by permutation from the words.
+
+// largest pattern of either half over N words, signs left out; a NaN passes on
+template <int N>
+__device__ __forceinline__ uint32_t max_words(const uint32_t (&w)[N]) {
+  uint32_t m = w[0];
+#pragma unroll
+  for (int i = 1; i < N; ++i) asm("max.NaN.xorsign.abs.bf16x2 %0, %0, %1;" : "+r"(m) : "r"(w[i]));
+  return m & 0x7FFF7FFFu;
+}
+// Sums of eight words' elements: lo[i], hi[i] of word i, scaled by r0 and r1.  `fits`: no product is above 6 or a NaN; else the products are
+// clamped (a NaN to 6) and the signs of the words' elements whose product is a NaN cleared.
+__device__ __forceinline__ void sr_words(uint32_t (&w)[8], const uint32_t (&draw)[8], float r0, float r1, bool fits, uint32_t (&lo)[8], uint32_t (&hi)[8]) {
+  float z0[8], z1[8];
+  if (fits) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t m = w[i] & 0x7FFF7FFFu;
+      asm("{ .reg .b64 a, b, c, d;\n"
+          "mov.b64 a, {%2, %3};\n"
+          "mov.b64 b, {%4, %5};\n"
+          "mov.b64 c, {%6, %6};\n"
+          "mul.rn.f32x2 d, a, b;\n"
+          "mul.rp.f32x2 d, d, c;\n"
+          "mov.b64 {%0, %1}, d; }"
+          : "=f"(z0[i]), "=f"(z1[i]) : "f"(__uint_as_float(m << 16)), "f"(__uint_as_float(m & 0xFFFF0000u)), "f"(r0), "f"(r1), "f"(SR_SCALE));
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float a = __fmul_rn(__uint_as_float((w[i] << 16) & 0x7FFFFFFFu), r0), b = __fmul_rn(__uint_as_float(w[i] & 0x7FFF0000u), r1);
+      if (isnan(a)) w[i] &= ~0x8000u;
+      if (isnan(b)) w[i] &= ~0x80000000u;
+      z0[i] = __fmul_ru(fminf(a, 6.0f), SR_SCALE);
+      z1[i] = __fmul_ru(fminf(b, 6.0f), SR_SCALE);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    lo[i] = sr_sum<false>(z0[i], sr_term<false>(draw[i], false));
+    hi[i] = sr_sum<false>(z1[i], sr_term<false>(draw[i], true));
+  }
+}
+// the scale byte of a block whose maximum is a NaN is that of its other elements (448 where there are none)
+__device__ __forceinline__ uint32_t scale_byte_bf16(uint32_t pattern, const BlockScaler& q) { return scale_byte(__uint_as_float(pattern << 16), q); }
+__device__ __forceinline__ float max_no_nan(float m, uint32_t pattern) { return fmaxf(m, fabsf(__uint_as_float(pattern << 16))); }
+
+// a block of 16 in eight words
+__device__ __forceinline__ uint32_t encode_words_sr(uint32_t (&w)[8], const uint32_t (&draw)[8], const BlockScaler& q, const float* r_tab, uint32_t (&packed)[2]) {
+  const uint32_t m2 = max_words(w), m = max(m2 & 0xFFFFu, m2 >> 16);
+  uint32_t byte = scale_byte_bf16(m, q);
+  float r = r_tab[byte];
+  const bool fits = __fmul_rn(__uint_as_float(m << 16), r) <= 6.0f;
+  if (!fits && m > 0x7F80u) {
+    float o = __int_as_float(0x7FC00000);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) o = max_no_nan(max_no_nan(o, w[i] & 0xFFFFu), w[i] >> 16);
+    byte = scale_byte(o, q);
+    r = r_tab[byte];
+  }
+  uint32_t lo[8], hi[8];
+  sr_words(w, draw, r, r, fits, lo, hi);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t s[8] = {lo[4 * h], hi[4 * h], lo[4 * h + 1], hi[4 * h + 1], lo[4 * h + 2], hi[4 * h + 2], lo[4 * h + 3], hi[4 * h + 3]};
+    const uint32_t a = __byte_perm(w[4 * h], w[4 * h + 1], 0x7351u), b = __byte_perm(w[4 * h + 2], w[4 * h + 3], 0x7351u);   // top bytes: lo, lo, hi, hi
+    const uint32_t e = __byte_perm(a, b, 0x5410u) >> 4, o = __byte_perm(a, b, 0x7632u);
+    packed[h] = e2m1x8_gather<false>(s, (e & 0x0F0F0F0Fu) | (o & 0xF0F0F0F0u));
+  }
+  return byte;
+}
+
+// two blocks side by side, of the lo and of the hi elements of 16 words; the draws' words stand 64 words apart
+__device__ __forceinline__ void encode_columns_sr(uint32_t (&w)[16], const uint32_t* draws, const BlockScaler& q, const float* r_tab, uint32_t& byte0, uint32_t& byte1,
+                                                  uint32_t (&p0)[2], uint32_t (&p1)[2]) {
+  const uint32_t m = max_words(w), m0 = m & 0xFFFFu, m1 = m >> 16;
+  byte0 = scale_byte_bf16(m0, q); byte1 = scale_byte_bf16(m1, q);
+  float r0 = r_tab[byte0], r1 = r_tab[byte1];
+  const bool fits = __fmul_rn(__uint_as_float(m0 << 16), r0) <= 6.0f && __fmul_rn(__uint_as_float(m1 << 16), r1) <= 6.0f;
+  if (!fits && (m0 > 0x7F80u || m1 > 0x7F80u)) {
+    float o0 = __int_as_float(0x7FC00000), o1 = o0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) { o0 = max_no_nan(o0, w[i] & 0xFFFFu); o1 = max_no_nan(o1, w[i] >> 16); }
+    byte0 = scale_byte(o0, q); byte1 = scale_byte(o1, q);
+    r0 = r_tab[byte0]; r1 = r_tab[byte1];
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t wh[8], draw[8], s0[8], s1[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { wh[i] = w[8 * h + i]; draw[i] = draws[(8 * h + i) * 64]; }
+    sr_words(wh, draw, r0, r1, fits, s0, s1);
+    const uint32_t a = __byte_perm(wh[0], wh[2], 0x7351u), b = __byte_perm(wh[4], wh[6], 0x7351u);     // top bytes: lo, lo, hi, hi
+    const uint32_t c = __byte_perm(wh[1], wh[3], 0x7351u), d = __byte_perm(wh[5], wh[7], 0x7351u);
+    const uint32_t e0 = __byte_perm(a, b, 0x5410u) >> 4, o0 = __byte_perm(c, d, 0x5410u), e1 = __byte_perm(a, b, 0x7632u) >> 4, o1 = __byte_perm(c, d, 0x7632u);
+    p0[h] = e2m1x8_gather<false>(s0, (e0 & 0x0F0F0F0Fu) | (o0 & 0xF0F0F0F0u));
+    p1[h] = e2m1x8_gather<false>(s1, (e1 & 0x0F0F0F0Fu) | (o1 & 0xF0F0F0F0u));
+  }
 }
 
 }  // namespace metis_qt

@@ -187,7 +187,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     static_assert(PATCH_F * 4 % 128 == 0 && PATCH_F * 4 >= 1024, "a warp's patch is the source of tensor copies");
     const int c_layout = FAST ? (int)METIS_SF_TILED : p.c_layout, r_layout = FAST ? (int)METIS_SF_TILED : p.r_layout;
     const float s_T = metis_tensor_scale(*g.amax_src);
-    const float six_s_T = __fmul_rn(6.0f, s_T);
+    const metis_qt::BlockScaler scaler = metis_qt::block_scaler(s_T);
     metis_qt::fill_r_table(r_tab, s_T, (int)threadIdx.x - 64, 32 * N_EW);
     asm volatile("bar.sync 1, %0;" ::"n"(32 * N_EW) : "memory");       // the epilogue warps only
     if (blockIdx.x == 0 && threadIdx.x == 64) {
@@ -266,8 +266,8 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         uint32_t u0[16], u1[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) { v0[i] = v[i]; v1[i] = v[16 + i]; u0[i] = sr ? metis_qt::sr_term<true>(nw[i >> 1], i & 1) : 0u; u1[i] = sr ? metis_qt::sr_term<true>(nw[8 + (i >> 1)], i & 1) : 0u; }
-        const uint32_t sb0 = encode_block_tab<true>(v0, u0, sr, six_s_T, r_tab, pk0);
-        const uint32_t sb1 = encode_block_tab<true>(v1, u1, sr, six_s_T, r_tab, pk1);
+        const uint32_t sb0 = encode_block_tab<true>(v0, u0, sr, scaler, r_tab, pk0);
+        const uint32_t sb1 = encode_block_tab<true>(v1, u1, sr, scaler, r_tab, pk1);
         if (!FAST && row_ok) {
           uint8_t* cp = p.c_codes + row * c_kbytes + c0 / 2;
           METIS_DBG_GUARD(g.dev_status, row * c_kbytes + c0 / 2, blk1_ok ? 16 : 8, p.rows * c_kbytes) {
@@ -320,7 +320,7 @@ residual_tc_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
             d[i] = sr ? __byte_perm(upatch[rb * 176 + i * 10 + (cb >> 1)], 0xFFu, term_sel) : 0u;   // sr_term of this column's half
           }
           uint32_t pk[2];
-          const uint32_t sb = encode_block_tab<true>(t, d, sr, six_s_T, r_tab, pk);
+          const uint32_t sb = encode_block_tab<true>(t, d, sr, scaler, r_tab, pk);
           pkr[hf][0] = pk[0]; pkr[hf][1] = pk[1];
           if (!FAST && col_ok && rb_ok) METIS_DBG_GUARD(g.dev_status, col * r_kbytes + (slab_row0 + 16 * rb) / 2, 8, p.cols * r_kbytes)
             *reinterpret_cast<uint2*>(p.r_codes + col * r_kbytes + (slab_row0 + 16 * rb) / 2) = make_uint2(pk[0], pk[1]);

@@ -226,3 +226,32 @@ def test_a_nan_is_stored_as_six_and_its_block_is_scaled_by_the_others(ctx, dtype
         os_ = np.where(at.reshape(at.shape[0], -1, 16).all(axis=2), np.uint8(126), os_)
         assert np.array_equal(s, os_)
         assert np.array_equal(c[~at], oc[~at]) and bool((c[at] == 7).all())
+
+
+@pytest.mark.parametrize("tensor_scale", [1.0 / 448, 0.013, 2.0 ** -80, 2.0 ** 98])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("rounding", [onv.ROUND_RNE, onv.ROUND_SR])
+def test_whole_tiles_and_block_scales_at_their_edges(ctx, dtype, rounding, tensor_scale):
+    """Matrices of whole tiles have a kernel of their own, and the block scale's quotient is formed from a reciprocal where the tensor scale
+    allows it and divided where not (2^-80): blocks whose maximum is every E4M3 value times 6 tensor scales, the numbers beside it, and
+    ones far below the smallest scale, byte for byte the oracle's codes, from a contiguous operand and from a view with rows off the
+    32-byte boundary (the general kernel)."""
+    B, h = ctx
+    rng = np.random.default_rng(79)
+    ts = np.float32(tensor_scale)
+    x = rng.uniform(-1, 1, (256, 384)).astype(np.float32)
+    grid = np.array([onv.E4M3_POS[b] for b in range(1, 127)], dtype=np.float32) * (np.float32(6) * ts)
+    edge = np.stack([grid, np.nextafter(grid, np.float32(0)), np.nextafter(grid, np.float32(np.inf)), grid * np.float32(2.0 ** -25)]).reshape(-1)
+    blocks = x.reshape(-1, 16)
+    blocks[: edge.size] *= edge[:, None]
+    blocks[: edge.size, 5] = edge
+    blocks[edge.size:] *= ts * np.float32(40)
+    blocks[-3:] *= np.float32(2.0 ** -36)
+    if dtype == torch.bfloat16:
+        x = synth.to_bf16_values(x)
+    xd = torch.from_numpy(x).to(dtype).cuda()
+    _compare(B, h, x, xd, B.BLOCKS_BOTH, rounding, B.SF_TILED, tensor_scale=ts)
+    wide = torch.zeros((256, 384 + 8), dtype=dtype, device="cuda")
+    wide[:, 8:] = xd
+    _compare(B, h, x, wide[:, 8:], B.BLOCKS_BOTH, rounding, B.SF_TILED, tensor_scale=ts)
+    _compare(B, h, x[:128, :128].copy(), xd[:128, :128].contiguous(), B.BLOCKS_ALONG_ROWS, rounding, B.SF_TILED, tensor_scale=ts)
