@@ -10,7 +10,9 @@ namespace {
 // so that narrow rows do not idle the block, and one 32-bit division per unit finds the unit's place (a 64-bit division per
 // vector and scalar FP32 loads held the kernel at 3.6 TB/s for BF16 and 1.1 TB/s for FP32).  Units are walked
 // from the end of the tensor to its start: the quantizer that follows reads from the start, which is then what L2 holds.
-template <int DTYPE>
+// STREAM: a tensor well beyond the L2 is loaded evict-first, so that what the L2 holds of others is not written back or lost for lines nobody finds
+// again (16384 x 14336 BF16: 83 -> 69 us, the quantizer behind it as before).
+template <int DTYPE, bool STREAM>
 __global__ void __launch_bounds__(256)
 amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, int tpr, int narrow, uint32_t segs, uint32_t units, float* __restrict__ out) {
   // |x| as a bit pattern: non-negative floats order like their bit patterns, infinity above every number and a
@@ -30,7 +32,10 @@ amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, 
       // rows of at most tpr vectors: the unit is UNROLL row groups; longer rows: UNROLL steps along the row
       const int64_t r = narrow ? r0 + (int64_t)j * rpp : r0, c = narrow ? c0 : c0 + (int64_t)j * tpr;
       q[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (r < rows && c < vecs) q[j] = __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(x) + (r * ld + c * E) * (16 / E)));
+      if (r < rows && c < vecs) {
+        const uint4* at = reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(x) + (r * ld + c * E) * (16 / E));
+        q[j] = STREAM ? __ldcs(at) : __ldg(at);
+      }
     }
 #pragma unroll
     for (int j = 0; j < UNROLL; ++j) {
@@ -333,6 +338,8 @@ metis_status_t metis_quantize_set_attrs() {
   return METIS_OK;
 }
 
+constexpr int64_t METIS_L2_BYTES = 126ll << 20;
+
 metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t cols, int64_t ld, float* amax_out,
                                  cudaStream_t s, bool zeroed) {
   const bool bf = dtype == METIS_BF16;
@@ -346,13 +353,24 @@ metis_status_t metis_launch_amax(const void* x, int dtype, int64_t rows, int64_t
   int tpr = 256;
   while (tpr > 1 && tpr / 2 >= vecs) tpr /= 2;
   const bool narrow = vecs <= tpr;                                              // rows of at most one step of the block
+  // Longer rows: a unit is 8 tpr vectors of each of 256 / tpr rows, and what lies beyond a row's end or the last row is not loaded.  Of at least 32
+  // threads a row (512 bytes side by side) the count that makes the fewest units, the largest of equals.
+  auto units_of = [&](int t) { return metis_ceil_div(rows, 256 / t) * metis_ceil_div(vecs, (int64_t)t * 8); };
+  if (!narrow)
+    for (int t = 128; t >= 32; t /= 2)
+      if (units_of(t) < units_of(tpr)) tpr = t;
   const int64_t segs = narrow ? 1 : metis_ceil_div(vecs, (int64_t)tpr * 8);
-  const int64_t groups = narrow ? metis_ceil_div(rows, (int64_t)(256 / tpr) * 8) : rows;
+  const int64_t groups = metis_ceil_div(rows, (int64_t)(256 / tpr) * (narrow ? 8 : 1));
   const int64_t units = groups * segs;
   if (units > 0xFFFFFFFFll) return METIS_ERR_SHAPE;
-  const unsigned grid = (unsigned)(units < 148 * 8 ? units : 148 * 8);
-  if (bf) METIS_CUDA_TRY(metis_launch_pdl((amax_kernel<METIS_BF16>), dim3(grid), dim3(256), (size_t)0, s, x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out));
-  else METIS_CUDA_TRY(metis_launch_pdl((amax_kernel<METIS_FP32>), dim3(grid), dim3(256), (size_t)0, s, x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out));
+  // Resident CTAs that walk the units (one reduction and one atomic each) up to 5/4 of the L2 (8192 x 4160 FP32, 136 MB: 66.1 us, streamed 66.4).  Beyond a CTA per unit: 12 and 13 units a CTA
+  // left an eighth of the last round idle (16384 x 14336 BF16, with its quantizer: 224 -> 214 us, evict-first 208; 16384 x 8192 134 -> 123; of
+  // tensors that fit, 4160 x 2752 FP32 29.0 -> 29.1, evict-first 32.2: the quantizer finds less).
+  const bool stream = rows * cols * (bf ? 2 : 4) > METIS_L2_BYTES / 4 * 5 && units <= 0x7FFFFFFFll;
+  const unsigned grid = (unsigned)(stream || units < 148 * 8 ? units : 148 * 8);
+  auto launch = [&](auto kernel) { return metis_launch_pdl(kernel, dim3(grid), dim3(256), (size_t)0, s, x, rows, cols, ld, tpr, narrow ? 1 : 0, (uint32_t)segs, (uint32_t)units, amax_out); };
+  if (bf) METIS_CUDA_TRY(stream ? launch(amax_kernel<METIS_BF16, true>) : launch(amax_kernel<METIS_BF16, false>));
+  else METIS_CUDA_TRY(stream ? launch(amax_kernel<METIS_FP32, true>) : launch(amax_kernel<METIS_FP32, false>));
   METIS_COUNT_LAUNCH();
   METIS_CUDA_TRY(cudaGetLastError());
   return METIS_OK;

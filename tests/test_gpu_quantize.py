@@ -255,3 +255,23 @@ def test_whole_tiles_and_block_scales_at_their_edges(ctx, dtype, rounding, tenso
     wide[:, 8:] = xd
     _compare(B, h, x, wide[:, 8:], B.BLOCKS_BOTH, rounding, B.SF_TILED, tensor_scale=ts)
     _compare(B, h, x[:128, :128].copy(), xd[:128, :128].contiguous(), B.BLOCKS_ALONG_ROWS, rounding, B.SF_TILED, tensor_scale=ts)
+
+
+@pytest.mark.parametrize("dtype,rows,cols,pad", [(torch.float32, 37, 1088, 64), (torch.float32, 41, 2752, 64), (torch.bfloat16, 5, 2112, 64), (torch.bfloat16, 9, 6208, 8),
+                                                 (torch.bfloat16, 10083, 8192, 16), (torch.float32, 10081, 4096, 0)])
+def test_tensor_amax_of_few_threads_a_row_and_beyond_the_l2(ctx, dtype, rows, cols, pad):
+    """Strided rows that are cut into units of 32, 64 or 128 threads (with rows left over in the last unit), and tensors just above 5/4 of the
+    L2, a CTA per unit: the largest element counts wherever it stands, and those beyond the operand's columns do not."""
+    B, h = ctx
+    full = torch.rand((rows, cols + pad), device="cuda").to(dtype)
+    full[:, cols:] = 1000.0
+    x = full[:, :cols]
+    step = 16 // x.element_size()
+    spots = {(0, 0), (0, cols - 1), (rows - 1, 0), (rows - 1, cols - 1)} | {(rows - 1 - i, (i * 37 * step + i) % cols) for i in range(min(rows, 24))} | {(rows // 2, c) for c in range(0, cols, max(step, cols // 24))}
+    out = h.quantize_nvfp4(x, layout=B.SF_LINEAR)
+    for r, c in sorted(spots):
+        old = x[r, c].clone()
+        x[r, c] = -7.0
+        t, _ = h.quantize_nvfp4(x, layout=B.SF_LINEAR, out=out)
+        assert t.tensor_scale.item() == float(np.float32(7.0) / np.float32(2688.0)), (r, c)
+        x[r, c] = old
