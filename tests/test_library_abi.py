@@ -84,3 +84,22 @@ def test_launch_helpers_keep_no_process_wide_state():
             if re.match(r"\s+static\s+(bool|int|unsigned|size_t|long)\b", line) and "(" not in line.split("=")[0]:
                 bad.append("%s:%d: %s" % (name, i, line.strip()))
     assert not bad, bad
+
+
+@pytest.mark.parametrize("k,axes", [(0, 3), (4, 1), (72, 2), (256, 3)])
+def test_operand_structures_hold_their_members(k, axes):
+    """What is handed to the library, packed as one row, reads back member by member through the ctypes structures."""
+    from paper_2509_00404_b200 import binding as B
+    op = B.Operand(64, 128, k, axes, device="cpu")
+
+    def nvfp4(t, rows):
+        return (t.codes.data_ptr(), t.scales.data_ptr(), t.tensor_scale.data_ptr(), rows, t.k_len, t.layout, 0) if t is not None else (None, None, None, 0, 0, 0, 0)
+
+    def members(s):
+        return tuple(getattr(s, name) for name, _ in s._fields_)
+
+    st = op.struct()
+    assert members(st)[:7] == (k, 0, 64, 128, op.left.data_ptr(), op.sigma.data_ptr(), op.right.data_ptr())
+    assert members(st.left_q) == nvfp4(op.left_q, k) and members(st.right_q) == nvfp4(op.right_q, k)
+    assert members(st.res_by_cols) == nvfp4(op.res_by_cols, 64) and members(st.res_by_rows) == nvfp4(op.res_by_rows, 128)
+    assert members(op.right_q.struct()) == nvfp4(op.right_q, max(k, 1))
