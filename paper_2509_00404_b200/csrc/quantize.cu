@@ -48,7 +48,7 @@ amax_kernel(const void* __restrict__ x, int64_t rows, int64_t cols, int64_t ld, 
     }
   }
   // The launch of the quantizer behind this kernel overlaps its end.  (At the head, the quantizer's CTAs, which need the result for
-  // all they do, would stand on SMs for as long as this kernel runs: up to 81 us, out of the reach of other streams.)
+  // all they do, would stand on SMs for as long as this kernel runs: up to 67 us, out of the reach of other streams.)
   metis_pdl_trigger();
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
