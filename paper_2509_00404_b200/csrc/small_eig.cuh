@@ -289,7 +289,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
   __shared__ double gmax_s;
   __shared__ int flags[EIG_MAX_SWEEPS], flags64[EIG_MAX_SWEEPS];
   __shared__ __align__(16) double2 te[N8 + 8];          // diagonal and squared subdiagonal of the tridiagonal matrix (a block beyond it is read ahead)
-  __shared__ __align__(16) double ys[N8], rs[2][N8], us[N8], ps[N8], qs[N8];
+  __shared__ __align__(16) double ys[N8], rs[2][N8], us[N8], ps[2][N8], qs[N8];
   __shared__ double eo[N8 + 1], beta_s[N8], v1_s[N8];
   __shared__ int pos[N8];
   __shared__ unsigned char grid_count[EIG_THREADS / 2];
@@ -368,7 +368,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
         arrive(Y_READY);
         await(U_READY);
         if (live) {
-          const double2 c = *reinterpret_cast<const double2*>(ps + i0);
+          const double2 c = *reinterpret_cast<const double2*>(ps[j & 1] + i0);
 #pragma unroll
           for (int t = T0; t < NT8; ++t) {
             const double u = us[s8 + 8 * t];
@@ -412,7 +412,10 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
     // A v = u = y - alpha r,  v^T A v = x^T y - 2 alpha y_1 + alpha^2 r_1;  w = beta u - K v,  A -= v w^T + w v^T = p u^T + q v^T.
     // p and u, which do not depend on K, go ahead of q; the next column it updates by itself, so that the others go from the update
     // to the next product without a barrier, and works out that column's reflector meanwhile.  Column j + 1 is not read again
-    // except for its first entry, so x stands for v in the others' last term ----
+    // except for its first entry, so x stands for v in the others' last term.
+    // What orders the vectors (this warp only arrives at U_READY and X_READY, so the others may be a step behind): ys and rs of a step are written
+    // behind its predecessor's X_READY and read behind its Y_READY; us and qs are written behind Y_READY, which the others reach when they have
+    // read those of the step before; p goes out ahead of Y_READY, while they may still read the step before's, so it has two halves, like rs ----
     constexpr int OWN = (N8 + 31) / 32;
     // the sum of a warp, in each lane: sums of four lanes first as columns (each lane gets two of the eight), then as rows
     auto sum32 = [](double v) {
@@ -438,7 +441,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
       for (int k = 0; k < OWN; ++k) {
         const int e = lane + 32 * k;
         v[k] = e == j + 1 ? v1 : x[k];
-        if (e < N8) ps[e] = -beta * v[k];
+        if (e < N8) ps[j & 1][e] = -beta * v[k];
       }
       eo[j] = alpha; beta_s[j] = beta; v1_s[j] = v1;
       await(Y_READY);                                   // the product and row j + 1 are there

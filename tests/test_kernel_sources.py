@@ -110,3 +110,76 @@ def test_shared_arrays_accessed_in_vectors_are_declared_aligned():
                         found.append((os.path.basename(path), type_, name))
     assert wanted >= 10
     assert found == []
+
+
+def _body(text, head):
+    """What stands between the braces behind `head`."""
+    at = text.index("{", text.index(head) + len(head) - 1)
+    depth, end = 0, at
+    while True:
+        depth += {"{": 1, "}": -1}.get(text[end], 0)
+        end += 1
+        if depth == 0:
+            return text[at + 1:end - 1]
+
+
+def _shared_events(body, pairs, step):
+    """The barrier calls and the accesses to shared vectors of one step of a loop, in order: ("arrive" | "await", barrier) and
+    ("read" | "write", vector, half).  pairs: the vectors with two halves; a pointer that is set to one of them stands for it."""
+    def value(expr):
+        return eval(expr, {}, {"j": step})
+
+    alias, events = {}, []
+    name = r"ys|us|ps|qs|rs|V"
+    for m in re.finditer(r"\b(?P<decl>\w+) = (?P<of>rs|ps)\[(?P<dh>[^\]]*)\](?: \+ \w+)?[,;]|\b(?P<sync>arrive|await)\((?P<bar>\w+)\)"
+                         r"|reinterpret_cast<(?P<const>const )?double2\*>\((?P<cast>%s)(?:\[(?P<ch>[^\]]*)\])? \+ [^)]*\)"
+                         r"|\b(?P<vec>%s|rj|out)\[(?P<idx>[^\]]*)\](?:\[[^\]]*\])?(?P<set> = )?" % (name, name), body):
+        if m["decl"]:
+            alias[m["decl"]] = (m["of"], value(m["dh"]))
+        elif m["sync"]:
+            events.append((m["sync"], m["bar"]))
+        elif m["cast"]:
+            events.append(("read" if m["const"] else "write", m["cast"], value(m["ch"]) if m["cast"] in pairs else 0))
+        else:
+            vec, half = alias.get(m["vec"], (m["vec"], None))
+            if half is None:
+                half = value(m["idx"]) if vec in pairs else (value(m["idx"].split(" * P")[0]) if vec == "V" else 0)
+            events.append(("write" if m["set"] else "read", vec, half))
+    return events
+
+
+def test_vectors_of_the_one_cta_reduction_change_hands_behind_a_barrier():
+    """The rows' warps and the scalars' warp of eig_kernel run a step or so apart, joined by one-sided barriers: of two accesses to a
+    shared vector from either side, one of which writes, one has to happen before the other by the barriers alone, whatever the warps' pace."""
+    with open(os.path.join(CSRC, "small_eig.cuh")) as f:
+        text = re.sub(r"//[^\n]*", "", f.read())
+    kernel = text[text.index("eig_kernel(const double"):]
+    pairs = set(re.findall(r"\b(\w+)\[2\]\[N8\]", re.search(r"__shared__[^;]*\bps\[[^;]*;", kernel).group(0)))
+    loops = {"rows": _body(kernel, "for (int j = from; j < to; ++j) {"), "scalars": _body(kernel, "for (int j = 0; j + 2 < n; ++j) {")}
+    # every event's position in its own side's order, and what of the other side has happened before it
+    order, signals, steps = {}, {}, 6
+    for side, body in loops.items():
+        order[side] = [e for step in range(steps) for e in _shared_events(body, pairs, step)]
+        seen = {}
+        for at, e in enumerate(order[side]):
+            if e[0] == "arrive":
+                seen[e[1]] = seen.get(e[1], 0) + 1
+                signals[side, e[1], seen[e[1]]] = at
+    other = {"rows": "scalars", "scalars": "rows"}
+    before = {}
+    for side in order:                                     # before[side][at]: events of the other side up to here have happened
+        seen, known, before[side] = {}, -1, []
+        for e in order[side]:
+            if e[0] == "await":
+                seen[e[1]] = seen.get(e[1], 0) + 1
+                known = max(known, signals[other[side], e[1], seen[e[1]]])
+            before[side].append(known)
+    found, shared = [], set()
+    for a, x in enumerate(order["rows"]):
+        for b, y in enumerate(order["scalars"]):
+            if x[0] in ("read", "write") and x[1:] == y[1:] and "write" in (x[0], y[0]) and y[0] in ("read", "write"):
+                shared.add(x[1])
+                if before["rows"][a] < b and before["scalars"][b] < a:
+                    found.append((x, a, y, b))
+    assert shared == {"ys", "us", "ps", "qs", "rs", "V"}
+    assert found == []
