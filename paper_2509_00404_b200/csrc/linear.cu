@@ -72,8 +72,10 @@ lowrank_finish_kernel(const __grid_constant__ FinishArgs first, const __grid_con
   metis_pdl_trigger();                                      // the large GEMM behind this kernel sets itself up meanwhile
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int kc = ka + kb;
-  const int64_t i0 = ((int64_t)((int)blockIdx.x - (is_first ? 0 : n_first)) * 8 + warp) * R;     // (M and N are multiples of 16)
-  const bool in_m = i0 < M, in_n = i0 < N;
+  const int64_t i0 = ((int64_t)((int)blockIdx.x - (is_first ? 0 : n_first)) * 8 + warp) * R;
+  // An extent is a multiple of 64 where that side has factors (they are quantized in blocks along it); a plain operand may have any number of
+  // rows, so each of the warp's rows is held against its extent.
+  const int rows_m = (int)max(min(M - i0, (int64_t)R), (int64_t)0), rows_n = (int)max(min(N - i0, (int64_t)R), (int64_t)0);
   // ---- loads (ka, kb <= 64: two vectors per lane and operand) ----
   uint32_t a_code[J] = {}, a_sfb[J] = {}, b_code[J] = {}, b_sfb[J] = {};
   float sa_v[J] = {}, sb_v[J] = {}, g1[J][R] = {}, wt[J][R] = {};
@@ -82,21 +84,19 @@ lowrank_finish_kernel(const __grid_constant__ FinishArgs first, const __grid_con
     const int u = lane + 32 * j;
     if (u < ka) {
       sa_v[j] = sa[u];
-      if (in_m) {
+      if (rows_m > 0) {
         const uint8_t* src = foa_codes + (int64_t)u * (M / 2) + i0 / 2;
         a_code[j] = R == 4 ? src[0] | (uint32_t)src[1] << 8 : (R == 2 ? src[0] : src[0] >> (4 * (int)(i0 & 1)));
         a_sfb[j] = foa_sf[metis_sf_offset(u, i0 / 16, M / 16, foa_layout)];
       }
-      if (in_n)
 #pragma unroll
-        for (int r = 0; r < R; ++r) wt[j][r] = rcat[(i0 + r) * kc + kb + u];
+      for (int r = 0; r < R; ++r) if (r < rows_n) wt[j][r] = rcat[(i0 + r) * kc + kb + u];
     }
     if (u < kb) {
       sb_v[j] = sb[u];
-      if (in_m)
 #pragma unroll
-        for (int r = 0; r < R; ++r) g1[j][r] = lcat[(i0 + r) * kc + u];
-      if (in_n) {
+      for (int r = 0; r < R; ++r) if (r < rows_m) g1[j][r] = lcat[(i0 + r) * kc + u];
+      if (rows_n > 0) {
         const uint8_t* src = fob_codes + (int64_t)u * (N / 2) + i0 / 2;
         b_code[j] = R == 4 ? src[0] | (uint32_t)src[1] << 8 : (R == 2 ? src[0] : src[0] >> (4 * (int)(i0 & 1)));
         b_sfb[j] = fob_sf[metis_sf_offset(u, i0 / 16, N / 16, fob_layout)];
@@ -134,7 +134,7 @@ lowrank_finish_kernel(const __grid_constant__ FinishArgs first, const __grid_con
     for (int r = 0; r < R; ++r) fa[warp][lane + 32 * j][r] = raw_a[j][r] * tsa * sa_v[j];
   }
   __syncthreads();
-  if (in_m) {
+  if (rows_m > 0) {
 #pragma unroll 4
     for (int u = 0; u < ka; ++u) {
       float fr[R];
@@ -153,6 +153,7 @@ lowrank_finish_kernel(const __grid_constant__ FinishArgs first, const __grid_con
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     const int64_t i = i0 + r;
+    const bool in_m = r < rows_m, in_n = r < rows_n;
 #pragma unroll
     for (int j = 0; j < J; ++j) {
       const int u = lane + 32 * j;

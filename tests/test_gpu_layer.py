@@ -339,6 +339,41 @@ def test_skinny_products_in_one_launch(ctx, l, n, m, kd, kx, kw):
     assert rel_fro(dw.cpu().numpy(), (ld + rdr).T @ (lx + rxr)) < 2e-5
 
 
+@pytest.mark.parametrize("side", ["x", "w", "dy"])
+@pytest.mark.parametrize("rows,k", [(7107, 32), (7107, 48), (14211, 12), (14211, 64), (16386, 32)])
+def test_plain_operand_of_any_number_of_rows_beside_a_factored_one(ctx, side, rows, k):
+    """metis_quantize_nvfp4 takes any number of rows, so a plain activation, weight or gradient may leave the finishing kernel (two rows a warp
+    from 7105 on, four from 14209 on) a warp that the extent cuts.  Products against float64 ones of the library's own codes, in a workspace of exactly the
+    plan's bytes between guard bytes."""
+    from gpu_util import to_dev_bf16, rel_fro, nv_dequant, Guarded
+    B, h = ctx
+    few, inner = 320, 256
+    t = synth.planted(rows, inner, 8, 100 * (np.sqrt(rows) + 16), 10 * (np.sqrt(rows) + 16), 1.0, 75)[0]
+    plain = B.Operand(rows, inner, 0, B.BLOCKS_ALONG_COLS)
+    plain.res_by_cols, _ = h.quantize_nvfp4(to_dev_bf16(t), axes=B.BLOCKS_ALONG_COLS)
+    shape = (inner, few) if side == "dy" else (few, inner)
+    wide = h.split(to_dev_bf16(synth.planted(*shape, 8, 60.0, 6.0, 0.02, 76)[0]), k, 4, sketch=B.SKETCH_FULL, seed=3)
+    low, by_cols, by_rows = _oracle_from_gpu_operand(wide, k)
+    q = nv_dequant(plain.res_by_cols)
+    kx, up = (2 * k + 63) // 64 * 64, lambda n: (n + 255) // 256 * 256
+    ws = Guarded((4 * 64 * 64 + sum(up(4 * r * k) + up(2 * r * kx) for r in (rows, few)),), torch.uint8)
+    own, h.workspace = h.workspace, lambda n: ws.view
+    try:
+        if side == "dy":
+            got, _ = h.linear_bwd(plain, None, wide, need_dw=False)
+            want = q @ (low + by_rows)
+        elif side == "x":
+            got, want = h.linear_fwd(plain, wide), q @ (low + by_cols).T
+        else:
+            got, want = h.linear_fwd(wide, plain), (low + by_cols) @ q.T
+        torch.cuda.synchronize()
+    finally:
+        h.workspace = own
+    assert h.device_status() == 0
+    assert rel_fro(got.cpu().numpy(), want) < 2e-5
+    ws.check("workspace")
+
+
 def test_bf16_output(ctx):
     from gpu_util import to_dev_bf16, rel_fro
     B, h = ctx
