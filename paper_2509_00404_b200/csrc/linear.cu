@@ -842,7 +842,7 @@ metis_status_t split_gemm_prologue(metis_context* ctx, const Side* const* a, con
   FinishArgs f[2] = {};
   int n_jobs = 0, n_f = 0;
   bool wide = false, fused = false;
-  int64_t mx[2] = {0, 0};
+  int64_t mx[2] = {0, 0}, m_max = 0;
   int kx = 0, kb_max = 0, k_max = 0;
   for (int i = 0; i < n; ++i) {
     if (pl[i]->kc == 0) continue;
@@ -863,6 +863,7 @@ metis_status_t split_gemm_prologue(metis_context* ctx, const Side* const* a, con
     o.sa = sa.sigma; o.sb = sb.sigma; o.pm = p.pm; o.lcat = p.lcat; o.rcat = p.rcat; o.lx = p.lx; o.rx = p.rx;
     o.res_a_ts = sa.res->tensor_scale; o.res_b_ts = sb.res->tensor_scale;
     mx[n_f] = p.M > p.N ? p.M : p.N;
+    if (p.M > m_max) m_max = p.M;
     wide |= ka > 64 || kb > 64; fused |= p.lx != nullptr;
     if (p.kx > kx) kx = p.kx;
     if (kb > kb_max) kb_max = kb;
@@ -874,8 +875,8 @@ metis_status_t split_gemm_prologue(metis_context* ctx, const Side* const* a, con
   const int64_t longest = mx[0] > mx[1] ? mx[0] : mx[1];
   if (wide) {
     METIS_CUDA_TRY(metis_launch_pdl(lowrank_deq_wide_kernel, dim3((unsigned)metis_ceil_div(longest, 32), (unsigned)n_f), dim3(256), 0, s, f[0], f[1])); METIS_COUNT_LAUNCH();
-    if (kb_max) {
-      METIS_CUDA_TRY(metis_launch_pdl(lowrank_gemm_wide_kernel, dim3((unsigned)metis_ceil_div(kb_max, 64), (unsigned)metis_ceil_div(longest, 64), (unsigned)n_f), dim3(256), 0, s,
+    if (kb_max) {                                           // (blocks of the rows of A alone: N may be beyond what a grid has in y)
+      METIS_CUDA_TRY(metis_launch_pdl(lowrank_gemm_wide_kernel, dim3((unsigned)metis_ceil_div(kb_max, 64), (unsigned)metis_ceil_div(m_max, 64), (unsigned)n_f), dim3(256), 0, s,
                                       f[0], f[1])); METIS_COUNT_LAUNCH();
     }
     if (fused) {

@@ -374,6 +374,39 @@ def test_plain_operand_of_any_number_of_rows_beside_a_factored_one(ctx, side, ro
     ws.check("workspace")
 
 
+def test_wide_rank_beside_more_columns_than_a_grid_has_rows_of_blocks(ctx):
+    """A product of few rows (256) and 2^22 columns at a rank above 64: the tiled step on the rows' operand counts its blocks by the rows.  The
+    first and the last 256 columns are, bit for bit, those of the same call on a weight of these rows alone."""
+    B, h = ctx
+    l, n, m, k = 256, 1 << 22, 64, 72
+    g = torch.Generator(device="cuda").manual_seed(77)
+    xo, wo = B.Operand(l, m, 0, B.BLOCKS_ALONG_COLS), B.Operand(n, m, k, B.BLOCKS_ALONG_COLS)
+    for t in (xo.res_by_cols, wo.res_by_cols, wo.left_q, wo.right_q):
+        t.codes.random_(0, 256, generator=g)
+        t.scales.random_(0x28, 0x40, generator=g)
+        t.tensor_scale.fill_(0.01)
+    wo.sigma.uniform_(0.5, 2.0, generator=g)
+
+    def part(rows):
+        p = B.Operand(256, m, k, B.BLOCKS_ALONG_COLS)
+        p.right_q, p.sigma = wo.right_q, wo.sigma
+        p.res_by_cols.codes, p.left_q.codes = wo.res_by_cols.codes[rows], wo.left_q.codes[:, rows.start // 2: rows.stop // 2].contiguous()
+        p.res_by_cols.scales, p.left_q.scales = (t.scales[rows.start * 4 * u: rows.stop * 4 * u] for t, u in ((wo.res_by_cols, 1), (wo.left_q, 2)))
+        p.res_by_cols.tensor_scale, p.left_q.tensor_scale = wo.res_by_cols.tensor_scale, wo.left_q.tensor_scale
+        return h.linear_fwd(xo, p, out_dtype=torch.bfloat16)
+
+    first, last = part(slice(0, 256)), part(slice(n - 256, n))
+    ws = torch.empty(4 * 8192 + (n + l) * (4 * k + 2 * 192) + 2048, dtype=torch.uint8, device="cuda")
+    own, h.workspace = h.workspace, lambda nbytes: ws
+    try:
+        y = h.linear_fwd(xo, wo, out_dtype=torch.bfloat16)
+        torch.cuda.synchronize()
+    finally:
+        h.workspace = own
+    assert h.device_status() == 0 and bool(torch.isfinite(first).all()) and float(first.float().std()) > 0
+    assert torch.equal(y[:, :256], first) and torch.equal(y[:, n - 256:], last)
+
+
 def test_bf16_output(ctx):
     from gpu_util import to_dev_bf16, rel_fro
     B, h = ctx
