@@ -838,9 +838,9 @@ metis_status_t make_plan(const Side& a, const Side& b, void* ws, size_t ws_bytes
 // Everything of one or two products that comes before their large GEMMs: the skinny products (straight into their slots of the concatenated
 // operands; of a layer with fewer than 256 rows the residual product too) in one launch and the finishing kernels.
 metis_status_t split_gemm_prologue(metis_context* ctx, const Side* const* a, const Side* const* b, const Plan* const* pl, int n, cudaStream_t s) {
-  metis_gemm_job jobs[8];
+  metis_gemm_job jobs[8], large[4];
   FinishArgs f[2] = {};
-  int n_jobs = 0, n_f = 0;
+  int n_jobs = 0, n_large = 0, n_f = 0;
   bool wide = false, fused = false;
   int64_t mx[2] = {0, 0}, m_max = 0;
   int kx = 0, kb_max = 0, k_max = 0;
@@ -853,8 +853,16 @@ metis_status_t split_gemm_prologue(metis_context* ctx, const Side* const* a, con
       if (metis_ceil_div(p.M, 128) * metis_ceil_div(p.N, 64) <= ctx->sm_count) jobs[n_jobs++] = {sa.res, sb.res, p.y0, p.N, false};
       else METIS_TRY(metis_launch_gemm_tc(ctx, sa.res, sb.res, p.y0, METIS_FP32, p.N, s));
     }
-    if (kb) jobs[n_jobs++] = {sa.res, sb.fc, p.lcat, kc, true};
-    if (ka) jobs[n_jobs++] = {sb.res, sa.fc, p.rcat + kb, kc, true};
+    // Rank 256, long and deep: 128 x 128 tiles read 140 bytes a cycle and SM, beyond what the L2 delivers, so such products keep the 256 x 256 tiles of the
+    // two-CTA kernel, beside the group on the side stream or behind it.  Weight gradient of 16384 x 8192 x 8192: all in the group 664 us, so 641;
+    // input and weight gradient 1492 and 1427; 16384 x 4096 x 14336 1318 and 1271.  With 4096 rows (half as many tiles as SMs) the group is the faster: 222
+    // against 233 us at 16384 x 4096 x 4096; at K = 4096 they are equal.
+    auto skinny = [&](const metis_nvfp4_t* r, const metis_nvfp4_t* fc, float* d) {
+      const bool square = fc->rows >= 256 && r->rows >= 8192 && r->rows * r->k_len >= (int64_t)1 << 26;
+      (square ? large[n_large++] : jobs[n_jobs++]) = {r, fc, d, kc, true};
+    };
+    if (kb) skinny(sa.res, sb.fc, p.lcat);
+    if (ka) skinny(sb.res, sa.fc, p.rcat + kb);
     if (ka && kb) jobs[n_jobs++] = {sa.fc, sb.fc, p.pm, kb, true};
     FinishArgs& o = f[n_f];
     o.M = p.M; o.N = p.N; o.ka = ka; o.kb = kb; o.kx = p.kx;
@@ -871,7 +879,11 @@ metis_status_t split_gemm_prologue(metis_context* ctx, const Side* const* a, con
     ++n_f;
   }
   if (n_f == 0) return METIS_OK;
+  if (n_large) METIS_TRY(metis_fork(ctx, s, 1));           // (the group first: its CTAs are few and soon done)
   METIS_TRY(metis_launch_gemm_group(ctx, jobs, n_jobs, s));
+  for (int i = 0; i < n_large; ++i)
+    METIS_TRY(metis_launch_gemm_tc(ctx, large[i].a, large[i].b, large[i].d, METIS_FP32, large[i].ldd, i & 1 ? s : ctx->side[0]));
+  if (n_large) METIS_TRY(metis_join(ctx, s, 0));
   const int64_t longest = mx[0] > mx[1] ? mx[0] : mx[1];
   if (wide) {
     METIS_CUDA_TRY(metis_launch_pdl(lowrank_deq_wide_kernel, dim3((unsigned)metis_ceil_div(longest, 32), (unsigned)n_f), dim3(256), 0, s, f[0], f[1])); METIS_COUNT_LAUNCH();

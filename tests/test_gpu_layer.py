@@ -407,6 +407,39 @@ def test_wide_rank_beside_more_columns_than_a_grid_has_rows_of_blocks(ctx):
     assert torch.equal(y[:, :256], first) and torch.equal(y[:, n - 256:], last)
 
 
+@pytest.mark.parametrize("kd,kx", [(256, 256), (0, 256), (256, 8)])
+def test_rank_256_products_of_long_and_deep_operands(ctx, kd, kx):
+    """From 8192 rows and 2^26 residual elements on, the products with 256 factor vectors run beside the grouped ones, on two streams: weight
+    gradient of operands with random codes against their float64 product (exact codes, FP32 sums)."""
+    B, h = ctx
+    n = 8192
+    g = torch.Generator(device="cuda").manual_seed(79)
+    e2m1 = torch.tensor([0, .5, 1, 1.5, 2, 3, 4, 6, 0, -.5, -1, -1.5, -2, -3, -4, -6], dtype=torch.float64, device="cuda")
+
+    def value(t):
+        c = torch.stack((t.codes & 15, t.codes >> 4), dim=2).reshape(t.rows, -1).int()
+        s = t.linear_scales().cuda().view(torch.float8_e4m3fn).double()
+        return (e2m1[c].reshape(t.rows, -1, 16) * s[:, :, None]).reshape(t.rows, -1) * t.tensor_scale.double()
+
+    def operand(k):
+        op = B.Operand(n, n, k, B.BLOCKS_ALONG_ROWS)
+        for t, scale in ((op.res_by_rows, 0.01), (op.left_q, 0.003), (op.right_q, 0.003)):
+            t.codes.random_(0, 256, generator=g)
+            t.scales.random_(0x28, 0x40, generator=g)
+            t.tensor_scale.fill_(scale)
+        op.sigma.uniform_(0.5, 2.0, generator=g)
+        v = value(op.res_by_rows).T
+        return op, v + (value(op.left_q).T * op.sigma.double()) @ value(op.right_q) if k else v
+
+    do, d = operand(kd)
+    xo, x = operand(kx)
+    _, dw = h.linear_bwd(do, xo, None, need_dx=False)
+    torch.cuda.synchronize()
+    assert h.device_status() == 0
+    want = d.T @ x
+    assert float((dw.double() - want).norm() / want.norm()) < 2e-5
+
+
 def test_bf16_output(ctx):
     from gpu_util import to_dev_bf16, rel_fro
     B, h = ctx
