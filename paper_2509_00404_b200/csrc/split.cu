@@ -811,22 +811,27 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
 // products less the sum, is an accumulator of its own with the smaller terms.
 // With M whole in the CTA its Gram matrix follows from shared memory (see gram_add).  As FP32 multiply-adds over ten slabs of rows, their sum, a
 // Gram kernel and its reduction this was four launches, 21 us at 160 x 4096 with q = 40; now 7.
-constexpr int PG_COLS = 64, PG_K = 64, PG_STAGES = 4, PG_XP = PG_COLS + 8, PG_HP = PG_K + 8;
-__host__ __device__ constexpr size_t pg_smem(int mt) {
-  const size_t ring = (size_t)PG_STAGES * (PG_K * PG_XP * 2 + 3 * mt * 16 * PG_HP * 2), post = sizeof(float) * mt * 16 * (PG_COLS + 4) + SG_SMEM;
+// PARTS (a long sample, see launch_project_gram): a CTA takes one of gridDim.y parts of the rows for its 64 columns and leaves mp[part][col][16 MT];
+// sum_gram_kernel does the rest.  These are many CTAs, so two of them share an SM.
+constexpr int PG_COLS = 64, PG_K = 64, PG_XP = PG_COLS + 8, PG_HP = PG_K + 8;
+__host__ __device__ constexpr int pg_stages(bool in_parts) { return in_parts ? 3 : 4; }
+__host__ __device__ constexpr size_t pg_smem(int mt, bool in_parts) {
+  const size_t ring = (size_t)pg_stages(in_parts) * (PG_K * PG_XP * 2 + 3 * mt * 16 * PG_HP * 2), post = sizeof(float) * mt * 16 * (PG_COLS + 4) + (in_parts ? 0 : SG_SMEM);
   return ring > post ? ring : post;
 }
-template <int MT>                                       // sketch columns / 16, rounded up
-__global__ void __launch_bounds__(256)
+template <int MT, bool PARTS>                           // sketch columns / 16, rounded up
+__global__ void __launch_bounds__(256, PARTS && MT <= 4 ? 2 : 1)
 project_gram_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, RowSample rs, int n_s, int q, const __nv_bfloat16* __restrict__ hsp, int ldh,
-                    float* __restrict__ m, double* __restrict__ gram_part) {
+                    float* __restrict__ m, double* __restrict__ gram_part, float* __restrict__ mp) {
   extern __shared__ __align__(16) unsigned char psm[];
+  constexpr int PG_STAGES = pg_stages(PARTS);
   constexpr int XS_BYTES = PG_K * PG_XP * 2, HS_BYTES = 3 * MT * 16 * PG_HP * 2, STAGE = XS_BYTES + HS_BYTES, MP = PG_COLS + 4;
   float* Ms = reinterpret_cast<float*>(psm);            // [MT * 16][MP], over the ring, which has been read by then
   double *tile = reinterpret_cast<double*>(psm + sizeof(float) * MT * 16 * MP), *gp = tile + GR_TILE * LP;
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(psm);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3, wn = warp & 3, kh = warp >> 2, n8 = (q + 7) & ~7;
-  const int n_chunks = (n_s + PG_K - 1) / PG_K;
+  const int all_chunks = (n_s + PG_K - 1) / PG_K, chunk0 = PARTS ? all_chunks * (int)blockIdx.y / (int)gridDim.y : 0;
+  const int n_chunks = PARTS ? all_chunks * ((int)blockIdx.y + 1) / (int)gridDim.y - chunk0 : all_chunks;       // of this CTA's part of the rows
   const int64_t tiles = (cols + PG_COLS - 1) / PG_COLS;
   __shared__ int ids[256];                              // the first rows of the sample (beyond them each copy works its row out)
   ids[tid] = tid < n_s ? sample_row(rs, tid) : 0;
@@ -834,7 +839,7 @@ project_gram_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, RowSample
     const uint32_t xs = sbase + (uint32_t)(c % PG_STAGES) * STAGE;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int rr = (tid >> 3) + 32 * u, c8 = (tid & 7) * 8, r = c * PG_K + rr;
+      const int rr = (tid >> 3) + 32 * u, c8 = (tid & 7) * 8, r = (chunk0 + c) * PG_K + rr;
       const bool ok = r < n_s && col0 + c8 + 8 <= cols;
       cp_async16(xs + (uint32_t)(rr * PG_XP + c8) * 2u, ok ? x + (int64_t)(r < 256 ? ids[r] : sample_row(rs, r)) * cols + col0 + c8 : x, ok);
     }
@@ -843,7 +848,7 @@ project_gram_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, RowSample
     const uint32_t hs = sbase + (uint32_t)(c % PG_STAGES) * STAGE + XS_BYTES;
     for (int i = tid; i < 3 * MT * 16 * (PG_K / 8); i += 256) {
       const int row = i >> 3, k8 = (i & 7) * 8;          // row = term * MT * 16 + j
-      cp_async16(hs + (uint32_t)(row * PG_HP + k8) * 2u, hsp + (int64_t)row * ldh + c * PG_K + k8, true);
+      cp_async16(hs + (uint32_t)(row * PG_HP + k8) * 2u, hsp + (int64_t)row * ldh + (chunk0 + c) * PG_K + k8, true);
     }
   };
   GramTiles gt;
@@ -928,6 +933,15 @@ project_gram_kernel(const __nv_bfloat16* __restrict__ x, int64_t cols, RowSample
               o = half ? o + total[a][n][e] : total[a][n][e];
             }
       __syncthreads();
+    }
+    if constexpr (PARTS) {                                 // (a tile per CTA)
+      for (int o = tid; o < PG_COLS * 4 * MT; o += 256) {
+        const int c = o / (4 * MT), j = 4 * (o - c * 4 * MT);
+        if (col0 + c < cols)
+          *reinterpret_cast<float4*>(mp + ((int64_t)blockIdx.y * cols + col0 + c) * (16 * MT) + j) =
+              make_float4(Ms[j * MP + c], Ms[(j + 1) * MP + c], Ms[(j + 2) * MP + c], Ms[(j + 3) * MP + c]);
+      }
+      return;
     }
     for (int o = tid; o < q * (PG_COLS / 4); o += 256) {
       const int j = o >> 4, c4 = (o & 15) * 4;
@@ -1144,9 +1158,11 @@ int sketch_tc_cols(int q) { return q <= 48 ? 48 : 96; }
 // Column chunks of a sampled sketch: 64 columns each (a 160-row sketch has one row block, so narrow chunks are what gives it CTAs), wider ones or more than
 // one to a CTA beyond 128 CTAs, so that the clusters leave at most GR_PARTS partials.
 struct SketchGrid { int ccols, chunks, ctas, csize, parts; };
-SketchGrid sketch_grid(int64_t cols) {
+SketchGrid sketch_grid(int64_t cols, int64_t n_s) {
   SketchGrid s{};
   s.ccols = cols <= 64 * 128 ? 64 : (cols <= 128 * 128 ? 128 : SKM_COLS);
+  // a long sample has its CTAs from its rows: fewer sums to exchange
+  while (n_s > GC_MAX_ROWS && s.ccols < SKM_COLS && metis_ceil_div(n_s, SKM_ROWS) * metis_ceil_div(cols, 2 * s.ccols) >= 296) s.ccols *= 2;
   s.chunks = (int)metis_ceil_div(cols, s.ccols);
   gram_grid(s.chunks, &s.ctas, &s.csize);
   s.parts = s.ctas / s.csize;
@@ -1214,18 +1230,35 @@ metis_status_t launch_sum_gram(cudaStream_t s, const float* part, int slices, in
   METIS_CUDA_TRY(metis_launch_pdl_cluster(sum_gram_kernel<TRANS>, dim3((unsigned)ctas), dim3(256), SG_SMEM, s, 0, csize, part, slices, n_pos, width, q, out, gram, skip)); METIS_COUNT_LAUNCH();
   return METIS_OK;
 }
-metis_status_t launch_project_gram(cudaStream_t s, const __nv_bfloat16* x, int64_t cols, const RowSample& rs, int n_s, int q, const __nv_bfloat16* hsp, int ldh, float* m, double* gram, int* parts) {
-  int ctas, csize;
-  gram_grid(metis_ceil_div(cols, PG_COLS), &ctas, &csize);
+// M = H^T x of sampled rows and its Gram partials.  A tile's CTA walks all rows; where that is long, up to eight CTAs take a part of the rows each and
+// sum_gram_kernel adds the parts (mp).  The rule counts rounds of CTAs times chunks of 64 rows behind one another (1.4 us, a third more with two CTAs on an
+// SM), six more for a CTA's start and end and twelve for the launch behind; samples of up to 1024 rows have no use for it.  Whole split, all rows in one CTA -> in
+// parts (and as slabs of 512 rows with FP32 partials, before both): p = 8, 8192 of 16384 x 1024, k = 32 355 -> 201 us (230); 4096 of 16384 x 4096 341 -> 269
+// (282); every row of 16384 x 4096 in a sample, k = 64 1247 -> 816 (881); 1312 of 131072 x 256, k = 8 171 -> 153 (270); 8192 of 16384 x 14336 1030 -> 826 (796).
+metis_status_t launch_project_gram(metis_context* ctx, cudaStream_t s, const __nv_bfloat16* x, int64_t cols, const RowSample& rs, int n_s, int q, const __nv_bfloat16* hsp, int ldh, float* m, double* gram,
+                                   float* mp, int* parts) {
+  const int64_t tiles = metis_ceil_div(cols, PG_COLS), chunks = metis_ceil_div(n_s, PG_K);
+  int ctas, csize, slices = 1;
+  gram_grid(tiles, &ctas, &csize);
+  const bool two = q <= 64;                             // CTAs on an SM
+  int64_t best = (chunks + 6) * metis_ceil_div(tiles, ctas < 120 ? ctas : 120) * 3;                  // (fifteen clusters of eight are resident)
+  for (int n = 2; n <= 8 && chunks > 16; ++n) {
+    const int64_t load = tiles * n, sms = ctx->sm_count, rounds = load <= sms || !two ? 3 * metis_ceil_div(load, sms) : 4 * metis_ceil_div(load, 2 * sms);
+    const int64_t cost = (metis_ceil_div(chunks, n) + 6) * rounds + 36;
+    if (cost < best) { best = cost; slices = n; }
+  }
   *parts = ctas / csize;
-#define METIS_PG(MT) case MT: METIS_CUDA_TRY(metis_launch_pdl_cluster(project_gram_kernel<MT>, dim3((unsigned)ctas), dim3(256), pg_smem(MT), s, 0, csize, x, cols, rs, n_s, q, hsp, ldh, m, gram)); break
+#define METIS_PG(MT) case MT: \
+    if (slices > 1) METIS_CUDA_TRY(metis_launch_pdl(project_gram_kernel<MT, true>, dim3((unsigned)tiles, (unsigned)slices), dim3(256), pg_smem(MT, true), s, x, cols, rs, n_s, q, hsp, ldh, m, gram, mp)); \
+    else METIS_CUDA_TRY(metis_launch_pdl_cluster(project_gram_kernel<MT, false>, dim3((unsigned)ctas), dim3(256), pg_smem(MT, false), s, 0, csize, x, cols, rs, n_s, q, hsp, ldh, m, gram, (float*)nullptr)); \
+    break
   switch ((q + 15) / 16) {
     METIS_PG(1); METIS_PG(2); METIS_PG(3); METIS_PG(4); METIS_PG(5);
     default: return METIS_ERR_SHAPE;
   }
 #undef METIS_PG
   METIS_COUNT_LAUNCH();
-  return METIS_OK;
+  return slices > 1 ? launch_sum_gram<true>(s, mp, slices, cols, (q + 15) / 16 * 16, q, m, gram, nullptr, parts) : METIS_OK;
 }
 metis_status_t launch_sketch(cudaStream_t s, const SketchGrid& sk, const __nv_bfloat16* x, int64_t cols, const RowSample& rs, int n_s, int q, uint64_t seed, const __nv_bfloat16* lut, float* zp,
                              float* amax, unsigned long long* keys) {
@@ -1653,7 +1686,8 @@ metis_status_t metis_split_set_attrs() {
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::chol_mid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::cm_smem(metis_wide::CM_MAX)));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::chol_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::CW_SMEM));
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::trsm_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::TW_SMEM));
-#define METIS_PP_ATTR(MT) METIS_CUDA_TRY(cudaFuncSetAttribute(project_gram_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pg_smem(MT)))
+#define METIS_PP_ATTR(MT) METIS_CUDA_TRY(cudaFuncSetAttribute(project_gram_kernel<MT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pg_smem(MT, false))); \
+  METIS_CUDA_TRY(cudaFuncSetAttribute(project_gram_kernel<MT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pg_smem(MT, true)))
   METIS_PP_ATTR(1); METIS_PP_ATTR(2); METIS_PP_ATTR(3); METIS_PP_ATTR(4); METIS_PP_ATTR(5);
 #undef METIS_PP_ATTR
   return METIS_OK;
@@ -1818,7 +1852,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     METIS_TRY(metis_launch_coeff_tc(ctx, x, rows, cols, omt, nb_sk / 3, zp, amax, 1, s));
     slices_z = metis_coeff_slices(rows, cols, nullptr); width_z = nb_sk;
   } else {
-    const SketchGrid sk = sketch_grid(cols);
+    const SketchGrid sk = sketch_grid(cols, n_s);
     METIS_TRY(launch_sketch(s, sk, x, cols, rs, (int)n_s, q, seed, ctx->quantile_lut, zp, amax, keys));
     if (src_amax != nullptr) METIS_CUDA_TRY(cudaMemcpyAsync(amax, src_amax, sizeof(float), cudaMemcpyDeviceToDevice, s));
     slices_z = sk.parts;
@@ -1841,7 +1875,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     METIS_TRY(metis_launch_project_tc(ctx, x, rows, cols, hsp, jp, ldh, mp, s));
     METIS_TRY(launch_sum_gram<true>(s, mp, metis_project_slices(rows, cols), cols, jp, q, m, gram, nullptr, &parts));
   } else {
-    METIS_TRY(launch_project_gram(s, x, cols, rs, (int)n_s, q, hsp, ldh, m, gram, &parts));
+    METIS_TRY(launch_project_gram(ctx, s, x, cols, rs, (int)n_s, q, hsp, ldh, m, gram, mp, &parts));
   }
   METIS_TRY(launch_eig(s, gram, parts, q, q, evals, evecs));
   // (5) right basis and its splits; coefficients of every row in the basis, (6) fused residual + quantizer

@@ -117,6 +117,8 @@ def test_wide_ranks_on_the_cluster_solver(ctx, case, mode_name):
     (2048, 512, 20, 5, "sampled", 1040),      # a long sample: partials of a width that is no multiple of four
     (4160, 320, 16, 8, "sampled", 0),         # more Gram partials of the coefficients than the eigen-solver adds
     (1088, 576, 64, 8, "sampled", 304),       # 38 groups of rows for eight CTAs
+    (1152, 192, 4, 4, "sampled", 1152), (2176, 320, 64, 8, "sampled", 2064),         # projection in parts of the rows, the last chunk cut
+    (2304, 4288, 32, 8, "sampled", 2064),     # the same on more columns than two CTAs an SM take at once, 128-column chunks of a long sketch
 ])
 def test_chain_kernels_at_their_edges(ctx, rows, cols, k, p, mode_name, n_sample):
     B, h = ctx
