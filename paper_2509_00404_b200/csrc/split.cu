@@ -144,8 +144,10 @@ inline void gram_grid(int64_t tiles, int* ctas, int* csize) {
 // Sums column slices of a tensor-core pass in a fixed order, v[position][i] = sum over s of part[s][position][i] (rows `width` wide, i < q), stores them
 // row by row (TRANS = 0: out[position][i]) or vector by vector (TRANS = 1: out[i][position]) and forms the Gram matrix of the q vectors.
 // out may be null (the slices are then the vectors themselves).
+// SOME: of rows that are wider than the q vectors take, only these are read.  For CTAs of several tiles, which are bound by their bytes (every row of 2^20 x 64,
+// q = 8 of 48 columns: split 1633 -> 1271 us; 16384 x 4096 at q = 40 of 48: step of the k / v projection 677 -> 669); a CTA of one tile takes half a us longer so.
 constexpr size_t SG_SMEM = sizeof(double) * (GR_TILE * LP + 64 * 45);
-template <bool TRANS>
+template <bool TRANS, bool SOME>
 __global__ void __launch_bounds__(256)
 sum_gram_kernel(const float* __restrict__ part, int slices, int64_t n_pos, int width, int q, float* __restrict__ out, double* __restrict__ gram_part,
                 const int* __restrict__ skip) {
@@ -161,23 +163,24 @@ sum_gram_kernel(const float* __restrict__ part, int slices, int64_t n_pos, int w
     const int64_t p0 = ti * GR_TILE;
     if ((width & 3) == 0) {
       // the tile is one run of 64 * width floats per slice: groups of four, two groups' slices in flight (columns from q on are zeros)
-      const int w4 = width >> 2, n_o = (int)min((int64_t)GR_TILE, n_pos - p0) * w4;
+      const int w4 = width >> 2, n4 = SOME ? n8 >> 2 : w4, n_o = (int)min((int64_t)GR_TILE, n_pos - p0) * n4;
       const float4* src = reinterpret_cast<const float4*>(part) + p0 * w4;
       const int64_t stride = n_pos * w4;
-      for (int o0 = tid; o0 < GR_TILE * w4; o0 += 512) {
+      auto place = [&](int o) { return SOME ? o + o / n4 * (w4 - n4) : o; };
+      for (int o0 = tid; o0 < GR_TILE * n4; o0 += 512) {
         float4 v[2][8];
 #pragma unroll
         for (int u = 0; u < 2; ++u)
 #pragma unroll
-          for (int sl = 0; sl < 8; ++sl) v[u][sl] = sl < slices && o0 + 256 * u < n_o ? src[sl * stride + o0 + 256 * u] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          for (int sl = 0; sl < 8; ++sl) v[u][sl] = sl < slices && o0 + 256 * u < n_o ? src[sl * stride + place(o0 + 256 * u)] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
-          const int o = o0 + 256 * u, p = o / w4, j = 4 * (o - p * w4);
-          if (o >= GR_TILE * w4) break;
+          const int o = o0 + 256 * u, p = o / n4, j = 4 * (o - p * n4);
+          if (o >= GR_TILE * n4) break;
           float4 x = v[u][0];
 #pragma unroll
           for (int sl = 1; sl < 8; ++sl) { x.x += v[u][sl].x; x.y += v[u][sl].y; x.z += v[u][sl].z; x.w += v[u][sl].w; }
-          for (int sl = 8; sl < slices && o < n_o; ++sl) { const float4 y = src[sl * stride + o]; x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w; }
+          for (int sl = 8; sl < slices && o < n_o; ++sl) { const float4 y = src[sl * stride + place(o)]; x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w; }
           if (j < n8) {
             *reinterpret_cast<double2*>(tile + p * LP + j) = make_double2((double)x.x, (double)x.y);
             *reinterpret_cast<double2*>(tile + p * LP + j + 2) = make_double2((double)x.z, (double)x.w);
@@ -1227,7 +1230,9 @@ metis_status_t launch_sum_gram(cudaStream_t s, const float* part, int slices, in
   int ctas, csize;
   gram_grid(metis_ceil_div(n_pos, GR_TILE), &ctas, &csize);
   *parts = ctas / csize;
-  METIS_CUDA_TRY(metis_launch_pdl_cluster(sum_gram_kernel<TRANS>, dim3((unsigned)ctas), dim3(256), SG_SMEM, s, 0, csize, part, slices, n_pos, width, q, out, gram, skip)); METIS_COUNT_LAUNCH();
+  const bool some = metis_ceil_div(n_pos, GR_TILE) > ctas && width % 4 == 0 && (q + 7) / 8 * 8 < width;
+  METIS_CUDA_TRY(metis_launch_pdl_cluster(some ? sum_gram_kernel<TRANS, true> : sum_gram_kernel<TRANS, false>, dim3((unsigned)ctas), dim3(256), SG_SMEM, s, 0, csize, part, slices, n_pos,
+                                          width, q, out, gram, skip)); METIS_COUNT_LAUNCH();
   return METIS_OK;
 }
 // M = H^T x of sampled rows and its Gram partials.  A tile's CTA walks all rows; where that is long, up to eight CTAs take a part of the rows each and
@@ -1672,8 +1677,9 @@ metis_status_t metis_split_set_attrs() {
   METIS_CUDA_TRY(cudaFuncSetAttribute(sketch_mma_kernel<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)skm_smem(KT, SKM_COLS)))
   METIS_GC_ATTR(1); METIS_GC_ATTR(2); METIS_GC_ATTR(3); METIS_GC_ATTR(4); METIS_GC_ATTR(5); METIS_GC_ATTR(6); METIS_GC_ATTR(7); METIS_GC_ATTR(8); METIS_GC_ATTR(9);
 #undef METIS_GC_ATTR
-  METIS_CUDA_TRY(cudaFuncSetAttribute(sum_gram_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SG_SMEM));
-  METIS_CUDA_TRY(cudaFuncSetAttribute(sum_gram_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SG_SMEM));
+#define METIS_SG_ATTR(T, S) METIS_CUDA_TRY(cudaFuncSetAttribute(sum_gram_kernel<T, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SG_SMEM))
+  METIS_SG_ATTR(false, false); METIS_SG_ATTR(false, true); METIS_SG_ATTR(true, false); METIS_SG_ATTR(true, true);
+#undef METIS_SG_ATTR
   METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::jacobi_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::JC_SMEM));
 #define METIS_WT_ATTR(R, C, T) METIS_CUDA_TRY(cudaFuncSetAttribute(metis_wide::tridiag_chol_kernel<R, C, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)metis_wide::cm_smem(metis_wide::WT_MAX)))
   METIS_WT_ATTR(6, 3, false); METIS_WT_ATTR(9, 3, false); METIS_WT_ATTR(9, 4, false); METIS_WT_ATTR(10, 4, true);

@@ -119,6 +119,7 @@ def test_wide_ranks_on_the_cluster_solver(ctx, case, mode_name):
     (1088, 576, 64, 8, "sampled", 304),       # 38 groups of rows for eight CTAs
     (1152, 192, 4, 4, "sampled", 1152), (2176, 320, 64, 8, "sampled", 2064),         # projection in parts of the rows, the last chunk cut
     (2304, 4288, 32, 8, "sampled", 2064),     # the same on more columns than two CTAs an SM take at once, 128-column chunks of a long sketch
+    (8320, 64, 8, 4, "full", 0), (1088, 8256, 4, 1, "full", 0),           # more tiles than CTAs of the slices' sum: of wider rows only the sketch's columns
 ])
 def test_chain_kernels_at_their_edges(ctx, rows, cols, k, p, mode_name, n_sample):
     B, h = ctx
