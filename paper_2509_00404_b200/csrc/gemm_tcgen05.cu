@@ -1007,7 +1007,9 @@ metis_status_t metis_launch_gemm_tc_fused(metis_context* ctx, const metis_nvfp4_
 
 // FP32 products of one launch (see gemm_nvfp4_group_kernel).  Split of the contractions: the problem whose CTAs have the most K blocks is halved again while
 // that fills SMs that have nothing, or while those CTAs alone would run a quarter longer than an
-// even share of all the work.
+// even share of all the work.  With tiles of 128 columns, one CTA to an SM, of the splits on this way the one with the fewest K blocks behind one another: a second
+// round of CTAs costs more than the halves save (forward 4096 x 2048 -> 7168, k = 128 99.0 -> 89.4 us, both gradients 141.9 -> 131.4; 8192 x
+// 1024 -> 4096, k = 100 92 -> 84 and 113 -> 105).
 metis_status_t metis_launch_gemm_group(metis_context* ctx, const metis_gemm_job* jobs, int n, cudaStream_t s) {
   if (n <= 0) return METIS_OK;
   if (n > GROUP_MAX) return METIS_ERR_INVALID_ARG;
@@ -1029,16 +1031,42 @@ metis_status_t metis_launch_gemm_group(metis_context* ctx, const metis_gemm_job*
     split[i] = 0; order[i] = i;
     total += tiles[i] * kb[i]; ctas += tiles[i];
   }
+  // 128 columns leave room for one CTA on an SM: K blocks behind one another, a second round of CTAs with ten more for its set-up and end
+  auto behind_one_another = [&]() -> int64_t {
+    int64_t longest = 0, last = 0, next = 0, left = ctx->sm_count;
+    bool taken[GROUP_MAX] = {};
+    for (int r = 0; r < n; ++r) {                          // by falling shares
+      int i = -1;
+      for (int j = 0; j < n; ++j) if (!taken[j] && (i < 0 || kb[j] >> split[j] > kb[i] >> split[i])) i = j;
+      taken[i] = true;
+      const int64_t share = kb[i] >> split[i], count = tiles[i] << split[i];
+      if (r == 0) longest = share;
+      if (left > 0) last = share;
+      if (left >= 0 && count > left) next = share;
+      left = count > left ? -1 : left - count;
+      if (left < 0) break;
+    }
+    if (ctas <= ctx->sm_count) return longest;
+    const int64_t even = total / ctx->sm_count + longest / 2;
+    return (last + next > even ? last + next : even) + 10 * ((ctas - 1) / ctx->sm_count);
+  };
+  int64_t best = block_n == 128 ? behind_one_another() : 0;
+  int best_split[GROUP_MAX] = {};
   for (;;) {
     int top = -1;
     for (int i = 0; i < n; ++i)
       if (split[i] < 3 && kb[i] >> split[i] >= 4 && (top < 0 || kb[i] >> split[i] > kb[top] >> split[top])) top = i;
     if (top < 0) break;
     const int64_t more = tiles[top] << split[top], share = kb[top] >> split[top];
-    // (GPCs hold clusters of four and eight on 128 SMs)
+    // (one CTA to an SM, clusters of four find room on 132 SMs, of eight on 120)
     if (ctas + more > (split[top] >= 1 ? 128 : ctx->sm_count) && 4 * share * ctx->sm_count <= 5 * total) break;
     ctas += more; ++split[top];
+    if (block_n == 128) {
+      const int64_t now = behind_one_another() + 1;        // (a divided contraction is put together again)
+      if (now < best) { best = now; for (int i = 0; i < n; ++i) best_split[i] = split[i]; }
+    }
   }
+  if (block_n == 128) for (int i = 0; i < n; ++i) split[i] = best_split[i];
   int log_c = 0;
   for (int i = 0; i < n; ++i) if (split[i] > log_c) log_c = split[i];
   for (int i = 1; i < n; ++i)                              // the longest shares first
