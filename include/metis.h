@@ -151,7 +151,7 @@ int32_t metis_debug_build(void);
 metis_status_t metis_debug_index_check(metis_handle_t h, int64_t offset, int64_t nbytes, int64_t extent, metis_stream_t stream);
 
 /* Test hook: rcp[i] and rsqrt[i] (device, n values each) are the FP64 reciprocal and reciprocal square root of x[i] as the dense kernels of
- * a decomposition form them (Newton-Raphson; for normal values whose results are normal). */
+ * a decomposition form them (a step of third order; for normal values whose results are normal). */
 metis_status_t metis_debug_reciprocals(metis_handle_t h, const double* x, int64_t n, double* rcp, double* rsqrt, metis_stream_t stream);
 
 /* Test hook: eigenvalues (n, descending) and eigenvectors (columns of the n x n evecs) of a symmetric positive semi-definite matrix of order

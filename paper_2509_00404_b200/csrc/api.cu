@@ -141,8 +141,8 @@ namespace {
 __global__ void reciprocals_kernel(const double* __restrict__ x, int64_t n, double* __restrict__ rcp, double* __restrict__ rsq) {
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= n) return;
-  rcp[i] = metis_small::rcp_newton(x[i]);
-  rsq[i] = metis_small::rsqrt_newton(x[i]);
+  rcp[i] = metis_small::rcp_cubic(x[i]);
+  rsq[i] = metis_small::rsqrt_cubic(x[i]);
 }
 }  // namespace
 

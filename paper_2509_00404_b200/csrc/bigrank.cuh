@@ -227,13 +227,13 @@ chol_wide_kernel(const double* __restrict__ g, int n, double tol_rel, double* l_
 #pragma unroll
       for (int c = 0; c < CW_NB; ++c) {
         const double d = __shfl_sync(0xFFFFFFFFu, v[c], c);
-        const double l = v[c] * (d > tol ? metis_small::rcp_newton(d) : 0.0);
+        const double l = v[c] * (d > tol ? metis_small::rcp_cubic(d) : 0.0);
         if (lane == c) pivot = d;
 #pragma unroll
         for (int c2 = c + 1; c2 < CW_NB; ++c2) v[c2] = fma(-l, __shfl_sync(0xFFFFFFFFu, v[c], c2), v[c2]);
       }
       const bool ok = pivot > tol;
-      const double rinv = ok ? metis_small::rsqrt_newton(pivot) : 0.0;               // lane c: 1 / L[c][c]
+      const double rinv = ok ? metis_small::rsqrt_cubic(pivot) : 0.0;               // lane c: 1 / L[c][c]
       if (ok) dmin = fmin(dmin, pivot);
 #pragma unroll
       for (int c = 0; c < CW_NB; ++c) {
@@ -714,7 +714,7 @@ jacobi_fp32_kernel(const double* __restrict__ l, int n, double* __restrict__ x) 
     for (int t = 0; t < R; ++t) { const float2 v = y[row_of(t)]; sx = fma((double)v.x, (double)v.x, sx); sy = fma((double)v.y, (double)v.y, sy); }
 #pragma unroll
     for (int o = LANES / 2; o > 0; o >>= 1) { sx += __shfl_xor_sync(0xFFFFFFFFu, sx, o); sy += __shfl_xor_sync(0xFFFFFFFFu, sy, o); }
-    const double rx = sx > 0.0 ? metis_small::rsqrt_newton(sx) : 0.0, ry = sy > 0.0 ? metis_small::rsqrt_newton(sy) : 0.0;
+    const double rx = sx > 0.0 ? metis_small::rsqrt_cubic(sx) : 0.0, ry = sy > 0.0 ? metis_small::rsqrt_cubic(sy) : 0.0;
     const int c = rank * JF_COLS + 2 * (s * JF_MB + m);
 #pragma unroll
     for (int t = 0; t < R; ++t) {
@@ -1023,7 +1023,7 @@ tridiag_vectors_kernel(const double* __restrict__ tri, const double* __restrict_
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const double pn = fma(d[u], p, -e2[u] * pm);
-        d[u] = pn * metis_small::rcp_newton(p + 1e-290);
+        d[u] = pn * metis_small::rcp_cubic(p + 1e-290);
         pm = p; p = pn;
       }
 #pragma unroll
@@ -1051,7 +1051,7 @@ tridiag_vectors_kernel(const double* __restrict__ tri, const double* __restrict_
     if (other < best || (other == best && oi < at)) { best = other; at = oi; }
   }
   for (int i = lane; i < n; i += 32) {
-    const double f = eo[i < at ? i : max(i - 1, 0)] * metis_small::rcp_newton((i < at ? Dp[i] : Dm[i]) + 1e-60);
+    const double f = eo[i < at ? i : max(i - 1, 0)] * metis_small::rcp_cubic((i < at ? Dp[i] : Dm[i]) + 1e-60);
     Dm[i] = i == at ? 1.0 : -f;
   }
   __syncwarp();
@@ -1074,7 +1074,7 @@ tridiag_vectors_kernel(const double* __restrict__ tri, const double* __restrict_
   }
   __syncwarp();
   zz += __shfl_xor_sync(0xFFFFFFFFu, zz, 1);
-  const double rz = metis_small::rsqrt_newton(__shfl_sync(0xFFFFFFFFu, zz, 0));
+  const double rz = metis_small::rsqrt_cubic(__shfl_sync(0xFFFFFFFFu, zz, 0));
   for (int i = lane; i < n; i += 32) zt[(int64_t)e * n + i] = Dm[i] * rz;
 }
 

@@ -26,8 +26,8 @@ __device__ __forceinline__ double rcp_step(double x, double y) {
   const double e = fma(-x, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ double rcp_newton(double x) { return rcp_step(x, rcp_seed(x)); }
-__device__ __forceinline__ double rsqrt_newton(double x) {
+__device__ __forceinline__ double rcp_cubic(double x) { return rcp_step(x, rcp_seed(x)); }
+__device__ __forceinline__ double rsqrt_cubic(double x) {
   const double y = rsqrt_seed(x), r = fma(-x * y, y, 1.0);
   return fma(y * r, fma(r, 0.375, 0.5), y);
 }

@@ -56,7 +56,7 @@ __device__ __forceinline__ void group_cholesky(double* Y, int n, double tol, dou
       for (int c = 0; c < 8; ++c) v[c] = r < n8 ? Y[r * P + c0 + c] : 0.0;
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const double d = a[j][j], rs = rsqrt_newton(d);  // (selected, not branched around)
+        const double d = a[j][j], rs = rsqrt_cubic(d);  // (selected, not branched around)
         const bool on = d > tol;
         inv[j] = on ? rs : 0.0;
         dmin = min(dmin, on ? __double2hiint(d) : 0x7FE00000);
@@ -562,7 +562,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
           const double pn = fma(d[u], p, -e2[u] * pm);
-          d[u] = pn * rcp_newton(p + 1e-290);
+          d[u] = pn * rcp_cubic(p + 1e-290);
           pm = p; p = pn;
         }
 #pragma unroll
@@ -600,7 +600,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
 #pragma unroll
       for (int t = 0; t < 2 * NT8; ++t) {
         const int i = s + 4 * t;
-        const double f = eo[i < at ? i : max(i - 1, 0)] * rcp_newton((i < at ? du[t] : dd[t]) + 1e-60);
+        const double f = eo[i < at ? i : max(i - 1, 0)] * rcp_cubic((i < at ? du[t] : dd[t]) + 1e-60);
         Z[i * P + e] = i < n ? (i == at ? 1.0 : -f) : 0.0;
       }
     }
@@ -623,7 +623,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
         i += 4 * step;
       }
       zz += __shfl_xor_sync(0xFFFFFFFFu, zz, 1);
-      if (step > 0 && e < N8) ys[e] = e < rank ? rsqrt_newton(zz) : 0.0;         // a dependent column of the factor: no vector
+      if (step > 0 && e < N8) ys[e] = e < rank ? rsqrt_cubic(zz) : 0.0;         // a dependent column of the factor: no vector
     }
   } else {
     // ---- meanwhile: the reflectors in panels of eight, H_8b ... H_8b+7 = I - V_b^T T_b V_b (T_b: inverse of diag(1 / beta) + the
@@ -784,7 +784,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
           for (int o = 4; o > 0; o >>= 1) { sx += __shfl_xor_sync(0xFFFFFFFFu, sx, o); sy += __shfl_xor_sync(0xFFFFFFFFu, sy, o); }
           if (active && sub < 2) {
             const double v = sub == 0 ? sx : sy;
-            inv_s[2 * (2 * m + h) + sub] = v > 0.0 ? rsqrt_newton(v) : 0.0;
+            inv_s[2 * (2 * m + h) + sub] = v > 0.0 ? rsqrt_cubic(v) : 0.0;
           }
         }
       }
@@ -854,7 +854,7 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
                 const double ro = 0.5 * r * (lam[i] + lam[j]);                     // what orthonormalising alone adds to S_ij
                 if (fmax(sv[u][e] * sv[u][e], ro * ro) > 1e-28 * fabs(lam[i] * lam[j])) {    // else orthogonal to FP64 rounding, and stays so
                   if (fabs(a) < 0.0625 * fabs(gap) && fabs(b) < 0.0625 * fabs(gap)) {
-                    const double rg = rcp_newton(gap);
+                    const double rg = rcp_cubic(gap);
                     e_ij = a * rg; e_ji = -b * rg;
                   } else if (sv[u][e] * sv[u][e] > 1e-24 * fabs(lam[i] * lam[j])) open = true;
                 }
@@ -931,8 +931,8 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
         __syncwarp();
         if (active && c * c > 1e-30 * (a * b)) {
           above |= c * c > 1e-13 * (a * b);
-          const double d = b - a, rh = rsqrt_newton(fma(4.0 * c, c, d * d));
-          const double cc = fma(0.5 * fabs(d), rh, 0.5), rs = rsqrt_newton(cc);
+          const double d = b - a, rh = rsqrt_cubic(fma(4.0 * c, c, d * d));
+          const double cc = fma(0.5 * fabs(d), rh, 0.5), rs = rsqrt_cubic(cc);
           const double cs = cc * rs, sn = (d < 0.0 ? -c : c) * rh * rs;
 #pragma unroll
           for (int t = 0; t < NT8; ++t) {

@@ -585,21 +585,26 @@ def test_a_wide_split_repeats_itself(ctx, k, p):
 
 def test_reciprocals_against_cuda_and_extended_precision(ctx):
     """The FP64 reciprocal and reciprocal square root of the dense kernels, from 2^-1000 to 2^1000 with 1e-290 and 1e-60 (what keeps a
-    pivot from zero) among them.  Error bounds: one rounding for the reciprocal, three halves of one for the root (its product is rounded
-    before it is subtracted), against 80-bit arithmetic; CUDA's own results are within one rounding (division) and two (root)."""
+    pivot from zero) among them, and both ends of every interval of 20 mantissa bits, over two binades: the hardware's approximation takes no more of
+    them, so its largest errors are there.  Error bounds, against 80-bit arithmetic: one rounding for the reciprocal, three halves of one
+    for the root (its product is rounded before it is subtracted), and the cube of the approximation's error, 2^-59 and 5/16 2^-57 (less than 2^-6
+    and 2^-5 of them); CUDA's own results are within one rounding (division) and two (root)."""
     B, h = ctx
     rng = np.random.default_rng(17)
     x = np.ldexp(rng.uniform(1.0, 2.0, 1 << 20), rng.integers(-1000, 1000, 1 << 20))
     x[:6] = [1e-290, 1e-60, 1.0, 2.0, 4.0, 1.0 - 2.0 ** -53]
     x[6:1024] = np.ldexp(1.0 + rng.integers(0, 64, 1018) * 2.0 ** -52, rng.integers(-600, 600, 1018))       # just above powers of two
+    ends = (np.int64(0x3FF00000) + np.arange(1 << 21, dtype=np.int64)) << 32                                # 1 to 4
+    x = np.concatenate((x, ends.view(np.float64), (ends + 0xFFFFFFFF).view(np.float64)))
     dx = torch.from_numpy(x).cuda()
     rcp, rsq = h.reciprocals(dx)
     wide = x.astype(np.longdouble)
-    for got, ref, bound in ((rcp, 1.0 / wide, 1.0), (rsq, 1.0 / np.sqrt(wide), 1.5)):
+    for got, ref, bound in ((rcp, 1.0 / wide, 1.0 + 2.0 ** -6), (rsq, 1.0 / np.sqrt(wide), 1.5 * (1.0 + 2.0 ** -5))):
         err = np.max(np.abs(got.cpu().numpy().astype(np.longdouble) - ref) / ref)
-        assert err <= bound * 2.0 ** -53 * (1.0 + 2.0 ** -10), float(err * 2.0 ** 53)
-    for got, ref, bound in ((rcp, 1.0 / dx, 2.0), (rsq, torch.rsqrt(dx), 3.5)):
-        assert ((got - ref).abs() / ref).max() <= bound * 2.0 ** -53 * (1.0 + 2.0 ** -10)
+        print("largest error in units of 2^-53: %.4f (bound %.4f)" % (float(err * 2.0 ** 53), bound))
+        assert err <= bound * 2.0 ** -53, float(err * 2.0 ** 53)
+    for got, ref, bound in ((rcp, 1.0 / dx, 2.0 + 2.0 ** -6), (rsq, torch.rsqrt(dx), 3.5 + 1.5 * 2.0 ** -5)):
+        assert ((got - ref).abs() / ref).max() <= bound * 2.0 ** -53
     neg = h.reciprocals(-dx)[0]
     assert torch.equal(neg, -rcp)
 
