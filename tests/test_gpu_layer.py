@@ -316,9 +316,11 @@ def test_ragged_layer_through_the_two_cta_gemm(ctx):
     (128, 448, 192, 8, 12, 4),            # residual product in the group, unequal ranks
     (320, 2112, 576, 36, 32, 40),         # 33-vector remainders of the finishing kernel, ragged K
     (512, 256, 4160, 16, 16, 16),         # contractions of 17 K blocks divided by eight, of one and of two beside them
-    (4096, 256, 320, 64, 48, 64),         # more than one CTA per SM, two rows per warp of the finishing kernel
-    (9216, 256, 256, 16, 20, 12),         # four rows per warp
+    (4096, 256, 320, 64, 48, 64),         # 64 vectors beside 48: two 32-vector groups, one row per warp
+    (9216, 256, 256, 16, 20, 12), (9216, 256, 256, 40, 36, 64),           # two rows per warp (from 7105 rows on), one and two 32-vector groups
+    (19200, 256, 256, 16, 20, 12), (19200, 256, 256, 40, 36, 64),         # four rows per warp (from 14209 on); more CTAs than SMs: four stages, two CTAs an SM
     (256, 512, 768, 72, 64, 64),          # a rank above 64 beside ranks below it
+    (1024, 4096, 4096, 128, 100, 128),    # ranks above 64 whose contractions would fill a second round of CTAs
 ])
 def test_skinny_products_in_one_launch(ctx, l, n, m, kd, kx, kw):
     """Forward and both gradients against float64 products of the library's own codes (exact codes, FP32 sums: 2e-5)."""
