@@ -1153,13 +1153,19 @@ factors_kernel(FactorsArgs f, int n_right) {
   }
 }
 
-// Columns per sketch CTA: a sampled sketch has few rows, so narrow chunks are what gives it enough CTAs; a full
-// sketch has one CTA per 256 rows already and wide chunks keep the partial buffer small.
+// CTAs and cluster of coef_finish_kernel, 32 rows to a CTA, a Gram partial to a cluster
+void coef_grid(int64_t rows, int* ctas, int* csize) {
+  const int64_t n = metis_ceil_div(rows, 32);
+  int c = 1;
+  while (c < GR_CLUSTER && c < n) c *= 2;
+  *csize = c; *ctas = (int)(metis_ceil_div(n, c) * c);
+}
 // accumulator columns of the tensor-core sketch: k + p rounded up to what the coefficient kernel is built for
 int sketch_tc_cols(int q) { return q <= 48 ? 48 : 96; }
 
 // Column chunks of a sampled sketch: 64 columns each (a 160-row sketch has one row block, so narrow chunks are what gives it CTAs), wider ones or more than
 // one to a CTA beyond 128 CTAs, so that the clusters leave at most GR_PARTS partials.
+// (of any length of the sample the shortest leaves the most)
 struct SketchGrid { int ccols, chunks, ctas, csize, parts; };
 SketchGrid sketch_grid(int64_t cols, int64_t n_s) {
   SketchGrid s{};
@@ -1185,7 +1191,7 @@ SplitWs split_ws_layout(int64_t rows, int64_t cols, int k, int p, int64_t n_s) {
   w.amax = take(256);
   // the full-mode tensor-core sketch writes slices x rows x nb partials into the buffer of the sampled one's
   const int nb_sk = sketch_tc_cols(q);
-  const size_t zp_mma = (size_t)GR_PARTS * n_s * q, zp_tc = (size_t)metis_coeff_slices(rows, cols, nullptr) * rows * nb_sk;
+  const size_t zp_mma = (size_t)sketch_grid(cols, 0).parts * n_s * q, zp_tc = (size_t)metis_coeff_slices(rows, cols, nullptr) * rows * nb_sk;
   w.zp = take(sizeof(float) * (zp_mma > zp_tc ? zp_mma : zp_tc));
   w.omt = take(sizeof(__nv_bfloat16) * (size_t)nb_sk * cols);
   w.z = take(sizeof(float) * (size_t)n_s * q);
@@ -1204,7 +1210,9 @@ SplitWs split_ws_layout(int64_t rows, int64_t cols, int k, int p, int64_t n_s) {
   w.b6 = take(sizeof(__nv_bfloat16) * (size_t)metis_residual_kx(kp) * cols);
   w.hsp = take(sizeof(__nv_bfloat16) * 3 * (size_t)((q + 15) / 16 * 16) * (size_t)((n_s + 63) / 64 * 64));
   w.bs = take(sizeof(__nv_bfloat16) * 3 * (size_t)kp * cols);
-  w.gram_c = take(sizeof(double) * (size_t)metis_ceil_div(rows, 32) * kp * kp);
+  int ctas_c, csize_c;
+  coef_grid(rows, &ctas_c, &csize_c);
+  w.gram_c = take(sizeof(double) * (size_t)(ctas_c / csize_c) * kp * kp);
   w.keys = take(sizeof(unsigned long long) * MAXQ);
   w.evals2 = take(sizeof(double) * MAXQ);
   w.evecs2 = take(sizeof(double) * MAXQ * MAXQ);
@@ -1885,8 +1893,8 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   }
   METIS_TRY(launch_eig(s, gram, parts, q, q, evals, evecs));
   // (5) right basis and its splits; coefficients of every row in the basis, (6) fused residual + quantizer
-  const int n_cta_c = (int)metis_ceil_div(rows, 32);
-  int csize_c = 1;                                        // CTAs of the coefficients' last kernel to a Gram partial
+  int ctas_c, csize_c;                                    // of the coefficients' last kernel
+  coef_grid(rows, &ctas_c, &csize_c);
   const int n_cta_cols = (int)metis_ceil_div(cols, FR_POS), n_cta_rows = (int)metis_ceil_div(rows, FR_POS);
   float* rb = full ? out->right : basis;
   METIS_TRY(launch_basis(s, n_cta_cols, fr_smem(q), m, cols, q, k, kp, evals, evecs, rb, full ? (__nv_bfloat16*)nullptr : bs, b6, kx6, full ? out->sigma : nullptr, full ? keys : nullptr, amax + 2));
@@ -1901,9 +1909,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
     // tensor-core pass over x (column slices), then the slices are summed and the Gram partials formed
     METIS_TRY(metis_launch_coeff_tc(ctx, x, rows, cols, bs, kp, part, amax, 0, s));
     const int slices = metis_coeff_slices(rows, cols, nullptr);
-    while (csize_c < GR_CLUSTER && csize_c < n_cta_c) csize_c *= 2;
-    const dim3 grid_c((unsigned)metis_ceil_div(n_cta_c, csize_c) * (unsigned)csize_c);
-#define METIS_CF(KP) METIS_CUDA_TRY(metis_launch_pdl_cluster((coef_finish_kernel<KP>), grid_c, dim3(256), (size_t)(0), s, 0, csize_c, (const float*)part, slices, rows, coef, gram_c, a6, kx6)); break
+#define METIS_CF(KP) METIS_CUDA_TRY(metis_launch_pdl_cluster((coef_finish_kernel<KP>), dim3((unsigned)ctas_c), dim3(256), (size_t)(0), s, 0, csize_c, (const float*)part, slices, rows, coef, gram_c, a6, kx6)); break
     switch (kp) {
       case 16: METIS_CF(16);
       case 32: METIS_CF(32);
@@ -1928,7 +1934,7 @@ metis_status_t metis_split(metis_handle_t h, const void* xv, int32_t dtype, int6
   cudaStream_t sf = ctx->side[0];
   if (!full) {
     // (7) Rayleigh-Ritz on C^T C (Gram partials came out of the broadcast pass), rotate both factors
-    int parts_c = (int)metis_ceil_div(n_cta_c, csize_c);
+    int parts_c = ctas_c / csize_c;
     const double* g2 = gram_c;
     if (parts_c > GR_PARTS) {                             // more than 4096 rows: summed on many CTAs first
       METIS_CUDA_TRY(metis_launch_pdl((reduce_gram_kernel), dim3((unsigned)metis_ceil_div(kp * kp, 32)), dim3(128), (size_t)(0), sf, (const double*)gram_c, parts_c, kp * kp, gram1, (const int*)nullptr)); METIS_COUNT_LAUNCH();

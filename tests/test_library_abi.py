@@ -103,3 +103,11 @@ def test_operand_structures_hold_their_members(k, axes):
     assert members(st.left_q) == nvfp4(op.left_q, k) and members(st.right_q) == nvfp4(op.right_q, k)
     assert members(st.res_by_cols) == nvfp4(op.res_by_cols, 64) and members(st.res_by_rows) == nvfp4(op.res_by_rows, 128)
     assert members(op.right_q.struct()) == nvfp4(op.right_q, max(k, 1))
+
+
+@pytest.mark.parametrize("rows,cols,k,p,reserved", [(1 << 20, 64, 4, 4, 812388608), (131072, 256, 8, 8, 108606720), (524288, 512, 64, 8, 1920849152),
+                                                    (16384, 128, 16, 8, 22562048), (65536, 1024, 32, 8, 136713472), (4096, 4096, 32, 8, 35345664)])
+def test_splits_run_in_the_scratch_that_callers_have_reserved(rows, cols, k, p, reserved):
+    """A caller that keeps its workspace at a fixed size keeps its calls: no later layout asks for more than these."""
+    from paper_2509_00404_b200 import binding as B
+    assert B.workspace_bytes(1, rows, cols, k, p) <= reserved
