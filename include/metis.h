@@ -15,7 +15,7 @@
  * General rules
  *  - Every pointer is a DEVICE pointer unless its comment says "host".  The caller owns every
  *    buffer (inputs, outputs, workspace); the library allocates device memory only inside
- *    metis_create (a 128 KiB quantile table and a status word; it also creates five streams and six
+ *    metis_create (a 128 KiB quantile table and a status word; it also creates one stream and two
  *    events there and sets the per-device kernel attributes) and frees it in metis_destroy.
  *  - All work is enqueued on the caller's stream (a cudaStream_t passed as void*); calls return
  *    without synchronising.  Inside a call, independent sub-chains may run on streams the handle owns;
@@ -227,8 +227,8 @@ metis_status_t metis_quantize_rht_nvfp4(metis_handle_t h, const void* x, int32_t
  * reduction of its own, i.e. a second read of x that a supplied value saves.  The value is trusted: a value below
  * the true maximum makes the largest elements saturate.
  * Requires rows % 16 == 0, cols % 64 == 0 (tiled scales), k % 4 == 0, k <= 256 and k + p <= 272.
- * Up to k = 64 and k + p = 72 the orthonormalisation and the two small eigen-solvers each run in one CTA's
- * shared memory; above that (the 1.5 % rank of an 8192-wide layer is 128) they run on FP64 kernels tiled over the
+ * Up to k = 64 and k + p = 72 the two small eigen-solvers each run in one CTA's shared memory and the orthonormalisation of up
+ * to 1024 rows in a cluster of eight; above that (the 1.5 % rank of an 8192-wide layer is 128) they run on FP64 kernels tiled over the
  * rank and on an eight-CTA cluster, which additionally needs rows % 64 == 0.  Larger ranks are refused with
  * METIS_ERR_SHAPE.
  * Workspace: metis_workspace_bytes(1, rows, cols, k, p) (for the wide ranks: sized for the default sample count;

@@ -496,9 +496,11 @@ constexpr int NUM_THREADS = 384;                            // producer, MMA iss
 constexpr int OUT_STAGE_BYTES = 8 * 4096;                   // per epilogue warp: 32 rows x 128 bytes of converted output
 constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + OUT_STAGE_BYTES + 1024 + 256;
 
-// Arrive on the barrier at the same shared-memory offset in CTA `rank` of the cluster.  What it announces are tensor-memory reads, which
-// tcgen05.wait::ld has completed and tcgen05.fence::before_thread_sync puts in front of it; there are no writes for the other CTA to see, and a release at
-// cluster scope, which waits for all of the thread's, held the accumulator for 1650 of the 2600 cycles between two tiles' products.
+// Arrive on the barrier at the same shared-memory offset in CTA `rank` of the cluster.  What it announces are tensor-memory reads, and nothing that was
+// written: tcgen05.wait::ld, tcgen05.fence::before_thread_sync, this relaxed arrive, and on the other side the wait, tcgen05.fence::after_thread_sync and the
+// next MMA are the pattern that the PTX manual gives for tcgen05 operations of different threads that complete by a wait (tcgen05 memory consistency model,
+// canonical synchronization patterns); the loads are the whole warp's, and __syncwarp stands between its fences and the one lane that arrives.  A
+// release at cluster scope waits for all stores of the thread as well and held the accumulator for 1650 of the 2600 cycles between two tiles' products.
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t local_bar, uint32_t rank) {
   asm volatile(
       "{ .reg .b32 ra; mapa.shared::cluster.u32 ra, %0, %1;\n"

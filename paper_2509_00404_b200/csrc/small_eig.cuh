@@ -528,8 +528,8 @@ eig_kernel(const double* __restrict__ gm, int parts, int n, int ld, double* __re
   __syncthreads();
   double *Dp = E, *Z = U;                               // column e of each: vector e
   constexpr int TV = 4 * N8;                            // four threads per vector
-  // Lanes per eigenvalue in the multisection, two points each, so that a warp (or two) runs on each of the four schedulers: a round costs 25 cycles per
-  // row and warp there (three points on fewer warps: n = 40 1290 -> 1650 cycles a round).
+  // Lanes per eigenvalue in the multisection, two points each, so that a warp (or two) runs on each of the four schedulers: a round at n = 40 is 1290
+  // cycles, 1180 of them the Sturm sequences (three points on fewer warps: 1650).
   constexpr int LE = N8 <= 32 ? 4 : (N8 <= 40 || N8 > 64 ? 3 : 2), PW = 32 / LE, TE = (N8 + PW - 1) / PW * 32;
   {
     if (tid < TE) {

@@ -41,15 +41,11 @@ __global__ void sample_rows_kernel(int* __restrict__ idx, int n_s, RowSample rs)
 }
 
 // ------------------------------------------------------------------------------------------------
-// Device-detected conditions of a split: amax|x| not finite (a NaN or an infinity in the operand: amax is kept as
-// an ordered bit pattern, so a NaN ranks above every number), a non-finite eigenvalue.  One warp.
-__global__ void split_status_kernel(const float* __restrict__ amax, const double* __restrict__ evals, int k, uint32_t* dev_status) {
+// amax|x| not finite: a NaN or an infinity in the operand (amax is kept as an ordered bit pattern, so a NaN ranks above every number).  For a quantizer
+// that does not look itself; a split's amax and eigenvalues are looked at by its factor quantizer.
+__global__ void amax_status_kernel(const float* __restrict__ amax, uint32_t* dev_status) {
   metis_pdl_wait_trigger();
-  uint32_t bits = 0u;
-  if (threadIdx.x == 0 && !(fabsf(*amax) <= 3.0e38f)) bits |= METIS_DEV_NONFINITE;
-  for (int j = threadIdx.x; j < k; j += 32)
-    if (!(fabs(evals[j]) <= 1.0e300)) bits |= METIS_DEV_NUMERIC;
-  if (bits) atomicOr(dev_status, bits);
+  if (threadIdx.x == 0 && !(fabsf(*amax) <= 3.0e38f)) atomicOr(dev_status, METIS_DEV_NONFINITE);
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -1709,7 +1705,7 @@ metis_status_t metis_split_set_attrs() {
 
 // flags METIS_DEV_NONFINITE when *amax (the amax of a tensor about to be quantized) is not a finite number
 metis_status_t metis_launch_amax_check(metis_context* ctx, const float* amax, cudaStream_t s) {
-  METIS_CUDA_TRY(metis_launch_pdl((split_status_kernel), dim3(1), dim3(32), (size_t)(0), s, amax, (const double*)nullptr, 0, ctx->dev_status));
+  METIS_CUDA_TRY(metis_launch_pdl(amax_status_kernel, dim3(1), dim3(32), (size_t)0, s, amax, ctx->dev_status));
   METIS_COUNT_LAUNCH();
   return METIS_OK;
 }
