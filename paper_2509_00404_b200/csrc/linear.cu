@@ -207,7 +207,7 @@ lowrank_deq_wide_kernel(const __grid_constant__ FinishArgs first, const __grid_c
   float *__restrict__ lcat = f.lcat, *__restrict__ rcat = f.rcat;
   __nv_bfloat16 *__restrict__ lx = f.lx, *__restrict__ rx = f.rx;
   const int tid = threadIdx.x, kc = ka + kb;
-  const int64_t i0 = (int64_t)blockIdx.x * 32 + 8 * (tid & 3);      // this thread's eight rows (M, N are multiples of 16)
+  const int64_t i0 = (int64_t)blockIdx.x * 32 + 8 * (tid & 3);      // this thread's eight rows (an extent with factors is a multiple of 64)
   const float tsa = ka ? *foa_ts : 0.0f, tsb = kb ? *fob_ts : 0.0f;
   for (int u = tid >> 2; u < ka; u += 64) {
     if (i0 >= M) break;

@@ -1243,7 +1243,7 @@ metis_status_t launch_sum_gram(cudaStream_t s, const float* part, int slices, in
 // sum_gram_kernel adds the parts (mp).  The rule counts rounds of CTAs times chunks of 64 rows behind one another (1.4 us, a third more with two CTAs on an
 // SM), six more for a CTA's start and end and twelve for the launch behind; samples of up to 1024 rows have no use for it.  Whole split, all rows in one CTA -> in
 // parts (and as slabs of 512 rows with FP32 partials, before both): p = 8, 8192 of 16384 x 1024, k = 32 355 -> 201 us (230); 4096 of 16384 x 4096 341 -> 269
-// (282); every row of 16384 x 4096 in a sample, k = 64 1247 -> 816 (881); 1312 of 131072 x 256, k = 8 171 -> 153 (270); 8192 of 16384 x 14336 1030 -> 826 (796).
+// (282); every row of 16384 x 4096 in a sample, k = 64 1247 -> 816 (881); 1312 of 131072 x 256, k = 8 171 -> 153 (270); 8192 of 16384 x 14336 1030 -> 830 (797).
 metis_status_t launch_project_gram(metis_context* ctx, cudaStream_t s, const __nv_bfloat16* x, int64_t cols, const RowSample& rs, int n_s, int q, const __nv_bfloat16* hsp, int ldh, float* m, double* gram,
                                    float* mp, int* parts) {
   const int64_t tiles = metis_ceil_div(cols, PG_COLS), chunks = metis_ceil_div(n_s, PG_K);
