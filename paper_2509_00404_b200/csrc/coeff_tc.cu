@@ -233,10 +233,6 @@ int metis_coeff_slices(int64_t rows, int64_t cols, int* chunks_per_slice) {
   return (int)metis_ceil_div(chunks, cps);                // every slice has work
 }
 
-bool metis_coeff_tc_usable(const void* x, const void* bs, int64_t cols, int kp) {
-  return metis_aligned16(x) && metis_aligned16(bs) && cols % 8 == 0 && (kp == 16 || kp == 32 || kp == 48 || kp == 64);
-}
-
 // part: [metis_coeff_slices(rows, cols, ..)][rows][kp] FP32; bs: [3][kp][cols] BF16 (three-term split of the basis).
 // raw = 1: the operand is a single (3 * kp) x cols BF16 matrix and the accumulator columns are written unsummed,
 // part[slice][rows][3 * kp] (the sketch Z = X Omega of a full-mode split).

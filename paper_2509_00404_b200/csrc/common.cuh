@@ -293,7 +293,6 @@ metis_status_t metis_launch_quantize(const void* x, int dtype, int64_t rows, int
                                      const float* tscale_src, int tscale_is_amax, const metis_nvfp4_t* by_cols,
                                      const metis_nvfp4_t* by_rows, cudaStream_t s, uint32_t* dbg_status = nullptr);
 int metis_coeff_slices(int64_t rows, int64_t cols, int* chunks_per_slice);
-bool metis_coeff_tc_usable(const void* x, const void* bs, int64_t cols, int kp);
 metis_status_t metis_launch_coeff_tc(metis_context* ctx, const void* x, int64_t rows, int64_t cols, const void* bs, int kp,
                                      float* part, float* amax, int raw, cudaStream_t s);
 // what a split reports in the status word: an amax that is not finite, an eigenvalue that is not finite
